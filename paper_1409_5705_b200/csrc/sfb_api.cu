@@ -1,5 +1,6 @@
 // C ABI of libsfb: argument checking, workspace carve-up, and the sequencing of one SFB step
 // (Section 3, Figure 1: compute factors -> broadcast/gather -> reconstruct and apply -> prox).
+#include <algorithm>
 #include <new>
 
 #include "sfb_internal.h"
@@ -24,6 +25,21 @@ int sm_count() {
 
 static size_t up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
 
+// The coder's iterations a <- soft(a - W^T (W a - x) / L) either take two products with W each, or one with the Gram matrix
+// W^T W, formed once per step (half of it: it is symmetric), and W^T x.  The Gram form wins when the dictionary has at most
+// about twice as many atoms as features and the mini-batch is large enough to repay W^T W; decided by the cost of the
+// products themselves.
+bool sc_use_gram(const sfb_config& c) {
+  const int64_t K = static_cast<int64_t>(c.workers) * c.batch, D = c.rows, A = c.cols;
+  const double it = c.sc_ista_iters - 1;
+  if (it < 1 || A > (32 << 10)) return false;        // (the power iteration keeps a vector of A values on chip)
+  auto cost = [](int64_t M, int64_t N, int64_t Kc, bool sym) {
+    const GemmShape g = pick_gemm_shape(M, N, Kc, sym);
+    return std::min(gemm_cost(128, g.split, M, N, Kc, sym), gemm_cost(64, g.split, M, N, Kc, sym));
+  };
+  return cost(A, A, D, true) + it * cost(K, A, A, false) < it * (cost(K, D, A, false) + cost(K, A, D, false));
+}
+
 Layout make_layout(const sfb_config& cfg) {
   sfb_config c = cfg;
   if (c.model == SFB_L2MLR) c.model = SFB_MLR;        // same buffers: the factors differ, the products do not
@@ -40,16 +56,21 @@ Layout make_layout(const sfb_config& cfg) {
   L.stageY = take(c.model == SFB_DML ? K * cols * 4 : 0);
   L.stageL = take(K * 4);
   L.colpart = take(c.model == SFB_SC ? static_cast<size_t>(kProxSlabs) * cols * 8 : 0);
-  L.pib = take(c.model == SFB_SC ? cols * 4 : 0);
-  L.piy = take(c.model == SFB_SC ? rows * 4 : 0);
+  L.pi = take(c.model == SFB_SC && !(c.sc_lipschitz > 0.f) ? power_scratch_bytes(c.cols) : 0);
   L.Kp = static_cast<int64_t>(K);
   L.colsb = static_cast<int64_t>(cols);
   L.ldu = static_cast<int64_t>(rows);
   if (use_tf32(cfg)) {
     tc32_extend_layout(c, L, off);
   } else if (c.precision != SFB_PREC_BF16) {
+    L.ldu = round_up(c.rows, 4);                      // 16-byte row pitch
     L.V = take(K * cols * 4);
-    L.U = take(K * rows * 4);
+    L.U = take(K * static_cast<size_t>(L.ldu) * 4);
+    if (c.model == SFB_SC && sc_use_gram(c)) {
+      L.G = take(cols * cols * 4);
+      L.Bx = take(K * cols * 4);
+    }
+    if (c.model == SFB_SC) L.V2 = take(K * cols * 4);
   } else {
     tc_extend_layout(c, L, off);
   }
@@ -185,42 +206,80 @@ extern "C" int sfb_destroy(sfb_ctx* ctx) {
 static int factors_fp32(sfb_ctx* ctx, int64_t off, int64_t n, const float* X, const float* Y,
                         const int32_t* labels, bool sparse_fwd = false, float* dml_norm_out = nullptr) {
   const sfb_config& c = ctx->cfg;
-  const int64_t rows = c.rows, cols = c.cols;
+  const int64_t rows = c.rows, cols = c.cols, ldu = ctx->lay.ldu, K = ctx->K;
   float* V = ctx->at<float>(ctx->lay.V) + off * cols;
-  float* U = ctx->at<float>(ctx->lay.U) + off * rows;
+  float* U = ctx->at<float>(ctx->lay.U) + off * ldu;
   Scalars* sc = ctx->at<Scalars>(ctx->lay.scalars);
   uint32_t* status = ctx->at<uint32_t>(ctx->lay.status);
   cudaStream_t s = ctx->stream;
   EpiArgs e{};
   if (c.model == SFB_MLR || c.model == SFB_DML) {
     CK(pack_copy(s, V, X, c.model == SFB_DML ? Y : nullptr, n * cols));                 // v = x | x - y
-    e.C = U; e.ldc = rows;
+    e.C = U; e.ldc = ldu;
     if (sparse_fwd) {                                                                   // z_i = W v_i over the non-zeros of v_i
-      const int rc = sparse_forward(ctx, off, n, ctx->at<float>(ctx->lay.U), rows);
+      const int rc = sparse_forward(ctx, off, n, ctx->at<float>(ctx->lay.U), ldu);
       if (rc) return rc;
     } else {
-      CK(sgemm(s, true, true, EPI_STORE, n, rows, cols, V, cols, ctx->W, cols, e));     // z_i = W v_i
+      CK(sgemm(s, true, true, EPI_STORE, n, rows, cols, V, cols, ctx->W, cols, e, K));  // z_i = W v_i
       ctx->stats.flops += 2.0 * n * rows * cols;
     }
     if (c.model == SFB_MLR)
-      CK(mlr_softmax_rows(s, U, n, rows, labels, ctx->at<float>(ctx->lay.loss) + off, status));
+      CK(mlr_softmax_rows(s, U, n, rows, ldu, labels, ctx->at<float>(ctx->lay.loss) + off, status));
     else
-      CK(dml_scale_rows(s, U, n, rows, rows, labels, c.dml_margin, nullptr, dml_norm_out));
+      CK(dml_scale_rows(s, U, n, rows, ldu, labels, c.dml_margin, nullptr, dml_norm_out));
     return SFB_OK;
   }
-  // sparse coding: ISTA from a = 0, then u = W a - x, v = a
-  CK(fill_zero(s, V, n * cols));
-  for (int it = 0; it <= c.sc_ista_iters; ++it) {
-    e = EpiArgs{};
-    e.C = U; e.ldc = rows; e.aux = X;
-    CK(sgemm(s, true, true, EPI_SUB, n, rows, cols, V, cols, ctx->W, cols, e));         // r = W a - x
-    ctx->stats.flops += 2.0 * n * rows * cols;
-    if (it == c.sc_ista_iters) break;
-    e = EpiArgs{};
-    e.C = V; e.ldc = cols; e.sc = sc; e.lam = c.sc_lambda;
-    CK(sgemm(s, true, false, EPI_ISTA, n, cols, rows, U, rows, ctx->W, cols, e));       // a <- soft(a - W^T r / L)
+  // Sparse coding: ISTA from a = 0, then u = W a - x, v = a.  The first iterate is soft(W^T x / L).
+  const int T = c.sc_ista_iters;
+  const bool gram = ctx->lay.G != 0;
+  float* V2 = ctx->at<float>(ctx->lay.V2) + off * cols;
+  float* Bx = gram ? ctx->at<float>(ctx->lay.Bx) + off * cols : nullptr;
+  const float* G = ctx->at<float>(ctx->lay.G);
+  auto iterate = [&](int t) { return ((T - t) & 1) == 0 ? V : V2; };                    // where a_t goes: a_T to V
+  if (T == 0) {
+    CK(fill_zero(s, V, n * cols));
+  } else {
+    e.C = iterate(1); e.ldc = cols; e.C2 = Bx; e.ldc2 = cols; e.sc = sc; e.lam = c.sc_lambda;
+    CK(sgemm(s, true, false, EPI_ISTA0, n, cols, rows, X, rows, ctx->W, cols, e, K));   // W^T x, a_1
     ctx->stats.flops += 2.0 * n * rows * cols;
   }
+  for (int t = 2; t <= T; ++t) {
+    EpiArgs q{};
+    q.C = iterate(t); q.ldc = cols; q.cur = iterate(t - 1); q.ldcur = cols; q.sc = sc; q.lam = c.sc_lambda;
+    if (gram) {
+      q.aux = Bx; q.ldaux = cols;
+      CK(sgemm(s, true, false, EPI_ISTA, n, cols, cols, q.cur, cols, G, cols, q, K));   // a <- soft(a - (W^T W a - W^T x) / L)
+      ctx->stats.flops += 2.0 * n * cols * cols;
+    } else {
+      e = EpiArgs{};
+      e.C = U; e.ldc = ldu; e.aux = X; e.ldaux = rows;
+      CK(sgemm(s, true, true, EPI_SUB, n, rows, cols, q.cur, cols, ctx->W, cols, e, K));    // r = W a - x
+      CK(sgemm(s, true, false, EPI_ISTA, n, cols, rows, U, ldu, ctx->W, cols, q, K));       // a <- soft(a - W^T r / L)
+      ctx->stats.flops += 4.0 * n * rows * cols;
+    }
+  }
+  e = EpiArgs{};
+  e.C = U; e.ldc = ldu; e.aux = X; e.ldaux = rows;
+  CK(sgemm(s, true, true, EPI_SUB, n, rows, cols, V, cols, ctx->W, cols, e, K));        // u = W a - x
+  ctx->stats.flops += 2.0 * n * rows * cols;
+  return SFB_OK;
+}
+
+// What the factors of every worker of a step share, formed from the W that they all see (bulk-synchronous consistency):
+// the coder's Gram matrix and its step size.
+static int begin_step(sfb_ctx* ctx) {
+  const sfb_config& c = ctx->cfg;
+  if (c.model != SFB_SC) return SFB_OK;
+  float* G = ctx->lay.G ? ctx->at<float>(ctx->lay.G) : nullptr;
+  if (c.precision == SFB_PREC_FP32 && G) {
+    EpiArgs e{};
+    e.C = G; e.ldc = c.cols;
+    CK(sgemm(ctx->stream, false, false, EPI_SYM, c.cols, c.cols, c.rows, ctx->W, c.cols, ctx->W, c.cols, e));
+    ctx->stats.flops += static_cast<double>(c.cols) * c.cols * c.rows;
+  }
+  if (!(c.sc_lipschitz > 0.f))
+    CK(estimate_lipschitz(ctx->stream, ctx->W, G, c.rows, c.cols, ctx->at<char>(ctx->lay.pi),
+                          ctx->at<Scalars>(ctx->lay.scalars), ctx->at<uint32_t>(ctx->lay.status), 50));
   return SFB_OK;
 }
 
@@ -230,7 +289,7 @@ static int update_fp32(sfb_ctx* ctx) {
   EpiArgs e{};
   e.C = ctx->W; e.ldc = c.cols; e.alpha = -ctx->step;
   e.prox_kind = ctx->prox_kind; e.prox_a = ctx->prox_a;
-  CK(sgemm(ctx->stream, false, false, EPI_RMW, c.rows, c.cols, ctx->K, ctx->at<float>(ctx->lay.U), c.rows,
+  CK(sgemm(ctx->stream, false, false, EPI_RMW, c.rows, c.cols, ctx->K, ctx->at<float>(ctx->lay.U), ctx->lay.ldu,
            ctx->at<float>(ctx->lay.V), c.cols, e));
   return SFB_OK;
 }
@@ -257,11 +316,7 @@ extern "C" int sfb_compute_factors(sfb_ctx* ctx, int32_t worker, const float* X_
     ctx->sparse_mask = 0;
     ctx->csr_fill = 0;
     CK(cudaEventRecord(ctx->ev[0], ctx->stream));
-    // the coder's step size comes from the W every worker sees at the start of the step (BSP)
-    if (c.model == SFB_SC && !(c.sc_lipschitz > 0.f))
-      CK(estimate_lipschitz(ctx->stream, ctx->W, c.rows, c.cols, ctx->at<float>(ctx->lay.pib),
-                            ctx->at<float>(ctx->lay.piy), ctx->at<float>(ctx->lay.colpart),
-                            ctx->at<Scalars>(ctx->lay.scalars), 50));
+    if ((rc = begin_step(ctx)) != SFB_OK) return rc;
   }
   // bf16 mode: every product runs on the tensor cores; DML and SC, whose u comes from a cancelling residual,
   // carry each value as a (hi, lo) pair of bf16 (fp32-class products)
@@ -359,13 +414,14 @@ extern "C" int sfb_forward_partials(sfb_ctx* ctx, const float* X_dev, const int3
     float* U = ctx->at<float>(ctx->lay.U);
     CK(pack_copy(ctx->stream, V, X_dev, nullptr, K * c.cols));                                    // v = x
     EpiArgs e{};
-    e.C = U; e.ldc = c.rows;
+    const int64_t ldu = ctx->lay.ldu;
+    e.C = U; e.ldc = ldu;
     CK(sgemm(ctx->stream, true, true, EPI_STORE, K, c.rows, c.cols, V, c.cols, ctx->W, c.cols, e));   // z_i = W_shard x_i
     ctx->stats.flops += 2.0 * K * c.rows * c.cols;
     // the class ids are kept for the finish (the caller's buffer may change before it)
     CK(cudaMemcpyAsync(ctx->at<int32_t>(ctx->lay.stageL), labels_dev, static_cast<size_t>(K) * 4, cudaMemcpyDeviceToDevice,
                        ctx->stream));
-    CK(mlr_shard_partials(ctx->stream, U, K, c.rows, c.rows, ctx->at<int32_t>(ctx->lay.stageL), ctx->row_offset,
+    CK(mlr_shard_partials(ctx->stream, U, K, c.rows, ldu, ctx->at<int32_t>(ctx->lay.stageL), ctx->row_offset,
                           partials_dev));
   }
   ctx->partials_ready = true;
@@ -403,7 +459,7 @@ extern "C" int sfb_finish_factors(sfb_ctx* ctx, const float* partials_all_dev, i
   if (!ctx->partials_ready) return SFB_ERR_STATE;
   const sfb_config& c = ctx->cfg;
   if (c.model == SFB_DML) {
-    const int64_t ldu = c.precision == SFB_PREC_FP32 ? c.rows : ctx->lay.ldu;
+    const int64_t ldu = ctx->lay.ldu;
     CK(dml_scale_rows(ctx->stream, ctx->at<float>(ctx->lay.U), ctx->K, c.rows, ldu, ctx->at<int32_t>(ctx->lay.stageL),
                       c.dml_margin, nullptr, nullptr, partials_all_dev, shards, ctx->K));
     ctx->partials_ready = false;
@@ -416,7 +472,7 @@ extern "C" int sfb_finish_factors(sfb_ctx* ctx, const float* partials_all_dev, i
                              : tc_finish_factors(ctx, partials_all_dev, shards);
     if (rc) return rc;
   } else {
-    CK(mlr_shard_finish(ctx->stream, ctx->at<float>(ctx->lay.U), ctx->K, c.rows, c.rows, ctx->at<int32_t>(ctx->lay.stageL),
+    CK(mlr_shard_finish(ctx->stream, ctx->at<float>(ctx->lay.U), ctx->K, c.rows, ctx->lay.ldu, ctx->at<int32_t>(ctx->lay.stageL),
                         ctx->row_offset, partials_all_dev, shards, ctx->at<float>(ctx->lay.loss),
                         ctx->at<uint32_t>(ctx->lay.status)));
   }
@@ -444,7 +500,7 @@ extern "C" int sfb_set_factors(sfb_ctx* ctx, int32_t worker, const float* U_dev,
     ctx->gathered = false;
     return SFB_OK;
   }
-  const int64_t ldu = c.precision == SFB_PREC_FP32 ? c.rows : ctx->lay.ldu;
+  const int64_t ldu = ctx->lay.ldu;
   float* U = ctx->at<float>(ctx->lay.U) + off * ldu;
   float* V = ctx->at<float>(ctx->lay.V) + off * c.cols;
   CK(cudaMemcpy2DAsync(U, static_cast<size_t>(ldu) * 4, U_dev, static_cast<size_t>(c.rows) * 4, static_cast<size_t>(c.rows) * 4,
@@ -464,7 +520,7 @@ extern "C" int sfb_export_factors(sfb_ctx* ctx, int32_t worker, float* U_out_dev
   if (!(ctx->committed & (1ull << worker))) return SFB_ERR_STATE;
   const int64_t off = static_cast<int64_t>(worker) * c.batch;
   if (c.precision == SFB_PREC_BF16 && c.model == SFB_MLR) return tc_export_factors(ctx, off, c.batch, U_out_dev, V_out_dev);
-  const int64_t ldu = c.precision == SFB_PREC_FP32 ? c.rows : ctx->lay.ldu;
+  const int64_t ldu = ctx->lay.ldu;
   CK(cudaMemcpy2DAsync(U_out_dev, static_cast<size_t>(c.rows) * 4, ctx->at<float>(ctx->lay.U) + off * ldu,
                        static_cast<size_t>(ldu) * 4, static_cast<size_t>(c.rows) * 4, static_cast<size_t>(c.batch),
                        cudaMemcpyDeviceToDevice, ctx->stream));
@@ -577,13 +633,14 @@ extern "C" int sfb_sdca_compute_factors(sfb_ctx* ctx, int32_t worker, const floa
     if (rc) return rc;
   } else if (c.precision == SFB_PREC_FP32) {
     float* V = ctx->at<float>(ctx->lay.V) + off * c.cols;
-    float* U = ctx->at<float>(ctx->lay.U) + off * c.rows;
+    const int64_t ldu = ctx->lay.ldu;
+    float* U = ctx->at<float>(ctx->lay.U) + off * ldu;
     CK(pack_copy(ctx->stream, V, X_dev, nullptr, n * c.cols));                                        // v = a_i
     EpiArgs e{};
-    e.C = U; e.ldc = c.rows;
-    CK(sgemm(ctx->stream, true, true, EPI_STORE, n, c.rows, c.cols, V, c.cols, ctx->W, c.cols, e));   // z_i = W a_i
+    e.C = U; e.ldc = ldu;
+    CK(sgemm(ctx->stream, true, true, EPI_STORE, n, c.rows, c.cols, V, c.cols, ctx->W, c.cols, e, ctx->K));   // z_i = W a_i
     ctx->stats.flops += 2.0 * n * c.rows * c.cols;
-    CK(sdca_dual_rows(ctx->stream, U, n, c.rows, c.rows, X_dev, c.cols, labels_dev, sample_ids_dev, ctx->dualQ, ctx->dual_n,
+    CK(sdca_dual_rows(ctx->stream, U, n, c.rows, ldu, X_dev, c.cols, labels_dev, sample_ids_dev, ctx->dualQ, ctx->dual_n,
                       inv_lam_n, c.eta, nullptr, loss, status));                                      // u_i = du_i
   } else {
     const int rc = tc_sdca_factors(ctx, off, n, X_dev, labels_dev, sample_ids_dev, inv_lam_n);
@@ -684,8 +741,8 @@ extern "C" int sfb_dense_sync_step(sfb_ctx* ctx, const float* X_dev, const float
     // worker p's dense update matrix, as it would be sent to the server
     EpiArgs e{};
     e.C = p == 0 ? sum : one; e.ldc = c.cols;
-    CK(sgemm(ctx->stream, false, false, EPI_STORE, c.rows, c.cols, c.batch, U + static_cast<int64_t>(p) * c.batch * c.rows,
-             c.rows, V + static_cast<int64_t>(p) * c.batch * c.cols, c.cols, e));
+    CK(sgemm(ctx->stream, false, false, EPI_STORE, c.rows, c.cols, c.batch, U + static_cast<int64_t>(p) * c.batch * ctx->lay.ldu,
+             ctx->lay.ldu, V + static_cast<int64_t>(p) * c.batch * c.cols, c.cols, e));
     if (p > 0) CK(axpy(ctx->stream, sum, one, 1.f, static_cast<int64_t>(mat)));          // server-side aggregation
   }
   CK(axpy(ctx->stream, ctx->W, sum, -c.eta, static_cast<int64_t>(mat)));                 // W <- W - eta * sum_p dW_p
@@ -709,7 +766,7 @@ extern "C" int sfb_get_factors(sfb_ctx* ctx, const void** U_dev, const void** V_
     if (V_dev) *V_dev = ctx->at<float>(ctx->lay.V);
     if (dtype) *dtype = 0;
     if (layout) *layout = 0;
-    if (ldu) *ldu = ctx->cfg.rows;
+    if (ldu) *ldu = ctx->lay.ldu;
     if (ldv) *ldv = ctx->cfg.cols;
     return SFB_OK;
   }

@@ -1,6 +1,8 @@
 // Bandwidth-bound kernels of the SFB step in fp32: factor packing, the row softmax of multiclass logistic
 // regression, the pair residual of distance metric learning, the column-norm prox of sparse coding and the
 // power iteration that estimates the coder's step size.
+#include <algorithm>
+
 #include "sfb_internal.h"
 
 namespace sfb {
@@ -84,11 +86,11 @@ __global__ void axpy_kernel(float* __restrict__ y, const float* __restrict__ x, 
 // (Section 1: u is the prediction vector; Section 2.1: u = d f / d (W a)).  A class id outside [0, rows)
 // sets a status bit and subtracts nothing.  loss = log sum exp z - z_y.
 template <int NTHREADS>
-__global__ void __launch_bounds__(NTHREADS) mlr_softmax_kernel(float* __restrict__ Z, int64_t rows,
+__global__ void __launch_bounds__(NTHREADS) mlr_softmax_kernel(float* __restrict__ Z, int64_t rows, int64_t ldz,
                                                                const int32_t* __restrict__ labels,
                                                                float* __restrict__ loss, uint32_t* status) {
   __shared__ float sh[32];
-  float* z = Z + static_cast<int64_t>(blockIdx.x) * rows;
+  float* z = Z + static_cast<int64_t>(blockIdx.x) * ldz;
   float m = -INFINITY;
   for (int64_t j = threadIdx.x; j < rows; j += NTHREADS) m = fmaxf(m, z[j]);
   m = block_max<NTHREADS>(m, sh);
@@ -315,44 +317,6 @@ __global__ void mean_kernel(const float* __restrict__ v, int64_t n, float* out) 
   if (threadIdx.x == 0) *out = s / static_cast<float>(n);
 }
 
-// Column reductions over W [rows x cols] in a fixed order: block (slab, column group of 128) sums
-// w^2 (MODE 0) or w * yvec[row] (MODE 1) over its row slab into part[slab][col].
-template <int MODE>
-__global__ void __launch_bounds__(kThreads) col_partial_kernel(const float* __restrict__ W, int64_t rows,
-                                                               int64_t cols, const float* __restrict__ yvec,
-                                                               float* __restrict__ part, int64_t slab_rows) {
-  __shared__ float sh[8][128];
-  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-  const int64_t c0 = static_cast<int64_t>(blockIdx.x) * 128 + tx * 4;
-  const int64_t r0 = static_cast<int64_t>(blockIdx.y) * slab_rows;
-  const int64_t r1 = min(rows, r0 + slab_rows);
-  float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-  if (c0 < cols) {                       // cols is a multiple of 4, so a quad is in range as a whole
-    for (int64_t r = r0 + ty; r < r1; r += 8) {
-      const float4 w = *reinterpret_cast<const float4*>(W + r * cols + c0);
-      if (MODE == 0) {
-        acc.x = fmaf(w.x, w.x, acc.x); acc.y = fmaf(w.y, w.y, acc.y);
-        acc.z = fmaf(w.z, w.z, acc.z); acc.w = fmaf(w.w, w.w, acc.w);
-      } else {
-        const float yv = yvec[r];
-        acc.x = fmaf(w.x, yv, acc.x); acc.y = fmaf(w.y, yv, acc.y);
-        acc.z = fmaf(w.z, yv, acc.z); acc.w = fmaf(w.w, yv, acc.w);
-      }
-    }
-  }
-  *reinterpret_cast<float4*>(&sh[ty][tx * 4]) = acc;
-  __syncthreads();
-  if (threadIdx.x < 128) {
-    const int64_t c = static_cast<int64_t>(blockIdx.x) * 128 + threadIdx.x;
-    if (c < cols) {
-      float s = 0.f;
-#pragma unroll
-      for (int k = 0; k < 8; ++k) s += sh[k][threadIdx.x];
-      part[static_cast<int64_t>(blockIdx.y) * cols + c] = s;
-    }
-  }
-}
-
 // Column sums of squares in fp64 (the prox must resolve norms to far better than fp32's 6e-8, because the
 // rescaling multiplies every entry of W while the step's update is ~1e-3 of ||W||).
 __global__ void __launch_bounds__(kThreads) col_sumsq_kernel(const float* __restrict__ W, int64_t rows, int64_t cols,
@@ -416,51 +380,189 @@ __global__ void __launch_bounds__(kThreads) prox_scale_kernel(float* __restrict_
   }
 }
 
-// y = W b : one warp per row.
-__global__ void __launch_bounds__(kThreads) matvec_rows_kernel(const float* __restrict__ W, int64_t rows,
-                                                               int64_t cols, const float* __restrict__ b,
-                                                               float* __restrict__ y) {
-  const int64_t r = static_cast<int64_t>(blockIdx.x) * (kThreads / 32) + (threadIdx.x >> 5);
-  if (r >= rows) return;
-  const int lane = threadIdx.x & 31;
-  float s = 0.f;
-  for (int64_t c = lane * 4; c < cols; c += 128) {
-    const float4 w = *reinterpret_cast<const float4*>(W + r * cols + c);
-    const float4 v = *reinterpret_cast<const float4*>(b + c);
-    s = fmaf(w.x, v.x, s); s = fmaf(w.y, v.y, s); s = fmaf(w.z, v.z, s); s = fmaf(w.w, v.w, s);
+// ---------------------------------------------------------------------------------------------------------
+// Power iteration for the coder's step size: one cooperative kernel runs all iterations, one block per SM, with a barrier
+// over the grid where an iteration needs the others' results (separate launches, three per iteration, cost more than the
+// arithmetic: 640 us against the figure below for a 2,000 x 1,000 dictionary).  Sums are in a fixed order.
+// ---------------------------------------------------------------------------------------------------------
+constexpr int kPiThreads = 512, kPiWarps = kPiThreads / 32;
+constexpr int kPiBlocks = 148;                        // most blocks of the grid (the scratch is sized for it)
+constexpr int kPiSmem = 200 << 10;
+
+struct PowerParams {
+  const float* W;                                     // [rows x cols]; with GRAM the symmetric [cols x cols] W^T W, rows = cols
+  int64_t rows, cols;
+  float* vec;                                         // [2][cols]: the unnormalised vectors of odd and even iterations
+  float* part;                                        // [blocks][cols]: column sums over a block's rows (not GRAM)
+  double* norms;                                      // [3][blocks]
+  unsigned long long* barrier;
+  Scalars* sc;
+  uint32_t* status;
+  int iters;
+  int smem_rows;                                      // GRAM: rows of G a block keeps in shared memory
+};
+
+// All blocks of a cooperative launch.  Gives up after about two seconds (the others then do the same).
+__device__ __forceinline__ bool grid_barrier(unsigned long long* count, uint32_t* status) {
+  __shared__ int ok;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    const unsigned long long n = gridDim.x, old = atomicAdd(count, 1ull), target = (old / n + 1) * n;
+    const long long t0 = clock64();
+    ok = 1;
+    while (*reinterpret_cast<volatile unsigned long long*>(count) < target)
+      if (clock64() - t0 > 4000000000ll) { ok = 0; atomicOr(status, SFB_STATUS_TIMEOUT); break; }
+    __threadfence();
   }
-  s = warp_sum(s);
-  if (lane == 0) y[r] = s;
+  __syncthreads();
+  return ok != 0;
 }
 
-// One block: c = sum of the slab partials; b = c / ||c||.
-__global__ void __launch_bounds__(1024) pi_normalise_kernel(const float* __restrict__ part, int nslabs, int64_t cols,
-                                                            float* __restrict__ b) {
-  __shared__ float sh[32];
-  float ss = 0.f;
-  for (int64_t c = threadIdx.x; c < cols; c += 1024) {
-    float s = 0.f;
-    for (int k = 0; k < nslabs; ++k) s += part[static_cast<int64_t>(k) * cols + c];
-    b[c] = s;
-    ss = fmaf(s, s, ss);
+__device__ __forceinline__ double warp_sum_d(double v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+// sum of v over the block, in every thread
+__device__ __forceinline__ double block_sum_d(double v, double* sh) {
+  v = warp_sum_d(v);
+  __syncthreads();
+  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
+  __syncthreads();
+  double s = 0.;
+  for (int w = 0; w < kPiWarps; ++w) s += sh[w];
+  return s;
+}
+__device__ __forceinline__ float dot4(const float4 a, const float4 b, float s) {
+  return fmaf(a.w, b.w, fmaf(a.z, b.z, fmaf(a.y, b.y, fmaf(a.x, b.x, s))));
+}
+
+// GRAM: v <- G v with one barrier an iteration.  A block keeps its rows of G in shared memory for all iterations if they fit
+// (smem_rows), reads the whole vector and forms its norm itself.  Otherwise v <- W^T (W v): a block takes its rows of W once
+// per iteration for both products and leaves its column sums, which a second phase adds (two barriers).
+template <bool GRAM>
+__global__ void __launch_bounds__(kPiThreads) power_kernel(const PowerParams p) {
+  extern __shared__ __align__(16) float pi_smem[];     // GRAM: [cols] vector, then [smem_rows][cols] rows of G
+  __shared__ double sh[kPiWarps];
+  __shared__ float yrow[kPiWarps];
+  const int t = threadIdx.x, warp = t >> 5, lane = t & 31, nb = gridDim.x, blk = blockIdx.x;
+  const int64_t r0 = p.rows * blk / nb, r1 = p.rows * (blk + 1) / nb;
+  const int quads = static_cast<int>(p.cols / 4);
+  const float start = rsqrtf(static_cast<float>(p.cols));
+  if (GRAM) {
+    float4* vs = reinterpret_cast<float4*>(pi_smem);
+    float4* gs = vs + quads;
+    const int keep = static_cast<int>(r1 - r0 < p.smem_rows ? r1 - r0 : p.smem_rows);
+    for (int q = t; q < keep * quads; q += kPiThreads) gs[q] = reinterpret_cast<const float4*>(p.W + r0 * p.cols)[q];
+    for (int it = 0; it <= p.iters; ++it) {           // the last pass forms v^T G v = ||W v||^2
+      const float4* v4 = reinterpret_cast<const float4*>(p.vec + static_cast<int64_t>(it & 1) * p.cols);
+      float* out = p.vec + static_cast<int64_t>((it + 1) & 1) * p.cols;
+      const bool last = it == p.iters;
+      double ss = 0.;
+      for (int q = t; q < quads; q += kPiThreads) {
+        const float4 v = it == 0 ? make_float4(start, start, start, start) : __ldcg(v4 + q);
+        vs[q] = v;
+        ss += static_cast<double>(dot4(v, v, 0.f));
+      }
+      ss = block_sum_d(ss, sh);                       // also: the vector is in shared memory for everyone
+      const float scale = it == 0 ? 1.f : static_cast<float>(1. / sqrt(ss));
+      double acc = 0.;
+      for (int64_t r = r0 + warp; r < r1; r += kPiWarps) {
+        const int k = static_cast<int>(r - r0);
+        const float4* w4 = k < keep ? gs + static_cast<int64_t>(k) * quads : reinterpret_cast<const float4*>(p.W + r * p.cols);
+        float s0 = 0.f, s1 = 0.f;
+        int q = lane;
+        for (; q + 32 < quads; q += 64) { s0 = dot4(w4[q], vs[q], s0); s1 = dot4(w4[q + 32], vs[q + 32], s1); }
+        if (q < quads) s0 = dot4(w4[q], vs[q], s0);
+        const float y = warp_sum(s0 + s1) * scale;    // (G v)_r for the normalised v
+        if (lane == 0) {
+          if (last) acc += static_cast<double>(y) * static_cast<double>(pi_smem[r] * scale);
+          else out[r] = y;
+        }
+      }
+      if (last) {
+        acc = block_sum_d(acc, sh);
+        if (t == 0) p.norms[blk] = acc;
+      }
+      if (!grid_barrier(p.barrier, p.status)) return;
+    }
+  } else {
+    float scale = 1.f;                                // 1 / ||v|| of the stored vector
+    for (int it = 0; it <= p.iters; ++it) {           // the last pass only forms ||W v||^2
+      const float4* v4 = reinterpret_cast<const float4*>(p.vec + static_cast<int64_t>(it & 1) * p.cols);
+      auto vat = [&](int q) { return it == 0 ? make_float4(start, start, start, start) : __ldcg(v4 + q); };
+      float* out = p.vec + static_cast<int64_t>((it + 1) & 1) * p.cols;
+      const bool last = it == p.iters;
+      double acc = 0.;
+      // rows in groups of one per warp: y_r = W[r] v, then the group's contribution to the column sums
+      float* part = p.part + static_cast<int64_t>(blk) * p.cols;
+      for (int64_t g = r0; g < r1 || g == r0; g += kPiWarps) {
+        const int64_t r = g + warp;
+        float y = 0.f;
+        if (r < r1) {
+          const float4* w4 = reinterpret_cast<const float4*>(p.W + r * p.cols);
+          float s0 = 0.f, s1 = 0.f;
+          int q = lane;
+          for (; q + 32 < quads; q += 64) { s0 = dot4(w4[q], vat(q), s0); s1 = dot4(w4[q + 32], vat(q + 32), s1); }
+          if (q < quads) s0 = dot4(w4[q], vat(q), s0);
+          y = warp_sum(s0 + s1) * scale;
+        }
+        if (last) {
+          if (lane == 0) acc += static_cast<double>(y) * y;
+          continue;
+        }
+        __syncthreads();
+        if (lane == 0) yrow[warp] = y;
+        __syncthreads();
+        const int n = static_cast<int>(r1 - g < kPiWarps ? r1 - g : kPiWarps);
+        for (int q = t; q < quads; q += kPiThreads) {
+          float4 z = g == r0 ? make_float4(0.f, 0.f, 0.f, 0.f) : *reinterpret_cast<float4*>(part + 4 * q);
+          for (int k = 0; k < n; ++k) {
+            const float4 w = *reinterpret_cast<const float4*>(p.W + (g + k) * p.cols + 4 * q);
+            z.x = fmaf(w.x, yrow[k], z.x); z.y = fmaf(w.y, yrow[k], z.y);
+            z.z = fmaf(w.z, yrow[k], z.z); z.w = fmaf(w.w, yrow[k], z.w);
+          }
+          *reinterpret_cast<float4*>(part + 4 * q) = z;
+        }
+      }
+      if (!last) {
+        if (!grid_barrier(p.barrier, p.status)) return;
+        // this block's columns: the sum over the blocks' parts, one warp per quad of columns
+        const int q0 = static_cast<int>(static_cast<int64_t>(quads) * blk / nb), q1 = static_cast<int>(static_cast<int64_t>(quads) * (blk + 1) / nb);
+        for (int q = q0 + warp; q < q1; q += kPiWarps) {
+          float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
+          for (int b = lane; b < nb; b += 32) {
+            const float4 w = __ldcg(reinterpret_cast<const float4*>(p.part + static_cast<int64_t>(b) * p.cols + 4 * q));
+            z.x += w.x; z.y += w.y; z.z += w.z; z.w += w.w;
+          }
+          z.x = warp_sum(z.x); z.y = warp_sum(z.y); z.z = warp_sum(z.z); z.w = warp_sum(z.w);
+          if (lane == 0) {
+            *reinterpret_cast<float4*>(out + 4 * q) = z;
+            acc += static_cast<double>(z.x) * z.x + static_cast<double>(z.y) * z.y + static_cast<double>(z.z) * z.z +
+                   static_cast<double>(z.w) * z.w;
+          }
+        }
+      }
+      acc = block_sum_d(acc, sh);
+      if (t == 0) p.norms[(last ? 0 : 1 + (it & 1)) * kPiBlocks + blk] = acc;
+      if (!grid_barrier(p.barrier, p.status)) return;
+      if (last) break;
+      double s = 0.;
+      for (int b = lane; b < nb; b += 32) s += __ldcg(p.norms + (1 + (it & 1)) * kPiBlocks + b);
+      scale = static_cast<float>(1. / sqrt(warp_sum_d(s)));
+    }
   }
-  ss = block_sum<1024>(ss, sh);
-  const float inv = rsqrtf(ss);
-  for (int64_t c = threadIdx.x; c < cols; c += 1024) b[c] *= inv;
-}
-
-__global__ void __launch_bounds__(1024) pi_init_kernel(float* __restrict__ b, int64_t cols) {
-  const float v = rsqrtf(static_cast<float>(cols));
-  for (int64_t c = threadIdx.x; c < cols; c += 1024) b[c] = v;
-}
-
-// L = ||W b||^2 (Rayleigh quotient of W^T W at the unit vector b).
-__global__ void __launch_bounds__(1024) pi_rayleigh_kernel(const float* __restrict__ y, int64_t rows, Scalars* sc) {
-  __shared__ float sh[32];
-  float ss = 0.f;
-  for (int64_t r = threadIdx.x; r < rows; r += 1024) ss = fmaf(y[r], y[r], ss);
-  ss = block_sum<1024>(ss, sh);
-  if (threadIdx.x == 0) { sc->L = ss; sc->invL = 1.f / ss; }
+  if (blk == 0 && warp == 0) {
+    double s = 0.;
+    for (int b = lane; b < nb; b += 32) s += __ldcg(p.norms + b);
+    s = warp_sum_d(s);
+    if (lane == 0) {
+      const float L = static_cast<float>(s);
+      p.sc->L = L;
+      p.sc->invL = 1.f / L;
+    }
+  }
 }
 
 __global__ void set_L_kernel(Scalars* sc, float L) { sc->L = L; sc->invL = 1.f / L; }
@@ -497,10 +599,10 @@ cudaError_t axpy(cudaStream_t s, float* y, const float* x, float alpha, int64_t 
   return cudaGetLastError();
 }
 
-cudaError_t mlr_softmax_rows(cudaStream_t s, float* Z, int64_t nsamp, int64_t rows, const int32_t* labels,
+cudaError_t mlr_softmax_rows(cudaStream_t s, float* Z, int64_t nsamp, int64_t rows, int64_t ldz, const int32_t* labels,
                              float* loss, uint32_t* status) {
   if (nsamp <= 0) return cudaSuccess;
-  mlr_softmax_kernel<512><<<static_cast<unsigned>(nsamp), 512, 0, s>>>(Z, rows, labels, loss, status);
+  mlr_softmax_kernel<512><<<static_cast<unsigned>(nsamp), 512, 0, s>>>(Z, rows, ldz, labels, loss, status);
   count_launch();
   return cudaGetLastError();
 }
@@ -567,26 +669,38 @@ cudaError_t prox_unit_columns(cudaStream_t s, float* W, int64_t rows, int64_t co
   return cudaGetLastError();
 }
 
-cudaError_t estimate_lipschitz(cudaStream_t s, const float* W, int64_t rows, int64_t cols, float* b, float* y,
-                               float* colpart, Scalars* sc, int iters) {
-  const int64_t sr = slab_rows_for(rows);
-  dim3 cgrid(static_cast<unsigned>((cols + 127) / 128), kProxSlabs);
-  const unsigned rgrid = static_cast<unsigned>((rows + kThreads / 32 - 1) / (kThreads / 32));
-  pi_init_kernel<<<1, 1024, 0, s>>>(b, cols);
+size_t power_scratch_bytes(int64_t cols) {
+  return 1024 + static_cast<size_t>(3) * kPiBlocks * 8 + static_cast<size_t>(cols) * 4 * (2 + kPiBlocks);
+}
+
+cudaError_t estimate_lipschitz(cudaStream_t s, const float* W, const float* G, int64_t rows, int64_t cols, void* scratch,
+                               Scalars* sc, uint32_t* status, int iters) {
+  PowerParams p{};
+  char* base = static_cast<char*>(scratch);
+  p.barrier = reinterpret_cast<unsigned long long*>(base);
+  p.vec = reinterpret_cast<float*>(base + 1024);
+  p.part = p.vec + 2 * cols;
+  p.norms = reinterpret_cast<double*>(p.part + static_cast<int64_t>(kPiBlocks) * cols);
+  p.W = G ? G : W;
+  p.rows = G ? cols : rows;
+  p.cols = cols;
+  p.sc = sc; p.status = status; p.iters = iters;
+  cudaError_t e = cudaMemsetAsync(p.barrier, 0, 8, s);
+  if (e != cudaSuccess) return e;
+  // a row per warp and block: small dictionaries synchronise fewer blocks
+  const int64_t want = (p.rows + kPiWarps - 1) / kPiWarps, most = std::min(sm_count(), kPiBlocks);
+  const int blocks = static_cast<int>(std::max<int64_t>(1, std::min(want, most)));
+  const int64_t row = cols * 4, room = kPiSmem - row;
+  if (G && room < 0) return cudaErrorInvalidValue;    // the vector has to fit: the callers form no Gram matrix that wide
+  p.smem_rows = G ? static_cast<int>(std::min<int64_t>((p.rows + blocks - 1) / blocks, room / row)) : 0;
+  const size_t smem = G ? static_cast<size_t>(row * (1 + p.smem_rows)) : 0;
+  if ((e = allow_smem<power_kernel<true>>(kPiSmem)) != cudaSuccess) return e;
+  void* args[] = {&p};
+  const dim3 grid(static_cast<unsigned>(blocks)), block(kPiThreads);
+  e = G ? cudaLaunchCooperativeKernel(power_kernel<true>, grid, block, args, smem, s)
+        : cudaLaunchCooperativeKernel(power_kernel<false>, grid, block, args, smem, s);
   count_launch();
-  for (int it = 0; it < iters; ++it) {
-    matvec_rows_kernel<<<rgrid, kThreads, 0, s>>>(W, rows, cols, b, y);
-    count_launch();
-    col_partial_kernel<1><<<cgrid, kThreads, 0, s>>>(W, rows, cols, y, colpart, sr);
-    count_launch();
-    pi_normalise_kernel<<<1, 1024, 0, s>>>(colpart, kProxSlabs, cols, b);
-    count_launch();
-  }
-  matvec_rows_kernel<<<rgrid, kThreads, 0, s>>>(W, rows, cols, b, y);
-  count_launch();
-  pi_rayleigh_kernel<<<1, 1024, 0, s>>>(y, rows, sc);
-  count_launch();
-  return cudaGetLastError();
+  return e;
 }
 
 cudaError_t set_lipschitz(cudaStream_t s, Scalars* sc, float L) {

@@ -18,13 +18,60 @@ inline void count_launch(int n = 1) { g_kernel_launches.fetch_add(n, std::memory
 int sm_count();
 
 // ---------------------------------------------------------------------------------------------------------
+// Launches.  A step is a chain of dependent kernels, several of them only microseconds long: each is launched with
+// programmatic stream serialisation, so that its blocks are scheduled and its set-up runs while the kernel before it
+// drains.  Every kernel launched this way calls pdl_wait() before it touches memory (it returns when the kernels before it
+// have completed and their writes are visible) and pdl_launch_dependents() early (the next kernel may then start its own
+// set-up once all blocks of this one are running).
+// ---------------------------------------------------------------------------------------------------------
+#ifdef __CUDACC__
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+template <typename... KArgs, typename... Args>
+cudaError_t launch_kernel(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, int cluster,
+                          const Args&... args) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[2]{};
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = static_cast<unsigned>(cluster);
+  attr[1].val.clusterDim.y = 1;
+  attr[1].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = cluster > 1 ? 2 : 1;
+  count_launch();
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
+}
+
+// The shared-memory opt-in of a kernel, once per device.
+template <auto Kernel>
+cudaError_t allow_smem(int bytes) {
+  static std::atomic<uint64_t> done{0};                // one bit per device ordinal
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  const uint64_t bit = 1ull << (dev & 63);
+  if (done.load(std::memory_order_acquire) & bit) return cudaSuccess;
+  e = cudaFuncSetAttribute(Kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  if (e == cudaSuccess) done.fetch_or(bit, std::memory_order_release);
+  return e;
+}
+#endif
+
+// ---------------------------------------------------------------------------------------------------------
 // Workspace carve-up.  Every offset is a multiple of 1024 bytes so that any sub-buffer can be a TMA base.
 // ---------------------------------------------------------------------------------------------------------
 constexpr size_t kAlign = 1024;
 constexpr int kProxSlabs = 64;        // row slabs of the deterministic column reductions
 
 struct Layout {
-  size_t status, scalars, loss, V, U, colpart, pib, piy, stageX, stageY, stageL;
+  size_t status, scalars, loss, V, U, colpart, stageX, stageY, stageL;
   // bf16 tensor-core mode
   size_t Wb, Xb, VT, ZT, UT, part, Xf, labels, coef, lse;
   // bf16 mode, DML and SC: (hi | lo) bf16 operands of the split products
@@ -32,7 +79,10 @@ struct Layout {
   size_t U2;                          // DML: second partial of z when the forward product splits its contraction
   // sparse factors (MLR, csr_nnz_max > 0): the step's (sample, column, value) triples and their column-major form
   size_t coo_i, coo_c, coo_x, coo_cx, row_beg, row_end, csc_cnt, csc_cur, csc_ptr, csc_tmp, csc_ent;
-  int64_t ldu;                        // row pitch of the fp32 U buffer (rows rounded up to 4 in bf16 mode)
+  // sparse coding: the dictionary's Gram matrix (when the coder iterates on it), W^T x, the codes of odd iterations, and
+  // the scratch of the power iteration
+  size_t G, Bx, V2, pi;
+  int64_t ldu;                        // row pitch of the fp32 U buffer (rows rounded up to 4; rows itself with tf32 pairs)
   int64_t colsp, rowsp;               // cols, rows rounded up to 64
   int64_t Kp;                         // K rounded up to the contraction block of the update product
   int64_t colsb;                      // cols rounded up to the contraction block of the forward product
@@ -40,6 +90,8 @@ struct Layout {
 };
 
 Layout make_layout(const sfb_config& c);
+bool sc_use_gram(const sfb_config& c);
+inline int64_t round_up(int64_t x, int64_t m) { return (x + m - 1) / m * m; }
 
 // fp32 mode runs its products of multiclass logistic regression on the tensor cores (every fp32 value as a pair of
 // tf32 words, three products per term) when asked to, or by itself when the shape is large enough to be worth the
@@ -100,8 +152,11 @@ namespace sfb {
 // ---------------------------------------------------------------------------------------------------------
 // fp32 FMA matrix products:  C (M x N) = sum_k A(m,k) * B(n,k)  followed by an epilogue.
 // A_KC: A(m,k) at A[m*lda + k] (k contiguous), else at A[k*lda + m].  Same for B with n.
+//   EPI_STORE  C = acc                                     EPI_SUB    C = acc - aux
+//   EPI_RMW    C = prox(C + alpha acc)                     EPI_SYM    C = acc for a symmetric result (half of the tiles)
+//   EPI_ISTA   C = soft(cur - (acc - aux) / L, lam / L)    EPI_ISTA0  C = soft(acc / L, lam / L), C2 = acc
 // ---------------------------------------------------------------------------------------------------------
-enum Epilogue { EPI_STORE = 0, EPI_SUB = 1, EPI_RMW = 2, EPI_ISTA = 3 };
+enum Epilogue { EPI_STORE = 0, EPI_SUB = 1, EPI_RMW = 2, EPI_ISTA = 3, EPI_ISTA0 = 4, EPI_SYM = 5 };
 
 // Entry-wise proximal operator fused into the update: kind 1 soft-threshold by a, kind 2 multiply by a.
 __host__ __device__ __forceinline__ float prox_entry(float w, int kind, float a) {
@@ -115,23 +170,34 @@ __host__ __device__ __forceinline__ float prox_entry(float w, int kind, float a)
 struct EpiArgs {
   int32_t prox_kind;   // EPI_RMW: entry-wise prox applied to the updated value (0 none)
   float prox_a;
+  float alpha;         // EPI_RMW
+  float lam;           // EPI_ISTA, EPI_ISTA0
   float* C;            // output, row-major [M x ldc]
   int64_t ldc;
-  const float* aux;    // EPI_SUB: the matrix subtracted, same shape and ld as C
-  float alpha;         // EPI_RMW: C += alpha * acc
-  const Scalars* sc;   // EPI_ISTA: reads invL
-  float lam;           // EPI_ISTA: C = soft(C - acc*invL, lam*invL)
+  float* C2;           // EPI_ISTA0 (may be null)
+  int64_t ldc2;
+  const float* aux;    // EPI_SUB, EPI_ISTA (there: may be null)
+  int64_t ldaux;
+  const float* cur;    // EPI_ISTA
+  int64_t ldcur;
+  const Scalars* sc;   // EPI_ISTA, EPI_ISTA0: reads invL
 };
 
+struct GemmShape { int tile, split; };               // tile edge; parts the contraction is cut into
+double gemm_cost(int tile, int split, int64_t M, int64_t N, int64_t Kc, bool sym);
+GemmShape pick_gemm_shape(int64_t M, int64_t N, int64_t Kc, bool sym = false);
+
+// M_split (0: M): the row count that decides how the contraction is split; callers that compute a product in slices of
+// rows pass the whole product's, so that a row has the same bits whichever slice it is computed in.
 cudaError_t sgemm(cudaStream_t s, bool a_kc, bool b_kc, Epilogue epi, int64_t M, int64_t N, int64_t Kc,
-                  const float* A, int64_t lda, const float* B, int64_t ldb, const EpiArgs& e);
+                  const float* A, int64_t lda, const float* B, int64_t ldb, const EpiArgs& e, int64_t M_split = 0);
 
 // ---------------------------------------------------------------------------------------------------------
 // Factor kernels (pack, softmax, pair residual, prox, power iteration)
 // ---------------------------------------------------------------------------------------------------------
 cudaError_t pack_copy(cudaStream_t s, float* dst, const float* x, const float* y_or_null, int64_t n);
 cudaError_t fill_zero(cudaStream_t s, float* dst, int64_t n);
-cudaError_t mlr_softmax_rows(cudaStream_t s, float* Z, int64_t nsamp, int64_t rows, const int32_t* labels,
+cudaError_t mlr_softmax_rows(cudaStream_t s, float* Z, int64_t nsamp, int64_t rows, int64_t ldz, const int32_t* labels,
                              float* loss_per_sample, uint32_t* status);
 // Row-sharded MLR: per-sample softmax partials (max, sum exp, label logit, owner flag) of a shard, and the finish with
 // the partials of all shards ([shards][nsamp] float4).
@@ -153,8 +219,11 @@ cudaError_t dml_scale_rows(cudaStream_t s, float* Z, int64_t nsamp, int64_t rows
                            const float* norms_all = nullptr, int shards = 0, int64_t nstride = 0);
 cudaError_t mean_of(cudaStream_t s, const float* v, int64_t n, float* out);
 cudaError_t prox_unit_columns(cudaStream_t s, float* W, int64_t rows, int64_t cols, float* colpart);
-cudaError_t estimate_lipschitz(cudaStream_t s, const float* W, int64_t rows, int64_t cols, float* b, float* y,
-                               float* colpart, Scalars* sc, int iters);
+// L = ||W||_2^2 by power iterations from the normalised all-ones vector, on W^T W itself when G is given, else on W.
+// scratch: power_scratch_bytes(cols).
+cudaError_t estimate_lipschitz(cudaStream_t s, const float* W, const float* G, int64_t rows, int64_t cols, void* scratch,
+                               Scalars* sc, uint32_t* status, int iters);
+size_t power_scratch_bytes(int64_t cols);
 cudaError_t set_lipschitz(cudaStream_t s, Scalars* sc, float L);
 cudaError_t axpy(cudaStream_t s, float* y, const float* x, float alpha, int64_t n);  // y += alpha*x
 cudaError_t prox_entries(cudaStream_t s, float* w, int64_t n, int kind, float a);      // w <- prox(w), entry-wise

@@ -676,7 +676,7 @@ int sparse_update(sfb_ctx* ctx) {
     p.copy_counters = &ctx->at<Scalars>(L.scalars)->copy_pieces;
     CKS((launch_sparse_update<1, 1>(ctx->stream, p, smem)));
   } else {
-    p.U = ctx->at<float>(L.U); p.ldu = c.rows;
+    p.U = ctx->at<float>(L.U); p.ldu = L.ldu;
     if (ctx->tf32) {
       p.shadow32 = ctx->at<float>(L.Ws); p.shadow32_ld = 2 * L.colsp; p.shadow_half = L.colsp;
       CKS((launch_sparse_update<0, 2>(ctx->stream, p, smem)));

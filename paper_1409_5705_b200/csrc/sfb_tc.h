@@ -48,8 +48,6 @@ struct TcState {
   int max_pairs;             // CTA pairs (clusters of 2) of the update kernel that can be resident at once
 };
 
-inline int64_t round_up(int64_t x, int64_t m) { return (x + m - 1) / m * m; }
-
 // 2-D row-major tensor [outer x inner] with row pitch `pitch_bytes`, box [box_outer x box_inner], 128-byte swizzle.
 inline bool make_map(const TcState* st, CUtensorMap* m, CUtensorMapDataType dt, void* base, int64_t inner,
                      int64_t outer, int64_t pitch_bytes, int box_inner, int box_outer) {
