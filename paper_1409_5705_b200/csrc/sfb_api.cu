@@ -26,14 +26,19 @@ int sm_count() {
 static size_t up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
 
 // The coder's iterations a <- soft(a - W^T (W a - x) / L) either take two products with W each, or one with the Gram matrix
-// W^T W, formed once per step (half of it: it is symmetric), and W^T x.  The Gram form wins when the dictionary has at most
-// about twice as many atoms as features and the mini-batch is large enough to repay W^T W; decided by the cost of the
-// products themselves.
+// W^T W, formed once per step (half of it: it is symmetric), and W^T x.  The Gram form wins when the mini-batch is large enough
+// to repay W^T W; decided by the cost of the products themselves (10,000 x 5,000, K = 512, 20 iterations, bf16: 5.0 -> 2.2 ms
+// for the coder; error of the codes 2.9e-5, with two products 1.1e-4 while they had one accumulator).  In bf16 mode it is kept
+// to dictionaries with no more atoms than features: the residual of an overcomplete one becomes small against x, and the
+// two-product form then rounds relative to it where W^T W a - W^T x rounds relative to W^T x (500 x 1,400: 4.8e-6 against
+// 1.2e-5).
 bool sc_use_gram(const sfb_config& c) {
   const int64_t K = static_cast<int64_t>(c.workers) * c.batch, D = c.rows, A = c.cols;
   const double it = c.sc_ista_iters - 1;
-  if (it < 1 || A > (32 << 10)) return false;        // (the power iteration keeps a vector of A values on chip)
-  auto cost = [](int64_t M, int64_t N, int64_t Kc, bool sym) {
+  if (it < 1 || (c.precision == SFB_PREC_BF16 && A > D)) return false;
+  if (A > (32 << 10)) return false;        // (the power iteration keeps a vector of A values on chip)
+  auto cost = [&](int64_t M, int64_t N, int64_t Kc, bool sym) {
+    if (c.precision == SFB_PREC_BF16) return split_product_cost(M, N, Kc, sym);
     const GemmShape g = pick_gemm_shape(M, N, Kc, sym);
     return std::min(gemm_cost(128, g.split, M, N, Kc, sym), gemm_cost(64, g.split, M, N, Kc, sym));
   };
@@ -161,6 +166,7 @@ extern "C" int sfb_init(const sfb_config* cfg, float* W_dev, void* workspace_dev
   ctx->K = static_cast<int64_t>(cfg->workers) * cfg->batch;
   ctx->in_dim = cfg->model == SFB_SC ? cfg->rows : cfg->cols;
   ctx->committed = 0;
+  ctx->begun = false;
   ctx->sparse_mask = 0;
   ctx->csr_fill = 0;
   ctx->sparse_v = false;
@@ -269,6 +275,10 @@ static int factors_fp32(sfb_ctx* ctx, int64_t off, int64_t n, const float* X, co
 // the coder's Gram matrix and its step size.
 static int begin_step(sfb_ctx* ctx) {
   const sfb_config& c = ctx->cfg;
+  if (c.precision == SFB_PREC_BF16) {
+    const int rc = tc_begin_step(ctx);
+    if (rc) return rc;
+  }
   if (c.model != SFB_SC) return SFB_OK;
   float* G = ctx->lay.G ? ctx->at<float>(ctx->lay.G) : nullptr;
   if (c.precision == SFB_PREC_FP32 && G) {
@@ -316,7 +326,11 @@ extern "C" int sfb_compute_factors(sfb_ctx* ctx, int32_t worker, const float* X_
     ctx->sparse_mask = 0;
     ctx->csr_fill = 0;
     CK(cudaEventRecord(ctx->ev[0], ctx->stream));
+    ctx->begun = false;
+  }
+  if (!ctx->begun) {
     if ((rc = begin_step(ctx)) != SFB_OK) return rc;
+    ctx->begun = true;
   }
   // bf16 mode: every product runs on the tensor cores; DML and SC, whose u comes from a cancelling residual,
   // carry each value as a (hi, lo) pair of bf16 (fp32-class products)
@@ -444,6 +458,7 @@ extern "C" int sfb_forward_partials_pairs(sfb_ctx* ctx, const float* X_dev, cons
   // the flags are kept for the finish (the caller's buffer may change before it)
   CK(cudaMemcpyAsync(ctx->at<int32_t>(ctx->lay.stageL), similar_dev, static_cast<size_t>(ctx->K) * 4, cudaMemcpyDeviceToDevice,
                      ctx->stream));
+  if ((rc = begin_step(ctx)) != SFB_OK) return rc;
   rc = c.precision == SFB_PREC_FP32 ? factors_fp32(ctx, 0, ctx->K, X_dev, Y_dev, similar_dev, false, partials_dev)
                                     : tc_factors(ctx, 0, ctx->K, X_dev, Y_dev, similar_dev, partials_dev);
   if (rc) return rc;
@@ -592,6 +607,7 @@ extern "C" int sfb_apply_update(sfb_ctx* ctx) {
   if (rc) return rc;
   CK(cudaEventRecord(ctx->ev[3], ctx->stream));
   ctx->committed = 0;
+  ctx->begun = false;
   ctx->sparse_mask = 0;               // the next step starts with no sparse samples staged
   ctx->csr_fill = 0;
   ctx->gathered = false;
@@ -752,6 +768,7 @@ extern "C" int sfb_dense_sync_step(sfb_ctx* ctx, const float* X_dev, const float
   if (rc) return rc;
   CK(cudaEventRecord(ctx->ev[3], ctx->stream));
   ctx->committed = 0;
+  ctx->begun = false;
   ctx->gathered = false;
   ctx->stats.steps += 1;
   ctx->stats.samples += ctx->K;

@@ -81,7 +81,7 @@ struct Layout {
   size_t coo_i, coo_c, coo_x, coo_cx, row_beg, row_end, csc_cnt, csc_cur, csc_ptr, csc_tmp, csc_ent;
   // sparse coding: the dictionary's Gram matrix (when the coder iterates on it), W^T x, the codes of odd iterations, and
   // the scratch of the power iteration
-  size_t G, Bx, V2, pi;
+  size_t G, Gs, Bx, V2, As2, pi;
   int64_t ldu;                        // row pitch of the fp32 U buffer (rows rounded up to 4; rows itself with tf32 pairs)
   int64_t colsp, rowsp;               // cols, rows rounded up to 64
   int64_t Kp;                         // K rounded up to the contraction block of the update product
@@ -133,6 +133,7 @@ struct sfb_ctx {
   int32_t prox_kind;                  // entry-wise prox of the update pass and its parameter (threshold or factor)
   float prox_a;
   uint64_t committed;                 // bit p set: worker p has written its factors since the last update
+  bool begun;                         // what the workers' factors of this step share has been derived from W
   uint64_t sparse_mask;               // bit p set: worker p's samples of this step came in compressed-sparse-row form
   int64_t csr_fill;                   // triples staged so far in this step
   int64_t last_stage_nnz;             // entries of the last staged block of samples

@@ -44,7 +44,13 @@ constexpr int kSmem = S * (kBytesA + kBytesB) + kEpiWarps * R * kSlotBytes + kBa
 //   F_STORE    store D as fp32                                                                     (DML: z = W v)
 //   F_SUB      store D - aux as fp32 and as a (hi | lo) bf16 pair                                  (SC: r = W a - x)
 //   F_ISTA     C <- soft(C - D / L, lambda / L) in place, also as a (hi | lo) bf16 pair            (SC: ISTA step)
-enum FwdEpi { F_SOFTMAX = 0, F_STORE = 1, F_SUB = 2, F_ISTA = 3 };
+//   F_ISTAG    C <- soft(C - (D - C2) / L, lambda / L) in place, also as a pair                     (SC: on W^T W)
+//   F_ISTA0    C2 = D and C = soft(D / L, lambda / L), also as a pair                               (SC: first iterate)
+//   F_GRAM     C (unless null) = D and D as a pair, of a symmetric D: only the tiles that reach the diagonal or lie above
+//              it are formed, the others are written as their mirror images                          (SC: W^T W)
+enum FwdEpi { F_SOFTMAX = 0, F_STORE = 1, F_SUB = 2, F_ISTA = 3, F_ISTAG = 4, F_ISTA0 = 5, F_GRAM = 6 };
+template <int EPI>
+constexpr bool kIsta = EPI == F_ISTA || EPI == F_ISTAG || EPI == F_ISTA0;
 
 struct TcParams {
   int32_t M, N, Kc;            // extents of the product: samples, output columns, contraction
@@ -60,14 +66,16 @@ struct TcParams {
   int32_t a_off0, a_off1, a_off2, b_off0, b_off1, b_off2;
   float2* part;                // F_SOFTMAX: [tilesN][part_ld] (max, sum exp) per sample and 256-row block
   int64_t part_ld;
-  const float* aux;            // F_SUB: the matrix subtracted, [M x ldaux]; F_ISTA: the matrix updated, [M x ldaux]
+  const float* aux;            // F_SUB: the matrix subtracted, [M x ldaux]; F_ISTA, F_ISTAG: the matrix updated
   int64_t ldaux;
+  float* C2;                   // F_ISTA0 (may be null), F_ISTAG: W^T x, [M x ldc]
   int32_t prefetch;            // k-blocks by which the producer asks L2 for the B operand ahead of its loads (0: off)
   int32_t ksplit;              // forward_split_kernel, F_STORE: the contraction is cut into this many parts, each a work
   int64_t c_split_stride;      //   unit of its own writing its partial product to C + part * c_split_stride (else 1, 0)
-  const Scalars* sc;           // F_ISTA: 1 / L
-  float lam;                   // F_ISTA: lambda
-  __nv_bfloat16* split;        // F_SUB, F_ISTA: [M x ld_split] receives hi at column n and lo at column split_half + n
+  int32_t four;                // F_GRAM: with the fourth term A_lo B_lo
+  const Scalars* sc;           // F_ISTA*: 1 / L
+  float lam;                   // F_ISTA*: lambda
+  __nv_bfloat16* split;        // all but F_STORE: [M x ld_split] receives hi at column n and lo at column split_half + n
   int64_t ld_split;
   int32_t split_half;          // padded N (a multiple of 64); columns N..split_half-1 are written as zeros
   uint32_t* status;
@@ -78,6 +86,26 @@ struct TcParams {
 __device__ __forceinline__ void tile_coords(const TcParams& p, int tile, int& m0, int& n0) {
   const int tm = tile % p.tilesM, tn = tile / p.tilesM;
   m0 = p.m_off + tm * BM;
+  n0 = tn * p.bn;
+}
+
+// F_GRAM: the tiles of column block tn that are formed are row blocks 0 .. sym_row_blocks - 1 (those that begin above the
+// column block's end); numbered column block by column block.
+__host__ __device__ __forceinline__ int sym_row_blocks(int tilesM, int bn, int tn) {
+  const int n = ((tn + 1) * bn - 1) / BM + 1;
+  return n < tilesM ? n : tilesM;
+}
+__host__ __device__ __forceinline__ int sym_tiles(int tilesM, int tilesN, int bn) {
+  int n = 0;
+  for (int tn = 0; tn < tilesN; ++tn) n += sym_row_blocks(tilesM, bn, tn);
+  return n;
+}
+template <int EPI>
+__device__ __forceinline__ void split_tile_coords(const TcParams& p, int tile, int& m0, int& n0) {
+  if (EPI != F_GRAM) return tile_coords(p, tile, m0, n0);
+  int tn = 0;
+  for (int n; tile >= (n = sym_row_blocks(p.tilesM, p.bn, tn)); ++tn) tile -= n;
+  m0 = tile * BM;
   n0 = tn * p.bn;
 }
 
@@ -259,7 +287,9 @@ forward_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
 // k-block are issued from it: 72 KB of operands per three k-blocks of tensor work instead of 108 KB when the three
 // products run as separate passes over the contraction (these products are bound by their operand loads: a 128 x 160
 // tile takes 36 KB per 320 cycles of MMA).  Three stages of 72 KB fill the shared memory, so the epilogue writes its
-// results straight from registers (the outputs are small: samples x N).
+// results straight from registers (the outputs are small: samples x N).  The cross terms have an accumulator of their own: the
+// tensor core rounds an fp32 accumulator at every instruction relative to what it holds, so two thirds of the roundings happen
+// at a 2^-8 of the size.
 // Roles as in forward_kernel: warp 0 TMA producer, warp 1 MMA issuer and TMEM owner, warps 2-5 epilogue.
 // ---------------------------------------------------------------------------------------------------------
 constexpr int FS_BN = 160;                          // widest tile of this kernel (columns of the accumulator)
@@ -285,8 +315,11 @@ forward_split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int S = p.ksplit > 1 ? p.ksplit : 1;
-  const int ntiles = p.tilesM * p.tilesN * S;       // work units: (tile, part of the contraction), parts of a tile adjacent
+  const int ntiles = (EPI == F_GRAM ? sym_tiles(p.tilesM, p.tilesN, p.bn) : p.tilesM * p.tilesN) * S;   // work units: (tile, part of the contraction), parts of a tile adjacent
   const int numKall = p.kseg;                       // k-blocks of the contraction (each serves three products)
+  // Two accumulators per tile: A_hi B_hi, and the cross terms at column `cross` of it.  Tiles of at most 128 columns have room
+  // for two such pairs (the epilogue of one tile then overlaps the products of the next), wider ones for one.
+  const int nacc = p.bn <= 128 ? 2 : 1, cross = p.bn <= 128 ? 128 : 256;
   const int a_hi = p.a_off0, a_lo = p.a_off2, b_hi = p.b_off0, b_lo = p.b_off1;
 
   if (threadIdx.x == 0) {
@@ -311,7 +344,7 @@ forward_split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
       bool ok = true;
       for (int tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x) {
         int m0, n0;
-        tile_coords(p, tile / S, m0, n0);
+        split_tile_coords<EPI>(p, tile / S, m0, n0);
         const int part = tile % S, kbeg = part * numKall / S, numK = (part + 1) * numKall / S;
         for (int kl = kbeg; kl < numK; ++kl, ++it) {
           const uint32_t s = it % FS_STAGES, ph = (it / FS_STAGES) & 1;
@@ -336,10 +369,10 @@ forward_split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
       uint32_t it = 0, tl = 0;
       bool ok = true;
       for (int tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x, ++tl) {
-        const uint32_t a = tl & 1, aph = (tl >> 1) & 1;
+        const uint32_t a = tl % nacc, aph = (tl / nacc) & 1;
         if (!mbar_wait(&tempty[a], aph ^ 1, abort_flag)) { ok = false; break; }
         tc_fence_after();
-        const uint32_t d_tmem = tmem_base + a * BN;
+        const uint32_t d_tmem = tmem_base + a * BN, d_cross = d_tmem + cross;
         const int part = tile % S, numK = (part + 1) * numKall / S - part * numKall / S;
         for (int kb = 0; kb < numK; ++kb, ++it) {
           const uint32_t s = it % FS_STAGES, ph = (it / FS_STAGES) & 1;
@@ -353,9 +386,11 @@ forward_split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
 #pragma unroll
           for (int k = 0; k < BK / UMMA_K; ++k) {
             const uint64_t adv = static_cast<uint64_t>(k * UMMA_K * 2 / 16);
-            umma_bf16(d_tmem, dal + adv, dbh + adv, idesc, (kb | k) != 0 ? 1u : 0u);     // A_lo B_hi
-            umma_bf16(d_tmem, dah + adv, dbl + adv, idesc, 1u);                          // A_hi B_lo
-            umma_bf16(d_tmem, dah + adv, dbh + adv, idesc, 1u);                          // A_hi B_hi
+            const uint32_t more = (kb | k) != 0 ? 1u : 0u;
+            umma_bf16(d_cross, dal + adv, dbh + adv, idesc, more);                       // A_lo B_hi
+            umma_bf16(d_cross, dah + adv, dbl + adv, idesc, 1u);                         // A_hi B_lo
+            if (EPI == F_GRAM && p.four) umma_bf16(d_cross, dal + adv, dbl + adv, idesc, 1u);    // A_lo B_lo
+            umma_bf16(d_tmem, dah + adv, dbh + adv, idesc, more);                        // A_hi B_hi
           }
           umma_commit(&empty[s]);
         }
@@ -368,13 +403,13 @@ forward_split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
     const int my_tiles = blockIdx.x < ntiles ? (ntiles - 1 - blockIdx.x) / gridDim.x + 1 : 0;
     bool ok = true;
     float invL = 0.f, thr = 0.f;
-    if (EPI == F_ISTA) { invL = p.sc->invL; thr = p.lam * invL; }
+    if (kIsta<EPI>) { invL = p.sc->invL; thr = p.lam * invL; }
     for (int tl = 0; tl < my_tiles && ok; ++tl) {
       int m0, n0;
       const int unit = blockIdx.x + tl * gridDim.x;
-      tile_coords(p, unit / S, m0, n0);
+      split_tile_coords<EPI>(p, unit / S, m0, n0);
       float* Cp = C + static_cast<int64_t>(unit % S) * p.c_split_stride;
-      const uint32_t a = tl & 1, aph = (tl >> 1) & 1;
+      const uint32_t a = tl % nacc, aph = (tl / nacc) & 1;
       if (!__all_sync(0xffffffffu, mbar_wait(&tfull[a], aph, abort_flag))) { ok = false; break; }
       tc_fence_after();
       const int row = m0 + q * 32 + lane;
@@ -382,31 +417,62 @@ forward_split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
       const int nlim = min(p.N, n0 + p.bn);
       for (int c = 0; c < (p.bn + kChunk - 1) / kChunk; ++c) {
         uint32_t acc[32];
-        tmem_ld_32x32(tmem_base + (static_cast<uint32_t>(q * 32) << 16) + a * BN + c * kChunk, acc);
-        tmem_ld_wait();
+        {
+          uint32_t small[32];
+          const uint32_t at = tmem_base + (static_cast<uint32_t>(q * 32) << 16) + a * BN + c * kChunk;
+          tmem_ld_32x32(at, acc);
+          tmem_ld_32x32(at + cross, small);
+          tmem_ld_wait();
+#pragma unroll
+          for (int j = 0; j < 32; ++j) acc[j] = __float_as_uint(__uint_as_float(acc[j]) + __uint_as_float(small[j]));
+        }
         const int col0 = n0 + c * kChunk;
         if (col0 >= nlim || row >= p.M) continue;
-        if constexpr (EPI == F_SUB || EPI == F_ISTA) {
-          // the sample's values of aux (x, or the current code a) are contiguous: up to 128 bytes per lane
-          float xv[32];
-          const float* ap = p.aux + static_cast<int64_t>(row) * p.ldaux + col0;
-          const bool ap16 = (reinterpret_cast<uintptr_t>(ap) & 15u) == 0;
+        if constexpr (EPI == F_ISTAG || EPI == F_ISTA0) {
+          // W^T x of the sample (N, hence every pitch, is a multiple of 4 for the products over atoms)
+          float* bp = p.C2 ? p.C2 + static_cast<int64_t>(row) * ldc + col0 : nullptr;
 #pragma unroll
           for (int j = 0; j < 8; ++j) {
-            if (ap16 && col0 + 4 * j + 4 <= nlim) {
-              const float4 v4 = *reinterpret_cast<const float4*>(ap + 4 * j);
-              xv[4 * j] = v4.x; xv[4 * j + 1] = v4.y; xv[4 * j + 2] = v4.z; xv[4 * j + 3] = v4.w;
+            if (!bp || col0 + 4 * j + 4 > nlim) continue;
+            if constexpr (EPI == F_ISTAG) {
+              const float4 b4 = *reinterpret_cast<const float4*>(bp + 4 * j);
+              acc[4 * j] = __float_as_uint(__uint_as_float(acc[4 * j]) - b4.x);
+              acc[4 * j + 1] = __float_as_uint(__uint_as_float(acc[4 * j + 1]) - b4.y);
+              acc[4 * j + 2] = __float_as_uint(__uint_as_float(acc[4 * j + 2]) - b4.z);
+              acc[4 * j + 3] = __float_as_uint(__uint_as_float(acc[4 * j + 3]) - b4.w);
             } else {
-#pragma unroll
-              for (int e = 0; e < 4; ++e) xv[4 * j + e] = col0 + 4 * j + e < nlim ? ap[4 * j + e] : 0.f;
+              *reinterpret_cast<uint4*>(bp + 4 * j) = make_uint4(acc[4 * j], acc[4 * j + 1], acc[4 * j + 2], acc[4 * j + 3]);
             }
           }
+        }
+        if constexpr (EPI != F_STORE) {
+          if constexpr (EPI == F_SUB || EPI == F_ISTA || EPI == F_ISTAG) {
+            // the sample's values of aux (x, or the current code a) are contiguous: up to 128 bytes per lane
+            float xv[32];
+            const float* ap = p.aux + static_cast<int64_t>(row) * p.ldaux + col0;
+            const bool ap16 = (reinterpret_cast<uintptr_t>(ap) & 15u) == 0;
 #pragma unroll
-          for (int j = 0; j < 32; ++j) {
-            const float d = __uint_as_float(acc[j]);
-            const float v = EPI == F_SUB ? d - xv[j] : soft_threshold(fmaf(-d, invL, xv[j]), thr);
-            acc[j] = __float_as_uint(col0 + j < p.N ? v : 0.f);
+            for (int j = 0; j < 8; ++j) {
+              if (ap16 && col0 + 4 * j + 4 <= nlim) {
+                const float4 v4 = *reinterpret_cast<const float4*>(ap + 4 * j);
+                xv[4 * j] = v4.x; xv[4 * j + 1] = v4.y; xv[4 * j + 2] = v4.z; xv[4 * j + 3] = v4.w;
+              } else {
+#pragma unroll
+                for (int e = 0; e < 4; ++e) xv[4 * j + e] = col0 + 4 * j + e < nlim ? ap[4 * j + e] : 0.f;
+              }
+            }
+#pragma unroll
+            for (int j = 0; j < 32; ++j) {
+              const float d = __uint_as_float(acc[j]);
+              acc[j] = __float_as_uint(EPI == F_SUB ? d - xv[j] : soft_threshold(fmaf(-d, invL, xv[j]), thr));
+            }
           }
+          if constexpr (EPI == F_ISTA0) {
+#pragma unroll
+            for (int j = 0; j < 32; ++j) acc[j] = __float_as_uint(soft_threshold(__uint_as_float(acc[j]) * invL, thr));
+          }
+#pragma unroll
+          for (int j = 0; j < 32; ++j) acc[j] = col0 + j < p.N ? acc[j] : 0u;
           // (hi | lo) bf16 pair of the result: the operand of the next product (zero in the padding past N; the
           // columns past this tile's width belong to the next tile)
           __nv_bfloat16* hp = p.split + static_cast<int64_t>(row) * p.ld_split + col0;
@@ -428,6 +494,22 @@ forward_split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
               *reinterpret_cast<uint4*>(hp + p.split_half + 8 * j) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
             }
           }
+        }
+        if constexpr (EPI == F_GRAM) {
+          // the mirror images of the entries whose own tile is not formed: lanes are neighbouring columns there
+          const int own_end = (row / p.bn + 1) * p.bn;              // end of the column block that row lies in
+#pragma unroll
+          for (int j = 0; j < 32; ++j) {
+            const int n = col0 + j;
+            if (n >= nlim || own_end > n / BM * BM) continue;
+            const float f = __uint_as_float(acc[j]);
+            const __nv_bfloat16 hi = __float2bfloat16_rn(f);
+            __nv_bfloat16* hp = p.split + static_cast<int64_t>(n) * p.ld_split + row;
+            hp[0] = hi;
+            hp[p.split_half] = __float2bfloat16_rn(f - __bfloat162float(hi));
+            if (C) C[static_cast<int64_t>(n) * ldc + row] = f;
+          }
+          if (!C) continue;
         }
         // the fp32 result: this lane's consecutive columns of its row
         float* cp = Cp + static_cast<int64_t>(row) * ldc + col0;
@@ -574,14 +656,24 @@ __global__ void __launch_bounds__(256) pack_split_t_kernel(const float* __restri
 
 // fp32 [n x dim] (row pitch ld) -> the (hi | lo) bf16 operand [n x 2*dimp], no transpose: dst[r][c] = hi,
 // dst[r][dimp + c] = lo with hi = bf16(f), lo = bf16(f - hi).  Columns dim..dimp-1 are left as they are (zero since
-// set-up).  dim and ld are multiples of 4.
+// set-up).
 __global__ void __launch_bounds__(256) pack_split_rows_kernel(const float* __restrict__ F, int64_t n, int64_t dim,
                                                               int64_t ld, __nv_bfloat16* __restrict__ dst, int64_t dimp) {
-  const int64_t quads = dim / 4, total = n * quads;
+  const int64_t quads = (dim + 3) / 4, total = n * quads;
   const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
+  const bool vec = ld % 4 == 0 && dim % 4 == 0;          // else (samples with an odd number of features) value by value
   for (int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; i < total; i += stride) {
     const int64_t r = i / quads, qd = i % quads;
-    const float4 v = *reinterpret_cast<const float4*>(F + r * ld + qd * 4);
+    const float* src = F + r * ld + qd * 4;
+    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (vec) {
+      v = *reinterpret_cast<const float4*>(src);
+    } else {
+      v.x = src[0];
+      if (qd * 4 + 1 < dim) v.y = src[1];
+      if (qd * 4 + 2 < dim) v.z = src[2];
+      if (qd * 4 + 3 < dim) v.w = src[3];
+    }
     const __nv_bfloat16 h0 = __float2bfloat16_rn(v.x), h1 = __float2bfloat16_rn(v.y), h2 = __float2bfloat16_rn(v.z),
                         h3 = __float2bfloat16_rn(v.w);
     __nv_bfloat16* d = dst + r * 2 * dimp + qd * 4;
@@ -834,7 +926,8 @@ cudaError_t launch_forward(sfb_ctx* ctx, const CUtensorMap& a, const CUtensorMap
 template <int EPI>
 cudaError_t launch_forward_split(sfb_ctx* ctx, const CUtensorMap& a, const CUtensorMap& b, float* C, int64_t ldc, TcParams p) {
   const TcState* st = static_cast<const TcState*>(ctx->tc);
-  const int64_t tiles = static_cast<int64_t>(p.tilesM) * p.tilesN * (p.ksplit > 1 ? p.ksplit : 1);
+  const int64_t tiles = EPI == F_GRAM ? sym_tiles(p.tilesM, p.tilesN, p.bn)
+                                      : static_cast<int64_t>(p.tilesM) * p.tilesN * (p.ksplit > 1 ? p.ksplit : 1);
   if (tiles <= 0) return cudaSuccess;
   const int grid = static_cast<int>(tiles < st->sms ? tiles : st->sms);
   forward_split_kernel<EPI><<<grid, kThreads, kFsSmem, ctx->stream>>>(a, b, C, ldc, p);
@@ -849,6 +942,9 @@ cudaError_t prepare_forward_kernels() {
   if (e == cudaSuccess) e = cudaFuncSetAttribute(forward_split_kernel<F_STORE>, cudaFuncAttributeMaxDynamicSharedMemorySize, kFsSmem);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(forward_split_kernel<F_SUB>, cudaFuncAttributeMaxDynamicSharedMemorySize, kFsSmem);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(forward_split_kernel<F_ISTA>, cudaFuncAttributeMaxDynamicSharedMemorySize, kFsSmem);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(forward_split_kernel<F_ISTAG>, cudaFuncAttributeMaxDynamicSharedMemorySize, kFsSmem);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(forward_split_kernel<F_ISTA0>, cudaFuncAttributeMaxDynamicSharedMemorySize, kFsSmem);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(forward_split_kernel<F_GRAM>, cudaFuncAttributeMaxDynamicSharedMemorySize, kFsSmem);
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(forward_kernel<F_SOFTMAX, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
   return e;
@@ -907,7 +1003,13 @@ void tc_extend_layout(const sfb_config& c, Layout& L, size_t& off) {
     L.As = take(K * 2 * static_cast<size_t>(L.colsp) * 2);              // v (DML) or the codes a (SC)
     if (c.model == SFB_SC) {
       L.WTs = take(static_cast<size_t>(c.cols) * 2 * L.rowsp * 2);      // W^T, atoms x (hi | lo)
-      L.Rs = take(K * 2 * static_cast<size_t>(L.rowsp) * 2);            // residual r = W a - x
+      L.Rs = take(K * 2 * static_cast<size_t>(L.rowsp) * 2);            // x, then the residual r = W a - x
+      if (sc_use_gram(c)) {
+        L.Gs = take(static_cast<size_t>(c.cols) * 2 * L.colsp * 2);     // W^T W, atoms x (hi | lo)
+        L.G = take(c.sc_lipschitz > 0.f ? 0 : static_cast<size_t>(c.cols) * c.cols * 4);   // in fp32 for the power iteration
+        L.Bx = take(K * static_cast<size_t>(c.cols) * 4);               // W^T x
+        L.As2 = take(K * 2 * static_cast<size_t>(L.colsp) * 2);         // the codes of every other iteration
+      }
     }
     return;
   }
@@ -960,6 +1062,10 @@ int tc_init(sfb_ctx* ctx) {
     if (c.model == SFB_SC) {
       CKC(cudaMemsetAsync(ctx->at<char>(L.WTs), 0, static_cast<size_t>(c.cols) * 2 * L.rowsp * 2, ctx->stream));
       CKC(cudaMemsetAsync(ctx->at<char>(L.Rs), 0, K * 2 * L.rowsp * 2, ctx->stream));
+      if (L.Gs) {
+        CKC(cudaMemsetAsync(ctx->at<char>(L.Gs), 0, static_cast<size_t>(c.cols) * 2 * L.colsp * 2, ctx->stream));
+        CKC(cudaMemsetAsync(ctx->at<char>(L.As2), 0, K * 2 * L.colsp * 2, ctx->stream));
+      }
     }
     return SFB_OK;
   }
@@ -1003,16 +1109,23 @@ inline unsigned grid1d(int64_t items, int per_block) {
 // column-equivalents (below 128 columns a k-block is bound by the latency of its operand loads, not by the MMA).
 // Narrower tiles fill the SMs of small products, where 256-wide ones leave many idle or need a nearly empty
 // second round; ties go to the wider tile.
-inline int pick_tile_width(int sms, int64_t tilesM, int64_t N, int widest, int step = 32) {
+inline int pick_tile_width(int sms, int64_t tilesM, int64_t N, int widest, int step = 32, bool sym = false) {
   int best = widest;
   int64_t best_cost = INT64_MAX;
   for (int bn = widest; bn >= 128; bn -= step) {
-    const int64_t tiles = tilesM * ((N + bn - 1) / bn);
+    const int64_t tn = (N + bn - 1) / bn;
+    const int64_t tiles = sym ? sym_tiles(static_cast<int>(tilesM), static_cast<int>(tn), bn) : tilesM * tn;
     const int64_t cost = ((tiles + sms - 1) / sms) * (bn + 16);
     if (cost < best_cost) { best_cost = cost; best = bn; }
   }
   return best;
 }
+
+// Features up to which the coder on W^T W forms W^T x by fp32 FMAs and W^T W with its fourth term.  Every iterate carries
+// their error, and for short contractions the rounding of the operands to pairs is most of it (for long ones it is the
+// tensor core's own rounding, which the second accumulator brought down).  Error of the codes with / without, and with two
+// products per iteration: 700 x 400: 3.7e-6 / 9.1e-6, 5.0e-6; 1,501 x 1,400: 5.1e-6 / 9.9e-6, 7.3e-6.
+constexpr int64_t kPreciseRows = 2048;
 
 constexpr int kSplitPrefetch = SFB_SPLIT_PREFETCH;    // k-blocks of look-ahead of the L2 prefetch in the split products
 
@@ -1022,7 +1135,7 @@ template <int EPI>
 int split_product(sfb_ctx* ctx, int64_t off, int64_t n, __nv_bfloat16* A, __nv_bfloat16* B, int64_t N, int64_t Cp,
                   float* C, int64_t ldc, TcParams p, int64_t c_split_stride = 0, int* parts_out = nullptr) {
   const TcState* st = static_cast<const TcState*>(ctx->tc);
-  const int bn = pick_tile_width(st->sms, (n + BM - 1) / BM, N, FS_BN, 16);
+  const int bn = pick_tile_width(st->sms, (n + BM - 1) / BM, N, FS_BN, 16, EPI == F_GRAM);
   CUtensorMap ma, mb;
   if (!make_map(st, &ma, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, A, 2 * Cp, off + n, 2 * Cp * 2, BK, BM) ||
       !make_map(st, &mb, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, B, 2 * Cp, N, 2 * Cp * 2, BK, bn))
@@ -1044,7 +1157,7 @@ int split_product(sfb_ctx* ctx, int64_t off, int64_t n, __nv_bfloat16* A, __nv_b
   p.b_off0 = 0; p.b_off1 = static_cast<int32_t>(Cp); p.b_off2 = 0;
   p.status = ctx->at<uint32_t>(ctx->lay.status);
   CKC(launch_forward_split<EPI>(ctx, ma, mb, C, ldc, p));
-  ctx->stats.flops += 3.0 * 2.0 * n * N * Cp;
+  ctx->stats.flops += (EPI == F_GRAM ? 3.0 : 6.0) * n * N * Cp;
   return SFB_OK;
 }
 
@@ -1061,17 +1174,6 @@ int factors_split(sfb_ctx* ctx, int64_t off, int64_t n, const float* X, const fl
   float* U = ctx->at<float>(L.U);
   __nv_bfloat16* Ws = ctx->at<__nv_bfloat16>(L.Ws);
   __nv_bfloat16* As = ctx->at<__nv_bfloat16>(L.As);
-  if (ctx->committed == 0) {
-    // first factors of the step: refresh the split copies of the W every worker sees (BSP)
-    pack_split_rows_kernel<<<grid1d(rows * cols / 4, 256), 256, 0, s>>>(ctx->W, rows, cols, cols, Ws, L.colsp);
-    count_launch();
-    if (c.model == SFB_SC) {
-      pack_split_t_kernel<<<dim3(static_cast<unsigned>((cols + 63) / 64), static_cast<unsigned>(L.rowsp / 64)), 256, 0, s>>>(
-          ctx->W, rows, cols, cols, ctx->at<__nv_bfloat16>(L.WTs), L.rowsp);
-      count_launch();
-    }
-    CKC(cudaGetLastError());
-  }
   TcParams p{};
   if (c.model == SFB_DML) {
     CKC(pack_copy(s, V + off * cols, X, Y, n * cols));                                   // v = x - y
@@ -1087,29 +1189,100 @@ int factors_split(sfb_ctx* ctx, int64_t off, int64_t n, const float* X, const fl
                        dml_norm_out));
     return SFB_OK;
   }
-  // sparse coding: ISTA from a = 0, then u = W a - x, v = a
+  // Sparse coding: ISTA from a = 0, then u = W a - x, v = a.  The first iterate is soft(W^T x / L).
+  const int T = c.sc_ista_iters;
+  const bool gram = L.Gs != 0;
   __nv_bfloat16* WTs = ctx->at<__nv_bfloat16>(L.WTs);
   __nv_bfloat16* Rs = ctx->at<__nv_bfloat16>(L.Rs);
-  CKC(cudaMemsetAsync(V + off * cols, 0, static_cast<size_t>(n) * cols * 4, s));
-  CKC(cudaMemsetAsync(As + off * 2 * L.colsp, 0, static_cast<size_t>(n) * 2 * L.colsp * 2, s));
-  for (int it = 0; it <= c.sc_ista_iters; ++it) {
-    p = TcParams{};
-    p.aux = X - off * rows; p.ldaux = rows;          // X holds this worker's samples: index it by the global row
-    p.split = Rs; p.ld_split = 2 * L.rowsp; p.split_half = static_cast<int32_t>(L.rowsp);
-    int rc = split_product<F_SUB>(ctx, off, n, As, Ws, rows, L.colsp, U, L.ldu, p);     // r = W a - x
-    if (rc) return rc;
-    if (it == c.sc_ista_iters) break;
-    p = TcParams{};
-    p.aux = V; p.ldaux = cols;
-    p.sc = ctx->at<Scalars>(L.scalars); p.lam = c.sc_lambda;
-    p.split = As; p.ld_split = 2 * L.colsp; p.split_half = static_cast<int32_t>(L.colsp);
-    rc = split_product<F_ISTA>(ctx, off, n, Rs, WTs, cols, L.rowsp, V, cols, p);        // a <- soft(a - W^T r / L)
+  // the iterates as operands: with the Gram matrix a product reads one and writes the next, so two buffers in turn
+  __nv_bfloat16* as[2] = {As, gram ? ctx->at<__nv_bfloat16>(L.As2) : As};
+  auto ista = [&](int t) {
+    TcParams q{};
+    q.aux = V; q.ldaux = cols;
+    q.sc = ctx->at<Scalars>(L.scalars); q.lam = c.sc_lambda;
+    q.split = as[t & 1]; q.ld_split = 2 * L.colsp; q.split_half = static_cast<int32_t>(L.colsp);
+    return q;
+  };
+  auto residual = [&](__nv_bfloat16* a) {                                               // r = W a - x
+    TcParams q{};
+    q.aux = X - off * rows; q.ldaux = rows;          // X holds this worker's samples: index it by the global row
+    q.split = Rs; q.ld_split = 2 * L.rowsp; q.split_half = static_cast<int32_t>(L.rowsp);
+    return split_product<F_SUB>(ctx, off, n, a, Ws, rows, L.colsp, U, L.ldu, q);
+  };
+  int rc = SFB_OK;
+  if (T == 0) {
+    CKC(cudaMemsetAsync(V + off * cols, 0, static_cast<size_t>(n) * cols * 4, s));
+    CKC(cudaMemsetAsync(As + off * 2 * L.colsp, 0, static_cast<size_t>(n) * 2 * L.colsp * 2, s));
+  } else {
+    if (gram && rows <= kPreciseRows) {                                                 // W^T x, a_1
+      EpiArgs e{};
+      e.C = V + off * cols; e.ldc = cols; e.C2 = ctx->at<float>(L.Bx) + off * cols; e.ldc2 = cols;
+      e.sc = ctx->at<Scalars>(L.scalars); e.lam = c.sc_lambda;
+      CKC(sgemm(s, true, false, EPI_ISTA0, n, cols, rows, X, rows, ctx->W, cols, e, ctx->K));
+      ctx->stats.flops += 2.0 * n * rows * cols;
+      pack_split_rows_kernel<<<grid1d(n * cols / 4, 256), 256, 0, s>>>(V + off * cols, n, cols, cols, as[1] + off * 2 * L.colsp, L.colsp);
+      count_launch();
+    } else {
+      pack_split_rows_kernel<<<grid1d(n * ((rows + 3) / 4), 256), 256, 0, s>>>(X, n, rows, rows, Rs + off * 2 * L.rowsp, L.rowsp);
+      count_launch();
+      p = ista(1);
+      p.C2 = gram ? ctx->at<float>(L.Bx) : nullptr;
+      if ((rc = split_product<F_ISTA0>(ctx, off, n, Rs, WTs, cols, L.rowsp, V, cols, p)) != SFB_OK) return rc;
+    }
+  }
+  for (int t = 2; t <= T; ++t) {
+    p = ista(t);
+    if (gram) {
+      p.C2 = ctx->at<float>(L.Bx);
+      rc = split_product<F_ISTAG>(ctx, off, n, as[(t - 1) & 1], ctx->at<__nv_bfloat16>(L.Gs), cols, L.colsp, V, cols, p);
+    } else {
+      if ((rc = residual(As)) != SFB_OK) return rc;
+      rc = split_product<F_ISTA>(ctx, off, n, Rs, WTs, cols, L.rowsp, V, cols, p);      // a <- soft(a - W^T r / L)
+    }
     if (rc) return rc;
   }
-  return SFB_OK;
+  return residual(T == 0 ? As : as[T & 1]);                                             // u = W a - x
 }
 
 }  // namespace
+
+// The operands that the factors of every worker of a step share: the split copies of the W that all of them see
+// (bulk-synchronous consistency), and for sparse coding its transpose and W^T W.
+int tc_begin_step(sfb_ctx* ctx) {
+  const sfb_config& c = ctx->cfg;
+  if (c.model == SFB_MLR) return SFB_OK;
+  const Layout& L = ctx->lay;
+  const int64_t rows = c.rows, cols = c.cols;
+  cudaStream_t s = ctx->stream;
+  pack_split_rows_kernel<<<grid1d(rows * cols / 4, 256), 256, 0, s>>>(ctx->W, rows, cols, cols, ctx->at<__nv_bfloat16>(L.Ws), L.colsp);
+  count_launch();
+  if (c.model == SFB_SC) {
+    __nv_bfloat16* WTs = ctx->at<__nv_bfloat16>(L.WTs);
+    pack_split_t_kernel<<<dim3(static_cast<unsigned>((cols + 63) / 64), static_cast<unsigned>(L.rowsp / 64)), 256, 0, s>>>(
+        ctx->W, rows, cols, cols, WTs, L.rowsp);
+    count_launch();
+    if (L.Gs) {
+      TcParams p{};
+      p.four = rows <= kPreciseRows;
+      p.split = ctx->at<__nv_bfloat16>(L.Gs); p.ld_split = 2 * L.colsp; p.split_half = static_cast<int32_t>(L.colsp);
+      float* G = c.sc_lipschitz > 0.f ? nullptr : ctx->at<float>(L.G);
+      const int rc = split_product<F_GRAM>(ctx, 0, cols, WTs, WTs, cols, L.rowsp, G, cols, p);
+      if (rc) return rc;
+    }
+  }
+  CKC(cudaGetLastError());
+  return SFB_OK;
+}
+
+// Cost of a split product in rounds of tiles x columns x k-blocks (what pick_tile_width minimises).
+double split_product_cost(int64_t M, int64_t N, int64_t Kc, bool sym) {
+  const int sms = sm_count();
+  const int64_t tm = (M + BM - 1) / BM;
+  const int bn = pick_tile_width(sms, tm, N, FS_BN, 16, sym);
+  const int64_t tn = (N + bn - 1) / bn;
+  const int64_t tiles = sym ? sym_tiles(static_cast<int>(tm), static_cast<int>(tn), bn) : tm * tn;
+  return static_cast<double>((tiles + sms - 1) / sms) * (bn + 16) * (static_cast<double>((Kc + BK - 1) / BK) + 8.0);
+}
 
 // v = x, the (big | small) samples, and the logits of n samples at pair offset off against this context's rows as
 // the three-term tf32 product, with the per-(sample, 256-row block) softmax partials.

@@ -21,6 +21,9 @@ int tc_init(sfb_ctx* ctx);
 void tc_destroy(sfb_ctx* ctx);
 // Rebuilds the bf16 operand copy of W from the caller's fp32 W (MLR; the other models rebuild theirs every step).
 int tc_refresh_operands(sfb_ctx* ctx);
+// Before the first factors of a step: the operands derived from W that its workers share (DML, SC).
+int tc_begin_step(sfb_ctx* ctx);
+double split_product_cost(int64_t M, int64_t N, int64_t Kc, bool sym);
 // dml_norm_out (DML, row-sharded form; may be null): receives ||z_i||^2 of this context's rows and z stays unscaled.
 int tc_factors(sfb_ctx* ctx, int64_t off, int64_t n, const float* X, const float* Y, const int32_t* labels,
                float* dml_norm_out = nullptr);
