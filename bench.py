@@ -696,8 +696,8 @@ def main():
     if args.context_library_update and rank == 0 and prec == S.PREC_BF16 and wl.model == I.MLR and not sparse:
         Uq, Vq, dt_, lo_, ldu_, ldv_ = ctx.sfb_get_factors()
         ws0 = ctx.workspace.data_ptr()
-        UT = ctx.workspace[Uq - ws0:Uq - ws0 + wl.rows * ldu_ * 2].view(torch.bfloat16).view(wl.rows, ldu_)[:, :wl.K]
-        VT = ctx.workspace[Vq - ws0:Vq - ws0 + wl.cols * ldv_ * 2].view(torch.bfloat16).view(wl.cols, ldv_)[:, :wl.K]
+        UT = ctx.workspace[Uq - ws0:Uq - ws0 + wl.K * ldu_ * 2].view(torch.bfloat16).view(wl.K, ldu_)[:, :wl.rows].t()
+        VT = ctx.workspace[Vq - ws0:Vq - ws0 + wl.K * ldv_ * 2].view(torch.bfloat16).view(wl.K, ldv_)[:, :wl.cols].t()
         def library_loop(reps):
             e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
             e0.record()

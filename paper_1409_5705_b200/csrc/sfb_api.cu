@@ -232,7 +232,7 @@ static int factors_fp32(sfb_ctx* ctx, int64_t off, int64_t n, const float* X, co
     if (c.model == SFB_MLR)
       CK(mlr_softmax_rows(s, U, n, rows, ldu, labels, ctx->at<float>(ctx->lay.loss) + off, status));
     else
-      CK(dml_scale_rows(s, U, n, rows, ldu, labels, c.dml_margin, nullptr, dml_norm_out));
+      CK(dml_scale_rows(s, U, n, rows, ldu, labels, c.dml_margin, nullptr, 0, nullptr, dml_norm_out));
     return SFB_OK;
   }
   // Sparse coding: ISTA from a = 0, then u = W a - x, v = a.  The first iterate is soft(W^T x / L).
@@ -476,7 +476,8 @@ extern "C" int sfb_finish_factors(sfb_ctx* ctx, const float* partials_all_dev, i
   if (c.model == SFB_DML) {
     const int64_t ldu = ctx->lay.ldu;
     CK(dml_scale_rows(ctx->stream, ctx->at<float>(ctx->lay.U), ctx->K, c.rows, ldu, ctx->at<int32_t>(ctx->lay.stageL),
-                      c.dml_margin, nullptr, nullptr, partials_all_dev, shards, ctx->K));
+                      c.dml_margin, c.precision == SFB_PREC_BF16 ? ctx->at<char>(ctx->lay.Rs) : nullptr, ctx->lay.rowsp, nullptr,
+                      nullptr, partials_all_dev, shards, ctx->K));
     ctx->partials_ready = false;
     ctx->committed = c.workers == 64 ? ~0ull : ((1ull << c.workers) - 1);
     ctx->gathered = false;
@@ -521,6 +522,10 @@ extern "C" int sfb_set_factors(sfb_ctx* ctx, int32_t worker, const float* U_dev,
   CK(cudaMemcpy2DAsync(U, static_cast<size_t>(ldu) * 4, U_dev, static_cast<size_t>(c.rows) * 4, static_cast<size_t>(c.rows) * 4,
                        static_cast<size_t>(c.batch), cudaMemcpyDeviceToDevice, ctx->stream));
   CK(cudaMemcpyAsync(V, V_dev, static_cast<size_t>(c.batch) * c.cols * 4, cudaMemcpyDeviceToDevice, ctx->stream));
+  if (c.precision == SFB_PREC_BF16) {
+    const int rc = tc_pack_received(ctx, off, c.batch);
+    if (rc) return rc;
+  }
   ctx->committed |= 1ull << worker;
   ctx->sparse_mask &= ~(1ull << worker);             // received factors are dense
   ctx->gathered = false;
@@ -569,8 +574,8 @@ extern "C" int sfb_gather_factors(sfb_ctx* ctx) {
   if (ctx->sparse_v) {
     int rc = sparse_build_csc(ctx);
     if (rc) return rc;
-  } else if (c.precision == SFB_PREC_BF16 || ctx->tf32) {
-    int rc = ctx->tf32 ? tc32_gather(ctx) : tc_gather(ctx);
+  } else if (ctx->tf32) {
+    int rc = tc32_gather(ctx);
     if (rc) return rc;
   }
   if (c.model == SFB_MLR)

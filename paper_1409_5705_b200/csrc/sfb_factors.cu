@@ -3,6 +3,8 @@
 // power iteration that estimates the coder's step size.
 #include <algorithm>
 
+#include <cuda_bf16.h>
+
 #include "sfb_internal.h"
 
 namespace sfb {
@@ -286,7 +288,8 @@ __global__ void __launch_bounds__(NTHREADS) dml_scale_kernel(float* __restrict__
                                                              int64_t rows, int64_t ld,
                                                              const int32_t* __restrict__ similar, float margin,
                                                              float* __restrict__ norm_out, const float* __restrict__ norms_all,
-                                                             int shards, int64_t nstride) {
+                                                             int shards, int64_t nstride, __nv_bfloat16* __restrict__ split,
+                                                             int64_t split_half) {
   __shared__ float sh[32];
   float* z = Z + static_cast<int64_t>(blockIdx.x) * ld;
   if (Z2) {                      // z arrives as two partial sums over halves of the contraction (fixed order: Z + Z2)
@@ -306,7 +309,16 @@ __global__ void __launch_bounds__(NTHREADS) dml_scale_kernel(float* __restrict__
     return;
   }
   const float c = similar[blockIdx.x] != 0 ? 2.f : (q < margin ? -2.f : 0.f);
-  for (int64_t j = threadIdx.x; j < rows; j += NTHREADS) z[j] = c * z[j];
+  __nv_bfloat16* hp = split ? split + static_cast<int64_t>(blockIdx.x) * 2 * split_half : nullptr;
+  for (int64_t j = threadIdx.x; j < rows; j += NTHREADS) {
+    const float u = c * z[j];
+    z[j] = u;
+    if (hp) {
+      const __nv_bfloat16 hi = __float2bfloat16_rn(u);
+      hp[j] = hi;
+      hp[split_half + j] = __float2bfloat16_rn(u - __bfloat162float(hi));
+    }
+  }
 }
 
 __global__ void mean_kernel(const float* __restrict__ v, int64_t n, float* out) {
@@ -643,11 +655,12 @@ cudaError_t sdca_dual_rows(cudaStream_t s, float* Z, int64_t nsamp, int64_t rows
 }
 
 cudaError_t dml_scale_rows(cudaStream_t s, float* Z, int64_t nsamp, int64_t rows, int64_t ld,
-                           const int32_t* similar, float margin, const float* Z2, float* norm_out, const float* norms_all,
+                           const int32_t* similar, float margin, void* split, int64_t split_half, const float* Z2, float* norm_out, const float* norms_all,
                            int shards, int64_t nstride) {
   if (nsamp <= 0) return cudaSuccess;
   dml_scale_kernel<256><<<static_cast<unsigned>(nsamp), 256, 0, s>>>(Z, Z2, rows, ld, similar, margin, norm_out, norms_all,
-                                                                     shards, nstride);
+                                                                     shards, nstride, static_cast<__nv_bfloat16*>(split),
+                                                                     split_half);
   count_launch();
   return cudaGetLastError();
 }

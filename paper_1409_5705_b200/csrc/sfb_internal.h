@@ -73,7 +73,7 @@ constexpr int kProxSlabs = 64;        // row slabs of the deterministic column r
 struct Layout {
   size_t status, scalars, loss, V, U, colpart, stageX, stageY, stageL;
   // bf16 tensor-core mode
-  size_t Wb, Xb, VT, ZT, UT, part, Xf, labels, coef, lse;
+  size_t Wb, Xb, VT, ZT, UT, P, part, Xf, labels, coef, lse;   // VT, UT: tf32 words only; P: probabilities [K x ldp]
   // bf16 mode, DML and SC: (hi | lo) bf16 operands of the split products
   size_t Ws, WTs, As, Rs;             // W by rows, W transposed, the A operand (v or the codes), the residual
   size_t U2;                          // DML: second partial of z when the forward product splits its contraction
@@ -85,6 +85,7 @@ struct Layout {
   int64_t ldu;                        // row pitch of the fp32 U buffer (rows rounded up to 4; rows itself with tf32 pairs)
   int64_t colsp, rowsp;               // cols, rows rounded up to 64
   int64_t Kp;                         // K rounded up to the contraction block of the update product
+  int64_t ldp;                        // row pitch of P: rows rounded up to 64
   int64_t colsb;                      // cols rounded up to the contraction block of the forward product
   size_t total;
 };
@@ -215,8 +216,9 @@ cudaError_t sdca_dual_rows(cudaStream_t s, float* Z, int64_t nsamp, int64_t rows
 // Z2 (may be null): a second partial of z (the other half of the contraction), added to Z first.  Row-sharded form:
 // norm_out (may be null) receives the shard's ||z_i||^2 and z is left unscaled; norms_all (may be null), [shards][nstride],
 // supplies ||z_i||^2 as the sum over the shards instead of this context's own.
+// split (may be null): the scaled rows also as (hi | lo) bf16 pairs, row pitch 2 * split_half.
 cudaError_t dml_scale_rows(cudaStream_t s, float* Z, int64_t nsamp, int64_t rows, int64_t ld,
-                           const int32_t* similar, float margin, const float* Z2 = nullptr, float* norm_out = nullptr,
+                           const int32_t* similar, float margin, void* split, int64_t split_half, const float* Z2 = nullptr, float* norm_out = nullptr,
                            const float* norms_all = nullptr, int shards = 0, int64_t nstride = 0);
 cudaError_t mean_of(cudaStream_t s, const float* v, int64_t n, float* out);
 cudaError_t prox_unit_columns(cudaStream_t s, float* W, int64_t rows, int64_t cols, float* colpart);

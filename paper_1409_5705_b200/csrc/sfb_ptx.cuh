@@ -155,6 +155,17 @@ __device__ __forceinline__ uint64_t umma_desc_k128(uint32_t smem_addr) {
   return d;
 }
 
+// The same for an MN-major operand tile: the contraction is the outer dimension.  A TMA box {64 elements of M or N, 64 of the
+// contraction} with the 128-byte swizzle is one 8 KB atom column: rows (of the contraction) of 128 bytes, groups of 8 of them
+// 1024 bytes apart (stride byte offset); the next 64 elements of M or N are the next box, 8 KB on (leading byte offset).
+// A step of 16 along the contraction advances the start address by 2048 bytes.
+__device__ __forceinline__ uint64_t umma_desc_mn128(uint32_t smem_addr) {
+  uint64_t d = umma_desc_k128(smem_addr);
+  d |= static_cast<uint64_t>(8192 >> 4) << 16;                    // bits 16-29: leading byte offset >> 4
+  return d;
+}
+constexpr uint32_t kIdescMnMajor = (1u << 15) | (1u << 16);       // A and B are MN-major (default: K-major)
+
 // Instruction descriptor of kind::f16 with bf16 A and B (both K-major), fp32 accumulator, tile M x N.
 __device__ __forceinline__ uint32_t umma_idesc_bf16(uint32_t M, uint32_t N) {
   uint32_t d = 0;

@@ -287,8 +287,8 @@ __global__ void __launch_bounds__(kSfThreads, 1) sparse_forward_kernel(const flo
 // for each of the 32 columns it sums x_id * u[i][row] over the column's entries (the entries are read by all lanes at
 // once, the slab row by row without bank conflicts).  The 32 x 32 sums are then transposed through shared memory so
 // that a lane is a COLUMN and each row's 32 entries of W leave as one 128-byte piece.
-//   USRC 0: factors fp32, sample-major [K x ldu] (fp32 modes);  1: bf16, transposed [rows x ldut] (bf16 mode, whose
-//           label entries are applied separately in fp32).
+//   USRC 0: factors fp32, sample-major [K x ldu] (fp32 modes);  1: bf16, sample-major [K x ldp] (bf16 mode, whose label
+//           entries are applied separately in fp32).
 //   SHADOW 0: none;  1: bf16 operand copy of W, a 64-byte row piece rewritten only if one of its roundings changed;
 //           2: the (big | small) tf32 copy.
 // ---------------------------------------------------------------------------------------------------------
@@ -299,8 +299,8 @@ struct SuParams {
   const int2* ent;
   const float* U;
   int64_t ldu;
-  const __nv_bfloat16* UT;
-  int64_t ldut;
+  const __nv_bfloat16* P;
+  int64_t ldp;
   int32_t K;
   float alpha;
   int32_t prox_kind;
@@ -358,13 +358,11 @@ __global__ void __launch_bounds__(kSuThreads, 1) sparse_update_kernel(const SuPa
       for (int i = warp; i < p.K; i += kSuWarps)
         *reinterpret_cast<float*>(us + i * S::kPitch + lane * 4) = rv ? p.U[static_cast<int64_t>(i) * p.ldu + r0 + lane] : 0.f;
     } else {
-      for (int r = warp; r < 32; r += kSuWarps) {
-        const bool rv = r < nrows;
-        const uint16_t* src = reinterpret_cast<const uint16_t*>(p.UT) + (r0 + r) * p.ldut;
+      const bool rv = lane < nrows;
 #pragma unroll 8
-        for (int i = lane; i < p.K; i += 32)
-          *reinterpret_cast<uint16_t*>(us + i * S::kPitch + r * 2) = rv ? src[i] : static_cast<uint16_t>(0);
-      }
+      for (int i = warp; i < p.K; i += kSuWarps)
+        *reinterpret_cast<uint16_t*>(us + i * S::kPitch + lane * 2) =
+            rv ? reinterpret_cast<const uint16_t*>(p.P)[static_cast<int64_t>(i) * p.ldp + r0 + lane] : static_cast<uint16_t>(0);
     }
     if (threadIdx.x == 0) next_cb = 0;
     __syncthreads();
@@ -671,7 +669,7 @@ int sparse_update(sfb_ctx* ctx) {
   p.alpha = -ctx->step;
   p.prox_kind = ctx->prox_kind; p.prox_a = ctx->prox_a;
   if (bf16) {
-    p.UT = ctx->at<__nv_bfloat16>(L.UT); p.ldut = L.Kp;
+    p.P = ctx->at<__nv_bfloat16>(L.P); p.ldp = L.ldp;
     p.shadow = ctx->at<__nv_bfloat16>(L.Wb); p.shadow_ld = L.colsb;
     p.copy_counters = &ctx->at<Scalars>(L.scalars)->copy_pieces;
     CKS((launch_sparse_update<1, 1>(ctx->stream, p, smem)));

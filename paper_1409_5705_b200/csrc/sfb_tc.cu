@@ -565,52 +565,28 @@ __global__ void __launch_bounds__(256) convert_rows_kernel(const float* __restri
 }
 
 // Pack of the inputs of n samples starting at pair index off (Section 2.1: v = a_i):
-//   Xb[off + i][:]  = bf16(x_i)          forward operand, sample-major
-//   VT[:][off + i]  = bf16(x_i)          update operand, feature-major (V^T)
-// 64 x 64 tiles through shared memory so that both sides are written in 16-byte pieces.
+//   Xb[off + i][:]  = bf16(x_i), the operand of the forward product and of the update (which contracts over the samples and
+//                     takes it as an MN-major operand),   Xf = the fp32 sample for the label rows,   labels.
+// One read of X, 6 bytes written per value; bound by HBM (1,024 x 20,000: 33 us with a transposed copy beside it, 24 without).
 __global__ void __launch_bounds__(256) pack_mlr_kernel(const float* __restrict__ X, int64_t n, int64_t cols,
-                                                       __nv_bfloat16* __restrict__ Xb, int64_t ldx,
-                                                       __nv_bfloat16* __restrict__ VT, int64_t ldv, int64_t off,
+                                                       __nv_bfloat16* __restrict__ Xb, int64_t ldx, int64_t off,
                                                        float* __restrict__ Xf, const int32_t* __restrict__ labels,
                                                        int32_t* __restrict__ labels_out) {
-  __shared__ float tile[64][65];
-  const int64_t i0 = static_cast<int64_t>(blockIdx.y) * 64, c0 = static_cast<int64_t>(blockIdx.x) * 64;
-  const int t = threadIdx.x;
-#pragma unroll
-  for (int v = 0; v < 4; ++v) {
-    const int idx = t + v * 256;            // 64 samples x 16 quads
-    const int i = idx / 16, cq = (idx % 16) * 4;
-    float4 val = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (i0 + i < n && c0 + cq < cols) val = *reinterpret_cast<const float4*>(X + (i0 + i) * cols + c0 + cq);
-    tile[i][cq + 0] = val.x; tile[i][cq + 1] = val.y; tile[i][cq + 2] = val.z; tile[i][cq + 3] = val.w;
-    if (i0 + i < n && c0 + cq < cols) {
-      *reinterpret_cast<uint2*>(Xb + (off + i0 + i) * ldx + c0 + cq) =
-          make_uint2(pack_bf16(val.x, val.y), pack_bf16(val.z, val.w));
-      *reinterpret_cast<float4*>(Xf + (off + i0 + i) * cols + c0 + cq) = val;
-    }
+  const uint32_t quads = static_cast<uint32_t>(cols / 4);
+  const int64_t total = n * quads, stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
+  const int64_t t0 = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
+  for (int64_t q = t0; q < total; q += stride) {
+    const int64_t i = q / quads, c = (q - i * quads) * 4;
+    const float4 v = *reinterpret_cast<const float4*>(X + i * cols + c);
+    *reinterpret_cast<uint2*>(Xb + (off + i) * ldx + c) = make_uint2(pack_bf16(v.x, v.y), pack_bf16(v.z, v.w));
+    *reinterpret_cast<float4*>(Xf + (off + i) * cols + c) = v;
   }
-  if (blockIdx.x == 0 && t < 64 && i0 + t < n) labels_out[off + i0 + t] = labels[i0 + t];
-  __syncthreads();
-#pragma unroll
-  for (int v = 0; v < 2; ++v) {
-    const int idx = t + v * 256;            // 64 features x 8 groups of 8 samples
-    const int c = idx / 8, ig = (idx % 8) * 8;
-    if (c0 + c >= cols) continue;
-    __nv_bfloat16* dst = VT + (c0 + c) * ldv + off + i0 + ig;
-    if (i0 + ig + 7 < n && ((off + i0 + ig) & 7) == 0) {
-      *reinterpret_cast<uint4*>(dst) =
-          make_uint4(pack_bf16(tile[ig][c], tile[ig + 1][c]), pack_bf16(tile[ig + 2][c], tile[ig + 3][c]),
-                     pack_bf16(tile[ig + 4][c], tile[ig + 5][c]), pack_bf16(tile[ig + 6][c], tile[ig + 7][c]));
-    } else {
-      for (int k = 0; k < 8; ++k)
-        if (i0 + ig + k < n) dst[k] = __float2bfloat16_rn(tile[ig + k][c]);
-    }
-  }
+  for (int64_t i = t0; i < n; i += stride) labels_out[off + i] = labels[i];
 }
 
-// Gathered fp32 factors F [n x dim] (pair-major) -> the split-bf16 operand of the update product,
-// FT [dim x 2*Kp] (samples contiguous): FT[c][i] = hi(F[i][c]), FT[c][Kp + i] = lo(F[i][c]) with
-// hi = bf16(f), lo = bf16(f - hi); samples n..Kp-1 are written as zeros.  64 x 64 tiles through shared memory.
+// W [n x dim] -> its transpose as a (hi | lo) bf16 operand FT [dim x 2*Kp] (the coder's W^T): FT[c][i] = hi(F[i][c]),
+// FT[c][Kp + i] = lo(F[i][c]) with hi = bf16(f), lo = bf16(f - hi); rows n..Kp-1 are written as zeros.  64 x 64 tiles through
+// shared memory.
 __global__ void __launch_bounds__(256) pack_split_t_kernel(const float* __restrict__ F, int64_t n, int64_t dim,
                                                            int64_t ld, __nv_bfloat16* __restrict__ FT, int64_t Kp) {
   __shared__ float tile[64][65];
@@ -783,59 +759,29 @@ __global__ void __launch_bounds__(256) mlr_shard_finish_tc_kernel(const float4* 
   labels[i] = mine ? static_cast<int32_t>(yl) : -1;
 }
 
-// P^T[r][off + i] = bf16( exp(z_ir - lse_i) ) for r != y_i and 0 for r = y_i: 64 samples x 64 rows per block,
-// transposed through shared memory (Z is sample-major, the update operand is row-major with samples
-// contiguous).  The factor is u_i = p_i - onehot(y_i); its label entry u_iy = p_iy - 1 is left out of the bf16
-// operand and applied to W in fp32 by label_rows_kernel, because bf16 cannot hold it when p_iy is close to 1
-// (spacing 2^-8 next to 1) and a rounded p_iy with an exact -1 would not cancel.
-// PLAIN: the values of Z themselves instead of exp(z - lse) (the dual changes of the SDCA step), same layout and
-// the same zero at the label entry.
+// P[off + i][r] = bf16( exp(z_ir - lse_i) ) for r != y_i and 0 for r = y_i, from the logits Z (row pitch a multiple of 32).
+// The factor is u_i = p_i - onehot(y_i); its label entry u_iy = p_iy - 1 is left out of the bf16 operand and applied to W in
+// fp32 by label_rows_kernel, because bf16 cannot hold it when p_iy is close to 1 (spacing 2^-8 next to 1) and a rounded p_iy
+// with an exact -1 would not cancel.  Eight values per thread; 6 bytes per value, bound by HBM.
+// PLAIN: the values of Z themselves instead of exp(z - lse) (the dual changes of the SDCA step), with the same zero at the
+// label entry.
 template <bool PLAIN>
-__global__ void __launch_bounds__(256) mlr_emit_ut_kernel(const float* __restrict__ Z, int64_t ldz, int64_t rows,
-                                                          const float* __restrict__ lse, int64_t off, int64_t n,
-                                                          const int32_t* __restrict__ labels,
-                                                          __nv_bfloat16* __restrict__ UT, int64_t ldu) {
-  __shared__ float tile[64][65];
-  const int64_t i0 = static_cast<int64_t>(blockIdx.y) * 64, r0 = static_cast<int64_t>(blockIdx.x) * 64;
-  const int t = threadIdx.x;
-  const bool vec = (ldz % 4) == 0;
-#pragma unroll
-  for (int v = 0; v < 4; ++v) {
-    const int idx = t + v * 256;
-    const int i = idx / 16, rq = (idx % 16) * 4;
-    if (i0 + i >= n) continue;
-    const int64_t s = off + i0 + i;
+__global__ void __launch_bounds__(256) mlr_emit_p_kernel(const float* __restrict__ Z, int64_t ldz, int64_t rows,
+                                                         const float* __restrict__ lse, int64_t off, int64_t n,
+                                                         const int32_t* __restrict__ labels, __nv_bfloat16* __restrict__ P,
+                                                         int64_t ldp) {
+  const uint32_t octs = static_cast<uint32_t>((rows + 7) / 8);
+  const int64_t total = n * octs, stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
+  for (int64_t q = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; q < total; q += stride) {
+    const int64_t i = q / octs, r = (q - i * octs) * 8, s = off + i;
     const float l = PLAIN ? 0.f : lse[s];
-    const int64_t yrel = static_cast<int64_t>(labels[i0 + i]) - (r0 + rq);     // label row relative to this quad
-    const float* zp = Z + s * ldz + r0 + rq;
-    float z[4] = {0.f, 0.f, 0.f, 0.f};
-    if (vec && r0 + rq + 3 < rows) {
-      const float4 q4 = *reinterpret_cast<const float4*>(zp);
-      z[0] = q4.x; z[1] = q4.y; z[2] = q4.z; z[3] = q4.w;
-    } else {
-      for (int k = 0; k < 4; ++k)
-        if (r0 + rq + k < rows) z[k] = zp[k];
-    }
+    const int64_t yrel = static_cast<int64_t>(labels[i]) - r;           // label row relative to this group of eight
+    const float4 a = *reinterpret_cast<const float4*>(Z + s * ldz + r), b = *reinterpret_cast<const float4*>(Z + s * ldz + r + 4);
+    float z[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      tile[i][rq + k] = k == yrel ? 0.f : (PLAIN ? z[k] : __expf(z[k] - l));
-    }
-  }
-  __syncthreads();
-#pragma unroll
-  for (int v = 0; v < 2; ++v) {
-    const int idx = t + v * 256;
-    const int r = idx / 8, ig = (idx % 8) * 8;
-    if (r0 + r >= rows) continue;
-    __nv_bfloat16* dst = UT + (r0 + r) * ldu + off + i0 + ig;
-    if (i0 + ig + 7 < n && ((off + i0 + ig) & 7) == 0) {
-      *reinterpret_cast<uint4*>(dst) =
-          make_uint4(pack_bf16(tile[ig][r], tile[ig + 1][r]), pack_bf16(tile[ig + 2][r], tile[ig + 3][r]),
-                     pack_bf16(tile[ig + 4][r], tile[ig + 5][r]), pack_bf16(tile[ig + 6][r], tile[ig + 7][r]));
-    } else {
-      for (int k = 0; k < 8; ++k)
-        if (i0 + ig + k < n) dst[k] = __float2bfloat16_rn(tile[ig + k][r]);
-    }
+    for (int k = 0; k < 8; ++k) z[k] = k == yrel ? 0.f : (PLAIN ? z[k] : __expf(z[k] - l));
+    *reinterpret_cast<uint4*>(P + s * ldp + r) =
+        make_uint4(pack_bf16(z[0], z[1]), pack_bf16(z[2], z[3]), pack_bf16(z[4], z[5]), pack_bf16(z[6], z[7]));
   }
 }
 
@@ -989,21 +935,18 @@ void tc_extend_layout(const sfb_config& c, Layout& L, size_t& off) {
   L.Kp = round_up(static_cast<int64_t>(K), 64);
   L.colsb = round_up(c.cols, 64);
   if (c.model != SFB_MLR) {
-    // fp32 factors as the workers write them, their split-bf16 transposes for the update product, and the
-    // split-bf16 operands of the forward products
+    // fp32 factors as the workers write them, and the split-bf16 operands of the forward and update products
     L.colsp = round_up(c.cols, 64);
     L.rowsp = round_up(c.rows, 64);
     L.ldu = round_up(c.rows, 4);                                        // TMA stores need a 16-byte row pitch
     L.V = take(K * static_cast<size_t>(c.cols) * 4);
     L.U = take(K * static_cast<size_t>(L.ldu) * 4);
     L.U2 = take(c.model == SFB_DML ? K * static_cast<size_t>(L.ldu) * 4 : 0);
-    L.UT = take(static_cast<size_t>(c.rows) * 2 * L.Kp * 2);
-    L.VT = take(static_cast<size_t>(c.cols) * 2 * L.Kp * 2);
+    L.Rs = take(K * 2 * static_cast<size_t>(L.rowsp) * 2);              // u (SC: first x, then the residuals)
     L.Ws = take(static_cast<size_t>(c.rows) * 2 * L.colsp * 2);         // W, rows x (hi | lo)
     L.As = take(K * 2 * static_cast<size_t>(L.colsp) * 2);              // v (DML) or the codes a (SC)
     if (c.model == SFB_SC) {
       L.WTs = take(static_cast<size_t>(c.cols) * 2 * L.rowsp * 2);      // W^T, atoms x (hi | lo)
-      L.Rs = take(K * 2 * static_cast<size_t>(L.rowsp) * 2);            // x, then the residual r = W a - x
       if (sc_use_gram(c)) {
         L.Gs = take(static_cast<size_t>(c.cols) * 2 * L.colsp * 2);     // W^T W, atoms x (hi | lo)
         L.G = take(c.sc_lipschitz > 0.f ? 0 : static_cast<size_t>(c.cols) * c.cols * 4);   // in fp32 for the power iteration
@@ -1017,9 +960,9 @@ void tc_extend_layout(const sfb_config& c, Layout& L, size_t& off) {
   const size_t nblk = static_cast<size_t>((c.rows + BN - 1) / BN);
   L.Wb = take(static_cast<size_t>(c.rows) * L.colsb * 2);
   L.Xb = take(K * L.colsb * 2);
-  L.VT = take(static_cast<size_t>(c.cols) * L.Kp * 2);
   L.ZT = take(K * ldz * 4);                      // logits Z, sample-major [K x ldz]
-  L.UT = take(static_cast<size_t>(c.rows) * L.Kp * 2);
+  L.ldp = round_up(c.rows, 64);
+  L.P = take(K * static_cast<size_t>(L.ldp) * 2);
   L.part = take(nblk * K * 8);
   L.V = take(K * 4);                             // log-sum-exp per sample
   L.Xf = take(K * static_cast<size_t>(c.cols) * 4);   // fp32 copy of the K samples (exact label-row term)
@@ -1059,9 +1002,9 @@ int tc_init(sfb_ctx* ctx) {
     const size_t K = static_cast<size_t>(ctx->K);
     CKC(cudaMemsetAsync(ctx->at<char>(L.Ws), 0, static_cast<size_t>(c.rows) * 2 * L.colsp * 2, ctx->stream));
     CKC(cudaMemsetAsync(ctx->at<char>(L.As), 0, K * 2 * L.colsp * 2, ctx->stream));
+    CKC(cudaMemsetAsync(ctx->at<char>(L.Rs), 0, K * 2 * L.rowsp * 2, ctx->stream));
     if (c.model == SFB_SC) {
       CKC(cudaMemsetAsync(ctx->at<char>(L.WTs), 0, static_cast<size_t>(c.cols) * 2 * L.rowsp * 2, ctx->stream));
-      CKC(cudaMemsetAsync(ctx->at<char>(L.Rs), 0, K * 2 * L.rowsp * 2, ctx->stream));
       if (L.Gs) {
         CKC(cudaMemsetAsync(ctx->at<char>(L.Gs), 0, static_cast<size_t>(c.cols) * 2 * L.colsp * 2, ctx->stream));
         CKC(cudaMemsetAsync(ctx->at<char>(L.As2), 0, K * 2 * L.colsp * 2, ctx->stream));
@@ -1185,7 +1128,8 @@ int factors_split(sfb_ctx* ctx, int64_t off, int64_t n, const float* X, const fl
     int parts = 1;
     int rc = split_product<F_STORE>(ctx, off, n, As, Ws, rows, L.colsp, U, L.ldu, p, U2 - U, &parts);   // z_i = W v_i
     if (rc) return rc;
-    CKC(dml_scale_rows(s, U + off * L.ldu, n, rows, L.ldu, labels, c.dml_margin, parts > 1 ? U2 + off * L.ldu : nullptr,
+    CKC(dml_scale_rows(s, U + off * L.ldu, n, rows, L.ldu, labels, c.dml_margin,
+                       ctx->at<__nv_bfloat16>(L.Rs) + off * 2 * L.rowsp, L.rowsp, parts > 1 ? U2 + off * L.ldu : nullptr,
                        dml_norm_out));
     return SFB_OK;
   }
@@ -1415,9 +1359,8 @@ static int mlr_forward(sfb_ctx* ctx, int64_t off, int64_t n, const float* X, con
   const int64_t rows = c.rows, cols = c.cols, K = ctx->K;
   const int64_t ldz = round_up(rows, 32);
   __nv_bfloat16* Xb = ctx->at<__nv_bfloat16>(L.Xb);
-  dim3 pgrid(static_cast<unsigned>((cols + 63) / 64), static_cast<unsigned>((n + 63) / 64));
-  pack_mlr_kernel<<<pgrid, 256, 0, ctx->stream>>>(X, n, cols, Xb, L.colsb, ctx->at<__nv_bfloat16>(L.VT), L.Kp, off,
-                                                  ctx->at<float>(L.Xf), labels, ctx->at<int32_t>(L.labels));
+  pack_mlr_kernel<<<grid1d(n * cols / 4, 256), 256, 0, ctx->stream>>>(X, n, cols, Xb, L.colsb, off, ctx->at<float>(L.Xf), labels,
+                                                                      ctx->at<int32_t>(L.labels));
   count_launch();
   CKC(cudaGetLastError());
   // samples on the lanes (A), rows of W on the accumulator columns (B)
@@ -1462,9 +1405,9 @@ int tc_finish_factors(sfb_ctx* ctx, const float* parts, int shards) {
       reinterpret_cast<const float4*>(parts), shards, K, c.rows, ctx->row_offset, ctx->at<int32_t>(L.labels),
       ctx->at<float>(L.V), ctx->at<float>(L.loss), ctx->at<float>(L.coef), ctx->at<uint32_t>(L.status));
   count_launch();
-  dim3 egrid(static_cast<unsigned>((c.rows + 63) / 64), static_cast<unsigned>((K + 63) / 64));
-  mlr_emit_ut_kernel<false><<<egrid, 256, 0, ctx->stream>>>(ctx->at<float>(L.ZT), round_up(c.rows, 32), c.rows, ctx->at<float>(L.V), 0, K,
-                                                     ctx->at<int32_t>(L.labels), ctx->at<__nv_bfloat16>(L.UT), L.Kp);
+  mlr_emit_p_kernel<false><<<grid1d(K * ((c.rows + 7) / 8), 256), 256, 0, ctx->stream>>>(
+      ctx->at<float>(L.ZT), round_up(c.rows, 32), c.rows, ctx->at<float>(L.V), 0, K, ctx->at<int32_t>(L.labels),
+      ctx->at<__nv_bfloat16>(L.P), L.ldp);
   count_launch();
   CKC(cudaGetLastError());
   return SFB_OK;
@@ -1548,12 +1491,11 @@ int tc_import_factors(sfb_ctx* ctx, int64_t off, int64_t n, const float* U_in, c
   float* Z = ctx->at<float>(L.ZT);
   CKC(cudaMemcpy2DAsync(Z + off * ldz, static_cast<size_t>(ldz) * 4, U_in, static_cast<size_t>(rows) * 4,
                         static_cast<size_t>(rows) * 4, static_cast<size_t>(n), cudaMemcpyDeviceToDevice, s));
-  dim3 pgrid(static_cast<unsigned>((cols + 63) / 64), static_cast<unsigned>((n + 63) / 64));
-  pack_mlr_kernel<<<pgrid, 256, 0, s>>>(V_in, n, cols, ctx->at<__nv_bfloat16>(L.Xb), L.colsb, ctx->at<__nv_bfloat16>(L.VT), L.Kp,
-                                        off, ctx->at<float>(L.Xf), labels + off, labels);
+  pack_mlr_kernel<<<grid1d(n * cols / 4, 256), 256, 0, s>>>(V_in, n, cols, ctx->at<__nv_bfloat16>(L.Xb), L.colsb, off,
+                                                            ctx->at<float>(L.Xf), labels + off, labels);
   count_launch();
-  dim3 egrid(static_cast<unsigned>((rows + 63) / 64), static_cast<unsigned>((n + 63) / 64));
-  mlr_emit_ut_kernel<true><<<egrid, 256, 0, s>>>(Z, ldz, rows, nullptr, off, n, labels + off, ctx->at<__nv_bfloat16>(L.UT), L.Kp);
+  mlr_emit_p_kernel<true><<<grid1d(n * ((rows + 7) / 8), 256), 256, 0, s>>>(Z, ldz, rows, nullptr, off, n, labels + off,
+                                                                            ctx->at<__nv_bfloat16>(L.P), L.ldp);
   count_launch();
   CKC(cudaGetLastError());
   return SFB_OK;
@@ -1573,9 +1515,8 @@ int tc_sdca_factors(sfb_ctx* ctx, int64_t off, int64_t n, const float* X, const 
   if (rc) return rc;
   CKC(sdca_dual_rows(ctx->stream, Z + off * ldz, n, rows, ldz, X, c.cols, labels, ids, ctx->dualQ, ctx->dual_n, inv_lam_n,
                      c.eta, ctx->at<float>(L.coef) + off, ctx->at<float>(L.loss) + off, ctx->at<uint32_t>(L.status)));
-  dim3 egrid(static_cast<unsigned>((rows + 63) / 64), static_cast<unsigned>((n + 63) / 64));
-  mlr_emit_ut_kernel<true><<<egrid, 256, 0, ctx->stream>>>(Z, ldz, rows, nullptr, off, n, labels, ctx->at<__nv_bfloat16>(L.UT),
-                                                           L.Kp);
+  mlr_emit_p_kernel<true><<<grid1d(n * ((rows + 7) / 8), 256), 256, 0, ctx->stream>>>(Z, ldz, rows, nullptr, off, n, labels,
+                                                                                      ctx->at<__nv_bfloat16>(L.P), L.ldp);
   count_launch();
   CKC(cudaGetLastError());
   return SFB_OK;
@@ -1597,25 +1538,30 @@ int tc_factors(sfb_ctx* ctx, int64_t off, int64_t n, const float* X, const float
       ctx->at<float2>(L.part), K, tiles_n, Z, ldz, rows, labels, off, n, lse, ctx->at<float>(L.loss), ctx->at<float>(L.coef),
       ctx->at<uint32_t>(L.status));
   count_launch();
-  dim3 egrid(static_cast<unsigned>((rows + 63) / 64), static_cast<unsigned>((n + 63) / 64));
-  mlr_emit_ut_kernel<false><<<egrid, 256, 0, ctx->stream>>>(Z, ldz, rows, lse, off, n, labels, ctx->at<__nv_bfloat16>(L.UT), L.Kp);
+  mlr_emit_p_kernel<false><<<grid1d(n * ((rows + 7) / 8), 256), 256, 0, ctx->stream>>>(Z, ldz, rows, lse, off, n, labels,
+                                                                                       ctx->at<__nv_bfloat16>(L.P), L.ldp);
   count_launch();
   CKC(cudaGetLastError());
   return SFB_OK;
 }
 
-// MLR: every worker wrote at its offset of U^T and V^T, nothing to move.  DML, SC: the workers' fp32 factors
-// are transposed into the split-bf16 operands of the update product.
-int tc_gather(sfb_ctx* ctx) {
-  const sfb_config& c = ctx->cfg;
-  if (c.model == SFB_MLR) return SFB_OK;
+// The (hi | lo) codes or pair differences: the operand V of the update.
+__nv_bfloat16* tc_split_v(const sfb_ctx* ctx) {
   const Layout& L = ctx->lay;
-  const unsigned gy = static_cast<unsigned>(L.Kp / 64);
-  pack_split_t_kernel<<<dim3(static_cast<unsigned>((c.rows + 63) / 64), gy), 256, 0, ctx->stream>>>(
-      ctx->at<float>(L.U), ctx->K, c.rows, L.ldu, ctx->at<__nv_bfloat16>(L.UT), L.Kp);
+  const bool odd = ctx->cfg.model == SFB_SC && L.Gs != 0 && (ctx->cfg.sc_ista_iters & 1);     // which buffer the last iterate is in
+  return ctx->at<__nv_bfloat16>(odd ? L.As2 : L.As);
+}
+
+// Factors computed elsewhere (DML, SC): fp32 pairs in U and V -> the operands of the update.
+int tc_pack_received(sfb_ctx* ctx, int64_t off, int64_t n) {
+  const sfb_config& c = ctx->cfg;
+  const Layout& L = ctx->lay;
+  cudaStream_t s = ctx->stream;
+  pack_split_rows_kernel<<<grid1d(n * ((c.rows + 3) / 4), 256), 256, 0, s>>>(ctx->at<float>(L.U) + off * L.ldu, n, c.rows, L.ldu,
+                                                                            ctx->at<__nv_bfloat16>(L.Rs) + off * 2 * L.rowsp, L.rowsp);
   count_launch();
-  pack_split_t_kernel<<<dim3(static_cast<unsigned>((c.cols + 63) / 64), gy), 256, 0, ctx->stream>>>(
-      ctx->at<float>(L.V), ctx->K, c.cols, c.cols, ctx->at<__nv_bfloat16>(L.VT), L.Kp);
+  pack_split_rows_kernel<<<grid1d(n * c.cols / 4, 256), 256, 0, s>>>(ctx->at<float>(L.V) + off * c.cols, n, c.cols, c.cols,
+                                                                     tc_split_v(ctx) + off * 2 * L.colsp, L.colsp);
   count_launch();
   CKC(cudaGetLastError());
   return SFB_OK;
@@ -1632,12 +1578,12 @@ int tc_get_factors(sfb_ctx* ctx, const void** U, const void** V, int32_t* dtype,
     if (ldv) *ldv = ctx->cfg.cols;
     return SFB_OK;
   }
-  if (U) *U = ctx->at<__nv_bfloat16>(ctx->lay.UT);
-  if (V) *V = ctx->at<__nv_bfloat16>(ctx->lay.VT);
+  if (U) *U = ctx->at<__nv_bfloat16>(ctx->lay.P);
+  if (V) *V = ctx->at<__nv_bfloat16>(ctx->lay.Xb);
   if (dtype) *dtype = 1;
-  if (layout) *layout = 1;
-  if (ldu) *ldu = ctx->lay.Kp;
-  if (ldv) *ldv = ctx->lay.Kp;
+  if (layout) *layout = 0;
+  if (ldu) *ldu = ctx->lay.ldp;
+  if (ldv) *ldv = ctx->lay.colsb;
   return SFB_OK;
 }
 

@@ -2,6 +2,7 @@
 // the tensor-core translation units share (sfb_tc.cu: factors and forward product; sfb_update.cu: the update).
 #pragma once
 #include <cuda.h>
+#include <cuda_bf16.h>
 
 #include "sfb_internal.h"
 
@@ -36,7 +37,9 @@ int tc_sdca_factors(sfb_ctx* ctx, int64_t off, int64_t n, const float* X, const 
 // MLR, bf16 mode: a worker's factors in fp32 as they are sent, and received fp32 factors put into the bf16 layout.
 int tc_export_factors(sfb_ctx* ctx, int64_t off, int64_t n, float* U_out, float* V_out);
 int tc_import_factors(sfb_ctx* ctx, int64_t off, int64_t n, const float* U_in, const float* V_in);
-int tc_gather(sfb_ctx* ctx);
+// DML, SC in bf16 mode: fp32 factors put into the U and V buffers by the caller become (hi | lo) operands; the operand of V.
+int tc_pack_received(sfb_ctx* ctx, int64_t off, int64_t n);
+__nv_bfloat16* tc_split_v(const sfb_ctx* ctx);
 int tc_update(sfb_ctx* ctx);
 int tc_get_factors(sfb_ctx* ctx, const void** U, const void** V, int32_t* dtype, int32_t* layout, int64_t* ldu,
                    int64_t* ldv);

@@ -8,6 +8,9 @@
 // stages of 256 columns), loads its own 128 x 64 slice of U^T and its own 128 x 64 half of the V^T slice per
 // k-block (32 KB per stage instead of the 48 KB a single-CTA 128 x 256 tile needs), and streams its own
 // 128 x 256 fp32 half of the W tile.
+// The bf16 operands are the gathered factors as the forward side leaves them, U [pairs x rows] and V [pairs x columns]: the
+// contraction runs over pairs, so both are MN-major operands and no transposed copy of either exists (the transposes were
+// a sixth of a step of metric learning at 1,000 x 20,000).  The tf32 words are K-major (U^T, V^T).
 // Warps of a CTA: 0 = TMA producer, 1 = MMA issuer (leader CTA only) and TMEM owner, 2..9 = epilogue.
 // Epilogue warp (q, h): TMEM lane quarter q (32 rows of W), column half h (128 columns), in four chunks of
 // 32 x 32.  Each warp owns a ring of three 4 KB slots: the W chunk lands there by TMA (two chunks in flight per
@@ -117,6 +120,7 @@ update_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
   const int ntiles = p.tilesM * p.tilesN;
   const int my_tiles = pair < ntiles ? (ntiles - 1 - pair) / npairs + 1 : 0;
   const int numK = p.nseg * p.kseg;
+  constexpr bool MN = !TF32;                   // the operands are MN-major
 
   if (threadIdx.x == 0) {
     for (int i = 0; i < kStages; ++i) { mbar_init(&full[i], 1); mbar_init(&empty[i], 1); }
@@ -149,10 +153,19 @@ update_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
             if (!mbar_wait(&empty[s], ph ^ 1, abort_flag)) { ok = false; break; }
             if (rank == 0) mbar_expect_tx(&full[s], 2 * kStageBytes);
             const uint32_t full_leader = mapa_u32(smem_u32(&full[s]), 0);
-            const int xa = (seg == 0 ? p.a_off0 : seg == 1 ? p.a_off1 : p.a_off2) + kl * (TF32 ? UK / 2 : UK);
-            const int xb = (seg == 0 ? p.b_off0 : seg == 1 ? p.b_off1 : p.b_off2) + kl * (TF32 ? UK / 2 : UK);
-            tma_load_2d_pair(sA + s * kBytesA, &tmA, xa, m0 + static_cast<int>(rank) * UM, full_leader, pol_norm);
-            tma_load_2d_pair(sB + s * kBytesB, &tmB, xb, n0 + static_cast<int>(rank) * (UN / 2), full_leader, pol_keep);
+            const int xa = seg == 0 ? p.a_off0 : seg == 1 ? p.a_off1 : p.a_off2;
+            const int xb = seg == 0 ? p.b_off0 : seg == 1 ? p.b_off1 : p.b_off2;
+            const int ma = m0 + static_cast<int>(rank) * UM, nb = n0 + static_cast<int>(rank) * (UN / 2);
+            if (MN) {                          // two boxes of 64 rows (columns) of W x 64 pairs per operand
+#pragma unroll
+              for (int h = 0; h < 2; ++h) {
+                tma_load_2d_pair(sA + s * kBytesA + h * (kBytesA / 2), &tmA, xa + ma + 64 * h, kl * UK, full_leader, pol_norm);
+                tma_load_2d_pair(sB + s * kBytesB + h * (kBytesB / 2), &tmB, xb + nb + 64 * h, kl * UK, full_leader, pol_keep);
+              }
+            } else {
+              tma_load_2d_pair(sA + s * kBytesA, &tmA, xa + kl * (UK / 2), ma, full_leader, pol_norm);
+              tma_load_2d_pair(sB + s * kBytesB, &tmB, xb + kl * (UK / 2), nb, full_leader, pol_keep);
+            }
           }
         }
       }
@@ -160,7 +173,7 @@ update_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
   } else if (warp == 1) {
     // ---------------- MMA issuer: one thread of the leader CTA drives both SMs ----------------
     if (lane == 0 && rank == 0) {
-      const uint32_t idesc = TF32 ? umma_idesc_tf32(2 * UM, UN) : umma_idesc_bf16(2 * UM, UN);
+      const uint32_t idesc = TF32 ? umma_idesc_tf32(2 * UM, UN) : umma_idesc_bf16(2 * UM, UN) | kIdescMnMajor;
       uint32_t it = 0;
       bool ok = true;
       for (int tl = 0; tl < my_tiles && ok; ++tl) {
@@ -172,11 +185,11 @@ update_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
           const uint32_t s = it % kStages, ph = (it / kStages) & 1;
           if (!mbar_wait(&full[s], ph, abort_flag)) { ok = false; break; }
           tc_fence_after();
-          const uint64_t da = umma_desc_k128(smem_u32(sA + s * kBytesA));
-          const uint64_t db = umma_desc_k128(smem_u32(sB + s * kBytesB));
+          const uint64_t da = MN ? umma_desc_mn128(smem_u32(sA + s * kBytesA)) : umma_desc_k128(smem_u32(sA + s * kBytesA));
+          const uint64_t db = MN ? umma_desc_mn128(smem_u32(sB + s * kBytesB)) : umma_desc_k128(smem_u32(sB + s * kBytesB));
 #pragma unroll
-          for (int k = 0; k < UK / UMMA_K; ++k) {          // four MMAs of 32 bytes of contraction each, either kind
-            const uint64_t adv = static_cast<uint64_t>(k * UMMA_K * 2 / 16);
+          for (int k = 0; k < UK / UMMA_K; ++k) {          // four MMAs of 16 pairs (bf16) or 8 (tf32) each
+            const uint64_t adv = static_cast<uint64_t>(MN ? k * 2048 / 16 : k * 32 / 16);
             if (TF32) umma_tf32_pair(d_tmem, da + adv, db + adv, idesc, (kb | k) != 0 ? 1u : 0u);
             else umma_bf16_pair(d_tmem, da + adv, db + adv, idesc, (kb | k) != 0 ? 1u : 0u);
           }
@@ -500,18 +513,21 @@ int tc_update(sfb_ctx* ctx) {
   const TcState* st = static_cast<const TcState*>(ctx->tc);
   const Layout& L = ctx->lay;
   const bool split = c.model != SFB_MLR;
-  const int64_t kw = split ? 2 * L.Kp : ctx->K;       // operand width in elements; pitch is Kp or 2*Kp
-  const int64_t pitch = (split ? 2 * L.Kp : L.Kp) * 2;
+  // U and V pair-major; the split products have (hi | lo) halves side by side
+  const int64_t ldu = split ? 2 * L.rowsp : L.ldp, ldv = split ? 2 * L.colsp : L.colsb;
+  const int64_t wu = split ? 2 * L.rowsp : c.rows, wv = split ? 2 * L.colsp : c.cols;
+  __nv_bfloat16* U = ctx->at<__nv_bfloat16>(split ? L.Rs : L.P);
+  __nv_bfloat16* V = split ? tc_split_v(ctx) : ctx->at<__nv_bfloat16>(L.Xb);
   CUtensorMap ma, mb, mc;
-  if (!make_map(st, &ma, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, ctx->at<__nv_bfloat16>(L.UT), kw, c.rows, pitch, UK, UM) ||
-      !make_map(st, &mb, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, ctx->at<__nv_bfloat16>(L.VT), kw, c.cols, pitch, UK, UN / 2) ||
+  if (!make_map(st, &ma, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, U, wu, ctx->K, ldu * 2, 64, UK) ||
+      !make_map(st, &mb, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, V, wv, ctx->K, ldv * 2, 64, UK) ||
       !make_map(st, &mc, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, ctx->W, c.cols, c.rows, c.cols * 4, kChunk, 32))
     return SFB_ERR_CUDA;
   UpdParams p{};
   p.rows = static_cast<int32_t>(c.rows); p.cols = static_cast<int32_t>(c.cols);
   p.tilesM = static_cast<int32_t>((c.rows + 2 * UM - 1) / (2 * UM));
   p.tilesN = static_cast<int32_t>((c.cols + UN - 1) / UN);
-  p.kseg = static_cast<int32_t>(L.Kp / UK);
+  p.kseg = static_cast<int32_t>((ctx->K + UK - 1) / UK);
   p.alpha = -ctx->step;
   p.prox_kind = ctx->prox_kind; p.prox_a = ctx->prox_a;
   p.status = ctx->at<uint32_t>(L.status);
@@ -520,8 +536,8 @@ int tc_update(sfb_ctx* ctx) {
   if (split) {
     // U^T V = Uhi Vhi + Uhi Vlo + Ulo Vhi (+ Ulo Vlo, dropped: 2^-16 of the product)
     p.nseg = 3;
-    p.a_off0 = 0; p.a_off1 = 0; p.a_off2 = static_cast<int32_t>(L.Kp);
-    p.b_off0 = 0; p.b_off1 = static_cast<int32_t>(L.Kp); p.b_off2 = 0;
+    p.a_off0 = 0; p.a_off1 = 0; p.a_off2 = static_cast<int32_t>(L.rowsp);
+    p.b_off0 = 0; p.b_off1 = static_cast<int32_t>(L.colsp); p.b_off2 = 0;
     p.shadow = nullptr; p.shadow_ld = 0;
     update_pair_kernel<0><<<grid, kThreads, kSmem, ctx->stream>>>(ma, mb, mc, p);
     count_launch();
