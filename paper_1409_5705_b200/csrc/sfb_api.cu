@@ -97,6 +97,13 @@ using namespace sfb;
     }                                                   \
   } while (0)
 
+// The phase that begins now (0 the step, 1 its gather, 2 its update) takes the time of the next kernel that can stamp it.
+static void begin_phase(sfb_ctx* ctx, int phase) {
+  unsigned long long* at = &ctx->at<Scalars>(ctx->lay.scalars)->ns[phase];
+  if (ctx->pending.n > 0 && ctx->pending.at + ctx->pending.n == at) ctx->pending.n += 1;     // nothing ran in between
+  else ctx->pending = Stamp{at, 1};
+}
+
 static bool al16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
 static int check_config(const sfb_config* c) {
@@ -177,11 +184,8 @@ extern "C" int sfb_init(const sfb_config* cfg, float* W_dev, void* workspace_dev
   ctx->last_cuda = 0;
   ctx->stats = sfb_stats{};
   ctx->tc = nullptr;
-  for (auto& e : ctx->ev) e = nullptr;
-  for (auto& e : ctx->ev) {
-    cudaError_t ce = cudaEventCreate(&e);
-    if (ce != cudaSuccess) { sfb_destroy(ctx); return SFB_ERR_CUDA; }
-  }
+  ctx->labels = sfb_ctx::kLabelsNone;
+  ctx->pending = Stamp{};
   // status word, scalars and per-sample losses are the first three (contiguous) regions
   cudaError_t ce = cudaMemsetAsync(ctx->ws + lay.status, 0, lay.stageX - lay.status, ctx->stream);
   if (ce != cudaSuccess) { sfb_destroy(ctx); return SFB_ERR_CUDA; }
@@ -199,8 +203,6 @@ extern "C" int sfb_init(const sfb_config* cfg, float* W_dev, void* workspace_dev
 
 extern "C" int sfb_destroy(sfb_ctx* ctx) {
   if (!ctx) return SFB_ERR_ARG;
-  for (auto& e : ctx->ev)
-    if (e) cudaEventDestroy(e);
   tc_destroy(ctx);
   delete ctx;
   return SFB_OK;
@@ -220,7 +222,7 @@ static int factors_fp32(sfb_ctx* ctx, int64_t off, int64_t n, const float* X, co
   cudaStream_t s = ctx->stream;
   EpiArgs e{};
   if (c.model == SFB_MLR || c.model == SFB_DML) {
-    CK(pack_copy(s, V, X, c.model == SFB_DML ? Y : nullptr, n * cols));                 // v = x | x - y
+    CK(pack_copy(s, V, X, c.model == SFB_DML ? Y : nullptr, n * cols, take_stamp(ctx)));      // v = x | x - y
     e.C = U; e.ldc = ldu;
     if (sparse_fwd) {                                                                   // z_i = W v_i over the non-zeros of v_i
       const int rc = sparse_forward(ctx, off, n, ctx->at<float>(ctx->lay.U), ldu);
@@ -280,6 +282,7 @@ static int begin_step(sfb_ctx* ctx) {
     if (rc) return rc;
   }
   if (c.model != SFB_SC) return SFB_OK;
+  CK(stamp(ctx->stream, take_stamp(ctx)));
   float* G = ctx->lay.G ? ctx->at<float>(ctx->lay.G) : nullptr;
   if (c.precision == SFB_PREC_FP32 && G) {
     EpiArgs e{};
@@ -299,6 +302,7 @@ static int update_fp32(sfb_ctx* ctx) {
   EpiArgs e{};
   e.C = ctx->W; e.ldc = c.cols; e.alpha = -ctx->step;
   e.prox_kind = ctx->prox_kind; e.prox_a = ctx->prox_a;
+  e.begin = take_stamp(ctx); e.end = &ctx->at<Scalars>(ctx->lay.scalars)->ns[3];
   CK(sgemm(ctx->stream, false, false, EPI_RMW, c.rows, c.cols, ctx->K, ctx->at<float>(ctx->lay.U), ctx->lay.ldu,
            ctx->at<float>(ctx->lay.V), c.cols, e));
   return SFB_OK;
@@ -313,8 +317,9 @@ static int check_inputs(sfb_ctx* ctx, const float* X, const float* Y, const int3
   return SFB_OK;
 }
 
-extern "C" int sfb_compute_factors(sfb_ctx* ctx, int32_t worker, const float* X_dev, const float* Y_dev,
-                                   const int32_t* labels_dev) {
+// fused: the call belongs to one that goes on to the update.
+static int compute_factors(sfb_ctx* ctx, int32_t worker, const float* X_dev, const float* Y_dev, const int32_t* labels_dev,
+                           bool fused) {
   int rc = check_inputs(ctx, X_dev, Y_dev, labels_dev);
   if (rc) return rc;
   const sfb_config& c = ctx->cfg;
@@ -325,7 +330,7 @@ extern "C" int sfb_compute_factors(sfb_ctx* ctx, int32_t worker, const float* X_
   if (ctx->committed == 0) {
     ctx->sparse_mask = 0;
     ctx->csr_fill = 0;
-    CK(cudaEventRecord(ctx->ev[0], ctx->stream));
+    begin_phase(ctx, 0);
     ctx->begun = false;
   }
   if (!ctx->begun) {
@@ -336,7 +341,7 @@ extern "C" int sfb_compute_factors(sfb_ctx* ctx, int32_t worker, const float* X_
   // carry each value as a (hi, lo) pair of bf16 (fp32-class products)
   rc = ctx->tf32 ? tc32_factors(ctx, off, n, X_dev, labels_dev, nullptr, 0.f)
        : c.precision == SFB_PREC_FP32 ? factors_fp32(ctx, off, n, X_dev, Y_dev, labels_dev)
-                                      : tc_factors(ctx, off, n, X_dev, Y_dev, labels_dev);
+                                      : tc_factors(ctx, off, n, X_dev, Y_dev, labels_dev, fused);
   if (rc) return rc;
   const uint64_t all = c.workers == 64 ? ~0ull : ((1ull << c.workers) - 1);
   ctx->committed |= worker < 0 ? all : (1ull << worker);
@@ -345,12 +350,17 @@ extern "C" int sfb_compute_factors(sfb_ctx* ctx, int32_t worker, const float* X_
   return SFB_OK;
 }
 
+extern "C" int sfb_compute_factors(sfb_ctx* ctx, int32_t worker, const float* X_dev, const float* Y_dev,
+                                   const int32_t* labels_dev) {
+  return compute_factors(ctx, worker, X_dev, Y_dev, labels_dev, false);
+}
+
 // ---------------------------------------------------------------------------------------------------------
 // Samples in compressed-sparse-row form (MLR): scattered for the dense forward product, and kept as triples for the
 // column-major form that the update reads
 // ---------------------------------------------------------------------------------------------------------
-extern "C" int sfb_compute_factors_csr(sfb_ctx* ctx, int32_t worker, const int64_t* indptr_dev, const int32_t* indices_dev,
-                                       const float* values_dev, int64_t nnz, const int32_t* labels_dev) {
+static int compute_factors_csr(sfb_ctx* ctx, int32_t worker, const int64_t* indptr_dev, const int32_t* indices_dev,
+                               const float* values_dev, int64_t nnz, const int32_t* labels_dev, bool fused) {
   if (!ctx || !indptr_dev || !labels_dev || nnz < 0) return SFB_ERR_ARG;
   if (nnz > 0 && (!indices_dev || !values_dev)) return SFB_ERR_ARG;
   const sfb_config& c = ctx->cfg;
@@ -367,13 +377,13 @@ extern "C" int sfb_compute_factors_csr(sfb_ctx* ctx, int32_t worker, const int64
   if (ctx->csr_fill + nnz > c.csr_nnz_max) return SFB_ERR_SHAPE;
   const int64_t off = worker < 0 ? 0 : static_cast<int64_t>(worker) * c.batch;
   const int64_t n = worker < 0 ? ctx->K : c.batch;
-  if (ctx->committed == 0) CK(cudaEventRecord(ctx->ev[0], ctx->stream));
+  if (ctx->committed == 0) begin_phase(ctx, 0);
   int rc = sparse_stage(ctx, off, n, indptr_dev, indices_dev, values_dev, nnz);
   if (rc) return rc;
   const float* X = ctx->at<float>(ctx->lay.stageX) + off * c.cols;
   rc = ctx->tf32 ? tc32_factors(ctx, off, n, X, labels_dev, nullptr, 0.f)
        : c.precision == SFB_PREC_FP32 ? factors_fp32(ctx, off, n, X, nullptr, labels_dev, sparse_forward_rows(ctx, n) > 0)
-                                      : tc_factors(ctx, off, n, X, nullptr, labels_dev);
+                                      : tc_factors(ctx, off, n, X, nullptr, labels_dev, fused);
   if (rc) return rc;
   ctx->csr_fill += nnz;
   ctx->sparse_mask |= bits;
@@ -382,11 +392,16 @@ extern "C" int sfb_compute_factors_csr(sfb_ctx* ctx, int32_t worker, const int64
   return SFB_OK;
 }
 
+extern "C" int sfb_compute_factors_csr(sfb_ctx* ctx, int32_t worker, const int64_t* indptr_dev, const int32_t* indices_dev,
+                                       const float* values_dev, int64_t nnz, const int32_t* labels_dev) {
+  return compute_factors_csr(ctx, worker, indptr_dev, indices_dev, values_dev, nnz, labels_dev, false);
+}
+
 extern "C" int sfb_step_csr(sfb_ctx* ctx, const int64_t* indptr_dev, const int32_t* indices_dev, const float* values_dev,
                             int64_t nnz, const int32_t* labels_dev) {
   if (!ctx) return SFB_ERR_ARG;
   ctx->committed = 0;
-  int rc = sfb_compute_factors_csr(ctx, -1, indptr_dev, indices_dev, values_dev, nnz, labels_dev);
+  int rc = compute_factors_csr(ctx, -1, indptr_dev, indices_dev, values_dev, nnz, labels_dev, true);
   if (rc) return rc;
   rc = sfb_gather_factors(ctx);
   if (rc) return rc;
@@ -417,7 +432,7 @@ extern "C" int sfb_forward_partials(sfb_ctx* ctx, const float* X_dev, const int3
   ctx->sparse_mask = 0;
   ctx->csr_fill = 0;
   ctx->gathered = false;
-  CK(cudaEventRecord(ctx->ev[0], ctx->stream));
+  begin_phase(ctx, 0);
   if (c.precision == SFB_PREC_BF16 || ctx->tf32) {
     rc = ctx->tf32 ? tc32_forward_partials(ctx, X_dev, labels_dev, partials_dev)
                    : tc_forward_partials(ctx, X_dev, labels_dev, partials_dev);
@@ -426,7 +441,7 @@ extern "C" int sfb_forward_partials(sfb_ctx* ctx, const float* X_dev, const int3
     const int64_t K = ctx->K;
     float* V = ctx->at<float>(ctx->lay.V);
     float* U = ctx->at<float>(ctx->lay.U);
-    CK(pack_copy(ctx->stream, V, X_dev, nullptr, K * c.cols));                                    // v = x
+    CK(pack_copy(ctx->stream, V, X_dev, nullptr, K * c.cols, take_stamp(ctx)));                                    // v = x
     EpiArgs e{};
     const int64_t ldu = ctx->lay.ldu;
     e.C = U; e.ldc = ldu;
@@ -454,13 +469,13 @@ extern "C" int sfb_forward_partials_pairs(sfb_ctx* ctx, const float* X_dev, cons
   ctx->sparse_mask = 0;
   ctx->csr_fill = 0;
   ctx->gathered = false;
-  CK(cudaEventRecord(ctx->ev[0], ctx->stream));
+  begin_phase(ctx, 0);
   // the flags are kept for the finish (the caller's buffer may change before it)
   CK(cudaMemcpyAsync(ctx->at<int32_t>(ctx->lay.stageL), similar_dev, static_cast<size_t>(ctx->K) * 4, cudaMemcpyDeviceToDevice,
                      ctx->stream));
   if ((rc = begin_step(ctx)) != SFB_OK) return rc;
   rc = c.precision == SFB_PREC_FP32 ? factors_fp32(ctx, 0, ctx->K, X_dev, Y_dev, similar_dev, false, partials_dev)
-                                    : tc_factors(ctx, 0, ctx->K, X_dev, Y_dev, similar_dev, partials_dev);
+                                    : tc_factors(ctx, 0, ctx->K, X_dev, Y_dev, similar_dev, false, partials_dev);
   if (rc) return rc;
   ctx->partials_ready = true;
   return SFB_OK;
@@ -506,7 +521,7 @@ extern "C" int sfb_set_factors(sfb_ctx* ctx, int32_t worker, const float* U_dev,
   if (worker < 0 || worker >= c.workers) return SFB_ERR_SHAPE;
   if (ctx->sdca) return SFB_ERR_UNSUPPORTED;
   if (ctx->partials_ready) return SFB_ERR_STATE;
-  if (ctx->committed == 0) CK(cudaEventRecord(ctx->ev[0], ctx->stream));
+  if (ctx->committed == 0) begin_phase(ctx, 0);
   const int64_t off = static_cast<int64_t>(worker) * c.batch;
   if (c.precision == SFB_PREC_BF16 && c.model == SFB_MLR) {
     const int rc = tc_import_factors(ctx, off, c.batch, U_dev, V_dev);
@@ -566,21 +581,24 @@ extern "C" int sfb_gather_factors(sfb_ctx* ctx) {
   const sfb_config& c = ctx->cfg;
   const uint64_t all = c.workers == 64 ? ~0ull : ((1ull << c.workers) - 1);
   if (ctx->committed != all) return SFB_ERR_STATE;
-  CK(cudaEventRecord(ctx->ev[1], ctx->stream));
+  begin_phase(ctx, 1);
   // Every worker wrote its pairs at row offset p*B of the shared buffers, so the gathered operands are
   // complete; what remains is the per-step read-out over all K pairs.
   // all K samples sparse: the v become their column-major form (and the dense update operands are not needed)
   ctx->sparse_v = c.model == SFB_MLR && c.csr_nnz_max > 0 && ctx->sparse_mask == all && sparse_update_wanted(ctx);
   if (ctx->sparse_v) {
+    CK(stamp(ctx->stream, take_stamp(ctx)));
     int rc = sparse_build_csc(ctx);
     if (rc) return rc;
   } else if (ctx->tf32) {
+    CK(stamp(ctx->stream, take_stamp(ctx)));
     int rc = tc32_gather(ctx);
     if (rc) return rc;
   }
-  if (c.model == SFB_MLR)
+  if (c.model == SFB_MLR && c.precision == SFB_PREC_FP32) {        // (bf16 mode: with the label rows)
     CK(mean_of(ctx->stream, ctx->at<float>(ctx->lay.loss), ctx->K,
-               &ctx->at<Scalars>(ctx->lay.scalars)->loss_mean));
+               &ctx->at<Scalars>(ctx->lay.scalars)->loss_mean, take_stamp(ctx)));
+  }
   // bytes per gathered value: fp32, bf16, or a (hi, lo) pair of bf16 for the split operands of DML and SC
   const double esz = (c.precision == SFB_PREC_FP32 || c.model != SFB_MLR) ? 4.0 : 2.0;
   // sparse v: 8 bytes (index, value) per non-zero instead of cols values per sample
@@ -590,14 +608,15 @@ extern "C" int sfb_gather_factors(sfb_ctx* ctx) {
   ctx->stats.gather_bytes_p2p += static_cast<double>(c.workers) * (c.workers - 1) * c.batch * pair;
   ctx->stats.dense_sync_bytes += static_cast<double>(c.workers) * c.rows * c.cols * 4.0;
   ctx->gathered = true;
-  CK(cudaEventRecord(ctx->ev[2], ctx->stream));
+  begin_phase(ctx, 2);
   return SFB_OK;
 }
 
 static int apply_prox(sfb_ctx* ctx) {
   const sfb_config& c = ctx->cfg;
   if (c.model == SFB_SC && c.sc_prox == 1)
-    CK(prox_unit_columns(ctx->stream, ctx->W, c.rows, c.cols, ctx->at<float>(ctx->lay.colpart)));
+    CK(prox_unit_columns(ctx->stream, ctx->W, c.rows, c.cols, ctx->at<float>(ctx->lay.colpart),
+                         &ctx->at<Scalars>(ctx->lay.scalars)->ns[3]));
   return SFB_OK;
 }
 
@@ -610,7 +629,6 @@ extern "C" int sfb_apply_update(sfb_ctx* ctx) {
   ctx->stats.flops += 2.0 * c.rows * c.cols * ctx->K;
   rc = apply_prox(ctx);
   if (rc) return rc;
-  CK(cudaEventRecord(ctx->ev[3], ctx->stream));
   ctx->committed = 0;
   ctx->begun = false;
   ctx->sparse_mask = 0;               // the next step starts with no sparse samples staged
@@ -635,8 +653,8 @@ extern "C" int sfb_sdca_set_dual(sfb_ctx* ctx, float* Q_dev, int64_t n_samples) 
   return SFB_OK;
 }
 
-extern "C" int sfb_sdca_compute_factors(sfb_ctx* ctx, int32_t worker, const float* X_dev, const int32_t* labels_dev,
-                                        const int32_t* sample_ids_dev) {
+static int sdca_compute_factors(sfb_ctx* ctx, int32_t worker, const float* X_dev, const int32_t* labels_dev,
+                                const int32_t* sample_ids_dev, bool fused) {
   if (!ctx || !X_dev || !labels_dev || !sample_ids_dev) return SFB_ERR_ARG;
   if (!ctx->sdca) return SFB_ERR_UNSUPPORTED;
   if (!ctx->dualQ) return SFB_ERR_STATE;
@@ -645,7 +663,7 @@ extern "C" int sfb_sdca_compute_factors(sfb_ctx* ctx, int32_t worker, const floa
   if (worker < -1 || worker >= c.workers) return SFB_ERR_SHAPE;
   const int64_t off = worker < 0 ? 0 : static_cast<int64_t>(worker) * c.batch;
   const int64_t n = worker < 0 ? ctx->K : c.batch;
-  if (ctx->committed == 0) CK(cudaEventRecord(ctx->ev[0], ctx->stream));
+  if (ctx->committed == 0) begin_phase(ctx, 0);
   const float inv_lam_n = static_cast<float>(1.0 / (static_cast<double>(c.sdca_lambda) * static_cast<double>(c.sdca_n)));
   uint32_t* status = ctx->at<uint32_t>(ctx->lay.status);
   float* loss = ctx->at<float>(ctx->lay.loss) + off;
@@ -656,7 +674,7 @@ extern "C" int sfb_sdca_compute_factors(sfb_ctx* ctx, int32_t worker, const floa
     float* V = ctx->at<float>(ctx->lay.V) + off * c.cols;
     const int64_t ldu = ctx->lay.ldu;
     float* U = ctx->at<float>(ctx->lay.U) + off * ldu;
-    CK(pack_copy(ctx->stream, V, X_dev, nullptr, n * c.cols));                                        // v = a_i
+    CK(pack_copy(ctx->stream, V, X_dev, nullptr, n * c.cols, take_stamp(ctx)));                                        // v = a_i
     EpiArgs e{};
     e.C = U; e.ldc = ldu;
     CK(sgemm(ctx->stream, true, true, EPI_STORE, n, c.rows, c.cols, V, c.cols, ctx->W, c.cols, e, ctx->K));   // z_i = W a_i
@@ -664,7 +682,7 @@ extern "C" int sfb_sdca_compute_factors(sfb_ctx* ctx, int32_t worker, const floa
     CK(sdca_dual_rows(ctx->stream, U, n, c.rows, ldu, X_dev, c.cols, labels_dev, sample_ids_dev, ctx->dualQ, ctx->dual_n,
                       inv_lam_n, c.eta, nullptr, loss, status));                                      // u_i = du_i
   } else {
-    const int rc = tc_sdca_factors(ctx, off, n, X_dev, labels_dev, sample_ids_dev, inv_lam_n);
+    const int rc = tc_sdca_factors(ctx, off, n, X_dev, labels_dev, sample_ids_dev, inv_lam_n, fused);
     if (rc) return rc;
   }
   const uint64_t all = c.workers == 64 ? ~0ull : ((1ull << c.workers) - 1);
@@ -673,10 +691,15 @@ extern "C" int sfb_sdca_compute_factors(sfb_ctx* ctx, int32_t worker, const floa
   return SFB_OK;
 }
 
+extern "C" int sfb_sdca_compute_factors(sfb_ctx* ctx, int32_t worker, const float* X_dev, const int32_t* labels_dev,
+                                        const int32_t* sample_ids_dev) {
+  return sdca_compute_factors(ctx, worker, X_dev, labels_dev, sample_ids_dev, false);
+}
+
 extern "C" int sfb_sdca_step(sfb_ctx* ctx, const float* X_dev, const int32_t* labels_dev, const int32_t* sample_ids_dev) {
   if (!ctx) return SFB_ERR_ARG;
   ctx->committed = 0;
-  int rc = sfb_sdca_compute_factors(ctx, -1, X_dev, labels_dev, sample_ids_dev);
+  int rc = sdca_compute_factors(ctx, -1, X_dev, labels_dev, sample_ids_dev, true);
   if (rc) return rc;
   rc = sfb_gather_factors(ctx);
   if (rc) return rc;
@@ -694,20 +717,19 @@ extern "C" int sfb_replay_update(sfb_ctx* ctx) {
   if (!ctx) return SFB_ERR_ARG;
   if (ctx->stats.steps < 1 || ctx->committed != 0 || ctx->partials_ready) return SFB_ERR_STATE;
   const sfb_config& c = ctx->cfg;
-  CK(cudaEventRecord(ctx->ev[2], ctx->stream));
+  begin_phase(ctx, 2);
   int rc = ctx->tf32 ? tc32_update(ctx) : c.precision == SFB_PREC_FP32 ? update_fp32(ctx) : tc_update(ctx);
   if (rc) return rc;
   ctx->stats.flops += 2.0 * c.rows * c.cols * ctx->K;
   rc = apply_prox(ctx);
   if (rc) return rc;
-  CK(cudaEventRecord(ctx->ev[3], ctx->stream));
   return SFB_OK;
 }
 
 extern "C" int sfb_step(sfb_ctx* ctx, const float* X_dev, const float* Y_dev, const int32_t* labels_dev) {
   if (!ctx) return SFB_ERR_ARG;
   ctx->committed = 0;
-  int rc = sfb_compute_factors(ctx, -1, X_dev, Y_dev, labels_dev);
+  int rc = compute_factors(ctx, -1, X_dev, Y_dev, labels_dev, true);
   if (rc) return rc;
   rc = sfb_gather_factors(ctx);
   if (rc) return rc;
@@ -758,6 +780,7 @@ extern "C" int sfb_dense_sync_step(sfb_ctx* ctx, const float* X_dev, const float
   float* one = scratch_dev + mat;
   const float* U = ctx->at<float>(ctx->lay.U);
   const float* V = ctx->at<float>(ctx->lay.V);
+  CK(stamp(ctx->stream, take_stamp(ctx)));
   for (int p = 0; p < c.workers; ++p) {
     // worker p's dense update matrix, as it would be sent to the server
     EpiArgs e{};
@@ -768,10 +791,10 @@ extern "C" int sfb_dense_sync_step(sfb_ctx* ctx, const float* X_dev, const float
   }
   CK(axpy(ctx->stream, ctx->W, sum, -c.eta, static_cast<int64_t>(mat)));                 // W <- W - eta * sum_p dW_p
   CK(prox_entries(ctx->stream, ctx->W, static_cast<int64_t>(mat), ctx->prox_kind, ctx->prox_a));
+  CK(stamp(ctx->stream, Stamp{&ctx->at<Scalars>(ctx->lay.scalars)->ns[3], 1}));
   ctx->stats.flops += 2.0 * c.rows * c.cols * ctx->K;
   rc = apply_prox(ctx);
   if (rc) return rc;
-  CK(cudaEventRecord(ctx->ev[3], ctx->stream));
   ctx->committed = 0;
   ctx->begun = false;
   ctx->gathered = false;
@@ -815,13 +838,12 @@ extern "C" int sfb_get_stats(sfb_ctx* ctx, sfb_stats* out) {
   if (!ctx || !out) return SFB_ERR_ARG;
   CK(cudaStreamSynchronize(ctx->stream));
   if (ctx->stats.steps > 0) {
-    float ms = 0.f;
-    if (cudaEventElapsedTime(&ms, ctx->ev[0], ctx->ev[1]) == cudaSuccess) ctx->stats.ms_factors = ms;
-    if (cudaEventElapsedTime(&ms, ctx->ev[1], ctx->ev[2]) == cudaSuccess) ctx->stats.ms_gather = ms;
-    if (cudaEventElapsedTime(&ms, ctx->ev[2], ctx->ev[3]) == cudaSuccess) ctx->stats.ms_update = ms;
-    cudaGetLastError();
     Scalars h{};
     CK(cudaMemcpy(&h, ctx->at<Scalars>(ctx->lay.scalars), sizeof(h), cudaMemcpyDeviceToHost));
+    auto ms = [&](int from, int to) { return h.ns[to] > h.ns[from] ? static_cast<float>(h.ns[to] - h.ns[from]) * 1e-6f : 0.f; };
+    ctx->stats.ms_factors = ms(0, 1);
+    ctx->stats.ms_gather = ms(1, 2);
+    ctx->stats.ms_update = ms(2, 3);
     ctx->stats.last_loss = h.loss_mean;
     ctx->stats.sc_lipschitz = h.L;
     ctx->stats.copy_pieces = static_cast<int64_t>(h.copy_pieces);

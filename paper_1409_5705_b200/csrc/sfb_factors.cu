@@ -7,6 +7,12 @@
 
 #include "sfb_internal.h"
 
+#define SFB_TRY(call)                         \
+  do {                                        \
+    const cudaError_t e__ = (call);           \
+    if (e__ != cudaSuccess) return e__;       \
+  } while (0)
+
 namespace sfb {
 namespace {
 
@@ -53,7 +59,10 @@ __device__ __forceinline__ float block_max(float v, float* sh) {
 
 // v = x (MLR) or v = x - y (DML pair difference, Section 2), 16-byte vectors with a scalar tail.
 __global__ void pack_kernel(float* __restrict__ dst, const float* __restrict__ x, const float* __restrict__ y,
-                            int64_t n4, int64_t n) {
+                            int64_t n4, int64_t n, const Stamp st) {
+  pdl_launch_dependents();
+  pdl_wait();
+  stamp_begin(st);
   const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
   for (int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; i < n4; i += stride) {
     float4 a = reinterpret_cast<const float4*>(x)[i];
@@ -68,17 +77,23 @@ __global__ void pack_kernel(float* __restrict__ dst, const float* __restrict__ x
 }
 
 __global__ void zero_kernel(float* __restrict__ dst, int64_t n) {
+  pdl_launch_dependents();
+  pdl_wait();
   const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
   for (int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; i < n; i += stride) dst[i] = 0.f;
 }
 
 __global__ void prox_entries_kernel(float* __restrict__ w, int64_t n, int kind, float a) {
+  pdl_launch_dependents();
+  pdl_wait();
   const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
   for (int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; i < n; i += stride)
     w[i] = prox_entry(w[i], kind, a);
 }
 
 __global__ void axpy_kernel(float* __restrict__ y, const float* __restrict__ x, float alpha, int64_t n) {
+  pdl_launch_dependents();
+  pdl_wait();
   const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
   for (int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; i < n; i += stride)
     y[i] = fmaf(alpha, x[i], y[i]);
@@ -91,6 +106,8 @@ template <int NTHREADS>
 __global__ void __launch_bounds__(NTHREADS) mlr_softmax_kernel(float* __restrict__ Z, int64_t rows, int64_t ldz,
                                                                const int32_t* __restrict__ labels,
                                                                float* __restrict__ loss, uint32_t* status) {
+  pdl_launch_dependents();
+  pdl_wait();
   __shared__ float sh[32];
   float* z = Z + static_cast<int64_t>(blockIdx.x) * ldz;
   float m = -INFINITY;
@@ -123,6 +140,8 @@ template <int NTHREADS>
 __global__ void __launch_bounds__(NTHREADS) mlr_shard_partials_kernel(const float* __restrict__ Z, int64_t rows, int64_t ldz,
                                                                       const int32_t* __restrict__ labels, int64_t row_off,
                                                                       float4* __restrict__ part) {
+  pdl_launch_dependents();
+  pdl_wait();
   __shared__ float sh[32];
   const float* z = Z + static_cast<int64_t>(blockIdx.x) * ldz;
   float m = -INFINITY;
@@ -163,6 +182,8 @@ __global__ void __launch_bounds__(NTHREADS) mlr_shard_finish_kernel(float* __res
                                                                     const int32_t* __restrict__ labels, int64_t row_off,
                                                                     const float4* __restrict__ parts, int shards, int64_t K,
                                                                     float* __restrict__ loss, uint32_t* status) {
+  pdl_launch_dependents();
+  pdl_wait();
   __shared__ float sh_lse;
   float* z = Z + static_cast<int64_t>(blockIdx.x) * ldz;
   if (threadIdx.x == 0) {
@@ -210,7 +231,9 @@ __global__ void __launch_bounds__(NTHREADS) sdca_dual_kernel(float* __restrict__
                                                              const int32_t* __restrict__ ids, float* __restrict__ Q,
                                                              int64_t n_samples, float inv_lam_n, float gamma,
                                                              float* __restrict__ coef, float* __restrict__ loss,
-                                                             uint32_t* status) {
+                                                             uint32_t* status, int32_t* __restrict__ slot, int64_t off) {
+  pdl_launch_dependents();
+  pdl_wait();
   __shared__ float sh[32];
   const int64_t i = blockIdx.x;
   float* z = Z + i * ldz;
@@ -247,6 +270,7 @@ __global__ void __launch_bounds__(NTHREADS) sdca_dual_kernel(float* __restrict__
   s = block_sum<NTHREADS>(s, sh);
   sz = block_sum<NTHREADS>(sz, sh);
   const float lse = m + logf(s);
+  if (threadIdx.x == 0 && slot) atomicMin(&slot[y], static_cast<int32_t>(off + i));
   if (threadIdx.x == 0) loss[i] = (mz + logf(sz)) - z[y];        // the sample's logistic loss at the W of this step
   // safeguarded Newton on nu: G(nu) = sum_j q_j(nu) is decreasing and convex, G(lse - kappa) >= 1 >= G(lse)
   float lo = lse - kappa, hi = lse, nu = lse;
@@ -287,9 +311,12 @@ template <int NTHREADS>
 __global__ void __launch_bounds__(NTHREADS) dml_scale_kernel(float* __restrict__ Z, const float* __restrict__ Z2,
                                                              int64_t rows, int64_t ld,
                                                              const int32_t* __restrict__ similar, float margin,
-                                                             float* __restrict__ norm_out, const float* __restrict__ norms_all,
+                                                             float* __restrict__ norm_out,
+                                                             const float* __restrict__ norms_all,
                                                              int shards, int64_t nstride, __nv_bfloat16* __restrict__ split,
                                                              int64_t split_half) {
+  pdl_launch_dependents();
+  pdl_wait();
   __shared__ float sh[32];
   float* z = Z + static_cast<int64_t>(blockIdx.x) * ld;
   if (Z2) {                      // z arrives as two partial sums over halves of the contraction (fixed order: Z + Z2)
@@ -321,7 +348,10 @@ __global__ void __launch_bounds__(NTHREADS) dml_scale_kernel(float* __restrict__
   }
 }
 
-__global__ void mean_kernel(const float* __restrict__ v, int64_t n, float* out) {
+__global__ void mean_kernel(const float* __restrict__ v, int64_t n, float* out, const Stamp st) {
+  pdl_launch_dependents();
+  pdl_wait();
+  stamp_begin(st);
   __shared__ float sh[32];
   float s = 0.f;
   for (int64_t i = threadIdx.x; i < n; i += 256) s += v[i];
@@ -333,6 +363,8 @@ __global__ void mean_kernel(const float* __restrict__ v, int64_t n, float* out) 
 // rescaling multiplies every entry of W while the step's update is ~1e-3 of ||W||).
 __global__ void __launch_bounds__(kThreads) col_sumsq_kernel(const float* __restrict__ W, int64_t rows, int64_t cols,
                                                              double* __restrict__ part, int64_t slab_rows) {
+  pdl_launch_dependents();
+  pdl_wait();
   __shared__ double sh[8][128];
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
   const int64_t c0 = static_cast<int64_t>(blockIdx.x) * 128 + tx * 4;
@@ -364,7 +396,9 @@ __global__ void __launch_bounds__(kThreads) col_sumsq_kernel(const float* __rest
 // Prox of Figure 3: b <- b / ||b|| for the columns with ||b|| > 1, others untouched (bit-identical).
 __global__ void __launch_bounds__(kThreads) prox_scale_kernel(float* __restrict__ W, int64_t rows, int64_t cols,
                                                               const double* __restrict__ part, int nslabs,
-                                                              int64_t slab_rows) {
+                                                              int64_t slab_rows, unsigned long long* end) {
+  pdl_launch_dependents();
+  pdl_wait();
   __shared__ double scale[128];
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
   if (threadIdx.x < 128) {
@@ -376,6 +410,7 @@ __global__ void __launch_bounds__(kThreads) prox_scale_kernel(float* __restrict_
   }
   __syncthreads();
   const int64_t c0 = static_cast<int64_t>(blockIdx.x) * 128 + tx * 4;
+  stamp_end(end);                     // (the kernel is a single wave of short blocks)
   if (c0 >= cols) return;
   const double s0 = scale[tx * 4], s1 = scale[tx * 4 + 1], s2 = scale[tx * 4 + 2], s3 = scale[tx * 4 + 3];
   if (s0 == 1. && s1 == 1. && s2 == 1. && s3 == 1.) return;
@@ -577,7 +612,7 @@ __global__ void __launch_bounds__(kPiThreads) power_kernel(const PowerParams p) 
   }
 }
 
-__global__ void set_L_kernel(Scalars* sc, float L) { sc->L = L; sc->invL = 1.f / L; }
+__global__ void set_L_kernel(Scalars* sc, float L) { pdl_launch_dependents(); pdl_wait(); sc->L = L; sc->invL = 1.f / L; }
 
 inline unsigned grid_for(int64_t n, int per_block) {
   int64_t g = (n + per_block - 1) / per_block;
@@ -590,96 +625,86 @@ inline int64_t slab_rows_for(int64_t rows) { return (rows + kProxSlabs - 1) / kP
 
 }  // namespace
 
-cudaError_t pack_copy(cudaStream_t s, float* dst, const float* x, const float* y, int64_t n) {
+__global__ void stamp_kernel(const Stamp st) {
+  pdl_launch_dependents();
+  pdl_wait();
+  stamp_begin(st);
+}
+
+cudaError_t stamp(cudaStream_t s, const Stamp& st) {
+  if (st.n <= 0) return cudaSuccess;
+  return launch_kernel(stamp_kernel, dim3(1), dim3(32), 0, s, 1, st);
+}
+
+cudaError_t pack_copy(cudaStream_t s, float* dst, const float* x, const float* y, int64_t n, const Stamp& st) {
   if (n <= 0) return cudaSuccess;
-  pack_kernel<<<grid_for(n / 4 + 1, kThreads), kThreads, 0, s>>>(dst, x, y, n / 4, n);
-  count_launch();
-  return cudaGetLastError();
+  return launch_kernel(pack_kernel, dim3(grid_for(n / 4 + 1, kThreads)), dim3(kThreads), 0, s, 1, dst, x, y, n / 4, n, st);
 }
 
 cudaError_t fill_zero(cudaStream_t s, float* dst, int64_t n) {
   if (n <= 0) return cudaSuccess;
-  zero_kernel<<<grid_for(n, kThreads), kThreads, 0, s>>>(dst, n);
-  count_launch();
-  return cudaGetLastError();
+  return launch_kernel(zero_kernel, dim3(grid_for(n, kThreads)), dim3(kThreads), 0, s, 1, dst, n);
 }
 
 cudaError_t axpy(cudaStream_t s, float* y, const float* x, float alpha, int64_t n) {
   if (n <= 0) return cudaSuccess;
-  axpy_kernel<<<grid_for(n, kThreads), kThreads, 0, s>>>(y, x, alpha, n);
-  count_launch();
-  return cudaGetLastError();
+  return launch_kernel(axpy_kernel, dim3(grid_for(n, kThreads)), dim3(kThreads), 0, s, 1, y, x, alpha, n);
 }
 
 cudaError_t mlr_softmax_rows(cudaStream_t s, float* Z, int64_t nsamp, int64_t rows, int64_t ldz, const int32_t* labels,
                              float* loss, uint32_t* status) {
   if (nsamp <= 0) return cudaSuccess;
-  mlr_softmax_kernel<512><<<static_cast<unsigned>(nsamp), 512, 0, s>>>(Z, rows, ldz, labels, loss, status);
-  count_launch();
-  return cudaGetLastError();
+  return launch_kernel(mlr_softmax_kernel<512>, dim3(static_cast<unsigned>(nsamp)), dim3(512), 0, s, 1, Z, rows, ldz,
+                       labels, loss, status);
 }
 
 cudaError_t prox_entries(cudaStream_t s, float* w, int64_t n, int kind, float a) {
   if (n <= 0 || kind == 0) return cudaSuccess;
-  prox_entries_kernel<<<grid_for(n, kThreads), kThreads, 0, s>>>(w, n, kind, a);
-  count_launch();
-  return cudaGetLastError();
+  return launch_kernel(prox_entries_kernel, dim3(grid_for(n, kThreads)), dim3(kThreads), 0, s, 1, w, n, kind, a);
 }
 
 cudaError_t mlr_shard_partials(cudaStream_t s, const float* Z, int64_t nsamp, int64_t rows, int64_t ldz,
                                const int32_t* labels, int64_t row_off, float* part) {
   if (nsamp <= 0) return cudaSuccess;
-  mlr_shard_partials_kernel<512><<<static_cast<unsigned>(nsamp), 512, 0, s>>>(Z, rows, ldz, labels, row_off,
-                                                                           reinterpret_cast<float4*>(part));
-  count_launch();
-  return cudaGetLastError();
+  return launch_kernel(mlr_shard_partials_kernel<512>, dim3(static_cast<unsigned>(nsamp)), dim3(512), 0, s, 1, Z, rows,
+                       ldz, labels, row_off, reinterpret_cast<float4*>(part));
 }
 
 cudaError_t mlr_shard_finish(cudaStream_t s, float* Z, int64_t nsamp, int64_t rows, int64_t ldz, const int32_t* labels,
                              int64_t row_off, const float* parts, int shards, float* loss, uint32_t* status) {
   if (nsamp <= 0) return cudaSuccess;
-  mlr_shard_finish_kernel<512><<<static_cast<unsigned>(nsamp), 512, 0, s>>>(
-      Z, rows, ldz, labels, row_off, reinterpret_cast<const float4*>(parts), shards, nsamp, loss, status);
-  count_launch();
-  return cudaGetLastError();
+  return launch_kernel(mlr_shard_finish_kernel<512>, dim3(static_cast<unsigned>(nsamp)), dim3(512), 0, s, 1,  Z, rows,
+                       ldz, labels, row_off, reinterpret_cast<const float4*>(parts), shards, nsamp, loss, status);
 }
 
 cudaError_t sdca_dual_rows(cudaStream_t s, float* Z, int64_t nsamp, int64_t rows, int64_t ldz, const float* X, int64_t cols,
                            const int32_t* labels, const int32_t* ids, float* Q, int64_t n_samples, float inv_lam_n,
-                           float gamma, float* coef, float* loss, uint32_t* status) {
+                           float gamma, float* coef, float* loss, uint32_t* status, int32_t* slot, int64_t off) {
   if (nsamp <= 0) return cudaSuccess;
-  sdca_dual_kernel<512><<<static_cast<unsigned>(nsamp), 512, 0, s>>>(Z, rows, ldz, X, cols, labels, ids, Q, n_samples,
-                                                                  inv_lam_n, gamma, coef, loss, status);
-  count_launch();
-  return cudaGetLastError();
+  return launch_kernel(sdca_dual_kernel<512>, dim3(static_cast<unsigned>(nsamp)), dim3(512), 0, s, 1, Z, rows, ldz, X,
+                       cols, labels, ids, Q, n_samples, inv_lam_n, gamma, coef, loss, status, slot, off);
 }
 
 cudaError_t dml_scale_rows(cudaStream_t s, float* Z, int64_t nsamp, int64_t rows, int64_t ld,
-                           const int32_t* similar, float margin, void* split, int64_t split_half, const float* Z2, float* norm_out, const float* norms_all,
+                           const int32_t* similar, float margin, void* split, int64_t split_half, const float* Z2,
+                           float* norm_out, const float* norms_all,
                            int shards, int64_t nstride) {
   if (nsamp <= 0) return cudaSuccess;
-  dml_scale_kernel<256><<<static_cast<unsigned>(nsamp), 256, 0, s>>>(Z, Z2, rows, ld, similar, margin, norm_out, norms_all,
-                                                                     shards, nstride, static_cast<__nv_bfloat16*>(split),
-                                                                     split_half);
-  count_launch();
-  return cudaGetLastError();
+  return launch_kernel(dml_scale_kernel<256>, dim3(static_cast<unsigned>(nsamp)), dim3(256), 0, s, 1, Z, Z2, rows, ld,
+                       similar, margin, norm_out, norms_all, shards, nstride, static_cast<__nv_bfloat16*>(split),
+                       split_half);
 }
 
-cudaError_t mean_of(cudaStream_t s, const float* v, int64_t n, float* out) {
-  mean_kernel<<<1, 256, 0, s>>>(v, n, out);
-  count_launch();
-  return cudaGetLastError();
+cudaError_t mean_of(cudaStream_t s, const float* v, int64_t n, float* out, const Stamp& st) {
+  return launch_kernel(mean_kernel, dim3(1), dim3(256), 0, s, 1, v, n, out, st);
 }
 
-cudaError_t prox_unit_columns(cudaStream_t s, float* W, int64_t rows, int64_t cols, float* colpart) {
+cudaError_t prox_unit_columns(cudaStream_t s, float* W, int64_t rows, int64_t cols, float* colpart, unsigned long long* end) {
   const int64_t sr = slab_rows_for(rows);
   dim3 grid(static_cast<unsigned>((cols + 127) / 128), kProxSlabs);
   double* part = reinterpret_cast<double*>(colpart);
-  col_sumsq_kernel<<<grid, kThreads, 0, s>>>(W, rows, cols, part, sr);
-  count_launch();
-  prox_scale_kernel<<<grid, kThreads, 0, s>>>(W, rows, cols, part, kProxSlabs, sr);
-  count_launch();
-  return cudaGetLastError();
+  SFB_TRY(launch_kernel(col_sumsq_kernel, grid, dim3(kThreads), 0, s, 1, W, rows, cols, part, sr));
+  return launch_kernel(prox_scale_kernel, grid, dim3(kThreads), 0, s, 1, W, rows, cols, part, kProxSlabs, sr, end);
 }
 
 size_t power_scratch_bytes(int64_t cols) {
@@ -717,9 +742,7 @@ cudaError_t estimate_lipschitz(cudaStream_t s, const float* W, const float* G, i
 }
 
 cudaError_t set_lipschitz(cudaStream_t s, Scalars* sc, float L) {
-  set_L_kernel<<<1, 1, 0, s>>>(sc, L);
-  count_launch();
-  return cudaGetLastError();
+  return launch_kernel(set_L_kernel, dim3(1), dim3(1), 0, s, 1, sc, L);
 }
 
 }  // namespace sfb
@@ -781,9 +804,11 @@ extern "C" int sfb_prox_columns_noalloc(float* W_dev, int64_t rows, int64_t cols
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   const int64_t sr = sfb::slab_rows_for(rows);
   dim3 grid(static_cast<unsigned>((cols + 127) / 128), sfb::kProxSlabs);
-  sfb::col_sumsq_kernel<<<grid, sfb::kThreads, 0, s>>>(W_dev, rows, cols, part, sr);
-  sfb::count_launch();
-  sfb::prox_scale_kernel<<<grid, sfb::kThreads, 0, s>>>(W_dev, rows, cols, part, sfb::kProxSlabs, sr);
-  sfb::count_launch();
-  return cudaGetLastError() == cudaSuccess ? SFB_OK : SFB_ERR_CUDA;
+  if (sfb::launch_kernel(sfb::col_sumsq_kernel, grid, dim3(sfb::kThreads), 0, s, 1, W_dev, rows, cols, part,
+                         sr) != cudaSuccess)
+    return SFB_ERR_CUDA;
+  const cudaError_t e = sfb::launch_kernel(sfb::prox_scale_kernel, grid, dim3(sfb::kThreads), 0, s, 1, W_dev, rows, cols,
+                                           part, sfb::kProxSlabs, sr,
+                                           nullptr);
+  return e == cudaSuccess ? SFB_OK : SFB_ERR_CUDA;
 }

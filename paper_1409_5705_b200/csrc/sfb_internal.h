@@ -22,15 +22,38 @@ int sm_count();
 // programmatic stream serialisation, so that its blocks are scheduled and its set-up runs while the kernel before it
 // drains.  Every kernel launched this way calls pdl_wait() before it touches memory (it returns when the kernels before it
 // have completed and their writes are visible) and pdl_launch_dependents() early (the next kernel may then start its own
-// set-up once all blocks of this one are running).
+// set-up once all blocks of this one are running).  The tile kernels are launched this way only when they have at most one
+// tile per SM: started while the SMs fall free one by one, their blocks land on them in that order, neighbours apart, and the
+// operands that neighbours share are read across the dies (3-4 % of a step at 325,000 x 10,000).
 // ---------------------------------------------------------------------------------------------------------
+struct Stamp {                        // the first block stores the time to at[0] .. at[n - 1]
+  unsigned long long* at;
+  int32_t n;
+};
 #ifdef __CUDACC__
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
+// Time stamps of the phases of a step (sfb_stats.ms_*), written by the kernels themselves: events between them would keep a
+// kernel from being scheduled before the one ahead of it has drained.
+__device__ __forceinline__ unsigned long long global_ns() {
+  unsigned long long t;
+  asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
+  return t;
+}
+__device__ __forceinline__ void stamp_begin(const Stamp& s) {
+  if (s.n > 0 && threadIdx.x == 0 && blockIdx.x == 0 && blockIdx.y == 0) {
+    const unsigned long long t = global_ns();
+    for (int i = 0; i < s.n; ++i) s.at[i] = t;
+  }
+}
+__device__ __forceinline__ void stamp_end(unsigned long long* at) {      // the latest block's time stays
+  if (at && threadIdx.x == 0) atomicMax(at, global_ns());
+}
+
 template <typename... KArgs, typename... Args>
-cudaError_t launch_kernel(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, int cluster,
-                          const Args&... args) {
+cudaError_t launch_kernel_if(bool early, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+                             int cluster, const Args&... args) {
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = grid;
   cfg.blockDim = block;
@@ -38,7 +61,7 @@ cudaError_t launch_kernel(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_
   cfg.stream = s;
   cudaLaunchAttribute attr[2]{};
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[0].val.programmaticStreamSerializationAllowed = early ? 1 : 0;
   attr[1].id = cudaLaunchAttributeClusterDimension;
   attr[1].val.clusterDim.x = static_cast<unsigned>(cluster);
   attr[1].val.clusterDim.y = 1;
@@ -47,6 +70,11 @@ cudaError_t launch_kernel(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_
   cfg.numAttrs = cluster > 1 ? 2 : 1;
   count_launch();
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
+}
+template <typename... KArgs, typename... Args>
+cudaError_t launch_kernel(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, int cluster,
+                          const Args&... args) {
+  return launch_kernel_if(true, kernel, grid, block, smem, s, cluster, args...);
 }
 
 // The shared-memory opt-in of a kernel, once per device.
@@ -73,7 +101,7 @@ constexpr int kProxSlabs = 64;        // row slabs of the deterministic column r
 struct Layout {
   size_t status, scalars, loss, V, U, colpart, stageX, stageY, stageL;
   // bf16 tensor-core mode
-  size_t Wb, Xb, VT, ZT, UT, P, part, Xf, labels, coef, lse;   // VT, UT: tf32 words only; P: probabilities [K x ldp]
+  size_t Wb, Xb, VT, ZT, UT, P, part, Xf, labels, coef, lse, slot, dL;   // VT, UT: tf32 words only; P: probabilities [K x ldp]; slot, dL: label rows
   // bf16 mode, DML and SC: (hi | lo) bf16 operands of the split products
   size_t Ws, WTs, As, Rs;             // W by rows, W transposed, the A operand (v or the codes), the residual
   size_t U2;                          // DML: second partial of z when the forward product splits its contraction
@@ -85,6 +113,7 @@ struct Layout {
   int64_t ldu;                        // row pitch of the fp32 U buffer (rows rounded up to 4; rows itself with tf32 pairs)
   int64_t colsp, rowsp;               // cols, rows rounded up to 64
   int64_t Kp;                         // K rounded up to the contraction block of the update product
+  int32_t pw;                         // columns per softmax partial of the bf16 forward product
   int64_t ldp;                        // row pitch of P: rows rounded up to 64
   int64_t colsb;                      // cols rounded up to the contraction block of the forward product
   size_t total;
@@ -111,6 +140,7 @@ struct Scalars {                      // device-resident scalars
   float tmp;
   unsigned long long copy_pieces;     // 64-byte row pieces of the bf16 operand copy the update passes went over ...
   unsigned long long copy_written;    // ... and how many of them they had to rewrite (the others already held bf16(W))
+  unsigned long long ns[4];           // global time at the start of the step, of its gather and of its update, and at its end
 };
 
 }  // namespace sfb
@@ -141,15 +171,23 @@ struct sfb_ctx {
   bool sparse_v;                      // the gathered v are in column-major sparse form: the update sums only the non-zeros
   bool gathered;
   int last_cuda;
-  cudaEvent_t ev[4];
+  // MLR, bf16 mode: the label entries of the step's factors are not in W; in W by the factors call; were in a past update,
+  // their sums kept
+  enum Labels : int8_t { kLabelsNone, kLabelsApplied, kLabelsKept } labels;
+  sfb::Stamp pending;                 // phases whose beginning the next kernel that can will stamp
   sfb_stats stats;
   void* tc;                           // tensor-core path state (tensor maps), owned
+
+  // the stamps that the next kernel takes along (their phases begin with it)
+  sfb::Stamp take_pending() { const sfb::Stamp s = pending; pending = sfb::Stamp{}; return s; }
 
   template <typename T>
   T* at(size_t off) const { return reinterpret_cast<T*>(ws + off); }
 };
 
 namespace sfb {
+
+inline Stamp take_stamp(sfb_ctx* ctx) { return ctx->take_pending(); }
 
 // ---------------------------------------------------------------------------------------------------------
 // fp32 FMA matrix products:  C (M x N) = sum_k A(m,k) * B(n,k)  followed by an epilogue.
@@ -174,6 +212,8 @@ struct EpiArgs {
   float prox_a;
   float alpha;         // EPI_RMW
   float lam;           // EPI_ISTA, EPI_ISTA0
+  Stamp begin;         // EPI_RMW: time stamps
+  unsigned long long* end;
   float* C;            // output, row-major [M x ldc]
   int64_t ldc;
   float* C2;           // EPI_ISTA0 (may be null)
@@ -197,7 +237,8 @@ cudaError_t sgemm(cudaStream_t s, bool a_kc, bool b_kc, Epilogue epi, int64_t M,
 // ---------------------------------------------------------------------------------------------------------
 // Factor kernels (pack, softmax, pair residual, prox, power iteration)
 // ---------------------------------------------------------------------------------------------------------
-cudaError_t pack_copy(cudaStream_t s, float* dst, const float* x, const float* y_or_null, int64_t n);
+cudaError_t stamp(cudaStream_t s, const Stamp& st);
+cudaError_t pack_copy(cudaStream_t s, float* dst, const float* x, const float* y_or_null, int64_t n, const Stamp& st);
 cudaError_t fill_zero(cudaStream_t s, float* dst, int64_t n);
 cudaError_t mlr_softmax_rows(cudaStream_t s, float* Z, int64_t nsamp, int64_t rows, int64_t ldz, const int32_t* labels,
                              float* loss_per_sample, uint32_t* status);
@@ -209,10 +250,10 @@ cudaError_t mlr_shard_finish(cudaStream_t s, float* Z, int64_t nsamp, int64_t ro
                              int64_t row_off, const float* parts, int shards, float* loss, uint32_t* status);
 // SDCA (l2-regularised MLR): per sample, from its logits z (row of Z, overwritten with du), its dual row of Q (advanced
 // by gamma * du) and its features x: the change of the dual vector that minimises the dual objective.  coef (may be
-// null) receives -du at the label entry.
+// null) receives -du at the label entry; slot (may be null) the smallest index, from off on, of a sample of each class.
 cudaError_t sdca_dual_rows(cudaStream_t s, float* Z, int64_t nsamp, int64_t rows, int64_t ldz, const float* X, int64_t cols,
                            const int32_t* labels, const int32_t* ids, float* Q, int64_t n_samples, float inv_lam_n,
-                           float gamma, float* coef, float* loss, uint32_t* status);
+                           float gamma, float* coef, float* loss, uint32_t* status, int32_t* slot = nullptr, int64_t off = 0);
 // Z2 (may be null): a second partial of z (the other half of the contraction), added to Z first.  Row-sharded form:
 // norm_out (may be null) receives the shard's ||z_i||^2 and z is left unscaled; norms_all (may be null), [shards][nstride],
 // supplies ||z_i||^2 as the sum over the shards instead of this context's own.
@@ -220,8 +261,8 @@ cudaError_t sdca_dual_rows(cudaStream_t s, float* Z, int64_t nsamp, int64_t rows
 cudaError_t dml_scale_rows(cudaStream_t s, float* Z, int64_t nsamp, int64_t rows, int64_t ld,
                            const int32_t* similar, float margin, void* split, int64_t split_half, const float* Z2 = nullptr, float* norm_out = nullptr,
                            const float* norms_all = nullptr, int shards = 0, int64_t nstride = 0);
-cudaError_t mean_of(cudaStream_t s, const float* v, int64_t n, float* out);
-cudaError_t prox_unit_columns(cudaStream_t s, float* W, int64_t rows, int64_t cols, float* colpart);
+cudaError_t mean_of(cudaStream_t s, const float* v, int64_t n, float* out, const Stamp& st);
+cudaError_t prox_unit_columns(cudaStream_t s, float* W, int64_t rows, int64_t cols, float* colpart, unsigned long long* end);
 // L = ||W||_2^2 by power iterations from the normalised all-ones vector, on W^T W itself when G is given, else on W.
 // scratch: power_scratch_bytes(cols).
 cudaError_t estimate_lipschitz(cudaStream_t s, const float* W, const float* G, int64_t rows, int64_t cols, void* scratch,

@@ -162,6 +162,7 @@ __global__ void __launch_bounds__(NT, 2) sgemm_kernel(const __grid_constant__ Ge
   const int tm = tile % p.tilesM, tn = tile / p.tilesM;
   pdl_launch_dependents();
   pdl_wait();
+  if (EPI == EPI_RMW) stamp_begin(p.e.begin);
   if (EPI == EPI_SYM && tn < tm) return;              // the mirror image of (tn, tm): uniform over the cluster
   const int m0 = tm * BT, n0 = tn * BT;
   // parts of the contraction end at multiples of 32 whatever the tile, so that a product has one summation order
@@ -232,6 +233,7 @@ __global__ void __launch_bounds__(NT, 2) sgemm_kernel(const __grid_constant__ Ge
         if (n < p.N) epilogue4<EPI>(p, m, n, make_float4(lo.x, lo.y, hi.x, hi.y), invL, mirror);
       }
     }
+    if (EPI == EPI_RMW) stamp_end(p.e.end);
     return;
   }
   // The parts of a split contraction: every CTA of the cluster puts its partial tile into its shared memory, then adds up
@@ -263,6 +265,7 @@ __global__ void __launch_bounds__(NT, 2) sgemm_kernel(const __grid_constant__ Ge
     }
     epilogue4<EPI>(p, m, n, v, invL, mirror);
   }
+  if (EPI == EPI_RMW) stamp_end(p.e.end);
   // no CTA leaves while a peer still reads its tile
   asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
   asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");

@@ -66,8 +66,11 @@ __global__ void __launch_bounds__(256) csr_stage_kernel(const int64_t* __restric
                                                         const float* __restrict__ val, int64_t n, int64_t nnz, int64_t cols,
                                                         int64_t off, float* __restrict__ Xd, int32_t* __restrict__ coo_i,
                                                         int32_t* __restrict__ coo_c, float* __restrict__ coo_x,
-                                                        int2* __restrict__ coo_cx, int32_t fill, int32_t* __restrict__ row_beg,
+                                                        int2* __restrict__ coo_cx, int32_t fill,
+                                                        int32_t* __restrict__ row_beg,
                                                         int32_t* __restrict__ row_end, uint32_t* __restrict__ status) {
+  pdl_launch_dependents();
+  pdl_wait();
   const int64_t i = (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (i >= n) return;
@@ -107,6 +110,8 @@ __global__ void __launch_bounds__(256) csr_stage_kernel(const int64_t* __restric
 // (sample K, value 0) entry, which points at an all-zero row of the factor slab.
 // ---------------------------------------------------------------------------------------------------------
 __global__ void __launch_bounds__(256) csc_count_kernel(const int32_t* __restrict__ coo_c, int64_t nnz, int32_t* __restrict__ cnt) {
+  pdl_launch_dependents();
+  pdl_wait();
   const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
   for (int64_t t = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; t < nnz; t += stride) {
     const int32_t c = coo_c[t];
@@ -115,6 +120,8 @@ __global__ void __launch_bounds__(256) csc_count_kernel(const int32_t* __restric
 }
 
 __global__ void __launch_bounds__(1024) csc_scan_kernel(const int32_t* __restrict__ cnt, int64_t cols, int32_t* __restrict__ ptr) {
+  pdl_launch_dependents();
+  pdl_wait();
   __shared__ int32_t part[1024];
   const int t = threadIdx.x;
   const int64_t chunk = (cols + 1023) / 1024;
@@ -141,6 +148,8 @@ __global__ void __launch_bounds__(256) csc_fill_kernel(const int32_t* __restrict
                                                        const float* __restrict__ coo_x, int64_t nnz,
                                                        const int32_t* __restrict__ ptr, int32_t* __restrict__ cur,
                                                        int2* __restrict__ tmp) {
+  pdl_launch_dependents();
+  pdl_wait();
   const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
   for (int64_t t = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; t < nnz; t += stride) {
     const int32_t c = coo_c[t];
@@ -154,6 +163,8 @@ __global__ void __launch_bounds__(256) csc_fill_kernel(const int32_t* __restrict
 __global__ void __launch_bounds__(128) csc_sort_kernel(const int2* __restrict__ tmp, const int32_t* __restrict__ ptr,
                                                        const int32_t* __restrict__ cnt, int64_t cols, int32_t K,
                                                        int2* __restrict__ ent) {
+  pdl_launch_dependents();
+  pdl_wait();
   for (int64_t d = blockIdx.x; d < cols; d += gridDim.x) {
     const int32_t n = cnt[d], b = ptr[d];
     for (int32_t e = threadIdx.x; e < n; e += blockDim.x) {
@@ -212,6 +223,8 @@ __global__ void __launch_bounds__(kSfThreads, 1) sparse_forward_kernel(const flo
                                                                        const int32_t* __restrict__ row_end,
                                                                        const int2* __restrict__ cx, int64_t off, int32_t n,
                                                                        float* __restrict__ Z, int64_t ldz) {
+  pdl_launch_dependents();
+  pdl_wait();
   extern __shared__ __align__(16) uint8_t sf_smem[];
   constexpr int EP = 32 / RB;                        // entries of a sample worked on at once
   float* ws = reinterpret_cast<float*>(sf_smem);     // RB rows of W, row pitch `pitch` floats
@@ -309,6 +322,8 @@ struct SuParams {
   int64_t shadow_ld;
   float* shadow32;
   int64_t shadow32_ld, shadow_half;
+  Stamp begin;
+  unsigned long long* end;
   unsigned long long* copy_counters;
 };
 
@@ -330,6 +345,9 @@ __device__ __forceinline__ float tf32_round(float x) {
 
 template <int USRC, int SHADOW, bool PROX>
 __global__ void __launch_bounds__(kSuThreads, 1) sparse_update_kernel(const SuParams p) {
+  pdl_launch_dependents();
+  pdl_wait();
+  stamp_begin(p.begin);
   extern __shared__ __align__(16) uint8_t su_smem[];
   __shared__ int next_cb;
   using S = Slab<USRC>;
@@ -474,6 +492,7 @@ __global__ void __launch_bounds__(kSuThreads, 1) sparse_update_kernel(const SuPa
       __syncwarp();                                    // the buffer of sums is free again
     }
   }
+  stamp_end(p.end);
   if (SHADOW == 1 && p.copy_counters) {
     if (lane == 0) atomicAdd(p.copy_counters, pieces);
     if (jj == 0 && written) atomicAdd(p.copy_counters + 1, written);
@@ -482,20 +501,11 @@ __global__ void __launch_bounds__(kSuThreads, 1) sparse_update_kernel(const SuPa
 
 template <int USRC, int SHADOW, bool PROX>
 cudaError_t launch_sparse_update_k(cudaStream_t s, const SuParams& p, int smem) {
-  static std::atomic<uint64_t> prepared{0};            // one bit per device ordinal
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
+  const cudaError_t e = allow_smem<sparse_update_kernel<USRC, SHADOW, PROX>>(kSmemOptIn);
   if (e != cudaSuccess) return e;
-  const uint64_t bit = 1ull << (dev & 63);
-  if (!(prepared.load(std::memory_order_acquire) & bit)) {
-    e = cudaFuncSetAttribute(sparse_update_kernel<USRC, SHADOW, PROX>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemOptIn);
-    if (e != cudaSuccess) return e;
-    prepared.fetch_or(bit, std::memory_order_release);
-  }
   const int nrb = static_cast<int>((p.rows + 31) / 32);
-  sparse_update_kernel<USRC, SHADOW, PROX><<<std::min(nrb, sm_count()), kSuThreads, smem, s>>>(p);
-  count_launch();
-  return cudaGetLastError();
+  return launch_kernel(sparse_update_kernel<USRC, SHADOW, PROX>, dim3(std::min(nrb, sm_count())), dim3(kSuThreads), smem,
+                       s, 1, p);
 }
 
 template <int USRC, int SHADOW>
@@ -560,13 +570,11 @@ int sparse_stage(sfb_ctx* ctx, int64_t off, int64_t n, const int64_t* indptr, co
   float* Xd = ctx->at<float>(L.stageX);
   CKS(cudaMemsetAsync(Xd + off * cols, 0, static_cast<size_t>(n) * cols * 4, s));
   if (nnz > 0) CKS(cudaMemsetAsync(ctx->at<int32_t>(L.coo_c) + ctx->csr_fill, 0xff, static_cast<size_t>(nnz) * 4, s));   // "no entry"
-  csr_stage_kernel<<<static_cast<unsigned>((n * 32 + 255) / 256), 256, 0, s>>>(
-      indptr, idx, val, n, nnz, cols, off, Xd, ctx->at<int32_t>(L.coo_i) + ctx->csr_fill,
-      ctx->at<int32_t>(L.coo_c) + ctx->csr_fill, ctx->at<float>(L.coo_x) + ctx->csr_fill,
-      ctx->at<int2>(L.coo_cx) + ctx->csr_fill, static_cast<int32_t>(ctx->csr_fill), ctx->at<int32_t>(L.row_beg),
-      ctx->at<int32_t>(L.row_end), ctx->at<uint32_t>(L.status));
-  count_launch();
-  CKS(cudaGetLastError());
+  CKS(launch_kernel(csr_stage_kernel, dim3(static_cast<unsigned>((n * 32 + 255) / 256)), dim3(256), 0, s, 1, indptr, idx,
+                    val, n, nnz, cols, off, Xd, ctx->at<int32_t>(L.coo_i) + ctx->csr_fill,
+                    ctx->at<int32_t>(L.coo_c) + ctx->csr_fill, ctx->at<float>(L.coo_x) + ctx->csr_fill,
+                    ctx->at<int2>(L.coo_cx) + ctx->csr_fill, static_cast<int32_t>(ctx->csr_fill),
+                    ctx->at<int32_t>(L.row_beg), ctx->at<int32_t>(L.row_end), ctx->at<uint32_t>(L.status)));
   ctx->last_stage_nnz = nnz;
   return SFB_OK;
 }
@@ -575,24 +583,16 @@ namespace {
 
 template <int RB>
 cudaError_t launch_sparse_forward(sfb_ctx* ctx, int64_t off, int64_t n, float* Z, int64_t ldz, int pitch, int smem) {
-  static std::atomic<uint64_t> prepared{0};            // one bit per device ordinal
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
+  const cudaError_t e = allow_smem<sparse_forward_kernel<RB>>(kSmemOptIn);
   if (e != cudaSuccess) return e;
-  const uint64_t bit = 1ull << (dev & 63);
-  if (!(prepared.load(std::memory_order_acquire) & bit)) {
-    e = cudaFuncSetAttribute(sparse_forward_kernel<RB>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemOptIn);
-    if (e != cudaSuccess) return e;
-    prepared.fetch_or(bit, std::memory_order_release);
-  }
   const Layout& L = ctx->lay;
   const sfb_config& c = ctx->cfg;
   const int64_t nblk = (c.rows + RB - 1) / RB;
-  sparse_forward_kernel<RB><<<static_cast<unsigned>(std::min<int64_t>(nblk, sm_count())), kSfThreads, smem, ctx->stream>>>(
-      ctx->W, c.rows, c.cols, pitch, ctx->at<int32_t>(L.row_beg), ctx->at<int32_t>(L.row_end), ctx->at<int2>(L.coo_cx), off,
-      static_cast<int32_t>(n), Z, ldz);
-  count_launch();
-  return cudaGetLastError();
+  return launch_kernel(sparse_forward_kernel<RB>, dim3(static_cast<unsigned>(std::min<int64_t>(nblk, sm_count()))),
+                       dim3(kSfThreads),
+                       smem, ctx->stream, 1, ctx->W, c.rows, c.cols, pitch, ctx->at<int32_t>(L.row_beg),
+                       ctx->at<int32_t>(L.row_end),
+                       ctx->at<int2>(L.coo_cx), off, static_cast<int32_t>(n), Z, ldz);
 }
 
 // Row pitch (floats) of the rows of W in shared memory: at least cols, and congruent to 32/RB modulo 32 so that the RB
@@ -637,20 +637,15 @@ int sparse_build_csc(sfb_ctx* ctx) {
   CKS(cudaMemsetAsync(cnt, 0, static_cast<size_t>(cols + 1) * 4, s));
   CKS(cudaMemsetAsync(cur, 0, static_cast<size_t>(cols + 1) * 4, s));
   if (nnz > 0) {
-    csc_count_kernel<<<grid1d(nnz, 256), 256, 0, s>>>(ctx->at<int32_t>(L.coo_c), nnz, cnt);
-    count_launch();
+    CKS(launch_kernel(csc_count_kernel, dim3(grid1d(nnz, 256)), dim3(256), 0, s, 1, ctx->at<int32_t>(L.coo_c), nnz, cnt));
   }
-  csc_scan_kernel<<<1, 1024, 0, s>>>(cnt, cols, ptr);
-  count_launch();
+  CKS(launch_kernel(csc_scan_kernel, dim3(1), dim3(1024), 0, s, 1, cnt, cols, ptr));
   if (nnz > 0) {
-    csc_fill_kernel<<<grid1d(nnz, 256), 256, 0, s>>>(ctx->at<int32_t>(L.coo_i), ctx->at<int32_t>(L.coo_c), ctx->at<float>(L.coo_x),
-                                                     nnz, ptr, cur, ctx->at<int2>(L.csc_tmp));
-    count_launch();
-    csc_sort_kernel<<<grid1d(cols, 1, 148 * 16), 128, 0, s>>>(ctx->at<int2>(L.csc_tmp), ptr, cnt, cols,
-                                                              static_cast<int32_t>(ctx->K), ctx->at<int2>(L.csc_ent));
-    count_launch();
+    CKS(launch_kernel(csc_fill_kernel, dim3(grid1d(nnz, 256)), dim3(256), 0, s, 1, ctx->at<int32_t>(L.coo_i),
+                      ctx->at<int32_t>(L.coo_c), ctx->at<float>(L.coo_x), nnz, ptr, cur, ctx->at<int2>(L.csc_tmp)));
+    CKS(launch_kernel(csc_sort_kernel, dim3(grid1d(cols, 1, 148 * 16)), dim3(128), 0, s, 1, ctx->at<int2>(L.csc_tmp), ptr,
+                      cnt, cols, static_cast<int32_t>(ctx->K), ctx->at<int2>(L.csc_ent)));
   }
-  CKS(cudaGetLastError());
   return SFB_OK;
 }
 
@@ -668,6 +663,7 @@ int sparse_update(sfb_ctx* ctx) {
   p.K = static_cast<int32_t>(ctx->K);
   p.alpha = -ctx->step;
   p.prox_kind = ctx->prox_kind; p.prox_a = ctx->prox_a;
+  p.begin = take_stamp(ctx); p.end = &ctx->at<Scalars>(L.scalars)->ns[3];
   if (bf16) {
     p.P = ctx->at<__nv_bfloat16>(L.P); p.ldp = L.ldp;
     p.shadow = ctx->at<__nv_bfloat16>(L.Wb); p.shadow_ld = L.colsb;

@@ -31,15 +31,16 @@ constexpr int kBytesA = BM * BK * 2, kBytesB = BN * BK * 2;
 constexpr int kChunk = 32;                 // accumulator columns handled per epilogue step
 constexpr int kSlotBytes = 32 * kChunk * 4;  // one warp's 32 rows x 32 fp32 columns
 constexpr int kTmemCols = 512;
-constexpr int S = 4;                      // operand pipeline stages
+constexpr int S = 4;                      // operand pipeline stages of a full-width tile (narrower ones: see forward_stages)
+constexpr int S_MAX = 8;
 constexpr int R = 2;                      // epilogue ring slots per warp
 constexpr int kEpiWarps = 4;
 constexpr int kThreads = 64 + 32 * kEpiWarps;
-constexpr int kBars = 2 * S + 4;
+constexpr int kBars = 2 * S_MAX + 4;
 constexpr int kSmem = S * (kBytesA + kBytesB) + kEpiWarps * R * kSlotBytes + kBars * 8 + 16 + 1024;
 
 // Epilogues of the product  D (samples x N) = A * B^T:
-//   F_SOFTMAX  store D as fp32 logits and the per (sample, 256-column block) softmax partials      (MLR; forward_kernel)
+//   F_SOFTMAX  store D as fp32 logits and the softmax partials per (sample, pw columns)            (MLR; forward_kernel)
 // and, in forward_split_kernel:
 //   F_STORE    store D as fp32                                                                     (DML: z = W v)
 //   F_SUB      store D - aux as fp32 and as a (hi | lo) bf16 pair                                  (SC: r = W a - x)
@@ -56,6 +57,10 @@ struct TcParams {
   int32_t M, N, Kc;            // extents of the product: samples, output columns, contraction
   int32_t m_off;               // first sample handled by this launch (per-worker slices)
   int32_t tilesM, tilesN;
+  int32_t a_rows;              // forward_kernel: rows of A per box (fewer than 128 for a slice of few samples; the rest of a
+                               // tile's samples are then never stored)
+  int32_t stages;              // forward_kernel: stages of the operand ring
+  int32_t pw;                  // F_SOFTMAX: columns per softmax partial, a divisor of bn
   int32_t bn;                  // columns per tile, at most BN (chosen so that the tiles fill the SMs): a multiple of 32
                                // in forward_kernel, of 16 in forward_split_kernel
   // The contraction runs over nseg segments of kseg k-blocks; segment s reads A from column a_off<s> and B from
@@ -64,7 +69,7 @@ struct TcParams {
   // parameter block to local memory.)
   int32_t nseg, kseg;
   int32_t a_off0, a_off1, a_off2, b_off0, b_off1, b_off2;
-  float2* part;                // F_SOFTMAX: [tilesN][part_ld] (max, sum exp) per sample and 256-row block
+  float2* part;                // F_SOFTMAX: [N / pw][part_ld] (max, sum exp) per sample and pw rows of W
   int64_t part_ld;
   const float* aux;            // F_SUB: the matrix subtracted, [M x ldaux]; F_ISTA, F_ISTAG: the matrix updated
   int64_t ldaux;
@@ -122,23 +127,24 @@ forward_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                const __grid_constant__ CUtensorMap tmC, const TcParams p) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  uint8_t* sA = smem;
-  uint8_t* sB = smem + S * kBytesA;
+  const int ST = p.stages;
+  const int stage_bytes = kBytesA + p.bn * BK * 2;       // A, then B: all multiples of 1024
   uint8_t* sRing = smem + S * (kBytesA + kBytesB);
   uint64_t* bars = reinterpret_cast<uint64_t*>(sRing + 4 * R * kSlotBytes);
   uint64_t* full = bars;
-  uint64_t* empty = bars + S;
-  uint64_t* tfull = bars + 2 * S;
-  uint64_t* tempty = bars + 2 * S + 2;
+  uint64_t* empty = bars + S_MAX;
+  uint64_t* tfull = bars + 2 * S_MAX;
+  uint64_t* tempty = bars + 2 * S_MAX + 2;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + kBars);
   volatile uint32_t* abort_flag = tmem_slot + 1;
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int ntiles = p.tilesM * p.tilesN;
   const int numK = p.nseg * p.kseg;
+  pdl_launch_dependents();
 
   if (threadIdx.x == 0) {
-    for (int i = 0; i < S; ++i) { mbar_init(&full[i], 1); mbar_init(&empty[i], 1); }
+    for (int i = 0; i < ST; ++i) { mbar_init(&full[i], 1); mbar_init(&empty[i], 1); }
     for (int i = 0; i < 2; ++i) { mbar_init(&tfull[i], 1); mbar_init(&tempty[i], 4); }
     *abort_flag = 0;
     fence_barrier_init();
@@ -149,13 +155,14 @@ forward_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  pdl_wait();
 
   if (warp == 0) {
     // ---------------- TMA producer ----------------
     if (lane == 0) {
       // A (the K samples) is the small operand every tile re-reads: pinned in L2.
       const uint64_t pol_keep = policy_evict_last();
-      uint32_t it = 0;
+      uint32_t s = 0, ph = 0;
       bool ok = true;
       for (int tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x) {
         int m0, n0;
@@ -163,16 +170,17 @@ forward_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         for (int seg = 0; seg < p.nseg && ok; ++seg) {
           const int xa0 = seg == 0 ? p.a_off0 : seg == 1 ? p.a_off1 : p.a_off2;
           const int xb0 = seg == 0 ? p.b_off0 : seg == 1 ? p.b_off1 : p.b_off2;
-          for (int kl = 0; kl < p.kseg; ++kl, ++it) {
-            const uint32_t s = it % S, ph = (it / S) & 1;
+          for (int kl = 0; kl < p.kseg; ++kl) {
             if (!mbar_wait(&empty[s], ph ^ 1, abort_flag)) { ok = false; break; }
             // B streams from HBM when it is larger than L2: with the box asked for a few k-blocks early, the load
             // that fills the stage finds it in L2 and the four stages cover the latency
             if (p.prefetch > 0 && kl + p.prefetch < p.kseg)
               tma_prefetch_2d(&tmB, xb0 + (kl + p.prefetch) * (TF32 ? BK / 2 : BK), n0);
-            mbar_expect_tx(&full[s], kBytesA + p.bn * BK * 2);
-            tma_load_2d_hint(sA + s * kBytesA, &tmA, xa0 + kl * (TF32 ? BK / 2 : BK), m0, &full[s], pol_keep);
-            tma_load_2d(sB + s * kBytesB, &tmB, xb0 + kl * (TF32 ? BK / 2 : BK), n0, &full[s]);
+            uint8_t* st = smem + s * stage_bytes;
+            mbar_expect_tx(&full[s], (p.a_rows + p.bn) * BK * 2);
+            tma_load_2d_hint(st, &tmA, xa0 + kl * (TF32 ? BK / 2 : BK), m0, &full[s], pol_keep);
+            tma_load_2d(st + kBytesA, &tmB, xb0 + kl * (TF32 ? BK / 2 : BK), n0, &full[s]);
+            if (++s == static_cast<uint32_t>(ST)) { s = 0; ph ^= 1; }
           }
         }
       }
@@ -181,19 +189,18 @@ forward_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     // ---------------- MMA issuer ----------------
     if (lane == 0) {
       const uint32_t idesc = TF32 ? umma_idesc_tf32(BM, p.bn) : umma_idesc_bf16(BM, p.bn);
-      uint32_t it = 0, tl = 0;
+      uint32_t s = 0, ph = 0, tl = 0;
       bool ok = true;
       for (int tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x, ++tl) {
         const uint32_t a = tl & 1, aph = (tl >> 1) & 1;
         if (!mbar_wait(&tempty[a], aph ^ 1, abort_flag)) { ok = false; break; }
         tc_fence_after();
         const uint32_t d_tmem = tmem_base + a * BN;
-        for (int kb = 0; kb < numK; ++kb, ++it) {
-          const uint32_t s = it % S, ph = (it / S) & 1;
+        for (int kb = 0; kb < numK; ++kb) {
           if (!mbar_wait(&full[s], ph, abort_flag)) { ok = false; break; }
           tc_fence_after();
-          const uint64_t da = umma_desc_k128(smem_u32(sA + s * kBytesA));
-          const uint64_t db = umma_desc_k128(smem_u32(sB + s * kBytesB));
+          const uint64_t da = umma_desc_k128(smem_u32(smem + s * stage_bytes));
+          const uint64_t db = umma_desc_k128(smem_u32(smem + s * stage_bytes + kBytesA));
 #pragma unroll
           for (int k = 0; k < BK / UMMA_K; ++k) {          // four MMAs of 32 bytes of contraction each, either kind
             const uint64_t adv = static_cast<uint64_t>(k * UMMA_K * 2 / 16);
@@ -201,6 +208,7 @@ forward_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
             else umma_bf16(d_tmem, da + adv, db + adv, idesc, (kb | k) != 0 ? 1u : 0u);
           }
           umma_commit(&empty[s]);          // the stage is free once these MMAs have read it
+          if (++s == static_cast<uint32_t>(ST)) { s = 0; ph ^= 1; }
         }
         if (ok) umma_commit(&tfull[a]);    // the accumulator is complete once every MMA of the tile is
       }
@@ -257,11 +265,16 @@ forward_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
             }
             ++gs;
           }
+          if (EPI == F_SOFTMAX && ((c + 1) * kChunk) % p.pw == 0) {      // the end of a group of pw columns
+            const int grp = (n0 + (c + 1) * kChunk) / p.pw - 1;
+            if (grp * p.pw < p.N && row < p.M) p.part[static_cast<int64_t>(grp) * p.part_ld + row] = make_float2(mx, sum);
+            mx = -INFINITY;
+            sum = 0.f;
+          }
         }
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive(&tempty[a]);
-        if (EPI == F_SOFTMAX && row < p.M) p.part[static_cast<int64_t>(n0 / p.bn) * p.part_ld + row] = make_float2(mx, sum);
       }
       if (lane == 0) tma_wait_group<0>();
     }
@@ -322,6 +335,7 @@ forward_split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
   const int nacc = p.bn <= 128 ? 2 : 1, cross = p.bn <= 128 ? 128 : 256;
   const int a_hi = p.a_off0, a_lo = p.a_off2, b_hi = p.b_off0, b_lo = p.b_off1;
 
+  pdl_launch_dependents();
   if (threadIdx.x == 0) {
     for (int i = 0; i < FS_STAGES; ++i) { mbar_init(&full[i], 1); mbar_init(&empty[i], 1); }
     for (int i = 0; i < 2; ++i) { mbar_init(&tfull[i], 1); mbar_init(&tempty[i], 4); }
@@ -334,6 +348,7 @@ forward_split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  pdl_wait();
 
   if (warp == 0) {
     // ---------------- TMA producer: the four operand halves of a k-block per stage ----------------
@@ -554,6 +569,8 @@ __device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
 // fp32 [rows x cols] -> bf16 [rows x ld] (row-major), 8 elements per thread; cols is a multiple of 4.
 __global__ void __launch_bounds__(256) convert_rows_kernel(const float* __restrict__ src, int64_t rows, int64_t cols,
                                                            __nv_bfloat16* __restrict__ dst, int64_t ld) {
+  pdl_launch_dependents();
+  pdl_wait();
   const int64_t quads = cols / 4;
   const int64_t total = rows * quads;
   const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
@@ -566,12 +583,18 @@ __global__ void __launch_bounds__(256) convert_rows_kernel(const float* __restri
 
 // Pack of the inputs of n samples starting at pair index off (Section 2.1: v = a_i):
 //   Xb[off + i][:]  = bf16(x_i), the operand of the forward product and of the update (which contracts over the samples and
-//                     takes it as an MN-major operand),   Xf = the fp32 sample for the label rows,   labels.
-// One read of X, 6 bytes written per value; bound by HBM (1,024 x 20,000: 33 us with a transposed copy beside it, 24 without).
+//                     takes it as an MN-major operand),   Xf (may be null) = the fp32 sample for the label rows,   labels.
+// The label-row slots of the classes that these samples had in the step before are cleared.
+// One read of X, 6 bytes written per value, 2 without Xf; bound by HBM (1,024 x 20,000: 33 us with a transposed copy beside
+// it, 28 without, 20 without Xf).
+constexpr int32_t kNoSlot = 0x7f7f7f7f;              // above every sample index (K <= 2^20)
 __global__ void __launch_bounds__(256) pack_mlr_kernel(const float* __restrict__ X, int64_t n, int64_t cols,
                                                        __nv_bfloat16* __restrict__ Xb, int64_t ldx, int64_t off,
-                                                       float* __restrict__ Xf, const int32_t* __restrict__ labels,
-                                                       int32_t* __restrict__ labels_out) {
+                                                       float* __restrict__ Xf, const int32_t* labels, int32_t* labels_out,
+                                                       int32_t* __restrict__ slot, int64_t rows, const Stamp stamp) {
+  pdl_launch_dependents();
+  pdl_wait();
+  stamp_begin(stamp);
   const uint32_t quads = static_cast<uint32_t>(cols / 4);
   const int64_t total = n * quads, stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
   const int64_t t0 = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
@@ -579,9 +602,13 @@ __global__ void __launch_bounds__(256) pack_mlr_kernel(const float* __restrict__
     const int64_t i = q / quads, c = (q - i * quads) * 4;
     const float4 v = *reinterpret_cast<const float4*>(X + i * cols + c);
     *reinterpret_cast<uint2*>(Xb + (off + i) * ldx + c) = make_uint2(pack_bf16(v.x, v.y), pack_bf16(v.z, v.w));
-    *reinterpret_cast<float4*>(Xf + (off + i) * cols + c) = v;
+    if (Xf) *reinterpret_cast<float4*>(Xf + (off + i) * cols + c) = v;
   }
-  for (int64_t i = t0; i < n; i += stride) labels_out[off + i] = labels[i];
+  for (int64_t i = t0; i < n; i += stride) {
+    const int32_t old = labels_out[off + i];
+    if (old >= 0 && old < rows) slot[old] = kNoSlot;
+    labels_out[off + i] = labels[i];
+  }
 }
 
 // W [n x dim] -> its transpose as a (hi | lo) bf16 operand FT [dim x 2*Kp] (the coder's W^T): FT[c][i] = hi(F[i][c]),
@@ -589,6 +616,8 @@ __global__ void __launch_bounds__(256) pack_mlr_kernel(const float* __restrict__
 // shared memory.
 __global__ void __launch_bounds__(256) pack_split_t_kernel(const float* __restrict__ F, int64_t n, int64_t dim,
                                                            int64_t ld, __nv_bfloat16* __restrict__ FT, int64_t Kp) {
+  pdl_launch_dependents();
+  pdl_wait();
   __shared__ float tile[64][65];
   const int64_t i0 = static_cast<int64_t>(blockIdx.y) * 64, c0 = static_cast<int64_t>(blockIdx.x) * 64;
   const int t = threadIdx.x;
@@ -634,7 +663,11 @@ __global__ void __launch_bounds__(256) pack_split_t_kernel(const float* __restri
 // dst[r][dimp + c] = lo with hi = bf16(f), lo = bf16(f - hi).  Columns dim..dimp-1 are left as they are (zero since
 // set-up).
 __global__ void __launch_bounds__(256) pack_split_rows_kernel(const float* __restrict__ F, int64_t n, int64_t dim,
-                                                              int64_t ld, __nv_bfloat16* __restrict__ dst, int64_t dimp) {
+                                                              int64_t ld, __nv_bfloat16* __restrict__ dst, int64_t dimp,
+                                                              const Stamp stamp) {
+  pdl_launch_dependents();
+  pdl_wait();
+  stamp_begin(stamp);
   const int64_t quads = (dim + 3) / 4, total = n * quads;
   const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
   const bool vec = ld % 4 == 0 && dim % 4 == 0;          // else (samples with an odd number of features) value by value
@@ -661,6 +694,30 @@ __global__ void __launch_bounds__(256) pack_split_rows_kernel(const float* __res
   }
 }
 
+// DML: v = x - y of n pairs (Section 2) in fp32 and as the (hi | lo) operand, one pass (16 bytes per value; as two kernels 24).
+__global__ void __launch_bounds__(256) pack_pairs_kernel(const float* __restrict__ X, const float* __restrict__ Y, int64_t n,
+                                                         int64_t dim, float* __restrict__ V,
+                                                         __nv_bfloat16* __restrict__ dst,
+                                                         int64_t dimp, const Stamp stamp) {
+  pdl_launch_dependents();
+  pdl_wait();
+  stamp_begin(stamp);
+  const uint32_t quads = static_cast<uint32_t>(dim / 4);
+  const int64_t total = n * quads, stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
+  for (int64_t q = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; q < total; q += stride) {
+    const int64_t i = q / quads, c = (q - i * quads) * 4;
+    const float4 x = reinterpret_cast<const float4*>(X)[q], y = reinterpret_cast<const float4*>(Y)[q];
+    const float4 v = make_float4(x.x - y.x, x.y - y.y, x.z - y.z, x.w - y.w);
+    reinterpret_cast<float4*>(V)[q] = v;
+    const uint32_t h01 = pack_bf16(v.x, v.y), h23 = pack_bf16(v.z, v.w);
+    const float2 f01 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&h01));
+    const float2 f23 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&h23));
+    __nv_bfloat16* d = dst + i * 2 * dimp + c;
+    *reinterpret_cast<uint2*>(d) = make_uint2(h01, h23);
+    *reinterpret_cast<uint2*>(d + dimp) = make_uint2(pack_bf16(v.x - f01.x, v.y - f01.y), pack_bf16(v.z - f23.x, v.w - f23.y));
+  }
+}
+
 __device__ __forceinline__ float warp_sum(float v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
@@ -673,12 +730,15 @@ __device__ __forceinline__ float warp_max(float v) {
 }
 
 // One warp per sample: merge the per-block (max, sum exp) partials into log sum exp; loss = lse - z_y;
-// coef = 1 - p_y, the size of the label entry of u, kept in fp32 for label_rows_kernel.
+// coef = 1 - p_y, the size of the label entry of u, kept in fp32.
 __global__ void __launch_bounds__(256) mlr_lse_kernel(const float2* __restrict__ part, int64_t part_ld, int nblocks,
                                                       const float* __restrict__ Z, int64_t ldz, int64_t rows,
                                                       const int32_t* __restrict__ labels, int64_t off, int64_t n,
                                                       float* __restrict__ lse, float* __restrict__ loss,
-                                                      float* __restrict__ coef, uint32_t* status) {
+                                                      float* __restrict__ coef, int32_t* __restrict__ slot,
+                                                      uint32_t* status) {
+  pdl_launch_dependents();
+  pdl_wait();
   const int64_t i = static_cast<int64_t>(blockIdx.x) * 8 + (threadIdx.x >> 5);
   if (i >= n) return;
   const int lane = threadIdx.x & 31;
@@ -701,7 +761,160 @@ __global__ void __launch_bounds__(256) mlr_lse_kernel(const float2* __restrict__
     const float zy = okl ? Z[s * ldz + y] : 0.f;
     loss[s] = okl ? l - zy : 0.f;
     coef[s] = okl ? -expm1f(zy - l) : 0.f;        // 1 - p_y = -u_y, formed in fp32 without cancellation
+    if (okl && slot) atomicMin(&slot[y], static_cast<int32_t>(s));      // the first sample of its class (see label_delta)
   }
+}
+
+// The label entries of the K factors, u_iy = p_iy - 1, which the bf16 operand leaves out (it holds 0 there).  Per class that
+// the mini-batch has, in fp32 and in ascending sample order (no atomics: one order):
+//     dL[f] = sum_{i : y_i = y} (1 - p_iy) x_i,   W[y] <- W[y] + step * dL[f],   f = slot[y] the class's first sample,
+// and the bf16 copy of the row with it; dL is kept for a repeated update.  Work units (first sample, 1024 columns) are dealt
+// to nblk blocks; the last block also forms the mean loss.  A popular class (130 of 1,024 samples under Zipf labels) is what
+// the kernel waits for, so a unit has eight samples in flight.  It shares a launch with the probabilities where it can.
+// (Adding dL in the epilogue of the update, which has the row on chip, cost that kernel 100 us at 10,000 x 20,000: its W
+// stream is bound by latency, and any work between a tile's arrival and its departure adds to it.)
+// Eight loads in one statement: issued together, whatever the compiler thinks of the registers.
+__device__ __forceinline__ void load8(float4 (&x)[8], const float* const (&p)[8]) {
+  asm volatile(
+      "ld.global.nc.v4.f32 {%0, %1, %2, %3}, [%32];\n\tld.global.nc.v4.f32 {%4, %5, %6, %7}, [%33];\n\t"
+      "ld.global.nc.v4.f32 {%8, %9, %10, %11}, [%34];\n\tld.global.nc.v4.f32 {%12, %13, %14, %15}, [%35];\n\t"
+      "ld.global.nc.v4.f32 {%16, %17, %18, %19}, [%36];\n\tld.global.nc.v4.f32 {%20, %21, %22, %23}, [%37];\n\t"
+      "ld.global.nc.v4.f32 {%24, %25, %26, %27}, [%38];\n\tld.global.nc.v4.f32 {%28, %29, %30, %31}, [%39];"
+      : "=&f"(x[0].x), "=&f"(x[0].y), "=&f"(x[0].z), "=&f"(x[0].w), "=&f"(x[1].x), "=&f"(x[1].y), "=&f"(x[1].z), "=&f"(x[1].w),
+        "=&f"(x[2].x), "=&f"(x[2].y), "=&f"(x[2].z), "=&f"(x[2].w), "=&f"(x[3].x), "=&f"(x[3].y), "=&f"(x[3].z), "=&f"(x[3].w),
+        "=&f"(x[4].x), "=&f"(x[4].y), "=&f"(x[4].z), "=&f"(x[4].w), "=&f"(x[5].x), "=&f"(x[5].y), "=&f"(x[5].z), "=&f"(x[5].w),
+        "=&f"(x[6].x), "=&f"(x[6].y), "=&f"(x[6].z), "=&f"(x[6].w), "=&f"(x[7].x), "=&f"(x[7].y), "=&f"(x[7].z), "=&f"(x[7].w)
+      : "l"(p[0]), "l"(p[1]), "l"(p[2]), "l"(p[3]), "l"(p[4]), "l"(p[5]), "l"(p[6]), "l"(p[7]));
+}
+constexpr int kLabelList = 1024, kLabelCols = 1024, kLabelBatch = 8;
+struct LabelArgs {
+  const float* X;              // the K samples, fp32
+  const int32_t* labels;
+  const int32_t* slot;
+  const float* coef;
+  float* dL;                   // [K x cols]
+  float* W;                    // [rows x cols]
+  __nv_bfloat16* Wb;           // its operand copy, row pitch ldw
+  int64_t ldw;
+  float step;
+  int32_t again;               // dL is there: add it to W once more
+  const float* loss;
+  float* loss_mean;
+  int64_t rows, cols;
+  int32_t K;
+};
+__device__ __forceinline__ void label_delta(const LabelArgs& a, int blk, int nblk) {
+  __shared__ int nunits;
+  __shared__ int32_t unit[256];
+  __shared__ int32_t list[kLabelList];
+  __shared__ float lcoef[kLabelList];
+  __shared__ int warp_tot[8];
+  __shared__ float lsum[8];
+  const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
+  if (blk == nblk - 1) {
+    float v = 0.f;
+    for (int i = t; i < a.K; i += 256) v += a.loss[i];
+    v = warp_sum(v);
+    if (lane == 0) lsum[wid] = v;
+    __syncthreads();
+    if (t == 0) {
+      float m = 0.f;
+      for (int w = 0; w < 8; ++w) m += lsum[w];
+      *a.loss_mean = m / static_cast<float>(a.K);
+    }
+  }
+  const int64_t chunks = (a.cols + kLabelCols - 1) / kLabelCols, total = a.K * chunks;
+  for (int64_t base = 0; base * nblk < total; base += 256) {
+    if (t == 0) nunits = 0;
+    __syncthreads();
+    const int64_t u = (base + t) * nblk + blk;
+    if (u < total) {
+      const int32_t i = static_cast<int32_t>(u / chunks), y = a.labels[i];
+      if (y >= 0 && y < a.rows && a.slot[y] == i) unit[atomicAdd(&nunits, 1)] = t;
+    }
+    __syncthreads();
+    const int todo = nunits;
+    for (int k = 0; k < todo; ++k) {
+      const int64_t v = (base + unit[k]) * nblk + blk;
+      const int32_t i = static_cast<int32_t>(v / chunks), y = a.labels[i];
+      const int64_t c = (v % chunks) * kLabelCols + 4 * t;
+      float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+      float* d = a.dL + static_cast<int64_t>(i) * a.cols + c;
+      float* wp = a.W + static_cast<int64_t>(y) * a.cols + c;
+      float4 w = s;
+      if (c < a.cols) {
+        w = *reinterpret_cast<const float4*>(wp);
+        if (a.again) s = *reinterpret_cast<const float4*>(d);
+      }
+      for (int j0 = a.again ? a.K : i; j0 < a.K; j0 += kLabelList) {
+        // ordered compaction of the class's samples in [j0, j0 + kLabelList): a warp looks at 128 labels
+        unsigned hit[4];
+        int mine = 0;
+#pragma unroll
+        for (int o = 0; o < 4; ++o) {
+          const int j = j0 + wid * 128 + o * 32 + lane;
+          hit[o] = __ballot_sync(0xffffffffu, j < a.K && a.labels[j] == y);
+          mine += __popc(hit[o]);
+        }
+        if (lane == 0) warp_tot[wid] = mine;
+        __syncthreads();
+        int pre = 0, n = 0;
+#pragma unroll
+        for (int w = 0; w < 8; ++w) {
+          if (w < wid) pre += warp_tot[w];
+          n += warp_tot[w];
+        }
+#pragma unroll
+        for (int o = 0; o < 4; ++o) {
+          if ((hit[o] >> lane) & 1u) {
+            const int at = pre + __popc(hit[o] & ((1u << lane) - 1)), j = j0 + wid * 128 + o * 32 + lane;
+            list[at] = j;
+            lcoef[at] = a.coef[j];
+          }
+          pre += __popc(hit[o]);
+        }
+        __syncthreads();
+        if (c < a.cols)
+          for (int q0 = 0; q0 < n; q0 += kLabelBatch) {
+            float4 x[kLabelBatch];
+            const float* xp[kLabelBatch];
+#pragma unroll
+            for (int e = 0; e < kLabelBatch; ++e) xp[e] = a.X + static_cast<int64_t>(list[min(q0 + e, n - 1)]) * a.cols + c;
+            load8(x, xp);
+#pragma unroll
+            for (int e = 0; e < kLabelBatch; ++e) {
+              const float cf = q0 + e < n ? lcoef[q0 + e] : 0.f;
+              s.x = fmaf(cf, x[e].x, s.x); s.y = fmaf(cf, x[e].y, s.y);
+              s.z = fmaf(cf, x[e].z, s.z); s.w = fmaf(cf, x[e].w, s.w);
+            }
+          }
+        __syncthreads();
+      }
+      if (c < a.cols) {
+        if (!a.again) *reinterpret_cast<float4*>(d) = s;
+        w.x = fmaf(a.step, s.x, w.x); w.y = fmaf(a.step, s.y, w.y); w.z = fmaf(a.step, s.z, w.z); w.w = fmaf(a.step, s.w, w.w);
+        *reinterpret_cast<float4*>(wp) = w;
+        *reinterpret_cast<uint2*>(a.Wb + static_cast<int64_t>(y) * a.ldw + c) = make_uint2(pack_bf16(w.x, w.y), pack_bf16(w.z, w.w));
+      }
+    }
+    __syncthreads();
+  }
+}
+__global__ void __launch_bounds__(256) label_delta_kernel(const LabelArgs a) {
+  pdl_launch_dependents();
+  pdl_wait();
+  label_delta(a, blockIdx.x, gridDim.x);
+}
+// slot[y] = the smallest index of a sample of class y, for factors that came in several calls.
+__global__ void __launch_bounds__(256) label_slots_kernel(const int32_t* __restrict__ labels, int32_t K, int64_t rows,
+                                                          int32_t* __restrict__ slot, const Stamp stamp) {
+  pdl_launch_dependents();
+  pdl_wait();
+  stamp_begin(stamp);
+  const int i = blockIdx.x * 256 + threadIdx.x;
+  if (i >= K) return;
+  const int32_t y = labels[i];
+  if (y >= 0 && y < rows) atomicMin(&slot[y], i);
 }
 
 // Row-sharded form, first half: one warp per sample merges the forward's per-block (max, sum exp) partials over the
@@ -711,6 +924,8 @@ __global__ void __launch_bounds__(256) mlr_shard_partials_tc_kernel(const float2
                                                                     const float* __restrict__ Z, int64_t ldz, int64_t rows,
                                                                     const int32_t* __restrict__ labels, int64_t row_off,
                                                                     int64_t n, float4* __restrict__ out) {
+  pdl_launch_dependents();
+  pdl_wait();
   const int64_t i = static_cast<int64_t>(blockIdx.x) * 8 + (threadIdx.x >> 5);
   if (i >= n) return;
   const int lane = threadIdx.x & 31;
@@ -734,9 +949,12 @@ __global__ void __launch_bounds__(256) mlr_shard_partials_tc_kernel(const float2
 // log-partition; loss = lse - z_y; coef = 1 - p_y for the samples whose class this shard owns (0 otherwise); the class
 // ids are rewritten as row indices of this shard (-1: another shard's row).  A class no shard owns sets the status bit.
 __global__ void __launch_bounds__(256) mlr_shard_finish_tc_kernel(const float4* __restrict__ parts, int shards, int64_t n,
-                                                                  int64_t rows, int64_t row_off, int32_t* __restrict__ labels,
+                                                                  int64_t rows, int64_t row_off,
+                                                                  int32_t* __restrict__ labels,
                                                                   float* __restrict__ lse, float* __restrict__ loss,
                                                                   float* __restrict__ coef, uint32_t* status) {
+  pdl_launch_dependents();
+  pdl_wait();
   const int64_t i = static_cast<int64_t>(blockIdx.x) * 256 + threadIdx.x;
   if (i >= n) return;
   float M = -INFINITY;
@@ -761,18 +979,22 @@ __global__ void __launch_bounds__(256) mlr_shard_finish_tc_kernel(const float4* 
 
 // P[off + i][r] = bf16( exp(z_ir - lse_i) ) for r != y_i and 0 for r = y_i, from the logits Z (row pitch a multiple of 32).
 // The factor is u_i = p_i - onehot(y_i); its label entry u_iy = p_iy - 1 is left out of the bf16 operand and applied to W in
-// fp32 by label_rows_kernel, because bf16 cannot hold it when p_iy is close to 1 (spacing 2^-8 next to 1) and a rounded p_iy
+// fp32 (label_delta), because bf16 cannot hold it when p_iy is close to 1 (spacing 2^-8 next to 1) and a rounded p_iy
 // with an exact -1 would not cancel.  Eight values per thread; 6 bytes per value, bound by HBM.
 // PLAIN: the values of Z themselves instead of exp(z - lse) (the dual changes of the SDCA step), with the same zero at the
 // label entry.
+// With K label entries to sum (lab.K > 0) the first lab_blocks blocks do that instead, see label_delta.
 template <bool PLAIN>
 __global__ void __launch_bounds__(256) mlr_emit_p_kernel(const float* __restrict__ Z, int64_t ldz, int64_t rows,
                                                          const float* __restrict__ lse, int64_t off, int64_t n,
                                                          const int32_t* __restrict__ labels, __nv_bfloat16* __restrict__ P,
-                                                         int64_t ldp) {
+                                                         int64_t ldp, int lab_blocks, const LabelArgs lab) {
+  pdl_launch_dependents();
+  pdl_wait();
+  if (static_cast<int>(blockIdx.x) < lab_blocks) return label_delta(lab, blockIdx.x, lab_blocks);
   const uint32_t octs = static_cast<uint32_t>((rows + 7) / 8);
-  const int64_t total = n * octs, stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
-  for (int64_t q = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; q < total; q += stride) {
+  const int64_t total = n * octs, stride = static_cast<int64_t>(gridDim.x - lab_blocks) * blockDim.x;
+  for (int64_t q = (blockIdx.x - lab_blocks) * static_cast<int64_t>(blockDim.x) + threadIdx.x; q < total; q += stride) {
     const int64_t i = q / octs, r = (q - i * octs) * 8, s = off + i;
     const float l = PLAIN ? 0.f : lse[s];
     const int64_t yrel = static_cast<int64_t>(labels[i]) - r;           // label row relative to this group of eight
@@ -799,6 +1021,8 @@ __device__ __forceinline__ float to_tf32(float x) {
 // dim..dimp-1 keep the zeros of set-up.  dim and ld are multiples of 4.
 __global__ void __launch_bounds__(256) split32_rows_kernel(const float* __restrict__ F, int64_t n, int64_t dim, int64_t ld,
                                                            float* __restrict__ dst, int64_t dimp) {
+  pdl_launch_dependents();
+  pdl_wait();
   const int64_t quads = dim / 4, total = n * quads;
   const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
   for (int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; i < total; i += stride) {
@@ -816,6 +1040,8 @@ __global__ void __launch_bounds__(256) split32_rows_kernel(const float* __restri
 // FT[c][i] = big, FT[c][Kp + i] = small; pairs n..Kp-1 are written as zeros.  64 x 64 tiles through shared memory.
 __global__ void __launch_bounds__(256) split32_t_kernel(const float* __restrict__ F, int64_t n, int64_t dim, int64_t ld,
                                                         float* __restrict__ FT, int64_t Kp) {
+  pdl_launch_dependents();
+  pdl_wait();
   __shared__ float tile[64][65];
   const int64_t i0 = static_cast<int64_t>(blockIdx.y) * 64, c0 = static_cast<int64_t>(blockIdx.x) * 64;
   const int t = threadIdx.x;
@@ -843,8 +1069,11 @@ __global__ void __launch_bounds__(256) split32_t_kernel(const float* __restrict_
 // (Section 2.1: u = d f / d (W a)).  PLAIN copies Z instead (the dual changes of the SDCA step already are the factors).
 template <bool PLAIN>
 __global__ void __launch_bounds__(256) mlr_finish_u_kernel(const float* __restrict__ Z, int64_t ldz, int64_t rows,
-                                                           const float* __restrict__ lse, const int32_t* __restrict__ labels,
+                                                           const float* __restrict__ lse,
+                                                           const int32_t* __restrict__ labels,
                                                            float* __restrict__ U) {
+  pdl_launch_dependents();
+  pdl_wait();
   const int64_t i = blockIdx.y;
   const float l = PLAIN ? 0.f : lse[i];
   const int64_t y = PLAIN ? -1 : static_cast<int64_t>(labels[i]);
@@ -860,25 +1089,21 @@ __global__ void __launch_bounds__(256) mlr_finish_u_kernel(const float* __restri
 // ---------------------------------------------------------------------------------------------------------
 template <int EPI, bool TF32 = false>
 cudaError_t launch_forward(sfb_ctx* ctx, const CUtensorMap& a, const CUtensorMap& b, const CUtensorMap& c, TcParams p) {
-  const TcState* st = static_cast<const TcState*>(ctx->tc);
+  TcState* st = static_cast<TcState*>(ctx->tc);
   const int64_t tiles = static_cast<int64_t>(p.tilesM) * p.tilesN;
   if (tiles <= 0) return cudaSuccess;
   const int grid = static_cast<int>(tiles < st->sms ? tiles : st->sms);
-  forward_kernel<EPI, TF32><<<grid, kThreads, kSmem, ctx->stream>>>(a, b, c, p);
-  count_launch();
-  return cudaGetLastError();
+  return launch_kernel_if(tiles <= st->sms, forward_kernel<EPI, TF32>, dim3(grid), dim3(kThreads), kSmem, ctx->stream, 1, a, b, c, p);
 }
 
 template <int EPI>
 cudaError_t launch_forward_split(sfb_ctx* ctx, const CUtensorMap& a, const CUtensorMap& b, float* C, int64_t ldc, TcParams p) {
-  const TcState* st = static_cast<const TcState*>(ctx->tc);
+  TcState* st = static_cast<TcState*>(ctx->tc);
   const int64_t tiles = EPI == F_GRAM ? sym_tiles(p.tilesM, p.tilesN, p.bn)
                                       : static_cast<int64_t>(p.tilesM) * p.tilesN * (p.ksplit > 1 ? p.ksplit : 1);
   if (tiles <= 0) return cudaSuccess;
   const int grid = static_cast<int>(tiles < st->sms ? tiles : st->sms);
-  forward_split_kernel<EPI><<<grid, kThreads, kFsSmem, ctx->stream>>>(a, b, C, ldc, p);
-  count_launch();
-  return cudaGetLastError();
+  return launch_kernel_if(tiles <= st->sms, forward_split_kernel<EPI>, dim3(grid), dim3(kThreads), kFsSmem, ctx->stream, 1, a, b, C, ldc, p);
 }
 
 // The shared-memory opt-in is a per-device attribute of each kernel: set for every instantiation when a context is
@@ -906,6 +1131,28 @@ cudaError_t prepare_forward_kernels() {
       return SFB_ERR_CUDA;                              \
     }                                                   \
   } while (0)
+
+// Stages of the operand ring for tiles of bn columns (192 KB).
+static int forward_stages(int bn) { return std::min(S_MAX, S * (kBytesA + kBytesB) / (kBytesA + bn * BK * 2)); }
+
+// Tile width of the forward product of n samples with a rows x cols matrix, a power of two from `least` to 256.  A k-block of a
+// tile takes the longest of its MMAs (2 cycles per column), its bytes at about 60 a cycle and the latency of its loads over
+// the stages in flight; wide tiles read the samples less often, narrow ones occupy more SMs when W has few rows (a worker's
+// 37 samples against 4,999 x 3,004: 23 us with 256-wide tiles on 20 SMs).
+static int pick_forward_width(int64_t n, int64_t rows, int64_t cols, int least) {
+  const int sms = sm_count();
+  const double kb = static_cast<double>((cols + BK - 1) / BK), ar = static_cast<double>(std::min<int64_t>(BM, round_up(n, 8)));
+  int best = 256;
+  double best_cost = 0.;
+  for (int bn = 256; bn >= least; bn /= 2) {
+    const int64_t tiles = ((n + BM - 1) / BM) * ((rows + bn - 1) / bn);
+    const double rounds = static_cast<double>((tiles + sms - 1) / sms);
+    const double per_kb = std::max(std::max(2.0 * bn, (ar + bn) * BK * 2 / 60.0), 1200.0 / forward_stages(bn));
+    const double cost = rounds * (kb * per_kb + 2500.0);
+    if (bn == 256 || cost < 0.97 * best_cost) { best = bn; best_cost = cost; }
+  }
+  return best;
+}
 
 // fp32 mode on the tensor cores (MLR): fp32 pair-major factors as in the FFMA path, plus the (big | small) tf32
 // operands of the two products and the logits.
@@ -957,7 +1204,8 @@ void tc_extend_layout(const sfb_config& c, Layout& L, size_t& off) {
     return;
   }
   const size_t ldz = static_cast<size_t>(round_up(c.rows, 32));
-  const size_t nblk = static_cast<size_t>((c.rows + BN - 1) / BN);
+  L.pw = pick_forward_width(c.batch, c.rows, c.cols, 32);
+  const size_t nblk = static_cast<size_t>((c.rows + L.pw - 1) / L.pw);
   L.Wb = take(static_cast<size_t>(c.rows) * L.colsb * 2);
   L.Xb = take(K * L.colsb * 2);
   L.ZT = take(K * ldz * 4);                      // logits Z, sample-major [K x ldz]
@@ -968,6 +1216,8 @@ void tc_extend_layout(const sfb_config& c, Layout& L, size_t& off) {
   L.Xf = take(K * static_cast<size_t>(c.cols) * 4);   // fp32 copy of the K samples (exact label-row term)
   L.labels = take(K * 4);                        // class ids of the K samples
   L.coef = take(K * 4);                          // 1 - p_y per sample (fp32 label entry of u)
+  L.slot = take(static_cast<size_t>(c.rows) * 4);     // per class of W: its first sample in the mini-batch (kNoSlot: none)
+  L.dL = take(K * static_cast<size_t>(c.cols) * 4);   // per such sample: the fp32 sum that the class's row of W takes
   L.U = 0;
 }
 
@@ -1012,6 +1262,8 @@ int tc_init(sfb_ctx* ctx) {
     }
     return SFB_OK;
   }
+  CKC(cudaMemsetAsync(ctx->at<char>(ctx->lay.labels), 0xff, static_cast<size_t>(ctx->K) * 4, ctx->stream));
+  CKC(cudaMemsetAsync(ctx->at<char>(ctx->lay.slot), 0x7f, static_cast<size_t>(c.rows) * 4, ctx->stream));
   // bf16 copy of W for the forward product; afterwards the update's epilogue keeps it current
   return tc_refresh_operands(ctx);
 }
@@ -1019,18 +1271,14 @@ int tc_init(sfb_ctx* ctx) {
 int tc_refresh_operands(sfb_ctx* ctx) {
   const sfb_config& c = ctx->cfg;
   if (c.model != SFB_MLR) return SFB_OK;          // the split copies of W are rebuilt by the first factors call of a step
-  const TcState* st = static_cast<const TcState*>(ctx->tc);
+  TcState* st = static_cast<TcState*>(ctx->tc);
   if (ctx->tf32) {
-    split32_rows_kernel<<<static_cast<unsigned>(st->sms * 16), 256, 0, ctx->stream>>>(ctx->W, c.rows, c.cols, c.cols,
-                                                                                     ctx->at<float>(ctx->lay.Ws), ctx->lay.colsp);
-    count_launch();
-    CKC(cudaGetLastError());
-    return SFB_OK;
+    CKC(launch_kernel(split32_rows_kernel, dim3(static_cast<unsigned>(st->sms * 16)), dim3(256), 0, ctx->stream, 1,
+                      ctx->W, c.rows, c.cols, c.cols, ctx->at<float>(ctx->lay.Ws), ctx->lay.colsp));
+      return SFB_OK;
   }
-  convert_rows_kernel<<<st->sms * 8, 256, 0, ctx->stream>>>(ctx->W, c.rows, c.cols, ctx->at<__nv_bfloat16>(ctx->lay.Wb),
-                                                            ctx->lay.colsb);
-  count_launch();
-  CKC(cudaGetLastError());
+  CKC(launch_kernel(convert_rows_kernel, dim3(st->sms * 8), dim3(256), 0, ctx->stream, 1, ctx->W, c.rows, c.cols,
+                    ctx->at<__nv_bfloat16>(ctx->lay.Wb), ctx->lay.colsb));
   return SFB_OK;
 }
 
@@ -1077,7 +1325,7 @@ constexpr int kSplitPrefetch = SFB_SPLIT_PREFETCH;    // k-blocks of look-ahead 
 template <int EPI>
 int split_product(sfb_ctx* ctx, int64_t off, int64_t n, __nv_bfloat16* A, __nv_bfloat16* B, int64_t N, int64_t Cp,
                   float* C, int64_t ldc, TcParams p, int64_t c_split_stride = 0, int* parts_out = nullptr) {
-  const TcState* st = static_cast<const TcState*>(ctx->tc);
+  TcState* st = static_cast<TcState*>(ctx->tc);
   const int bn = pick_tile_width(st->sms, (n + BM - 1) / BM, N, FS_BN, 16, EPI == F_GRAM);
   CUtensorMap ma, mb;
   if (!make_map(st, &ma, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, A, 2 * Cp, off + n, 2 * Cp * 2, BK, BM) ||
@@ -1119,12 +1367,9 @@ int factors_split(sfb_ctx* ctx, int64_t off, int64_t n, const float* X, const fl
   __nv_bfloat16* As = ctx->at<__nv_bfloat16>(L.As);
   TcParams p{};
   if (c.model == SFB_DML) {
-    CKC(pack_copy(s, V + off * cols, X, Y, n * cols));                                   // v = x - y
-    pack_split_rows_kernel<<<grid1d(n * cols / 4, 256), 256, 0, s>>>(V + off * cols, n, cols, cols,
-                                                                     As + off * 2 * L.colsp, L.colsp);
-    count_launch();
-    CKC(cudaGetLastError());
-    float* U2 = ctx->at<float>(L.U2);
+    CKC(launch_kernel(pack_pairs_kernel, dim3(grid1d(n * cols / 4, 256)), dim3(256), 0, s, 1, X, Y, n, cols,
+                      V + off * cols, As + off * 2 * L.colsp, L.colsp, Stamp{}));
+      float* U2 = ctx->at<float>(L.U2);
     int parts = 1;
     int rc = split_product<F_STORE>(ctx, off, n, As, Ws, rows, L.colsp, U, L.ldu, p, U2 - U, &parts);   // z_i = W v_i
     if (rc) return rc;
@@ -1164,11 +1409,11 @@ int factors_split(sfb_ctx* ctx, int64_t off, int64_t n, const float* X, const fl
       e.sc = ctx->at<Scalars>(L.scalars); e.lam = c.sc_lambda;
       CKC(sgemm(s, true, false, EPI_ISTA0, n, cols, rows, X, rows, ctx->W, cols, e, ctx->K));
       ctx->stats.flops += 2.0 * n * rows * cols;
-      pack_split_rows_kernel<<<grid1d(n * cols / 4, 256), 256, 0, s>>>(V + off * cols, n, cols, cols, as[1] + off * 2 * L.colsp, L.colsp);
-      count_launch();
+      CKC(launch_kernel(pack_split_rows_kernel, dim3(grid1d(n * cols / 4, 256)), dim3(256), 0, s, 1, V + off * cols, n,
+                        cols, cols, as[1] + off * 2 * L.colsp, L.colsp, Stamp{}));
     } else {
-      pack_split_rows_kernel<<<grid1d(n * ((rows + 3) / 4), 256), 256, 0, s>>>(X, n, rows, rows, Rs + off * 2 * L.rowsp, L.rowsp);
-      count_launch();
+      CKC(launch_kernel(pack_split_rows_kernel, dim3(grid1d(n * ((rows + 3) / 4), 256)), dim3(256), 0, s, 1, X, n, rows,
+                        rows, Rs + off * 2 * L.rowsp, L.rowsp, Stamp{}));
       p = ista(1);
       p.C2 = gram ? ctx->at<float>(L.Bx) : nullptr;
       if ((rc = split_product<F_ISTA0>(ctx, off, n, Rs, WTs, cols, L.rowsp, V, cols, p)) != SFB_OK) return rc;
@@ -1198,13 +1443,12 @@ int tc_begin_step(sfb_ctx* ctx) {
   const Layout& L = ctx->lay;
   const int64_t rows = c.rows, cols = c.cols;
   cudaStream_t s = ctx->stream;
-  pack_split_rows_kernel<<<grid1d(rows * cols / 4, 256), 256, 0, s>>>(ctx->W, rows, cols, cols, ctx->at<__nv_bfloat16>(L.Ws), L.colsp);
-  count_launch();
+  CKC(launch_kernel(pack_split_rows_kernel, dim3(grid1d(rows * cols / 4, 256)), dim3(256), 0, s, 1, ctx->W, rows, cols,
+                    cols, ctx->at<__nv_bfloat16>(L.Ws), L.colsp, take_stamp(ctx)));
   if (c.model == SFB_SC) {
     __nv_bfloat16* WTs = ctx->at<__nv_bfloat16>(L.WTs);
-    pack_split_t_kernel<<<dim3(static_cast<unsigned>((cols + 63) / 64), static_cast<unsigned>(L.rowsp / 64)), 256, 0, s>>>(
-        ctx->W, rows, cols, cols, WTs, L.rowsp);
-    count_launch();
+    CKC(launch_kernel(pack_split_t_kernel, dim3(static_cast<unsigned>((cols + 63) / 64),
+                      static_cast<unsigned>(L.rowsp / 64)), dim3(256), 0, s, 1, ctx->W, rows, cols, cols, WTs, L.rowsp));
     if (L.Gs) {
       TcParams p{};
       p.four = rows <= kPreciseRows;
@@ -1214,7 +1458,6 @@ int tc_begin_step(sfb_ctx* ctx) {
       if (rc) return rc;
     }
   }
-  CKC(cudaGetLastError());
   return SFB_OK;
 }
 
@@ -1232,7 +1475,7 @@ double split_product_cost(int64_t M, int64_t N, int64_t Kc, bool sym) {
 // the three-term tf32 product, with the per-(sample, 256-row block) softmax partials.
 static int mlr32_forward(sfb_ctx* ctx, int64_t off, int64_t n, const float* X, int* tiles_n) {
   const sfb_config& c = ctx->cfg;
-  const TcState* st = static_cast<const TcState*>(ctx->tc);
+  TcState* st = static_cast<TcState*>(ctx->tc);
   const Layout& L = ctx->lay;
   const int64_t rows = c.rows, cols = c.cols, K = ctx->K;
   const int64_t ldz = round_up(rows, 32);
@@ -1242,10 +1485,9 @@ static int mlr32_forward(sfb_ctx* ctx, int64_t off, int64_t n, const float* X, i
   float* Z = ctx->at<float>(L.ZT);
   float* V = ctx->at<float>(L.V) + off * cols;
   // Ws, the (big | small) copy of W, is built at set-up and rewritten by the update's epilogue together with W
-  CKC(pack_copy(s, V, X, nullptr, n * cols));                                              // v = x
-  split32_rows_kernel<<<grid1d(n * cols / 4, 256), 256, 0, s>>>(X, n, cols, cols, As + off * 2 * L.colsp, L.colsp);
-  count_launch();
-  CKC(cudaGetLastError());
+  CKC(pack_copy(s, V, X, nullptr, n * cols, take_stamp(ctx)));                             // v = x
+  CKC(launch_kernel(split32_rows_kernel, dim3(grid1d(n * cols / 4, 256)), dim3(256), 0, s, 1, X, n, cols, cols,
+                    As + off * 2 * L.colsp, L.colsp));
   CUtensorMap ma, mb, mc;
   if (!make_map(st, &ma, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, As, 2 * L.colsp, off + n, 2 * L.colsp * 4, BK / 2, BM) ||
       !make_map(st, &mb, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, Ws, 2 * L.colsp, rows, 2 * L.colsp * 4, BK / 2, BN) ||
@@ -1255,7 +1497,7 @@ static int mlr32_forward(sfb_ctx* ctx, int64_t off, int64_t n, const float* X, i
   p.M = static_cast<int32_t>(off + n); p.N = static_cast<int32_t>(rows); p.Kc = static_cast<int32_t>(L.colsp);
   p.m_off = static_cast<int32_t>(off);
   p.tilesM = static_cast<int32_t>((n + BM - 1) / BM);
-  p.bn = BN;
+  p.bn = BN; p.pw = BN; p.a_rows = BM; p.stages = S;
   p.tilesN = static_cast<int32_t>((rows + BN - 1) / BN);
   p.part = ctx->at<float2>(L.part); p.part_ld = K; p.status = ctx->at<uint32_t>(L.status);
   p.nseg = 3; p.kseg = static_cast<int32_t>(L.colsp / (BK / 2));          // cross terms first, big*big last
@@ -1275,11 +1517,9 @@ int tc32_forward_partials(sfb_ctx* ctx, const float* X, const int32_t* labels, f
   const int rc = mlr32_forward(ctx, 0, ctx->K, X, &tiles_n);
   if (rc) return rc;
   CKC(cudaMemcpyAsync(ctx->at<int32_t>(L.labels), labels, static_cast<size_t>(ctx->K) * 4, cudaMemcpyDeviceToDevice, ctx->stream));
-  mlr_shard_partials_tc_kernel<<<static_cast<unsigned>((ctx->K + 7) / 8), 256, 0, ctx->stream>>>(
-      ctx->at<float2>(L.part), ctx->K, tiles_n, ctx->at<float>(L.ZT), round_up(c.rows, 32), c.rows,
-      ctx->at<int32_t>(L.labels), ctx->row_offset, ctx->K, reinterpret_cast<float4*>(part_out));
-  count_launch();
-  CKC(cudaGetLastError());
+  CKC(launch_kernel(mlr_shard_partials_tc_kernel, dim3(static_cast<unsigned>((ctx->K + 7) / 8)), dim3(256), 0,
+                    ctx->stream, 1, ctx->at<float2>(L.part), ctx->K, tiles_n, ctx->at<float>(L.ZT), round_up(c.rows, 32),
+                    c.rows, ctx->at<int32_t>(L.labels), ctx->row_offset, ctx->K, reinterpret_cast<float4*>(part_out)));
   return SFB_OK;
 }
 
@@ -1288,15 +1528,13 @@ int tc32_finish_factors(sfb_ctx* ctx, const float* parts, int shards) {
   const sfb_config& c = ctx->cfg;
   const Layout& L = ctx->lay;
   const int64_t K = ctx->K, rows = c.rows;
-  mlr_shard_finish_tc_kernel<<<static_cast<unsigned>((K + 255) / 256), 256, 0, ctx->stream>>>(
-      reinterpret_cast<const float4*>(parts), shards, K, rows, ctx->row_offset, ctx->at<int32_t>(L.labels),
-      ctx->at<float>(L.lse), ctx->at<float>(L.loss), ctx->at<float>(L.coef), ctx->at<uint32_t>(L.status));
-  count_launch();
+  CKC(launch_kernel(mlr_shard_finish_tc_kernel, dim3(static_cast<unsigned>((K + 255) / 256)), dim3(256), 0, ctx->stream,
+                    1, reinterpret_cast<const float4*>(parts), shards, K, rows, ctx->row_offset,
+                    ctx->at<int32_t>(L.labels), ctx->at<float>(L.lse), ctx->at<float>(L.loss), ctx->at<float>(L.coef),
+                    ctx->at<uint32_t>(L.status)));
   dim3 ugrid(static_cast<unsigned>(std::min<int64_t>((rows + 255) / 256, 64)), static_cast<unsigned>(K));
-  mlr_finish_u_kernel<false><<<ugrid, 256, 0, ctx->stream>>>(ctx->at<float>(L.ZT), round_up(rows, 32), rows, ctx->at<float>(L.lse),
-                                                             ctx->at<int32_t>(L.labels), ctx->at<float>(L.U));
-  count_launch();
-  CKC(cudaGetLastError());
+  CKC(launch_kernel(mlr_finish_u_kernel<false>, ugrid, dim3(256), 0, ctx->stream, 1, ctx->at<float>(L.ZT), round_up(rows,
+                    32), rows, ctx->at<float>(L.lse), ctx->at<int32_t>(L.labels), ctx->at<float>(L.U)));
   return SFB_OK;
 }
 
@@ -1321,17 +1559,15 @@ int tc32_factors(sfb_ctx* ctx, int64_t off, int64_t n, const float* X, const int
   if (sdca_ids) {
     CKC(sdca_dual_rows(s, Z + off * ldz, n, rows, ldz, X, cols, labels, sdca_ids, ctx->dualQ, ctx->dual_n, inv_lam_n, c.eta,
                        nullptr, ctx->at<float>(L.loss) + off, ctx->at<uint32_t>(L.status)));
-    mlr_finish_u_kernel<true><<<ugrid, 256, 0, s>>>(Z + off * ldz, ldz, rows, nullptr, nullptr, U);
+    CKC(launch_kernel(mlr_finish_u_kernel<true>, ugrid, dim3(256), 0, s, 1, Z + off * ldz, ldz, rows, nullptr, nullptr, U));
   } else {
     float* lse = ctx->at<float>(L.lse);
-    mlr_lse_kernel<<<static_cast<unsigned>((n + 7) / 8), 256, 0, s>>>(ctx->at<float2>(L.part), K, tiles_n, Z, ldz, rows, labels,
-                                                                     off, n, lse, ctx->at<float>(L.loss),
-                                                                     ctx->at<float>(L.coef), ctx->at<uint32_t>(L.status));
-    count_launch();
-    mlr_finish_u_kernel<false><<<ugrid, 256, 0, s>>>(Z + off * ldz, ldz, rows, lse + off, labels, U);
+    CKC(launch_kernel(mlr_lse_kernel, dim3(static_cast<unsigned>((n + 7) / 8)), dim3(256), 0, s, 1,
+                      ctx->at<float2>(L.part), K, tiles_n, Z, ldz, rows, labels, off, n, lse, ctx->at<float>(L.loss),
+                      ctx->at<float>(L.coef), nullptr, ctx->at<uint32_t>(L.status)));
+    CKC(launch_kernel(mlr_finish_u_kernel<false>, ugrid, dim3(256), 0, s, 1, Z + off * ldz, ldz, rows, lse + off, labels,
+                      U));
   }
-  count_launch();
-  CKC(cudaGetLastError());
   return SFB_OK;
 }
 
@@ -1340,46 +1576,92 @@ int tc32_gather(sfb_ctx* ctx) {
   const sfb_config& c = ctx->cfg;
   const Layout& L = ctx->lay;
   const unsigned gy = static_cast<unsigned>((L.Kp + 63) / 64);
-  split32_t_kernel<<<dim3(static_cast<unsigned>((c.rows + 63) / 64), gy), 256, 0, ctx->stream>>>(
-      ctx->at<float>(L.U), ctx->K, c.rows, c.rows, ctx->at<float>(L.UT), L.Kp);
-  count_launch();
-  split32_t_kernel<<<dim3(static_cast<unsigned>((c.cols + 63) / 64), gy), 256, 0, ctx->stream>>>(
-      ctx->at<float>(L.V), ctx->K, c.cols, c.cols, ctx->at<float>(L.VT), L.Kp);
-  count_launch();
-  CKC(cudaGetLastError());
+  CKC(launch_kernel(split32_t_kernel, dim3(static_cast<unsigned>((c.rows + 63) / 64), gy), dim3(256), 0, ctx->stream, 1,
+                    ctx->at<float>(L.U), ctx->K, c.rows, c.rows, ctx->at<float>(L.UT), L.Kp));
+  CKC(launch_kernel(split32_t_kernel, dim3(static_cast<unsigned>((c.cols + 63) / 64), gy), dim3(256), 0, ctx->stream, 1,
+                    ctx->at<float>(L.V), ctx->K, c.cols, c.cols, ctx->at<float>(L.VT), L.Kp));
   return SFB_OK;
 }
 
 // Pack of n samples at pair offset off and their logits against the rows of this context's W:
-// Z[off .. off+n) = X W^T with the per-(sample, 256-row block) softmax partials.
-static int mlr_forward(sfb_ctx* ctx, int64_t off, int64_t n, const float* X, const int32_t* labels, int* tiles_n) {
+// Z[off .. off+n) = X W^T with the softmax partials.  fused: see tc_factors.
+static int mlr_forward(sfb_ctx* ctx, int64_t off, int64_t n, const float* X, const int32_t* labels, bool fused, int* parts) {
   const sfb_config& c = ctx->cfg;
-  const TcState* st = static_cast<const TcState*>(ctx->tc);
+  TcState* st = static_cast<TcState*>(ctx->tc);
   const Layout& L = ctx->lay;
   const int64_t rows = c.rows, cols = c.cols, K = ctx->K;
   const int64_t ldz = round_up(rows, 32);
   __nv_bfloat16* Xb = ctx->at<__nv_bfloat16>(L.Xb);
-  pack_mlr_kernel<<<grid1d(n * cols / 4, 256), 256, 0, ctx->stream>>>(X, n, cols, Xb, L.colsb, off, ctx->at<float>(L.Xf), labels,
-                                                                      ctx->at<int32_t>(L.labels));
-  count_launch();
-  CKC(cudaGetLastError());
+  ctx->labels = sfb_ctx::kLabelsNone;
+  CKC(launch_kernel(pack_mlr_kernel, dim3(grid1d(n * cols / 4, 256)), dim3(256), 0, ctx->stream, 1, X, n, cols, Xb,
+                    L.colsb, off,
+                    fused ? nullptr : ctx->at<float>(L.Xf), labels, ctx->at<int32_t>(L.labels), ctx->at<int32_t>(L.slot),
+                    rows,
+                    take_stamp(ctx)));
   // samples on the lanes (A), rows of W on the accumulator columns (B)
+  const int bn = pick_forward_width(n, rows, cols, L.pw);
+  const int ar = static_cast<int>(std::min<int64_t>(BM, round_up(n, 8)));
   CUtensorMap ma, mb, mc;
-  if (!make_map(st, &ma, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, Xb, cols, off + n, L.colsb * 2, BK, BM) ||
-      !make_map(st, &mb, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, ctx->at<__nv_bfloat16>(L.Wb), cols, rows, L.colsb * 2, BK, BN) ||
+  if (!make_map(st, &ma, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, Xb, cols, K, L.colsb * 2, BK, ar) ||
+      !make_map(st, &mb, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, ctx->at<__nv_bfloat16>(L.Wb), cols, rows, L.colsb * 2, BK, bn) ||
       !make_map(st, &mc, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, ctx->at<float>(L.ZT), rows, off + n, ldz * 4, kChunk, 32))
     return SFB_ERR_CUDA;
   TcParams p{};
   p.M = static_cast<int32_t>(off + n); p.N = static_cast<int32_t>(rows); p.Kc = static_cast<int32_t>(cols);
   p.m_off = static_cast<int32_t>(off);
   p.tilesM = static_cast<int32_t>((n + BM - 1) / BM);
-  p.bn = BN;
-  p.tilesN = static_cast<int32_t>((rows + BN - 1) / BN);
+  p.bn = bn; p.pw = L.pw; p.a_rows = ar; p.stages = forward_stages(bn);
+  p.tilesN = static_cast<int32_t>((rows + bn - 1) / bn);
   p.part = ctx->at<float2>(L.part); p.part_ld = K; p.status = ctx->at<uint32_t>(L.status);
   p.nseg = 1; p.kseg = (p.Kc + BK - 1) / BK;
   CKC(launch_forward<F_SOFTMAX>(ctx, ma, mb, mc, p));
   ctx->stats.flops += 2.0 * n * rows * cols;
-  *tiles_n = p.tilesN;
+  *parts = static_cast<int>((rows + L.pw - 1) / L.pw);
+  return SFB_OK;
+}
+
+static LabelArgs label_args(sfb_ctx* ctx, const float* X) {
+  const Layout& L = ctx->lay;
+  LabelArgs a{};
+  a.X = X;
+  a.labels = ctx->at<int32_t>(L.labels); a.slot = ctx->at<int32_t>(L.slot); a.coef = ctx->at<float>(L.coef);
+  a.dL = ctx->at<float>(L.dL);
+  a.loss = ctx->at<float>(L.loss); a.loss_mean = &ctx->at<Scalars>(L.scalars)->loss_mean;
+  a.rows = ctx->cfg.rows; a.cols = ctx->cfg.cols; a.K = static_cast<int32_t>(ctx->K);
+  a.W = ctx->W; a.Wb = ctx->at<__nv_bfloat16>(L.Wb); a.ldw = L.colsb; a.step = ctx->step;
+  return a;
+}
+static int label_blocks(const sfb_ctx* ctx) {
+  return static_cast<int>(std::min<int64_t>(ctx->K * ((ctx->cfg.cols + kLabelCols - 1) / kLabelCols), 6 * sm_count()));
+}
+
+// Probabilities (or, PLAIN, the values of Z) of n samples as the operand of the update; fused: and the label rows applied.
+template <bool PLAIN>
+static int emit_p(sfb_ctx* ctx, int64_t off, int64_t n, const int32_t* labels, const float* fused_X) {
+  const Layout& L = ctx->lay;
+  const int64_t rows = ctx->cfg.rows;
+  const int lab = fused_X ? label_blocks(ctx) : 0;
+  CKC(launch_kernel(mlr_emit_p_kernel<PLAIN>, dim3(grid1d(n * ((rows + 7) / 8), 256) + lab), dim3(256), 0, ctx->stream, 1,
+                    ctx->at<float>(L.ZT), round_up(rows, 32), rows, ctx->at<float>(L.V), off, n, labels,
+                    ctx->at<__nv_bfloat16>(L.P), L.ldp, lab, label_args(ctx, fused_X)));
+  if (fused_X) ctx->labels = sfb_ctx::kLabelsApplied;
+  return SFB_OK;
+}
+
+int tc_labels(sfb_ctx* ctx) {
+  if (ctx->labels == sfb_ctx::kLabelsApplied) {           // by the factors call of this step
+    ctx->labels = sfb_ctx::kLabelsKept;
+    return SFB_OK;
+  }
+  const Layout& L = ctx->lay;
+  LabelArgs a = label_args(ctx, ctx->at<float>(L.Xf));
+  a.again = ctx->labels == sfb_ctx::kLabelsKept;          // a repeated update
+  if (!a.again)
+    CKC(launch_kernel(label_slots_kernel, dim3(static_cast<unsigned>((ctx->K + 255) / 256)), dim3(256), 0, ctx->stream, 1,
+                      ctx->at<int32_t>(L.labels), static_cast<int32_t>(ctx->K), ctx->cfg.rows, ctx->at<int32_t>(L.slot),
+                      take_stamp(ctx)));
+  CKC(launch_kernel(label_delta_kernel, dim3(static_cast<unsigned>(label_blocks(ctx))), dim3(256), 0, ctx->stream, 1, a));
+  ctx->labels = sfb_ctx::kLabelsKept;
   return SFB_OK;
 }
 
@@ -1387,13 +1669,11 @@ int tc_forward_partials(sfb_ctx* ctx, const float* X, const int32_t* labels, flo
   const sfb_config& c = ctx->cfg;
   const Layout& L = ctx->lay;
   int tiles_n = 0;
-  const int rc = mlr_forward(ctx, 0, ctx->K, X, labels, &tiles_n);
+  const int rc = mlr_forward(ctx, 0, ctx->K, X, labels, false, &tiles_n);
   if (rc) return rc;
-  mlr_shard_partials_tc_kernel<<<static_cast<unsigned>((ctx->K + 7) / 8), 256, 0, ctx->stream>>>(
-      ctx->at<float2>(L.part), ctx->K, tiles_n, ctx->at<float>(L.ZT), round_up(c.rows, 32), c.rows,
-      ctx->at<int32_t>(L.labels), ctx->row_offset, ctx->K, reinterpret_cast<float4*>(part_out));
-  count_launch();
-  CKC(cudaGetLastError());
+  CKC(launch_kernel(mlr_shard_partials_tc_kernel, dim3(static_cast<unsigned>((ctx->K + 7) / 8)), dim3(256), 0,
+                    ctx->stream, 1, ctx->at<float2>(L.part), ctx->K, tiles_n, ctx->at<float>(L.ZT), round_up(c.rows, 32),
+                    c.rows, ctx->at<int32_t>(L.labels), ctx->row_offset, ctx->K, reinterpret_cast<float4*>(part_out)));
   return SFB_OK;
 }
 
@@ -1401,23 +1681,21 @@ int tc_finish_factors(sfb_ctx* ctx, const float* parts, int shards) {
   const sfb_config& c = ctx->cfg;
   const Layout& L = ctx->lay;
   const int64_t K = ctx->K;
-  mlr_shard_finish_tc_kernel<<<static_cast<unsigned>((K + 255) / 256), 256, 0, ctx->stream>>>(
-      reinterpret_cast<const float4*>(parts), shards, K, c.rows, ctx->row_offset, ctx->at<int32_t>(L.labels),
-      ctx->at<float>(L.V), ctx->at<float>(L.loss), ctx->at<float>(L.coef), ctx->at<uint32_t>(L.status));
-  count_launch();
-  mlr_emit_p_kernel<false><<<grid1d(K * ((c.rows + 7) / 8), 256), 256, 0, ctx->stream>>>(
-      ctx->at<float>(L.ZT), round_up(c.rows, 32), c.rows, ctx->at<float>(L.V), 0, K, ctx->at<int32_t>(L.labels),
-      ctx->at<__nv_bfloat16>(L.P), L.ldp);
-  count_launch();
-  CKC(cudaGetLastError());
-  return SFB_OK;
+  CKC(launch_kernel(mlr_shard_finish_tc_kernel, dim3(static_cast<unsigned>((K + 255) / 256)), dim3(256), 0, ctx->stream,
+                    1, reinterpret_cast<const float4*>(parts), shards, K, c.rows, ctx->row_offset,
+                    ctx->at<int32_t>(L.labels), ctx->at<float>(L.V), ctx->at<float>(L.loss), ctx->at<float>(L.coef),
+                    ctx->at<uint32_t>(L.status)));
+  return emit_p<false>(ctx, 0, K, ctx->at<int32_t>(L.labels), nullptr);
 }
 
 // What a worker sends (Section 3) in bf16 mode: u_ij = exp(z_ij - lse_i) - [j = y_i] in fp32 from the logits and the
 // log-partition it holds; one block row per sample.
 __global__ void __launch_bounds__(256) mlr_export_u_kernel(const float* __restrict__ Z, int64_t ldz, int64_t rows,
-                                                           const float* __restrict__ lse, const int32_t* __restrict__ labels,
+                                                           const float* __restrict__ lse,
+                                                           const int32_t* __restrict__ labels,
                                                            int64_t off, float* __restrict__ U_out) {
+  pdl_launch_dependents();
+  pdl_wait();
   const int64_t i = blockIdx.y;
   const float l = lse[off + i];
   const int32_t y = labels[off + i];
@@ -1433,7 +1711,9 @@ __global__ void __launch_bounds__(256) mlr_export_u_kernel(const float* __restri
 // ties (none for a valid u) go to the smaller index.
 __global__ void __launch_bounds__(256) mlr_import_labels_kernel(const float* __restrict__ U_in, int64_t rows, int64_t off,
                                                                 int32_t* __restrict__ labels, float* __restrict__ coef,
-                                                                float* __restrict__ loss) {
+                                                                float* __restrict__ loss, int32_t* __restrict__ slot) {
+  pdl_launch_dependents();
+  pdl_wait();
   __shared__ float sv[256];
   __shared__ int32_t si[256];
   const int64_t i = blockIdx.x;
@@ -1456,6 +1736,8 @@ __global__ void __launch_bounds__(256) mlr_import_labels_kernel(const float* __r
   }
   if (threadIdx.x == 0) {
     const float c = fminf(fmaxf(-sv[0], 0.f), 1.f);
+    const int32_t old = labels[off + i];
+    if (old >= 0 && old < rows) slot[old] = kNoSlot;
     labels[off + i] = si[0];
     coef[off + i] = c;
     loss[off + i] = -logf(fmaxf(1.f - c, 1e-37f));
@@ -1467,10 +1749,8 @@ int tc_export_factors(sfb_ctx* ctx, int64_t off, int64_t n, float* U_out, float*
   const Layout& L = ctx->lay;
   const int64_t ldz = round_up(c.rows, 32);
   dim3 grid(static_cast<unsigned>(std::min<int64_t>((c.rows + 255) / 256, 64)), static_cast<unsigned>(n));
-  mlr_export_u_kernel<<<grid, 256, 0, ctx->stream>>>(ctx->at<float>(L.ZT), ldz, c.rows, ctx->at<float>(L.V),
-                                                     ctx->at<int32_t>(L.labels), off, U_out);
-  count_launch();
-  CKC(cudaGetLastError());
+  CKC(launch_kernel(mlr_export_u_kernel, grid, dim3(256), 0, ctx->stream, 1, ctx->at<float>(L.ZT), ldz, c.rows,
+                    ctx->at<float>(L.V), ctx->at<int32_t>(L.labels), off, U_out));
   CKC(cudaMemcpyAsync(V_out, ctx->at<float>(L.Xf) + off * c.cols, static_cast<size_t>(n) * c.cols * 4, cudaMemcpyDeviceToDevice,
                       ctx->stream));
   return SFB_OK;
@@ -1485,44 +1765,37 @@ int tc_import_factors(sfb_ctx* ctx, int64_t off, int64_t n, const float* U_in, c
   const int64_t ldz = round_up(rows, 32);
   cudaStream_t s = ctx->stream;
   int32_t* labels = ctx->at<int32_t>(L.labels);
-  mlr_import_labels_kernel<<<static_cast<unsigned>(n), 256, 0, s>>>(U_in, rows, off, labels, ctx->at<float>(L.coef),
-                                                                   ctx->at<float>(L.loss));
-  count_launch();
+  ctx->labels = sfb_ctx::kLabelsNone;
+  CKC(launch_kernel(mlr_import_labels_kernel, dim3(static_cast<unsigned>(n)), dim3(256), 0, s, 1, U_in, rows, off, labels,
+                    ctx->at<float>(L.coef), ctx->at<float>(L.loss), ctx->at<int32_t>(L.slot)));
   float* Z = ctx->at<float>(L.ZT);
   CKC(cudaMemcpy2DAsync(Z + off * ldz, static_cast<size_t>(ldz) * 4, U_in, static_cast<size_t>(rows) * 4,
                         static_cast<size_t>(rows) * 4, static_cast<size_t>(n), cudaMemcpyDeviceToDevice, s));
-  pack_mlr_kernel<<<grid1d(n * cols / 4, 256), 256, 0, s>>>(V_in, n, cols, ctx->at<__nv_bfloat16>(L.Xb), L.colsb, off,
-                                                            ctx->at<float>(L.Xf), labels + off, labels);
-  count_launch();
-  mlr_emit_p_kernel<true><<<grid1d(n * ((rows + 7) / 8), 256), 256, 0, s>>>(Z, ldz, rows, nullptr, off, n, labels + off,
-                                                                            ctx->at<__nv_bfloat16>(L.P), L.ldp);
-  count_launch();
-  CKC(cudaGetLastError());
-  return SFB_OK;
+  CKC(launch_kernel(pack_mlr_kernel, dim3(grid1d(n * cols / 4, 256)), dim3(256), 0, s, 1, V_in, n, cols,
+                    ctx->at<__nv_bfloat16>(L.Xb), L.colsb, off, ctx->at<float>(L.Xf), labels + off, labels,
+                    ctx->at<int32_t>(L.slot), rows, Stamp{}));
+  return emit_p<true>(ctx, off, n, labels + off, nullptr);
 }
 
 // SDCA factors in bf16 mode: logits by the forward product, the dual changes in fp32 in place of the logits, then the
 // bf16 operand U^T = du (0 at the label entry, which goes to W in fp32 through coef, as for MLR).
 int tc_sdca_factors(sfb_ctx* ctx, int64_t off, int64_t n, const float* X, const int32_t* labels, const int32_t* ids,
-                    float inv_lam_n) {
+                    float inv_lam_n, bool fused) {
   const sfb_config& c = ctx->cfg;
   const Layout& L = ctx->lay;
   const int64_t rows = c.rows;
   const int64_t ldz = round_up(rows, 32);
   float* Z = ctx->at<float>(L.ZT);
   int tiles_n = 0;
-  const int rc = mlr_forward(ctx, off, n, X, labels, &tiles_n);
+  const int rc = mlr_forward(ctx, off, n, X, labels, fused, &tiles_n);
   if (rc) return rc;
   CKC(sdca_dual_rows(ctx->stream, Z + off * ldz, n, rows, ldz, X, c.cols, labels, ids, ctx->dualQ, ctx->dual_n, inv_lam_n,
-                     c.eta, ctx->at<float>(L.coef) + off, ctx->at<float>(L.loss) + off, ctx->at<uint32_t>(L.status)));
-  mlr_emit_p_kernel<true><<<grid1d(n * ((rows + 7) / 8), 256), 256, 0, ctx->stream>>>(Z, ldz, rows, nullptr, off, n, labels,
-                                                                                      ctx->at<__nv_bfloat16>(L.P), L.ldp);
-  count_launch();
-  CKC(cudaGetLastError());
-  return SFB_OK;
+                     c.eta, ctx->at<float>(L.coef) + off, ctx->at<float>(L.loss) + off, ctx->at<uint32_t>(L.status),
+                     fused ? ctx->at<int32_t>(L.slot) : nullptr, off));
+  return emit_p<true>(ctx, off, n, labels, fused ? X : nullptr);
 }
 
-int tc_factors(sfb_ctx* ctx, int64_t off, int64_t n, const float* X, const float* Y, const int32_t* labels,
+int tc_factors(sfb_ctx* ctx, int64_t off, int64_t n, const float* X, const float* Y, const int32_t* labels, bool fused,
                float* dml_norm_out) {
   if (ctx->cfg.model != SFB_MLR) return factors_split(ctx, off, n, X, Y, labels, dml_norm_out);
   const sfb_config& c = ctx->cfg;
@@ -1532,17 +1805,12 @@ int tc_factors(sfb_ctx* ctx, int64_t off, int64_t n, const float* X, const float
   float* Z = ctx->at<float>(L.ZT);
   float* lse = ctx->at<float>(L.V);
   int tiles_n = 0;
-  const int rc = mlr_forward(ctx, off, n, X, labels, &tiles_n);
+  const int rc = mlr_forward(ctx, off, n, X, labels, fused, &tiles_n);
   if (rc) return rc;
-  mlr_lse_kernel<<<static_cast<unsigned>((n + 7) / 8), 256, 0, ctx->stream>>>(
-      ctx->at<float2>(L.part), K, tiles_n, Z, ldz, rows, labels, off, n, lse, ctx->at<float>(L.loss), ctx->at<float>(L.coef),
-      ctx->at<uint32_t>(L.status));
-  count_launch();
-  mlr_emit_p_kernel<false><<<grid1d(n * ((rows + 7) / 8), 256), 256, 0, ctx->stream>>>(Z, ldz, rows, lse, off, n, labels,
-                                                                                       ctx->at<__nv_bfloat16>(L.P), L.ldp);
-  count_launch();
-  CKC(cudaGetLastError());
-  return SFB_OK;
+  CKC(launch_kernel(mlr_lse_kernel, dim3(static_cast<unsigned>((n + 7) / 8)), dim3(256), 0, ctx->stream, 1,
+                    ctx->at<float2>(L.part), K, tiles_n, Z, ldz, rows, labels, off, n, lse, ctx->at<float>(L.loss),
+                    ctx->at<float>(L.coef), fused ? ctx->at<int32_t>(L.slot) : nullptr, ctx->at<uint32_t>(L.status)));
+  return emit_p<false>(ctx, off, n, labels, fused ? X : nullptr);
 }
 
 // The (hi | lo) codes or pair differences: the operand V of the update.
@@ -1557,13 +1825,12 @@ int tc_pack_received(sfb_ctx* ctx, int64_t off, int64_t n) {
   const sfb_config& c = ctx->cfg;
   const Layout& L = ctx->lay;
   cudaStream_t s = ctx->stream;
-  pack_split_rows_kernel<<<grid1d(n * ((c.rows + 3) / 4), 256), 256, 0, s>>>(ctx->at<float>(L.U) + off * L.ldu, n, c.rows, L.ldu,
-                                                                            ctx->at<__nv_bfloat16>(L.Rs) + off * 2 * L.rowsp, L.rowsp);
-  count_launch();
-  pack_split_rows_kernel<<<grid1d(n * c.cols / 4, 256), 256, 0, s>>>(ctx->at<float>(L.V) + off * c.cols, n, c.cols, c.cols,
-                                                                     tc_split_v(ctx) + off * 2 * L.colsp, L.colsp);
-  count_launch();
-  CKC(cudaGetLastError());
+  CKC(launch_kernel(pack_split_rows_kernel, dim3(grid1d(n * ((c.rows + 3) / 4), 256)), dim3(256), 0, s, 1,
+                    ctx->at<float>(L.U) + off * L.ldu, n, c.rows, L.ldu, ctx->at<__nv_bfloat16>(L.Rs) + off * 2 * L.rowsp,
+                    L.rowsp, Stamp{}));
+  CKC(launch_kernel(pack_split_rows_kernel, dim3(grid1d(n * c.cols / 4, 256)), dim3(256), 0, s, 1,
+                    ctx->at<float>(L.V) + off * c.cols, n, c.cols, c.cols, tc_split_v(ctx) + off * 2 * L.colsp, L.colsp,
+                    Stamp{}));
   return SFB_OK;
 }
 

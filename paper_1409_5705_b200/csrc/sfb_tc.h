@@ -26,14 +26,18 @@ int tc_refresh_operands(sfb_ctx* ctx);
 int tc_begin_step(sfb_ctx* ctx);
 double split_product_cost(int64_t M, int64_t N, int64_t Kc, bool sym);
 // dml_norm_out (DML, row-sharded form; may be null): receives ||z_i||^2 of this context's rows and z stays unscaled.
-int tc_factors(sfb_ctx* ctx, int64_t off, int64_t n, const float* X, const float* Y, const int32_t* labels,
+// fused: the call is part of one that goes on to the update, so X stays as it is until then.
+int tc_factors(sfb_ctx* ctx, int64_t off, int64_t n, const float* X, const float* Y, const int32_t* labels, bool fused,
                float* dml_norm_out = nullptr);
 // Row-sharded MLR: logits and softmax partials of all K samples against this context's rows; then the factors from
 // the partials of all shards.
 int tc_forward_partials(sfb_ctx* ctx, const float* X, const int32_t* labels, float* part_out);
 int tc_finish_factors(sfb_ctx* ctx, const float* parts, int shards);
 int tc_sdca_factors(sfb_ctx* ctx, int64_t off, int64_t n, const float* X, const int32_t* labels, const int32_t* ids,
-                    float inv_lam_n);
+                    float inv_lam_n, bool fused);
+// MLR in bf16 mode: the fp32 label entries of all K samples into W and the mean loss, unless the factors call has done that
+// (fused); before the update.
+int tc_labels(sfb_ctx* ctx);
 // MLR, bf16 mode: a worker's factors in fp32 as they are sent, and received fp32 factors put into the bf16 layout.
 int tc_export_factors(sfb_ctx* ctx, int64_t off, int64_t n, float* U_out, float* V_out);
 int tc_import_factors(sfb_ctx* ctx, int64_t off, int64_t n, const float* U_in, const float* V_in);
@@ -48,23 +52,49 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t,
                                   const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
                                   CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
+struct MapKey {
+  void* base;
+  int64_t inner, outer, pitch;
+  int32_t dt, box_inner, box_outer;
+  bool operator==(const MapKey& o) const {
+    return base == o.base && inner == o.inner && outer == o.outer && pitch == o.pitch && dt == o.dt && box_inner == o.box_inner &&
+           box_outer == o.box_outer;
+  }
+};
+
 struct TcState {
+  // tensor maps made so far: the buffers of a context stay where they are, so a step finds all of its maps here
+  static constexpr int kMaps = 256;
+  MapKey key[kMaps];
+  CUtensorMap map[kMaps];
   EncodeTiledFn encode;      // cuTensorMapEncodeTiled, obtained through the runtime's driver entry point query
   int sms;                   // multiprocessors of the device
   int max_pairs;             // CTA pairs (clusters of 2) of the update kernel that can be resident at once
 };
 
 // 2-D row-major tensor [outer x inner] with row pitch `pitch_bytes`, box [box_outer x box_inner], 128-byte swizzle.
-inline bool make_map(const TcState* st, CUtensorMap* m, CUtensorMapDataType dt, void* base, int64_t inner,
+inline bool make_map(TcState* st, CUtensorMap* m, CUtensorMapDataType dt, void* base, int64_t inner,
                      int64_t outer, int64_t pitch_bytes, int box_inner, int box_outer) {
   if (inner <= 0 || outer <= 0) return false;
-  cuuint64_t dims[2] = {static_cast<cuuint64_t>(inner), static_cast<cuuint64_t>(outer)};
-  cuuint64_t strides[1] = {static_cast<cuuint64_t>(pitch_bytes)};
-  cuuint32_t box[2] = {static_cast<cuuint32_t>(box_inner), static_cast<cuuint32_t>(box_outer)};
-  cuuint32_t estr[2] = {1, 1};
-  return st->encode(m, dt, 2, base, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                    CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+  const MapKey k{base, inner, outer, pitch_bytes, static_cast<int32_t>(dt), box_inner, box_outer};
+  uint64_t h = reinterpret_cast<uintptr_t>(base) / 1024 * 31 + static_cast<uint64_t>(outer) * 7 + static_cast<uint64_t>(inner) * 3 +
+               static_cast<uint64_t>(box_outer);
+  const int slot = static_cast<int>((h ^ (h >> 17)) % TcState::kMaps);
+  if (!(st->key[slot] == k)) {
+    cuuint64_t dims[2] = {static_cast<cuuint64_t>(inner), static_cast<cuuint64_t>(outer)};
+    cuuint64_t strides[1] = {static_cast<cuuint64_t>(pitch_bytes)};
+    cuuint32_t box[2] = {static_cast<cuuint32_t>(box_inner), static_cast<cuuint32_t>(box_outer)};
+    cuuint32_t estr[2] = {1, 1};
+    if (st->encode(&st->map[slot], dt, 2, base, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                   CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS) {
+      st->key[slot] = MapKey{};
+      return false;
+    }
+    st->key[slot] = k;
+  }
+  *m = st->map[slot];
+  return true;
 }
 
 // Fills st->max_pairs (occupancy query of the update kernel); defined beside that kernel.

@@ -32,7 +32,7 @@ namespace {
 using namespace ptx;
 
 constexpr int UM = 128;                 // rows of W per CTA (256 per pair)
-constexpr int UN = 256;                 // columns of W per tile
+constexpr int UN = 256;                 // columns of W per tile, at most (128 for small matrices, see tile_width)
 constexpr int UK = 64, UMMA_K = 16;
 constexpr int kStages = 4;
 constexpr int kBytesA = UM * UK * 2;          // 16 KB: this CTA's rows of U^T
@@ -44,14 +44,14 @@ constexpr int kRing = 3;                      // slots per epilogue warp
 constexpr int kPend = 1;                      // TMA stores of a warp that may still be reading their slots
 constexpr int kEpiWarps = 8;
 constexpr int kThreads = 64 + 32 * kEpiWarps;
-constexpr int kChunksPerWarp = (UN / 2) / kChunk;   // 4
 constexpr int kTmemCols = 512;
 constexpr int kBars = 2 * kStages + 4 + kEpiWarps * kRing;
 constexpr int kSmem = kStages * kStageBytes + kEpiWarps * kRing * kSlotBytes + kBars * 8 + 16 + 1024;
 
 struct UpdParams {
   int32_t rows, cols;          // shape of W
-  int32_t tilesM, tilesN;      // pair tiles: 256 rows x 256 columns
+  int32_t tilesM, tilesN;      // pair tiles: 256 rows x bn columns
+  int32_t bn;                  // 256 or 128
   int32_t nseg, kseg;          // contraction: nseg segments of kseg k-blocks (3 segments: split-bf16 product)
   // Segment s reads U^T from column a_off<s> and V^T from column b_off<s>.  Scalars, not arrays: indexing an
   // array of a kernel parameter with a run-time index moves the whole parameter block to local memory.
@@ -63,6 +63,8 @@ struct UpdParams {
   float* shadow32;             // (big | small) tf32 copy of the updated W: big at column c, small at shadow_half + c
   int64_t shadow_ld;
   int64_t shadow_half;
+  Stamp begin;
+  unsigned long long* end;
   uint32_t* status;
   unsigned long long* copy_counters;   // [0] row pieces of the bf16 copy visited, [1] of them rewritten (or null)
 };
@@ -90,7 +92,7 @@ __device__ __forceinline__ void tile_origin(const UpdParams& p, int tile, int& m
   const int gsz = min(kGroup, p.tilesM - grp * kGroup);       // the last group may be smaller
   const int tm = grp * kGroup + within % gsz, tn = within / gsz;
   m0 = tm * (2 * UM);
-  n0 = tn * UN;
+  n0 = tn * p.bn;
 }
 
 // TF32: the operands are 32-bit words read as tf32 (32 elements per 128-byte k-block), see the forward kernel.
@@ -121,6 +123,8 @@ update_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
   const int my_tiles = pair < ntiles ? (ntiles - 1 - pair) / npairs + 1 : 0;
   const int numK = p.nseg * p.kseg;
   constexpr bool MN = !TF32;                   // the operands are MN-major
+  const int half = p.bn / 2;                   // columns per CTA of the V^T slice, and per epilogue warp
+  pdl_launch_dependents();
 
   if (threadIdx.x == 0) {
     for (int i = 0; i < kStages; ++i) { mbar_init(&full[i], 1); mbar_init(&empty[i], 1); }
@@ -137,6 +141,8 @@ update_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
   cluster_wait();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  pdl_wait();
+  stamp_begin(p.begin);
 
   if (warp == 0) {
     // ---------------- TMA producer (each CTA loads its own rows of U^T and its own half of the V^T rows) ---------
@@ -151,16 +157,18 @@ update_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
           for (int kl = 0; kl < p.kseg; ++kl, ++it) {
             const uint32_t s = it % kStages, ph = (it / kStages) & 1;
             if (!mbar_wait(&empty[s], ph ^ 1, abort_flag)) { ok = false; break; }
-            if (rank == 0) mbar_expect_tx(&full[s], 2 * kStageBytes);
+            if (rank == 0) mbar_expect_tx(&full[s], 2 * (kBytesA + half * UK * 2));
             const uint32_t full_leader = mapa_u32(smem_u32(&full[s]), 0);
             const int xa = seg == 0 ? p.a_off0 : seg == 1 ? p.a_off1 : p.a_off2;
             const int xb = seg == 0 ? p.b_off0 : seg == 1 ? p.b_off1 : p.b_off2;
-            const int ma = m0 + static_cast<int>(rank) * UM, nb = n0 + static_cast<int>(rank) * (UN / 2);
-            if (MN) {                          // two boxes of 64 rows (columns) of W x 64 pairs per operand
+            const int ma = m0 + static_cast<int>(rank) * UM, nb = n0 + static_cast<int>(rank) * half;
+            if (MN) {                          // boxes of 64 rows (columns) of W x 64 pairs
 #pragma unroll
               for (int h = 0; h < 2; ++h) {
                 tma_load_2d_pair(sA + s * kBytesA + h * (kBytesA / 2), &tmA, xa + ma + 64 * h, kl * UK, full_leader, pol_norm);
-                tma_load_2d_pair(sB + s * kBytesB + h * (kBytesB / 2), &tmB, xb + nb + 64 * h, kl * UK, full_leader, pol_keep);
+                if (64 * h < half)
+                  tma_load_2d_pair(sB + s * kBytesB + h * (kBytesB / 2), &tmB, xb + nb + 64 * h, kl * UK, full_leader,
+                  pol_keep);
               }
             } else {
               tma_load_2d_pair(sA + s * kBytesA, &tmA, xa + kl * (UK / 2), ma, full_leader, pol_norm);
@@ -173,7 +181,7 @@ update_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
   } else if (warp == 1) {
     // ---------------- MMA issuer: one thread of the leader CTA drives both SMs ----------------
     if (lane == 0 && rank == 0) {
-      const uint32_t idesc = TF32 ? umma_idesc_tf32(2 * UM, UN) : umma_idesc_bf16(2 * UM, UN) | kIdescMnMajor;
+      const uint32_t idesc = TF32 ? umma_idesc_tf32(2 * UM, p.bn) : umma_idesc_bf16(2 * UM, p.bn) | kIdescMnMajor;
       uint32_t it = 0;
       bool ok = true;
       for (int tl = 0; tl < my_tiles && ok; ++tl) {
@@ -203,7 +211,8 @@ update_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
     const int e = warp - 2, q = warp & 3, h = e >> 2;
     uint8_t* ring = sRing + e * kRing * kSlotBytes;
     uint64_t* rf = rfull + e * kRing;
-    const uint32_t nchunks = static_cast<uint32_t>(my_tiles) * kChunksPerWarp;
+    const int cshift = p.bn == 256 ? 2 : 1, cpw = 1 << cshift;       // chunks per warp and tile: 4 or 2
+    const uint32_t nchunks = static_cast<uint32_t>(my_tiles * cpw);
     // Default L2 priority for the tiles of W: with evict_first on this traffic the written lines are pushed to
     // HBM at once, in small pieces between the reads, and the measured rate drops by a quarter.
     const uint64_t pol_w = policy_evict_normal();
@@ -215,10 +224,10 @@ update_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
     auto issue_load = [&]() {
       if (lg >= nchunks) return;
       int m0, n0;
-      tile_origin(p, pair + static_cast<int>(lg / kChunksPerWarp) * npairs, m0, n0);
+      tile_origin(p, pair + static_cast<int>(lg >> cshift) * npairs, m0, n0);
       const uint32_t slot = lg % kRing;
       mbar_expect_tx(&rf[slot], kSlotBytes);
-      tma_load_2d_hint(ring + slot * kSlotBytes, &tmC, n0 + h * (UN / 2) + static_cast<int>(lg % kChunksPerWarp) * kChunk,
+      tma_load_2d_hint(ring + slot * kSlotBytes, &tmC, n0 + h * half + static_cast<int>(lg & (cpw - 1)) * kChunk,
                        m0 + row_in_tile, &rf[slot], pol_w);
       ++lg;
     };
@@ -229,25 +238,25 @@ update_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
       int m0, n0;
       tile_origin(p, pair + tl * npairs, m0, n0);
       const uint32_t a = tl & 1, aph = (tl >> 1) & 1;
+      const int y0 = m0 + row_in_tile;
       if (!__all_sync(0xffffffffu, mbar_wait(&tfull[a], aph, abort_flag))) { ok = false; break; }
       tc_fence_after();
-      const int y0 = m0 + row_in_tile;
-      const uint32_t t_addr = tmem_base + (static_cast<uint32_t>(q * 32) << 16) + a * UN + h * (UN / 2);
+      const uint32_t t_addr = tmem_base + (static_cast<uint32_t>(q * 32) << 16) + a * UN + h * half;
       uint32_t acc0[32], acc1[32];
       tmem_ld_32x32(t_addr, acc0);
       auto process = [&](uint32_t (&acc)[32], uint32_t (&nxt)[32], int c) -> bool {
         tmem_ld_wait();                                      // chunk c's accumulators are in registers
-        if (c + 1 < kChunksPerWarp) {
+        if (c + 1 < cpw) {
           tmem_ld_32x32(t_addr + (c + 1) * kChunk, nxt);     // chunk c+1 streams in during this chunk's work
         } else {
           tc_fence_before();                                 // last TMEM read of the tile by this warp: hand the
           __syncwarp();                                      // accumulator stage back to the leader's MMA warp
           if (lane == 0) mbar_arrive_cluster(a ? tempty_leader1 : tempty_leader0);
         }
-        const uint32_t slot = g % kRing;
-        uint8_t* sl = ring + slot * kSlotBytes;
-        if (!__all_sync(0xffffffffu, mbar_wait(&rf[slot], (g / kRing) & 1, abort_flag))) return false;
-        const int x0 = n0 + h * (UN / 2) + c * kChunk;
+        const uint32_t rs = g % kRing;
+        uint8_t* sl = ring + rs * kSlotBytes;
+        const int x0 = n0 + h * half + c * kChunk;
+        if (!__all_sync(0xffffffffu, mbar_wait(&rf[rs], (g / kRing) & 1, abort_flag))) return false;
         uint32_t differs = 0;      // SHADOW == 1: does the bf16 rounding of any of this row's 32 values change?
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
@@ -266,7 +275,7 @@ update_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
           *wp = w;
           if (SHADOW == 1) differs |= (o01 ^ pack2(w.x, w.y)) | (o23 ^ pack2(w.z, w.w));
         }
-        // The bf16 copy holds bf16(W) when the pass starts (set-up, refresh, label rows and this kernel keep it so): a
+        // The bf16 copy holds bf16(W) when the pass starts (set-up, refresh and this kernel keep it so): a
         // row piece whose 32 roundings all stay the same already holds bf16 of the new values and is not rewritten.
         // With updates of a few fp32 spacings per entry that is most of the matrix; the copy stays exact either way.
         const uint32_t rowmask = SHADOW == 1 ? __ballot_sync(0xffffffffu, differs != 0) : 0u;
@@ -332,7 +341,7 @@ update_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
         return true;
       };
 #pragma unroll 1
-      for (int c = 0; c < kChunksPerWarp && ok; c += 2) {
+      for (int c = 0; c < cpw && ok; c += 2) {
         ok = process(acc0, acc1, c);
         if (ok) ok = process(acc1, acc0, c + 1);
       }
@@ -356,77 +365,18 @@ update_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
   }
   cluster_arrive();          // neither CTA frees its TMEM or exits while the other may still signal or write it
   cluster_wait();
+  stamp_end(p.end);
   if (warp == 1) { tc_fence_after(); tmem_dealloc_pair(tmem_base, kTmemCols); }
 }
 
-// The label entries of the K factors, u_iy = p_iy - 1, which the bf16 operand leaves out (it holds 0 there):
-//   W[y] <- W[y] + eta * sum_{i : y_i = y} (1 - p_iy) x_i     in fp32, from the fp32 copy of the samples.
-// One block per (sample, 1024 columns); the blocks of the first sample of each class list that class's samples
-// (ascending, so the sum has the same order every run; no atomics), sum them and refresh the bf16 copy of the row.
-constexpr int kLabelList = 1024;
-__global__ void __launch_bounds__(256) label_rows_kernel(float* __restrict__ W, int64_t rows, int64_t cols,
-                                                         const float* __restrict__ Xf, const int32_t* __restrict__ labels,
-                                                         const float* __restrict__ coef, int K, float eta, __nv_bfloat16* __restrict__ shadow,
-                                                         int64_t shadow_ld) {
-  __shared__ int first;
-  __shared__ int count;
-  __shared__ int list[kLabelList];
-  __shared__ int warp_tot[8];
-  const int i = blockIdx.x;
-  const int32_t y = labels[i];
-  if (y < 0 || y >= rows) return;              // out-of-range ids were flagged by the softmax pass
-  if (threadIdx.x == 0) first = 1;
-  __syncthreads();
-  for (int j = threadIdx.x; j < i; j += 256)
-    if (labels[j] == y) first = 0;
-  __syncthreads();
-  if (!first) return;
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  const int64_t c = static_cast<int64_t>(threadIdx.x) * 4 + static_cast<int64_t>(blockIdx.y) * 1024;
-  float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-  for (int base = i; base < K; base += kLabelList) {
-    // ordered compaction of the matching sample indices in [base, base + kLabelList)
-    if (threadIdx.x == 0) count = 0;
-    __syncthreads();
-    for (int off = 0; off < kLabelList; off += 256) {
-      const int j = base + off + threadIdx.x;
-      const bool hit = j < K && labels[j] == y;
-      const unsigned m = __ballot_sync(0xffffffffu, hit);
-      if (lane == 0) warp_tot[wid] = __popc(m);
-      __syncthreads();
-      int pre = count;
-      for (int w = 0; w < wid; ++w) pre += warp_tot[w];
-      if (hit) list[pre + __popc(m & ((1u << lane) - 1))] = j;
-      __syncthreads();
-      if (threadIdx.x == 0) {
-        int t = 0;
-        for (int w = 0; w < 8; ++w) t += warp_tot[w];
-        count += t;
-      }
-      __syncthreads();
-    }
-    if (c < cols) {
-      const int n = count;
-      for (int k = 0; k < n; ++k) {
-        const int j = list[k];
-        const float4 x = *reinterpret_cast<const float4*>(Xf + static_cast<int64_t>(j) * cols + c);
-        const float cf = coef[j];
-        acc.x = fmaf(cf, x.x, acc.x); acc.y = fmaf(cf, x.y, acc.y);
-        acc.z = fmaf(cf, x.z, acc.z); acc.w = fmaf(cf, x.w, acc.w);
-      }
-    }
-    __syncthreads();
-  }
-  if (c < cols) {
-    float4* wp = reinterpret_cast<float4*>(W + static_cast<int64_t>(y) * cols + c);
-    float4 w = *wp;
-    w.x = fmaf(eta, acc.x, w.x); w.y = fmaf(eta, acc.y, w.y);
-    w.z = fmaf(eta, acc.z, w.z); w.w = fmaf(eta, acc.w, w.w);
-    *wp = w;
-    if (shadow)
-      *reinterpret_cast<uint2*>(shadow + static_cast<int64_t>(y) * shadow_ld + c) =
-          make_uint2(pack2(w.x, w.y), pack2(w.z, w.w));
-  }
+// Tile width: 128 where 256-wide tiles leave the pairs short of work.  Cycles of a tile: its k-blocks at the MMA or operand
+// rate (measured about 620 a k-block for 256 columns, 450 for 128) and its epilogue.
+int tile_width(int64_t rows, int64_t cols, int64_t kblocks, int pairs) {
+  auto cost = [&](int bn) {
+    const int64_t tiles = ((rows + 2 * UM - 1) / (2 * UM)) * ((cols + bn - 1) / bn);
+    return static_cast<double>((tiles + pairs - 1) / pairs) * (kblocks * (bn == 256 ? 620. : 450.) + (bn == 256 ? 2500. : 1800.));
+  };
+  return cost(128) < 0.97 * cost(256) ? 128 : 256;
 }
 
 }  // namespace
@@ -476,7 +426,7 @@ int tc_update_init(sfb_ctx* ctx, TcState* st) {
 int tc32_update(sfb_ctx* ctx) {
   if (ctx->sparse_v) return sparse_update(ctx);         // writes the (big | small) copy as well
   const sfb_config& c = ctx->cfg;
-  const TcState* st = static_cast<const TcState*>(ctx->tc);
+  TcState* st = static_cast<TcState*>(ctx->tc);
   const Layout& L = ctx->lay;
   const int64_t Kp = L.Kp;                                  // a multiple of 32
   CUtensorMap ma, mb, mc;
@@ -487,8 +437,10 @@ int tc32_update(sfb_ctx* ctx) {
   UpdParams p{};
   p.rows = static_cast<int32_t>(c.rows); p.cols = static_cast<int32_t>(c.cols);
   p.tilesM = static_cast<int32_t>((c.rows + 2 * UM - 1) / (2 * UM));
+  p.bn = UN;
   p.tilesN = static_cast<int32_t>((c.cols + UN - 1) / UN);
   p.kseg = static_cast<int32_t>(Kp / (UK / 2));
+  p.begin = take_stamp(ctx); p.end = &ctx->at<Scalars>(L.scalars)->ns[3];
   p.alpha = -ctx->step;
   p.prox_kind = ctx->prox_kind; p.prox_a = ctx->prox_a;
   p.status = ctx->at<uint32_t>(L.status);
@@ -502,15 +454,18 @@ int tc32_update(sfb_ctx* ctx) {
   p.shadow = nullptr; p.shadow32 = ctx->at<float>(L.Ws); p.shadow_ld = 2 * L.colsp; p.shadow_half = L.colsp;
   const int64_t tiles = static_cast<int64_t>(p.tilesM) * p.tilesN;
   const unsigned grid = 2u * static_cast<unsigned>(std::min<int64_t>(tiles, st->max_pairs));
-  update_pair_kernel<2, true><<<grid, kThreads, kSmem, ctx->stream>>>(ma, mb, mc, p);
-  count_launch();
-  CKC(cudaGetLastError());
+  CKC(launch_kernel_if(tiles <= st->max_pairs, (update_pair_kernel<2, true>), dim3(grid), dim3(kThreads), kSmem, ctx->stream, 1, ma, mb, mc, p));
   return SFB_OK;
 }
 
 int tc_update(sfb_ctx* ctx) {
+  if (ctx->cfg.model == SFB_MLR) {
+    const int rc = tc_labels(ctx);                     // the fp32 label entries, unless the factors call has applied them
+    if (rc) return rc;
+  }
+  if (ctx->sparse_v) return sparse_update(ctx);
   const sfb_config& c = ctx->cfg;
-  const TcState* st = static_cast<const TcState*>(ctx->tc);
+  TcState* st = static_cast<TcState*>(ctx->tc);
   const Layout& L = ctx->lay;
   const bool split = c.model != SFB_MLR;
   // U and V pair-major; the split products have (hi | lo) halves side by side
@@ -526,8 +481,10 @@ int tc_update(sfb_ctx* ctx) {
   UpdParams p{};
   p.rows = static_cast<int32_t>(c.rows); p.cols = static_cast<int32_t>(c.cols);
   p.tilesM = static_cast<int32_t>((c.rows + 2 * UM - 1) / (2 * UM));
-  p.tilesN = static_cast<int32_t>((c.cols + UN - 1) / UN);
   p.kseg = static_cast<int32_t>((ctx->K + UK - 1) / UK);
+  p.bn = tile_width(c.rows, c.cols, (split ? 3 : 1) * p.kseg, st->max_pairs);
+  p.tilesN = static_cast<int32_t>((c.cols + p.bn - 1) / p.bn);
+  p.begin = take_stamp(ctx); p.end = &ctx->at<Scalars>(L.scalars)->ns[3];
   p.alpha = -ctx->step;
   p.prox_kind = ctx->prox_kind; p.prox_a = ctx->prox_a;
   p.status = ctx->at<uint32_t>(L.status);
@@ -539,35 +496,13 @@ int tc_update(sfb_ctx* ctx) {
     p.a_off0 = 0; p.a_off1 = 0; p.a_off2 = static_cast<int32_t>(L.rowsp);
     p.b_off0 = 0; p.b_off1 = static_cast<int32_t>(L.colsp); p.b_off2 = 0;
     p.shadow = nullptr; p.shadow_ld = 0;
-    update_pair_kernel<0><<<grid, kThreads, kSmem, ctx->stream>>>(ma, mb, mc, p);
-    count_launch();
-    CKC(cudaGetLastError());
+    CKC(launch_kernel_if(tiles <= st->max_pairs, update_pair_kernel<0>, dim3(grid), dim3(kThreads), kSmem, ctx->stream, 1, ma, mb, mc, p));
     return SFB_OK;
   }
   p.nseg = 1;
   p.shadow = ctx->at<__nv_bfloat16>(L.Wb); p.shadow_ld = L.colsb;
   p.copy_counters = &ctx->at<Scalars>(L.scalars)->copy_pieces;
-  if ((c.cols + 1023) / 1024 > 65535) return SFB_ERR_SHAPE;
-  dim3 lgrid(static_cast<unsigned>(ctx->K), static_cast<unsigned>((c.cols + 1023) / 1024));
-  // With a fused prox the fp32 label-row term has to be in W before the pass that applies the operator, so it goes
-  // first (both terms are sums into W).  Either way the label-row kernel rewrites the bf16 copy of its rows, so the
-  // copy equals bf16(W) whenever the main pass starts.
-  const bool labels_first = ctx->prox_kind != 0;
-  for (int pass = 0; pass < 2; ++pass) {
-    if ((pass == 0) == labels_first) {
-      label_rows_kernel<<<lgrid, 256, 0, ctx->stream>>>(
-          ctx->W, c.rows, c.cols, ctx->at<float>(L.Xf), ctx->at<int32_t>(L.labels), ctx->at<float>(L.coef),
-          static_cast<int>(ctx->K), ctx->step, ctx->at<__nv_bfloat16>(L.Wb), L.colsb);   // keeps the copy = bf16(W)
-    } else if (ctx->sparse_v) {
-      const int rc = sparse_update(ctx);                                                // the same sum over the non-zeros of V
-      if (rc) return rc;
-      continue;
-    } else {
-      update_pair_kernel<1><<<grid, kThreads, kSmem, ctx->stream>>>(ma, mb, mc, p);     // W += -eta * P^T V
-    }
-    count_launch();
-    CKC(cudaGetLastError());
-  }
+  CKC(launch_kernel_if(tiles <= st->max_pairs, update_pair_kernel<1>, dim3(grid), dim3(kThreads), kSmem, ctx->stream, 1, ma, mb, mc, p));
   return SFB_OK;
 }
 
