@@ -653,6 +653,17 @@ extern "C" int sfb_sdca_set_dual(sfb_ctx* ctx, float* Q_dev, int64_t n_samples) 
   return SFB_OK;
 }
 
+namespace sfb {
+SdcaArgs sdca_args(const sfb_ctx* ctx, int64_t off, int64_t n, const float* X, const int32_t* labels, const int32_t* ids,
+                   float inv_lam_n) {
+  SdcaArgs a{};
+  a.n = n; a.rows = ctx->cfg.rows; a.X = X; a.cols = ctx->cfg.cols; a.labels = labels; a.ids = ids;
+  a.Q = ctx->dualQ; a.n_samples = ctx->dual_n; a.inv_lam_n = inv_lam_n; a.gamma = ctx->cfg.eta;
+  a.loss = ctx->at<float>(ctx->lay.loss) + off; a.status = ctx->at<uint32_t>(ctx->lay.status); a.off = off;
+  return a;
+}
+}  // namespace sfb
+
 static int sdca_compute_factors(sfb_ctx* ctx, int32_t worker, const float* X_dev, const int32_t* labels_dev,
                                 const int32_t* sample_ids_dev, bool fused) {
   if (!ctx || !X_dev || !labels_dev || !sample_ids_dev) return SFB_ERR_ARG;
@@ -665,8 +676,6 @@ static int sdca_compute_factors(sfb_ctx* ctx, int32_t worker, const float* X_dev
   const int64_t n = worker < 0 ? ctx->K : c.batch;
   if (ctx->committed == 0) begin_phase(ctx, 0);
   const float inv_lam_n = static_cast<float>(1.0 / (static_cast<double>(c.sdca_lambda) * static_cast<double>(c.sdca_n)));
-  uint32_t* status = ctx->at<uint32_t>(ctx->lay.status);
-  float* loss = ctx->at<float>(ctx->lay.loss) + off;
   if (ctx->tf32) {
     const int rc = tc32_factors(ctx, off, n, X_dev, labels_dev, sample_ids_dev, inv_lam_n);
     if (rc) return rc;
@@ -679,8 +688,9 @@ static int sdca_compute_factors(sfb_ctx* ctx, int32_t worker, const float* X_dev
     e.C = U; e.ldc = ldu;
     CK(sgemm(ctx->stream, true, true, EPI_STORE, n, c.rows, c.cols, V, c.cols, ctx->W, c.cols, e, ctx->K));   // z_i = W a_i
     ctx->stats.flops += 2.0 * n * c.rows * c.cols;
-    CK(sdca_dual_rows(ctx->stream, U, n, c.rows, ldu, X_dev, c.cols, labels_dev, sample_ids_dev, ctx->dualQ, ctx->dual_n,
-                      inv_lam_n, c.eta, nullptr, loss, status));                                      // u_i = du_i
+    SdcaArgs a = sdca_args(ctx, off, n, X_dev, labels_dev, sample_ids_dev, inv_lam_n);
+    a.Z = U; a.ldz = ldu; a.out = U; a.ldo = ldu;                                                     // u_i = du_i
+    CK(sdca_dual_rows(ctx->stream, a));
   } else {
     const int rc = tc_sdca_factors(ctx, off, n, X_dev, labels_dev, sample_ids_dev, inv_lam_n, fused);
     if (rc) return rc;

@@ -208,99 +208,158 @@ __global__ void __launch_bounds__(NTHREADS) mlr_shard_finish_kernel(float* __res
 // the new dual row q minimises  sum_j q_j log q_j - q.(z + kappa q_old) + kappa/2 ||q||^2  over the simplex, kappa =
 // ||x||^2 / (lam N).  Stationarity: log q_j + kappa q_j = t_j - nu with t = z + kappa q_old, and nu such that the q_j sum
 // to 1; nu lies in [lse(t) - kappa, lse(t)].
-// q_j(nu): Newton on y = log q for  y + kappa e^y = c  (increasing and convex in y, so the iteration is monotone from
-// the right of the root, where it starts).
+// q_j(nu) with c = t_j - nu: kappa q = W(kappa e^c), W the Lambert function.  Nearly every class has kappa e^c << 1, where four
+// terms of its series at 0 (Corless et al., "On the Lambert W function", 1996) are exact to 5 e^4 < 1e-11; else Newton on
+// y = log q for  y + kappa e^y = c  (increasing and convex in y, so monotone from the right of the root, where it starts).
 __device__ __forceinline__ float sdca_coordinate(float c, float kappa) {
-  if (kappa <= 0.f) return expf(c);
+  const float ec = expf(c), e = kappa * ec;
+  if (e < 1e-3f) return ec * fmaf(e, fmaf(e, fmaf(e, -8.f / 3.f, 1.5f), -1.f), 1.f);
   float y = c;                                       // y + kappa e^y - c = kappa e^c >= 0 here: right of the root
   if (c > 0.f) y = fminf(c, logf((c + 1.f) / kappa));
 #pragma unroll 1
   for (int it = 0; it < 24; ++it) {
-    const float e = kappa * expf(y);
-    const float d = (y + e - c) / (1.f + e);
+    const float f = kappa * expf(y);
+    const float d = (y + f - c) / (1.f + f);
     y -= d;
     if (fabsf(d) <= 1e-7f * fmaxf(1.f, fabsf(y))) break;
   }
   return expf(y);
 }
 
+// Sums of three values over the block in a fixed order, in every thread.
 template <int NTHREADS>
-__global__ void __launch_bounds__(NTHREADS) sdca_dual_kernel(float* __restrict__ Z, int64_t rows, int64_t ldz,
-                                                             const float* __restrict__ X, int64_t cols,
-                                                             const int32_t* __restrict__ labels,
-                                                             const int32_t* __restrict__ ids, float* __restrict__ Q,
-                                                             int64_t n_samples, float inv_lam_n, float gamma,
-                                                             float* __restrict__ coef, float* __restrict__ loss,
-                                                             uint32_t* status, int32_t* __restrict__ slot, int64_t off) {
+__device__ __forceinline__ float3 block_sum3(float a, float b, float c, float3* sh) {
+  a = warp_sum(a); b = warp_sum(b); c = warp_sum(c);
+  __syncthreads();
+  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = make_float3(a, b, c);
+  __syncthreads();
+  float3 r = make_float3(0.f, 0.f, 0.f);
+#pragma unroll
+  for (int w = 0; w < NTHREADS / 32; ++w) { r.x += sh[w].x; r.y += sh[w].y; r.z += sh[w].z; }
+  return r;
+}
+
+struct SdcaParams {
+  const float* Z;              // logits [n x ldz]
+  int64_t rows, ldz;
+  const float* X;
+  int64_t cols;
+  const int32_t* labels;
+  const int32_t* ids;
+  float* Q;
+  int64_t n_samples;
+  float inv_lam_n, gamma;
+  float* out;                  // du in fp32 [n x ldo] (may be Z itself), or null with
+  int64_t ldo;
+  __nv_bfloat16* P;            //   du in bf16 [n x ldp], 0 at the label entry, whose value goes to coef
+  int64_t ldp;
+  float* coef;
+  float* loss;
+  uint32_t* status;
+  int32_t* slot;               // may be null
+  int64_t off;                 // first sample's index (slot)
+};
+
+// What bounds it: the exponentials, one per class and pass over a sample's classes.  The passes: t and its maximum; the sums
+// behind lse(t), lse(z) and the first step of nu; two or three of the outer Newton; the write-out.  t - lse stays in shared
+// memory (KEEP; up to 50,000 classes), and nu is carried as its distance from lse(t): as a number near lse(t) its own spacing
+// (1e-6) is above the tolerance of the sum, and the iteration ran to its limit of twelve passes.
+// 512 samples x 10,000 classes: 76 us; 420 us with a Newton solve per class and pass and those twelve passes.
+template <int NTHREADS, bool KEEP>
+__global__ void __launch_bounds__(NTHREADS) sdca_dual_kernel(const __grid_constant__ SdcaParams p) {
   pdl_launch_dependents();
   pdl_wait();
+  extern __shared__ float base[];                    // KEEP: t_j, then t_j - lse(t)
   __shared__ float sh[32];
+  __shared__ float3 sh3[NTHREADS / 32];
+  const int t = threadIdx.x, rows = static_cast<int>(p.rows);
   const int64_t i = blockIdx.x;
-  float* z = Z + i * ldz;
-  const int64_t id = ids[i];
-  const int32_t y = labels[i];
-  const bool ok = id >= 0 && id < n_samples && y >= 0 && y < rows;
+  const float* z = p.Z + i * p.ldz;
+  float* out = p.out ? p.out + i * p.ldo : nullptr;
+  __nv_bfloat16* P = p.P ? p.P + i * p.ldp : nullptr;
+  const int64_t id = p.ids[i];
+  const int32_t y = p.labels[i];
+  const bool ok = id >= 0 && id < p.n_samples && y >= 0 && y < rows;
   if (!ok) {                                         // uniform over the block: skip the sample, contribute nothing
-    if (threadIdx.x == 0) {
-      atomicOr(status, (id >= 0 && id < n_samples) ? SFB_STATUS_LABEL_RANGE : SFB_STATUS_SAMPLE_RANGE);
-      if (coef) coef[i] = 0.f;
-      loss[i] = 0.f;
+    if (t == 0) {
+      atomicOr(p.status, (id >= 0 && id < p.n_samples) ? SFB_STATUS_LABEL_RANGE : SFB_STATUS_SAMPLE_RANGE);
+      if (p.coef) p.coef[i] = 0.f;
+      p.loss[i] = 0.f;
     }
-    for (int64_t j = threadIdx.x; j < rows; j += NTHREADS) z[j] = 0.f;
+    for (int j = t; j < rows; j += NTHREADS) {
+      if (out) out[j] = 0.f;
+      if (P) P[j] = __float2bfloat16_rn(0.f);
+    }
     return;
   }
-  float* q = Q + id * rows;
-  const float* x = X + i * cols;
+  float* q = p.Q + id * p.rows;
+  const float4* x = reinterpret_cast<const float4*>(p.X + i * p.cols);
   float ss = 0.f;
-  for (int64_t d = threadIdx.x; d < cols; d += NTHREADS) ss = fmaf(x[d], x[d], ss);
-  const float kappa = block_sum<NTHREADS>(ss, sh) * inv_lam_n;
-  // lse(t) and, for the read-out, lse(z)
+  for (int d = t; d < p.cols / 4; d += NTHREADS) {
+    const float4 v = x[d];
+    ss = fmaf(v.x, v.x, ss); ss = fmaf(v.y, v.y, ss); ss = fmaf(v.z, v.z, ss); ss = fmaf(v.w, v.w, ss);
+  }
+  const float kappa = block_sum<NTHREADS>(ss, sh) * p.inv_lam_n;
   float m = -INFINITY, mz = -INFINITY;
-  for (int64_t j = threadIdx.x; j < rows; j += NTHREADS) {
-    m = fmaxf(m, fmaf(kappa, q[j], z[j]));
-    mz = fmaxf(mz, z[j]);
+#pragma unroll 4
+  for (int j = t; j < rows; j += NTHREADS) {
+    const float zj = z[j], tj = fmaf(kappa, q[j], zj);
+    if (KEEP) base[j] = tj;
+    m = fmaxf(m, tj);
+    mz = fmaxf(mz, zj);
   }
   m = block_max<NTHREADS>(m, sh);
   mz = block_max<NTHREADS>(mz, sh);
-  float s = 0.f, sz = 0.f;
-  for (int64_t j = threadIdx.x; j < rows; j += NTHREADS) {
-    s += expf(fmaf(kappa, q[j], z[j]) - m);
-    sz += expf(z[j] - mz);
+  float s1 = 0.f, s2 = 0.f, sz = 0.f;
+#pragma unroll 4
+  for (int j = t; j < rows; j += NTHREADS) {
+    const float zj = z[j], e = expf((KEEP ? base[j] : fmaf(kappa, q[j], zj)) - m);
+    s1 += e;
+    s2 = fmaf(e, e, s2);
+    sz += expf(zj - mz);
   }
-  s = block_sum<NTHREADS>(s, sh);
-  sz = block_sum<NTHREADS>(sz, sh);
-  const float lse = m + logf(s);
-  if (threadIdx.x == 0 && slot) atomicMin(&slot[y], static_cast<int32_t>(off + i));
-  if (threadIdx.x == 0) loss[i] = (mz + logf(sz)) - z[y];        // the sample's logistic loss at the W of this step
-  // safeguarded Newton on nu: G(nu) = sum_j q_j(nu) is decreasing and convex, G(lse - kappa) >= 1 >= G(lse)
-  float lo = lse - kappa, hi = lse, nu = lse;
+  const float3 r = block_sum3<NTHREADS>(s1, s2, sz, sh3);
+  const float lse = m + logf(r.x);
+  if (t == 0) {
+    p.loss[i] = (mz + logf(r.z)) - z[y];             // the sample's logistic loss at the W of this step
+    if (p.slot) atomicMin(&p.slot[y], static_cast<int32_t>(p.off + i));
+  }
+  if (KEEP)
+    for (int j = t; j < rows; j += NTHREADS) base[j] -= lse;
+  auto dist = [&](int j) { return KEEP ? base[j] : fmaf(kappa, q[j], z[j]) - lse; };
+  // safeguarded Newton on d = nu - lse(t): G(d) = sum_j q_j is decreasing and convex, G(-kappa) >= 1 >= G(0); to first order
+  // in kappa G(d) = 1 - kappa sum p^2 - d with p = softmax(t)
+  float lo = -kappa, hi = 0.f, d = -kappa * r.y / (r.x * r.x), S = 1.f;
 #pragma unroll 1
   for (int it = 0; it < 12; ++it) {
     float G = 0.f, Dv = 0.f;
-    for (int64_t j = threadIdx.x; j < rows; j += NTHREADS) {
-      const float qj = sdca_coordinate(fmaf(kappa, q[j], z[j]) - nu, kappa);
+#pragma unroll 4
+    for (int j = t; j < rows; j += NTHREADS) {
+      const float qj = sdca_coordinate(dist(j) - d, kappa);
       G += qj;
-      Dv += qj / fmaf(kappa, qj, 1.f);
+      Dv += __fdividef(qj, fmaf(kappa, qj, 1.f));    // (only steers the iteration)
     }
-    G = block_sum<NTHREADS>(G, sh);
-    Dv = block_sum<NTHREADS>(Dv, sh);
-    const float g = G - 1.f;
-    if (fabsf(g) <= 2e-7f) break;                    // uniform over the block: every thread holds the same sums
-    if (g > 0.f) lo = fmaxf(lo, nu); else hi = fminf(hi, nu);
-    float next = nu + g / Dv;
+    const float3 v = block_sum3<NTHREADS>(G, Dv, 0.f, sh3);
+    S = v.x;
+    const float g = S - 1.f;
+    // the write-out divides by S: what is left of an error g in the sum is g kappa q_j / (1 + kappa q_j) of an entry
+    if (fabsf(g) <= 2e-7f || (fabsf(g) <= 1e-4f && fabsf(g) * kappa <= 5e-8f)) break;   // uniform over the block
+    if (it == 11) break;
+    if (g > 0.f) lo = fmaxf(lo, d); else hi = fminf(hi, d);
+    float next = d + g / v.y;
     if (!(next > lo && next < hi)) next = 0.5f * (lo + hi);
-    nu = next;
+    if (next == d) break;
+    d = next;
   }
-  float S = 0.f;
-  for (int64_t j = threadIdx.x; j < rows; j += NTHREADS) S += sdca_coordinate(fmaf(kappa, q[j], z[j]) - nu, kappa);
-  S = block_sum<NTHREADS>(S, sh);
   const float invS = 1.f / S;
-  for (int64_t j = threadIdx.x; j < rows; j += NTHREADS) {
+#pragma unroll 4
+  for (int j = t; j < rows; j += NTHREADS) {
     const float qo = q[j];
-    const float du = sdca_coordinate(fmaf(kappa, qo, z[j]) - nu, kappa) * invS - qo;      // du = q_new - q_old
-    z[j] = du;
-    q[j] = fmaf(gamma, du, qo);
-    if (coef && j == y) coef[i] = -du;
+    const float du = fmaf(sdca_coordinate(dist(j) - d, kappa), invS, -qo);      // du = q_new - q_old
+    if (out) out[j] = du;
+    if (P) P[j] = __float2bfloat16_rn(j == y ? 0.f : du);
+    q[j] = fmaf(p.gamma, du, qo);
+    if (p.coef && j == y) p.coef[i] = -du;
   }
 }
 
@@ -677,12 +736,19 @@ cudaError_t mlr_shard_finish(cudaStream_t s, float* Z, int64_t nsamp, int64_t ro
                        ldz, labels, row_off, reinterpret_cast<const float4*>(parts), shards, nsamp, loss, status);
 }
 
-cudaError_t sdca_dual_rows(cudaStream_t s, float* Z, int64_t nsamp, int64_t rows, int64_t ldz, const float* X, int64_t cols,
-                           const int32_t* labels, const int32_t* ids, float* Q, int64_t n_samples, float inv_lam_n,
-                           float gamma, float* coef, float* loss, uint32_t* status, int32_t* slot, int64_t off) {
-  if (nsamp <= 0) return cudaSuccess;
-  return launch_kernel(sdca_dual_kernel<512>, dim3(static_cast<unsigned>(nsamp)), dim3(512), 0, s, 1, Z, rows, ldz, X,
-                       cols, labels, ids, Q, n_samples, inv_lam_n, gamma, coef, loss, status, slot, off);
+cudaError_t sdca_dual_rows(cudaStream_t s, const SdcaArgs& a) {
+  if (a.n <= 0) return cudaSuccess;
+  SdcaParams p{};
+  p.Z = a.Z; p.rows = a.rows; p.ldz = a.ldz; p.X = a.X; p.cols = a.cols; p.labels = a.labels; p.ids = a.ids;
+  p.Q = a.Q; p.n_samples = a.n_samples; p.inv_lam_n = a.inv_lam_n; p.gamma = a.gamma;
+  p.out = a.out; p.ldo = a.ldo; p.P = static_cast<__nv_bfloat16*>(a.P); p.ldp = a.ldp;
+  p.coef = a.coef; p.loss = a.loss; p.status = a.status; p.slot = a.slot; p.off = a.off;
+  constexpr int kKeep = 200 << 10;
+  const dim3 grid(static_cast<unsigned>(a.n)), block(512);
+  if (a.rows * 4 > kKeep) return launch_kernel(sdca_dual_kernel<512, false>, grid, block, 0, s, 1, p);
+  const cudaError_t e = allow_smem<sdca_dual_kernel<512, true>>(kKeep);
+  if (e != cudaSuccess) return e;
+  return launch_kernel(sdca_dual_kernel<512, true>, grid, block, static_cast<size_t>(a.rows) * 4, s, 1, p);
 }
 
 cudaError_t dml_scale_rows(cudaStream_t s, float* Z, int64_t nsamp, int64_t rows, int64_t ld,

@@ -248,12 +248,33 @@ cudaError_t mlr_shard_partials(cudaStream_t s, const float* Z, int64_t nsamp, in
                                const int32_t* labels, int64_t row_off, float* part);
 cudaError_t mlr_shard_finish(cudaStream_t s, float* Z, int64_t nsamp, int64_t rows, int64_t ldz, const int32_t* labels,
                              int64_t row_off, const float* parts, int shards, float* loss, uint32_t* status);
-// SDCA (l2-regularised MLR): per sample, from its logits z (row of Z, overwritten with du), its dual row of Q (advanced
-// by gamma * du) and its features x: the change of the dual vector that minimises the dual objective.  coef (may be
-// null) receives -du at the label entry; slot (may be null) the smallest index, from off on, of a sample of each class.
-cudaError_t sdca_dual_rows(cudaStream_t s, float* Z, int64_t nsamp, int64_t rows, int64_t ldz, const float* X, int64_t cols,
-                           const int32_t* labels, const int32_t* ids, float* Q, int64_t n_samples, float inv_lam_n,
-                           float gamma, float* coef, float* loss, uint32_t* status, int32_t* slot = nullptr, int64_t off = 0);
+// SDCA (l2-regularised MLR): per sample, from its logits z, its dual row of Q (advanced by gamma * du) and its features x:
+// the change du of the dual vector that minimises the dual objective, written in fp32 to out (row pitch ldo; may be Z) or in
+// bf16 to P with a 0 at the label entry and -du there to coef.  slot (may be null): the smallest index, from off on, of a
+// sample of each class.
+struct SdcaArgs {
+  const float* Z;
+  int64_t n, rows, ldz;
+  const float* X;
+  int64_t cols;
+  const int32_t* labels;
+  const int32_t* ids;
+  float* Q;
+  int64_t n_samples;
+  float inv_lam_n, gamma;
+  float* out;
+  int64_t ldo;
+  void* P;
+  int64_t ldp;
+  float* coef;
+  float* loss;
+  uint32_t* status;
+  int32_t* slot;
+  int64_t off;
+};
+cudaError_t sdca_dual_rows(cudaStream_t s, const SdcaArgs& a);
+SdcaArgs sdca_args(const sfb_ctx* ctx, int64_t off, int64_t n, const float* X, const int32_t* labels, const int32_t* ids,
+                   float inv_lam_n);               // all but the logits and where du goes
 // Z2 (may be null): a second partial of z (the other half of the contraction), added to Z first.  Row-sharded form:
 // norm_out (may be null) receives the shard's ||z_i||^2 and z is left unscaled; norms_all (may be null), [shards][nstride],
 // supplies ||z_i||^2 as the sum over the shards instead of this context's own.

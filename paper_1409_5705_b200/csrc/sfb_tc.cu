@@ -981,8 +981,8 @@ __global__ void __launch_bounds__(256) mlr_shard_finish_tc_kernel(const float4* 
 // The factor is u_i = p_i - onehot(y_i); its label entry u_iy = p_iy - 1 is left out of the bf16 operand and applied to W in
 // fp32 (label_delta), because bf16 cannot hold it when p_iy is close to 1 (spacing 2^-8 next to 1) and a rounded p_iy
 // with an exact -1 would not cancel.  Eight values per thread; 6 bytes per value, bound by HBM.
-// PLAIN: the values of Z themselves instead of exp(z - lse) (the dual changes of the SDCA step), with the same zero at the
-// label entry.
+// PLAIN: the values of Z themselves instead of exp(z - lse) (factors received from elsewhere), with the same zero at the label
+// entry.
 // With K label entries to sum (lab.K > 0) the first lab_blocks blocks do that instead, see label_delta.
 template <bool PLAIN>
 __global__ void __launch_bounds__(256) mlr_emit_p_kernel(const float* __restrict__ Z, int64_t ldz, int64_t rows,
@@ -1066,8 +1066,7 @@ __global__ void __launch_bounds__(256) split32_t_kernel(const float* __restrict_
 }
 
 // u_ij = exp(z_ij - lse_i) - [j = y_i], from the logits Z [n x ldz] to the pair-major fp32 factors U [n x rows]
-// (Section 2.1: u = d f / d (W a)).  PLAIN copies Z instead (the dual changes of the SDCA step already are the factors).
-template <bool PLAIN>
+// (Section 2.1: u = d f / d (W a)).
 __global__ void __launch_bounds__(256) mlr_finish_u_kernel(const float* __restrict__ Z, int64_t ldz, int64_t rows,
                                                            const float* __restrict__ lse,
                                                            const int32_t* __restrict__ labels,
@@ -1075,12 +1074,12 @@ __global__ void __launch_bounds__(256) mlr_finish_u_kernel(const float* __restri
   pdl_launch_dependents();
   pdl_wait();
   const int64_t i = blockIdx.y;
-  const float l = PLAIN ? 0.f : lse[i];
-  const int64_t y = PLAIN ? -1 : static_cast<int64_t>(labels[i]);
+  const float l = lse[i];
+  const int64_t y = labels[i];
   const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
   for (int64_t j = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; j < rows; j += stride) {
     const float z = Z[i * ldz + j];
-    U[i * rows + j] = PLAIN ? z : expf(z - l) - (j == y ? 1.f : 0.f);
+    U[i * rows + j] = expf(z - l) - (j == y ? 1.f : 0.f);
   }
 }
 
@@ -1533,7 +1532,7 @@ int tc32_finish_factors(sfb_ctx* ctx, const float* parts, int shards) {
                     ctx->at<int32_t>(L.labels), ctx->at<float>(L.lse), ctx->at<float>(L.loss), ctx->at<float>(L.coef),
                     ctx->at<uint32_t>(L.status)));
   dim3 ugrid(static_cast<unsigned>(std::min<int64_t>((rows + 255) / 256, 64)), static_cast<unsigned>(K));
-  CKC(launch_kernel(mlr_finish_u_kernel<false>, ugrid, dim3(256), 0, ctx->stream, 1, ctx->at<float>(L.ZT), round_up(rows,
+  CKC(launch_kernel(mlr_finish_u_kernel, ugrid, dim3(256), 0, ctx->stream, 1, ctx->at<float>(L.ZT), round_up(rows,
                     32), rows, ctx->at<float>(L.lse), ctx->at<int32_t>(L.labels), ctx->at<float>(L.U)));
   return SFB_OK;
 }
@@ -1557,15 +1556,15 @@ int tc32_factors(sfb_ctx* ctx, int64_t off, int64_t n, const float* X, const int
   }
   dim3 ugrid(static_cast<unsigned>(std::min<int64_t>((rows + 255) / 256, 64)), static_cast<unsigned>(n));
   if (sdca_ids) {
-    CKC(sdca_dual_rows(s, Z + off * ldz, n, rows, ldz, X, cols, labels, sdca_ids, ctx->dualQ, ctx->dual_n, inv_lam_n, c.eta,
-                       nullptr, ctx->at<float>(L.loss) + off, ctx->at<uint32_t>(L.status)));
-    CKC(launch_kernel(mlr_finish_u_kernel<true>, ugrid, dim3(256), 0, s, 1, Z + off * ldz, ldz, rows, nullptr, nullptr, U));
+    SdcaArgs a = sdca_args(ctx, off, n, X, labels, sdca_ids, inv_lam_n);
+    a.Z = Z + off * ldz; a.ldz = ldz; a.out = U; a.ldo = rows;
+    CKC(sdca_dual_rows(s, a));
   } else {
     float* lse = ctx->at<float>(L.lse);
     CKC(launch_kernel(mlr_lse_kernel, dim3(static_cast<unsigned>((n + 7) / 8)), dim3(256), 0, s, 1,
                       ctx->at<float2>(L.part), K, tiles_n, Z, ldz, rows, labels, off, n, lse, ctx->at<float>(L.loss),
                       ctx->at<float>(L.coef), nullptr, ctx->at<uint32_t>(L.status)));
-    CKC(launch_kernel(mlr_finish_u_kernel<false>, ugrid, dim3(256), 0, s, 1, Z + off * ldz, ldz, rows, lse + off, labels,
+    CKC(launch_kernel(mlr_finish_u_kernel, ugrid, dim3(256), 0, s, 1, Z + off * ldz, ldz, rows, lse + off, labels,
                       U));
   }
   return SFB_OK;
@@ -1777,8 +1776,8 @@ int tc_import_factors(sfb_ctx* ctx, int64_t off, int64_t n, const float* U_in, c
   return emit_p<true>(ctx, off, n, labels + off, nullptr);
 }
 
-// SDCA factors in bf16 mode: logits by the forward product, the dual changes in fp32 in place of the logits, then the
-// bf16 operand U^T = du (0 at the label entry, which goes to W in fp32 through coef, as for MLR).
+// SDCA factors in bf16 mode: logits by the forward product, then the dual changes, solved in fp32, as the bf16 operand U (0 at
+// the label entry, which goes to W in fp32 through coef, as for MLR).
 int tc_sdca_factors(sfb_ctx* ctx, int64_t off, int64_t n, const float* X, const int32_t* labels, const int32_t* ids,
                     float inv_lam_n, bool fused) {
   const sfb_config& c = ctx->cfg;
@@ -1789,10 +1788,18 @@ int tc_sdca_factors(sfb_ctx* ctx, int64_t off, int64_t n, const float* X, const 
   int tiles_n = 0;
   const int rc = mlr_forward(ctx, off, n, X, labels, fused, &tiles_n);
   if (rc) return rc;
-  CKC(sdca_dual_rows(ctx->stream, Z + off * ldz, n, rows, ldz, X, c.cols, labels, ids, ctx->dualQ, ctx->dual_n, inv_lam_n,
-                     c.eta, ctx->at<float>(L.coef) + off, ctx->at<float>(L.loss) + off, ctx->at<uint32_t>(L.status),
-                     fused ? ctx->at<int32_t>(L.slot) : nullptr, off));
-  return emit_p<true>(ctx, off, n, labels, fused ? X : nullptr);
+  SdcaArgs a = sdca_args(ctx, off, n, X, labels, ids, inv_lam_n);
+  a.Z = Z + off * ldz; a.ldz = ldz;
+  a.P = ctx->at<__nv_bfloat16>(L.P) + off * L.ldp; a.ldp = L.ldp;
+  a.coef = ctx->at<float>(L.coef) + off;
+  a.slot = fused ? ctx->at<int32_t>(L.slot) : nullptr;
+  CKC(sdca_dual_rows(ctx->stream, a));
+  if (fused) {
+    CKC(launch_kernel(label_delta_kernel, dim3(static_cast<unsigned>(label_blocks(ctx))), dim3(256), 0, ctx->stream, 1,
+                      label_args(ctx, X)));
+    ctx->labels = sfb_ctx::kLabelsApplied;
+  }
+  return SFB_OK;
 }
 
 int tc_factors(sfb_ctx* ctx, int64_t off, int64_t n, const float* X, const float* Y, const int32_t* labels, bool fused,
