@@ -234,7 +234,7 @@ static int factors_fp32(sfb_ctx* ctx, int64_t off, int64_t n, const float* X, co
     if (c.model == SFB_MLR)
       CK(mlr_softmax_rows(s, U, n, rows, ldu, labels, ctx->at<float>(ctx->lay.loss) + off, status));
     else
-      CK(dml_scale_rows(s, U, n, rows, ldu, labels, c.dml_margin, nullptr, 0, nullptr, dml_norm_out));
+      CK(dml_scale_rows(s, U, n, rows, ldu, labels, c.dml_margin, nullptr, 0, dml_norm_out));
     return SFB_OK;
   }
   // Sparse coding: ISTA from a = 0, then u = W a - x, v = a.  The first iterate is soft(W^T x / L).
@@ -492,7 +492,7 @@ extern "C" int sfb_finish_factors(sfb_ctx* ctx, const float* partials_all_dev, i
     const int64_t ldu = ctx->lay.ldu;
     CK(dml_scale_rows(ctx->stream, ctx->at<float>(ctx->lay.U), ctx->K, c.rows, ldu, ctx->at<int32_t>(ctx->lay.stageL),
                       c.dml_margin, c.precision == SFB_PREC_BF16 ? ctx->at<char>(ctx->lay.Rs) : nullptr, ctx->lay.rowsp, nullptr,
-                      nullptr, partials_all_dev, shards, ctx->K));
+                      partials_all_dev, shards, ctx->K));
     ctx->partials_ready = false;
     ctx->committed = c.workers == 64 ? ~0ull : ((1ull << c.workers) - 1);
     ctx->gathered = false;

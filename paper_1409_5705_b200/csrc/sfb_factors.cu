@@ -364,11 +364,10 @@ __global__ void __launch_bounds__(NTHREADS) sdca_dual_kernel(const __grid_consta
 }
 
 // One block per pair: q = ||z||^2; similar: u = 2z; dissimilar: u = -2z if q < margin else 0 (Section 2, DML).
-// Row-sharded form: with norm_out the block only stores its shard's q (after merging Z2) and leaves z as it is; with
+// Row-sharded form: with norm_out the block only stores its shard's q and leaves z as it is; with
 // norms_all it takes q as the sum, in shard order, of the shards' values and scales.
 template <int NTHREADS>
-__global__ void __launch_bounds__(NTHREADS) dml_scale_kernel(float* __restrict__ Z, const float* __restrict__ Z2,
-                                                             int64_t rows, int64_t ld,
+__global__ void __launch_bounds__(NTHREADS) dml_scale_kernel(float* __restrict__ Z, int64_t rows, int64_t ld,
                                                              const int32_t* __restrict__ similar, float margin,
                                                              float* __restrict__ norm_out,
                                                              const float* __restrict__ norms_all,
@@ -378,11 +377,6 @@ __global__ void __launch_bounds__(NTHREADS) dml_scale_kernel(float* __restrict__
   pdl_wait();
   __shared__ float sh[32];
   float* z = Z + static_cast<int64_t>(blockIdx.x) * ld;
-  if (Z2) {                      // z arrives as two partial sums over halves of the contraction (fixed order: Z + Z2)
-    const float* z2 = Z2 + static_cast<int64_t>(blockIdx.x) * ld;
-    for (int64_t j = threadIdx.x; j < rows; j += NTHREADS) z[j] += z2[j];
-    __syncthreads();
-  }
   float q = 0.f;
   if (norms_all) {
     for (int g = 0; g < shards; ++g) q += norms_all[g * nstride + blockIdx.x];
@@ -752,11 +746,10 @@ cudaError_t sdca_dual_rows(cudaStream_t s, const SdcaArgs& a) {
 }
 
 cudaError_t dml_scale_rows(cudaStream_t s, float* Z, int64_t nsamp, int64_t rows, int64_t ld,
-                           const int32_t* similar, float margin, void* split, int64_t split_half, const float* Z2,
-                           float* norm_out, const float* norms_all,
+                           const int32_t* similar, float margin, void* split, int64_t split_half, float* norm_out, const float* norms_all,
                            int shards, int64_t nstride) {
   if (nsamp <= 0) return cudaSuccess;
-  return launch_kernel(dml_scale_kernel<256>, dim3(static_cast<unsigned>(nsamp)), dim3(256), 0, s, 1, Z, Z2, rows, ld,
+  return launch_kernel(dml_scale_kernel<256>, dim3(static_cast<unsigned>(nsamp)), dim3(256), 0, s, 1, Z, rows, ld,
                        similar, margin, norm_out, norms_all, shards, nstride, static_cast<__nv_bfloat16*>(split),
                        split_half);
 }

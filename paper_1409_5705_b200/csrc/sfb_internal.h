@@ -104,7 +104,6 @@ struct Layout {
   size_t Wb, Xb, VT, ZT, UT, P, part, Xf, labels, coef, lse, slot, dL;   // VT, UT: tf32 words only; P: probabilities [K x ldp]; slot, dL: label rows
   // bf16 mode, DML and SC: (hi | lo) bf16 operands of the split products
   size_t Ws, WTs, As, Rs;             // W by rows, W transposed, the A operand (v or the codes), the residual
-  size_t U2;                          // DML: second partial of z when the forward product splits its contraction
   // sparse factors (MLR, csr_nnz_max > 0): the step's (sample, column, value) triples and their column-major form
   size_t coo_i, coo_c, coo_x, coo_cx, row_beg, row_end, csc_cnt, csc_cur, csc_ptr, csc_tmp, csc_ent;
   // sparse coding: the dictionary's Gram matrix (when the coder iterates on it), W^T x, the codes of odd iterations, and
@@ -113,6 +112,7 @@ struct Layout {
   int64_t ldu;                        // row pitch of the fp32 U buffer (rows rounded up to 4; rows itself with tf32 pairs)
   int64_t colsp, rowsp;               // cols, rows rounded up to 64
   int64_t Kp;                         // K rounded up to the contraction block of the update product
+  int32_t split;                      // parts that the bf16 forward product of MLR cuts its contraction into
   int32_t pw;                         // columns per softmax partial of the bf16 forward product
   int64_t ldp;                        // row pitch of P: rows rounded up to 64
   int64_t colsb;                      // cols rounded up to the contraction block of the forward product
@@ -275,12 +275,11 @@ struct SdcaArgs {
 cudaError_t sdca_dual_rows(cudaStream_t s, const SdcaArgs& a);
 SdcaArgs sdca_args(const sfb_ctx* ctx, int64_t off, int64_t n, const float* X, const int32_t* labels, const int32_t* ids,
                    float inv_lam_n);               // all but the logits and where du goes
-// Z2 (may be null): a second partial of z (the other half of the contraction), added to Z first.  Row-sharded form:
-// norm_out (may be null) receives the shard's ||z_i||^2 and z is left unscaled; norms_all (may be null), [shards][nstride],
-// supplies ||z_i||^2 as the sum over the shards instead of this context's own.
+// Row-sharded form: norm_out (may be null) receives the shard's ||z_i||^2 and z is left unscaled; norms_all (may be null),
+// [shards][nstride], supplies ||z_i||^2 as the sum over the shards instead of this context's own.
 // split (may be null): the scaled rows also as (hi | lo) bf16 pairs, row pitch 2 * split_half.
 cudaError_t dml_scale_rows(cudaStream_t s, float* Z, int64_t nsamp, int64_t rows, int64_t ld,
-                           const int32_t* similar, float margin, void* split, int64_t split_half, const float* Z2 = nullptr, float* norm_out = nullptr,
+                           const int32_t* similar, float margin, void* split, int64_t split_half, float* norm_out = nullptr,
                            const float* norms_all = nullptr, int shards = 0, int64_t nstride = 0);
 cudaError_t mean_of(cudaStream_t s, const float* v, int64_t n, float* out, const Stamp& st);
 cudaError_t prox_unit_columns(cudaStream_t s, float* W, int64_t rows, int64_t cols, float* colpart, unsigned long long* end);

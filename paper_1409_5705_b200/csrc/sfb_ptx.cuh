@@ -251,6 +251,14 @@ __device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_addr) {
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 
+// 16 bytes from the shared memory of CTA `rank` of this cluster, at this CTA's address `own_addr`.
+__device__ __forceinline__ float4 ld_cluster_f4(uint32_t own_addr, uint32_t rank) {
+  float4 v;
+  asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
+               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(mapa_u32(own_addr, rank)) : "memory");
+  return v;
+}
+
 // TMA load into this CTA's shared memory whose completion is signalled on an mbarrier that may live in the
 // peer CTA of the pair (bar_cluster_addr is a shared::cluster address).  Every CTA fetches its own tile.
 __device__ __forceinline__ void tma_load_2d_pair(void* dst, const CUtensorMap* m, int32_t x, int32_t y,

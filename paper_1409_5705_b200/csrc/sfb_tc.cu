@@ -75,8 +75,7 @@ struct TcParams {
   int64_t ldaux;
   float* C2;                   // F_ISTA0 (may be null), F_ISTAG: W^T x, [M x ldc]
   int32_t prefetch;            // k-blocks by which the producer asks L2 for the B operand ahead of its loads (0: off)
-  int32_t ksplit;              // forward_split_kernel, F_STORE: the contraction is cut into this many parts, each a work
-  int64_t c_split_stride;      //   unit of its own writing its partial product to C + part * c_split_stride (else 1, 0)
+  int32_t kparts;              // the contraction of a tile is cut over a cluster of this many CTAs (1: persistent CTAs)
   int32_t four;                // F_GRAM: with the fourth term A_lo B_lo
   const Scalars* sc;           // F_ISTA*: 1 / L
   float lam;                   // F_ISTA*: lambda
@@ -114,6 +113,34 @@ __device__ __forceinline__ void split_tile_coords(const TcParams& p, int tile, i
   n0 = tn * p.bn;
 }
 
+// Exchange of the partial tiles of a split contraction through the shared memory of the cluster's CTAs, in chunks of 32
+// columns x 128 rows of fp32 (16 KB, the operand stages' memory, which nothing uses any more); a warp writes and reads its 32
+// rows with the 16-byte pieces of a row swizzled.  Rank r then finishes the chunks c = r, r + split, ...; the sums are in rank
+// order, so they do not depend on timing.
+constexpr int kXchgBytes = BM * kChunk * 4;
+__device__ __forceinline__ uint32_t xchg_addr(uint8_t* smem, int c, int row, int j) {
+  return smem_u32(smem) + c * kXchgBytes + row * (kChunk * 4) + ((j ^ (row & 7)) << 4);
+}
+__device__ __forceinline__ void xchg_put(uint8_t* smem, int c, int row, const uint32_t (&acc)[32]) {
+#pragma unroll
+  for (int j = 0; j < 8; ++j)
+    asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(xchg_addr(smem, c, row, j)), "r"(acc[4 * j]), "r"(acc[4 * j + 1]),
+                 "r"(acc[4 * j + 2]), "r"(acc[4 * j + 3]) : "memory");
+}
+__device__ __forceinline__ void xchg_sum(uint8_t* smem, int c, int row, int split, uint32_t (&acc)[32]) {
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    const uint32_t at = xchg_addr(smem, c, row, j);
+    float4 s = ld_cluster_f4(at, 0);
+    for (int g = 1; g < split; ++g) {
+      const float4 v = ld_cluster_f4(at, g);
+      s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w;
+    }
+    acc[4 * j] = __float_as_uint(s.x); acc[4 * j + 1] = __float_as_uint(s.y);
+    acc[4 * j + 2] = __float_as_uint(s.z); acc[4 * j + 3] = __float_as_uint(s.w);
+  }
+}
+
 __device__ __forceinline__ float soft_threshold(float w, float t) {
   const float a = fabsf(w) - t;
   return a > 0.f ? copysignf(a, w) : 0.f;
@@ -140,7 +167,12 @@ forward_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int ntiles = p.tilesM * p.tilesN;
-  const int numK = p.nseg * p.kseg;
+  // With a split contraction a CTA has one tile and the k-blocks [kbeg, kend) of its nseg * kseg; else all of them and the
+  // tiles blockIdx.x, blockIdx.x + gridDim.x, ...
+  const int split = p.kparts, part = split > 1 ? static_cast<int>(blockIdx.x) % split : 0;
+  const int tile0 = static_cast<int>(blockIdx.x) / split, tile_step = split > 1 ? ntiles : static_cast<int>(gridDim.x);
+  const int kall = p.nseg * p.kseg;
+  const int kbeg = part * kall / split, kend = (part + 1) * kall / split;
   pdl_launch_dependents();
 
   if (threadIdx.x == 0) {
@@ -164,13 +196,14 @@ forward_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       const uint64_t pol_keep = policy_evict_last();
       uint32_t s = 0, ph = 0;
       bool ok = true;
-      for (int tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x) {
+      for (int tile = tile0; tile < ntiles && ok; tile += tile_step) {
         int m0, n0;
         tile_coords(p, tile, m0, n0);
         for (int seg = 0; seg < p.nseg && ok; ++seg) {
           const int xa0 = seg == 0 ? p.a_off0 : seg == 1 ? p.a_off1 : p.a_off2;
           const int xb0 = seg == 0 ? p.b_off0 : seg == 1 ? p.b_off1 : p.b_off2;
-          for (int kl = 0; kl < p.kseg; ++kl) {
+          const int kl1 = min(p.kseg, kend - seg * p.kseg);
+          for (int kl = max(0, kbeg - seg * p.kseg); kl < kl1; ++kl) {
             if (!mbar_wait(&empty[s], ph ^ 1, abort_flag)) { ok = false; break; }
             // B streams from HBM when it is larger than L2: with the box asked for a few k-blocks early, the load
             // that fills the stage finds it in L2 and the four stages cover the latency
@@ -191,12 +224,12 @@ forward_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       const uint32_t idesc = TF32 ? umma_idesc_tf32(BM, p.bn) : umma_idesc_bf16(BM, p.bn);
       uint32_t s = 0, ph = 0, tl = 0;
       bool ok = true;
-      for (int tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x, ++tl) {
+      for (int tile = tile0; tile < ntiles && ok; tile += tile_step, ++tl) {
         const uint32_t a = tl & 1, aph = (tl >> 1) & 1;
         if (!mbar_wait(&tempty[a], aph ^ 1, abort_flag)) { ok = false; break; }
         tc_fence_after();
         const uint32_t d_tmem = tmem_base + a * BN;
-        for (int kb = 0; kb < numK; ++kb) {
+        for (int kb = 0; kb < kend - kbeg; ++kb) {
           if (!mbar_wait(&full[s], ph, abort_flag)) { ok = false; break; }
           tc_fence_after();
           const uint64_t da = umma_desc_k128(smem_u32(smem + s * stage_bytes));
@@ -217,67 +250,85 @@ forward_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     // ---------------- epilogue: warps 2..5, TMEM lane quarter q ----------------
     const int q = warp & 3;
     uint8_t* ring = sRing + q * R * kSlotBytes;
-    const int my_tiles = blockIdx.x < ntiles ? (ntiles - 1 - blockIdx.x) / gridDim.x + 1 : 0;
+    const int my_tiles = tile0 < ntiles ? (ntiles - 1 - tile0) / tile_step + 1 : 0;
     bool ok = true;
-
-    {
-      // The fp32 result goes out through the ring by TMA; F_SOFTMAX keeps a running (max, sum exp) per sample.
-      uint32_t gs = 0;                       // stores issued so far: consecutive stores alternate ring slots
-      for (int tl = 0; tl < my_tiles && ok; ++tl) {
-        int m0, n0;
-        tile_coords(p, blockIdx.x + tl * gridDim.x, m0, n0);
-        const uint32_t a = tl & 1, aph = (tl >> 1) & 1;
-        if (!__all_sync(0xffffffffu, mbar_wait(&tfull[a], aph, abort_flag))) { ok = false; break; }
-        tc_fence_after();
-        const int row = m0 + q * 32 + lane;
-        float mx = -INFINITY, sum = 0.f;
-        for (int c = 0; c < p.bn / kChunk; ++c) {
-          uint8_t* sl = ring + (gs % R) * kSlotBytes;
-          uint32_t acc[32];
-          tmem_ld_32x32(tmem_base + (static_cast<uint32_t>(q * 32) << 16) + a * BN + c * kChunk, acc);
-          tmem_ld_wait();
-          const int col0 = n0 + c * kChunk;
-          if (col0 < p.N) {
-            if constexpr (EPI == F_SOFTMAX) {
-              float cm = -INFINITY;
+    // The fp32 result goes out through the ring by TMA; F_SOFTMAX keeps a running (max, sum exp) per sample.
+    uint32_t gs = 0;                       // stores issued so far: consecutive stores alternate ring slots
+    float mx = -INFINITY, sum = 0.f;
+    auto finish = [&](uint32_t (&acc)[32], int m0, int n0, int c) {
+      uint8_t* sl = ring + (gs % R) * kSlotBytes;
+      const int col0 = n0 + c * kChunk, row = m0 + q * 32 + lane;
+      if (col0 < p.N) {
+        if constexpr (EPI == F_SOFTMAX) {
+          float cm = -INFINITY;
 #pragma unroll
-              for (int j = 0; j < 32; ++j)
-                if (col0 + j < p.N) cm = fmaxf(cm, __uint_as_float(acc[j]));
-              const float nm = fmaxf(mx, cm);
-              float cs = 0.f;
+          for (int j = 0; j < 32; ++j)
+            if (col0 + j < p.N) cm = fmaxf(cm, __uint_as_float(acc[j]));
+          const float nm = fmaxf(mx, cm);
+          float cs = 0.f;
 #pragma unroll
-              for (int j = 0; j < 32; ++j)
-                if (col0 + j < p.N) cs += __expf(__uint_as_float(acc[j]) - nm);
-              sum = sum * __expf(mx - nm) + cs;
-              mx = nm;
-            }
-            if (lane == 0) tma_wait_group_read<R - 1>();   // the store that last used this slot has read it
-            __syncwarp();
-#pragma unroll
-            for (int j = 0; j < 8; ++j)
-              *reinterpret_cast<uint4*>(sl + lane * 128 + ((j ^ (lane & 7)) << 4)) =
-                  make_uint4(acc[4 * j], acc[4 * j + 1], acc[4 * j + 2], acc[4 * j + 3]);
-            fence_proxy_async_smem();
-            __syncwarp();
-            if (lane == 0) {
-              tma_store_2d(&tmC, sl, col0, m0 + q * 32);
-              tma_commit_group();
-            }
-            ++gs;
-          }
-          if (EPI == F_SOFTMAX && ((c + 1) * kChunk) % p.pw == 0) {      // the end of a group of pw columns
-            const int grp = (n0 + (c + 1) * kChunk) / p.pw - 1;
-            if (grp * p.pw < p.N && row < p.M) p.part[static_cast<int64_t>(grp) * p.part_ld + row] = make_float2(mx, sum);
-            mx = -INFINITY;
-            sum = 0.f;
-          }
+          for (int j = 0; j < 32; ++j)
+            if (col0 + j < p.N) cs += __expf(__uint_as_float(acc[j]) - nm);
+          sum = sum * __expf(mx - nm) + cs;
+          mx = nm;
         }
-        tc_fence_before();
+        if (lane == 0) tma_wait_group_read<R - 1>();   // the store that last used this slot has read it
         __syncwarp();
-        if (lane == 0) mbar_arrive(&tempty[a]);
+#pragma unroll
+        for (int j = 0; j < 8; ++j)
+          *reinterpret_cast<uint4*>(sl + lane * 128 + ((j ^ (lane & 7)) << 4)) =
+              make_uint4(acc[4 * j], acc[4 * j + 1], acc[4 * j + 2], acc[4 * j + 3]);
+        fence_proxy_async_smem();
+        __syncwarp();
+        if (lane == 0) {
+          tma_store_2d(&tmC, sl, col0, m0 + q * 32);
+          tma_commit_group();
+        }
+        ++gs;
       }
-      if (lane == 0) tma_wait_group<0>();
+      if (EPI == F_SOFTMAX && ((c + 1) * kChunk) % p.pw == 0) {      // the end of a group of pw columns
+        const int grp = (n0 + (c + 1) * kChunk) / p.pw - 1;
+        if (grp * p.pw < p.N && row < p.M) p.part[static_cast<int64_t>(grp) * p.part_ld + row] = make_float2(mx, sum);
+        mx = -INFINITY;
+        sum = 0.f;
+      }
+    };
+    for (int tl = 0; tl < my_tiles && ok; ++tl) {
+      int m0, n0;
+      tile_coords(p, tile0 + tl * tile_step, m0, n0);
+      const uint32_t a = tl & 1, aph = (tl >> 1) & 1;
+      if (!__all_sync(0xffffffffu, mbar_wait(&tfull[a], aph, abort_flag))) { ok = false; break; }
+      tc_fence_after();
+      for (int c = 0; c < p.bn / kChunk; ++c) {
+        uint32_t acc[32];
+        tmem_ld_32x32(tmem_base + (static_cast<uint32_t>(q * 32) << 16) + a * BN + c * kChunk, acc);
+        tmem_ld_wait();
+        if (split > 1) xchg_put(smem, c, q * 32 + lane, acc);
+        else finish(acc, m0, n0, c);
+      }
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&tempty[a]);
     }
+    if (split > 1) {
+      __syncwarp();
+      cluster_arrive();
+      cluster_wait();
+      int m0, n0;
+      tile_coords(p, tile0, m0, n0);
+      for (int c = part; c < p.bn / kChunk && ok; c += split) {        // (pw is 32: a group is a chunk)
+        uint32_t acc[32];
+        xchg_sum(smem, c, q * 32 + lane, split, acc);
+        finish(acc, m0, n0, c);
+      }
+    }
+    if (lane == 0) tma_wait_group<0>();
+  }
+  if (split > 1) {
+    __syncwarp();
+    if (warp < 2) { cluster_arrive(); cluster_wait(); }                // (the epilogue warps have been there)
+    cluster_arrive();                                                  // no CTA leaves while a peer still reads its part
+    cluster_wait();
   }
 
   // ---------------- teardown ----------------
@@ -310,10 +361,12 @@ constexpr int FS_STAGES = 3;
 constexpr int kFsBytesB = FS_BN * BK * 2;           // 20 KB
 constexpr int kFsStage = 2 * kBytesA + 2 * kFsBytesB;
 constexpr int kFsBars = 2 * FS_STAGES + 4;
+constexpr int kFsEpi = 8;                           // epilogue warps: two per TMEM lane quarter, taking turns at the chunks
+constexpr int kFsThreads = 64 + 32 * kFsEpi;
 constexpr int kFsSmem = FS_STAGES * kFsStage + kFsBars * 8 + 16 + 1024;
 
 template <int EPI>
-__global__ void __launch_bounds__(kThreads, 1)
+__global__ void __launch_bounds__(kFsThreads, 1)
 forward_split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, float* __restrict__ C,
                      int64_t ldc, const TcParams p) {
   extern __shared__ uint8_t smem_raw[];
@@ -327,9 +380,11 @@ forward_split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
   volatile uint32_t* abort_flag = tmem_slot + 1;
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int S = p.ksplit > 1 ? p.ksplit : 1;
-  const int ntiles = (EPI == F_GRAM ? sym_tiles(p.tilesM, p.tilesN, p.bn) : p.tilesM * p.tilesN) * S;   // work units: (tile, part of the contraction), parts of a tile adjacent
-  const int numKall = p.kseg;                       // k-blocks of the contraction (each serves three products)
+  const int ntiles = EPI == F_GRAM ? sym_tiles(p.tilesM, p.tilesN, p.bn) : p.tilesM * p.tilesN;
+  // the tiles and k-blocks (each serves three products) of this CTA, as in forward_kernel
+  const int split = p.kparts, part = split > 1 ? static_cast<int>(blockIdx.x) % split : 0;
+  const int tile0 = static_cast<int>(blockIdx.x) / split, tile_step = split > 1 ? ntiles : static_cast<int>(gridDim.x);
+  const int kbeg = part * p.kseg / split, kend = (part + 1) * p.kseg / split;
   // Two accumulators per tile: A_hi B_hi, and the cross terms at column `cross` of it.  Tiles of at most 128 columns have room
   // for two such pairs (the epilogue of one tile then overlaps the products of the next), wider ones for one.
   const int nacc = p.bn <= 128 ? 2 : 1, cross = p.bn <= 128 ? 128 : 256;
@@ -338,7 +393,7 @@ forward_split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
   pdl_launch_dependents();
   if (threadIdx.x == 0) {
     for (int i = 0; i < FS_STAGES; ++i) { mbar_init(&full[i], 1); mbar_init(&empty[i], 1); }
-    for (int i = 0; i < 2; ++i) { mbar_init(&tfull[i], 1); mbar_init(&tempty[i], 4); }
+    for (int i = 0; i < 2; ++i) { mbar_init(&tfull[i], 1); mbar_init(&tempty[i], kFsEpi); }
     *abort_flag = 0;
     fence_barrier_init();
     prefetch_tmap(&tmA); prefetch_tmap(&tmB);
@@ -357,14 +412,13 @@ forward_split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
       const uint32_t stage_bytes = 2 * kBytesA + 2 * static_cast<uint32_t>(p.bn) * BK * 2;
       uint32_t it = 0;
       bool ok = true;
-      for (int tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x) {
+      for (int tile = tile0; tile < ntiles && ok; tile += tile_step) {
         int m0, n0;
-        split_tile_coords<EPI>(p, tile / S, m0, n0);
-        const int part = tile % S, kbeg = part * numKall / S, numK = (part + 1) * numKall / S;
-        for (int kl = kbeg; kl < numK; ++kl, ++it) {
+        split_tile_coords<EPI>(p, tile, m0, n0);
+        for (int kl = kbeg; kl < kend; ++kl, ++it) {
           const uint32_t s = it % FS_STAGES, ph = (it / FS_STAGES) & 1;
           if (!mbar_wait(&empty[s], ph ^ 1, abort_flag)) { ok = false; break; }
-          if (p.prefetch > 0 && kl + p.prefetch < numK) {          // B streams from HBM when it is larger than L2
+          if (p.prefetch > 0 && kl + p.prefetch < kend) {          // B streams from HBM when it is larger than L2
             tma_prefetch_2d(&tmB, b_hi + (kl + p.prefetch) * BK, n0);
             tma_prefetch_2d(&tmB, b_lo + (kl + p.prefetch) * BK, n0);
           }
@@ -383,13 +437,12 @@ forward_split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
       const uint32_t idesc = umma_idesc_bf16(BM, p.bn);
       uint32_t it = 0, tl = 0;
       bool ok = true;
-      for (int tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x, ++tl) {
+      for (int tile = tile0; tile < ntiles && ok; tile += tile_step, ++tl) {
         const uint32_t a = tl % nacc, aph = (tl / nacc) & 1;
         if (!mbar_wait(&tempty[a], aph ^ 1, abort_flag)) { ok = false; break; }
         tc_fence_after();
         const uint32_t d_tmem = tmem_base + a * BN, d_cross = d_tmem + cross;
-        const int part = tile % S, numK = (part + 1) * numKall / S - part * numKall / S;
-        for (int kb = 0; kb < numK; ++kb, ++it) {
+        for (int kb = 0; kb < kend - kbeg; ++kb, ++it) {
           const uint32_t s = it % FS_STAGES, ph = (it / FS_STAGES) & 1;
           if (!mbar_wait(&full[s], ph, abort_flag)) { ok = false; break; }
           tc_fence_after();
@@ -413,24 +466,123 @@ forward_split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
       }
     }
   } else {
-    // ---------------- epilogue: warps 2..5, TMEM lane quarter q; results leave straight from registers ----------------
-    const int q = warp & 3;
-    const int my_tiles = blockIdx.x < ntiles ? (ntiles - 1 - blockIdx.x) / gridDim.x + 1 : 0;
+    // ---------------- epilogue: warp (q, h) = TMEM lane quarter q, every second chunk; results leave straight from registers
+    const int q = warp & 3, h = (warp - 2) >> 2;
+    const int my_tiles = tile0 < ntiles ? (ntiles - 1 - tile0) / tile_step + 1 : 0;
     bool ok = true;
     float invL = 0.f, thr = 0.f;
     if (kIsta<EPI>) { invL = p.sc->invL; thr = p.lam * invL; }
-    for (int tl = 0; tl < my_tiles && ok; ++tl) {
-      int m0, n0;
-      const int unit = blockIdx.x + tl * gridDim.x;
-      split_tile_coords<EPI>(p, unit / S, m0, n0);
-      float* Cp = C + static_cast<int64_t>(unit % S) * p.c_split_stride;
-      const uint32_t a = tl % nacc, aph = (tl / nacc) & 1;
-      if (!__all_sync(0xffffffffu, mbar_wait(&tfull[a], aph, abort_flag))) { ok = false; break; }
-      tc_fence_after();
+    auto finish = [&](uint32_t (&acc)[32], int m0, int n0, int c) {
       const int row = m0 + q * 32 + lane;
       // the tile's columns end at nlim; its width is a multiple of 16, so the last 32-column chunk may be half used
       const int nlim = min(p.N, n0 + p.bn);
-      for (int c = 0; c < (p.bn + kChunk - 1) / kChunk; ++c) {
+      const int col0 = n0 + c * kChunk;
+      if (col0 >= nlim || row >= p.M) return;
+      if constexpr (EPI == F_ISTAG || EPI == F_ISTA0) {
+        // W^T x of the sample (N, hence every pitch, is a multiple of 4 for the products over atoms)
+        float* bp = p.C2 ? p.C2 + static_cast<int64_t>(row) * ldc + col0 : nullptr;
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+          if (!bp || col0 + 4 * j + 4 > nlim) continue;
+          if constexpr (EPI == F_ISTAG) {
+            const float4 b4 = *reinterpret_cast<const float4*>(bp + 4 * j);
+            acc[4 * j] = __float_as_uint(__uint_as_float(acc[4 * j]) - b4.x);
+            acc[4 * j + 1] = __float_as_uint(__uint_as_float(acc[4 * j + 1]) - b4.y);
+            acc[4 * j + 2] = __float_as_uint(__uint_as_float(acc[4 * j + 2]) - b4.z);
+            acc[4 * j + 3] = __float_as_uint(__uint_as_float(acc[4 * j + 3]) - b4.w);
+          } else {
+            *reinterpret_cast<uint4*>(bp + 4 * j) = make_uint4(acc[4 * j], acc[4 * j + 1], acc[4 * j + 2], acc[4 * j + 3]);
+          }
+        }
+      }
+      if constexpr (EPI != F_STORE) {
+        if constexpr (EPI == F_SUB || EPI == F_ISTA || EPI == F_ISTAG) {
+          // the sample's values of aux (x, or the current code a) are contiguous: up to 128 bytes per lane
+          float xv[32];
+          const float* ap = p.aux + static_cast<int64_t>(row) * p.ldaux + col0;
+          const bool ap16 = (reinterpret_cast<uintptr_t>(ap) & 15u) == 0;
+#pragma unroll
+          for (int j = 0; j < 8; ++j) {
+            if (ap16 && col0 + 4 * j + 4 <= nlim) {
+              const float4 v4 = *reinterpret_cast<const float4*>(ap + 4 * j);
+              xv[4 * j] = v4.x; xv[4 * j + 1] = v4.y; xv[4 * j + 2] = v4.z; xv[4 * j + 3] = v4.w;
+            } else {
+#pragma unroll
+              for (int e = 0; e < 4; ++e) xv[4 * j + e] = col0 + 4 * j + e < nlim ? ap[4 * j + e] : 0.f;
+            }
+          }
+#pragma unroll
+          for (int j = 0; j < 32; ++j) {
+            const float d = __uint_as_float(acc[j]);
+            acc[j] = __float_as_uint(EPI == F_SUB ? d - xv[j] : soft_threshold(fmaf(-d, invL, xv[j]), thr));
+          }
+        }
+        if constexpr (EPI == F_ISTA0) {
+#pragma unroll
+          for (int j = 0; j < 32; ++j) acc[j] = __float_as_uint(soft_threshold(__uint_as_float(acc[j]) * invL, thr));
+        }
+#pragma unroll
+        for (int j = 0; j < 32; ++j) acc[j] = col0 + j < p.N ? acc[j] : 0u;
+        // (hi | lo) bf16 pair of the result: the operand of the next product (zero in the padding past N; the
+        // columns past this tile's width belong to the next tile)
+        __nv_bfloat16* hp = p.split + static_cast<int64_t>(row) * p.ld_split + col0;
+        const int split_lim = min(p.split_half, n0 + p.bn);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          if (col0 + 8 * j < split_lim) {
+            uint32_t hi[4], lo[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+              const float f0 = __uint_as_float(acc[8 * j + 2 * e]), f1 = __uint_as_float(acc[8 * j + 2 * e + 1]);
+              const __nv_bfloat16 h0 = __float2bfloat16_rn(f0), h1 = __float2bfloat16_rn(f1);
+              hi[e] = static_cast<uint32_t>(__bfloat16_as_ushort(h0)) |
+                      (static_cast<uint32_t>(__bfloat16_as_ushort(h1)) << 16);
+              const __nv_bfloat162 l2 = __floats2bfloat162_rn(f0 - __bfloat162float(h0), f1 - __bfloat162float(h1));
+              lo[e] = *reinterpret_cast<const uint32_t*>(&l2);
+            }
+            *reinterpret_cast<uint4*>(hp + 8 * j) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+            *reinterpret_cast<uint4*>(hp + p.split_half + 8 * j) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+          }
+        }
+      }
+      if constexpr (EPI == F_GRAM) {
+        // the mirror images of the entries whose own tile is not formed: lanes are neighbouring columns there
+        const int own_end = (row / p.bn + 1) * p.bn;              // end of the column block that row lies in
+#pragma unroll
+        for (int j = 0; j < 32; ++j) {
+          const int n = col0 + j;
+          if (n >= nlim || own_end > n / BM * BM) continue;
+          const float f = __uint_as_float(acc[j]);
+          const __nv_bfloat16 hi = __float2bfloat16_rn(f);
+          __nv_bfloat16* hp = p.split + static_cast<int64_t>(n) * p.ld_split + row;
+          hp[0] = hi;
+          hp[p.split_half] = __float2bfloat16_rn(f - __bfloat162float(hi));
+          if (C) C[static_cast<int64_t>(n) * ldc + row] = f;
+        }
+        if (!C) return;
+      }
+      // the fp32 result: this lane's consecutive columns of its row
+      float* cp = C + static_cast<int64_t>(row) * ldc + col0;
+      const bool cp16 = (reinterpret_cast<uintptr_t>(cp) & 15u) == 0;
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        if (cp16 && col0 + 4 * j + 4 <= nlim) {
+          *reinterpret_cast<uint4*>(cp + 4 * j) = make_uint4(acc[4 * j], acc[4 * j + 1], acc[4 * j + 2], acc[4 * j + 3]);
+        } else {
+#pragma unroll
+          for (int e = 0; e < 4; ++e)
+            if (col0 + 4 * j + e < nlim) cp[4 * j + e] = __uint_as_float(acc[4 * j + e]);
+        }
+      }
+    };
+    const int chunks = (p.bn + kChunk - 1) / kChunk;
+    for (int tl = 0; tl < my_tiles && ok; ++tl) {
+      int m0, n0;
+      split_tile_coords<EPI>(p, tile0 + tl * tile_step, m0, n0);
+      const uint32_t a = tl % nacc, aph = (tl / nacc) & 1;
+      if (!__all_sync(0xffffffffu, mbar_wait(&tfull[a], aph, abort_flag))) { ok = false; break; }
+      tc_fence_after();
+      for (int c = h; c < chunks; c += 2) {
         uint32_t acc[32];
         {
           uint32_t small[32];
@@ -441,109 +593,31 @@ forward_split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
 #pragma unroll
           for (int j = 0; j < 32; ++j) acc[j] = __float_as_uint(__uint_as_float(acc[j]) + __uint_as_float(small[j]));
         }
-        const int col0 = n0 + c * kChunk;
-        if (col0 >= nlim || row >= p.M) continue;
-        if constexpr (EPI == F_ISTAG || EPI == F_ISTA0) {
-          // W^T x of the sample (N, hence every pitch, is a multiple of 4 for the products over atoms)
-          float* bp = p.C2 ? p.C2 + static_cast<int64_t>(row) * ldc + col0 : nullptr;
-#pragma unroll
-          for (int j = 0; j < 8; ++j) {
-            if (!bp || col0 + 4 * j + 4 > nlim) continue;
-            if constexpr (EPI == F_ISTAG) {
-              const float4 b4 = *reinterpret_cast<const float4*>(bp + 4 * j);
-              acc[4 * j] = __float_as_uint(__uint_as_float(acc[4 * j]) - b4.x);
-              acc[4 * j + 1] = __float_as_uint(__uint_as_float(acc[4 * j + 1]) - b4.y);
-              acc[4 * j + 2] = __float_as_uint(__uint_as_float(acc[4 * j + 2]) - b4.z);
-              acc[4 * j + 3] = __float_as_uint(__uint_as_float(acc[4 * j + 3]) - b4.w);
-            } else {
-              *reinterpret_cast<uint4*>(bp + 4 * j) = make_uint4(acc[4 * j], acc[4 * j + 1], acc[4 * j + 2], acc[4 * j + 3]);
-            }
-          }
-        }
-        if constexpr (EPI != F_STORE) {
-          if constexpr (EPI == F_SUB || EPI == F_ISTA || EPI == F_ISTAG) {
-            // the sample's values of aux (x, or the current code a) are contiguous: up to 128 bytes per lane
-            float xv[32];
-            const float* ap = p.aux + static_cast<int64_t>(row) * p.ldaux + col0;
-            const bool ap16 = (reinterpret_cast<uintptr_t>(ap) & 15u) == 0;
-#pragma unroll
-            for (int j = 0; j < 8; ++j) {
-              if (ap16 && col0 + 4 * j + 4 <= nlim) {
-                const float4 v4 = *reinterpret_cast<const float4*>(ap + 4 * j);
-                xv[4 * j] = v4.x; xv[4 * j + 1] = v4.y; xv[4 * j + 2] = v4.z; xv[4 * j + 3] = v4.w;
-              } else {
-#pragma unroll
-                for (int e = 0; e < 4; ++e) xv[4 * j + e] = col0 + 4 * j + e < nlim ? ap[4 * j + e] : 0.f;
-              }
-            }
-#pragma unroll
-            for (int j = 0; j < 32; ++j) {
-              const float d = __uint_as_float(acc[j]);
-              acc[j] = __float_as_uint(EPI == F_SUB ? d - xv[j] : soft_threshold(fmaf(-d, invL, xv[j]), thr));
-            }
-          }
-          if constexpr (EPI == F_ISTA0) {
-#pragma unroll
-            for (int j = 0; j < 32; ++j) acc[j] = __float_as_uint(soft_threshold(__uint_as_float(acc[j]) * invL, thr));
-          }
-#pragma unroll
-          for (int j = 0; j < 32; ++j) acc[j] = col0 + j < p.N ? acc[j] : 0u;
-          // (hi | lo) bf16 pair of the result: the operand of the next product (zero in the padding past N; the
-          // columns past this tile's width belong to the next tile)
-          __nv_bfloat16* hp = p.split + static_cast<int64_t>(row) * p.ld_split + col0;
-          const int split_lim = min(p.split_half, n0 + p.bn);
-#pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            if (col0 + 8 * j < split_lim) {
-              uint32_t hi[4], lo[4];
-#pragma unroll
-              for (int e = 0; e < 4; ++e) {
-                const float f0 = __uint_as_float(acc[8 * j + 2 * e]), f1 = __uint_as_float(acc[8 * j + 2 * e + 1]);
-                const __nv_bfloat16 h0 = __float2bfloat16_rn(f0), h1 = __float2bfloat16_rn(f1);
-                hi[e] = static_cast<uint32_t>(__bfloat16_as_ushort(h0)) |
-                        (static_cast<uint32_t>(__bfloat16_as_ushort(h1)) << 16);
-                const __nv_bfloat162 l2 = __floats2bfloat162_rn(f0 - __bfloat162float(h0), f1 - __bfloat162float(h1));
-                lo[e] = *reinterpret_cast<const uint32_t*>(&l2);
-              }
-              *reinterpret_cast<uint4*>(hp + 8 * j) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
-              *reinterpret_cast<uint4*>(hp + p.split_half + 8 * j) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
-            }
-          }
-        }
-        if constexpr (EPI == F_GRAM) {
-          // the mirror images of the entries whose own tile is not formed: lanes are neighbouring columns there
-          const int own_end = (row / p.bn + 1) * p.bn;              // end of the column block that row lies in
-#pragma unroll
-          for (int j = 0; j < 32; ++j) {
-            const int n = col0 + j;
-            if (n >= nlim || own_end > n / BM * BM) continue;
-            const float f = __uint_as_float(acc[j]);
-            const __nv_bfloat16 hi = __float2bfloat16_rn(f);
-            __nv_bfloat16* hp = p.split + static_cast<int64_t>(n) * p.ld_split + row;
-            hp[0] = hi;
-            hp[p.split_half] = __float2bfloat16_rn(f - __bfloat162float(hi));
-            if (C) C[static_cast<int64_t>(n) * ldc + row] = f;
-          }
-          if (!C) continue;
-        }
-        // the fp32 result: this lane's consecutive columns of its row
-        float* cp = Cp + static_cast<int64_t>(row) * ldc + col0;
-        const bool cp16 = (reinterpret_cast<uintptr_t>(cp) & 15u) == 0;
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-          if (cp16 && col0 + 4 * j + 4 <= nlim) {
-            *reinterpret_cast<uint4*>(cp + 4 * j) = make_uint4(acc[4 * j], acc[4 * j + 1], acc[4 * j + 2], acc[4 * j + 3]);
-          } else {
-#pragma unroll
-            for (int e = 0; e < 4; ++e)
-              if (col0 + 4 * j + e < nlim) cp[4 * j + e] = __uint_as_float(acc[4 * j + e]);
-          }
-        }
+        if (split > 1) xchg_put(smem, c, q * 32 + lane, acc);
+        else finish(acc, m0, n0, c);
       }
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(&tempty[a]);
     }
+    if (split > 1) {
+      __syncwarp();
+      cluster_arrive();
+      cluster_wait();
+      int m0, n0;
+      split_tile_coords<EPI>(p, tile0, m0, n0);
+      for (int c = part + split * h; c < chunks && ok; c += 2 * split) {
+        uint32_t acc[32];
+        xchg_sum(smem, c, q * 32 + lane, split, acc);
+        finish(acc, m0, n0, c);
+      }
+    }
+  }
+  if (split > 1) {
+    __syncwarp();
+    if (warp < 2) { cluster_arrive(); cluster_wait(); }                // (the epilogue warps have been there)
+    cluster_arrive();                                                  // no CTA leaves while a peer still reads its part
+    cluster_wait();
   }
 
   // ---------------- teardown ----------------
@@ -1091,18 +1165,19 @@ cudaError_t launch_forward(sfb_ctx* ctx, const CUtensorMap& a, const CUtensorMap
   TcState* st = static_cast<TcState*>(ctx->tc);
   const int64_t tiles = static_cast<int64_t>(p.tilesM) * p.tilesN;
   if (tiles <= 0) return cudaSuccess;
-  const int grid = static_cast<int>(tiles < st->sms ? tiles : st->sms);
-  return launch_kernel_if(tiles <= st->sms, forward_kernel<EPI, TF32>, dim3(grid), dim3(kThreads), kSmem, ctx->stream, 1, a, b, c, p);
+  const unsigned grid = static_cast<unsigned>(p.kparts > 1 ? tiles * p.kparts : std::min<int64_t>(tiles, st->sms));
+  return launch_kernel_if(tiles * p.kparts <= st->sms, forward_kernel<EPI, TF32>, dim3(grid), dim3(kThreads), kSmem, ctx->stream,
+                          p.kparts, a, b, c, p);
 }
 
 template <int EPI>
 cudaError_t launch_forward_split(sfb_ctx* ctx, const CUtensorMap& a, const CUtensorMap& b, float* C, int64_t ldc, TcParams p) {
   TcState* st = static_cast<TcState*>(ctx->tc);
-  const int64_t tiles = EPI == F_GRAM ? sym_tiles(p.tilesM, p.tilesN, p.bn)
-                                      : static_cast<int64_t>(p.tilesM) * p.tilesN * (p.ksplit > 1 ? p.ksplit : 1);
+  const int64_t tiles = EPI == F_GRAM ? sym_tiles(p.tilesM, p.tilesN, p.bn) : static_cast<int64_t>(p.tilesM) * p.tilesN;
   if (tiles <= 0) return cudaSuccess;
-  const int grid = static_cast<int>(tiles < st->sms ? tiles : st->sms);
-  return launch_kernel_if(tiles <= st->sms, forward_split_kernel<EPI>, dim3(grid), dim3(kThreads), kFsSmem, ctx->stream, 1, a, b, C, ldc, p);
+  const unsigned grid = static_cast<unsigned>(p.kparts > 1 ? tiles * p.kparts : std::min<int64_t>(tiles, st->sms));
+  return launch_kernel_if(tiles * p.kparts <= st->sms, forward_split_kernel<EPI>, dim3(grid), dim3(kFsThreads), kFsSmem, ctx->stream,
+                          p.kparts, a, b, C, ldc, p);
 }
 
 // The shared-memory opt-in is a per-device attribute of each kernel: set for every instantiation when a context is
@@ -1134,21 +1209,36 @@ cudaError_t prepare_forward_kernels() {
 // Stages of the operand ring for tiles of bn columns (192 KB).
 static int forward_stages(int bn) { return std::min(S_MAX, S * (kBytesA + kBytesB) / (kBytesA + bn * BK * 2)); }
 
-// Tile width of the forward product of n samples with a rows x cols matrix, a power of two from `least` to 256.  A k-block of a
-// tile takes the longest of its MMAs (2 cycles per column), its bytes at about 60 a cycle and the latency of its loads over
-// the stages in flight; wide tiles read the samples less often, narrow ones occupy more SMs when W has few rows (a worker's
-// 37 samples against 4,999 x 3,004: 23 us with 256-wide tiles on 20 SMs).
-static int pick_forward_width(int64_t n, int64_t rows, int64_t cols, int least) {
-  const int sms = sm_count();
+// Cycles of the forward product of n samples with a rows x cols matrix in tiles of bn columns and `split` parts.  A k-block of
+// a tile takes the longest of its MMAs (2 cycles per column), its bytes at about 60 a cycle and the latency of its loads over
+// the stages in flight; the exchange of the parts about 3000.
+static double forward_cost(int64_t n, int64_t rows, int64_t cols, int bn, int split) {
   const double kb = static_cast<double>((cols + BK - 1) / BK), ar = static_cast<double>(std::min<int64_t>(BM, round_up(n, 8)));
-  int best = 256;
-  double best_cost = 0.;
-  for (int bn = 256; bn >= least; bn /= 2) {
-    const int64_t tiles = ((n + BM - 1) / BM) * ((rows + bn - 1) / bn);
-    const double rounds = static_cast<double>((tiles + sms - 1) / sms);
-    const double per_kb = std::max(std::max(2.0 * bn, (ar + bn) * BK * 2 / 60.0), 1200.0 / forward_stages(bn));
-    const double cost = rounds * (kb * per_kb + 2500.0);
-    if (bn == 256 || cost < 0.97 * best_cost) { best = bn; best_cost = cost; }
+  const int64_t ctas = ((n + BM - 1) / BM) * ((rows + bn - 1) / bn) * split;
+  const double rounds = static_cast<double>((ctas + sm_count() - 1) / sm_count());
+  const double per_kb = std::max(std::max(2.0 * bn, (ar + bn) * BK * 2 / 60.0), 1200.0 / forward_stages(bn));
+  return rounds * (kb / split * per_kb + 2500.0 + (split > 1 ? 3000.0 : 0.0));
+}
+// Tile width: a power of two from `least` to 256 (128 with a split contraction, whose parts are exchanged through the operand
+// stages).  Wide tiles read the samples less often, narrow ones occupy more SMs when W has few rows (a worker's 37 samples
+// against 4,999 x 3,004: 23 us with 256-wide tiles on 20 SMs).
+static int pick_forward_width(int64_t n, int64_t rows, int64_t cols, int least, int split) {
+  int best = split > 1 ? 128 : 256;
+  double cost = forward_cost(n, rows, cols, best, split);
+  for (int bn = best / 2; bn >= least; bn /= 2) {
+    const double c = forward_cost(n, rows, cols, bn, split);
+    if (c < 0.97 * cost) { cost = c; best = bn; }
+  }
+  return best;
+}
+// Parts that the contraction of the forward product is cut into when the tiles of all K samples do not fill the SMs (72 rows of
+// 14,240 columns: 223 k-blocks in a row on one SM, 68 us).  One choice per context: it fixes the order of the sums.
+static int pick_forward_split(int64_t K, int64_t rows, int64_t cols) {
+  int best = 1;
+  double cost = forward_cost(K, rows, cols, pick_forward_width(K, rows, cols, 32, 1), 1);
+  for (int s = 2; s <= 8 && (cols + BK - 1) / BK >= 2 * s; s *= 2) {
+    const double c = forward_cost(K, rows, cols, pick_forward_width(K, rows, cols, 32, s), s);
+    if (c < 0.9 * cost) { cost = c; best = s; }
   }
   return best;
 }
@@ -1187,7 +1277,6 @@ void tc_extend_layout(const sfb_config& c, Layout& L, size_t& off) {
     L.ldu = round_up(c.rows, 4);                                        // TMA stores need a 16-byte row pitch
     L.V = take(K * static_cast<size_t>(c.cols) * 4);
     L.U = take(K * static_cast<size_t>(L.ldu) * 4);
-    L.U2 = take(c.model == SFB_DML ? K * static_cast<size_t>(L.ldu) * 4 : 0);
     L.Rs = take(K * 2 * static_cast<size_t>(L.rowsp) * 2);              // u (SC: first x, then the residuals)
     L.Ws = take(static_cast<size_t>(c.rows) * 2 * L.colsp * 2);         // W, rows x (hi | lo)
     L.As = take(K * 2 * static_cast<size_t>(L.colsp) * 2);              // v (DML) or the codes a (SC)
@@ -1203,7 +1292,8 @@ void tc_extend_layout(const sfb_config& c, Layout& L, size_t& off) {
     return;
   }
   const size_t ldz = static_cast<size_t>(round_up(c.rows, 32));
-  L.pw = pick_forward_width(c.batch, c.rows, c.cols, 32);
+  L.split = pick_forward_split(static_cast<int64_t>(K), c.rows, c.cols);
+  L.pw = L.split > 1 ? 32 : pick_forward_width(c.batch, c.rows, c.cols, 32, 1);
   const size_t nblk = static_cast<size_t>((c.rows + L.pw - 1) / L.pw);
   L.Wb = take(static_cast<size_t>(c.rows) * L.colsb * 2);
   L.Xb = take(K * L.colsb * 2);
@@ -1302,6 +1392,7 @@ inline unsigned grid1d(int64_t items, int per_block) {
 inline int pick_tile_width(int sms, int64_t tilesM, int64_t N, int widest, int step = 32, bool sym = false) {
   int best = widest;
   int64_t best_cost = INT64_MAX;
+  if (N <= 112) return static_cast<int>(round_up(N, step));
   for (int bn = widest; bn >= 128; bn -= step) {
     const int64_t tn = (N + bn - 1) / bn;
     const int64_t tiles = sym ? sym_tiles(static_cast<int>(tilesM), static_cast<int>(tn), bn) : tilesM * tn;
@@ -1319,13 +1410,36 @@ constexpr int64_t kPreciseRows = 2048;
 
 constexpr int kSplitPrefetch = SFB_SPLIT_PREFETCH;    // k-blocks of look-ahead of the L2 prefetch in the split products
 
+// Cost of a split product in rounds of tiles x columns x k-blocks, its contraction in `split` parts.
+double split_cost(int64_t M, int64_t N, int64_t Kc, bool sym, int split) {
+  const int sms = sm_count();
+  const int64_t tm = (M + BM - 1) / BM;
+  const int bn = pick_tile_width(sms / split, tm, N, FS_BN, 16, sym);
+  const int64_t tn = (N + bn - 1) / bn;
+  const int64_t tiles = sym ? sym_tiles(static_cast<int>(tm), static_cast<int>(tn), bn) : tm * tn;
+  const double kb = static_cast<double>((Kc + BK - 1) / BK) / split;
+  return static_cast<double>((tiles * split + sms - 1) / sms) * (std::max(bn, 128) + 16) * (kb + 8.0 + (split > 1 ? 6.0 : 0.0));
+}
+// Parts of the contraction for all M samples of the product (a slice of them takes the same: it fixes the order of the sums):
+// where the tiles leave SMs idle and the k-blocks of one follow each other on one SM.
+int split_parts(int64_t M, int64_t N, int64_t Kc) {
+  int best = 1;
+  double cost = split_cost(M, N, Kc, false, 1);
+  for (int s = 2; s <= 8 && Kc / BK >= 2 * s; s *= 2) {
+    const double c = split_cost(M, N, Kc, false, s);
+    if (c < 0.9 * cost) { cost = c; best = s; }
+  }
+  return best;
+}
+
 // One split-bf16 product  D[off..off+n) = A * B^T  with A = [*, 2*Cp] and B = [N x 2*Cp] (hi | lo) operands:
 // hi*hi + hi*lo + lo*hi over a contraction of Cp.
 template <int EPI>
 int split_product(sfb_ctx* ctx, int64_t off, int64_t n, __nv_bfloat16* A, __nv_bfloat16* B, int64_t N, int64_t Cp,
-                  float* C, int64_t ldc, TcParams p, int64_t c_split_stride = 0, int* parts_out = nullptr) {
+                  float* C, int64_t ldc, TcParams p) {
   TcState* st = static_cast<TcState*>(ctx->tc);
-  const int bn = pick_tile_width(st->sms, (n + BM - 1) / BM, N, FS_BN, 16, EPI == F_GRAM);
+  p.kparts = EPI == F_GRAM ? 1 : split_parts(ctx->K, N, Cp);
+  const int bn = pick_tile_width(st->sms / p.kparts, (n + BM - 1) / BM, N, FS_BN, 16, EPI == F_GRAM);
   CUtensorMap ma, mb;
   if (!make_map(st, &ma, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, A, 2 * Cp, off + n, 2 * Cp * 2, BK, BM) ||
       !make_map(st, &mb, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, B, 2 * Cp, N, 2 * Cp * 2, BK, bn))
@@ -1337,12 +1451,6 @@ int split_product(sfb_ctx* ctx, int64_t off, int64_t n, __nv_bfloat16* A, __nv_b
   p.tilesN = static_cast<int32_t>((N + bn - 1) / bn);
   p.nseg = 3; p.kseg = static_cast<int32_t>(Cp / BK);
   p.prefetch = kSplitPrefetch;
-  // a product whose tiles fill less than half of the SMs is cut along its contraction (plain store epilogue only: the
-  // partial products are added, in a fixed order, by the kernel that consumes them)
-  const int64_t tiles = static_cast<int64_t>(p.tilesM) * p.tilesN;
-  p.ksplit = (EPI == F_STORE && c_split_stride > 0 && 2 * tiles <= st->sms && p.kseg >= 8) ? 2 : 1;
-  p.c_split_stride = p.ksplit > 1 ? c_split_stride : 0;
-  if (parts_out) *parts_out = p.ksplit;
   p.a_off0 = 0; p.a_off1 = 0; p.a_off2 = static_cast<int32_t>(Cp);
   p.b_off0 = 0; p.b_off1 = static_cast<int32_t>(Cp); p.b_off2 = 0;
   p.status = ctx->at<uint32_t>(ctx->lay.status);
@@ -1368,13 +1476,10 @@ int factors_split(sfb_ctx* ctx, int64_t off, int64_t n, const float* X, const fl
   if (c.model == SFB_DML) {
     CKC(launch_kernel(pack_pairs_kernel, dim3(grid1d(n * cols / 4, 256)), dim3(256), 0, s, 1, X, Y, n, cols,
                       V + off * cols, As + off * 2 * L.colsp, L.colsp, Stamp{}));
-      float* U2 = ctx->at<float>(L.U2);
-    int parts = 1;
-    int rc = split_product<F_STORE>(ctx, off, n, As, Ws, rows, L.colsp, U, L.ldu, p, U2 - U, &parts);   // z_i = W v_i
+      int rc = split_product<F_STORE>(ctx, off, n, As, Ws, rows, L.colsp, U, L.ldu, p);    // z_i = W v_i
     if (rc) return rc;
     CKC(dml_scale_rows(s, U + off * L.ldu, n, rows, L.ldu, labels, c.dml_margin,
-                       ctx->at<__nv_bfloat16>(L.Rs) + off * 2 * L.rowsp, L.rowsp, parts > 1 ? U2 + off * L.ldu : nullptr,
-                       dml_norm_out));
+                       ctx->at<__nv_bfloat16>(L.Rs) + off * 2 * L.rowsp, L.rowsp, dml_norm_out));
     return SFB_OK;
   }
   // Sparse coding: ISTA from a = 0, then u = W a - x, v = a.  The first iterate is soft(W^T x / L).
@@ -1460,14 +1565,8 @@ int tc_begin_step(sfb_ctx* ctx) {
   return SFB_OK;
 }
 
-// Cost of a split product in rounds of tiles x columns x k-blocks (what pick_tile_width minimises).
 double split_product_cost(int64_t M, int64_t N, int64_t Kc, bool sym) {
-  const int sms = sm_count();
-  const int64_t tm = (M + BM - 1) / BM;
-  const int bn = pick_tile_width(sms, tm, N, FS_BN, 16, sym);
-  const int64_t tn = (N + bn - 1) / bn;
-  const int64_t tiles = sym ? sym_tiles(static_cast<int>(tm), static_cast<int>(tn), bn) : tm * tn;
-  return static_cast<double>((tiles + sms - 1) / sms) * (bn + 16) * (static_cast<double>((Kc + BK - 1) / BK) + 8.0);
+  return split_cost(M, N, Kc, sym, sym ? 1 : split_parts(M, N, Kc));
 }
 
 // v = x, the (big | small) samples, and the logits of n samples at pair offset off against this context's rows as
@@ -1496,7 +1595,7 @@ static int mlr32_forward(sfb_ctx* ctx, int64_t off, int64_t n, const float* X, i
   p.M = static_cast<int32_t>(off + n); p.N = static_cast<int32_t>(rows); p.Kc = static_cast<int32_t>(L.colsp);
   p.m_off = static_cast<int32_t>(off);
   p.tilesM = static_cast<int32_t>((n + BM - 1) / BM);
-  p.bn = BN; p.pw = BN; p.a_rows = BM; p.stages = S;
+  p.bn = BN; p.kparts = 1; p.pw = BN; p.a_rows = BM; p.stages = S;
   p.tilesN = static_cast<int32_t>((rows + BN - 1) / BN);
   p.part = ctx->at<float2>(L.part); p.part_ld = K; p.status = ctx->at<uint32_t>(L.status);
   p.nseg = 3; p.kseg = static_cast<int32_t>(L.colsp / (BK / 2));          // cross terms first, big*big last
@@ -1598,7 +1697,7 @@ static int mlr_forward(sfb_ctx* ctx, int64_t off, int64_t n, const float* X, con
                     rows,
                     take_stamp(ctx)));
   // samples on the lanes (A), rows of W on the accumulator columns (B)
-  const int bn = pick_forward_width(n, rows, cols, L.pw);
+  const int bn = pick_forward_width(n, rows, cols, L.pw, L.split);
   const int ar = static_cast<int>(std::min<int64_t>(BM, round_up(n, 8)));
   CUtensorMap ma, mb, mc;
   if (!make_map(st, &ma, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, Xb, cols, K, L.colsb * 2, BK, ar) ||
@@ -1609,7 +1708,7 @@ static int mlr_forward(sfb_ctx* ctx, int64_t off, int64_t n, const float* X, con
   p.M = static_cast<int32_t>(off + n); p.N = static_cast<int32_t>(rows); p.Kc = static_cast<int32_t>(cols);
   p.m_off = static_cast<int32_t>(off);
   p.tilesM = static_cast<int32_t>((n + BM - 1) / BM);
-  p.bn = bn; p.pw = L.pw; p.a_rows = ar; p.stages = forward_stages(bn);
+  p.bn = bn; p.kparts = L.split; p.pw = L.pw; p.a_rows = ar; p.stages = forward_stages(bn);
   p.tilesN = static_cast<int32_t>((rows + bn - 1) / bn);
   p.part = ctx->at<float2>(L.part); p.part_ld = K; p.status = ctx->at<uint32_t>(L.status);
   p.nseg = 1; p.kseg = (p.Kc + BK - 1) / BK;
