@@ -38,7 +38,7 @@ bool sc_use_gram(const sfb_config& c) {
   if (it < 1 || (c.precision == SFB_PREC_BF16 && A > D)) return false;
   if (A > (32 << 10)) return false;        // (the power iteration keeps a vector of A values on chip)
   auto cost = [&](int64_t M, int64_t N, int64_t Kc, bool sym) {
-    if (c.precision == SFB_PREC_BF16) return split_product_cost(M, N, Kc, sym);
+    if (c.precision == SFB_PREC_BF16 || use_h16(c)) return split_product_cost(M, N, Kc, sym);
     const GemmShape g = pick_gemm_shape(M, N, Kc, sym);
     return std::min(gemm_cost(128, g.split, M, N, Kc, sym), gemm_cost(64, g.split, M, N, Kc, sym));
   };
@@ -67,6 +67,8 @@ Layout make_layout(const sfb_config& cfg) {
   L.ldu = static_cast<int64_t>(rows);
   if (use_tf32(cfg)) {
     tc32_extend_layout(c, L, off);
+  } else if (use_h16(cfg)) {
+    split_extend_layout(c, L, off);
   } else if (c.precision != SFB_PREC_BF16) {
     L.ldu = round_up(c.rows, 4);                      // 16-byte row pitch
     L.V = take(K * cols * 4);
@@ -154,7 +156,8 @@ extern "C" int sfb_init(const sfb_config* cfg, float* W_dev, void* workspace_dev
   if (!ctx) return SFB_ERR_ARG;
   ctx->cfg = *cfg;
   ctx->tf32 = use_tf32(*cfg);
-  if (cfg->precision != SFB_PREC_BF16) ctx->cfg.precision = SFB_PREC_FP32;      // one fp32 family; tf32 says which kernels
+  ctx->h16 = use_h16(*cfg);
+  if (cfg->precision != SFB_PREC_BF16) ctx->cfg.precision = SFB_PREC_FP32;      // one fp32 family; tf32, h16 say which kernels
   ctx->sdca = cfg->model == SFB_L2MLR;
   if (ctx->sdca) ctx->cfg.model = SFB_MLR;            // the products, buffers and the update are those of MLR
   ctx->dualQ = nullptr;
@@ -193,7 +196,7 @@ extern "C" int sfb_init(const sfb_config* cfg, float* W_dev, void* workspace_dev
     ce = set_lipschitz(ctx->stream, ctx->at<Scalars>(lay.scalars), cfg->sc_lipschitz);
     if (ce != cudaSuccess) { sfb_destroy(ctx); return SFB_ERR_CUDA; }
   }
-  if (cfg->precision == SFB_PREC_BF16 || ctx->tf32) {
+  if (cfg->precision == SFB_PREC_BF16 || ctx->tf32 || ctx->h16) {
     rc = tc_init(ctx);
     if (rc) { sfb_destroy(ctx); return rc; }
   }
@@ -211,6 +214,19 @@ extern "C" int sfb_destroy(sfb_ctx* ctx) {
 // ---------------------------------------------------------------------------------------------------------
 // fp32-operand path
 // ---------------------------------------------------------------------------------------------------------
+// v = x (or x - y) of n pairs at offset off, and z = W v into U.
+static int logits_fp32(sfb_ctx* ctx, int64_t off, int64_t n, const float* X, const float* Y) {
+  if (ctx->h16) return split_logits(ctx, off, n, X, Y);
+  const sfb_config& c = ctx->cfg;
+  float* V = ctx->at<float>(ctx->lay.V) + off * c.cols;
+  CK(pack_copy(ctx->stream, V, X, Y, n * c.cols, take_stamp(ctx)));
+  EpiArgs e{};
+  e.C = ctx->at<float>(ctx->lay.U) + off * ctx->lay.ldu; e.ldc = ctx->lay.ldu;
+  CK(sgemm(ctx->stream, true, true, EPI_STORE, n, c.rows, c.cols, V, c.cols, ctx->W, c.cols, e, ctx->K));
+  ctx->stats.flops += 2.0 * n * c.rows * c.cols;
+  return SFB_OK;
+}
+
 static int factors_fp32(sfb_ctx* ctx, int64_t off, int64_t n, const float* X, const float* Y,
                         const int32_t* labels, bool sparse_fwd = false, float* dml_norm_out = nullptr) {
   const sfb_config& c = ctx->cfg;
@@ -222,21 +238,22 @@ static int factors_fp32(sfb_ctx* ctx, int64_t off, int64_t n, const float* X, co
   cudaStream_t s = ctx->stream;
   EpiArgs e{};
   if (c.model == SFB_MLR || c.model == SFB_DML) {
-    CK(pack_copy(s, V, X, c.model == SFB_DML ? Y : nullptr, n * cols, take_stamp(ctx)));      // v = x | x - y
-    e.C = U; e.ldc = ldu;
     if (sparse_fwd) {                                                                   // z_i = W v_i over the non-zeros of v_i
+      CK(pack_copy(s, V, X, nullptr, n * cols, take_stamp(ctx)));
       const int rc = sparse_forward(ctx, off, n, ctx->at<float>(ctx->lay.U), ldu);
       if (rc) return rc;
     } else {
-      CK(sgemm(s, true, true, EPI_STORE, n, rows, cols, V, cols, ctx->W, cols, e, K));  // z_i = W v_i
-      ctx->stats.flops += 2.0 * n * rows * cols;
+      const int rc = logits_fp32(ctx, off, n, X, c.model == SFB_DML ? Y : nullptr);
+      if (rc) return rc;
     }
     if (c.model == SFB_MLR)
       CK(mlr_softmax_rows(s, U, n, rows, ldu, labels, ctx->at<float>(ctx->lay.loss) + off, status));
     else
-      CK(dml_scale_rows(s, U, n, rows, ldu, labels, c.dml_margin, nullptr, 0, dml_norm_out));
+      CK(dml_scale_rows(s, U, n, rows, ldu, labels, c.dml_margin, nullptr, 0, ctx->h16 ? ctx->at<float>(ctx->lay.iA) + off : nullptr,
+                        ctx->h16 ? ctx->at<float>(ctx->lay.q) + off : nullptr, dml_norm_out));
     return SFB_OK;
   }
+  if (ctx->h16) return split_factors_sc(ctx, off, n, X);
   // Sparse coding: ISTA from a = 0, then u = W a - x, v = a.  The first iterate is soft(W^T x / L).
   const int T = c.sc_ista_iters;
   const bool gram = ctx->lay.G != 0;
@@ -277,14 +294,14 @@ static int factors_fp32(sfb_ctx* ctx, int64_t off, int64_t n, const float* X, co
 // the coder's Gram matrix and its step size.
 static int begin_step(sfb_ctx* ctx) {
   const sfb_config& c = ctx->cfg;
-  if (c.precision == SFB_PREC_BF16) {
-    const int rc = tc_begin_step(ctx);
+  if (ctx->h16 || (c.precision == SFB_PREC_BF16 && c.model != SFB_MLR)) {
+    const int rc = split_begin_step(ctx);
     if (rc) return rc;
   }
   if (c.model != SFB_SC) return SFB_OK;
   CK(stamp(ctx->stream, take_stamp(ctx)));
   float* G = ctx->lay.G ? ctx->at<float>(ctx->lay.G) : nullptr;
-  if (c.precision == SFB_PREC_FP32 && G) {
+  if (c.precision == SFB_PREC_FP32 && G && !ctx->h16) {
     EpiArgs e{};
     e.C = G; e.ldc = c.cols;
     CK(sgemm(ctx->stream, false, false, EPI_SYM, c.cols, c.cols, c.rows, ctx->W, c.cols, ctx->W, c.cols, e));
@@ -299,6 +316,7 @@ static int begin_step(sfb_ctx* ctx) {
 static int update_fp32(sfb_ctx* ctx) {
   const sfb_config& c = ctx->cfg;
   if (ctx->sparse_v) return sparse_update(ctx);
+  if (ctx->h16) return tc_update(ctx);
   EpiArgs e{};
   e.C = ctx->W; e.ldc = c.cols; e.alpha = -ctx->step;
   e.prox_kind = ctx->prox_kind; e.prox_a = ctx->prox_a;
@@ -377,12 +395,20 @@ static int compute_factors_csr(sfb_ctx* ctx, int32_t worker, const int64_t* indp
   if (ctx->csr_fill + nnz > c.csr_nnz_max) return SFB_ERR_SHAPE;
   const int64_t off = worker < 0 ? 0 : static_cast<int64_t>(worker) * c.batch;
   const int64_t n = worker < 0 ? ctx->K : c.batch;
-  if (ctx->committed == 0) begin_phase(ctx, 0);
-  int rc = sparse_stage(ctx, off, n, indptr_dev, indices_dev, values_dev, nnz);
+  if (ctx->committed == 0) {
+    begin_phase(ctx, 0);
+    ctx->begun = false;
+  }
+  int rc = SFB_OK;
+  if (!ctx->begun) {
+    if ((rc = begin_step(ctx)) != SFB_OK) return rc;
+    ctx->begun = true;
+  }
+  rc = sparse_stage(ctx, off, n, indptr_dev, indices_dev, values_dev, nnz);
   if (rc) return rc;
   const float* X = ctx->at<float>(ctx->lay.stageX) + off * c.cols;
   rc = ctx->tf32 ? tc32_factors(ctx, off, n, X, labels_dev, nullptr, 0.f)
-       : c.precision == SFB_PREC_FP32 ? factors_fp32(ctx, off, n, X, nullptr, labels_dev, sparse_forward_rows(ctx, n) > 0)
+       : c.precision == SFB_PREC_FP32 ? factors_fp32(ctx, off, n, X, nullptr, labels_dev, !ctx->h16 && sparse_forward_rows(ctx, n) > 0)
                                       : tc_factors(ctx, off, n, X, nullptr, labels_dev, fused);
   if (rc) return rc;
   ctx->csr_fill += nnz;
@@ -438,15 +464,9 @@ extern "C" int sfb_forward_partials(sfb_ctx* ctx, const float* X_dev, const int3
                    : tc_forward_partials(ctx, X_dev, labels_dev, partials_dev);
     if (rc) return rc;
   } else {
-    const int64_t K = ctx->K;
-    float* V = ctx->at<float>(ctx->lay.V);
+    const int64_t K = ctx->K, ldu = ctx->lay.ldu;
     float* U = ctx->at<float>(ctx->lay.U);
-    CK(pack_copy(ctx->stream, V, X_dev, nullptr, K * c.cols, take_stamp(ctx)));                                    // v = x
-    EpiArgs e{};
-    const int64_t ldu = ctx->lay.ldu;
-    e.C = U; e.ldc = ldu;
-    CK(sgemm(ctx->stream, true, true, EPI_STORE, K, c.rows, c.cols, V, c.cols, ctx->W, c.cols, e));   // z_i = W_shard x_i
-    ctx->stats.flops += 2.0 * K * c.rows * c.cols;
+    if ((rc = begin_step(ctx)) != SFB_OK || (rc = logits_fp32(ctx, 0, K, X_dev, nullptr)) != SFB_OK) return rc;    // z_i = W_shard x_i
     // the class ids are kept for the finish (the caller's buffer may change before it)
     CK(cudaMemcpyAsync(ctx->at<int32_t>(ctx->lay.stageL), labels_dev, static_cast<size_t>(K) * 4, cudaMemcpyDeviceToDevice,
                        ctx->stream));
@@ -491,7 +511,8 @@ extern "C" int sfb_finish_factors(sfb_ctx* ctx, const float* partials_all_dev, i
   if (c.model == SFB_DML) {
     const int64_t ldu = ctx->lay.ldu;
     CK(dml_scale_rows(ctx->stream, ctx->at<float>(ctx->lay.U), ctx->K, c.rows, ldu, ctx->at<int32_t>(ctx->lay.stageL),
-                      c.dml_margin, c.precision == SFB_PREC_BF16 ? ctx->at<char>(ctx->lay.Rs) : nullptr, ctx->lay.rowsp, nullptr,
+                      c.dml_margin, c.precision == SFB_PREC_BF16 ? ctx->at<char>(ctx->lay.Rs) : nullptr, ctx->lay.rowsp,
+                      ctx->h16 ? ctx->at<float>(ctx->lay.iA) : nullptr, ctx->h16 ? ctx->at<float>(ctx->lay.q) : nullptr, nullptr,
                       partials_all_dev, shards, ctx->K));
     ctx->partials_ready = false;
     ctx->committed = c.workers == 64 ? ~0ull : ((1ull << c.workers) - 1);
@@ -537,8 +558,8 @@ extern "C" int sfb_set_factors(sfb_ctx* ctx, int32_t worker, const float* U_dev,
   CK(cudaMemcpy2DAsync(U, static_cast<size_t>(ldu) * 4, U_dev, static_cast<size_t>(c.rows) * 4, static_cast<size_t>(c.rows) * 4,
                        static_cast<size_t>(c.batch), cudaMemcpyDeviceToDevice, ctx->stream));
   CK(cudaMemcpyAsync(V, V_dev, static_cast<size_t>(c.batch) * c.cols * 4, cudaMemcpyDeviceToDevice, ctx->stream));
-  if (c.precision == SFB_PREC_BF16) {
-    const int rc = tc_pack_received(ctx, off, c.batch);
+  if (c.precision == SFB_PREC_BF16 || ctx->h16) {
+    const int rc = split_pack_received(ctx, off, c.batch);
     if (rc) return rc;
   }
   ctx->committed |= 1ull << worker;
@@ -593,6 +614,9 @@ extern "C" int sfb_gather_factors(sfb_ctx* ctx) {
   } else if (ctx->tf32) {
     CK(stamp(ctx->stream, take_stamp(ctx)));
     int rc = tc32_gather(ctx);
+    if (rc) return rc;
+  } else if (ctx->h16) {
+    const int rc = split_gather(ctx);
     if (rc) return rc;
   }
   if (c.model == SFB_MLR && c.precision == SFB_PREC_FP32) {        // (bf16 mode: with the label rows)
@@ -674,20 +698,24 @@ static int sdca_compute_factors(sfb_ctx* ctx, int32_t worker, const float* X_dev
   if (worker < -1 || worker >= c.workers) return SFB_ERR_SHAPE;
   const int64_t off = worker < 0 ? 0 : static_cast<int64_t>(worker) * c.batch;
   const int64_t n = worker < 0 ? ctx->K : c.batch;
-  if (ctx->committed == 0) begin_phase(ctx, 0);
+  if (ctx->committed == 0) {
+    begin_phase(ctx, 0);
+    ctx->begun = false;
+  }
   const float inv_lam_n = static_cast<float>(1.0 / (static_cast<double>(c.sdca_lambda) * static_cast<double>(c.sdca_n)));
   if (ctx->tf32) {
     const int rc = tc32_factors(ctx, off, n, X_dev, labels_dev, sample_ids_dev, inv_lam_n);
     if (rc) return rc;
   } else if (c.precision == SFB_PREC_FP32) {
-    float* V = ctx->at<float>(ctx->lay.V) + off * c.cols;
     const int64_t ldu = ctx->lay.ldu;
     float* U = ctx->at<float>(ctx->lay.U) + off * ldu;
-    CK(pack_copy(ctx->stream, V, X_dev, nullptr, n * c.cols, take_stamp(ctx)));                                        // v = a_i
-    EpiArgs e{};
-    e.C = U; e.ldc = ldu;
-    CK(sgemm(ctx->stream, true, true, EPI_STORE, n, c.rows, c.cols, V, c.cols, ctx->W, c.cols, e, ctx->K));   // z_i = W a_i
-    ctx->stats.flops += 2.0 * n * c.rows * c.cols;
+    if (!ctx->begun) {
+      const int rc = begin_step(ctx);
+      if (rc) return rc;
+      ctx->begun = true;
+    }
+    const int rc = logits_fp32(ctx, off, n, X_dev, nullptr);                                          // z_i = W a_i
+    if (rc) return rc;
     SdcaArgs a = sdca_args(ctx, off, n, X_dev, labels_dev, sample_ids_dev, inv_lam_n);
     a.Z = U; a.ldz = ldu; a.out = U; a.ldo = ldu;                                                     // u_i = du_i
     CK(sdca_dual_rows(ctx->stream, a));
@@ -869,6 +897,7 @@ extern "C" int sfb_get_status(sfb_ctx* ctx, uint32_t* status_out) {
   CK(cudaMemcpyAsync(status_out, ctx->at<uint32_t>(ctx->lay.status), 4, cudaMemcpyDeviceToHost, ctx->stream));
   CK(cudaMemsetAsync(ctx->at<uint32_t>(ctx->lay.status), 0, 4, ctx->stream));
   CK(cudaStreamSynchronize(ctx->stream));
+  if ((*status_out & SFB_STATUS_TIMEOUT) && ctx->lay.ready) CK(split_reset(ctx));
   return SFB_OK;
 }
 

@@ -61,7 +61,7 @@ __device__ __forceinline__ float block_max(float v, float* sh) {
 __global__ void pack_kernel(float* __restrict__ dst, const float* __restrict__ x, const float* __restrict__ y,
                             int64_t n4, int64_t n, const Stamp st) {
   pdl_launch_dependents();
-  pdl_wait();
+  pdl_wait(x, y);
   stamp_begin(st);
   const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
   for (int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; i < n4; i += stride) {
@@ -93,7 +93,7 @@ __global__ void prox_entries_kernel(float* __restrict__ w, int64_t n, int kind, 
 
 __global__ void axpy_kernel(float* __restrict__ y, const float* __restrict__ x, float alpha, int64_t n) {
   pdl_launch_dependents();
-  pdl_wait();
+  pdl_wait(x);
   const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
   for (int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; i < n; i += stride)
     y[i] = fmaf(alpha, x[i], y[i]);
@@ -107,7 +107,7 @@ __global__ void __launch_bounds__(NTHREADS) mlr_softmax_kernel(float* __restrict
                                                                const int32_t* __restrict__ labels,
                                                                float* __restrict__ loss, uint32_t* status) {
   pdl_launch_dependents();
-  pdl_wait();
+  pdl_wait(labels);
   __shared__ float sh[32];
   float* z = Z + static_cast<int64_t>(blockIdx.x) * ldz;
   float m = -INFINITY;
@@ -141,7 +141,7 @@ __global__ void __launch_bounds__(NTHREADS) mlr_shard_partials_kernel(const floa
                                                                       const int32_t* __restrict__ labels, int64_t row_off,
                                                                       float4* __restrict__ part) {
   pdl_launch_dependents();
-  pdl_wait();
+  pdl_wait(Z, labels);
   __shared__ float sh[32];
   const float* z = Z + static_cast<int64_t>(blockIdx.x) * ldz;
   float m = -INFINITY;
@@ -183,7 +183,7 @@ __global__ void __launch_bounds__(NTHREADS) mlr_shard_finish_kernel(float* __res
                                                                     const float4* __restrict__ parts, int shards, int64_t K,
                                                                     float* __restrict__ loss, uint32_t* status) {
   pdl_launch_dependents();
-  pdl_wait();
+  pdl_wait(labels, parts);
   __shared__ float sh_lse;
   float* z = Z + static_cast<int64_t>(blockIdx.x) * ldz;
   if (threadIdx.x == 0) {
@@ -372,9 +372,10 @@ __global__ void __launch_bounds__(NTHREADS) dml_scale_kernel(float* __restrict__
                                                              float* __restrict__ norm_out,
                                                              const float* __restrict__ norms_all,
                                                              int shards, int64_t nstride, __nv_bfloat16* __restrict__ split,
-                                                             int64_t split_half) {
+                                                             int64_t split_half, const float* __restrict__ inv_v,
+                                                             float* __restrict__ most) {
   pdl_launch_dependents();
-  pdl_wait();
+  pdl_wait(similar, norms_all, inv_v);
   __shared__ float sh[32];
   float* z = Z + static_cast<int64_t>(blockIdx.x) * ld;
   float q = 0.f;
@@ -389,21 +390,27 @@ __global__ void __launch_bounds__(NTHREADS) dml_scale_kernel(float* __restrict__
     return;
   }
   const float c = similar[blockIdx.x] != 0 ? 2.f : (q < margin ? -2.f : 0.f);
+  float m = 0.f;
   __nv_bfloat16* hp = split ? split + static_cast<int64_t>(blockIdx.x) * 2 * split_half : nullptr;
   for (int64_t j = threadIdx.x; j < rows; j += NTHREADS) {
     const float u = c * z[j];
     z[j] = u;
+    m = fmaxf(m, fabsf(u));
     if (hp) {
       const __nv_bfloat16 hi = __float2bfloat16_rn(u);
       hp[j] = hi;
       hp[split_half + j] = __float2bfloat16_rn(u - __bfloat162float(hi));
     }
   }
+  if (most) {
+    m = block_max<NTHREADS>(m, sh);
+    if (threadIdx.x == 0) most[blockIdx.x] = m * inv_v[blockIdx.x];
+  }
 }
 
 __global__ void mean_kernel(const float* __restrict__ v, int64_t n, float* out, const Stamp st) {
   pdl_launch_dependents();
-  pdl_wait();
+  pdl_wait(v);
   stamp_begin(st);
   __shared__ float sh[32];
   float s = 0.f;
@@ -417,7 +424,7 @@ __global__ void mean_kernel(const float* __restrict__ v, int64_t n, float* out, 
 __global__ void __launch_bounds__(kThreads) col_sumsq_kernel(const float* __restrict__ W, int64_t rows, int64_t cols,
                                                              double* __restrict__ part, int64_t slab_rows) {
   pdl_launch_dependents();
-  pdl_wait();
+  pdl_wait(W);
   __shared__ double sh[8][128];
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
   const int64_t c0 = static_cast<int64_t>(blockIdx.x) * 128 + tx * 4;
@@ -451,7 +458,7 @@ __global__ void __launch_bounds__(kThreads) prox_scale_kernel(float* __restrict_
                                                               const double* __restrict__ part, int nslabs,
                                                               int64_t slab_rows, unsigned long long* end) {
   pdl_launch_dependents();
-  pdl_wait();
+  pdl_wait(part);
   __shared__ double scale[128];
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
   if (threadIdx.x < 128) {
@@ -746,12 +753,13 @@ cudaError_t sdca_dual_rows(cudaStream_t s, const SdcaArgs& a) {
 }
 
 cudaError_t dml_scale_rows(cudaStream_t s, float* Z, int64_t nsamp, int64_t rows, int64_t ld,
-                           const int32_t* similar, float margin, void* split, int64_t split_half, float* norm_out, const float* norms_all,
+                           const int32_t* similar, float margin, void* split, int64_t split_half, const float* inv_v,
+                           float* most, float* norm_out, const float* norms_all,
                            int shards, int64_t nstride) {
   if (nsamp <= 0) return cudaSuccess;
   return launch_kernel(dml_scale_kernel<256>, dim3(static_cast<unsigned>(nsamp)), dim3(256), 0, s, 1, Z, rows, ld,
                        similar, margin, norm_out, norms_all, shards, nstride, static_cast<__nv_bfloat16*>(split),
-                       split_half);
+                       split_half, inv_v, most);
 }
 
 cudaError_t mean_of(cudaStream_t s, const float* v, int64_t n, float* out, const Stamp& st) {

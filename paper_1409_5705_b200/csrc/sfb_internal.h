@@ -32,6 +32,15 @@ struct Stamp {                        // the first block stores the time to at[0
 };
 #ifdef __CUDACC__
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// ... with the kernel's `const __restrict__` parameters: the compiler may read through those at any time, before the wait too
+// (a scalar was), unless it cannot tell where they point until after it.
+template <typename T>
+__device__ __forceinline__ void pdl_hide(T& p) { asm volatile("" : "+l"(p) :: "memory"); }
+template <typename... P>
+__device__ __forceinline__ void pdl_wait(P&... p) {
+  pdl_wait();
+  (pdl_hide(p), ...);
+}
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 // Time stamps of the phases of a step (sfb_stats.ms_*), written by the kernels themselves: events between them would keep a
@@ -102,8 +111,10 @@ struct Layout {
   size_t status, scalars, loss, V, U, colpart, stageX, stageY, stageL;
   // bf16 tensor-core mode
   size_t Wb, Xb, VT, ZT, UT, P, part, Xf, labels, coef, lse, slot, dL;   // VT, UT: tf32 words only; P: probabilities [K x ldp]; slot, dL: label rows
-  // bf16 mode, DML and SC: (hi | lo) bf16 operands of the split products
+  // (hi | lo) operands of the split products
   size_t Ws, WTs, As, Rs;             // W by rows, W transposed, the A operand (v or the codes), the residual
+  size_t partial, ready;              // parts of the tiles of a split product
+  size_t iW, iA, iR, iC, q;           // fp32 mode: inverse scales of the rows of W, of the pairs; see sfb_split.cu
   // sparse factors (MLR, csr_nnz_max > 0): the step's (sample, column, value) triples and their column-major form
   size_t coo_i, coo_c, coo_x, coo_cx, row_beg, row_end, csc_cnt, csc_cur, csc_ptr, csc_tmp, csc_ent;
   // sparse coding: the dictionary's Gram matrix (when the coder iterates on it), W^T x, the codes of odd iterations, and
@@ -123,21 +134,22 @@ Layout make_layout(const sfb_config& c);
 bool sc_use_gram(const sfb_config& c);
 inline int64_t round_up(int64_t x, int64_t m) { return (x + m - 1) / m * m; }
 
-// fp32 mode runs its products of multiclass logistic regression on the tensor cores (every fp32 value as a pair of
-// tf32 words, three products per term) when asked to, or by itself when the shape is large enough to be worth the
-// operand copies; small shapes and the other models use the FFMA kernels.
+// Which kernels the products of an fp32 mode run on.  Pairs of tf32 words when asked for (logistic models).  SFB_PREC_FP32 runs
+// on pairs of fp16 words with fp32 scales (sfb_split.cu) where the products are large enough to repay the packing of their
+// operands, else on the FMA kernels: below about 10^8 multiply-adds a step is launches either way.
 inline bool use_tf32(const sfb_config& c) {
-  const bool mlr = c.model == SFB_MLR || c.model == SFB_L2MLR;
-  if (c.precision == SFB_PREC_TF32X3) return mlr;
-  if (c.precision != SFB_PREC_FP32 || !mlr) return false;
-  return c.rows >= 2048 && c.cols >= 512 && static_cast<int64_t>(c.workers) * c.batch >= 128;
+  return c.precision == SFB_PREC_TF32X3 && (c.model == SFB_MLR || c.model == SFB_L2MLR);
+}
+inline bool use_h16(const sfb_config& c) {
+  return c.precision == SFB_PREC_FP32 && c.rows >= 64 && c.cols >= 64 &&
+         static_cast<double>(c.workers) * c.batch * static_cast<double>(c.rows) * static_cast<double>(c.cols) >= 1e8;
 }
 
 struct Scalars {                      // device-resident scalars
   float loss_mean;
   float L;                            // ||W||_2^2 used by the coder
   float invL;
-  float tmp;
+  float iWT, iWT2, iG, iU;            // inverse scales: W^T and its square, W^T W, u (see sfb_split.cu)
   unsigned long long copy_pieces;     // 64-byte row pieces of the bf16 operand copy the update passes went over ...
   unsigned long long copy_written;    // ... and how many of them they had to rewrite (the others already held bf16(W))
   unsigned long long ns[4];           // global time at the start of the step, of its gather and of its update, and at its end
@@ -156,7 +168,7 @@ struct sfb_ctx {
   int64_t row_offset;                 // row-sharded MLR: this context's W holds rows [row_offset, row_offset + rows)
   int64_t global_rows;                //   of a matrix with global_rows rows (class ids are global); 0, rows when unsharded
   bool partials_ready;                // sfb_forward_partials has run since the last update
-  bool tf32;                          // fp32 mode with its products on the tensor cores (see use_tf32)
+  bool tf32, h16;                     // fp32 modes with their products on the tensor cores (see use_tf32, use_h16)
   bool sdca;                          // SFB_L2MLR: the factors are dual changes; cfg.model is kept as SFB_MLR internally
   float* dualQ;                       // SDCA dual state [dual_n x rows], caller-owned
   int64_t dual_n;
@@ -277,9 +289,11 @@ SdcaArgs sdca_args(const sfb_ctx* ctx, int64_t off, int64_t n, const float* X, c
                    float inv_lam_n);               // all but the logits and where du goes
 // Row-sharded form: norm_out (may be null) receives the shard's ||z_i||^2 and z is left unscaled; norms_all (may be null),
 // [shards][nstride], supplies ||z_i||^2 as the sum over the shards instead of this context's own.
-// split (may be null): the scaled rows also as (hi | lo) bf16 pairs, row pitch 2 * split_half.
+// split (may be null): the scaled rows also as (hi | lo) bf16 pairs, row pitch 2 * split_half.  most (may be null): receives
+// inv_v[i] * max_j |u_ij|.
 cudaError_t dml_scale_rows(cudaStream_t s, float* Z, int64_t nsamp, int64_t rows, int64_t ld,
-                           const int32_t* similar, float margin, void* split, int64_t split_half, float* norm_out = nullptr,
+                           const int32_t* similar, float margin, void* split = nullptr, int64_t split_half = 0,
+                           const float* inv_v = nullptr, float* most = nullptr, float* norm_out = nullptr,
                            const float* norms_all = nullptr, int shards = 0, int64_t nstride = 0);
 cudaError_t mean_of(cudaStream_t s, const float* v, int64_t n, float* out, const Stamp& st);
 cudaError_t prox_unit_columns(cudaStream_t s, float* W, int64_t rows, int64_t cols, float* colpart, unsigned long long* end);

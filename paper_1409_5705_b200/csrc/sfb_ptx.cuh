@@ -72,6 +72,24 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volati
   return false;
 }
 
+// A flag that another CTA of the grid sets (with st_release) to hand over data; bounded like mbar_wait.
+__device__ __forceinline__ void st_release(uint32_t* flag, uint32_t v) {
+  asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(flag), "r"(v) : "memory");
+}
+__device__ __forceinline__ bool flag_wait(const uint32_t* flag, volatile uint32_t* abort) {
+  const long long t0 = clock64();
+  for (uint32_t i = 0; i < kMaxPolls; ++i) {
+    uint32_t v;
+    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(flag) : "memory");
+    if (v) return true;
+    if (*abort) return false;
+    if (clock64() - t0 > kMaxWaitCycles) break;
+    __nanosleep(64);
+  }
+  *abort = 1;
+  return false;
+}
+
 // ---- fences ---------------------------------------------------------------------------------------------
 __device__ __forceinline__ void fence_proxy_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
@@ -177,6 +195,11 @@ __device__ __forceinline__ uint32_t umma_idesc_bf16(uint32_t M, uint32_t N) {
   return d;
 }
 
+// The same with fp16 A and B.
+__device__ __forceinline__ uint32_t umma_idesc_fp16(uint32_t M, uint32_t N) {
+  return umma_idesc_bf16(M, N) & ~((1u << 7) | (1u << 10));       // A, B format 0: f16
+}
+
 // Instruction descriptor of kind::tf32: A and B are 32-bit words read as tf32 (both K-major), fp32 accumulator.
 __device__ __forceinline__ uint32_t umma_idesc_tf32(uint32_t M, uint32_t N) {
   uint32_t d = 0;
@@ -252,6 +275,13 @@ __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 
 // 16 bytes from the shared memory of CTA `rank` of this cluster, at this CTA's address `own_addr`.
+__device__ __forceinline__ float4 ld_shared_f4(uint32_t addr) {
+  float4 v;
+  asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr) : "memory");
+  return v;
+}
+__device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
+
 __device__ __forceinline__ float4 ld_cluster_f4(uint32_t own_addr, uint32_t rank) {
   float4 v;
   asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"

@@ -70,7 +70,7 @@ __global__ void __launch_bounds__(256) csr_stage_kernel(const int64_t* __restric
                                                         int32_t* __restrict__ row_beg,
                                                         int32_t* __restrict__ row_end, uint32_t* __restrict__ status) {
   pdl_launch_dependents();
-  pdl_wait();
+  pdl_wait(indptr, idx, val);
   const int64_t i = (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (i >= n) return;
@@ -111,7 +111,7 @@ __global__ void __launch_bounds__(256) csr_stage_kernel(const int64_t* __restric
 // ---------------------------------------------------------------------------------------------------------
 __global__ void __launch_bounds__(256) csc_count_kernel(const int32_t* __restrict__ coo_c, int64_t nnz, int32_t* __restrict__ cnt) {
   pdl_launch_dependents();
-  pdl_wait();
+  pdl_wait(coo_c);
   const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
   for (int64_t t = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; t < nnz; t += stride) {
     const int32_t c = coo_c[t];
@@ -121,7 +121,7 @@ __global__ void __launch_bounds__(256) csc_count_kernel(const int32_t* __restric
 
 __global__ void __launch_bounds__(1024) csc_scan_kernel(const int32_t* __restrict__ cnt, int64_t cols, int32_t* __restrict__ ptr) {
   pdl_launch_dependents();
-  pdl_wait();
+  pdl_wait(cnt);
   __shared__ int32_t part[1024];
   const int t = threadIdx.x;
   const int64_t chunk = (cols + 1023) / 1024;
@@ -149,7 +149,7 @@ __global__ void __launch_bounds__(256) csc_fill_kernel(const int32_t* __restrict
                                                        const int32_t* __restrict__ ptr, int32_t* __restrict__ cur,
                                                        int2* __restrict__ tmp) {
   pdl_launch_dependents();
-  pdl_wait();
+  pdl_wait(coo_i, coo_c, coo_x, ptr);
   const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
   for (int64_t t = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; t < nnz; t += stride) {
     const int32_t c = coo_c[t];
@@ -164,7 +164,7 @@ __global__ void __launch_bounds__(128) csc_sort_kernel(const int2* __restrict__ 
                                                        const int32_t* __restrict__ cnt, int64_t cols, int32_t K,
                                                        int2* __restrict__ ent) {
   pdl_launch_dependents();
-  pdl_wait();
+  pdl_wait(tmp, ptr, cnt);
   for (int64_t d = blockIdx.x; d < cols; d += gridDim.x) {
     const int32_t n = cnt[d], b = ptr[d];
     for (int32_t e = threadIdx.x; e < n; e += blockDim.x) {
@@ -224,7 +224,7 @@ __global__ void __launch_bounds__(kSfThreads, 1) sparse_forward_kernel(const flo
                                                                        const int2* __restrict__ cx, int64_t off, int32_t n,
                                                                        float* __restrict__ Z, int64_t ldz) {
   pdl_launch_dependents();
-  pdl_wait();
+  pdl_wait(W, row_beg, row_end, cx);
   extern __shared__ __align__(16) uint8_t sf_smem[];
   constexpr int EP = 32 / RB;                        // entries of a sample worked on at once
   float* ws = reinterpret_cast<float*>(sf_smem);     // RB rows of W, row pitch `pitch` floats
@@ -556,11 +556,11 @@ bool sparse_update_wanted(const sfb_ctx* ctx) {
   const sfb_config& c = ctx->cfg;
   const bool bf16 = c.precision == SFB_PREC_BF16;
   if (c.csr_update == 2 || slab_smem(ctx->K, bf16) < 0) return false;
-  if (c.csr_update == 1 || (!bf16 && !ctx->tf32)) return true;
+  if (c.csr_update == 1 || (!bf16 && !ctx->tf32 && !ctx->h16)) return true;
   const double per_col = static_cast<double>(ctx->csr_fill) / static_cast<double>(c.cols);
   const double k = static_cast<double>(ctx->K) / 1024.0;
-  const double sparse = (bf16 ? 1.0 : 1.57) + 0.089 * per_col;
-  return sparse < (bf16 ? 1.0 : 4.4) * k;
+  const double sparse = (ctx->tf32 ? 1.57 : 1.0) + 0.089 * per_col;
+  return sparse < (bf16 ? 1.0 : ctx->tf32 ? 4.4 : 2.2) * k;
 }
 
 int sparse_stage(sfb_ctx* ctx, int64_t off, int64_t n, const int64_t* indptr, const int32_t* idx, const float* val,

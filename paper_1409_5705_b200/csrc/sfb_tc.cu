@@ -1,6 +1,6 @@
 // Tensor-core (bf16 operand) path of the SFB step on sm_100a: sufficient-factor computation for multiclass
 // logistic regression (Sections 1 and 2: u = softmax(W x) - onehot(y), v = x) and the operand packing of the
-// update product.  The update product itself is in sfb_update.cu.
+// update product.  The update product itself is in sfb_update.cu, the products of (hi | lo) pairs in sfb_split.cu.
 //
 // Forward product: one persistent, warp-specialised kernel computes  Z (K x rows) = X (K x cols) * W^T  with bf16
 // operands staged by TMA into 128-byte-swizzled shared memory, tcgen05.mma accumulating in TMEM (two 128 x 256
@@ -16,10 +16,7 @@
 
 #include "sfb_ptx.cuh"
 #include "sfb_tc.h"
-
-#ifndef SFB_SPLIT_PREFETCH
-#define SFB_SPLIT_PREFETCH 4
-#endif
+#include "sfb_tile.cuh"
 
 namespace sfb {
 namespace {
@@ -40,29 +37,18 @@ constexpr int kBars = 2 * S_MAX + 4;
 constexpr int kSmem = S * (kBytesA + kBytesB) + kEpiWarps * R * kSlotBytes + kBars * 8 + 16 + 1024;
 
 // Epilogues of the product  D (samples x N) = A * B^T:
-//   F_SOFTMAX  store D as fp32 logits and the softmax partials per (sample, pw columns)            (MLR; forward_kernel)
-// and, in forward_split_kernel:
-//   F_STORE    store D as fp32                                                                     (DML: z = W v)
-//   F_SUB      store D - aux as fp32 and as a (hi | lo) bf16 pair                                  (SC: r = W a - x)
-//   F_ISTA     C <- soft(C - D / L, lambda / L) in place, also as a (hi | lo) bf16 pair            (SC: ISTA step)
-//   F_ISTAG    C <- soft(C - (D - C2) / L, lambda / L) in place, also as a pair                     (SC: on W^T W)
-//   F_ISTA0    C2 = D and C = soft(D / L, lambda / L), also as a pair                               (SC: first iterate)
-//   F_GRAM     C (unless null) = D and D as a pair, of a symmetric D: only the tiles that reach the diagonal or lie above
-//              it are formed, the others are written as their mirror images                          (SC: W^T W)
-enum FwdEpi { F_SOFTMAX = 0, F_STORE = 1, F_SUB = 2, F_ISTA = 3, F_ISTAG = 4, F_ISTA0 = 5, F_GRAM = 6 };
-template <int EPI>
-constexpr bool kIsta = EPI == F_ISTA || EPI == F_ISTAG || EPI == F_ISTA0;
+//   F_SOFTMAX  store D as fp32 logits and the softmax partials per (sample, pw columns)
+enum FwdEpi { F_SOFTMAX = 0 };
 
 struct TcParams {
   int32_t M, N, Kc;            // extents of the product: samples, output columns, contraction
   int32_t m_off;               // first sample handled by this launch (per-worker slices)
   int32_t tilesM, tilesN;
-  int32_t a_rows;              // forward_kernel: rows of A per box (fewer than 128 for a slice of few samples; the rest of a
+  int32_t a_rows;              // rows of A per box (fewer than 128 for a slice of few samples; the rest of a
                                // tile's samples are then never stored)
   int32_t stages;              // forward_kernel: stages of the operand ring
   int32_t pw;                  // F_SOFTMAX: columns per softmax partial, a divisor of bn
-  int32_t bn;                  // columns per tile, at most BN (chosen so that the tiles fill the SMs): a multiple of 32
-                               // in forward_kernel, of 16 in forward_split_kernel
+  int32_t bn;                  // columns per tile, at most BN, a multiple of 32 (chosen so that the tiles fill the SMs)
   // The contraction runs over nseg segments of kseg k-blocks; segment s reads A from column a_off<s> and B from
   // column b_off<s> of their tensors: one segment is the plain product, three segments over [hi | lo] operand
   // halves form the split-bf16 product hi*hi + hi*lo + lo*hi.  (Scalars: an indexed array would send the whole
@@ -71,17 +57,8 @@ struct TcParams {
   int32_t a_off0, a_off1, a_off2, b_off0, b_off1, b_off2;
   float2* part;                // F_SOFTMAX: [N / pw][part_ld] (max, sum exp) per sample and pw rows of W
   int64_t part_ld;
-  const float* aux;            // F_SUB: the matrix subtracted, [M x ldaux]; F_ISTA, F_ISTAG: the matrix updated
-  int64_t ldaux;
-  float* C2;                   // F_ISTA0 (may be null), F_ISTAG: W^T x, [M x ldc]
   int32_t prefetch;            // k-blocks by which the producer asks L2 for the B operand ahead of its loads (0: off)
   int32_t kparts;              // the contraction of a tile is cut over a cluster of this many CTAs (1: persistent CTAs)
-  int32_t four;                // F_GRAM: with the fourth term A_lo B_lo
-  const Scalars* sc;           // F_ISTA*: 1 / L
-  float lam;                   // F_ISTA*: lambda
-  __nv_bfloat16* split;        // all but F_STORE: [M x ld_split] receives hi at column n and lo at column split_half + n
-  int64_t ld_split;
-  int32_t split_half;          // padded N (a multiple of 64); columns N..split_half-1 are written as zeros
   uint32_t* status;
 };
 
@@ -91,59 +68,6 @@ __device__ __forceinline__ void tile_coords(const TcParams& p, int tile, int& m0
   const int tm = tile % p.tilesM, tn = tile / p.tilesM;
   m0 = p.m_off + tm * BM;
   n0 = tn * p.bn;
-}
-
-// F_GRAM: the tiles of column block tn that are formed are row blocks 0 .. sym_row_blocks - 1 (those that begin above the
-// column block's end); numbered column block by column block.
-__host__ __device__ __forceinline__ int sym_row_blocks(int tilesM, int bn, int tn) {
-  const int n = ((tn + 1) * bn - 1) / BM + 1;
-  return n < tilesM ? n : tilesM;
-}
-__host__ __device__ __forceinline__ int sym_tiles(int tilesM, int tilesN, int bn) {
-  int n = 0;
-  for (int tn = 0; tn < tilesN; ++tn) n += sym_row_blocks(tilesM, bn, tn);
-  return n;
-}
-template <int EPI>
-__device__ __forceinline__ void split_tile_coords(const TcParams& p, int tile, int& m0, int& n0) {
-  if (EPI != F_GRAM) return tile_coords(p, tile, m0, n0);
-  int tn = 0;
-  for (int n; tile >= (n = sym_row_blocks(p.tilesM, p.bn, tn)); ++tn) tile -= n;
-  m0 = tile * BM;
-  n0 = tn * p.bn;
-}
-
-// Exchange of the partial tiles of a split contraction through the shared memory of the cluster's CTAs, in chunks of 32
-// columns x 128 rows of fp32 (16 KB, the operand stages' memory, which nothing uses any more); a warp writes and reads its 32
-// rows with the 16-byte pieces of a row swizzled.  Rank r then finishes the chunks c = r, r + split, ...; the sums are in rank
-// order, so they do not depend on timing.
-constexpr int kXchgBytes = BM * kChunk * 4;
-__device__ __forceinline__ uint32_t xchg_addr(uint8_t* smem, int c, int row, int j) {
-  return smem_u32(smem) + c * kXchgBytes + row * (kChunk * 4) + ((j ^ (row & 7)) << 4);
-}
-__device__ __forceinline__ void xchg_put(uint8_t* smem, int c, int row, const uint32_t (&acc)[32]) {
-#pragma unroll
-  for (int j = 0; j < 8; ++j)
-    asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(xchg_addr(smem, c, row, j)), "r"(acc[4 * j]), "r"(acc[4 * j + 1]),
-                 "r"(acc[4 * j + 2]), "r"(acc[4 * j + 3]) : "memory");
-}
-__device__ __forceinline__ void xchg_sum(uint8_t* smem, int c, int row, int split, uint32_t (&acc)[32]) {
-#pragma unroll
-  for (int j = 0; j < 8; ++j) {
-    const uint32_t at = xchg_addr(smem, c, row, j);
-    float4 s = ld_cluster_f4(at, 0);
-    for (int g = 1; g < split; ++g) {
-      const float4 v = ld_cluster_f4(at, g);
-      s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w;
-    }
-    acc[4 * j] = __float_as_uint(s.x); acc[4 * j + 1] = __float_as_uint(s.y);
-    acc[4 * j + 2] = __float_as_uint(s.z); acc[4 * j + 3] = __float_as_uint(s.w);
-  }
-}
-
-__device__ __forceinline__ float soft_threshold(float w, float t) {
-  const float a = fabsf(w) - t;
-  return a > 0.f ? copysignf(a, w) : 0.f;
 }
 
 // TF32: the operands are 32-bit words read as tf32 (a k-block of 128 bytes is then 32 elements and one MMA contracts
@@ -318,7 +242,7 @@ forward_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       tile_coords(p, tile0, m0, n0);
       for (int c = part; c < p.bn / kChunk && ok; c += split) {        // (pw is 32: a group is a chunk)
         uint32_t acc[32];
-        xchg_sum(smem, c, q * 32 + lane, split, acc);
+        xchg_sum(smem, c, q * 32 + lane, split, 0, 1, acc);
         finish(acc, m0, n0, c);
       }
     }
@@ -345,294 +269,6 @@ forward_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
 }
 
 // ---------------------------------------------------------------------------------------------------------
-// Split-bf16 products of distance metric learning and sparse coding:  D (samples x N) = A * B^T  with both operands
-// stored as [hi | lo] bf16 halves,  A_hi B_hi + A_lo B_hi + A_hi B_lo  (fp32-class accuracy; A_lo B_lo, 2^-16 of the
-// product, is dropped).  One pipeline stage holds the k-block of all four halves, and the three products of that
-// k-block are issued from it: 72 KB of operands per three k-blocks of tensor work instead of 108 KB when the three
-// products run as separate passes over the contraction (these products are bound by their operand loads: a 128 x 160
-// tile takes 36 KB per 320 cycles of MMA).  Three stages of 72 KB fill the shared memory, so the epilogue writes its
-// results straight from registers (the outputs are small: samples x N).  The cross terms have an accumulator of their own: the
-// tensor core rounds an fp32 accumulator at every instruction relative to what it holds, so two thirds of the roundings happen
-// at a 2^-8 of the size.
-// Roles as in forward_kernel: warp 0 TMA producer, warp 1 MMA issuer and TMEM owner, warps 2-5 epilogue.
-// ---------------------------------------------------------------------------------------------------------
-constexpr int FS_BN = 160;                          // widest tile of this kernel (columns of the accumulator)
-constexpr int FS_STAGES = 3;
-constexpr int kFsBytesB = FS_BN * BK * 2;           // 20 KB
-constexpr int kFsStage = 2 * kBytesA + 2 * kFsBytesB;
-constexpr int kFsBars = 2 * FS_STAGES + 4;
-constexpr int kFsEpi = 8;                           // epilogue warps: two per TMEM lane quarter, taking turns at the chunks
-constexpr int kFsThreads = 64 + 32 * kFsEpi;
-constexpr int kFsSmem = FS_STAGES * kFsStage + kFsBars * 8 + 16 + 1024;
-
-template <int EPI>
-__global__ void __launch_bounds__(kFsThreads, 1)
-forward_split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, float* __restrict__ C,
-                     int64_t ldc, const TcParams p) {
-  extern __shared__ uint8_t smem_raw[];
-  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + FS_STAGES * kFsStage);
-  uint64_t* full = bars;
-  uint64_t* empty = bars + FS_STAGES;
-  uint64_t* tfull = bars + 2 * FS_STAGES;
-  uint64_t* tempty = bars + 2 * FS_STAGES + 2;
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + kFsBars);
-  volatile uint32_t* abort_flag = tmem_slot + 1;
-
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int ntiles = EPI == F_GRAM ? sym_tiles(p.tilesM, p.tilesN, p.bn) : p.tilesM * p.tilesN;
-  // the tiles and k-blocks (each serves three products) of this CTA, as in forward_kernel
-  const int split = p.kparts, part = split > 1 ? static_cast<int>(blockIdx.x) % split : 0;
-  const int tile0 = static_cast<int>(blockIdx.x) / split, tile_step = split > 1 ? ntiles : static_cast<int>(gridDim.x);
-  const int kbeg = part * p.kseg / split, kend = (part + 1) * p.kseg / split;
-  // Two accumulators per tile: A_hi B_hi, and the cross terms at column `cross` of it.  Tiles of at most 128 columns have room
-  // for two such pairs (the epilogue of one tile then overlaps the products of the next), wider ones for one.
-  const int nacc = p.bn <= 128 ? 2 : 1, cross = p.bn <= 128 ? 128 : 256;
-  const int a_hi = p.a_off0, a_lo = p.a_off2, b_hi = p.b_off0, b_lo = p.b_off1;
-
-  pdl_launch_dependents();
-  if (threadIdx.x == 0) {
-    for (int i = 0; i < FS_STAGES; ++i) { mbar_init(&full[i], 1); mbar_init(&empty[i], 1); }
-    for (int i = 0; i < 2; ++i) { mbar_init(&tfull[i], 1); mbar_init(&tempty[i], kFsEpi); }
-    *abort_flag = 0;
-    fence_barrier_init();
-    prefetch_tmap(&tmA); prefetch_tmap(&tmB);
-  }
-  if (warp == 1) { tmem_alloc(tmem_slot, kTmemCols); tmem_relinquish(); }
-  tc_fence_before();
-  __syncthreads();
-  tc_fence_after();
-  const uint32_t tmem_base = *tmem_slot;
-  pdl_wait();
-
-  if (warp == 0) {
-    // ---------------- TMA producer: the four operand halves of a k-block per stage ----------------
-    if (lane == 0) {
-      const uint64_t pol_keep = policy_evict_last();
-      const uint32_t stage_bytes = 2 * kBytesA + 2 * static_cast<uint32_t>(p.bn) * BK * 2;
-      uint32_t it = 0;
-      bool ok = true;
-      for (int tile = tile0; tile < ntiles && ok; tile += tile_step) {
-        int m0, n0;
-        split_tile_coords<EPI>(p, tile, m0, n0);
-        for (int kl = kbeg; kl < kend; ++kl, ++it) {
-          const uint32_t s = it % FS_STAGES, ph = (it / FS_STAGES) & 1;
-          if (!mbar_wait(&empty[s], ph ^ 1, abort_flag)) { ok = false; break; }
-          if (p.prefetch > 0 && kl + p.prefetch < kend) {          // B streams from HBM when it is larger than L2
-            tma_prefetch_2d(&tmB, b_hi + (kl + p.prefetch) * BK, n0);
-            tma_prefetch_2d(&tmB, b_lo + (kl + p.prefetch) * BK, n0);
-          }
-          uint8_t* st = smem + s * kFsStage;
-          mbar_expect_tx(&full[s], stage_bytes);
-          tma_load_2d_hint(st, &tmA, a_hi + kl * BK, m0, &full[s], pol_keep);
-          tma_load_2d_hint(st + kBytesA, &tmA, a_lo + kl * BK, m0, &full[s], pol_keep);
-          tma_load_2d(st + 2 * kBytesA, &tmB, b_hi + kl * BK, n0, &full[s]);
-          tma_load_2d(st + 2 * kBytesA + kFsBytesB, &tmB, b_lo + kl * BK, n0, &full[s]);
-        }
-      }
-    }
-  } else if (warp == 1) {
-    // ---------------- MMA issuer: three products per stage ----------------
-    if (lane == 0) {
-      const uint32_t idesc = umma_idesc_bf16(BM, p.bn);
-      uint32_t it = 0, tl = 0;
-      bool ok = true;
-      for (int tile = tile0; tile < ntiles && ok; tile += tile_step, ++tl) {
-        const uint32_t a = tl % nacc, aph = (tl / nacc) & 1;
-        if (!mbar_wait(&tempty[a], aph ^ 1, abort_flag)) { ok = false; break; }
-        tc_fence_after();
-        const uint32_t d_tmem = tmem_base + a * BN, d_cross = d_tmem + cross;
-        for (int kb = 0; kb < kend - kbeg; ++kb, ++it) {
-          const uint32_t s = it % FS_STAGES, ph = (it / FS_STAGES) & 1;
-          if (!mbar_wait(&full[s], ph, abort_flag)) { ok = false; break; }
-          tc_fence_after();
-          uint8_t* st = smem + s * kFsStage;
-          const uint64_t dah = umma_desc_k128(smem_u32(st));
-          const uint64_t dal = umma_desc_k128(smem_u32(st + kBytesA));
-          const uint64_t dbh = umma_desc_k128(smem_u32(st + 2 * kBytesA));
-          const uint64_t dbl = umma_desc_k128(smem_u32(st + 2 * kBytesA + kFsBytesB));
-#pragma unroll
-          for (int k = 0; k < BK / UMMA_K; ++k) {
-            const uint64_t adv = static_cast<uint64_t>(k * UMMA_K * 2 / 16);
-            const uint32_t more = (kb | k) != 0 ? 1u : 0u;
-            umma_bf16(d_cross, dal + adv, dbh + adv, idesc, more);                       // A_lo B_hi
-            umma_bf16(d_cross, dah + adv, dbl + adv, idesc, 1u);                         // A_hi B_lo
-            if (EPI == F_GRAM && p.four) umma_bf16(d_cross, dal + adv, dbl + adv, idesc, 1u);    // A_lo B_lo
-            umma_bf16(d_tmem, dah + adv, dbh + adv, idesc, more);                        // A_hi B_hi
-          }
-          umma_commit(&empty[s]);
-        }
-        if (ok) umma_commit(&tfull[a]);
-      }
-    }
-  } else {
-    // ---------------- epilogue: warp (q, h) = TMEM lane quarter q, every second chunk; results leave straight from registers
-    const int q = warp & 3, h = (warp - 2) >> 2;
-    const int my_tiles = tile0 < ntiles ? (ntiles - 1 - tile0) / tile_step + 1 : 0;
-    bool ok = true;
-    float invL = 0.f, thr = 0.f;
-    if (kIsta<EPI>) { invL = p.sc->invL; thr = p.lam * invL; }
-    auto finish = [&](uint32_t (&acc)[32], int m0, int n0, int c) {
-      const int row = m0 + q * 32 + lane;
-      // the tile's columns end at nlim; its width is a multiple of 16, so the last 32-column chunk may be half used
-      const int nlim = min(p.N, n0 + p.bn);
-      const int col0 = n0 + c * kChunk;
-      if (col0 >= nlim || row >= p.M) return;
-      if constexpr (EPI == F_ISTAG || EPI == F_ISTA0) {
-        // W^T x of the sample (N, hence every pitch, is a multiple of 4 for the products over atoms)
-        float* bp = p.C2 ? p.C2 + static_cast<int64_t>(row) * ldc + col0 : nullptr;
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-          if (!bp || col0 + 4 * j + 4 > nlim) continue;
-          if constexpr (EPI == F_ISTAG) {
-            const float4 b4 = *reinterpret_cast<const float4*>(bp + 4 * j);
-            acc[4 * j] = __float_as_uint(__uint_as_float(acc[4 * j]) - b4.x);
-            acc[4 * j + 1] = __float_as_uint(__uint_as_float(acc[4 * j + 1]) - b4.y);
-            acc[4 * j + 2] = __float_as_uint(__uint_as_float(acc[4 * j + 2]) - b4.z);
-            acc[4 * j + 3] = __float_as_uint(__uint_as_float(acc[4 * j + 3]) - b4.w);
-          } else {
-            *reinterpret_cast<uint4*>(bp + 4 * j) = make_uint4(acc[4 * j], acc[4 * j + 1], acc[4 * j + 2], acc[4 * j + 3]);
-          }
-        }
-      }
-      if constexpr (EPI != F_STORE) {
-        if constexpr (EPI == F_SUB || EPI == F_ISTA || EPI == F_ISTAG) {
-          // the sample's values of aux (x, or the current code a) are contiguous: up to 128 bytes per lane
-          float xv[32];
-          const float* ap = p.aux + static_cast<int64_t>(row) * p.ldaux + col0;
-          const bool ap16 = (reinterpret_cast<uintptr_t>(ap) & 15u) == 0;
-#pragma unroll
-          for (int j = 0; j < 8; ++j) {
-            if (ap16 && col0 + 4 * j + 4 <= nlim) {
-              const float4 v4 = *reinterpret_cast<const float4*>(ap + 4 * j);
-              xv[4 * j] = v4.x; xv[4 * j + 1] = v4.y; xv[4 * j + 2] = v4.z; xv[4 * j + 3] = v4.w;
-            } else {
-#pragma unroll
-              for (int e = 0; e < 4; ++e) xv[4 * j + e] = col0 + 4 * j + e < nlim ? ap[4 * j + e] : 0.f;
-            }
-          }
-#pragma unroll
-          for (int j = 0; j < 32; ++j) {
-            const float d = __uint_as_float(acc[j]);
-            acc[j] = __float_as_uint(EPI == F_SUB ? d - xv[j] : soft_threshold(fmaf(-d, invL, xv[j]), thr));
-          }
-        }
-        if constexpr (EPI == F_ISTA0) {
-#pragma unroll
-          for (int j = 0; j < 32; ++j) acc[j] = __float_as_uint(soft_threshold(__uint_as_float(acc[j]) * invL, thr));
-        }
-#pragma unroll
-        for (int j = 0; j < 32; ++j) acc[j] = col0 + j < p.N ? acc[j] : 0u;
-        // (hi | lo) bf16 pair of the result: the operand of the next product (zero in the padding past N; the
-        // columns past this tile's width belong to the next tile)
-        __nv_bfloat16* hp = p.split + static_cast<int64_t>(row) * p.ld_split + col0;
-        const int split_lim = min(p.split_half, n0 + p.bn);
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          if (col0 + 8 * j < split_lim) {
-            uint32_t hi[4], lo[4];
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-              const float f0 = __uint_as_float(acc[8 * j + 2 * e]), f1 = __uint_as_float(acc[8 * j + 2 * e + 1]);
-              const __nv_bfloat16 h0 = __float2bfloat16_rn(f0), h1 = __float2bfloat16_rn(f1);
-              hi[e] = static_cast<uint32_t>(__bfloat16_as_ushort(h0)) |
-                      (static_cast<uint32_t>(__bfloat16_as_ushort(h1)) << 16);
-              const __nv_bfloat162 l2 = __floats2bfloat162_rn(f0 - __bfloat162float(h0), f1 - __bfloat162float(h1));
-              lo[e] = *reinterpret_cast<const uint32_t*>(&l2);
-            }
-            *reinterpret_cast<uint4*>(hp + 8 * j) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
-            *reinterpret_cast<uint4*>(hp + p.split_half + 8 * j) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
-          }
-        }
-      }
-      if constexpr (EPI == F_GRAM) {
-        // the mirror images of the entries whose own tile is not formed: lanes are neighbouring columns there
-        const int own_end = (row / p.bn + 1) * p.bn;              // end of the column block that row lies in
-#pragma unroll
-        for (int j = 0; j < 32; ++j) {
-          const int n = col0 + j;
-          if (n >= nlim || own_end > n / BM * BM) continue;
-          const float f = __uint_as_float(acc[j]);
-          const __nv_bfloat16 hi = __float2bfloat16_rn(f);
-          __nv_bfloat16* hp = p.split + static_cast<int64_t>(n) * p.ld_split + row;
-          hp[0] = hi;
-          hp[p.split_half] = __float2bfloat16_rn(f - __bfloat162float(hi));
-          if (C) C[static_cast<int64_t>(n) * ldc + row] = f;
-        }
-        if (!C) return;
-      }
-      // the fp32 result: this lane's consecutive columns of its row
-      float* cp = C + static_cast<int64_t>(row) * ldc + col0;
-      const bool cp16 = (reinterpret_cast<uintptr_t>(cp) & 15u) == 0;
-#pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        if (cp16 && col0 + 4 * j + 4 <= nlim) {
-          *reinterpret_cast<uint4*>(cp + 4 * j) = make_uint4(acc[4 * j], acc[4 * j + 1], acc[4 * j + 2], acc[4 * j + 3]);
-        } else {
-#pragma unroll
-          for (int e = 0; e < 4; ++e)
-            if (col0 + 4 * j + e < nlim) cp[4 * j + e] = __uint_as_float(acc[4 * j + e]);
-        }
-      }
-    };
-    const int chunks = (p.bn + kChunk - 1) / kChunk;
-    for (int tl = 0; tl < my_tiles && ok; ++tl) {
-      int m0, n0;
-      split_tile_coords<EPI>(p, tile0 + tl * tile_step, m0, n0);
-      const uint32_t a = tl % nacc, aph = (tl / nacc) & 1;
-      if (!__all_sync(0xffffffffu, mbar_wait(&tfull[a], aph, abort_flag))) { ok = false; break; }
-      tc_fence_after();
-      for (int c = h; c < chunks; c += 2) {
-        uint32_t acc[32];
-        {
-          uint32_t small[32];
-          const uint32_t at = tmem_base + (static_cast<uint32_t>(q * 32) << 16) + a * BN + c * kChunk;
-          tmem_ld_32x32(at, acc);
-          tmem_ld_32x32(at + cross, small);
-          tmem_ld_wait();
-#pragma unroll
-          for (int j = 0; j < 32; ++j) acc[j] = __float_as_uint(__uint_as_float(acc[j]) + __uint_as_float(small[j]));
-        }
-        if (split > 1) xchg_put(smem, c, q * 32 + lane, acc);
-        else finish(acc, m0, n0, c);
-      }
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(&tempty[a]);
-    }
-    if (split > 1) {
-      __syncwarp();
-      cluster_arrive();
-      cluster_wait();
-      int m0, n0;
-      split_tile_coords<EPI>(p, tile0, m0, n0);
-      for (int c = part + split * h; c < chunks && ok; c += 2 * split) {
-        uint32_t acc[32];
-        xchg_sum(smem, c, q * 32 + lane, split, acc);
-        finish(acc, m0, n0, c);
-      }
-    }
-  }
-  if (split > 1) {
-    __syncwarp();
-    if (warp < 2) { cluster_arrive(); cluster_wait(); }                // (the epilogue warps have been there)
-    cluster_arrive();                                                  // no CTA leaves while a peer still reads its part
-    cluster_wait();
-  }
-
-  // ---------------- teardown ----------------
-  __syncwarp();
-  tc_fence_before();
-  __syncthreads();
-  if (*abort_flag) {
-    if (threadIdx.x == 0) atomicOr(p.status, SFB_STATUS_TIMEOUT);
-    for (int i = 0; i < 64; ++i) __nanosleep(1000);
-    __syncthreads();
-  }
-  if (warp == 1) { tc_fence_after(); tmem_dealloc(tmem_base, kTmemCols); }
-}
-
-// ---------------------------------------------------------------------------------------------------------
 // Bandwidth-bound companions of the tensor-core products
 // ---------------------------------------------------------------------------------------------------------
 __device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
@@ -644,7 +280,7 @@ __device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
 __global__ void __launch_bounds__(256) convert_rows_kernel(const float* __restrict__ src, int64_t rows, int64_t cols,
                                                            __nv_bfloat16* __restrict__ dst, int64_t ld) {
   pdl_launch_dependents();
-  pdl_wait();
+  pdl_wait(src);
   const int64_t quads = cols / 4;
   const int64_t total = rows * quads;
   const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
@@ -667,7 +303,7 @@ __global__ void __launch_bounds__(256) pack_mlr_kernel(const float* __restrict__
                                                        float* __restrict__ Xf, const int32_t* labels, int32_t* labels_out,
                                                        int32_t* __restrict__ slot, int64_t rows, const Stamp stamp) {
   pdl_launch_dependents();
-  pdl_wait();
+  pdl_wait(X);
   stamp_begin(stamp);
   const uint32_t quads = static_cast<uint32_t>(cols / 4);
   const int64_t total = n * quads, stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
@@ -682,113 +318,6 @@ __global__ void __launch_bounds__(256) pack_mlr_kernel(const float* __restrict__
     const int32_t old = labels_out[off + i];
     if (old >= 0 && old < rows) slot[old] = kNoSlot;
     labels_out[off + i] = labels[i];
-  }
-}
-
-// W [n x dim] -> its transpose as a (hi | lo) bf16 operand FT [dim x 2*Kp] (the coder's W^T): FT[c][i] = hi(F[i][c]),
-// FT[c][Kp + i] = lo(F[i][c]) with hi = bf16(f), lo = bf16(f - hi); rows n..Kp-1 are written as zeros.  64 x 64 tiles through
-// shared memory.
-__global__ void __launch_bounds__(256) pack_split_t_kernel(const float* __restrict__ F, int64_t n, int64_t dim,
-                                                           int64_t ld, __nv_bfloat16* __restrict__ FT, int64_t Kp) {
-  pdl_launch_dependents();
-  pdl_wait();
-  __shared__ float tile[64][65];
-  const int64_t i0 = static_cast<int64_t>(blockIdx.y) * 64, c0 = static_cast<int64_t>(blockIdx.x) * 64;
-  const int t = threadIdx.x;
-  const bool vec = (ld % 4) == 0;
-#pragma unroll
-  for (int v = 0; v < 4; ++v) {
-    const int idx = t + v * 256;            // 64 samples x 16 quads
-    const int i = idx / 16, cq = (idx % 16) * 4;
-    float f[4] = {0.f, 0.f, 0.f, 0.f};
-    if (i0 + i < n) {
-      const float* src = F + (i0 + i) * ld + c0 + cq;
-      if (vec && c0 + cq + 3 < dim) {
-        const float4 q4 = *reinterpret_cast<const float4*>(src);
-        f[0] = q4.x; f[1] = q4.y; f[2] = q4.z; f[3] = q4.w;
-      } else {
-        for (int k = 0; k < 4; ++k)
-          if (c0 + cq + k < dim) f[k] = src[k];
-      }
-    }
-    tile[i][cq + 0] = f[0]; tile[i][cq + 1] = f[1]; tile[i][cq + 2] = f[2]; tile[i][cq + 3] = f[3];
-  }
-  __syncthreads();
-#pragma unroll
-  for (int v = 0; v < 2; ++v) {
-    const int idx = t + v * 256;            // 64 features x 8 groups of 8 samples
-    const int c = idx / 8, ig = (idx % 8) * 8;
-    if (c0 + c >= dim) continue;
-    uint32_t hi[4], lo[4];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      const float f0 = tile[ig + 2 * k][c], f1 = tile[ig + 2 * k + 1][c];
-      const __nv_bfloat16 h0 = __float2bfloat16_rn(f0), h1 = __float2bfloat16_rn(f1);
-      hi[k] = static_cast<uint32_t>(__bfloat16_as_ushort(h0)) | (static_cast<uint32_t>(__bfloat16_as_ushort(h1)) << 16);
-      lo[k] = pack_bf16(f0 - __bfloat162float(h0), f1 - __bfloat162float(h1));
-    }
-    __nv_bfloat16* dst = FT + (c0 + c) * 2 * Kp + i0 + ig;     // Kp is a multiple of 64: 16-byte aligned
-    *reinterpret_cast<uint4*>(dst) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
-    *reinterpret_cast<uint4*>(dst + Kp) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
-  }
-}
-
-// fp32 [n x dim] (row pitch ld) -> the (hi | lo) bf16 operand [n x 2*dimp], no transpose: dst[r][c] = hi,
-// dst[r][dimp + c] = lo with hi = bf16(f), lo = bf16(f - hi).  Columns dim..dimp-1 are left as they are (zero since
-// set-up).
-__global__ void __launch_bounds__(256) pack_split_rows_kernel(const float* __restrict__ F, int64_t n, int64_t dim,
-                                                              int64_t ld, __nv_bfloat16* __restrict__ dst, int64_t dimp,
-                                                              const Stamp stamp) {
-  pdl_launch_dependents();
-  pdl_wait();
-  stamp_begin(stamp);
-  const int64_t quads = (dim + 3) / 4, total = n * quads;
-  const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
-  const bool vec = ld % 4 == 0 && dim % 4 == 0;          // else (samples with an odd number of features) value by value
-  for (int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; i < total; i += stride) {
-    const int64_t r = i / quads, qd = i % quads;
-    const float* src = F + r * ld + qd * 4;
-    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (vec) {
-      v = *reinterpret_cast<const float4*>(src);
-    } else {
-      v.x = src[0];
-      if (qd * 4 + 1 < dim) v.y = src[1];
-      if (qd * 4 + 2 < dim) v.z = src[2];
-      if (qd * 4 + 3 < dim) v.w = src[3];
-    }
-    const __nv_bfloat16 h0 = __float2bfloat16_rn(v.x), h1 = __float2bfloat16_rn(v.y), h2 = __float2bfloat16_rn(v.z),
-                        h3 = __float2bfloat16_rn(v.w);
-    __nv_bfloat16* d = dst + r * 2 * dimp + qd * 4;
-    *reinterpret_cast<uint2*>(d) =
-        make_uint2(static_cast<uint32_t>(__bfloat16_as_ushort(h0)) | (static_cast<uint32_t>(__bfloat16_as_ushort(h1)) << 16),
-                   static_cast<uint32_t>(__bfloat16_as_ushort(h2)) | (static_cast<uint32_t>(__bfloat16_as_ushort(h3)) << 16));
-    *reinterpret_cast<uint2*>(d + dimp) = make_uint2(pack_bf16(v.x - __bfloat162float(h0), v.y - __bfloat162float(h1)),
-                                                     pack_bf16(v.z - __bfloat162float(h2), v.w - __bfloat162float(h3)));
-  }
-}
-
-// DML: v = x - y of n pairs (Section 2) in fp32 and as the (hi | lo) operand, one pass (16 bytes per value; as two kernels 24).
-__global__ void __launch_bounds__(256) pack_pairs_kernel(const float* __restrict__ X, const float* __restrict__ Y, int64_t n,
-                                                         int64_t dim, float* __restrict__ V,
-                                                         __nv_bfloat16* __restrict__ dst,
-                                                         int64_t dimp, const Stamp stamp) {
-  pdl_launch_dependents();
-  pdl_wait();
-  stamp_begin(stamp);
-  const uint32_t quads = static_cast<uint32_t>(dim / 4);
-  const int64_t total = n * quads, stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
-  for (int64_t q = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; q < total; q += stride) {
-    const int64_t i = q / quads, c = (q - i * quads) * 4;
-    const float4 x = reinterpret_cast<const float4*>(X)[q], y = reinterpret_cast<const float4*>(Y)[q];
-    const float4 v = make_float4(x.x - y.x, x.y - y.y, x.z - y.z, x.w - y.w);
-    reinterpret_cast<float4*>(V)[q] = v;
-    const uint32_t h01 = pack_bf16(v.x, v.y), h23 = pack_bf16(v.z, v.w);
-    const float2 f01 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&h01));
-    const float2 f23 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&h23));
-    __nv_bfloat16* d = dst + i * 2 * dimp + c;
-    *reinterpret_cast<uint2*>(d) = make_uint2(h01, h23);
-    *reinterpret_cast<uint2*>(d + dimp) = make_uint2(pack_bf16(v.x - f01.x, v.y - f01.y), pack_bf16(v.z - f23.x, v.w - f23.y));
   }
 }
 
@@ -812,7 +341,7 @@ __global__ void __launch_bounds__(256) mlr_lse_kernel(const float2* __restrict__
                                                       float* __restrict__ coef, int32_t* __restrict__ slot,
                                                       uint32_t* status) {
   pdl_launch_dependents();
-  pdl_wait();
+  pdl_wait(part, Z, labels);
   const int64_t i = static_cast<int64_t>(blockIdx.x) * 8 + (threadIdx.x >> 5);
   if (i >= n) return;
   const int lane = threadIdx.x & 31;
@@ -983,7 +512,7 @@ __global__ void __launch_bounds__(256) label_delta_kernel(const LabelArgs a) {
 __global__ void __launch_bounds__(256) label_slots_kernel(const int32_t* __restrict__ labels, int32_t K, int64_t rows,
                                                           int32_t* __restrict__ slot, const Stamp stamp) {
   pdl_launch_dependents();
-  pdl_wait();
+  pdl_wait(labels);
   stamp_begin(stamp);
   const int i = blockIdx.x * 256 + threadIdx.x;
   if (i >= K) return;
@@ -999,7 +528,7 @@ __global__ void __launch_bounds__(256) mlr_shard_partials_tc_kernel(const float2
                                                                     const int32_t* __restrict__ labels, int64_t row_off,
                                                                     int64_t n, float4* __restrict__ out) {
   pdl_launch_dependents();
-  pdl_wait();
+  pdl_wait(part, Z, labels);
   const int64_t i = static_cast<int64_t>(blockIdx.x) * 8 + (threadIdx.x >> 5);
   if (i >= n) return;
   const int lane = threadIdx.x & 31;
@@ -1028,7 +557,7 @@ __global__ void __launch_bounds__(256) mlr_shard_finish_tc_kernel(const float4* 
                                                                   float* __restrict__ lse, float* __restrict__ loss,
                                                                   float* __restrict__ coef, uint32_t* status) {
   pdl_launch_dependents();
-  pdl_wait();
+  pdl_wait(parts);
   const int64_t i = static_cast<int64_t>(blockIdx.x) * 256 + threadIdx.x;
   if (i >= n) return;
   float M = -INFINITY;
@@ -1064,7 +593,7 @@ __global__ void __launch_bounds__(256) mlr_emit_p_kernel(const float* __restrict
                                                          const int32_t* __restrict__ labels, __nv_bfloat16* __restrict__ P,
                                                          int64_t ldp, int lab_blocks, const LabelArgs lab) {
   pdl_launch_dependents();
-  pdl_wait();
+  pdl_wait(Z, lse, labels);
   if (static_cast<int>(blockIdx.x) < lab_blocks) return label_delta(lab, blockIdx.x, lab_blocks);
   const uint32_t octs = static_cast<uint32_t>((rows + 7) / 8);
   const int64_t total = n * octs, stride = static_cast<int64_t>(gridDim.x - lab_blocks) * blockDim.x;
@@ -1096,7 +625,7 @@ __device__ __forceinline__ float to_tf32(float x) {
 __global__ void __launch_bounds__(256) split32_rows_kernel(const float* __restrict__ F, int64_t n, int64_t dim, int64_t ld,
                                                            float* __restrict__ dst, int64_t dimp) {
   pdl_launch_dependents();
-  pdl_wait();
+  pdl_wait(F);
   const int64_t quads = dim / 4, total = n * quads;
   const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
   for (int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; i < total; i += stride) {
@@ -1115,7 +644,7 @@ __global__ void __launch_bounds__(256) split32_rows_kernel(const float* __restri
 __global__ void __launch_bounds__(256) split32_t_kernel(const float* __restrict__ F, int64_t n, int64_t dim, int64_t ld,
                                                         float* __restrict__ FT, int64_t Kp) {
   pdl_launch_dependents();
-  pdl_wait();
+  pdl_wait(F);
   __shared__ float tile[64][65];
   const int64_t i0 = static_cast<int64_t>(blockIdx.y) * 64, c0 = static_cast<int64_t>(blockIdx.x) * 64;
   const int t = threadIdx.x;
@@ -1146,7 +675,7 @@ __global__ void __launch_bounds__(256) mlr_finish_u_kernel(const float* __restri
                                                            const int32_t* __restrict__ labels,
                                                            float* __restrict__ U) {
   pdl_launch_dependents();
-  pdl_wait();
+  pdl_wait(Z, lse, labels);
   const int64_t i = blockIdx.y;
   const float l = lse[i];
   const int64_t y = labels[i];
@@ -1170,26 +699,10 @@ cudaError_t launch_forward(sfb_ctx* ctx, const CUtensorMap& a, const CUtensorMap
                           p.kparts, a, b, c, p);
 }
 
-template <int EPI>
-cudaError_t launch_forward_split(sfb_ctx* ctx, const CUtensorMap& a, const CUtensorMap& b, float* C, int64_t ldc, TcParams p) {
-  TcState* st = static_cast<TcState*>(ctx->tc);
-  const int64_t tiles = EPI == F_GRAM ? sym_tiles(p.tilesM, p.tilesN, p.bn) : static_cast<int64_t>(p.tilesM) * p.tilesN;
-  if (tiles <= 0) return cudaSuccess;
-  const unsigned grid = static_cast<unsigned>(p.kparts > 1 ? tiles * p.kparts : std::min<int64_t>(tiles, st->sms));
-  return launch_kernel_if(tiles * p.kparts <= st->sms, forward_split_kernel<EPI>, dim3(grid), dim3(kFsThreads), kFsSmem, ctx->stream,
-                          p.kparts, a, b, C, ldc, p);
-}
-
 // The shared-memory opt-in is a per-device attribute of each kernel: set for every instantiation when a context is
 // created (with its device current), not once per process.
 cudaError_t prepare_forward_kernels() {
   cudaError_t e = cudaFuncSetAttribute(forward_kernel<F_SOFTMAX>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(forward_split_kernel<F_STORE>, cudaFuncAttributeMaxDynamicSharedMemorySize, kFsSmem);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(forward_split_kernel<F_SUB>, cudaFuncAttributeMaxDynamicSharedMemorySize, kFsSmem);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(forward_split_kernel<F_ISTA>, cudaFuncAttributeMaxDynamicSharedMemorySize, kFsSmem);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(forward_split_kernel<F_ISTAG>, cudaFuncAttributeMaxDynamicSharedMemorySize, kFsSmem);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(forward_split_kernel<F_ISTA0>, cudaFuncAttributeMaxDynamicSharedMemorySize, kFsSmem);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(forward_split_kernel<F_GRAM>, cudaFuncAttributeMaxDynamicSharedMemorySize, kFsSmem);
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(forward_kernel<F_SOFTMAX, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
   return e;
@@ -1270,27 +783,7 @@ void tc_extend_layout(const sfb_config& c, Layout& L, size_t& off) {
   const size_t K = static_cast<size_t>(c.workers) * c.batch;
   L.Kp = round_up(static_cast<int64_t>(K), 64);
   L.colsb = round_up(c.cols, 64);
-  if (c.model != SFB_MLR) {
-    // fp32 factors as the workers write them, and the split-bf16 operands of the forward and update products
-    L.colsp = round_up(c.cols, 64);
-    L.rowsp = round_up(c.rows, 64);
-    L.ldu = round_up(c.rows, 4);                                        // TMA stores need a 16-byte row pitch
-    L.V = take(K * static_cast<size_t>(c.cols) * 4);
-    L.U = take(K * static_cast<size_t>(L.ldu) * 4);
-    L.Rs = take(K * 2 * static_cast<size_t>(L.rowsp) * 2);              // u (SC: first x, then the residuals)
-    L.Ws = take(static_cast<size_t>(c.rows) * 2 * L.colsp * 2);         // W, rows x (hi | lo)
-    L.As = take(K * 2 * static_cast<size_t>(L.colsp) * 2);              // v (DML) or the codes a (SC)
-    if (c.model == SFB_SC) {
-      L.WTs = take(static_cast<size_t>(c.cols) * 2 * L.rowsp * 2);      // W^T, atoms x (hi | lo)
-      if (sc_use_gram(c)) {
-        L.Gs = take(static_cast<size_t>(c.cols) * 2 * L.colsp * 2);     // W^T W, atoms x (hi | lo)
-        L.G = take(c.sc_lipschitz > 0.f ? 0 : static_cast<size_t>(c.cols) * c.cols * 4);   // in fp32 for the power iteration
-        L.Bx = take(K * static_cast<size_t>(c.cols) * 4);               // W^T x
-        L.As2 = take(K * 2 * static_cast<size_t>(L.colsp) * 2);         // the codes of every other iteration
-      }
-    }
-    return;
-  }
+  if (c.model != SFB_MLR) return split_extend_layout(c, L, off);
   const size_t ldz = static_cast<size_t>(round_up(c.rows, 32));
   L.split = pick_forward_split(static_cast<int64_t>(K), c.rows, c.cols);
   L.pw = L.split > 1 ? 32 : pick_forward_width(c.batch, c.rows, c.cols, 32, 1);
@@ -1335,22 +828,7 @@ int tc_init(sfb_ctx* ctx) {
     CKC(cudaMemsetAsync(ctx->at<char>(L.As), 0, static_cast<size_t>(ctx->K) * 2 * L.colsp * 4, ctx->stream));
     return tc_refresh_operands(ctx);
   }
-  if (c.model != SFB_MLR) {
-    // pad columns of the split operands are never written by the kernels: clear the buffers once
-    const Layout& L = ctx->lay;
-    const size_t K = static_cast<size_t>(ctx->K);
-    CKC(cudaMemsetAsync(ctx->at<char>(L.Ws), 0, static_cast<size_t>(c.rows) * 2 * L.colsp * 2, ctx->stream));
-    CKC(cudaMemsetAsync(ctx->at<char>(L.As), 0, K * 2 * L.colsp * 2, ctx->stream));
-    CKC(cudaMemsetAsync(ctx->at<char>(L.Rs), 0, K * 2 * L.rowsp * 2, ctx->stream));
-    if (c.model == SFB_SC) {
-      CKC(cudaMemsetAsync(ctx->at<char>(L.WTs), 0, static_cast<size_t>(c.cols) * 2 * L.rowsp * 2, ctx->stream));
-      if (L.Gs) {
-        CKC(cudaMemsetAsync(ctx->at<char>(L.Gs), 0, static_cast<size_t>(c.cols) * 2 * L.colsp * 2, ctx->stream));
-        CKC(cudaMemsetAsync(ctx->at<char>(L.As2), 0, K * 2 * L.colsp * 2, ctx->stream));
-      }
-    }
-    return SFB_OK;
-  }
+  if (c.model != SFB_MLR || ctx->h16) return split_init(ctx);
   CKC(cudaMemsetAsync(ctx->at<char>(ctx->lay.labels), 0xff, static_cast<size_t>(ctx->K) * 4, ctx->stream));
   CKC(cudaMemsetAsync(ctx->at<char>(ctx->lay.slot), 0x7f, static_cast<size_t>(c.rows) * 4, ctx->stream));
   // bf16 copy of W for the forward product; afterwards the update's epilogue keeps it current
@@ -1374,199 +852,6 @@ int tc_refresh_operands(sfb_ctx* ctx) {
 void tc_destroy(sfb_ctx* ctx) {
   delete static_cast<TcState*>(ctx->tc);
   ctx->tc = nullptr;
-}
-
-namespace {
-
-inline unsigned grid1d(int64_t items, int per_block) {
-  int64_t g = (items + per_block - 1) / per_block;
-  return static_cast<unsigned>(std::max<int64_t>(1, std::min<int64_t>(g, static_cast<int64_t>(sm_count()) * 16)));
-}
-
-// Tile width (a multiple of `step` columns, at most `widest`) for a product with tilesM row blocks and N columns on
-// `sms` SMs.  The
-// persistent kernel runs ceil(tiles / sms) rounds of tiles; measured, a tile costs about max(width, 128) + 16
-// column-equivalents (below 128 columns a k-block is bound by the latency of its operand loads, not by the MMA).
-// Narrower tiles fill the SMs of small products, where 256-wide ones leave many idle or need a nearly empty
-// second round; ties go to the wider tile.
-inline int pick_tile_width(int sms, int64_t tilesM, int64_t N, int widest, int step = 32, bool sym = false) {
-  int best = widest;
-  int64_t best_cost = INT64_MAX;
-  if (N <= 112) return static_cast<int>(round_up(N, step));
-  for (int bn = widest; bn >= 128; bn -= step) {
-    const int64_t tn = (N + bn - 1) / bn;
-    const int64_t tiles = sym ? sym_tiles(static_cast<int>(tilesM), static_cast<int>(tn), bn) : tilesM * tn;
-    const int64_t cost = ((tiles + sms - 1) / sms) * (bn + 16);
-    if (cost < best_cost) { best_cost = cost; best = bn; }
-  }
-  return best;
-}
-
-// Features up to which the coder on W^T W forms W^T x by fp32 FMAs and W^T W with its fourth term.  Every iterate carries
-// their error, and for short contractions the rounding of the operands to pairs is most of it (for long ones it is the
-// tensor core's own rounding, which the second accumulator brought down).  Error of the codes with / without, and with two
-// products per iteration: 700 x 400: 3.7e-6 / 9.1e-6, 5.0e-6; 1,501 x 1,400: 5.1e-6 / 9.9e-6, 7.3e-6.
-constexpr int64_t kPreciseRows = 2048;
-
-constexpr int kSplitPrefetch = SFB_SPLIT_PREFETCH;    // k-blocks of look-ahead of the L2 prefetch in the split products
-
-// Cost of a split product in rounds of tiles x columns x k-blocks, its contraction in `split` parts.
-double split_cost(int64_t M, int64_t N, int64_t Kc, bool sym, int split) {
-  const int sms = sm_count();
-  const int64_t tm = (M + BM - 1) / BM;
-  const int bn = pick_tile_width(sms / split, tm, N, FS_BN, 16, sym);
-  const int64_t tn = (N + bn - 1) / bn;
-  const int64_t tiles = sym ? sym_tiles(static_cast<int>(tm), static_cast<int>(tn), bn) : tm * tn;
-  const double kb = static_cast<double>((Kc + BK - 1) / BK) / split;
-  return static_cast<double>((tiles * split + sms - 1) / sms) * (std::max(bn, 128) + 16) * (kb + 8.0 + (split > 1 ? 6.0 : 0.0));
-}
-// Parts of the contraction for all M samples of the product (a slice of them takes the same: it fixes the order of the sums):
-// where the tiles leave SMs idle and the k-blocks of one follow each other on one SM.
-int split_parts(int64_t M, int64_t N, int64_t Kc) {
-  int best = 1;
-  double cost = split_cost(M, N, Kc, false, 1);
-  for (int s = 2; s <= 8 && Kc / BK >= 2 * s; s *= 2) {
-    const double c = split_cost(M, N, Kc, false, s);
-    if (c < 0.9 * cost) { cost = c; best = s; }
-  }
-  return best;
-}
-
-// One split-bf16 product  D[off..off+n) = A * B^T  with A = [*, 2*Cp] and B = [N x 2*Cp] (hi | lo) operands:
-// hi*hi + hi*lo + lo*hi over a contraction of Cp.
-template <int EPI>
-int split_product(sfb_ctx* ctx, int64_t off, int64_t n, __nv_bfloat16* A, __nv_bfloat16* B, int64_t N, int64_t Cp,
-                  float* C, int64_t ldc, TcParams p) {
-  TcState* st = static_cast<TcState*>(ctx->tc);
-  p.kparts = EPI == F_GRAM ? 1 : split_parts(ctx->K, N, Cp);
-  const int bn = pick_tile_width(st->sms / p.kparts, (n + BM - 1) / BM, N, FS_BN, 16, EPI == F_GRAM);
-  CUtensorMap ma, mb;
-  if (!make_map(st, &ma, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, A, 2 * Cp, off + n, 2 * Cp * 2, BK, BM) ||
-      !make_map(st, &mb, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, B, 2 * Cp, N, 2 * Cp * 2, BK, bn))
-    return SFB_ERR_CUDA;
-  p.M = static_cast<int32_t>(off + n); p.N = static_cast<int32_t>(N); p.Kc = static_cast<int32_t>(Cp);
-  p.m_off = static_cast<int32_t>(off);
-  p.tilesM = static_cast<int32_t>((n + BM - 1) / BM);
-  p.bn = bn;
-  p.tilesN = static_cast<int32_t>((N + bn - 1) / bn);
-  p.nseg = 3; p.kseg = static_cast<int32_t>(Cp / BK);
-  p.prefetch = kSplitPrefetch;
-  p.a_off0 = 0; p.a_off1 = 0; p.a_off2 = static_cast<int32_t>(Cp);
-  p.b_off0 = 0; p.b_off1 = static_cast<int32_t>(Cp); p.b_off2 = 0;
-  p.status = ctx->at<uint32_t>(ctx->lay.status);
-  CKC(launch_forward_split<EPI>(ctx, ma, mb, C, ldc, p));
-  ctx->stats.flops += (EPI == F_GRAM ? 3.0 : 6.0) * n * N * Cp;
-  return SFB_OK;
-}
-
-// Sufficient factors of distance metric learning and sparse coding in bf16 mode: the same steps as the fp32
-// path (Section 2: z = W v with v = x - y; Figure 3: ISTA codes, u = W a - x), every product on the tensor cores
-// with (hi | lo) bf16 operands.
-int factors_split(sfb_ctx* ctx, int64_t off, int64_t n, const float* X, const float* Y, const int32_t* labels,
-                  float* dml_norm_out = nullptr) {
-  const sfb_config& c = ctx->cfg;
-  const Layout& L = ctx->lay;
-  const int64_t rows = c.rows, cols = c.cols;
-  cudaStream_t s = ctx->stream;
-  float* V = ctx->at<float>(L.V);
-  float* U = ctx->at<float>(L.U);
-  __nv_bfloat16* Ws = ctx->at<__nv_bfloat16>(L.Ws);
-  __nv_bfloat16* As = ctx->at<__nv_bfloat16>(L.As);
-  TcParams p{};
-  if (c.model == SFB_DML) {
-    CKC(launch_kernel(pack_pairs_kernel, dim3(grid1d(n * cols / 4, 256)), dim3(256), 0, s, 1, X, Y, n, cols,
-                      V + off * cols, As + off * 2 * L.colsp, L.colsp, Stamp{}));
-      int rc = split_product<F_STORE>(ctx, off, n, As, Ws, rows, L.colsp, U, L.ldu, p);    // z_i = W v_i
-    if (rc) return rc;
-    CKC(dml_scale_rows(s, U + off * L.ldu, n, rows, L.ldu, labels, c.dml_margin,
-                       ctx->at<__nv_bfloat16>(L.Rs) + off * 2 * L.rowsp, L.rowsp, dml_norm_out));
-    return SFB_OK;
-  }
-  // Sparse coding: ISTA from a = 0, then u = W a - x, v = a.  The first iterate is soft(W^T x / L).
-  const int T = c.sc_ista_iters;
-  const bool gram = L.Gs != 0;
-  __nv_bfloat16* WTs = ctx->at<__nv_bfloat16>(L.WTs);
-  __nv_bfloat16* Rs = ctx->at<__nv_bfloat16>(L.Rs);
-  // the iterates as operands: with the Gram matrix a product reads one and writes the next, so two buffers in turn
-  __nv_bfloat16* as[2] = {As, gram ? ctx->at<__nv_bfloat16>(L.As2) : As};
-  auto ista = [&](int t) {
-    TcParams q{};
-    q.aux = V; q.ldaux = cols;
-    q.sc = ctx->at<Scalars>(L.scalars); q.lam = c.sc_lambda;
-    q.split = as[t & 1]; q.ld_split = 2 * L.colsp; q.split_half = static_cast<int32_t>(L.colsp);
-    return q;
-  };
-  auto residual = [&](__nv_bfloat16* a) {                                               // r = W a - x
-    TcParams q{};
-    q.aux = X - off * rows; q.ldaux = rows;          // X holds this worker's samples: index it by the global row
-    q.split = Rs; q.ld_split = 2 * L.rowsp; q.split_half = static_cast<int32_t>(L.rowsp);
-    return split_product<F_SUB>(ctx, off, n, a, Ws, rows, L.colsp, U, L.ldu, q);
-  };
-  int rc = SFB_OK;
-  if (T == 0) {
-    CKC(cudaMemsetAsync(V + off * cols, 0, static_cast<size_t>(n) * cols * 4, s));
-    CKC(cudaMemsetAsync(As + off * 2 * L.colsp, 0, static_cast<size_t>(n) * 2 * L.colsp * 2, s));
-  } else {
-    if (gram && rows <= kPreciseRows) {                                                 // W^T x, a_1
-      EpiArgs e{};
-      e.C = V + off * cols; e.ldc = cols; e.C2 = ctx->at<float>(L.Bx) + off * cols; e.ldc2 = cols;
-      e.sc = ctx->at<Scalars>(L.scalars); e.lam = c.sc_lambda;
-      CKC(sgemm(s, true, false, EPI_ISTA0, n, cols, rows, X, rows, ctx->W, cols, e, ctx->K));
-      ctx->stats.flops += 2.0 * n * rows * cols;
-      CKC(launch_kernel(pack_split_rows_kernel, dim3(grid1d(n * cols / 4, 256)), dim3(256), 0, s, 1, V + off * cols, n,
-                        cols, cols, as[1] + off * 2 * L.colsp, L.colsp, Stamp{}));
-    } else {
-      CKC(launch_kernel(pack_split_rows_kernel, dim3(grid1d(n * ((rows + 3) / 4), 256)), dim3(256), 0, s, 1, X, n, rows,
-                        rows, Rs + off * 2 * L.rowsp, L.rowsp, Stamp{}));
-      p = ista(1);
-      p.C2 = gram ? ctx->at<float>(L.Bx) : nullptr;
-      if ((rc = split_product<F_ISTA0>(ctx, off, n, Rs, WTs, cols, L.rowsp, V, cols, p)) != SFB_OK) return rc;
-    }
-  }
-  for (int t = 2; t <= T; ++t) {
-    p = ista(t);
-    if (gram) {
-      p.C2 = ctx->at<float>(L.Bx);
-      rc = split_product<F_ISTAG>(ctx, off, n, as[(t - 1) & 1], ctx->at<__nv_bfloat16>(L.Gs), cols, L.colsp, V, cols, p);
-    } else {
-      if ((rc = residual(As)) != SFB_OK) return rc;
-      rc = split_product<F_ISTA>(ctx, off, n, Rs, WTs, cols, L.rowsp, V, cols, p);      // a <- soft(a - W^T r / L)
-    }
-    if (rc) return rc;
-  }
-  return residual(T == 0 ? As : as[T & 1]);                                             // u = W a - x
-}
-
-}  // namespace
-
-// The operands that the factors of every worker of a step share: the split copies of the W that all of them see
-// (bulk-synchronous consistency), and for sparse coding its transpose and W^T W.
-int tc_begin_step(sfb_ctx* ctx) {
-  const sfb_config& c = ctx->cfg;
-  if (c.model == SFB_MLR) return SFB_OK;
-  const Layout& L = ctx->lay;
-  const int64_t rows = c.rows, cols = c.cols;
-  cudaStream_t s = ctx->stream;
-  CKC(launch_kernel(pack_split_rows_kernel, dim3(grid1d(rows * cols / 4, 256)), dim3(256), 0, s, 1, ctx->W, rows, cols,
-                    cols, ctx->at<__nv_bfloat16>(L.Ws), L.colsp, take_stamp(ctx)));
-  if (c.model == SFB_SC) {
-    __nv_bfloat16* WTs = ctx->at<__nv_bfloat16>(L.WTs);
-    CKC(launch_kernel(pack_split_t_kernel, dim3(static_cast<unsigned>((cols + 63) / 64),
-                      static_cast<unsigned>(L.rowsp / 64)), dim3(256), 0, s, 1, ctx->W, rows, cols, cols, WTs, L.rowsp));
-    if (L.Gs) {
-      TcParams p{};
-      p.four = rows <= kPreciseRows;
-      p.split = ctx->at<__nv_bfloat16>(L.Gs); p.ld_split = 2 * L.colsp; p.split_half = static_cast<int32_t>(L.colsp);
-      float* G = c.sc_lipschitz > 0.f ? nullptr : ctx->at<float>(L.G);
-      const int rc = split_product<F_GRAM>(ctx, 0, cols, WTs, WTs, cols, L.rowsp, G, cols, p);
-      if (rc) return rc;
-    }
-  }
-  return SFB_OK;
-}
-
-double split_product_cost(int64_t M, int64_t N, int64_t Kc, bool sym) {
-  return split_cost(M, N, Kc, sym, sym ? 1 : split_parts(M, N, Kc));
 }
 
 // v = x, the (big | small) samples, and the logits of n samples at pair offset off against this context's rows as
@@ -1793,7 +1078,7 @@ __global__ void __launch_bounds__(256) mlr_export_u_kernel(const float* __restri
                                                            const int32_t* __restrict__ labels,
                                                            int64_t off, float* __restrict__ U_out) {
   pdl_launch_dependents();
-  pdl_wait();
+  pdl_wait(Z, lse, labels);
   const int64_t i = blockIdx.y;
   const float l = lse[off + i];
   const int32_t y = labels[off + i];
@@ -1811,7 +1096,7 @@ __global__ void __launch_bounds__(256) mlr_import_labels_kernel(const float* __r
                                                                 int32_t* __restrict__ labels, float* __restrict__ coef,
                                                                 float* __restrict__ loss, int32_t* __restrict__ slot) {
   pdl_launch_dependents();
-  pdl_wait();
+  pdl_wait(U_in);
   __shared__ float sv[256];
   __shared__ int32_t si[256];
   const int64_t i = blockIdx.x;
@@ -1903,7 +1188,15 @@ int tc_sdca_factors(sfb_ctx* ctx, int64_t off, int64_t n, const float* X, const 
 
 int tc_factors(sfb_ctx* ctx, int64_t off, int64_t n, const float* X, const float* Y, const int32_t* labels, bool fused,
                float* dml_norm_out) {
-  if (ctx->cfg.model != SFB_MLR) return factors_split(ctx, off, n, X, Y, labels, dml_norm_out);
+  if (ctx->cfg.model == SFB_SC) return split_factors_sc(ctx, off, n, X);
+  if (ctx->cfg.model == SFB_DML) {
+    const Layout& L = ctx->lay;
+    const int rc = split_logits(ctx, off, n, X, Y);                                     // z_i = W v_i
+    if (rc) return rc;
+    CKC(dml_scale_rows(ctx->stream, ctx->at<float>(L.U) + off * L.ldu, n, ctx->cfg.rows, L.ldu, labels, ctx->cfg.dml_margin,
+                       ctx->at<uint16_t>(L.Rs) + off * 2 * L.rowsp, L.rowsp, nullptr, nullptr, dml_norm_out));
+    return SFB_OK;
+  }
   const sfb_config& c = ctx->cfg;
   const Layout& L = ctx->lay;
   const int64_t rows = c.rows, K = ctx->K;
@@ -1917,27 +1210,6 @@ int tc_factors(sfb_ctx* ctx, int64_t off, int64_t n, const float* X, const float
                     ctx->at<float2>(L.part), K, tiles_n, Z, ldz, rows, labels, off, n, lse, ctx->at<float>(L.loss),
                     ctx->at<float>(L.coef), fused ? ctx->at<int32_t>(L.slot) : nullptr, ctx->at<uint32_t>(L.status)));
   return emit_p<false>(ctx, off, n, labels, fused ? X : nullptr);
-}
-
-// The (hi | lo) codes or pair differences: the operand V of the update.
-__nv_bfloat16* tc_split_v(const sfb_ctx* ctx) {
-  const Layout& L = ctx->lay;
-  const bool odd = ctx->cfg.model == SFB_SC && L.Gs != 0 && (ctx->cfg.sc_ista_iters & 1);     // which buffer the last iterate is in
-  return ctx->at<__nv_bfloat16>(odd ? L.As2 : L.As);
-}
-
-// Factors computed elsewhere (DML, SC): fp32 pairs in U and V -> the operands of the update.
-int tc_pack_received(sfb_ctx* ctx, int64_t off, int64_t n) {
-  const sfb_config& c = ctx->cfg;
-  const Layout& L = ctx->lay;
-  cudaStream_t s = ctx->stream;
-  CKC(launch_kernel(pack_split_rows_kernel, dim3(grid1d(n * ((c.rows + 3) / 4), 256)), dim3(256), 0, s, 1,
-                    ctx->at<float>(L.U) + off * L.ldu, n, c.rows, L.ldu, ctx->at<__nv_bfloat16>(L.Rs) + off * 2 * L.rowsp,
-                    L.rowsp, Stamp{}));
-  CKC(launch_kernel(pack_split_rows_kernel, dim3(grid1d(n * c.cols / 4, 256)), dim3(256), 0, s, 1,
-                    ctx->at<float>(L.V) + off * c.cols, n, c.cols, c.cols, tc_split_v(ctx) + off * 2 * L.colsp, L.colsp,
-                    Stamp{}));
-  return SFB_OK;
 }
 
 int tc_get_factors(sfb_ctx* ctx, const void** U, const void** V, int32_t* dtype, int32_t* layout, int64_t* ldu,

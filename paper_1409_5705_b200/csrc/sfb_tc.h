@@ -22,9 +22,6 @@ int tc_init(sfb_ctx* ctx);
 void tc_destroy(sfb_ctx* ctx);
 // Rebuilds the bf16 operand copy of W from the caller's fp32 W (MLR; the other models rebuild theirs every step).
 int tc_refresh_operands(sfb_ctx* ctx);
-// Before the first factors of a step: the operands derived from W that its workers share (DML, SC).
-int tc_begin_step(sfb_ctx* ctx);
-double split_product_cost(int64_t M, int64_t N, int64_t Kc, bool sym);
 // dml_norm_out (DML, row-sharded form; may be null): receives ||z_i||^2 of this context's rows and z stays unscaled.
 // fused: the call is part of one that goes on to the update, so X stays as it is until then.
 int tc_factors(sfb_ctx* ctx, int64_t off, int64_t n, const float* X, const float* Y, const int32_t* labels, bool fused,
@@ -41,9 +38,20 @@ int tc_labels(sfb_ctx* ctx);
 // MLR, bf16 mode: a worker's factors in fp32 as they are sent, and received fp32 factors put into the bf16 layout.
 int tc_export_factors(sfb_ctx* ctx, int64_t off, int64_t n, float* U_out, float* V_out);
 int tc_import_factors(sfb_ctx* ctx, int64_t off, int64_t n, const float* U_in, const float* V_in);
-// DML, SC in bf16 mode: fp32 factors put into the U and V buffers by the caller become (hi | lo) operands; the operand of V.
-int tc_pack_received(sfb_ctx* ctx, int64_t off, int64_t n);
-__nv_bfloat16* tc_split_v(const sfb_ctx* ctx);
+// Products of (hi | lo) pairs (sfb_split.cu): metric learning and sparse coding in bf16 mode, every model in fp32 mode
+// (ctx->h16).  Layout and set-up; what a step's factors share, formed from W before the first of them; v and z = W v of n
+// pairs (v = x, or x - y with Y) into the fp32 factor buffers; the factors of sparse coding; fp32 factors that the caller has
+// put into the U and V buffers as operands; the rest of the update's operands once all pairs are there; the operand V.
+void split_extend_layout(const sfb_config& c, Layout& L, size_t& off);
+cudaError_t split_reset(sfb_ctx* ctx);
+int split_init(sfb_ctx* ctx);
+int split_begin_step(sfb_ctx* ctx);
+int split_logits(sfb_ctx* ctx, int64_t off, int64_t n, const float* X, const float* Y);
+int split_factors_sc(sfb_ctx* ctx, int64_t off, int64_t n, const float* X);
+int split_pack_received(sfb_ctx* ctx, int64_t off, int64_t n);
+int split_gather(sfb_ctx* ctx);
+const uint16_t* split_v(const sfb_ctx* ctx);
+double split_product_cost(int64_t M, int64_t N, int64_t Kc, bool sym);
 int tc_update(sfb_ctx* ctx);
 int tc_get_factors(sfb_ctx* ctx, const void** U, const void** V, int32_t* dtype, int32_t* layout, int64_t* ldu,
                    int64_t* ldv);

@@ -97,7 +97,7 @@ __device__ __forceinline__ void tile_origin(const UpdParams& p, int tile, int& m
 
 // TF32: the operands are 32-bit words read as tf32 (32 elements per 128-byte k-block), see the forward kernel.
 // SHADOW: the operand copy of the new W that the epilogue writes beside it for the next forward product:
-// 0 none, 1 bf16, 2 the (big | small) pair of tf32 words of the fp32-on-tensor-cores mode.
+// 1 bf16, 2 the (big | small) pair of tf32 words of the fp32-on-tensor-cores mode.
 template <int SHADOW, bool TF32 = false>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
 update_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
@@ -369,12 +369,251 @@ update_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
   if (warp == 1) { tc_fence_after(); tmem_dealloc_pair(tmem_base, kTmemCols); }
 }
 
+// ---------------------------------------------------------------------------------------------------------
+// The update of operands that are (hi | lo) pairs of 16-bit values (metric learning, sparse coding):
+//   W <- prox(W + alpha * (U_hi^T V_hi + U_lo^T V_hi + U_hi^T V_lo)).
+// As in forward_split_kernel, one stage holds a k-block of all four halves (64 KB in a CTA of the pair, 43 bytes per cycle of
+// tensor work where three passes over the contraction take 64: those were bound by their loads) and the cross terms have an
+// accumulator of their own; U_hi^T V_hi is added to sums in the epilogue warps' registers every eight k-blocks, while the
+// cross terms of the last of them run.  The sums also free both accumulators (all 512 columns of TMEM) before the pass over
+// W, which therefore runs beside the next tile's products although there is no second pair of accumulators.
+// Shared memory: three stages and one 4 KB slot of W per epilogue warp.  1,000 x 20,000, K = 1024: 114 us with three passes.
+// ---------------------------------------------------------------------------------------------------------
+constexpr int SU_STAGES = 3, SU_DRAIN = 16;
+constexpr int kSuBytes = 64 * 2 * UM;                // 16 KB: one operand half of a k-block in a CTA
+constexpr int kSuStage = 4 * kSuBytes;
+constexpr int kSuBars = 2 * SU_STAGES + 4 + kEpiWarps;
+constexpr int kSuSmem = SU_STAGES * kSuStage + kEpiWarps * kSlotBytes + kSuBars * 8 + 16 + 1024;
+
+struct SplitUpdParams {
+  UpdParams t;                 // rows, cols, tiles, bn, kseg, alpha, prox, stamps, status
+  int32_t u_lo, v_lo;          // column of the lo half of U and of V
+  bool fp16;                   // the form of the pairs
+  float lo_scale;              // what an accumulated cross term counts for
+  const float* inv;            // inverse scale of the whole sum (or null: 1)
+};
+
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
+update_split_kernel(const __grid_constant__ CUtensorMap tmU, const __grid_constant__ CUtensorMap tmV,
+                    const __grid_constant__ CUtensorMap tmC, const __grid_constant__ SplitUpdParams sp) {
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  uint8_t* sRing = smem + SU_STAGES * kSuStage;
+  uint64_t* bars = reinterpret_cast<uint64_t*>(sRing + kEpiWarps * kSlotBytes);
+  uint64_t* full = bars;                             // as in update_pair_kernel: full, mempty, cempty are the leader's
+  uint64_t* empty = bars + SU_STAGES;
+  uint64_t* mfull = bars + 2 * SU_STAGES;
+  uint64_t* mempty = mfull + 1;
+  uint64_t* cfull = mfull + 2;
+  uint64_t* cempty = mfull + 3;
+  uint64_t* rfull = mfull + 4;                       // per epilogue warp
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + kSuBars);
+  volatile uint32_t* abort_flag = tmem_slot + 1;
+
+  const UpdParams& p = sp.t;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const uint32_t rank = cluster_ctarank();
+  const int pair = blockIdx.x >> 1, npairs = gridDim.x >> 1;
+  const int ntiles = p.tilesM * p.tilesN;
+  const int my_tiles = pair < ntiles ? (ntiles - 1 - pair) / npairs + 1 : 0;
+  const int nk = p.kseg, half = p.bn / 2;
+  pdl_launch_dependents();
+
+  if (threadIdx.x == 0) {
+    for (int i = 0; i < SU_STAGES; ++i) { mbar_init(&full[i], 1); mbar_init(&empty[i], 1); }
+    mbar_init(mfull, 1); mbar_init(mempty, 2 * kEpiWarps);
+    mbar_init(cfull, 1); mbar_init(cempty, 2 * kEpiWarps);
+    for (int i = 0; i < kEpiWarps; ++i) mbar_init(&rfull[i], 1);
+    *abort_flag = 0;
+    fence_barrier_init();
+    prefetch_tmap(&tmU); prefetch_tmap(&tmV); prefetch_tmap(&tmC);
+  }
+  if (warp == 1) { tmem_alloc_pair(tmem_slot, kTmemCols); tmem_relinquish_pair(); }
+  tc_fence_before();
+  __syncthreads();
+  cluster_arrive();
+  cluster_wait();
+  tc_fence_after();
+  const uint32_t tmem_base = *tmem_slot;
+  pdl_wait();
+  stamp_begin(p.begin);
+
+  if (warp == 0) {
+    // ---------------- TMA producer: U_hi, U_lo, V_hi, V_lo of a k-block, boxes of 64 columns x 64 pairs ----------------
+    if (lane == 0) {
+      const uint64_t pol_keep = policy_evict_last(), pol_norm = policy_evict_normal();
+      uint32_t it = 0;
+      bool ok = true;
+      for (int tl = 0; tl < my_tiles && ok; ++tl) {
+        int m0, n0;
+        tile_origin(p, pair + tl * npairs, m0, n0);
+        const int mu = m0 + static_cast<int>(rank) * UM, nv = n0 + static_cast<int>(rank) * half;
+        for (int kb = 0; kb < nk; ++kb, ++it) {
+          const uint32_t s = it % SU_STAGES, ph = (it / SU_STAGES) & 1;
+          if (!mbar_wait(&empty[s], ph ^ 1, abort_flag)) { ok = false; break; }
+          if (rank == 0) mbar_expect_tx(&full[s], 2 * (2 * kSuBytes + 2 * half * UK * 2));
+          const uint32_t bar = mapa_u32(smem_u32(&full[s]), 0);
+          uint8_t* st = smem + s * kSuStage;
+#pragma unroll
+          for (int b = 0; b < 2; ++b) {
+            tma_load_2d_pair(st + b * 8192, &tmU, mu + 64 * b, kb * UK, bar, pol_norm);
+            tma_load_2d_pair(st + kSuBytes + b * 8192, &tmU, sp.u_lo + mu + 64 * b, kb * UK, bar, pol_norm);
+            if (64 * b < half) {
+              tma_load_2d_pair(st + 2 * kSuBytes + b * 8192, &tmV, nv + 64 * b, kb * UK, bar, pol_keep);
+              tma_load_2d_pair(st + 3 * kSuBytes + b * 8192, &tmV, sp.v_lo + nv + 64 * b, kb * UK, bar, pol_keep);
+            }
+          }
+        }
+      }
+    }
+  } else if (warp == 1) {
+    // ---------------- MMA issuer: one thread of the leader CTA ----------------
+    if (lane == 0 && rank == 0) {
+      const uint32_t idesc = (sp.fp16 ? umma_idesc_fp16(2 * UM, p.bn) : umma_idesc_bf16(2 * UM, p.bn)) | kIdescMnMajor;
+      const uint32_t d_main = tmem_base, d_cross = tmem_base + UN;
+      uint32_t it = 0, g = 0;
+      bool ok = true;
+      for (int tl = 0; tl < my_tiles && ok; ++tl) {
+        for (int kb = 0; kb < nk; ++kb, ++it) {
+          const uint32_t s = it % SU_STAGES, ph = (it / SU_STAGES) & 1;
+          const int kc = kb % SU_DRAIN;
+          if (!mbar_wait(&full[s], ph, abort_flag)) { ok = false; break; }
+          if (kc == 0 && !mbar_wait(mempty, (g & 1) ^ 1, abort_flag)) { ok = false; break; }
+          tc_fence_after();
+          uint8_t* st = smem + s * kSuStage;
+          const uint64_t duh = umma_desc_mn128(smem_u32(st)), dul = umma_desc_mn128(smem_u32(st + kSuBytes));
+          const uint64_t dvh = umma_desc_mn128(smem_u32(st + 2 * kSuBytes)), dvl = umma_desc_mn128(smem_u32(st + 3 * kSuBytes));
+#pragma unroll
+          for (int k = 0; k < UK / UMMA_K; ++k) {
+            const uint64_t adv = static_cast<uint64_t>(k * 2048 / 16);
+            umma_bf16_pair(d_main, duh + adv, dvh + adv, idesc, (kc | k) != 0 ? 1u : 0u);
+          }
+          if (kc == SU_DRAIN - 1 || kb + 1 == nk) {
+            umma_commit_pair(mfull, 3);
+            ++g;
+          }
+          if (kb == 0) {
+            if (!mbar_wait(cempty, (tl & 1) ^ 1, abort_flag)) { ok = false; break; }
+            tc_fence_after();
+          }
+#pragma unroll
+          for (int k = 0; k < UK / UMMA_K; ++k) {
+            const uint64_t adv = static_cast<uint64_t>(k * 2048 / 16);
+            umma_bf16_pair(d_cross, dul + adv, dvh + adv, idesc, (kb | k) != 0 ? 1u : 0u);
+            umma_bf16_pair(d_cross, duh + adv, dvl + adv, idesc, 1u);
+          }
+          umma_commit_pair(&empty[s], 3);
+        }
+        if (ok) umma_commit_pair(cfull, 3);
+      }
+    }
+  } else {
+    // ---------------- epilogue: warp (q, h) = TMEM lane quarter q, column half h ----------------
+    const int e = warp - 2, q = warp & 3, h = e >> 2;
+    uint8_t* sl = sRing + e * kSlotBytes;
+    const int cpw = half / kChunk;                   // chunks per warp and tile: 4 or 2
+    const uint64_t pol_w = policy_evict_normal();
+    const uint32_t mempty_leader = mapa_u32(smem_u32(mempty), 0), cempty_leader = mapa_u32(smem_u32(cempty), 0);
+    const int row_in_tile = static_cast<int>(rank) * UM + q * 32;
+    const uint32_t t_addr = tmem_base + (static_cast<uint32_t>(q * 32) << 16) + h * half;
+    bool ok = true;
+    auto issue_load = [&](int tl, int c) {           // (lane 0) chunk c of this pair's tile tl
+      if (tl >= my_tiles) return;
+      int m0, n0;
+      tile_origin(p, pair + tl * npairs, m0, n0);
+      mbar_expect_tx(&rfull[e], kSlotBytes);
+      tma_load_2d_hint(sl, &tmC, n0 + h * half + c * kChunk, m0 + row_in_tile, &rfull[e], pol_w);
+    };
+    if (lane == 0) issue_load(0, 0);
+    const float alpha = p.alpha * (sp.inv ? *sp.inv : 1.f);
+    uint32_t g = 0, r = 0;
+    for (int tl = 0; tl < my_tiles && ok; ++tl) {
+      int m0, n0;
+      tile_origin(p, pair + tl * npairs, m0, n0);
+      float sum[4][32];
+#pragma unroll
+      for (int c = 0; c < 4; ++c)
+#pragma unroll
+        for (int j = 0; j < 32; ++j) sum[c][j] = 0.f;
+      auto drain = [&](uint32_t at, float scale, uint32_t done) {     // sum += scale * the accumulator at column `at`
+        tc_fence_after();
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+          if (c >= cpw) break;
+          uint32_t acc[32];
+          tmem_ld_32x32(t_addr + at + c * kChunk, acc);
+          tmem_ld_wait();
+#pragma unroll
+          for (int j = 0; j < 32; ++j) sum[c][j] = fmaf(__uint_as_float(acc[j]), scale, sum[c][j]);
+        }
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive_cluster(done);
+      };
+      for (int kb = 0; kb < nk && ok; kb += SU_DRAIN, ++g) {
+        ok = __all_sync(0xffffffffu, mbar_wait(mfull, g & 1, abort_flag));
+        if (ok) drain(0, 1.f, mempty_leader);
+      }
+      if (ok) ok = __all_sync(0xffffffffu, mbar_wait(cfull, tl & 1, abort_flag));
+      if (!ok) break;
+      drain(UN, sp.lo_scale, cempty_leader);
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        if (c >= cpw || !ok) break;
+        const int x0 = n0 + h * half + c * kChunk, y0 = m0 + row_in_tile;
+        ok = __all_sync(0xffffffffu, mbar_wait(&rfull[e], r & 1, abort_flag));
+        if (!ok) break;
+        ++r;
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+          float4* wp = reinterpret_cast<float4*>(sl + lane * 128 + ((j ^ (lane & 7)) << 4));
+          float4 w = *wp;
+          w.x = fmaf(alpha, sum[c][4 * j + 0], w.x);
+          w.y = fmaf(alpha, sum[c][4 * j + 1], w.y);
+          w.z = fmaf(alpha, sum[c][4 * j + 2], w.z);
+          w.w = fmaf(alpha, sum[c][4 * j + 3], w.w);
+          if (p.prox_kind != 0) {
+            w.x = prox_entry(w.x, p.prox_kind, p.prox_a); w.y = prox_entry(w.y, p.prox_kind, p.prox_a);
+            w.z = prox_entry(w.z, p.prox_kind, p.prox_a); w.w = prox_entry(w.w, p.prox_kind, p.prox_a);
+          }
+          *wp = w;
+        }
+        fence_proxy_async_smem();
+        __syncwarp();
+        if (lane == 0) {
+          if (x0 < p.cols && y0 < p.rows) tma_store_2d_hint(&tmC, sl, x0, y0, pol_w);
+          tma_commit_group();
+          tma_wait_group_read<0>();                   // the slot has been read: the next chunk may land in it
+          issue_load(c + 1 < cpw ? tl : tl + 1, c + 1 < cpw ? c + 1 : 0);
+        }
+        __syncwarp();
+      }
+    }
+    if (lane == 0) tma_wait_group<0>();
+  }
+
+  // ---------------- teardown, as in update_pair_kernel ----------------
+  __syncwarp();
+  tc_fence_before();
+  __syncthreads();
+  if (*abort_flag) {
+    if (threadIdx.x == 0) atomicOr(p.status, SFB_STATUS_TIMEOUT);
+    for (int i = 0; i < 64; ++i) __nanosleep(1000);
+    __syncthreads();
+  }
+  cluster_arrive();
+  cluster_wait();
+  stamp_end(p.end);
+  if (warp == 1) { tc_fence_after(); tmem_dealloc_pair(tmem_base, kTmemCols); }
+}
+
 // Tile width: 128 where 256-wide tiles leave the pairs short of work.  Cycles of a tile: its k-blocks at the MMA or operand
-// rate (measured about 620 a k-block for 256 columns, 450 for 128) and its epilogue.
-int tile_width(int64_t rows, int64_t cols, int64_t kblocks, int pairs) {
+// rate (measured about 620 a k-block for 256 columns, 450 for 128; with four operand halves 1600 and 900) and its epilogue.
+int tile_width(int64_t rows, int64_t cols, int64_t kblocks, int pairs, bool split) {
   auto cost = [&](int bn) {
     const int64_t tiles = ((rows + 2 * UM - 1) / (2 * UM)) * ((cols + bn - 1) / bn);
-    return static_cast<double>((tiles + pairs - 1) / pairs) * (kblocks * (bn == 256 ? 620. : 450.) + (bn == 256 ? 2500. : 1800.));
+    const double kb = split ? (bn == 256 ? 1600. : 900.) : (bn == 256 ? 620. : 450.);
+    return static_cast<double>((tiles + pairs - 1) / pairs) * (kblocks * kb + (bn == 256 ? 2500. : 1800.));
   };
   return cost(128) < 0.97 * cost(256) ? 128 : 256;
 }
@@ -390,33 +629,33 @@ int tile_width(int64_t rows, int64_t cols, int64_t kblocks, int pairs) {
     }                                                   \
   } while (0)
 
-template <int SHADOW, bool TF32 = false>
-static cudaError_t prepare_kernel(int* max_pairs) {
-  cudaError_t e = cudaFuncSetAttribute(update_pair_kernel<SHADOW, TF32>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
+template <typename Kernel>
+static cudaError_t prepare_kernel(Kernel kernel, int smem, int* max_pairs) {
+  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3(2, 1, 1);
   cfg.blockDim = dim3(kThreads, 1, 1);
-  cfg.dynamicSmemBytes = kSmem;
+  cfg.dynamicSmemBytes = smem;
   cudaLaunchAttribute attr{};
   attr.id = cudaLaunchAttributeClusterDimension;
   attr.val.clusterDim.x = 2; attr.val.clusterDim.y = 1; attr.val.clusterDim.z = 1;
   cfg.attrs = &attr;
   cfg.numAttrs = 1;
   int n = 0;
-  e = cudaOccupancyMaxActiveClusters(&n, update_pair_kernel<SHADOW, TF32>, &cfg);
+  e = cudaOccupancyMaxActiveClusters(&n, kernel, &cfg);
   if (e != cudaSuccess) return e;
-  *max_pairs = n;
+  *max_pairs = std::min(*max_pairs, n);
   return cudaSuccess;
 }
 
 int tc_update_init(sfb_ctx* ctx, TcState* st) {
-  int a = 0, b = 0, t = 0;
-  CKC(prepare_kernel<1>(&a));
-  CKC(prepare_kernel<0>(&b));
-  CKC((prepare_kernel<2, true>(&t)));
-  st->max_pairs = std::min(std::min(a, b), t);
-  if (st->max_pairs < 1) return SFB_ERR_ARCH;     // the device cannot host a CTA pair of this kernel
+  int n = 1 << 30;
+  CKC(prepare_kernel(update_pair_kernel<1>, kSmem, &n));
+  CKC(prepare_kernel(update_split_kernel, kSuSmem, &n));
+  CKC(prepare_kernel(update_pair_kernel<2, true>, kSmem, &n));
+  st->max_pairs = n;
+  if (n < 1) return SFB_ERR_ARCH;                 // the device cannot host a CTA pair of these kernels
   return SFB_OK;
 }
 
@@ -459,7 +698,7 @@ int tc32_update(sfb_ctx* ctx) {
 }
 
 int tc_update(sfb_ctx* ctx) {
-  if (ctx->cfg.model == SFB_MLR) {
+  if (ctx->cfg.model == SFB_MLR && !ctx->h16) {
     const int rc = tc_labels(ctx);                     // the fp32 label entries, unless the factors call has applied them
     if (rc) return rc;
   }
@@ -467,12 +706,12 @@ int tc_update(sfb_ctx* ctx) {
   const sfb_config& c = ctx->cfg;
   TcState* st = static_cast<TcState*>(ctx->tc);
   const Layout& L = ctx->lay;
-  const bool split = c.model != SFB_MLR;
+  const bool split = c.model != SFB_MLR || ctx->h16;
   // U and V pair-major; the split products have (hi | lo) halves side by side
   const int64_t ldu = split ? 2 * L.rowsp : L.ldp, ldv = split ? 2 * L.colsp : L.colsb;
   const int64_t wu = split ? 2 * L.rowsp : c.rows, wv = split ? 2 * L.colsp : c.cols;
   __nv_bfloat16* U = ctx->at<__nv_bfloat16>(split ? L.Rs : L.P);
-  __nv_bfloat16* V = split ? tc_split_v(ctx) : ctx->at<__nv_bfloat16>(L.Xb);
+  void* V = split ? const_cast<uint16_t*>(split_v(ctx)) : ctx->at<uint16_t>(L.Xb);
   CUtensorMap ma, mb, mc;
   if (!make_map(st, &ma, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, U, wu, ctx->K, ldu * 2, 64, UK) ||
       !make_map(st, &mb, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, V, wv, ctx->K, ldv * 2, 64, UK) ||
@@ -482,7 +721,7 @@ int tc_update(sfb_ctx* ctx) {
   p.rows = static_cast<int32_t>(c.rows); p.cols = static_cast<int32_t>(c.cols);
   p.tilesM = static_cast<int32_t>((c.rows + 2 * UM - 1) / (2 * UM));
   p.kseg = static_cast<int32_t>((ctx->K + UK - 1) / UK);
-  p.bn = tile_width(c.rows, c.cols, (split ? 3 : 1) * p.kseg, st->max_pairs);
+  p.bn = tile_width(c.rows, c.cols, p.kseg, st->max_pairs, split);
   p.tilesN = static_cast<int32_t>((c.cols + p.bn - 1) / p.bn);
   p.begin = take_stamp(ctx); p.end = &ctx->at<Scalars>(L.scalars)->ns[3];
   p.alpha = -ctx->step;
@@ -491,12 +730,10 @@ int tc_update(sfb_ctx* ctx) {
   const int64_t tiles = static_cast<int64_t>(p.tilesM) * p.tilesN;
   const unsigned grid = 2u * static_cast<unsigned>(std::min<int64_t>(tiles, st->max_pairs));
   if (split) {
-    // U^T V = Uhi Vhi + Uhi Vlo + Ulo Vhi (+ Ulo Vlo, dropped: 2^-16 of the product)
-    p.nseg = 3;
-    p.a_off0 = 0; p.a_off1 = 0; p.a_off2 = static_cast<int32_t>(L.rowsp);
-    p.b_off0 = 0; p.b_off1 = static_cast<int32_t>(L.colsp); p.b_off2 = 0;
-    p.shadow = nullptr; p.shadow_ld = 0;
-    CKC(launch_kernel_if(tiles <= st->max_pairs, update_pair_kernel<0>, dim3(grid), dim3(kThreads), kSmem, ctx->stream, 1, ma, mb, mc, p));
+    SplitUpdParams sp{p, static_cast<int32_t>(L.rowsp), static_cast<int32_t>(L.colsp), ctx->h16, ctx->h16 ? 1.f / 2048.f : 1.f,
+                      ctx->h16 ? &ctx->at<Scalars>(L.scalars)->iU : nullptr};
+    CKC(launch_kernel_if(tiles <= st->max_pairs, update_split_kernel, dim3(grid), dim3(kThreads), kSuSmem, ctx->stream, 1, ma, mb,
+                         mc, sp));
     return SFB_OK;
   }
   p.nseg = 1;
