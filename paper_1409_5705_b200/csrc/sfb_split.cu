@@ -13,6 +13,8 @@
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
+#include <type_traits>
+
 #include "sfb_tc.h"
 #include "sfb_tile.cuh"
 
@@ -50,6 +52,8 @@ struct SplitParams {
   const float* aux;            // F_SUB: the matrix subtracted; F_ISTA, F_ISTAG: the matrix updated; [M x ldaux]
   int64_t ldaux;
   float* C2;                   // [M x ldc]
+  int32_t copies;              // F_SUB, F_ISTA, F_ISTAG: aux and C2 as tensor maps (16-byte pitch and address); the first row of
+  int32_t aux_row0;            // aux's map
   const Scalars* sc;           // F_ISTA*: 1 / L
   float lam;                   // F_ISTA*: lambda
   uint16_t* split;             // all but F_STORE: [M x ld_split] receives hi at column n and lo at column split_half + n
@@ -129,7 +133,9 @@ constexpr int kRegion = 192 << 10;                  // of the operand ring
 constexpr int kSlot = 32 * kChunk * 4;              // per epilogue warp: 32 rows x 32 columns of fp32
 constexpr int kDrain = 8;
 constexpr int kThreads = 128 + 32 * kEpi;
-constexpr int kBars = 2 * kStagesMax + 4;
+constexpr int kInputs = 3;                          // buffers per epilogue warp for what the end of the last tile reads
+static_assert((4 + kInputs - 1) * kEpi * kSlot <= kRegion, "see there");
+constexpr int kBars = 2 * kStagesMax + 4 + kEpi * kInputs;
 constexpr int kSmem = kRegion + kEpi * kSlot + kBars * 8 + 16 + 1024;
 constexpr int kTmemCols = 512;
 
@@ -202,6 +208,7 @@ struct Segments {
 template <int EPI, bool F16>
 __global__ void __launch_bounds__(kThreads, 1)
 split_product_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
+                     const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmY,
                      const __grid_constant__ SplitParams p) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -212,6 +219,7 @@ split_product_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
   uint64_t* mempty = mfull + 1;
   uint64_t* cfull = mfull + 2;
   uint64_t* cempty = mfull + 3;
+  uint64_t* ifull = mfull + 4;                       // per epilogue warp and buffer
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + kBars);
   volatile uint32_t* abort_flag = tmem_slot + 1;
 
@@ -228,6 +236,7 @@ split_product_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
     for (int i = 0; i < ST; ++i) { mbar_init(&full[i], 1); mbar_init(&empty[i], 1); }
     mbar_init(mfull, 1); mbar_init(mempty, 2 * kEpi);
     mbar_init(cfull, 1); mbar_init(cempty, 2 * kEpi);
+    for (int i = 0; i < kEpi * kInputs; ++i) mbar_init(&ifull[i], 1);
     *abort_flag = 0;
     fence_barrier_init();
     prefetch_tmap(&tmA); prefetch_tmap(&tmB);
@@ -323,87 +332,82 @@ split_product_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
     // of TMEM, every access touched 32 lines and the loads of an ISTA step waited for one another: 20 us at the end of each
     // product of 512 x 5,000.)
     const int rg = lane >> 3, cj = lane & 7;
-    auto finish = [&](int m0, int n0, int c) {
-      const int col0 = n0 + c * kChunk, col = col0 + 4 * cj;
-      if (col0 >= p.N) return;
-      const int row = m0 + row0 + rg;
-      const int nv = (p.M - row + 3) >> 2;                          // of the lane's rows row + 4 e inside the matrix
-      const bool in4 = col + 4 <= p.N;
-      float4 x[8], b[8];
-      float fa[8], so[8];
-      if constexpr (EPI == F_SUB || EPI == F_ISTA || EPI == F_ISTAG) {
-        const float* ap = p.aux + static_cast<int64_t>(row) * p.ldaux + col;
-        const bool vec = in4 && (reinterpret_cast<uintptr_t>(ap) & 15u) == 0;
-#pragma unroll
-        for (int e = 0; e < 8; ++e, ap += 4 * p.ldaux) {
-          x[e] = make_float4(0.f, 0.f, 0.f, 0.f);
-          if (e >= nv) continue;
-          if (vec) {
-            x[e] = *reinterpret_cast<const float4*>(ap);
-          } else {
-            if (col < p.N) x[e].x = ap[0];
-            if (col + 1 < p.N) x[e].y = ap[1];
-            if (col + 2 < p.N) x[e].z = ap[2];
-            if (col + 3 < p.N) x[e].w = ap[3];
-          }
-        }
-      }
-      // W^T x of the samples (N, hence every pitch, is a multiple of 4 for the products over atoms)
-      float* bp = EPI == F_ISTAG || EPI == F_ISTA0 ? p.C2 : nullptr;
-      if (bp) bp += static_cast<int64_t>(row) * p.ldc + col;
-      if constexpr (EPI == F_ISTAG) {
-#pragma unroll
-        for (int e = 0; e < 8; ++e) {
-          b[e] = make_float4(0.f, 0.f, 0.f, 0.f);
-          if (e < nv && in4) b[e] = *reinterpret_cast<const float4*>(bp + e * 4 * p.ldc);
-        }
-      }
-      float4 fb = make_float4(1.f, 1.f, 1.f, 1.f);
+    constexpr bool kAux = EPI == F_SUB || EPI == F_ISTA || EPI == F_ISTAG;
+    // Four columns of a row: the factors, what the epilogue does, the result and its pair.
+    struct Place { int col; bool in4; float4 fb; };
+    auto place = [&](int n0, int c) {
+      Place o;
+      o.col = n0 + c * kChunk + 4 * cj;
+      o.in4 = o.col + 4 <= p.N;
+      o.fb = make_float4(1.f, 1.f, 1.f, 1.f);
       if constexpr (F16) {
-        if (p.ib) fb = *reinterpret_cast<const float4*>(p.ib + col);                    // (padded to whole chunks)
-        const float all = p.iab ? *p.iab : 1.f;
-        fb = make_float4(fb.x * all, fb.y * all, fb.z * all, fb.w * all);
-        const float one = EPI == F_GRAM ? *p.ios : 1.f;
-#pragma unroll
-        for (int e = 0; e < 8; ++e) {
-          fa[e] = p.ia && e < nv ? p.ia[row + 4 * e] : 1.f;
-          if constexpr (EPI != F_STORE) so[e] = __frcp_rn(p.io && e < nv ? p.io[row + 4 * e] : one);
+        if (p.ib) o.fb = *reinterpret_cast<const float4*>(p.ib + o.col);                // (padded to whole chunks)
+        if (p.iab) o.fb = scale4(o.fb, *p.iab);
+      }
+      return o;
+    };
+    auto put = [&](const Place& o, int row, float4 v, const float4& x, const float4& b) {
+      float so = 1.f;
+      if constexpr (F16) {
+        if (p.ia) v = scale4(v, p.ia[row]);
+        v = make_float4(v.x * o.fb.x, v.y * o.fb.y, v.z * o.fb.z, v.w * o.fb.w);
+        if constexpr (EPI != F_STORE) so = __frcp_rn(p.io ? p.io[row] : *p.ios);
+      }
+      // (N, hence every pitch, is a multiple of 4 for the products over atoms)
+      if constexpr (EPI == F_ISTAG) v = make_float4(v.x - b.x, v.y - b.y, v.z - b.z, v.w - b.w);
+      if constexpr (EPI == F_ISTA0) {
+        if (p.C2 && o.in4) *reinterpret_cast<float4*>(p.C2 + static_cast<int64_t>(row) * p.ldc + o.col) = v;
+        v = make_float4(soft_threshold(v.x * invL, thr), soft_threshold(v.y * invL, thr), soft_threshold(v.z * invL, thr),
+                        soft_threshold(v.w * invL, thr));
+      }
+      if constexpr (EPI == F_SUB) v = make_float4(v.x - x.x, v.y - x.y, v.z - x.z, v.w - x.w);
+      if constexpr (EPI == F_ISTA || EPI == F_ISTAG)
+        v = make_float4(soft_threshold(fmaf(-v.x, invL, x.x), thr), soft_threshold(fmaf(-v.y, invL, x.y), thr),
+                        soft_threshold(fmaf(-v.z, invL, x.z), thr), soft_threshold(fmaf(-v.w, invL, x.w), thr));
+      if (p.C) {
+        float* to = p.C + static_cast<int64_t>(row) * p.ldc + o.col;
+        if (o.in4) {                                                // (its pitch is a multiple of 4)
+          *reinterpret_cast<float4*>(to) = v;
+        } else {
+          if (o.col < p.N) to[0] = v.x;
+          if (o.col + 1 < p.N) to[1] = v.y;
+          if (o.col + 2 < p.N) to[2] = v.z;
         }
       }
-      uint16_t* hp = EPI == F_STORE ? nullptr : p.split + static_cast<int64_t>(row) * p.ld_split + col;
-      float* cp = p.C ? p.C + static_cast<int64_t>(row) * p.ldc + col : nullptr;
+      if constexpr (EPI != F_STORE) {                // the operand of the next product, zero in the padding past N
+        if (o.col < p.split_half) {
+          if (!o.in4) v = make_float4(o.col < p.N ? v.x : 0.f, o.col + 1 < p.N ? v.y : 0.f, o.col + 2 < p.N ? v.z : 0.f, 0.f);
+          put_pair4<F16>(p.split + static_cast<int64_t>(row) * p.ld_split + o.col, p.split_half, F16 ? scale4(v, so) : v);
+        }
+      }
+    };
+    // A chunk from shared memory, with loads of what else it reads.
+    auto finish = [&](int m0, int n0, int c, uint32_t from) {
+      if (n0 + c * kChunk >= p.N) return;
+      const Place o = place(n0, c);
+      const int row = m0 + row0 + rg, nv = (p.M - row + 3) >> 2;    // nv: of the lane's rows row + 4 e inside the matrix
+      float4 x[8], b[8];
 #pragma unroll
       for (int e = 0; e < 8; ++e) {
+        x[e] = b[e] = make_float4(0.f, 0.f, 0.f, 0.f);
         if (e >= nv) continue;
-        float4 v = ld_shared_f4(slot_addr(slot, rg + 4 * e, cj));
-        if constexpr (F16) v = make_float4(v.x * fa[e] * fb.x, v.y * fa[e] * fb.y, v.z * fa[e] * fb.z, v.w * fa[e] * fb.w);
-        if constexpr (EPI == F_ISTAG) v = make_float4(v.x - b[e].x, v.y - b[e].y, v.z - b[e].z, v.w - b[e].w);
-        if constexpr (EPI == F_ISTA0) {
-          if (bp && in4) *reinterpret_cast<float4*>(bp + e * 4 * p.ldc) = v;
-          v = make_float4(soft_threshold(v.x * invL, thr), soft_threshold(v.y * invL, thr), soft_threshold(v.z * invL, thr),
-                          soft_threshold(v.w * invL, thr));
-        }
-        if constexpr (EPI == F_SUB) v = make_float4(v.x - x[e].x, v.y - x[e].y, v.z - x[e].z, v.w - x[e].w);
-        if constexpr (EPI == F_ISTA || EPI == F_ISTAG)
-          v = make_float4(soft_threshold(fmaf(-v.x, invL, x[e].x), thr), soft_threshold(fmaf(-v.y, invL, x[e].y), thr),
-                          soft_threshold(fmaf(-v.z, invL, x[e].z), thr), soft_threshold(fmaf(-v.w, invL, x[e].w), thr));
-        if (cp) {
-          float* o = cp + e * 4 * p.ldc;
-          if (in4) {                                                // (pitches are multiples of 4)
-            *reinterpret_cast<float4*>(o) = v;
+        if constexpr (kAux) {
+          const float* ap = p.aux + static_cast<int64_t>(row + 4 * e) * p.ldaux + o.col;
+          if (o.in4 && (reinterpret_cast<uintptr_t>(ap) & 15u) == 0) {
+            x[e] = *reinterpret_cast<const float4*>(ap);
           } else {
-            if (col < p.N) o[0] = v.x;
-            if (col + 1 < p.N) o[1] = v.y;
-            if (col + 2 < p.N) o[2] = v.z;
+            if (o.col < p.N) x[e].x = ap[0];
+            if (o.col + 1 < p.N) x[e].y = ap[1];
+            if (o.col + 2 < p.N) x[e].z = ap[2];
+            if (o.col + 3 < p.N) x[e].w = ap[3];
           }
         }
-        if constexpr (EPI != F_STORE) {              // the operand of the next product, zero in the padding past N
-          if (col < p.split_half) {
-            if (!in4) v = make_float4(col < p.N ? v.x : 0.f, col + 1 < p.N ? v.y : 0.f, col + 2 < p.N ? v.z : 0.f, 0.f);
-            put_pair4<F16>(hp + e * 4 * p.ld_split, p.split_half, F16 ? scale4(v, so[e]) : v);
-          }
-        }
+        if (EPI == F_ISTAG && o.in4)
+          b[e] = *reinterpret_cast<const float4*>(p.C2 + static_cast<int64_t>(row + 4 * e) * p.ldc + o.col);
       }
+#pragma unroll
+      for (int e = 0; e < 8; ++e)
+        if (e < nv) put(o, row + 4 * e, ld_shared_f4(slot_addr(from, rg + 4 * e, cj)), x[e], b[e]);
     };
     // F_GRAM: the mirror images of the entries whose own tile is not formed; a row per lane makes neighbouring columns there.
     auto mirror = [&](const uint32_t (&acc)[32], int m0, int n0, int c) {
@@ -434,19 +438,6 @@ split_product_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
       const int nk = sg.k1 - sg.k0;
       int m0, n0;
       tile_coords<EPI>(p, sg.tile, m0, n0);
-      if ((EPI == F_SUB || EPI == F_ISTA || EPI == F_ISTAG) && sg.k1 == p.kseg) {      // what the end of the tile reads, into L2
-        const int64_t row = m0 + row0 + lane;
-        for (int c = h; c < chunks && row < p.M; c += 2) {
-          const int col = n0 + c * kChunk;
-          if (col + kChunk > p.N) break;
-          prefetch_l2(p.aux + row * p.ldaux + col);
-          prefetch_l2(p.aux + row * p.ldaux + col + kChunk - 1);
-          if (EPI == F_ISTAG) {
-            prefetch_l2(p.C2 + row * p.ldc + col);
-            prefetch_l2(p.C2 + row * p.ldc + col + kChunk - 1);
-          }
-        }
-      }
       float sum[4][32];                              // chunks h, h + 2, h + 4, h + 6
 #pragma unroll
       for (int i = 0; i < 4; ++i)
@@ -476,51 +467,140 @@ split_product_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
       if (!ok) break;
       drain(kMaxN, F16 ? 1.f / kLoScale : 1.f, cempty_leader);
       const int at = static_cast<int>(rank) * kEpi + warp - 4;
-      if (sg.k1 < p.kseg) {                          // the rest of the tile is another pair's: leave it the sums
-        float4* out = reinterpret_cast<float4*>(p.partial) + (static_cast<int64_t>(pair) * 2 * kEpi + at) * 1024 + lane;
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          if (h + 2 * i >= chunks) break;
-#pragma unroll
-          for (int j = 0; j < 8; ++j)
-            out[i * 256 + j * 32] = make_float4(sum[i][4 * j], sum[i][4 * j + 1], sum[i][4 * j + 2], sum[i][4 * j + 3]);
-        }
-        __threadfence();
-        __syncwarp();
-        if (lane == 0) st_release(p.ready + pair * 2 * kEpi + at, 1u);
-        continue;
-      }
-      for (int from = segs.first_part(sg); from < pair && ok; ++from) {
-        uint32_t* flag = p.ready + from * 2 * kEpi + at;
-        ok = __all_sync(0xffffffffu, lane != 0 || flag_wait(flag, abort_flag));
-        if (!ok) break;
-        const float4* in = reinterpret_cast<const float4*>(p.partial) + (static_cast<int64_t>(from) * 2 * kEpi + at) * 1024 + lane;
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          if (h + 2 * i >= chunks) break;
-          float4 v[8];
-#pragma unroll
-          for (int j = 0; j < 8; ++j) v[j] = __ldcg(in + i * 256 + j * 32);
-#pragma unroll
-          for (int j = 0; j < 8; ++j) {
-            sum[i][4 * j] += v[j].x; sum[i][4 * j + 1] += v[j].y; sum[i][4 * j + 2] += v[j].z; sum[i][4 * j + 3] += v[j].w;
-          }
-        }
-        __syncwarp();
-        if (lane == 0) *flag = 0;                    // for the next launch
-      }
-      if (!ok) break;
-#pragma unroll 1
-      for (int i = 0; h + 2 * i < chunks; ++i) {
+      auto chunk_to_slot = [&](int i) {
         uint32_t acc[32];
 #pragma unroll
         for (int j = 0; j < 32; ++j)
           acc[j] = __float_as_uint(i == 0 ? sum[0][j] : i == 1 ? sum[1][j] : i == 2 ? sum[2][j] : sum[3][j]);
-        const int c = h + 2 * i;
-        if (EPI == F_GRAM) mirror(acc, m0, n0, c);
         slot_put(slot, lane, acc);
+      };
+      if (sg.k1 < p.kseg) {                          // the rest of the tile is another pair's: leave it the sums
+        float* out = p.partial + (static_cast<int64_t>(pair) * 2 * kEpi + at) * 4 * (kSlot / 4);
+#pragma unroll 1
+        for (int i = 0; h + 2 * i < chunks; ++i) {
+          chunk_to_slot(i);
+          fence_proxy_async_smem();
+          __syncwarp();
+          if (lane == 0) { bulk_store(out + i * (kSlot / 4), slot, kSlot); tma_commit_group(); tma_wait_group_read<0>(); }
+          __syncwarp();
+        }
+        if (lane == 0) {
+          tma_wait_group<0>();
+          fence_proxy_async_all();
+          __threadfence();
+          st_release(p.ready + pair * 2 * kEpi + at, 1u);
+        }
+        continue;
+      }
+      if (EPI != F_GRAM && sgi + 1 == segs.n) {
+        // The last tile, the one that may take parts from other pairs.  Nothing uses the operand ring any more: its memory takes
+        // the sums and, with the slot, what the end of the tile reads -- per chunk the parts, aux, C2 -- by bulk copies, kInputs
+        // of them under way per warp.
+        // (Loads go through what is left of L1, 28 KB, which held them to 14 bytes per cycle: 30,000 cycles at the end of an
+        // ISTA step of 512 x 5,000, 27,000 to add up five parts.)
+        const int from = segs.first_part(sg), parts = pair - from;
+        const bool copies = kAux && p.copies;
+        constexpr int kAfter = EPI == F_ISTAG ? 2 : 1;
+        const int per = parts + (copies ? kAfter : 0);
+        int mine = 0;
+        while (mine < 4 && h + 2 * mine < chunks && n0 + (h + 2 * mine) * kChunk < p.N) ++mine;
+        const uint32_t room = smem_u32(smem) + (warp - 4) * (4 + kInputs - 1) * kSlot;
+        auto buffer = [&](int k) { return k % kInputs == 0 ? slot : room + (3 + k % kInputs) * kSlot; };
+        uint64_t* bar = ifull + (warp - 4) * kInputs;
+        for (int j = from; j < pair && ok; ++j) ok = __all_sync(0xffffffffu, lane != 0 || flag_wait(p.ready + j * 2 * kEpi + at, abort_flag));
+        if (!ok) break;
+        int asked = 0, taken = 0;                    // copies
+        auto ask = [&]() {                           // (lane 0) the next one
+          if (asked >= mine * per) return;
+          const int i = asked / per, w = asked - i * per, buf = asked % kInputs;
+          const uint32_t to = buffer(asked);
+          const int x0 = n0 + (h + 2 * i) * kChunk;
+          mbar_expect_tx(&bar[buf], kSlot);
+          if (w < parts) bulk_load(to, p.partial + ((static_cast<int64_t>(from + w) * 2 * kEpi + at) * 4 + i) * (kSlot / 4), kSlot, &bar[buf]);
+          else if (w == parts) tma_load_2d_at(to, &tmX, x0, m0 + row0 - p.aux_row0, &bar[buf]);
+          else tma_load_2d_at(to, &tmY, x0, m0 + row0, &bar[buf]);
+          ++asked;
+        };
+        auto take = [&](int ahead) {                 // waits for the copy `ahead` places on; where it is
+          const int k = taken + ahead;
+          ok = ok && __all_sync(0xffffffffu, mbar_wait(&bar[k % kInputs], (k / kInputs) & 1, abort_flag));
+          return buffer(k);
+        };
+        auto give = [&](int n) {                     // their buffers are free
+          __syncwarp();
+          taken += n;
+          if (lane == 0) for (int k = 0; k < n; ++k) ask();
+        };
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          if (i >= mine) break;
+          uint32_t acc[32];
+#pragma unroll
+          for (int j = 0; j < 32; ++j) acc[j] = __float_as_uint(sum[i][j]);
+          slot_put(room + i * kSlot, lane, acc);
+        }
         __syncwarp();
-        finish(m0, n0, c);
+        if (lane == 0) {
+          for (int j = from; j < pair; ++j) p.ready[j * 2 * kEpi + at] = 0;             // for the next launch
+          fence_proxy_async_all();
+          for (int k = 0; k < kInputs; ++k) ask();
+        }
+#pragma unroll 1
+        for (int i = 0; i < mine && ok; ++i) {
+          const uint32_t own = room + i * kSlot;
+          const Place o = place(n0, h + 2 * i);
+          const int row = m0 + row0 + rg, nv = (p.M - row + 3) >> 2;
+          float4 v[8];
+#pragma unroll
+          for (int e = 0; e < 8; ++e) v[e] = ld_shared_f4(slot_addr(own, rg + 4 * e, cj));
+          for (int w = 0; w < parts && ok; ++w) {
+            const uint32_t a = take(0);
+            if (!ok) break;
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+              const float4 t = ld_shared_f4(slot_addr(a, rg + 4 * e, cj));
+              v[e] = make_float4(v[e].x + t.x, v[e].y + t.y, v[e].z + t.z, v[e].w + t.w);
+            }
+            give(1);
+          }
+          if (!ok) break;
+          const float4 none = make_float4(0.f, 0.f, 0.f, 0.f);
+          if (!kAux) {
+#pragma unroll
+            for (int e = 0; e < 8; ++e)
+              if (e < nv) put(o, row + 4 * e, v[e], none, none);
+          } else if (copies) {
+            const uint32_t xa = take(0), ba = kAfter > 1 ? take(1) : 0;
+            if (!ok) break;
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+              const float4 x = ld_shared_f4(slot_addr(xa, rg + 4 * e, cj));
+              const float4 b = kAfter > 1 ? ld_shared_f4(slot_addr(ba, rg + 4 * e, cj)) : none;
+              if (e < nv) put(o, row + 4 * e, v[e], x, b);
+            }
+            give(kAfter);
+          } else {
+#pragma unroll
+            for (int e = 0; e < 8; ++e) st_shared_f4(slot_addr(own, rg + 4 * e, cj), v[e]);
+            __syncwarp();
+            finish(m0, n0, h + 2 * i, own);
+          }
+        }
+        break;
+      }
+#pragma unroll 1
+      for (int i = 0; h + 2 * i < chunks; ++i) {
+        const int c = h + 2 * i;
+        if (EPI == F_GRAM) {
+          uint32_t acc[32];
+#pragma unroll
+          for (int j = 0; j < 32; ++j)
+            acc[j] = __float_as_uint(i == 0 ? sum[0][j] : i == 1 ? sum[1][j] : i == 2 ? sum[2][j] : sum[3][j]);
+          mirror(acc, m0, n0, c);
+        }
+        chunk_to_slot(i);
+        __syncwarp();
+        finish(m0, n0, c, slot);
         __syncwarp();
       }
     }
@@ -829,7 +909,7 @@ ProductPlan plan_width(int64_t M, int64_t N, int64_t Kc, bool sym, int bn, int64
   if (rest > 0) {
     const int64_t pairs = rounds > 0 ? max_pairs : std::max<int64_t>(1, std::min(max_pairs, rest * kseg / 4));
     const double cut = static_cast<double>(rounds * kseg + (rest * kseg + pairs - 1) / pairs);
-    if (rounds == 0 && (kb - cut) * per_kb > 8000.0 && rest * kseg >= 4 * pairs) {
+    if (!sym && rounds == 0 && (kb - cut) * per_kb > 8000.0) {
       p.whole = rounds * max_pairs;
       p.pairs = pairs;
       kb = cut + 8000.0 / per_kb;
@@ -864,6 +944,13 @@ int split_product(sfb_ctx* ctx, int64_t off, int64_t n, const uint16_t* A, const
   if (!make_map(st, &ma, CU_TENSOR_MAP_DATA_TYPE_UINT16, const_cast<uint16_t*>(A), 2 * Cp, off + n, 2 * Cp * 2, BK, p.a_rows) ||
       !make_map(st, &mb, CU_TENSOR_MAP_DATA_TYPE_UINT16, const_cast<uint16_t*>(B), 2 * Cp, N, 2 * Cp * 2, BK, p.bn / 2))
     return SFB_ERR_CUDA;
+  // aux ends with the last sample of this call; C2 covers all of them
+  CUtensorMap mx = ma, my = ma;
+  p.copies = p.aux && ((reinterpret_cast<uintptr_t>(p.aux + p.aux_row0 * p.ldaux) | static_cast<uintptr_t>(p.ldaux * 4)) & 15u) == 0;
+  if (p.copies && !make_map(st, &mx, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, const_cast<float*>(p.aux + p.aux_row0 * p.ldaux), N,
+                            off + n - p.aux_row0, p.ldaux * 4, kChunk, 32))
+    return SFB_ERR_CUDA;
+  if (EPI == F_ISTAG && !make_map(st, &my, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, p.C2, N, off + n, p.ldc * 4, kChunk, 32)) return SFB_ERR_CUDA;
   p.M = static_cast<int32_t>(off + n); p.N = static_cast<int32_t>(N);
   p.m_off = static_cast<int32_t>(off);
   p.tilesM = static_cast<int32_t>((n + PM - 1) / PM);
@@ -874,7 +961,7 @@ int split_product(sfb_ctx* ctx, int64_t off, int64_t n, const uint16_t* A, const
   if (plan.tiles <= 0) return SFB_OK;
   CKC((allow_smem<split_product_kernel<EPI, F16>>(kSmem)));
   CKC(launch_kernel_if(plan.tiles <= st->max_pairs, split_product_kernel<EPI, F16>, dim3(static_cast<unsigned>(2 * plan.pairs)),
-                       dim3(kThreads), kSmem, ctx->stream, 2, ma, mb, p));
+                       dim3(kThreads), kSmem, ctx->stream, 2, ma, mb, mx, my, p));
   ctx->stats.flops += (EPI == F_GRAM ? 3.0 : 6.0) * n * N * Cp;
   return SFB_OK;
 }
@@ -922,7 +1009,7 @@ int factors_sc(sfb_ctx* ctx, int64_t off, int64_t n, const float* X) {
   auto residual = [&](uint16_t* a) {                                                    // r = W a - x
     SplitParams q{};
     q.C = ctx->at<float>(L.U); q.ldc = L.ldu;
-    q.aux = X - off * rows; q.ldaux = rows;          // X holds this worker's samples: index it by the global row
+    q.aux = X - off * rows; q.ldaux = rows; q.aux_row0 = static_cast<int32_t>(off);          // X holds this worker's samples: index it by the global row
     q.split = Rs; q.ld_split = 2 * L.rowsp; q.split_half = static_cast<int32_t>(L.rowsp);
     if (F16) { q.ia = iC; q.ib = ctx->at<float>(L.iW); q.io = iR; }
     return split_product<F_SUB, F16>(ctx, off, n, a, Ws, rows, L.colsp, q);
