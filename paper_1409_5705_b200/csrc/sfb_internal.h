@@ -136,13 +136,18 @@ inline int64_t round_up(int64_t x, int64_t m) { return (x + m - 1) / m * m; }
 
 // Which kernels the products of an fp32 mode run on.  Pairs of tf32 words when asked for (logistic models).  SFB_PREC_FP32 runs
 // on pairs of fp16 words with fp32 scales (sfb_split.cu) where the products are large enough to repay the packing of their
-// operands, else on the FMA kernels: below about 10^8 multiply-adds a step is launches either way.
+// operands (W once per step, as much work as 24 more pairs), else on the FMA kernels.  us per step, fp16 pairs / FMAs: sparse
+// coding 2,000 x 1,000 K = 128 459 / 425, 6,000 x 3,000 K = 16 1242 / 2568; metric learning 300 x 1,000 K = 500 55 / 49,
+// 500 x 4,000 K = 100 66 / 77; regression 2,000 x 5,000 K = 16 128 / 90, 3,000 x 600 K = 130 50 / 64, 10,000 x 20,000 K = 16
+// 1306 / 1583, 50,000 x 64 K = 256 192 / 148 (bound by u, which is packed too).
 inline bool use_tf32(const sfb_config& c) {
   return c.precision == SFB_PREC_TF32X3 && (c.model == SFB_MLR || c.model == SFB_L2MLR);
 }
 inline bool use_h16(const sfb_config& c) {
-  return c.precision == SFB_PREC_FP32 && c.rows >= 64 && c.cols >= 64 &&
-         static_cast<double>(c.workers) * c.batch * static_cast<double>(c.rows) * static_cast<double>(c.cols) >= 1e8;
+  if (c.precision != SFB_PREC_FP32 || c.rows < 64 || c.cols < 64) return false;
+  const double K = static_cast<double>(c.workers) * c.batch, macs = K * static_cast<double>(c.rows) * static_cast<double>(c.cols);
+  if (c.model == SFB_SC) return macs >= 2.8e8;
+  return c.cols >= 256 && (macs >= 1e9 || macs * (1.0 - 24.0 / K) >= 1.8e8);
 }
 
 struct Scalars {                      // device-resident scalars
