@@ -408,7 +408,7 @@ static int compute_factors_csr(sfb_ctx* ctx, int32_t worker, const int64_t* indp
   if (rc) return rc;
   const float* X = ctx->at<float>(ctx->lay.stageX) + off * c.cols;
   rc = ctx->tf32 ? tc32_factors(ctx, off, n, X, labels_dev, nullptr, 0.f)
-       : c.precision == SFB_PREC_FP32 ? factors_fp32(ctx, off, n, X, nullptr, labels_dev, !ctx->h16 && sparse_forward_rows(ctx, n) > 0)
+       : c.precision == SFB_PREC_FP32 ? factors_fp32(ctx, off, n, X, nullptr, labels_dev, sparse_forward_wanted(ctx, n))
                                       : tc_factors(ctx, off, n, X, nullptr, labels_dev, fused);
   if (rc) return rc;
   ctx->csr_fill += nnz;

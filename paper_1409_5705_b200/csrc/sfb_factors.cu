@@ -61,7 +61,7 @@ __device__ __forceinline__ float block_max(float v, float* sh) {
 __global__ void pack_kernel(float* __restrict__ dst, const float* __restrict__ x, const float* __restrict__ y,
                             int64_t n4, int64_t n, const Stamp st) {
   pdl_launch_dependents();
-  pdl_wait(x, y);
+  pdl_wait();
   stamp_begin(st);
   const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
   for (int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; i < n4; i += stride) {
@@ -93,7 +93,7 @@ __global__ void prox_entries_kernel(float* __restrict__ w, int64_t n, int kind, 
 
 __global__ void axpy_kernel(float* __restrict__ y, const float* __restrict__ x, float alpha, int64_t n) {
   pdl_launch_dependents();
-  pdl_wait(x);
+  pdl_wait();
   const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
   for (int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; i < n; i += stride)
     y[i] = fmaf(alpha, x[i], y[i]);
@@ -141,7 +141,7 @@ __global__ void __launch_bounds__(NTHREADS) mlr_shard_partials_kernel(const floa
                                                                       const int32_t* __restrict__ labels, int64_t row_off,
                                                                       float4* __restrict__ part) {
   pdl_launch_dependents();
-  pdl_wait(Z, labels);
+  pdl_wait(labels);
   __shared__ float sh[32];
   const float* z = Z + static_cast<int64_t>(blockIdx.x) * ldz;
   float m = -INFINITY;
@@ -410,7 +410,7 @@ __global__ void __launch_bounds__(NTHREADS) dml_scale_kernel(float* __restrict__
 
 __global__ void mean_kernel(const float* __restrict__ v, int64_t n, float* out, const Stamp st) {
   pdl_launch_dependents();
-  pdl_wait(v);
+  pdl_wait();
   stamp_begin(st);
   __shared__ float sh[32];
   float s = 0.f;
@@ -424,7 +424,7 @@ __global__ void mean_kernel(const float* __restrict__ v, int64_t n, float* out, 
 __global__ void __launch_bounds__(kThreads) col_sumsq_kernel(const float* __restrict__ W, int64_t rows, int64_t cols,
                                                              double* __restrict__ part, int64_t slab_rows) {
   pdl_launch_dependents();
-  pdl_wait(W);
+  pdl_wait();
   __shared__ double sh[8][128];
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
   const int64_t c0 = static_cast<int64_t>(blockIdx.x) * 128 + tx * 4;

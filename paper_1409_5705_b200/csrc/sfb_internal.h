@@ -321,7 +321,8 @@ bool sparse_update_wanted(const sfb_ctx* ctx);
 int sparse_stage(sfb_ctx* ctx, int64_t off, int64_t n, const int64_t* indptr, const int32_t* idx, const float* val,
                  int64_t nnz);
 // fp32 FMA mode: rows of W per block of the row-wise forward over sparse samples (0: the rows do not fit), and that product
-int sparse_forward_rows(const sfb_ctx* ctx, int64_t n);
+bool sparse_forward_wanted(const sfb_ctx* ctx, int64_t n);
+double gemm_cycles(int64_t M, int64_t N, int64_t Kc);               // of a product on the FMA kernels
 int sparse_forward(sfb_ctx* ctx, int64_t off, int64_t n, float* Z, int64_t ldz);
 int sparse_build_csc(sfb_ctx* ctx);
 int sparse_update(sfb_ctx* ctx);

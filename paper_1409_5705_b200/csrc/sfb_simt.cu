@@ -341,6 +341,11 @@ GemmShape pick_gemm_shape(int64_t M, int64_t N, int64_t Kc, bool sym) {
   return best;
 }
 
+double gemm_cycles(int64_t M, int64_t N, int64_t Kc) {
+  const GemmShape g = pick_gemm_shape(M, N, Kc);
+  return std::min(gemm_cost(128, g.split, M, N, Kc, false), gemm_cost(64, g.split, M, N, Kc, false));
+}
+
 cudaError_t sgemm(cudaStream_t s, bool a_kc, bool b_kc, Epilogue epi, int64_t M, int64_t N, int64_t Kc,
                   const float* A, int64_t lda, const float* B, int64_t ldb, const EpiArgs& e, int64_t M_split) {
 #define SFB_GO(AK, BK_, E) return launch<AK, BK_, E>(s, M, N, Kc, A, lda, B, ldb, e, M_split)

@@ -70,7 +70,7 @@ __global__ void __launch_bounds__(256) csr_stage_kernel(const int64_t* __restric
                                                         int32_t* __restrict__ row_beg,
                                                         int32_t* __restrict__ row_end, uint32_t* __restrict__ status) {
   pdl_launch_dependents();
-  pdl_wait(indptr, idx, val);
+  pdl_wait();
   const int64_t i = (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (i >= n) return;
@@ -111,7 +111,7 @@ __global__ void __launch_bounds__(256) csr_stage_kernel(const int64_t* __restric
 // ---------------------------------------------------------------------------------------------------------
 __global__ void __launch_bounds__(256) csc_count_kernel(const int32_t* __restrict__ coo_c, int64_t nnz, int32_t* __restrict__ cnt) {
   pdl_launch_dependents();
-  pdl_wait(coo_c);
+  pdl_wait();
   const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
   for (int64_t t = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; t < nnz; t += stride) {
     const int32_t c = coo_c[t];
@@ -149,7 +149,7 @@ __global__ void __launch_bounds__(256) csc_fill_kernel(const int32_t* __restrict
                                                        const int32_t* __restrict__ ptr, int32_t* __restrict__ cur,
                                                        int2* __restrict__ tmp) {
   pdl_launch_dependents();
-  pdl_wait(coo_i, coo_c, coo_x, ptr);
+  pdl_wait(ptr);
   const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
   for (int64_t t = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; t < nnz; t += stride) {
     const int32_t c = coo_c[t];
@@ -164,7 +164,7 @@ __global__ void __launch_bounds__(128) csc_sort_kernel(const int2* __restrict__ 
                                                        const int32_t* __restrict__ cnt, int64_t cols, int32_t K,
                                                        int2* __restrict__ ent) {
   pdl_launch_dependents();
-  pdl_wait(tmp, ptr, cnt);
+  pdl_wait(ptr, cnt);
   for (int64_t d = blockIdx.x; d < cols; d += gridDim.x) {
     const int32_t n = cnt[d], b = ptr[d];
     for (int32_t e = threadIdx.x; e < n; e += blockDim.x) {
@@ -224,7 +224,7 @@ __global__ void __launch_bounds__(kSfThreads, 1) sparse_forward_kernel(const flo
                                                                        const int2* __restrict__ cx, int64_t off, int32_t n,
                                                                        float* __restrict__ Z, int64_t ldz) {
   pdl_launch_dependents();
-  pdl_wait(W, row_beg, row_end, cx);
+  pdl_wait();
   extern __shared__ __align__(16) uint8_t sf_smem[];
   constexpr int EP = 32 / RB;                        // entries of a sample worked on at once
   float* ws = reinterpret_cast<float*>(sf_smem);     // RB rows of W, row pitch `pitch` floats
@@ -613,6 +613,21 @@ int sparse_forward_rows(const sfb_ctx* ctx, int64_t n) {
     if (bytes <= kSmemOptIn) return rb;
   }
   return 0;
+}
+
+// Whether the row-wise forward is faster than the FMA product over the scattered samples, both in SM cycles.  Row-wise: a block's
+// 16 warps take the samples in turn, 900 cycles each and 40 more per entry and lane group, for rb rows of W at a time.
+// 91,238 x 148, K = 176, 13 entries: 1,770,000 cycles against 160,000.  For the whole mini-batch and the room for its entries, so
+// that a slice of it takes the same kernel.
+bool sparse_forward_wanted(const sfb_ctx* ctx, int64_t n) {
+  const int rb = sparse_forward_rows(ctx, n);
+  if (rb == 0 || ctx->h16) return false;
+  const sfb_config& c = ctx->cfg;
+  const double rounds = static_cast<double>(((c.rows + rb - 1) / rb + sm_count() - 1) / sm_count());
+  const double entries = static_cast<double>(c.csr_nnz_max) / static_cast<double>(ctx->K);
+  const double sparse = rounds * (static_cast<double>((ctx->K + kSfWarps - 1) / kSfWarps) * (900.0 + 40.0 * entries * rb / 32.0) +
+                                  static_cast<double>(rb * c.cols) * 4.0 / 25.0);
+  return sparse < gemm_cycles(ctx->K, c.rows, c.cols);
 }
 
 // Z[off .. off+n) = X W^T for the n staged sparse samples at pair offset off (fp32, row pitch ldz).

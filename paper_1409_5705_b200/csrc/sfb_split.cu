@@ -630,7 +630,7 @@ template <bool F16>
 __global__ void __launch_bounds__(256) pack_t_kernel(const float* __restrict__ F, int64_t n, int64_t dim, int64_t ld,
                                                      uint16_t* __restrict__ FT, int64_t Kp, const float* __restrict__ inv) {
   pdl_launch_dependents();
-  pdl_wait(F, inv);
+  pdl_wait(inv);
   __shared__ float tile[64][65];
   const int64_t i0 = static_cast<int64_t>(blockIdx.y) * 64, c0 = static_cast<int64_t>(blockIdx.x) * 64;
   const int t = threadIdx.x;
@@ -663,7 +663,7 @@ __global__ void __launch_bounds__(256) pack_t_kernel(const float* __restrict__ F
 __global__ void __launch_bounds__(256) pack_rows_kernel(const float* __restrict__ F, int64_t n, int64_t dim, int64_t ld,
                                                         uint16_t* __restrict__ dst, int64_t dimp, const Stamp stamp) {
   pdl_launch_dependents();
-  pdl_wait(F);
+  pdl_wait();
   stamp_begin(stamp);
   const int64_t quads = (dim + 3) / 4, total = n * quads;
   const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
@@ -690,7 +690,7 @@ __global__ void __launch_bounds__(256) pack_pairs_kernel(const float* __restrict
                                                          int64_t dim, float* __restrict__ V, uint16_t* __restrict__ dst,
                                                          int64_t dimp) {
   pdl_launch_dependents();
-  pdl_wait(X, Y);
+  pdl_wait();
   const uint32_t quads = static_cast<uint32_t>(dim / 4);
   const int64_t total = n * quads, stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
   for (int64_t q = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; q < total; q += stride) {
@@ -834,7 +834,7 @@ __global__ void __launch_bounds__(1024) sc_scales_kernel(const float* __restrict
 __global__ void __launch_bounds__(256) row_most_kernel(const float* __restrict__ U, int64_t ldu, int64_t rows,
                                                        const float* __restrict__ inv, float* __restrict__ q) {
   pdl_launch_dependents();
-  pdl_wait(U, inv);
+  pdl_wait(inv);
   __shared__ float sh[8];
   const float* u = U + static_cast<int64_t>(blockIdx.x) * ldu;
   float m = 0.f;
@@ -856,7 +856,7 @@ __global__ void __launch_bounds__(256) pack_u_kernel(const float* __restrict__ U
                                                      const float* __restrict__ q, const float* __restrict__ inv_v,
                                                      uint16_t* __restrict__ dst, int64_t rowsp, Scalars* sc, const Stamp stamp) {
   pdl_launch_dependents();
-  pdl_wait(U, q, inv_v);
+  pdl_wait(q, inv_v);
   stamp_begin(stamp);
   __shared__ float sh[8];
   float m = 0.f;
