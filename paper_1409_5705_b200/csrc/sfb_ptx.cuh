@@ -175,11 +175,11 @@ __device__ __forceinline__ uint64_t umma_desc_k128(uint32_t smem_addr) {
 
 // The same for an MN-major operand tile: the contraction is the outer dimension.  A TMA box {64 elements of M or N, 64 of the
 // contraction} with the 128-byte swizzle is one 8 KB atom column: rows (of the contraction) of 128 bytes, groups of 8 of them
-// 1024 bytes apart (stride byte offset); the next 64 elements of M or N are the next box, 8 KB on (leading byte offset).
-// A step of 16 along the contraction advances the start address by 2048 bytes.
-__device__ __forceinline__ uint64_t umma_desc_mn128(uint32_t smem_addr) {
+// 1024 bytes apart (stride byte offset); the next 64 elements of M or N are the next box, 8 KB on (leading byte offset; 4 KB
+// with 32 of the contraction).  A step of 16 along the contraction advances the start address by 2048 bytes.
+__device__ __forceinline__ uint64_t umma_desc_mn128(uint32_t smem_addr, uint32_t box_bytes = 8192) {
   uint64_t d = umma_desc_k128(smem_addr);
-  d |= static_cast<uint64_t>(8192 >> 4) << 16;                    // bits 16-29: leading byte offset >> 4
+  d |= static_cast<uint64_t>(box_bytes >> 4) << 16;                    // bits 16-29: leading byte offset >> 4
   return d;
 }
 constexpr uint32_t kIdescMnMajor = (1u << 15) | (1u << 16);       // A and B are MN-major (default: K-major)

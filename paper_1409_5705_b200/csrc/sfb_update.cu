@@ -372,18 +372,22 @@ update_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
 // ---------------------------------------------------------------------------------------------------------
 // The update of operands that are (hi | lo) pairs of 16-bit values (metric learning, sparse coding):
 //   W <- prox(W + alpha * (U_hi^T V_hi + U_lo^T V_hi + U_hi^T V_lo)).
-// As in forward_split_kernel, one stage holds a k-block of all four halves (64 KB in a CTA of the pair, 43 bytes per cycle of
-// tensor work where three passes over the contraction take 64: those were bound by their loads) and the cross terms have an
-// accumulator of their own; U_hi^T V_hi is added to sums in the epilogue warps' registers every eight k-blocks, while the
-// cross terms of the last of them run.  The sums also free both accumulators (all 512 columns of TMEM) before the pass over
-// W, which therefore runs beside the next tile's products although there is no second pair of accumulators.
-// Shared memory: three stages and one 4 KB slot of W per epilogue warp.  1,000 x 20,000, K = 1024: 114 us with three passes.
+// As in split_product_kernel, one stage holds a k-block of all four halves and the cross terms have an accumulator of their own;
+// U_hi^T V_hi is added to sums in the epilogue warps' registers every 1,024 pairs, while the cross terms of the last k-block
+// run.  The sums also free both accumulators (all 512 columns of TMEM) before the pass over W, which therefore runs beside the
+// next tile's products although there is no second pair of accumulators.
+// Shared memory, in two forms.  Many pairs: three stages of 64 of them (64 KB in a CTA), for the tensor cores' sake, and one 4 KB
+// slot of W per epilogue warp.  Few pairs, where the pass over W is what takes the time: three stages of 32 and four slots.
+// With one slot that pass waits for every load (2.7 TB/s); with stages of 32 there are twice the copies (K = 1024: 914 -> 980 us).
 // ---------------------------------------------------------------------------------------------------------
-constexpr int SU_STAGES = 3, SU_DRAIN = 16;
-constexpr int kSuBytes = 64 * 2 * UM;                // 16 KB: one operand half of a k-block in a CTA
-constexpr int kSuStage = 4 * kSuBytes;
-constexpr int kSuBars = 2 * SU_STAGES + 4 + kEpiWarps;
-constexpr int kSuSmem = SU_STAGES * kSuStage + kEpiWarps * kSlotBytes + kSuBars * 8 + 16 + 1024;
+constexpr int SU_STAGES = 3, kSuFewPairs = 384;
+template <bool FEW>
+struct SuShape {
+  static constexpr int kPairs = FEW ? 32 : 64, kDrain = 1024 / kPairs, kSlots = FEW ? 4 : 1, kPending = FEW ? 1 : 0;
+  static constexpr int kBox = 64 * kPairs * 2, kBytes = 2 * kBox, kStage = 4 * kBytes;     // 64 columns; an operand half; all four
+  static constexpr int kBars = 2 * SU_STAGES + 4 + kEpiWarps * kSlots;
+  static constexpr int kSmem = SU_STAGES * kStage + kEpiWarps * kSlots * kSlotBytes + kBars * 8 + 16 + 1024;
+};
 
 struct SplitUpdParams {
   UpdParams t;                 // rows, cols, tiles, bn, kseg, alpha, prox, stamps, status
@@ -393,20 +397,24 @@ struct SplitUpdParams {
   const float* inv;            // inverse scale of the whole sum (or null: 1)
 };
 
+template <bool FEW>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
 update_split_kernel(const __grid_constant__ CUtensorMap tmU, const __grid_constant__ CUtensorMap tmV,
                     const __grid_constant__ CUtensorMap tmC, const __grid_constant__ SplitUpdParams sp) {
+  using Shape = SuShape<FEW>;
+  constexpr int SU_UK = Shape::kPairs, SU_DRAIN = Shape::kDrain, SU_SLOTS = Shape::kSlots, SU_PENDING = Shape::kPending;
+  constexpr int kSuBox = Shape::kBox, kSuBytes = Shape::kBytes, kSuStage = Shape::kStage, kSuBars = Shape::kBars;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint8_t* sRing = smem + SU_STAGES * kSuStage;
-  uint64_t* bars = reinterpret_cast<uint64_t*>(sRing + kEpiWarps * kSlotBytes);
+  uint64_t* bars = reinterpret_cast<uint64_t*>(sRing + kEpiWarps * SU_SLOTS * kSlotBytes);
   uint64_t* full = bars;                             // as in update_pair_kernel: full, mempty, cempty are the leader's
   uint64_t* empty = bars + SU_STAGES;
   uint64_t* mfull = bars + 2 * SU_STAGES;
   uint64_t* mempty = mfull + 1;
   uint64_t* cfull = mfull + 2;
   uint64_t* cempty = mfull + 3;
-  uint64_t* rfull = mfull + 4;                       // per epilogue warp
+  uint64_t* rfull = mfull + 4;                       // per epilogue warp and slot
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + kSuBars);
   volatile uint32_t* abort_flag = tmem_slot + 1;
 
@@ -423,7 +431,7 @@ update_split_kernel(const __grid_constant__ CUtensorMap tmU, const __grid_consta
     for (int i = 0; i < SU_STAGES; ++i) { mbar_init(&full[i], 1); mbar_init(&empty[i], 1); }
     mbar_init(mfull, 1); mbar_init(mempty, 2 * kEpiWarps);
     mbar_init(cfull, 1); mbar_init(cempty, 2 * kEpiWarps);
-    for (int i = 0; i < kEpiWarps; ++i) mbar_init(&rfull[i], 1);
+    for (int i = 0; i < kEpiWarps * SU_SLOTS; ++i) mbar_init(&rfull[i], 1);
     *abort_flag = 0;
     fence_barrier_init();
     prefetch_tmap(&tmU); prefetch_tmap(&tmV); prefetch_tmap(&tmC);
@@ -439,7 +447,7 @@ update_split_kernel(const __grid_constant__ CUtensorMap tmU, const __grid_consta
   stamp_begin(p.begin);
 
   if (warp == 0) {
-    // ---------------- TMA producer: U_hi, U_lo, V_hi, V_lo of a k-block, boxes of 64 columns x 64 pairs ----------------
+    // ---------------- TMA producer: U_hi, U_lo, V_hi, V_lo of a k-block, boxes of 64 columns ----------------
     if (lane == 0) {
       const uint64_t pol_keep = policy_evict_last(), pol_norm = policy_evict_normal();
       uint32_t it = 0;
@@ -451,16 +459,16 @@ update_split_kernel(const __grid_constant__ CUtensorMap tmU, const __grid_consta
         for (int kb = 0; kb < nk; ++kb, ++it) {
           const uint32_t s = it % SU_STAGES, ph = (it / SU_STAGES) & 1;
           if (!mbar_wait(&empty[s], ph ^ 1, abort_flag)) { ok = false; break; }
-          if (rank == 0) mbar_expect_tx(&full[s], 2 * (2 * kSuBytes + 2 * half * UK * 2));
+          if (rank == 0) mbar_expect_tx(&full[s], 2 * (2 * kSuBytes + 2 * half * SU_UK * 2));
           const uint32_t bar = mapa_u32(smem_u32(&full[s]), 0);
           uint8_t* st = smem + s * kSuStage;
 #pragma unroll
           for (int b = 0; b < 2; ++b) {
-            tma_load_2d_pair(st + b * 8192, &tmU, mu + 64 * b, kb * UK, bar, pol_norm);
-            tma_load_2d_pair(st + kSuBytes + b * 8192, &tmU, sp.u_lo + mu + 64 * b, kb * UK, bar, pol_norm);
+            tma_load_2d_pair(st + b * kSuBox, &tmU, mu + 64 * b, kb * SU_UK, bar, pol_norm);
+            tma_load_2d_pair(st + kSuBytes + b * kSuBox, &tmU, sp.u_lo + mu + 64 * b, kb * SU_UK, bar, pol_norm);
             if (64 * b < half) {
-              tma_load_2d_pair(st + 2 * kSuBytes + b * 8192, &tmV, nv + 64 * b, kb * UK, bar, pol_keep);
-              tma_load_2d_pair(st + 3 * kSuBytes + b * 8192, &tmV, sp.v_lo + nv + 64 * b, kb * UK, bar, pol_keep);
+              tma_load_2d_pair(st + 2 * kSuBytes + b * kSuBox, &tmV, nv + 64 * b, kb * SU_UK, bar, pol_keep);
+              tma_load_2d_pair(st + 3 * kSuBytes + b * kSuBox, &tmV, sp.v_lo + nv + 64 * b, kb * SU_UK, bar, pol_keep);
             }
           }
         }
@@ -481,10 +489,10 @@ update_split_kernel(const __grid_constant__ CUtensorMap tmU, const __grid_consta
           if (kc == 0 && !mbar_wait(mempty, (g & 1) ^ 1, abort_flag)) { ok = false; break; }
           tc_fence_after();
           uint8_t* st = smem + s * kSuStage;
-          const uint64_t duh = umma_desc_mn128(smem_u32(st)), dul = umma_desc_mn128(smem_u32(st + kSuBytes));
-          const uint64_t dvh = umma_desc_mn128(smem_u32(st + 2 * kSuBytes)), dvl = umma_desc_mn128(smem_u32(st + 3 * kSuBytes));
+          const uint64_t duh = umma_desc_mn128(smem_u32(st), kSuBox), dul = umma_desc_mn128(smem_u32(st + kSuBytes), kSuBox);
+          const uint64_t dvh = umma_desc_mn128(smem_u32(st + 2 * kSuBytes), kSuBox), dvl = umma_desc_mn128(smem_u32(st + 3 * kSuBytes), kSuBox);
 #pragma unroll
-          for (int k = 0; k < UK / UMMA_K; ++k) {
+          for (int k = 0; k < SU_UK / UMMA_K; ++k) {
             const uint64_t adv = static_cast<uint64_t>(k * 2048 / 16);
             umma_bf16_pair(d_main, duh + adv, dvh + adv, idesc, (kc | k) != 0 ? 1u : 0u);
           }
@@ -497,7 +505,7 @@ update_split_kernel(const __grid_constant__ CUtensorMap tmU, const __grid_consta
             tc_fence_after();
           }
 #pragma unroll
-          for (int k = 0; k < UK / UMMA_K; ++k) {
+          for (int k = 0; k < SU_UK / UMMA_K; ++k) {
             const uint64_t adv = static_cast<uint64_t>(k * 2048 / 16);
             umma_bf16_pair(d_cross, dul + adv, dvh + adv, idesc, (kb | k) != 0 ? 1u : 0u);
             umma_bf16_pair(d_cross, duh + adv, dvl + adv, idesc, 1u);
@@ -510,23 +518,28 @@ update_split_kernel(const __grid_constant__ CUtensorMap tmU, const __grid_consta
   } else {
     // ---------------- epilogue: warp (q, h) = TMEM lane quarter q, column half h ----------------
     const int e = warp - 2, q = warp & 3, h = e >> 2;
-    uint8_t* sl = sRing + e * kSlotBytes;
+    uint8_t* slots = sRing + e * SU_SLOTS * kSlotBytes;
+    uint64_t* arrived = rfull + e * SU_SLOTS;
     const int cpw = half / kChunk;                   // chunks per warp and tile: 4 or 2
     const uint64_t pol_w = policy_evict_normal();
     const uint32_t mempty_leader = mapa_u32(smem_u32(mempty), 0), cempty_leader = mapa_u32(smem_u32(cempty), 0);
     const int row_in_tile = static_cast<int>(rank) * UM + q * 32;
     const uint32_t t_addr = tmem_base + (static_cast<uint32_t>(q * 32) << 16) + h * half;
     bool ok = true;
-    auto issue_load = [&](int tl, int c) {           // (lane 0) chunk c of this pair's tile tl
-      if (tl >= my_tiles) return;
+    const uint32_t last = static_cast<uint32_t>(my_tiles * cpw);
+    auto issue_load = [&](uint32_t n) {              // (lane 0) the n-th chunk of this warp
+      if (n >= last) return;
+      const int tl = static_cast<int>(n) / cpw, c = static_cast<int>(n) % cpw;
       int m0, n0;
       tile_origin(p, pair + tl * npairs, m0, n0);
-      mbar_expect_tx(&rfull[e], kSlotBytes);
-      tma_load_2d_hint(sl, &tmC, n0 + h * half + c * kChunk, m0 + row_in_tile, &rfull[e], pol_w);
+      const uint32_t at = n % SU_SLOTS;
+      mbar_expect_tx(&arrived[at], kSlotBytes);
+      tma_load_2d_hint(slots + at * kSlotBytes, &tmC, n0 + h * half + c * kChunk, m0 + row_in_tile, &arrived[at], pol_w);
     };
-    if (lane == 0) issue_load(0, 0);
+    if (lane == 0)
+      for (uint32_t n = 0; n < SU_SLOTS; ++n) issue_load(n);
     const float alpha = p.alpha * (sp.inv ? *sp.inv : 1.f);
-    uint32_t g = 0, r = 0;
+    uint32_t g = 0, r = 0;                           // drains and chunks behind
     for (int tl = 0; tl < my_tiles && ok; ++tl) {
       int m0, n0;
       tile_origin(p, pair + tl * npairs, m0, n0);
@@ -561,9 +574,9 @@ update_split_kernel(const __grid_constant__ CUtensorMap tmU, const __grid_consta
       for (int c = 0; c < 4; ++c) {
         if (c >= cpw || !ok) break;
         const int x0 = n0 + h * half + c * kChunk, y0 = m0 + row_in_tile;
-        ok = __all_sync(0xffffffffu, mbar_wait(&rfull[e], r & 1, abort_flag));
+        ok = __all_sync(0xffffffffu, mbar_wait(&arrived[r % SU_SLOTS], (r / SU_SLOTS) & 1, abort_flag));
         if (!ok) break;
-        ++r;
+        uint8_t* sl = slots + (r % SU_SLOTS) * kSlotBytes;
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
           float4* wp = reinterpret_cast<float4*>(sl + lane * 128 + ((j ^ (lane & 7)) << 4));
@@ -583,10 +596,11 @@ update_split_kernel(const __grid_constant__ CUtensorMap tmU, const __grid_consta
         if (lane == 0) {
           if (x0 < p.cols && y0 < p.rows) tma_store_2d_hint(&tmC, sl, x0, y0, pol_w);
           tma_commit_group();
-          tma_wait_group_read<0>();                   // the slot has been read: the next chunk may land in it
-          issue_load(c + 1 < cpw ? tl : tl + 1, c + 1 < cpw ? c + 1 : 0);
+          tma_wait_group_read<SU_PENDING>();          // an earlier chunk's slot (or this one's) has been read: refill it
+          if (r >= SU_PENDING) issue_load(r - SU_PENDING + SU_SLOTS);
         }
         __syncwarp();
+        ++r;
       }
     }
     if (lane == 0) tma_wait_group<0>();
@@ -608,7 +622,8 @@ update_split_kernel(const __grid_constant__ CUtensorMap tmU, const __grid_consta
 }
 
 // Tile width: 128 where 256-wide tiles leave the pairs short of work.  Cycles of a tile: its k-blocks at the MMA or operand
-// rate (measured about 620 a k-block for 256 columns, 450 for 128; with four operand halves 1600 and 900) and its epilogue.
+// rate (measured about 620 a k-block of 64 pairs for 256 columns, 450 for 128; 1600 and 900 with four operand halves) and its
+// epilogue.
 int tile_width(int64_t rows, int64_t cols, int64_t kblocks, int pairs, bool split) {
   auto cost = [&](int bn) {
     const int64_t tiles = ((rows + 2 * UM - 1) / (2 * UM)) * ((cols + bn - 1) / bn);
@@ -652,7 +667,8 @@ static cudaError_t prepare_kernel(Kernel kernel, int smem, int* max_pairs) {
 int tc_update_init(sfb_ctx* ctx, TcState* st) {
   int n = 1 << 30;
   CKC(prepare_kernel(update_pair_kernel<1>, kSmem, &n));
-  CKC(prepare_kernel(update_split_kernel, kSuSmem, &n));
+  CKC(prepare_kernel(update_split_kernel<false>, SuShape<false>::kSmem, &n));
+  CKC(prepare_kernel(update_split_kernel<true>, SuShape<true>::kSmem, &n));
   CKC(prepare_kernel(update_pair_kernel<2, true>, kSmem, &n));
   st->max_pairs = n;
   if (n < 1) return SFB_ERR_ARCH;                 // the device cannot host a CTA pair of these kernels
@@ -712,16 +728,18 @@ int tc_update(sfb_ctx* ctx) {
   const int64_t wu = split ? 2 * L.rowsp : c.rows, wv = split ? 2 * L.colsp : c.cols;
   __nv_bfloat16* U = ctx->at<__nv_bfloat16>(split ? L.Rs : L.P);
   void* V = split ? const_cast<uint16_t*>(split_v(ctx)) : ctx->at<uint16_t>(L.Xb);
+  const bool few = split && ctx->K <= kSuFewPairs;
+  const int uk = few ? SuShape<true>::kPairs : UK;
   CUtensorMap ma, mb, mc;
-  if (!make_map(st, &ma, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, U, wu, ctx->K, ldu * 2, 64, UK) ||
-      !make_map(st, &mb, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, V, wv, ctx->K, ldv * 2, 64, UK) ||
+  if (!make_map(st, &ma, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, U, wu, ctx->K, ldu * 2, 64, uk) ||
+      !make_map(st, &mb, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, V, wv, ctx->K, ldv * 2, 64, uk) ||
       !make_map(st, &mc, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, ctx->W, c.cols, c.rows, c.cols * 4, kChunk, 32))
     return SFB_ERR_CUDA;
   UpdParams p{};
   p.rows = static_cast<int32_t>(c.rows); p.cols = static_cast<int32_t>(c.cols);
   p.tilesM = static_cast<int32_t>((c.rows + 2 * UM - 1) / (2 * UM));
-  p.kseg = static_cast<int32_t>((ctx->K + UK - 1) / UK);
-  p.bn = tile_width(c.rows, c.cols, p.kseg, st->max_pairs, split);
+  p.kseg = static_cast<int32_t>((ctx->K + uk - 1) / uk);
+  p.bn = tile_width(c.rows, c.cols, (ctx->K + UK - 1) / UK, st->max_pairs, split);
   p.tilesN = static_cast<int32_t>((c.cols + p.bn - 1) / p.bn);
   p.begin = take_stamp(ctx); p.end = &ctx->at<Scalars>(L.scalars)->ns[3];
   p.alpha = -ctx->step;
@@ -732,8 +750,10 @@ int tc_update(sfb_ctx* ctx) {
   if (split) {
     SplitUpdParams sp{p, static_cast<int32_t>(L.rowsp), static_cast<int32_t>(L.colsp), ctx->h16, ctx->h16 ? 1.f / 2048.f : 1.f,
                       ctx->h16 ? &ctx->at<Scalars>(L.scalars)->iU : nullptr};
-    CKC(launch_kernel_if(tiles <= st->max_pairs, update_split_kernel, dim3(grid), dim3(kThreads), kSuSmem, ctx->stream, 1, ma, mb,
-                         mc, sp));
+    CKC(few ? launch_kernel_if(tiles <= st->max_pairs, update_split_kernel<true>, dim3(grid), dim3(kThreads), SuShape<true>::kSmem,
+                               ctx->stream, 1, ma, mb, mc, sp)
+            : launch_kernel_if(tiles <= st->max_pairs, update_split_kernel<false>, dim3(grid), dim3(kThreads), SuShape<false>::kSmem,
+                               ctx->stream, 1, ma, mb, mc, sp));
     return SFB_OK;
   }
   p.nseg = 1;
