@@ -658,47 +658,50 @@ __global__ void __launch_bounds__(256) pack_t_kernel(const float* __restrict__ F
   }
 }
 
-// bf16 form: fp32 [n x dim] (row pitch ld) -> the operand [n x 2*dimp].  Columns dim..dimp-1 are left as they are (zero since
-// set-up).
-__global__ void __launch_bounds__(256) pack_rows_kernel(const float* __restrict__ F, int64_t n, int64_t dim, int64_t ld,
-                                                        uint16_t* __restrict__ dst, int64_t dimp, const Stamp stamp) {
+// bf16 form: rows of F (or of F - Y, which then also go to V in fp32) -> the operand [n x 2*dimp].  TPR threads per row, four
+// quads of columns each at a time.  Columns dim..dimp-1 are left as they are (zero since set-up).  (Over one index for the whole
+// matrix, each quad paid for a 64-bit division: 1,000 x 20,000 47 us, 10,000 x 5,000 109.)
+template <int TPR, bool SUB>
+__global__ void __launch_bounds__(256) pack_rows_kernel(const float* __restrict__ F, const float* __restrict__ Y, int64_t n, int dim,
+                                                        int64_t ld, float* __restrict__ V, uint16_t* __restrict__ dst, int64_t dimp,
+                                                        const Stamp stamp) {
   pdl_launch_dependents();
   pdl_wait();
   stamp_begin(stamp);
-  const int64_t quads = (dim + 3) / 4, total = n * quads;
-  const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
-  const bool vec = ld % 4 == 0 && dim % 4 == 0;          // else (samples with an odd number of features) value by value
-  for (int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; i < total; i += stride) {
-    const int64_t r = i / quads, qd = i % quads;
-    const float* src = F + r * ld + qd * 4;
-    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (vec) {
-      v = *reinterpret_cast<const float4*>(src);
-    } else {
-      v.x = src[0];
-      if (qd * 4 + 1 < dim) v.y = src[1];
-      if (qd * 4 + 2 < dim) v.z = src[2];
-      if (qd * 4 + 3 < dim) v.w = src[3];
+  const int64_t r = static_cast<int64_t>(blockIdx.x) * (256 / TPR) + threadIdx.x / TPR;
+  const int t = threadIdx.x % TPR, quads = dim / 4;
+  if (r >= n) return;
+  uint16_t* d = dst + r * 2 * dimp;
+  if (ld % 4 == 0 && dim % 4 == 0) {
+    const float4* src = reinterpret_cast<const float4*>(F + r * ld);
+    const float4* sub = reinterpret_cast<const float4*>(Y + r * ld);
+    float4* v4 = reinterpret_cast<float4*>(V + r * dim);
+    for (int q0 = t; q0 < quads; q0 += 4 * TPR) {
+      float4 v[4], y[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        if (q0 + k * TPR < quads) v[k] = src[q0 + k * TPR];
+        if (SUB && q0 + k * TPR < quads) y[k] = sub[q0 + k * TPR];
+      }
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const int q = q0 + k * TPR;
+        if (q >= quads) continue;
+        if (SUB) {
+          v[k] = make_float4(v[k].x - y[k].x, v[k].y - y[k].y, v[k].z - y[k].z, v[k].w - y[k].w);
+          v4[q] = v[k];
+        }
+        put_pair4<false>(d + 4 * q, dimp, v[k]);
+      }
     }
-    put_pair4<false>(dst + r * 2 * dimp + qd * 4, dimp, v);
-  }
-}
-
-// bf16 form, metric learning: v = x - y of n pairs (Section 2) in fp32 and as the operand, one pass (16 bytes per value; as
-// two kernels 24).
-__global__ void __launch_bounds__(256) pack_pairs_kernel(const float* __restrict__ X, const float* __restrict__ Y, int64_t n,
-                                                         int64_t dim, float* __restrict__ V, uint16_t* __restrict__ dst,
-                                                         int64_t dimp) {
-  pdl_launch_dependents();
-  pdl_wait();
-  const uint32_t quads = static_cast<uint32_t>(dim / 4);
-  const int64_t total = n * quads, stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
-  for (int64_t q = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; q < total; q += stride) {
-    const int64_t i = q / quads, c = (q - i * quads) * 4;
-    const float4 x = reinterpret_cast<const float4*>(X)[q], y = reinterpret_cast<const float4*>(Y)[q];
-    const float4 v = make_float4(x.x - y.x, x.y - y.y, x.z - y.z, x.w - y.w);
-    reinterpret_cast<float4*>(V)[q] = v;
-    put_pair4<false>(dst + i * 2 * dimp + c, dimp, v);
+  } else {                                             // samples with an odd number of features: value by value
+    const float* src = F + r * ld;
+    for (int c = t; c < dim; c += TPR) {
+      uint32_t hi, lo;
+      split2<false>(src[c], 0.f, hi, lo);
+      d[c] = static_cast<uint16_t>(hi);
+      d[dimp + c] = static_cast<uint16_t>(lo);
+    }
   }
 }
 
@@ -723,6 +726,15 @@ struct Pack16 {
   float iters;
   Stamp stamp;
 };
+__device__ __forceinline__ void row_scales(const Pack16& p, int64_t r, float s, float ss) {
+  p.inv[r] = 1.f / s;
+  if (p.inv2) p.inv2[r] = 1.f / s;
+  if (p.inv_res) {
+    const float norm = sqrtf(ss);
+    p.inv_res[r] = 1.f / pow2_scale(norm, 4);
+    p.inv_code[r] = 1.f / pow2_scale(p.iters * norm * sqrtf(p.sc->invL), 4);
+  }
+}
 template <int TPR>
 __global__ void __launch_bounds__(256) pack16_kernel(const __grid_constant__ Pack16 p) {
   pdl_launch_dependents();
@@ -775,15 +787,7 @@ __global__ void __launch_bounds__(256) pack16_kernel(const __grid_constant__ Pac
     for (int w = 1; w < 8; ++w) { m = fmaxf(m, sh[w]); ss += sh[8 + w]; }
   }
   const float s = pow2_scale(m, 13);
-  if (t == 0) {
-    p.inv[r] = 1.f / s;
-    if (p.inv2) p.inv2[r] = 1.f / s;
-    if (p.inv_res) {
-      const float norm = sqrtf(ss);
-      p.inv_res[r] = 1.f / pow2_scale(norm, 4);
-      p.inv_code[r] = 1.f / pow2_scale(p.iters * norm * sqrtf(p.sc->invL), 4);
-    }
-  }
+  if (t == 0) row_scales(p, r, s, ss);
   uint16_t* d = p.dst + r * 2 * p.dimp;
   if (vec) {
     float4* v4 = p.V ? reinterpret_cast<float4*>(p.V + r * p.dim) : nullptr;
@@ -806,6 +810,73 @@ __global__ void __launch_bounds__(256) pack16_kernel(const __grid_constant__ Pac
       d[c] = static_cast<uint16_t>(hi);
       d[p.dimp + c] = static_cast<uint16_t>(lo);
     }
+  }
+}
+
+// The same for long rows, which come through shared memory: a block has the next rows under way by bulk copies while it looks for
+// the largest entry of one and converts it.  (Held in registers, a row's loads and stores took turns: 10,000 x 20,000 in 603 us.)
+constexpr int kPackRoom = 208 << 10, kPackThreads = 512, kPackBufs = 4;
+__global__ void __launch_bounds__(kPackThreads, 1) pack16_long_kernel(const __grid_constant__ Pack16 p, int bufs, uint32_t* status) {
+  extern __shared__ __align__(128) uint8_t rows_smem[];
+  __shared__ __align__(8) uint64_t full[kPackBufs];
+  __shared__ float sh[2 * kPackThreads / 32];
+  __shared__ uint32_t abort_word;
+  pdl_launch_dependents();
+  const int t = threadIdx.x, quads = static_cast<int>(p.dim / 4);
+  const uint32_t bytes = static_cast<uint32_t>(p.dim) * 4;
+  if (t == 0) {
+    for (int i = 0; i < kPackBufs; ++i) mbar_init(&full[i], 1);
+    abort_word = 0;
+    fence_barrier_init();
+  }
+  __syncthreads();
+  pdl_wait();
+  stamp_begin(p.stamp);
+  auto ask = [&](int64_t r, int b) {
+    mbar_expect_tx(&full[b], bytes);
+    bulk_load(smem_u32(rows_smem) + b * bytes, p.F + r * p.ld, bytes, &full[b]);
+  };
+  const int64_t step = gridDim.x;
+  if (t == 0)
+    for (int b = 0; b < bufs && blockIdx.x + b * step < p.n; ++b) ask(blockIdx.x + b * step, b);
+  int b = 0;
+  uint32_t ph = 0;
+  for (int64_t r = blockIdx.x; r < p.n; r += step) {
+    if (!__syncthreads_and(mbar_wait(&full[b], ph, &abort_word))) {
+      if (t == 0) atomicOr(status, SFB_STATUS_TIMEOUT);
+      for (int i = 0; i < 64; ++i) __nanosleep(1000);  // for copies in flight
+      return;
+    }
+    const float4* row = reinterpret_cast<const float4*>(rows_smem + b * bytes);
+    float m = 0.f, ss = 0.f;
+    for (int q = t; q < quads; q += kPackThreads) {
+      const float4 v = row[q];
+      m = fmaxf(m, fmaxf(fmaxf(fabsf(v.x), fabsf(v.y)), fmaxf(fabsf(v.z), fabsf(v.w))));
+      if (p.inv_res) ss = fmaf(v.x, v.x, fmaf(v.y, v.y, fmaf(v.z, v.z, fmaf(v.w, v.w, ss))));
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+      ss += __shfl_xor_sync(0xffffffffu, ss, o);
+    }
+    constexpr int kWarps = kPackThreads / 32;
+    if ((t & 31) == 0) { sh[t >> 5] = m; sh[kWarps + (t >> 5)] = ss; }
+    __syncthreads();
+    m = sh[0]; ss = sh[kWarps];
+#pragma unroll
+    for (int w = 1; w < kWarps; ++w) { m = fmaxf(m, sh[w]); ss += sh[kWarps + w]; }
+    const float s = pow2_scale(m, 13);
+    if (t == 0) row_scales(p, r, s, ss);
+    uint16_t* d = p.dst + r * 2 * p.dimp;
+    float4* v4 = p.V ? reinterpret_cast<float4*>(p.V + r * p.dim) : nullptr;
+    for (int q = t; q < quads; q += kPackThreads) {
+      const float4 v = row[q];
+      if (v4) v4[q] = v;
+      put_pair4<true>(d + 4 * q, p.dimp, scale4(v, s));
+    }
+    __syncthreads();                                   // the row (and sh) has been read
+    if (t == 0 && r + bufs * step < p.n) ask(r + bufs * step, b);
+    if (++b == bufs) { b = 0; ph ^= 1; }
   }
 }
 
@@ -966,10 +1037,29 @@ int split_product(sfb_ctx* ctx, int64_t off, int64_t n, const uint16_t* A, const
   return SFB_OK;
 }
 
-cudaError_t pack16(cudaStream_t s, const Pack16& p) {
+cudaError_t pack16(sfb_ctx* ctx, const Pack16& p) {
+  cudaStream_t s = ctx->stream;
   if (p.n <= 0) return cudaSuccess;
   if (p.dim <= 2048) return launch_kernel(pack16_kernel<32>, dim3(static_cast<unsigned>((p.n + 7) / 8)), dim3(256), 0, s, 1, p);
-  return launch_kernel(pack16_kernel<256>, dim3(static_cast<unsigned>(p.n)), dim3(256), 0, s, 1, p);
+  const int bufs = static_cast<int>(std::min<int64_t>(kPackBufs, kPackRoom / (p.dim * 4)));
+  if (bufs < 2 || p.Y || p.dim % 4 != 0 || p.ld % 4 != 0)
+    return launch_kernel(pack16_kernel<256>, dim3(static_cast<unsigned>(p.n)), dim3(256), 0, s, 1, p);
+  const cudaError_t e = allow_smem<pack16_long_kernel>(kPackRoom);
+  if (e != cudaSuccess) return e;
+  return launch_kernel(pack16_long_kernel, dim3(static_cast<unsigned>(std::min<int64_t>(p.n, sm_count()))), dim3(kPackThreads),
+                       static_cast<int>(bufs * p.dim * 4), s, 1, p, bufs, ctx->at<uint32_t>(ctx->lay.status));
+}
+
+// bf16 form; Y: subtracted, the difference also to V.
+cudaError_t pack_rows(cudaStream_t s, const float* F, const float* Y, int64_t n, int64_t dim, int64_t ld, float* V, uint16_t* dst,
+                      int64_t dimp, const Stamp& stamp) {
+  if (n <= 0) return cudaSuccess;
+  auto go = [&](auto kernel, int tpr) {
+    return launch_kernel(kernel, dim3(static_cast<unsigned>((n + 256 / tpr - 1) / (256 / tpr))), dim3(256), 0, s, 1, F, Y, n,
+                         static_cast<int>(dim), ld, V, dst, dimp, stamp);
+  };
+  if (dim <= 512) return Y ? go(pack_rows_kernel<32, true>, 32) : go(pack_rows_kernel<32, false>, 32);
+  return Y ? go(pack_rows_kernel<256, true>, 256) : go(pack_rows_kernel<256, false>, 256);
 }
 
 // Features up to which the coder on W^T W forms W^T x by fp32 FMAs and W^T W with its fourth term in the bf16 form.  Every
@@ -1021,7 +1111,7 @@ int factors_sc(sfb_ctx* ctx, int64_t off, int64_t n, const float* X) {
     p.inv = ctx->at<float>(L.iA) + off;
     p.inv_res = ctx->at<float>(L.iR) + off; p.inv_code = ctx->at<float>(L.iC) + off;
     p.sc = sc; p.iters = static_cast<float>(T);
-    CKC(pack16(s, p));
+    CKC(pack16(ctx, p));
   }
   if (T == 0) {
     CKC(cudaMemsetAsync(V + off * cols, 0, static_cast<size_t>(n) * cols * 4, s));
@@ -1032,12 +1122,10 @@ int factors_sc(sfb_ctx* ctx, int64_t off, int64_t n, const float* X) {
     e.sc = sc; e.lam = c.sc_lambda;
     CKC(sgemm(s, true, false, EPI_ISTA0, n, cols, rows, X, rows, ctx->W, cols, e, ctx->K));
     ctx->stats.flops += 2.0 * n * rows * cols;
-    CKC(launch_kernel(pack_rows_kernel, dim3(grid1d(n * cols / 4, 256)), dim3(256), 0, s, 1, V + off * cols, n, cols, cols,
-                      as[1] + off * 2 * L.colsp, L.colsp, Stamp{}));
+    CKC(pack_rows(s, V + off * cols, nullptr, n, cols, cols, nullptr, as[1] + off * 2 * L.colsp, L.colsp, Stamp{}));
   } else {
     if (!F16)
-      CKC(launch_kernel(pack_rows_kernel, dim3(grid1d(n * ((rows + 3) / 4), 256)), dim3(256), 0, s, 1, X, n, rows, rows,
-                        Rs + off * 2 * L.rowsp, L.rowsp, Stamp{}));
+      CKC(pack_rows(s, X, nullptr, n, rows, rows, nullptr, Rs + off * 2 * L.rowsp, L.rowsp, Stamp{}));
     if ((rc = split_product<F_ISTA0, F16>(ctx, off, n, Rs, WTs, cols, L.rowsp, ista(1, iX, &sc->iWT))) != SFB_OK) return rc;
   }
   for (int t = 2; t <= T; ++t) {
@@ -1064,10 +1152,9 @@ int begin_operands(sfb_ctx* ctx) {
     Pack16 p{};
     p.F = ctx->W; p.n = rows; p.dim = p.ld = cols; p.dst = Ws; p.dimp = L.colsp; p.inv = ctx->at<float>(L.iW);
     p.stamp = take_stamp(ctx);
-    CKC(pack16(s, p));
+    CKC(pack16(ctx, p));
   } else {
-    CKC(launch_kernel(pack_rows_kernel, dim3(grid1d(rows * cols / 4, 256)), dim3(256), 0, s, 1, ctx->W, rows, cols, cols, Ws,
-                      L.colsp, take_stamp(ctx)));
+    CKC(pack_rows(s, ctx->W, nullptr, rows, cols, cols, nullptr, Ws, L.colsp, take_stamp(ctx)));
   }
   if (c.model != SFB_SC) return SFB_OK;
   uint16_t* WTs = ctx->at<uint16_t>(L.WTs);
@@ -1158,15 +1245,14 @@ int split_logits(sfb_ctx* ctx, int64_t off, int64_t n, const float* X, const flo
   SplitParams p{};
   p.C = ctx->at<float>(L.U); p.ldc = L.ldu;
   if (!ctx->h16) {
-    CKC(launch_kernel(pack_pairs_kernel, dim3(grid1d(n * cols / 4, 256)), dim3(256), 0, ctx->stream, 1, X, Y, n, cols, V,
-                      As + off * 2 * L.colsp, L.colsp));
+    CKC(pack_rows(ctx->stream, X, Y, n, cols, cols, V, As + off * 2 * L.colsp, L.colsp, Stamp{}));
     return split_product<F_STORE, false>(ctx, off, n, As, ctx->at<uint16_t>(L.Ws), c.rows, L.colsp, p);
   }
   Pack16 k{};
   k.F = X; k.Y = Y; k.n = n; k.dim = k.ld = cols; k.V = V; k.dst = As + off * 2 * L.colsp; k.dimp = L.colsp;
   k.inv = ctx->at<float>(L.iA) + off;
   k.inv2 = ctx->at<float>(L.q) + off;                  // of u: |u| <= 1 for the logistic models; others set theirs later
-  CKC(pack16(ctx->stream, k));
+  CKC(pack16(ctx, k));
   p.ia = ctx->at<float>(L.iA); p.ib = ctx->at<float>(L.iW);
   return split_product<F_STORE, true>(ctx, off, n, As, ctx->at<uint16_t>(L.Ws), c.rows, L.colsp, p);
 }
@@ -1190,15 +1276,13 @@ int split_pack_received(sfb_ctx* ctx, int64_t off, int64_t n) {
   const float* V = ctx->at<float>(L.V) + off * c.cols;
   uint16_t* dst = const_cast<uint16_t*>(split_v(ctx)) + off * 2 * L.colsp;
   if (!ctx->h16) {
-    CKC(launch_kernel(pack_rows_kernel, dim3(grid1d(n * ((c.rows + 3) / 4), 256)), dim3(256), 0, s, 1, U, n, c.rows, L.ldu,
-                      ctx->at<uint16_t>(L.Rs) + off * 2 * L.rowsp, L.rowsp, Stamp{}));
-    CKC(launch_kernel(pack_rows_kernel, dim3(grid1d(n * c.cols / 4, 256)), dim3(256), 0, s, 1, V, n, c.cols, c.cols, dst, L.colsp,
-                      Stamp{}));
+    CKC(pack_rows(s, U, nullptr, n, c.rows, L.ldu, nullptr, ctx->at<uint16_t>(L.Rs) + off * 2 * L.rowsp, L.rowsp, Stamp{}));
+    CKC(pack_rows(s, V, nullptr, n, c.cols, c.cols, nullptr, dst, L.colsp, Stamp{}));
     return SFB_OK;
   }
   Pack16 k{};
   k.F = V; k.n = n; k.dim = k.ld = c.cols; k.dst = dst; k.dimp = L.colsp; k.inv = inv_v(ctx) + off;
-  CKC(pack16(s, k));
+  CKC(pack16(ctx, k));
   CKC(launch_kernel(row_most_kernel, dim3(static_cast<unsigned>(n)), dim3(256), 0, s, 1, U, L.ldu, c.rows, inv_v(ctx) + off,
                     ctx->at<float>(L.q) + off));
   return SFB_OK;
