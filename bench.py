@@ -252,17 +252,24 @@ def precision_code(S, name):
 
 
 def dtype_name(wl, name):
-    """The arithmetic type of the products: bf16, f32 (FFMA) or tf32x3 (fp32 values as pairs of tf32 words)."""
+    """The arithmetic type of the products: bf16, f32 (FFMA), or f16x3 / tf32x3 (fp32 values as pairs of fp16 or tf32 words)."""
     if name == "bf16":
         return "bf16"
-    return "tf32x3" if runs_tf32(wl, name) else "f32"
+    return "tf32x3" if runs_tf32(wl, name) else "f16x3" if runs_fp16_pairs(wl, name) else "f32"
 
 
 def runs_tf32(wl, name):
-    """Whether the fp32 mode runs this workload's products on the tensor cores (the library's own rule)."""
-    if wl.model != I.MLR or name in ("bf16", "ffma"):
+    return name == "tf32" and wl.model == I.MLR
+
+
+def runs_fp16_pairs(wl, name):
+    """Whether the fp32 mode runs this workload's products on the tensor cores as pairs of fp16 words (the library's own rule)."""
+    if name != "fp32" or wl.rows < 64 or wl.cols < 64:
         return False
-    return name == "tf32" or (wl.rows >= 2048 and wl.cols >= 512 and wl.K >= 128)
+    macs = float(wl.K) * wl.rows * wl.cols
+    if wl.model == I.SC:
+        return macs >= 2.8e8
+    return wl.cols >= 256 and (macs >= 1e9 or macs * (1 - 24 / wl.K) >= 1.8e8)
 
 
 NOMINAL_BF16_TFLOPS = 2250.0        # dense bf16, vendor figure (context only)
@@ -270,7 +277,7 @@ NOMINAL_TF32_OVER_BF16 = 1100.0 / 2250.0   # nominal ratio of the dense tf32 and
 NOMINAL_HBM_GBS = 7700.0
 
 
-def update_roofline(wl, prec_bf16, ms_u, peaks, clocks, sustained=True, tf32=False, copy_fraction=1.0):
+def update_roofline(wl, prec_bf16, ms_u, peaks, clocks, sustained=True, tf32=False, copy_fraction=1.0, pairs=False):
     """Roofline entry of the fused update W += -eta U^T V (one launch per step).  Algorithmic bytes per launch: W read
     and written once in fp32 plus U and V read once (what the method has to move).  The bf16 copy of W that this design
     writes alongside (the operand of the next forward product) is real traffic of the kernel and is reported beside
@@ -300,6 +307,11 @@ def update_roofline(wl, prec_bf16, ms_u, peaks, clocks, sustained=True, tf32=Fal
         roof = {"bound": "tensor", "achieved": 3.0 * upd_flops / (ms_u * 1e-3) / 1e12, "peak": peak, "unit": "TFLOP/s",
                 "note": "tf32 peak = measured bf16 x nominal ratio 1.1/2.25; achieved = executed flops (3 products per term)"}
         roof["roof_ms"] = max(3.0 * upd_flops / (peak * 1e12), upd_bytes / (peaks["hbm_gbs"] * 1e9)) * 1e3
+    elif pairs:
+        # fp32 operands as fp16 pairs: three products per term at the bf16 rate
+        roof = {"bound": "tensor", "achieved": 3.0 * upd_flops / (ms_u * 1e-3) / 1e12, "peak": tf_peak, "unit": "TFLOP/s",
+                "note": "achieved = executed flops (3 products per term)"}
+        roof["roof_ms"] = max(3.0 * upd_flops / (tf_peak * 1e12), upd_bytes / (peaks["hbm_gbs"] * 1e9)) * 1e3
     else:
         # fp32 FMA pipe: SMs x 128 lanes x 2 flop x max SM clock
         peak = 148 * 128 * 2 * ((clocks or {}).get("sm_max_mhz") or 1965.0) * 1e6 / 1e12
@@ -309,7 +321,7 @@ def update_roofline(wl, prec_bf16, ms_u, peaks, clocks, sustained=True, tf32=Fal
     roof["traffic"] = ncu_traffic_per_launch(wl, 0 if prec_bf16 else 1)
     roof["traffic_captured_at"] = NCU_UPDATE_TRAFFIC["kernel_unchanged_since"] if roof["traffic"] else None
     roof["kernel"] = "update_pair_kernel + label_rows_kernel (sfb_apply_update)" if prec_bf16 \
-        else "update_pair_kernel<tf32 pairs> (sfb_apply_update)" if tf32 else "sgemm_kernel EPI_RMW (sfb_apply_update)"
+        else "update_pair_kernel<tf32 pairs> (sfb_apply_update)" if tf32 else "update_split_kernel (sfb_apply_update)" if pairs else "sgemm_kernel EPI_RMW (sfb_apply_update)"
     roof["ms"] = ms_u
     roof["peaks"] = "of " + peaks["source"] + (" (sustained tensor figure: timed inside a long step)" if sustained
                                                else " (burst tensor figure: timed alone)")
@@ -425,7 +437,8 @@ def run_sharded(args, wl, rank, world, local):
     if rank == 0:
         value = K * args.steps / (total_ms * 1e-3)                          # one problem: K samples per step in all
         shard = I.scaled(wl, wl.name, rows=r1 - r0)
-        roof = update_roofline(shard, prec == S.PREC_BF16, ms_u, peaks, clocks, tf32=runs_tf32(shard, args.precision))
+        roof = update_roofline(shard, prec == S.PREC_BF16, ms_u, peaks, clocks, tf32=runs_tf32(shard, args.precision),
+                          pairs=runs_fp16_pairs(shard, args.precision))
         roof["traffic"] = None
         roof["traffic_captured_at"] = None
         model = exchange_model_bytes(wl.workers, wl.batch, wl.rows, wl.cols, world)
@@ -455,8 +468,8 @@ def main():
     ap.add_argument("--warmup", type=int, default=5)
     ap.add_argument("--impl", default="sfb", choices=["sfb", "reference"])
     ap.add_argument("--precision", default="bf16", choices=["bf16", "fp32", "tf32", "ffma"],
-                    help="bf16 operands (default); fp32 = the 1e-5 mode (tensor cores with tf32 pairs at large MLR "
-                         "shapes, FFMA otherwise); tf32 / ffma force either kernel family of that mode")
+                    help="bf16 operands (default); fp32 = the 1e-5 mode (tensor cores with fp16 pairs, "
+                         "FFMA for the smallest products); tf32 / ffma force either kernel family of that mode")
     ap.add_argument("--workload", default="mlr_large", choices=sorted(I.WORKLOADS))
     ap.add_argument("--no-cpu-baseline", action="store_true")
     ap.add_argument("--rows", type=int, default=0,
@@ -666,7 +679,7 @@ def main():
         update_loop = {"launches": reps, "ms": ms_loop, "seconds": ms_loop * reps * 1e-3, "clocks": ck,
                        "ms_x_sm_mhz": ms_loop * ck["sm_mhz"] if ck.get("sm_mhz") else None,
                        "roofline": update_roofline(wl, prec == S.PREC_BF16, ms_loop, peaks, ck,
-                                                   tf32=runs_tf32(wl, args.precision))}
+                                                   tf32=runs_tf32(wl, args.precision), pairs=runs_fp16_pairs(wl, args.precision))}
 
     # ---- end to end: host minibatch -> sfb_step_host -> loss back on the host, every step (sparse samples: the three
     # arrays and the labels copied from pinned memory, sfb_step_csr, the loss read back through sfb_get_stats)
@@ -735,7 +748,7 @@ def main():
         h2d = int(sum(8 * (K + 1) + 8 * n for _, _, _, n in hS) / nb) + K * 4
 
     # ---- roofline of the dominant kernel (the fused update), timed inside the long step: sustained tensor figure
-    roof = update_roofline(wl, prec == S.PREC_BF16, ms_u, peaks, clocks, tf32=runs_tf32(wl, args.precision),
+    roof = update_roofline(wl, prec == S.PREC_BF16, ms_u, peaks, clocks, tf32=runs_tf32(wl, args.precision), pairs=runs_fp16_pairs(wl, args.precision),
                            copy_fraction=min(1.0, copy_stats["rewritten_per_step"] / (wl.rows * math.ceil(wl.cols / 32)))
                            if copy_stats else 1.0)
     sparse_ran = sparse and st1.sparse_updates > st0.sparse_updates

@@ -42,8 +42,9 @@ enum sfb_model { SFB_MLR = 0, SFB_DML = 1, SFB_SC = 2, SFB_L2MLR = 3 };
  *                that cancels, so every product -- the forward W v, the products of the ISTA coder and the update --
  *                runs on the tensor cores with each value carried as a (hi, lo) pair of bf16, three bf16 products
  *                per term (about 2^-16 relative error per product).
- * SFB_PREC_FP32: fp32 operands.  MLR and SFB_L2MLR contexts of at least 2048 x 512 with K >= 128 run their two
- *                products on the tensor cores as SFB_PREC_TF32X3 does; everything else uses fp32 FMA kernels.
+ * SFB_PREC_FP32: fp32 operands.  Products large enough to repay the packing of their operands run on the tensor cores, every
+ *                value as a pair of fp16 words with a power-of-two scale per row (23 of its 24 bits, down to 2^-27 of the
+ *                row's largest entry), three fp16 products per term, partial sums in fp32; smaller ones on fp32 FMA kernels.
  * SFB_PREC_TF32X3: (MLR, SFB_L2MLR) fp32 operands on the tensor cores at any shape: every fp32 value x is carried as
  *                two tf32 words, big = tf32(x) and small = tf32(x - big), and a product runs as
  *                big*big + big*small + small*big with fp32 accumulation (relative error about 2^-21 per product);
@@ -135,8 +136,8 @@ int sfb_init(const sfb_config* cfg, float* W_dev, void* workspace_dev, size_t wo
  * Factors are written at the worker's row offset p*B of the gathered buffers.  All P workers of a step see the
  * same W (bulk-synchronous consistency, Section 4.1).
  * Copies of W that the library derives: in bf16 mode the forward product reads a bf16 operand copy of W.  DML and SC
- * rebuild theirs from W in the first factors call of every step.  MLR (and the tensor-core fp32 mode, whose copy is
- * the pair of tf32 words per entry) builds it once in sfb_init and afterwards the
+ * and SFB_PREC_FP32 rebuild theirs from W in the first factors call of every step.  MLR in bf16 mode (and with
+ * SFB_PREC_TF32X3, whose copy is the pair of tf32 words per entry) builds it once in sfb_init and afterwards the
  * update pass rewrites it together with W (W makes one trip through the SM per step), so it tracks every change the
  * LIBRARY makes to W -- but not writes the caller makes to W_dev between steps (loading weights, rescaling, a prox of
  * its own): after such a write call sfb_refresh_operands, or the next forward product runs on the stale copy. */
@@ -157,9 +158,9 @@ int sfb_compute_factors(sfb_ctx* ctx, int32_t worker, const float* X_dev, const 
  * be reused once later work on the stream may overwrite them.
  *
  * u is computed as for dense samples.  The logits need every column of W (the non-zero columns of a mini-batch cover
- * it), so in the tensor-core modes the forward product is the dense one over the scattered samples; in the fp32 FMA
- * mode it is a row-wise product over the non-zeros (z_ij = sum_t x_it W[j][c_it], rows of W held on chip, cols up to
- * about 55,000; the dense FMA product beyond).
+ * it), so on the tensor cores the forward product is the dense one over the scattered samples; on the fp32 FMA
+ * kernels it is that or a row-wise product over the non-zeros (z_ij = sum_t x_it W[j][c_it], rows of W held on chip, cols up
+ * to about 55,000), whichever is faster.
  * When every worker of the step committed in this form, sfb_gather_factors builds the column-major form of the K
  * samples (entries of a column in ascending sample order, so the result does not depend on scheduling) and
  * sfb_apply_update sums, per entry of W, only the samples that have a non-zero in that column:
@@ -169,7 +170,7 @@ int sfb_compute_factors(sfb_ctx* ctx, int32_t worker, const float* X_dev, const 
  * kernel's on-chip factor slab (K above about 1200 in the fp32 modes, 2400 in bf16 mode) takes the dense update, and
  * so does, unless cfg.csr_update says otherwise, one whose columns hold so many non-zeros that the tensor-core update
  * over the scattered samples is the faster of the two (in bf16 mode always up to K = 1024; in the fp32 modes from about
- * 30 non-zeros per column). */
+ * 30 non-zeros per column with tf32 pairs, fewer with fp16 pairs). */
 int sfb_compute_factors_csr(sfb_ctx* ctx, int32_t worker, const int64_t* indptr_dev, const int32_t* indices_dev,
                             const float* values_dev, int64_t nnz, const int32_t* labels_dev);
 
@@ -235,8 +236,7 @@ int sfb_apply_update(sfb_ctx* ctx);
 
 /* Re-derives the library's operand copies of W from the caller's W_dev (enqueued on the stream): to be called after
  * the caller itself has written W_dev between two steps.  MLR in bf16 mode: one conversion pass over W (reads 4,
- * writes 2 bytes per entry; 8 bytes in the tensor-core fp32 mode); a no-op for the other models and for the FFMA
- * kernels.  SFB_ERR_STATE in the middle of a step. */
+ * writes 2 bytes per entry; 8 bytes with SFB_PREC_TF32X3); a no-op for the other models and modes, which keep none.  SFB_ERR_STATE in the middle of a step. */
 int sfb_refresh_operands(sfb_ctx* ctx);
 
 /* Measurement hook (the paper has no counterpart): applies the factors gathered by the last completed step once
@@ -306,10 +306,10 @@ int sfb_dense_sync_step(sfb_ctx* ctx, const float* X_dev, const float* Y_dev, co
 int sfb_get_factors(sfb_ctx* ctx, const void** U_dev, const void** V_dev, int32_t* dtype, int32_t* layout,
                     int64_t* ldu, int64_t* ldv);
 
-/* The library's operand copy of W, for inspection: MLR in bf16 mode: dtype 1, the bf16 matrix [rows x ld]; the
- * tensor-core fp32 mode: dtype 2, fp32 words [rows x ld] holding tf32(w) at column c and tf32(w - tf32(w)) at column
- * ld/2 + c.  SFB_ERR_UNSUPPORTED where no persistent copy exists (the other models rebuild theirs every step; the FFMA
- * kernels read W itself). */
+/* The library's operand copy of W, for inspection: MLR in bf16 mode: dtype 1, the bf16 matrix [rows x ld]; with
+ * SFB_PREC_TF32X3: dtype 2, fp32 words [rows x ld] holding tf32(w) at column c and tf32(w - tf32(w)) at column
+ * ld/2 + c.  SFB_ERR_UNSUPPORTED where no persistent copy exists (the other models and SFB_PREC_FP32 rebuild theirs
+ * every step; the FFMA kernels read W itself). */
 int sfb_get_operand_copy(sfb_ctx* ctx, const void** copy_dev, int32_t* dtype, int64_t* ld);
 
 /* Waits for the stream, then fills the counters. */
