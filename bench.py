@@ -320,7 +320,7 @@ def update_roofline(wl, prec_bf16, ms_u, peaks, clocks, sustained=True, tf32=Fal
     roof["frac"] = roof["achieved"] / roof["peak"]
     roof["traffic"] = ncu_traffic_per_launch(wl, 0 if prec_bf16 else 1)
     roof["traffic_captured_at"] = NCU_UPDATE_TRAFFIC["kernel_unchanged_since"] if roof["traffic"] else None
-    roof["kernel"] = "update_pair_kernel + label_rows_kernel (sfb_apply_update)" if prec_bf16 \
+    roof["kernel"] = "update_pair_kernel (sfb_apply_update)" if prec_bf16 \
         else "update_pair_kernel<tf32 pairs> (sfb_apply_update)" if tf32 else "update_split_kernel (sfb_apply_update)" if pairs else "sgemm_kernel EPI_RMW (sfb_apply_update)"
     roof["ms"] = ms_u
     roof["peaks"] = "of " + peaks["source"] + (" (sustained tensor figure: timed inside a long step)" if sustained
@@ -760,7 +760,7 @@ def main():
         peak = peaks["hbm_gbs"]
         roof = {"bound": "hbm", "achieved": algo / (ms_u * 1e-3) / 1e9, "peak": peak, "unit": "GB/s",
                 "frac": algo / (ms_u * 1e-3) / 1e9 / peak, "traffic": None, "peak_source": peaks["source"],
-                "kernel": "sparse_update_kernel (+ label_rows_kernel in bf16 mode)", "ms": ms_u,
+                "kernel": "sparse_update_kernel", "ms": ms_u,
                 "algorithmic_bytes": algo, "fma_per_entry_of_W": nnz / wl.cols,
                 "note": "W read and written once in fp32, the factors u read once, 8 bytes per non-zero of v; "
                         "the operand copy of W is rewritten where its rounding changed (not counted)"}

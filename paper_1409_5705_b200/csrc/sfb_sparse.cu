@@ -551,7 +551,7 @@ void sparse_extend_layout(const sfb_config& c, Layout& L, size_t& off) {
 // sparse update costs a fixed 1.0 for its pass over W in bf16 mode (0.83 where the operand copy hardly changes, 1.4 at
 // 10,000 x 20,000 where all of it does, and the column-major form of the samples comes on top) and 1.57 in the tensor-core
 // fp32 mode, whose 8-byte operand copy it also writes, plus 0.089 per non-zero of an average column; the dense update costs
-// K/1024 in bf16 mode, 4.4 K/1024 with tf32 pairs, and far more on the FMA kernels.
+// K/1024 in bf16 mode, 4.4 K/1024 with tf32 pairs, 2.2 K/1024 with fp16 pairs, and far more on the FMA kernels.
 bool sparse_update_wanted(const sfb_ctx* ctx) {
   const sfb_config& c = ctx->cfg;
   const bool bf16 = c.precision == SFB_PREC_BF16;

@@ -119,7 +119,7 @@ __device__ __forceinline__ float4 scale4(float4 v, float s) { return make_float4
 // has a run of them that begins within one tile and ends within another (or the same).  The part at the end of a run, which
 // does not reach the end of its tile, is computed first and left in memory; the part at the beginning, which completes a tile,
 // last: the parts that it waits for come from the pairs before this one.  The sums are in the order of the pairs, so they do
-// not depend on timing.  512 x 5,000 over 5,000 (40 tiles of 256 x 256 on 74 pairs): see below.
+// not depend on timing.
 // Warps: 0 TMA producer, 1 MMA issuer (leader CTA) and TMEM owner, 4..11 epilogue; the first four give their registers to
 // the epilogue (384 threads x 168 = 128 x 40 + 256 x 232).
 // Rates: see pair_cost.

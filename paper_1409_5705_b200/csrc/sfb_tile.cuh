@@ -10,8 +10,7 @@ namespace sfb {
 
 // Exchange of the partial tiles of a split contraction through the shared memory of the cluster's CTAs, in chunks of 32
 // columns x 128 rows of fp32 (16 KB, the operand stages' memory, which nothing uses any more); a warp writes and reads its 32
-// rows with the 16-byte pieces of a row swizzled.  The parts are in the CTAs of rank first, first + step, ...; each of them
-// finishes every parts-th chunk.  The sums are in rank order, so they do not depend on timing.
+// rows with the 16-byte pieces of a row swizzled.  Each of them finishes every parts-th chunk.  The sums are in rank order, so they do not depend on timing.
 constexpr int kXchgCols = 32;
 constexpr int kXchgBytes = 128 * kXchgCols * 4;
 // the 16-byte piece j of a row of 32 fp32 values
@@ -30,13 +29,13 @@ __device__ __forceinline__ void slot_put(uint32_t base, int row, const uint32_t 
 __device__ __forceinline__ void xchg_put(uint8_t* smem, int c, int row, const uint32_t (&acc)[32]) {
   slot_put(ptx::smem_u32(smem) + c * kXchgBytes, row, acc);
 }
-__device__ __forceinline__ void xchg_sum(uint8_t* smem, int c, int row, int parts, int first, int step, uint32_t (&acc)[32]) {
+__device__ __forceinline__ void xchg_sum(uint8_t* smem, int c, int row, int parts, uint32_t (&acc)[32]) {
 #pragma unroll
   for (int j = 0; j < 8; ++j) {
     const uint32_t at = xchg_addr(smem, c, row, j);
-    float4 s = ptx::ld_cluster_f4(at, first);
+    float4 s = ptx::ld_cluster_f4(at, 0);
     for (int g = 1; g < parts; ++g) {
-      const float4 v = ptx::ld_cluster_f4(at, first + g * step);
+      const float4 v = ptx::ld_cluster_f4(at, g);
       s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w;
     }
     acc[4 * j] = __float_as_uint(s.x); acc[4 * j + 1] = __float_as_uint(s.y);
