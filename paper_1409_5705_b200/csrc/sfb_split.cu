@@ -814,7 +814,8 @@ __global__ void __launch_bounds__(256) pack16_kernel(const __grid_constant__ Pac
 }
 
 // The same for long rows, which come through shared memory: a block has the next rows under way by bulk copies while it looks for
-// the largest entry of one and converts it.  (Held in registers, a row's loads and stores took turns: 10,000 x 20,000 in 603 us.)
+// the largest entry of one and converts it.  (Held in registers, a row's loads and stores took turns: 10,000 x 20,000 in 603 us,
+// 290 now.  With Y both rows come; if only one such pair fits, its stores at least drain beside the next loads.)
 constexpr int kPackRoom = 208 << 10, kPackThreads = 512, kPackBufs = 4;
 __global__ void __launch_bounds__(kPackThreads, 1) pack16_long_kernel(const __grid_constant__ Pack16 p, int bufs, uint32_t* status) {
   extern __shared__ __align__(128) uint8_t rows_smem[];
@@ -823,7 +824,7 @@ __global__ void __launch_bounds__(kPackThreads, 1) pack16_long_kernel(const __gr
   __shared__ uint32_t abort_word;
   pdl_launch_dependents();
   const int t = threadIdx.x, quads = static_cast<int>(p.dim / 4);
-  const uint32_t bytes = static_cast<uint32_t>(p.dim) * 4;
+  const uint32_t bytes = static_cast<uint32_t>(p.dim) * 4, buf_bytes = (p.Y ? 2 : 1) * bytes;
   if (t == 0) {
     for (int i = 0; i < kPackBufs; ++i) mbar_init(&full[i], 1);
     abort_word = 0;
@@ -833,8 +834,9 @@ __global__ void __launch_bounds__(kPackThreads, 1) pack16_long_kernel(const __gr
   pdl_wait();
   stamp_begin(p.stamp);
   auto ask = [&](int64_t r, int b) {
-    mbar_expect_tx(&full[b], bytes);
-    bulk_load(smem_u32(rows_smem) + b * bytes, p.F + r * p.ld, bytes, &full[b]);
+    mbar_expect_tx(&full[b], buf_bytes);
+    bulk_load(smem_u32(rows_smem) + b * buf_bytes, p.F + r * p.ld, bytes, &full[b]);
+    if (p.Y) bulk_load(smem_u32(rows_smem) + b * buf_bytes + bytes, p.Y + r * p.ld, bytes, &full[b]);
   };
   const int64_t step = gridDim.x;
   if (t == 0)
@@ -847,10 +849,16 @@ __global__ void __launch_bounds__(kPackThreads, 1) pack16_long_kernel(const __gr
       for (int i = 0; i < 64; ++i) __nanosleep(1000);  // for copies in flight
       return;
     }
-    const float4* row = reinterpret_cast<const float4*>(rows_smem + b * bytes);
+    float4* row = reinterpret_cast<float4*>(rows_smem + b * buf_bytes);
+    const float4* sub = row + quads;
     float m = 0.f, ss = 0.f;
     for (int q = t; q < quads; q += kPackThreads) {
-      const float4 v = row[q];
+      float4 v = row[q];
+      if (p.Y) {
+        const float4 y = sub[q];
+        v = make_float4(v.x - y.x, v.y - y.y, v.z - y.z, v.w - y.w);
+        row[q] = v;                                    // (this thread reads it again)
+      }
       m = fmaxf(m, fmaxf(fmaxf(fabsf(v.x), fabsf(v.y)), fmaxf(fabsf(v.z), fabsf(v.w))));
       if (p.inv_res) ss = fmaf(v.x, v.x, fmaf(v.y, v.y, fmaf(v.z, v.z, fmaf(v.w, v.w, ss))));
     }
@@ -874,6 +882,7 @@ __global__ void __launch_bounds__(kPackThreads, 1) pack16_long_kernel(const __gr
       if (v4) v4[q] = v;
       put_pair4<true>(d + 4 * q, p.dimp, scale4(v, s));
     }
+    if (p.Y) fence_proxy_async_smem();                 // (written to, and to be overwritten by a copy)
     __syncthreads();                                   // the row (and sh) has been read
     if (t == 0 && r + bufs * step < p.n) ask(r + bufs * step, b);
     if (++b == bufs) { b = 0; ph ^= 1; }
@@ -1041,13 +1050,14 @@ cudaError_t pack16(sfb_ctx* ctx, const Pack16& p) {
   cudaStream_t s = ctx->stream;
   if (p.n <= 0) return cudaSuccess;
   if (p.dim <= 2048) return launch_kernel(pack16_kernel<32>, dim3(static_cast<unsigned>((p.n + 7) / 8)), dim3(256), 0, s, 1, p);
-  const int bufs = static_cast<int>(std::min<int64_t>(kPackBufs, kPackRoom / (p.dim * 4)));
-  if (bufs < 2 || p.Y || p.dim % 4 != 0 || p.ld % 4 != 0)
+  const int64_t buf = p.dim * (p.Y ? 8 : 4);
+  const int bufs = static_cast<int>(std::min<int64_t>(kPackBufs, kPackRoom / buf));
+  if (bufs < (p.Y ? 1 : 2) || p.dim % 4 != 0 || p.ld % 4 != 0)
     return launch_kernel(pack16_kernel<256>, dim3(static_cast<unsigned>(p.n)), dim3(256), 0, s, 1, p);
   const cudaError_t e = allow_smem<pack16_long_kernel>(kPackRoom);
   if (e != cudaSuccess) return e;
   return launch_kernel(pack16_long_kernel, dim3(static_cast<unsigned>(std::min<int64_t>(p.n, sm_count()))), dim3(kPackThreads),
-                       static_cast<int>(bufs * p.dim * 4), s, 1, p, bufs, ctx->at<uint32_t>(ctx->lay.status));
+                       static_cast<int>(bufs * buf), s, 1, p, bufs, ctx->at<uint32_t>(ctx->lay.status));
 }
 
 // bf16 form; Y: subtracted, the difference also to V.

@@ -57,7 +57,6 @@ struct TcParams {
   int32_t a_off0, a_off1, a_off2, b_off0, b_off1, b_off2;
   float2* part;                // F_SOFTMAX: [N / pw][part_ld] (max, sum exp) per sample and pw rows of W
   int64_t part_ld;
-  int32_t prefetch;            // k-blocks by which the producer asks L2 for the B operand ahead of its loads (0: off)
   int32_t kparts;              // the contraction of a tile is cut over a cluster of this many CTAs (1: persistent CTAs)
   uint32_t* status;
 };
@@ -129,10 +128,6 @@ forward_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
           const int kl1 = min(p.kseg, kend - seg * p.kseg);
           for (int kl = max(0, kbeg - seg * p.kseg); kl < kl1; ++kl) {
             if (!mbar_wait(&empty[s], ph ^ 1, abort_flag)) { ok = false; break; }
-            // B streams from HBM when it is larger than L2: with the box asked for a few k-blocks early, the load
-            // that fills the stage finds it in L2 and the four stages cover the latency
-            if (p.prefetch > 0 && kl + p.prefetch < p.kseg)
-              tma_prefetch_2d(&tmB, xb0 + (kl + p.prefetch) * (TF32 ? BK / 2 : BK), n0);
             uint8_t* st = smem + s * stage_bytes;
             mbar_expect_tx(&full[s], (p.a_rows + p.bn) * BK * 2);
             tma_load_2d_hint(st, &tmA, xa0 + kl * (TF32 ? BK / 2 : BK), m0, &full[s], pol_keep);
