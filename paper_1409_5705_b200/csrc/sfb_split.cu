@@ -659,8 +659,8 @@ __global__ void __launch_bounds__(256) pack_t_kernel(const float* __restrict__ F
 }
 
 // bf16 form: rows of F (or of F - Y, which then also go to V in fp32) -> the operand [n x 2*dimp].  TPR threads per row, four
-// quads of columns each at a time.  Columns dim..dimp-1 are left as they are (zero since set-up).  (Over one index for the whole
-// matrix, each quad paid for a 64-bit division: 1,000 x 20,000 47 us, 10,000 x 5,000 109.)
+// quads of columns each at a time.  Columns dim..dimp-1 are left as they are (zero since set-up).  For the rows that
+// pack_long_kernel does not take (1,000 x 20,000 there: 49 -> 42 us).
 template <int TPR, bool SUB>
 __global__ void __launch_bounds__(256) pack_rows_kernel(const float* __restrict__ F, const float* __restrict__ Y, int64_t n, int dim,
                                                         int64_t ld, float* __restrict__ V, uint16_t* __restrict__ dst, int64_t dimp,
@@ -813,11 +813,12 @@ __global__ void __launch_bounds__(256) pack16_kernel(const __grid_constant__ Pac
   }
 }
 
-// The same for long rows, which come through shared memory: a block has the next rows under way by bulk copies while it looks for
+// The same (and the bf16 form, which needs no scale) for long rows, which come through shared memory: a block has the next rows under way by bulk copies while it looks for
 // the largest entry of one and converts it.  (Held in registers, a row's loads and stores took turns: 10,000 x 20,000 in 603 us,
 // 290 now.  With Y both rows come; if only one such pair fits, its stores at least drain beside the next loads.)
 constexpr int kPackRoom = 208 << 10, kPackThreads = 512, kPackBufs = 4;
-__global__ void __launch_bounds__(kPackThreads, 1) pack16_long_kernel(const __grid_constant__ Pack16 p, int bufs, uint32_t* status) {
+template <bool F16>
+__global__ void __launch_bounds__(kPackThreads, 1) pack_long_kernel(const __grid_constant__ Pack16 p, int bufs, uint32_t* status) {
   extern __shared__ __align__(128) uint8_t rows_smem[];
   __shared__ __align__(8) uint64_t full[kPackBufs];
   __shared__ float sh[2 * kPackThreads / 32];
@@ -851,38 +852,45 @@ __global__ void __launch_bounds__(kPackThreads, 1) pack16_long_kernel(const __gr
     }
     float4* row = reinterpret_cast<float4*>(rows_smem + b * buf_bytes);
     const float4* sub = row + quads;
-    float m = 0.f, ss = 0.f;
-    for (int q = t; q < quads; q += kPackThreads) {
-      float4 v = row[q];
-      if (p.Y) {
-        const float4 y = sub[q];
-        v = make_float4(v.x - y.x, v.y - y.y, v.z - y.z, v.w - y.w);
-        row[q] = v;                                    // (this thread reads it again)
+    float s = 1.f;
+    if constexpr (F16) {
+      float m = 0.f, ss = 0.f;
+      for (int q = t; q < quads; q += kPackThreads) {
+        float4 v = row[q];
+        if (p.Y) {
+          const float4 y = sub[q];
+          v = make_float4(v.x - y.x, v.y - y.y, v.z - y.z, v.w - y.w);
+          row[q] = v;                                    // (this thread reads it again)
+        }
+        m = fmaxf(m, fmaxf(fmaxf(fabsf(v.x), fabsf(v.y)), fmaxf(fabsf(v.z), fabsf(v.w))));
+        if (p.inv_res) ss = fmaf(v.x, v.x, fmaf(v.y, v.y, fmaf(v.z, v.z, fmaf(v.w, v.w, ss))));
       }
-      m = fmaxf(m, fmaxf(fmaxf(fabsf(v.x), fabsf(v.y)), fmaxf(fabsf(v.z), fabsf(v.w))));
-      if (p.inv_res) ss = fmaf(v.x, v.x, fmaf(v.y, v.y, fmaf(v.z, v.z, fmaf(v.w, v.w, ss))));
-    }
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-      ss += __shfl_xor_sync(0xffffffffu, ss, o);
-    }
-    constexpr int kWarps = kPackThreads / 32;
-    if ((t & 31) == 0) { sh[t >> 5] = m; sh[kWarps + (t >> 5)] = ss; }
-    __syncthreads();
-    m = sh[0]; ss = sh[kWarps];
+      for (int o = 16; o > 0; o >>= 1) {
+        m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+        ss += __shfl_xor_sync(0xffffffffu, ss, o);
+      }
+      constexpr int kWarps = kPackThreads / 32;
+      if ((t & 31) == 0) { sh[t >> 5] = m; sh[kWarps + (t >> 5)] = ss; }
+      __syncthreads();
+      m = sh[0]; ss = sh[kWarps];
 #pragma unroll
-    for (int w = 1; w < kWarps; ++w) { m = fmaxf(m, sh[w]); ss += sh[kWarps + w]; }
-    const float s = pow2_scale(m, 13);
-    if (t == 0) row_scales(p, r, s, ss);
+      for (int w = 1; w < kWarps; ++w) { m = fmaxf(m, sh[w]); ss += sh[kWarps + w]; }
+      s = pow2_scale(m, 13);
+      if (t == 0) row_scales(p, r, s, ss);
+    }
     uint16_t* d = p.dst + r * 2 * p.dimp;
     float4* v4 = p.V ? reinterpret_cast<float4*>(p.V + r * p.dim) : nullptr;
     for (int q = t; q < quads; q += kPackThreads) {
-      const float4 v = row[q];
+      float4 v = row[q];
+      if (!F16 && p.Y) {
+        const float4 y = sub[q];
+        v = make_float4(v.x - y.x, v.y - y.y, v.z - y.z, v.w - y.w);
+      }
       if (v4) v4[q] = v;
-      put_pair4<true>(d + 4 * q, p.dimp, scale4(v, s));
+      put_pair4<F16>(d + 4 * q, p.dimp, F16 ? scale4(v, s) : v);
     }
-    if (p.Y) fence_proxy_async_smem();                 // (written to, and to be overwritten by a copy)
+    if (F16 && p.Y) fence_proxy_async_smem();                 // (written to, and to be overwritten by a copy)
     __syncthreads();                                   // the row (and sh) has been read
     if (t == 0 && r + bufs * step < p.n) ask(r + bufs * step, b);
     if (++b == bufs) { b = 0; ph ^= 1; }
@@ -1046,24 +1054,35 @@ int split_product(sfb_ctx* ctx, int64_t off, int64_t n, const uint16_t* A, const
   return SFB_OK;
 }
 
-cudaError_t pack16(sfb_ctx* ctx, const Pack16& p) {
-  cudaStream_t s = ctx->stream;
-  if (p.n <= 0) return cudaSuccess;
-  if (p.dim <= 2048) return launch_kernel(pack16_kernel<32>, dim3(static_cast<unsigned>((p.n + 7) / 8)), dim3(256), 0, s, 1, p);
+// Long rows with 16-byte pieces; false: the caller has to take another kernel.
+template <bool F16>
+bool pack_long(sfb_ctx* ctx, const Pack16& p, cudaError_t& e) {
   const int64_t buf = p.dim * (p.Y ? 8 : 4);
   const int bufs = static_cast<int>(std::min<int64_t>(kPackBufs, kPackRoom / buf));
-  if (bufs < (p.Y ? 1 : 2) || p.dim % 4 != 0 || p.ld % 4 != 0)
-    return launch_kernel(pack16_kernel<256>, dim3(static_cast<unsigned>(p.n)), dim3(256), 0, s, 1, p);
-  const cudaError_t e = allow_smem<pack16_long_kernel>(kPackRoom);
-  if (e != cudaSuccess) return e;
-  return launch_kernel(pack16_long_kernel, dim3(static_cast<unsigned>(std::min<int64_t>(p.n, sm_count()))), dim3(kPackThreads),
-                       static_cast<int>(bufs * buf), s, 1, p, bufs, ctx->at<uint32_t>(ctx->lay.status));
+  if (p.dim <= 2048 || bufs < (p.Y ? 1 : 2) || p.dim % 4 != 0 || p.ld % 4 != 0) return false;
+  if ((e = allow_smem<pack_long_kernel<F16>>(kPackRoom)) == cudaSuccess)
+    e = launch_kernel(pack_long_kernel<F16>, dim3(static_cast<unsigned>(std::min<int64_t>(p.n, sm_count()))), dim3(kPackThreads),
+                      static_cast<int>(bufs * buf), ctx->stream, 1, p, bufs, ctx->at<uint32_t>(ctx->lay.status));
+  return true;
+}
+cudaError_t pack16(sfb_ctx* ctx, const Pack16& p) {
+  cudaStream_t s = ctx->stream;
+  cudaError_t e = cudaSuccess;
+  if (p.n <= 0) return cudaSuccess;
+  if (p.dim <= 2048) return launch_kernel(pack16_kernel<32>, dim3(static_cast<unsigned>((p.n + 7) / 8)), dim3(256), 0, s, 1, p);
+  if (pack_long<true>(ctx, p, e)) return e;
+  return launch_kernel(pack16_kernel<256>, dim3(static_cast<unsigned>(p.n)), dim3(256), 0, s, 1, p);
 }
 
 // bf16 form; Y: subtracted, the difference also to V.
-cudaError_t pack_rows(cudaStream_t s, const float* F, const float* Y, int64_t n, int64_t dim, int64_t ld, float* V, uint16_t* dst,
+cudaError_t pack_rows(sfb_ctx* ctx, const float* F, const float* Y, int64_t n, int64_t dim, int64_t ld, float* V, uint16_t* dst,
                       int64_t dimp, const Stamp& stamp) {
+  cudaStream_t s = ctx->stream;
+  cudaError_t e = cudaSuccess;
   if (n <= 0) return cudaSuccess;
+  Pack16 p{};
+  p.F = F; p.Y = Y; p.n = n; p.dim = dim; p.ld = ld; p.V = V; p.dst = dst; p.dimp = dimp; p.stamp = stamp;
+  if (pack_long<false>(ctx, p, e)) return e;
   auto go = [&](auto kernel, int tpr) {
     return launch_kernel(kernel, dim3(static_cast<unsigned>((n + 256 / tpr - 1) / (256 / tpr))), dim3(256), 0, s, 1, F, Y, n,
                          static_cast<int>(dim), ld, V, dst, dimp, stamp);
@@ -1132,10 +1151,10 @@ int factors_sc(sfb_ctx* ctx, int64_t off, int64_t n, const float* X) {
     e.sc = sc; e.lam = c.sc_lambda;
     CKC(sgemm(s, true, false, EPI_ISTA0, n, cols, rows, X, rows, ctx->W, cols, e, ctx->K));
     ctx->stats.flops += 2.0 * n * rows * cols;
-    CKC(pack_rows(s, V + off * cols, nullptr, n, cols, cols, nullptr, as[1] + off * 2 * L.colsp, L.colsp, Stamp{}));
+    CKC(pack_rows(ctx, V + off * cols, nullptr, n, cols, cols, nullptr, as[1] + off * 2 * L.colsp, L.colsp, Stamp{}));
   } else {
     if (!F16)
-      CKC(pack_rows(s, X, nullptr, n, rows, rows, nullptr, Rs + off * 2 * L.rowsp, L.rowsp, Stamp{}));
+      CKC(pack_rows(ctx, X, nullptr, n, rows, rows, nullptr, Rs + off * 2 * L.rowsp, L.rowsp, Stamp{}));
     if ((rc = split_product<F_ISTA0, F16>(ctx, off, n, Rs, WTs, cols, L.rowsp, ista(1, iX, &sc->iWT))) != SFB_OK) return rc;
   }
   for (int t = 2; t <= T; ++t) {
@@ -1164,7 +1183,7 @@ int begin_operands(sfb_ctx* ctx) {
     p.stamp = take_stamp(ctx);
     CKC(pack16(ctx, p));
   } else {
-    CKC(pack_rows(s, ctx->W, nullptr, rows, cols, cols, nullptr, Ws, L.colsp, take_stamp(ctx)));
+    CKC(pack_rows(ctx, ctx->W, nullptr, rows, cols, cols, nullptr, Ws, L.colsp, take_stamp(ctx)));
   }
   if (c.model != SFB_SC) return SFB_OK;
   uint16_t* WTs = ctx->at<uint16_t>(L.WTs);
@@ -1255,7 +1274,7 @@ int split_logits(sfb_ctx* ctx, int64_t off, int64_t n, const float* X, const flo
   SplitParams p{};
   p.C = ctx->at<float>(L.U); p.ldc = L.ldu;
   if (!ctx->h16) {
-    CKC(pack_rows(ctx->stream, X, Y, n, cols, cols, V, As + off * 2 * L.colsp, L.colsp, Stamp{}));
+    CKC(pack_rows(ctx, X, Y, n, cols, cols, V, As + off * 2 * L.colsp, L.colsp, Stamp{}));
     return split_product<F_STORE, false>(ctx, off, n, As, ctx->at<uint16_t>(L.Ws), c.rows, L.colsp, p);
   }
   Pack16 k{};
@@ -1286,8 +1305,8 @@ int split_pack_received(sfb_ctx* ctx, int64_t off, int64_t n) {
   const float* V = ctx->at<float>(L.V) + off * c.cols;
   uint16_t* dst = const_cast<uint16_t*>(split_v(ctx)) + off * 2 * L.colsp;
   if (!ctx->h16) {
-    CKC(pack_rows(s, U, nullptr, n, c.rows, L.ldu, nullptr, ctx->at<uint16_t>(L.Rs) + off * 2 * L.rowsp, L.rowsp, Stamp{}));
-    CKC(pack_rows(s, V, nullptr, n, c.cols, c.cols, nullptr, dst, L.colsp, Stamp{}));
+    CKC(pack_rows(ctx, U, nullptr, n, c.rows, L.ldu, nullptr, ctx->at<uint16_t>(L.Rs) + off * 2 * L.rowsp, L.rowsp, Stamp{}));
+    CKC(pack_rows(ctx, V, nullptr, n, c.cols, c.cols, nullptr, dst, L.colsp, Stamp{}));
     return SFB_OK;
   }
   Pack16 k{};
