@@ -162,7 +162,20 @@ struct Scalars {                      // device-resident scalars
 
 }  // namespace sfb
 
+namespace sfb {
+// For sfb_step_host, made by its first call: a stream for the copies of the mini-batch's parts, an event per part (and one for the
+// work ahead of the call), page-locked memory for what is read back.
+struct HostSide {
+  static constexpr int kParts = 8;
+  cudaStream_t copies;
+  cudaEvent_t ahead, part[kParts];
+  char* back;
+  int parts;                          // of the call that is being enqueued (0: none, the samples are there)
+};
+}  // namespace sfb
+
 struct sfb_ctx {
+  sfb::HostSide* host;
   sfb_config cfg;
   sfb::Layout lay;
   float* W;

@@ -1235,6 +1235,25 @@ int tc_sdca_factors(sfb_ctx* ctx, int64_t off, int64_t n, const float* X, const 
   return SFB_OK;
 }
 
+// Parts of at least 128 samples: copied at about 45 GB/s; a part's product takes its tensor work or one pass over the bf16 W.  With
+// the copies and the products in line, first copy + the slower of the two per part + last product is what passes.
+int tc_host_parts(const sfb_ctx* ctx) {
+  const sfb_config& c = ctx->cfg;
+  if (c.model != SFB_MLR || c.precision != SFB_PREC_BF16 || ctx->lay.split > 1) return 1;
+  auto total = [&](int parts) {
+    const int64_t n = ctx->K / parts;
+    const double copy = 4.0 * static_cast<double>(n) * static_cast<double>(c.cols) / 45e9 + 4e-6;
+    const double cycles = forward_cost(n, c.rows, c.cols, pick_forward_width(n, c.rows, c.cols, ctx->lay.pw, 1), 1);
+    const double product = std::max(cycles / 1.7e9, 2.0 * static_cast<double>(c.rows) * static_cast<double>(c.cols) / 5e12) + 5e-6;
+    // (a product that takes much longer than its copy has little to gain, and a pass over W per part to lose)
+    return parts > 1 && product > 2. * copy ? 1e9 : copy + (parts - 1) * std::max(copy, product) + product;
+  };
+  int best = 1;
+  for (int parts = 2; parts <= HostSide::kParts && ctx->K % (parts * BM) == 0; parts *= 2)
+    if (total(parts) < 0.95 * total(best)) best = parts;
+  return best;
+}
+
 int tc_factors(sfb_ctx* ctx, int64_t off, int64_t n, const float* X, const float* Y, const int32_t* labels, bool fused,
                float* dml_norm_out) {
   if (ctx->cfg.model == SFB_SC) return split_factors_sc(ctx, off, n, X);
@@ -1253,8 +1272,13 @@ int tc_factors(sfb_ctx* ctx, int64_t off, int64_t n, const float* X, const float
   float* Z = ctx->at<float>(L.ZT);
   float* lse = ctx->at<float>(L.V);
   int tiles_n = 0;
-  const int rc = mlr_forward(ctx, off, n, X, labels, fused, &tiles_n);
-  if (rc) return rc;
+  const int parts = ctx->host && ctx->host->parts > 1 ? ctx->host->parts : 1;
+  for (int i = 0; i < parts; ++i) {                     // (parts: of samples that are still on their way, see sfb_step_host)
+    const int64_t m = n / parts;
+    if (parts > 1) CKC(cudaStreamWaitEvent(ctx->stream, ctx->host->part[i], 0));
+    const int rc = mlr_forward(ctx, off + i * m, m, X + i * m * c.cols, labels + i * m, fused, &tiles_n);
+    if (rc) return rc;
+  }
   if (!fused && n <= 65535) {
     const int64_t most = (rows + 2047) / 2048, want = (4 * sm_count() + n - 1) / n;      // blocks of at least one pass over 2,048 classes
     CKC(launch_kernel(mlr_lse_emit_kernel, dim3(static_cast<unsigned>(std::min(most, want)), static_cast<unsigned>(n)), dim3(256), 0,

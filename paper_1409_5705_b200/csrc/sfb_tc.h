@@ -28,6 +28,8 @@ int tc_factors(sfb_ctx* ctx, int64_t off, int64_t n, const float* X, const float
                float* dml_norm_out = nullptr);
 // Row-sharded MLR: logits and softmax partials of all K samples against this context's rows; then the factors from
 // the partials of all shards.
+// Parts in which sfb_step_host had better copy the K samples of MLR in bf16 mode (their logits follow part by part).
+int tc_host_parts(const sfb_ctx* ctx);
 int tc_forward_partials(sfb_ctx* ctx, const float* X, const int32_t* labels, float* part_out);
 int tc_finish_factors(sfb_ctx* ctx, const float* parts, int shards);
 int tc_sdca_factors(sfb_ctx* ctx, int64_t off, int64_t n, const float* X, const int32_t* labels, const int32_t* ids,
