@@ -169,3 +169,21 @@ def test_dual_solve_at_the_edge_of_shared_memory(classes):
         err = np.linalg.norm(W.cpu().numpy().astype(np.float64) - W_ref.astype(np.float32)) / np.linalg.norm(W_ref - W_t)
         assert err <= TOL[S.PREC_FP32] and np.abs(Q.cpu().numpy() - Q_ref).max() <= 2e-6
     ctx.close()
+
+
+# Samples from host memory: copied in parts beside the products of the parts before them (several times 128 samples), in one piece.
+@pytest.mark.parametrize("shape", [(2000, 8000, 4, 64), (1000, 8000, 1, 384), (333, 260, 3, 37)])
+def test_host_samples_in_parts(shape):
+    wl = workload("mlr", *shape, w_std=0.01)
+    W0, inp = I.initial_W(wl), I.step_inputs(wl, 1)
+    W = to_dev(W0, torch)
+    ctx = S.Context(config_for(wl, S.PREC_BF16), W)
+    X, lab = torch.from_numpy(inp.X).pin_memory(), torch.from_numpy(inp.labels).pin_memory()
+    Wt = W0
+    for _ in range(2):                                          # the second step copies over the first one's samples
+        loss, status = ctx.sfb_step_host(X, None, lab)
+        ref, Wg = oracle_step(wl, Wt, inp), W.cpu().numpy()
+        assert status == 0 and abs(loss - O.mlr_loss(Wt, inp.X, inp.labels).mean()) < 1e-3
+        assert rel_err(Wg, ref, Wt) <= TOL[S.PREC_BF16]
+        Wt = Wg
+    ctx.close()
