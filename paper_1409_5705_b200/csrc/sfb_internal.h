@@ -143,8 +143,9 @@ inline int64_t round_up(int64_t x, int64_t m) { return (x + m - 1) / m * m; }
 inline bool use_tf32(const sfb_config& c) {
   return c.precision == SFB_PREC_TF32X3 && (c.model == SFB_MLR || c.model == SFB_L2MLR);
 }
+bool sparse_on_fma(const sfb_config& c);      // sparse samples: see sfb_sparse.cu
 inline bool use_h16(const sfb_config& c) {
-  if (c.precision != SFB_PREC_FP32 || c.rows < 64 || c.cols < 64) return false;
+  if (c.precision != SFB_PREC_FP32 || c.rows < 64 || c.cols < 64 || sparse_on_fma(c)) return false;
   const double K = static_cast<double>(c.workers) * c.batch, macs = K * static_cast<double>(c.rows) * static_cast<double>(c.cols);
   if (c.model == SFB_SC) return macs >= 2.8e8;
   return c.cols >= 256 && (macs >= 1e9 || macs * (1.0 - 24.0 / K) >= 1.8e8);

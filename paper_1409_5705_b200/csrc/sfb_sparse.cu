@@ -12,8 +12,10 @@
 #include <cuda_bf16.h>
 
 #include <algorithm>
+#include <cmath>
 
 #include "sfb_internal.h"
+#include "sfb_tc.h"
 
 namespace sfb {
 
@@ -607,32 +609,46 @@ int forward_pitch(int64_t cols, int rb) {
 }  // namespace
 
 // Rows of W a block of the row-wise forward can hold (4, 2 or 1), or 0 when even one row does not fit.
-int sparse_forward_rows(const sfb_ctx* ctx, int64_t n) {
+int sparse_forward_rows(const sfb_config& c, int64_t n) {
   for (int rb = 4; rb >= 1; rb >>= 1) {
-    const int64_t bytes = static_cast<int64_t>(rb) * forward_pitch(ctx->cfg.cols, rb) * 4 + n * 8 + kSfWarps * kSfBufs * kSfChunk * 8;
+    const int64_t bytes = static_cast<int64_t>(rb) * forward_pitch(c.cols, rb) * 4 + n * 8 + kSfWarps * kSfBufs * kSfChunk * 8;
     if (bytes <= kSmemOptIn) return rb;
   }
   return 0;
 }
 
-// Whether the row-wise forward is faster than the FMA product over the scattered samples, both in SM cycles.  Row-wise: a block's
-// 16 warps take the samples in turn, 900 cycles each and 40 more per entry and lane group, for rb rows of W at a time.
-// 91,238 x 148, K = 176, 13 entries: 1,770,000 cycles against 160,000.  For the whole mini-batch and the room for its entries, so
-// that a slice of it takes the same kernel.
-bool sparse_forward_wanted(const sfb_ctx* ctx, int64_t n) {
-  const int rb = sparse_forward_rows(ctx, n);
-  if (rb == 0 || ctx->h16) return false;
-  const sfb_config& c = ctx->cfg;
+// SM cycles of the logits of all K samples row by row: a block's 16 warps take the samples in turn, 900 cycles each and 40 more
+// per entry and lane group, for rb rows of W at a time.  91,238 x 148, K = 176, 13 entries: 1,770,000, the FMA product over the
+// scattered samples 160,000.  For the room for entries, so that a slice of the mini-batch takes the same kernel.
+static double row_wise_cycles(const sfb_config& c, int rb) {
+  const double K = static_cast<double>(c.workers) * c.batch, entries = static_cast<double>(c.csr_nnz_max) / K;
   const double rounds = static_cast<double>(((c.rows + rb - 1) / rb + sm_count() - 1) / sm_count());
-  const double entries = static_cast<double>(c.csr_nnz_max) / static_cast<double>(ctx->K);
-  const double sparse = rounds * (static_cast<double>((ctx->K + kSfWarps - 1) / kSfWarps) * (900.0 + 40.0 * entries * rb / 32.0) +
-                                  static_cast<double>(rb * c.cols) * 4.0 / 25.0);
-  return sparse < gemm_cycles(ctx->K, c.rows, c.cols);
+  return rounds * (std::ceil(K / kSfWarps) * (900.0 + 40.0 * entries * rb / 32.0) + static_cast<double>(rb * c.cols) * 4.0 / 25.0);
+}
+// Whether the row-wise forward is faster than the FMA product.
+bool sparse_forward_wanted(const sfb_ctx* ctx, int64_t n) {
+  const int rb = sparse_forward_rows(ctx->cfg, n);
+  return rb > 0 && !ctx->h16 && row_wise_cycles(ctx->cfg, rb) < gemm_cycles(ctx->K, ctx->cfg.rows, ctx->cfg.cols);
+}
+// Whether sparse samples in fp32 mode are better off on the FMA kernels and the sparse update than on pairs of fp16 words (the
+// packing of W at 4.5 TB/s, the dense product, the cheaper update; in units of 2.6 ps per entry of W as below).  us per step, FMA / pairs:
+// 10,000 x 20,000 with 30 entries K = 128 873 / 1302, 20,000 x 4,000 K = 16 371 / 659; 50,000 x 1,000 with 10 K = 128 551 / 463,
+// 1,000 x 20,000 with 100 K = 256 335 / 251.
+bool sparse_on_fma(const sfb_config& c) {
+  const int64_t K = static_cast<int64_t>(c.workers) * c.batch;
+  if (c.model != SFB_MLR || c.csr_nnz_max <= 0 || c.csr_update == 2 || slab_smem(K, false) < 0) return false;
+  const int rb = sparse_forward_rows(c, K);
+  const double size = static_cast<double>(c.rows) * static_cast<double>(c.cols), unit = 2.6e-12 * 1.9e9 * size;
+  const double sparse = 1.0 + 0.089 * static_cast<double>(c.csr_nnz_max) / static_cast<double>(c.cols);
+  const double fma = (rb > 0 ? std::min(row_wise_cycles(c, rb), gemm_cycles(K, c.rows, c.cols)) : gemm_cycles(K, c.rows, c.cols)) + sparse * unit;
+  const double pairs = size * 8.0 / 4.5e12 * 1.9e9 + split_product_cost(K, c.rows, c.cols, false) +
+                       std::min(sparse, std::max(0.7, 1.75 * static_cast<double>(K) / 1024.0)) * unit;
+  return fma < 1.1 * pairs;
 }
 
 // Z[off .. off+n) = X W^T for the n staged sparse samples at pair offset off (fp32, row pitch ldz).
 int sparse_forward(sfb_ctx* ctx, int64_t off, int64_t n, float* Z, int64_t ldz) {
-  const int rb = sparse_forward_rows(ctx, n);
+  const int rb = sparse_forward_rows(ctx->cfg, n);
   if (rb == 0) return SFB_ERR_SHAPE;
   const int pitch = forward_pitch(ctx->cfg.cols, rb);
   const int smem = static_cast<int>(static_cast<int64_t>(rb) * pitch * 4 + n * 8 + kSfWarps * kSfBufs * kSfChunk * 8);

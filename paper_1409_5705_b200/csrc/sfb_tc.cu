@@ -1025,7 +1025,9 @@ static int mlr_forward(sfb_ctx* ctx, int64_t off, int64_t n, const float* X, con
   const int64_t ldz = round_up(rows, 32);
   __nv_bfloat16* Xb = ctx->at<__nv_bfloat16>(L.Xb);
   ctx->labels = sfb_ctx::kLabelsNone;
-  CKC(launch_kernel(pack_mlr_kernel, dim3(grid1d(n * cols / 4, 256)), dim3(256), 0, ctx->stream, 1, X, n, cols, Xb,
+  // (samples that come by a copy on another stream: that one has to be complete before the kernel starts at all)
+  const bool early = !ctx->host || ctx->host->parts <= 1;
+  CKC(launch_kernel_if(early, pack_mlr_kernel, dim3(grid1d(n * cols / 4, 256)), dim3(256), 0, ctx->stream, 1, X, n, cols, Xb,
                     L.colsb, off,
                     fused ? nullptr : ctx->at<float>(L.Xf), labels, ctx->at<int32_t>(L.labels), ctx->at<int32_t>(L.slot),
                     rows,

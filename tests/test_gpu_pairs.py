@@ -174,7 +174,8 @@ def test_dual_solve_at_the_edge_of_shared_memory(classes):
 # Samples from host memory: copied in parts beside the products of the parts before them (several times 128 samples), in one piece.
 @pytest.mark.parametrize("shape", [(2000, 8000, 4, 64), (1000, 8000, 1, 384), (333, 260, 3, 37)])
 def test_host_samples_in_parts(shape):
-    wl = workload("mlr", *shape, w_std=0.01)
+    # (samples of unit length: of 8,000 unit features, length 90, one step puts every p_y at 1 and leaves a second update of 0)
+    wl = workload("mlr", *shape, w_std=0.01, x_scale="inv_sqrt_d")
     W0, inp = I.initial_W(wl), I.step_inputs(wl, 1)
     W = to_dev(W0, torch)
     ctx = S.Context(config_for(wl, S.PREC_BF16), W)
