@@ -558,7 +558,16 @@ bool sparse_update_wanted(const sfb_ctx* ctx) {
   const sfb_config& c = ctx->cfg;
   const bool bf16 = c.precision == SFB_PREC_BF16;
   if (c.csr_update == 2 || slab_smem(ctx->K, bf16) < 0) return false;
-  if (c.csr_update == 1 || (!bf16 && !ctx->tf32 && !ctx->h16)) return true;
+  if (c.csr_update == 1) return true;
+  if (!bf16 && !ctx->tf32 && !ctx->h16) {
+    // FMA kernels, in SM cycles: the column-major form takes 38,000 (five small launches), the dense update at least its pass over W
+    // at 2.5 TB/s.  us per step, sparse / dense update: 1,000 x 1,000 K = 128 57 / 42, 91,238 x 148 K = 176 519 / 441, 20,000 x 4,000
+    // K = 16 371 / 458, 10,000 x 20,000 K = 128 874 / 1531.
+    const double size = static_cast<double>(c.rows) * static_cast<double>(c.cols);
+    const double sums = 1.0 + 0.089 * static_cast<double>(ctx->csr_fill) / static_cast<double>(c.cols);
+    const double sparse = 38000.0 + sums * 2.6e-12 * 1.9e9 * size + static_cast<double>(ctx->K) * static_cast<double>(c.rows) * 4.0 / 4e12 * 1.9e9;
+    return sparse < std::max(gemm_cycles(c.rows, c.cols, ctx->K), size * 8.0 / 2.5e12 * 1.9e9);
+  }
   const double per_col = static_cast<double>(ctx->csr_fill) / static_cast<double>(c.cols);
   const double k = static_cast<double>(ctx->K) / 1024.0;
   const double sparse = (ctx->tf32 ? 1.57 : 1.0) + 0.089 * per_col;
