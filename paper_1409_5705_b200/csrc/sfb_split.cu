@@ -959,9 +959,12 @@ __global__ void __launch_bounds__(256) pack_u_kernel(const float* __restrict__ U
   const int64_t quads = (rows + 3) / 4, total = K * quads, stride = static_cast<int64_t>(gridDim.x) * 256;
   for (int64_t t = blockIdx.x * 256ll + threadIdx.x; t < total; t += stride) {
     const int64_t i = t / quads, c = (t - i * quads) * 4;
-    // (the pitch is a multiple of 4; what a last quad holds past `rows` lands in the operand's padding, where it only meets
-    // rows of W that are not there)
-    const float4 u = *reinterpret_cast<const float4*>(U + i * ldu + c);
+    // (the pitch is a multiple of 4; the operand's padding stays zero: the coder contracts over the same buffer in the next step,
+    // and nothing ever writes the padding of U)
+    float4 u = *reinterpret_cast<const float4*>(U + i * ldu + c);
+    if (c + 1 >= rows) u.y = 0.f;
+    if (c + 2 >= rows) u.z = 0.f;
+    if (c + 3 >= rows) u.w = 0.f;
     put_pair4<true>(dst + i * 2 * rowsp + c, rowsp, scale4(u, fminf(a * inv_v[i], 1e36f)));
   }
 }

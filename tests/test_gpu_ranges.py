@@ -1,0 +1,45 @@
+"""Inputs at the ends of the ranges that the entry points take, and calls in orders that a program may use them in: workspace
+memory with anything in it, matrices of large and small norm, W written between two calls, steps in which a coder does not
+converge."""
+import numpy as np
+import pytest
+
+import paper_1409_5705_b200 as S
+import sfb_inputs as I
+from oracle import sfb_oracle as O
+from _parity import config_for, oracle_step, rel_err, step_tol, to_dev
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+
+
+def poisoned_context(cfg, W, monkeypatch):
+    """A context whose workspace holds NaN in every word at the start."""
+    empty = torch.empty
+    with monkeypatch.context() as m:
+        m.setattr(torch, "empty", lambda *a, **k: empty(*a, **k).fill_(255) if k.get("dtype") is torch.uint8 else empty(*a, **k))
+        return S.Context(cfg, W)
+
+
+def sc_workload(rows, cols, K, iters, **kw):
+    return I.scaled(I.WORKLOADS["sc"], "sc_ranges", rows=rows, cols=cols, workers=1, batch=K, eta=1e-2, sc_nnz=6, sc_iters=iters, **kw)
+
+
+# rows % 4 = 0 .. 3: what lies between `rows` and the pitch of u must not reach the products of the next step.
+@pytest.mark.parametrize("rows", [1500, 1501, 1502, 1503])
+@pytest.mark.parametrize("prec", [pytest.param(S.PREC_FP32, id="fp32"), pytest.param(S.PREC_BF16, id="bf16")])
+def test_second_step_on_a_workspace_of_nan(rows, prec, monkeypatch):
+    wl = sc_workload(rows, 600, 400, 3)
+    W0 = I.initial_W(wl)
+    L = float(np.float32(O.lipschitz_power_iteration(W0)))
+    W = to_dev(W0, torch)
+    ctx = poisoned_context(config_for(wl, prec, L), W, monkeypatch)
+    Wt, D = W0, I.sc_true_dictionary(wl)
+    for t in range(2):
+        inp = I.step_inputs(wl, t, D)
+        ctx.sfb_step(to_dev(inp.X, torch), None, None)
+        assert ctx.sfb_get_status() == 0
+        Wg, ref = W.cpu().numpy(), oracle_step(wl, Wt, inp, L=L)
+        assert rel_err(Wg, ref, Wt) <= step_tol(wl, prec, ref, Wt)
+        Wt = Wg
+    ctx.close()
