@@ -495,8 +495,11 @@ __global__ void __launch_bounds__(kThreads) prox_scale_kernel(float* __restrict_
 // a fence, an atomic, a poll and a load one after the other (4 us an iteration); here every value of the vector carries the
 // number of its iteration in the same 8 bytes, and who needs the vector reads it until it is all there.  Two buffers are enough:
 // a block writes iteration i + 2 when it has all of i + 1, which the others wrote when they had read all of i.
-// The norm is not waited for either: an iteration scales by the one before it, v <- G v / ||previous v||, which keeps the vector
-// within a factor of ||G|| of its length; only the last pass needs its own norm.  2,000 x 1,000: 200 -> 166 -> 125 us.
+// The norm is not waited for either: it is known one iteration later.  With rho_i = ||G v_i|| / ||v_i||, which settles, an iteration
+// scales by what rho_(i-2) says the next vector's length will be, so that lengths stay at rho_i rho_(i-1) / rho_(i-2)^2, near 1
+// whatever the norm of G (scaled by the length before alone they swing between 1 and ||G||^2, and their squares overflow from
+// ||W|| = 6e4 on).  Only the first vector, of length ||G v_0||, and the last are scaled by their own norm.
+// 2,000 x 1,000: 200 -> 166 -> 125 us.
 // ---------------------------------------------------------------------------------------------------------
 constexpr int kPiThreads = 512, kPiWarps = kPiThreads / 32;
 constexpr int kPiBlocks = 148;                        // most blocks of the grid (the scratch is sized for it)
@@ -609,7 +612,8 @@ __global__ void __launch_bounds__(kPiThreads) power_kernel(const PowerParams p) 
   const int keep = static_cast<int>(r1 - r0 < p.smem_rows ? r1 - r0 : p.smem_rows);
   if (GRAM)
     for (int q = t; q < keep * quads; q += kPiThreads) gs[q] = reinterpret_cast<const float4*>(p.W + r0 * p.cols)[q];
-  float scale = 1.f;                                   // 1 / ||v|| of the iteration before (of this one in the last pass)
+  float scale = 1.f;                                   // of G v in this iteration (1 / ||v|| in the last pass)
+  float iscale = 1.f, scale1 = 1.f, len1 = 1.f;        // its inverse; scale and ||v|| of the iteration before
   for (int it = 0; it <= p.iters; ++it) {              // the last pass only forms ||W v||^2
     const unsigned long long* in = p.vec + static_cast<int64_t>(it & 1) * p.cols;
     unsigned long long* out = p.vec + static_cast<int64_t>((it + 1) & 1) * p.cols;
@@ -622,14 +626,35 @@ __global__ void __launch_bounds__(kPiThreads) power_kernel(const PowerParams p) 
     } else {
       if (!get_vector(in, quads, it, vs, p.status, ss)) return;
     }
+    float unit = 1.f;                                  // of a vector that is not in shared memory
     auto vat = [&](int q) {
       if (GRAM || vs) return vs[q];
-      return it == 0 ? make_float4(start, start, start, start) : untagged(ld_pair(in + 4 * q), ld_pair(in + 4 * q + 2));
+      if (it == 0) return make_float4(start, start, start, start);
+      const float4 v = untagged(ld_pair(in + 4 * q), ld_pair(in + 4 * q + 2));
+      return make_float4(v.x * unit, v.y * unit, v.z * unit, v.w * unit);
     };
-    if (last && it > 0) {
+    if (it > 0 && (last || it == 1)) {
       double s = 0.;
-      for (int q = t; q < quads; q += kPiThreads) s += static_cast<double>(dot4(vat(q), vat(q), 0.f));
-      scale = static_cast<float>(1. / sqrt(block_sum_d(s, sh)));
+      for (int q = t; q < quads; q += kPiThreads) {
+        const float4 v = vat(q);
+        s += static_cast<double>(v.x) * v.x + static_cast<double>(v.y) * v.y + static_cast<double>(v.z) * v.z + static_cast<double>(v.w) * v.w;
+      }
+      const double n = sqrt(block_sum_d(s, sh));
+      if (last) {
+        scale = static_cast<float>(1. / n);
+      } else {                                         // v_1 / ||v_1||, as if v_0 had been scaled by it; rho_0 = ||v_1||
+        unit = static_cast<float>(1. / n);
+        if (vs) {
+          for (int q = t; q < quads; q += kPiThreads) {
+            const float4 v = vs[q];
+            vs[q] = make_float4(v.x * unit, v.y * unit, v.z * unit, v.w * unit);
+          }
+          unit = 1.f;
+        }
+        __syncthreads();
+        scale1 = scale = static_cast<float>(1. / n);
+        iscale = static_cast<float>(n);
+      }
     }
     auto dot_row = [&](const float4* w4) {             // in every lane
       float s0 = 0.f, s1 = 0.f;
@@ -691,8 +716,16 @@ __global__ void __launch_bounds__(kPiThreads) power_kernel(const PowerParams p) 
       }
     }
     // (any scale does but in the last pass; the vector has been read by everyone, too)
-    if (it > 0 && !last) scale = rsqrtf(fmaxf(block_sum_f(ss, shf), 1e-37f));
-    else if (!last) __syncthreads();
+    if (it > 1 && !last) {
+      const float sq = block_sum_f(ss, shf), ilen = rsqrtf(sq);
+      const float irho = len1 * scale1 * ilen;         // of the iteration before
+      scale1 = scale;
+      len1 = sq * ilen;
+      scale = irho * (irho * iscale) * ilen;           // 1 / (rho * (rho * len * scale))
+      iscale = 1.f / scale;
+    } else if (!last) {
+      __syncthreads();
+    }
     if (last) {
       acc = block_sum_d(acc, sh);
       if (t == 0) p.norms[blk] = acc;

@@ -43,3 +43,21 @@ def test_second_step_on_a_workspace_of_nan(rows, prec, monkeypatch):
         assert rel_err(Wg, ref, Wt) <= step_tol(wl, prec, ref, Wt)
         Wt = Wg
     ctx.close()
+
+
+# The estimate of L on W^T W, on W with the vector in shared memory, and beyond it (51,200 atoms), for dictionaries of any norm: the
+# lengths of the iterates must neither overflow nor vanish.  50 products of fp32 sums: 50 * 2^-24 of L.
+@pytest.mark.parametrize("scale", [1e-8, 1e-4, 1.0, 3e3, 1e5, 1e8])
+@pytest.mark.parametrize("rows,cols,K", [(400, 200, 64), (60, 700, 2), (40, 60000, 2)])
+def test_lipschitz_estimate_of_small_and_large_dictionaries(rows, cols, K, scale):
+    wl = sc_workload(rows, cols, K, 2)
+    W0 = (I.initial_W(wl) * np.float32(scale)).astype(np.float32)
+    X = np.random.default_rng(5).standard_normal((K, rows)).astype(np.float32)
+    W = to_dev(W0, torch)
+    ctx = S.Context(config_for(wl, S.PREC_FP32, 0.0, prox=0), W)
+    ctx.sfb_step(to_dev(X, torch), None, None)
+    assert ctx.sfb_get_status() == 0
+    L = ctx.sfb_get_stats().sc_lipschitz
+    ctx.close()
+    ref = O.lipschitz_power_iteration(W0)
+    assert abs(L - ref) <= 50 * 2.0 ** -24 * ref
