@@ -136,7 +136,8 @@ int sfb_init(const sfb_config* cfg, float* W_dev, void* workspace_dev, size_t wo
  * Factors are written at the worker's row offset p*B of the gathered buffers.  All P workers of a step see the
  * same W (bulk-synchronous consistency, Section 4.1).
  * Copies of W that the library derives: in bf16 mode the forward product reads a bf16 operand copy of W.  DML and SC
- * and SFB_PREC_FP32 rebuild theirs from W in the first factors call of every step.  MLR in bf16 mode (and with
+ * and SFB_PREC_FP32 rebuild theirs from W in the first factors call of every step, and in one that computes factors again (for
+ * all workers, or for a worker that has committed).  MLR in bf16 mode (and with
  * SFB_PREC_TF32X3, whose copy is the pair of tf32 words per entry) builds it once in sfb_init and afterwards the
  * update pass rewrites it together with W (W makes one trip through the SM per step), so it tracks every change the
  * LIBRARY makes to W -- but not writes the caller makes to W_dev between steps (loading weights, rescaling, a prox of

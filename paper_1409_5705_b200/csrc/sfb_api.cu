@@ -314,6 +314,12 @@ static int factors_fp32(sfb_ctx* ctx, int64_t off, int64_t n, const float* X, co
   return SFB_OK;
 }
 
+// A factors call with which the step begins, or begins anew: the first one, one for all workers, and one for a worker that has
+// its factors already (they are computed again, against the W of now).
+static bool starts_over(const sfb_ctx* ctx, int32_t worker) {
+  return ctx->committed == 0 || worker < 0 || ((ctx->committed >> worker) & 1u) != 0;
+}
+
 // What the factors of every worker of a step share, formed from the W that they all see (bulk-synchronous consistency):
 // the coder's Gram matrix and its step size.
 static int begin_step(sfb_ctx* ctx) {
@@ -373,8 +379,8 @@ static int compute_factors(sfb_ctx* ctx, int32_t worker, const float* X_dev, con
     ctx->sparse_mask = 0;
     ctx->csr_fill = 0;
     begin_phase(ctx, 0);
-    ctx->begun = false;
   }
+  if (starts_over(ctx, worker)) ctx->begun = false;
   if (!ctx->begun) {
     if ((rc = begin_step(ctx)) != SFB_OK) return rc;
     ctx->begun = true;
@@ -419,10 +425,8 @@ static int compute_factors_csr(sfb_ctx* ctx, int32_t worker, const int64_t* indp
   if (ctx->csr_fill + nnz > c.csr_nnz_max) return SFB_ERR_SHAPE;
   const int64_t off = worker < 0 ? 0 : static_cast<int64_t>(worker) * c.batch;
   const int64_t n = worker < 0 ? ctx->K : c.batch;
-  if (ctx->committed == 0) {
-    begin_phase(ctx, 0);
-    ctx->begun = false;
-  }
+  if (ctx->committed == 0) begin_phase(ctx, 0);
+  if (starts_over(ctx, worker)) ctx->begun = false;
   int rc = SFB_OK;
   if (!ctx->begun) {
     if ((rc = begin_step(ctx)) != SFB_OK) return rc;
@@ -722,10 +726,8 @@ static int sdca_compute_factors(sfb_ctx* ctx, int32_t worker, const float* X_dev
   if (worker < -1 || worker >= c.workers) return SFB_ERR_SHAPE;
   const int64_t off = worker < 0 ? 0 : static_cast<int64_t>(worker) * c.batch;
   const int64_t n = worker < 0 ? ctx->K : c.batch;
-  if (ctx->committed == 0) {
-    begin_phase(ctx, 0);
-    ctx->begun = false;
-  }
+  if (ctx->committed == 0) begin_phase(ctx, 0);
+  if (starts_over(ctx, worker)) ctx->begun = false;
   const float inv_lam_n = static_cast<float>(1.0 / (static_cast<double>(c.sdca_lambda) * static_cast<double>(c.sdca_n)));
   if (ctx->tf32) {
     const int rc = tc32_factors(ctx, off, n, X_dev, labels_dev, sample_ids_dev, inv_lam_n);

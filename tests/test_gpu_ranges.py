@@ -61,3 +61,33 @@ def test_lipschitz_estimate_of_small_and_large_dictionaries(rows, cols, K, scale
     ctx.close()
     ref = O.lipschitz_power_iteration(W0)
     assert abs(L - ref) <= 50 * 2.0 ** -24 * ref
+
+
+# Factors that are computed again before any update, after the caller has written W (a line search, a check of gradients): they
+# belong to the W of the second call, on every kind of kernel.  all: one call for all workers; else worker 0 again.
+@pytest.mark.parametrize("whole", [True, False])
+@pytest.mark.parametrize("model,shape,prec", [(S.MLR, (701, 1028, 2, 180), S.PREC_FP32), (S.MLR, (70, 260, 2, 20), S.PREC_FP32),
+                                              (S.DML, (300, 2500, 2, 150), S.PREC_FP32), (S.DML, (300, 2500, 2, 150), S.PREC_BF16),
+                                              (S.SC, (700, 400, 2, 512), S.PREC_FP32), (S.SC, (260, 132, 2, 40), S.PREC_FP32)])
+def test_factors_computed_again_see_the_w_of_now(model, shape, prec, whole):
+    rows, cols, P, B = shape
+    rng = np.random.default_rng(2)
+    K, ind = P * B, rows if model == S.SC else cols
+    W0 = (rng.standard_normal((rows, cols)) / np.sqrt(rows if model == S.SC else cols)).astype(np.float32)
+    X, Y = (rng.standard_normal((K, ind)).astype(np.float32) for _ in range(2))
+    lab = rng.integers(0, rows if model == S.MLR else 2, K).astype(np.int32)
+    W = to_dev(W0, torch)
+    cfg = S.make_config(model, rows, cols, P, B, 1e-3, prec, sc_ista_iters=4)
+    ctx = S.Context(cfg, W)
+    dev = [to_dev(a, torch) for a in (X, Y if model == S.DML else None, lab if model != S.SC else None)]
+    part = dev if whole else [None if a is None else a[:B] for a in dev]
+    ctx.sfb_compute_factors(-1, *dev)
+    W.mul_(0.5)
+    ctx.sfb_compute_factors(-1 if whole else 0, *part)
+    U, V = (t.cpu().numpy().astype(np.float64) for t in ctx.factors_as_tensors())
+    ctx.close()
+    n, Wn = K if whole else B, (W0 * np.float32(0.5)).astype(np.float64)
+    L = O.lipschitz_power_iteration(Wn.astype(np.float32)) if model == S.SC else None
+    Ur, Vr = O.sfb_step(model, Wn, X, Y, lab, workers=P, eta=1e-3, margin=1.0, lam=0.1, L=L, iters=4, prox=False, return_factors=True)[1:3]
+    for got, want in ((U[:n], Ur[:n]), (V[:n], Vr[:n])):
+        assert np.linalg.norm(got - want) <= (1e-5 if prec == S.PREC_FP32 else 1e-4) * np.linalg.norm(want)
