@@ -45,6 +45,7 @@ enum sfb_model { SFB_MLR = 0, SFB_DML = 1, SFB_SC = 2, SFB_L2MLR = 3 };
  * SFB_PREC_FP32: fp32 operands.  Products large enough to repay the packing of their operands run on the tensor cores, every
  *                value as a pair of fp16 words with a power-of-two scale per row (23 of its 24 bits, down to 2^-27 of the
  *                row's largest entry), three fp16 products per term, partial sums in fp32; smaller ones on fp32 FMA kernels.
+ *                Sparse coding may iterate on W^T W, in fp64, where that is the cheaper form.
  * SFB_PREC_TF32X3: (MLR, SFB_L2MLR) fp32 operands on the tensor cores at any shape: every fp32 value x is carried as
  *                two tf32 words, big = tf32(x) and small = tf32(x - big), and a product runs as
  *                big*big + big*small + small*big with fp32 accumulation (relative error about 2^-21 per product);

@@ -28,21 +28,56 @@ static size_t up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
 // The coder's iterations a <- soft(a - W^T (W a - x) / L) either take two products with W each, or one with the Gram matrix
 // W^T W, formed once per step (half of it: it is symmetric), and W^T x.  The Gram form wins when the mini-batch is large enough
 // to repay W^T W; decided by the cost of the products themselves (10,000 x 5,000, K = 512, 20 iterations, bf16: 5.0 -> 2.2 ms
-// for the coder; error of the codes 2.9e-5, with two products 1.1e-4 while they had one accumulator).  In bf16 mode it is kept
-// to dictionaries with no more atoms than features: the residual of an overcomplete one becomes small against x, and the
-// two-product form then rounds relative to it where W^T W a - W^T x rounds relative to W^T x (500 x 1,400: 4.8e-6 against
-// 1.2e-5).
+// for the coder).  In bf16 mode it is kept to dictionaries with no more atoms than features: the residual of an overcomplete one
+// becomes small against x, and the two-product form then rounds relative to it where W^T W a - W^T x rounds relative to W^T x
+// (500 x 1,400: 4.8e-6 against 1.2e-5).  The fp32 mode has it in fp64 only, on the FMA kernels, for the same reason (see
+// sfb_gram64.cu).
+static double sc_iterations(const sfb_config& c) { return c.sc_ista_iters - 1; }
+constexpr int64_t kMostAtoms = 32 << 10;     // (the power iteration keeps a vector of them on chip)
+
 bool sc_use_gram(const sfb_config& c) {
   const int64_t K = static_cast<int64_t>(c.workers) * c.batch, D = c.rows, A = c.cols;
-  const double it = c.sc_ista_iters - 1;
-  if (it < 1 || (c.precision == SFB_PREC_BF16 && A > D)) return false;
-  if (A > (32 << 10)) return false;        // (the power iteration keeps a vector of A values on chip)
-  auto cost = [&](int64_t M, int64_t N, int64_t Kc, bool sym) {
-    if (c.precision == SFB_PREC_BF16 || use_h16(c)) return split_product_cost(M, N, Kc, sym);
-    const GemmShape g = pick_gemm_shape(M, N, Kc, sym);
-    return std::min(gemm_cost(128, g.split, M, N, Kc, sym), gemm_cost(64, g.split, M, N, Kc, sym));
-  };
-  return cost(A, A, D, true) + it * cost(K, A, A, false) < it * (cost(K, D, A, false) + cost(K, A, D, false));
+  const double it = sc_iterations(c);
+  if (c.precision != SFB_PREC_BF16 || it < 1 || A > D || A > kMostAtoms) return false;
+  return split_product_cost(A, A, D, true) + it * split_product_cost(K, A, A, false) <
+         it * (split_product_cost(K, D, A, false) + split_product_cost(K, A, D, false));
+}
+
+// The power iteration on W^T W, whose rows stay on chip, or on W, which comes from L2 or memory twice an iteration, with a barrier
+// between (2,500 x 1,000: 2.6 us an iteration against 21).
+bool sc_estimate_on_gram(const sfb_config& c, double form) {
+  if (c.sc_lipschitz > 0.f || c.cols > kMostAtoms) return false;
+  const double D = static_cast<double>(c.rows), A = static_cast<double>(c.cols);
+  return form + 50.0 * (4000.0 + A * A * 4.0 / 3000.0) < 50.0 * (10000.0 + D * A * 8.0 / 640.0);
+}
+
+// SM cycles of the coder's products on the FMA kernels, in the cheaper of the two forms; W^T W is there where L is estimated on it.
+static double sc_fma_cost(const sfb_config& c, bool& gram64) {
+  const int64_t K = static_cast<int64_t>(c.workers) * c.batch, D = c.rows, A = c.cols;
+  const double it = sc_iterations(c), last = gemm_cycles(K, D, A), form = gram64_form_cost(D, A);
+  const double there = sc_estimate_on_gram(c, form) ? form : 0.0;
+  gram64 = false;
+  if (it < 0) return last + there;
+  const double two = gemm_cycles(K, A, D) + it * (gemm_cycles(K, D, A) + gemm_cycles(K, A, D)) + last + there;
+  if (it < 1 || A > kMostAtoms) return two;
+  const double one = form + gram64_cost(A, K, D) + it * gram64_cost(A, K, A) + last + 10000.0;
+  gram64 = one < two;
+  return std::min(one, two);
+}
+bool sc_use_gram64(const sfb_config& c) {
+  bool gram64 = false;
+  sc_fma_cost(c, gram64);
+  return gram64;
+}
+// Whether the products of sparse coding in fp32 mode are better off as pairs of fp16 words: the packing of W and W^T at 4.5 TB/s, two
+// products an iteration.
+bool sc_on_pairs(const sfb_config& c) {
+  const int64_t K = static_cast<int64_t>(c.workers) * c.batch, D = c.rows, A = c.cols;
+  const double it = sc_iterations(c), size = static_cast<double>(D) * static_cast<double>(A), form = split_product_cost(A, A, D, true, true);
+  const double toD = split_product_cost(K, D, A, false, true), toA = split_product_cost(K, A, D, false, true);
+  const double pairs = toD + size * 16.0 / 4.5e12 * 1.9e9 + 20000.0 + (it >= 0 ? toA + it * (toD + toA) : 0.0) + (sc_estimate_on_gram(c, form) ? form : 0.0);
+  bool gram64;
+  return pairs < sc_fma_cost(c, gram64);
 }
 
 Layout make_layout(const sfb_config& cfg) {
@@ -73,9 +108,10 @@ Layout make_layout(const sfb_config& cfg) {
     L.ldu = round_up(c.rows, 4);                      // 16-byte row pitch
     L.V = take(K * cols * 4);
     L.U = take(K * static_cast<size_t>(L.ldu) * 4);
-    if (c.model == SFB_SC && sc_use_gram(c)) {
-      L.G = take(cols * cols * 4);
-      L.Bx = take(K * cols * 4);
+    if (c.model == SFB_SC) {
+      const bool coder = sc_use_gram64(c), estimate = sc_estimate_on_gram(c, gram64_form_cost(c.rows, c.cols));
+      if (coder || estimate) gram64_extend_layout(c, coder, L, off);
+      if (estimate || (coder && !(c.sc_lipschitz > 0.f))) L.G = take(cols * cols * 4);      // in fp32 for the power iteration
     }
     if (c.model == SFB_SC) L.V2 = take(K * cols * 4);
   } else {
@@ -280,30 +316,23 @@ static int factors_fp32(sfb_ctx* ctx, int64_t off, int64_t n, const float* X, co
   if (ctx->h16) return split_factors_sc(ctx, off, n, X);
   // Sparse coding: ISTA from a = 0, then u = W a - x, v = a.  The first iterate is soft(W^T x / L).
   const int T = c.sc_ista_iters;
-  const bool gram = ctx->lay.G != 0;
   float* V2 = ctx->at<float>(ctx->lay.V2) + off * cols;
-  float* Bx = gram ? ctx->at<float>(ctx->lay.Bx) + off * cols : nullptr;
-  const float* G = ctx->at<float>(ctx->lay.G);
   auto iterate = [&](int t) { return ((T - t) & 1) == 0 ? V : V2; };                    // where a_t goes: a_T to V
   if (T == 0) {
     CK(fill_zero(s, V, n * cols));
+  } else if (ctx->lay.Xd) {
+    CK(gram64_codes(ctx, n, X, V));
   } else {
-    e.C = iterate(1); e.ldc = cols; e.C2 = Bx; e.ldc2 = cols; e.sc = sc; e.lam = c.sc_lambda;
-    CK(sgemm(s, true, false, EPI_ISTA0, n, cols, rows, X, rows, ctx->W, cols, e, K));   // W^T x, a_1
+    e.C = iterate(1); e.ldc = cols; e.sc = sc; e.lam = c.sc_lambda;
+    CK(sgemm(s, true, false, EPI_ISTA0, n, cols, rows, X, rows, ctx->W, cols, e, K));   // a_1
     ctx->stats.flops += 2.0 * n * rows * cols;
-  }
-  for (int t = 2; t <= T; ++t) {
-    EpiArgs q{};
-    q.C = iterate(t); q.ldc = cols; q.cur = iterate(t - 1); q.ldcur = cols; q.sc = sc; q.lam = c.sc_lambda;
-    if (gram) {
-      q.aux = Bx; q.ldaux = cols;
-      CK(sgemm(s, true, false, EPI_ISTA, n, cols, cols, q.cur, cols, G, cols, q, K));   // a <- soft(a - (W^T W a - W^T x) / L)
-      ctx->stats.flops += 2.0 * n * cols * cols;
-    } else {
+    for (int t = 2; t <= T; ++t) {
       e = EpiArgs{};
       e.C = U; e.ldc = ldu; e.aux = X; e.ldaux = rows;
-      CK(sgemm(s, true, true, EPI_SUB, n, rows, cols, q.cur, cols, ctx->W, cols, e, K));    // r = W a - x
-      CK(sgemm(s, true, false, EPI_ISTA, n, cols, rows, U, ldu, ctx->W, cols, q, K));       // a <- soft(a - W^T r / L)
+      CK(sgemm(s, true, true, EPI_SUB, n, rows, cols, iterate(t - 1), cols, ctx->W, cols, e, K));    // r = W a - x
+      e = EpiArgs{};
+      e.C = iterate(t); e.ldc = cols; e.cur = iterate(t - 1); e.ldcur = cols; e.sc = sc; e.lam = c.sc_lambda;
+      CK(sgemm(s, true, false, EPI_ISTA, n, cols, rows, U, ldu, ctx->W, cols, e, K));   // a <- soft(a - W^T r / L)
       ctx->stats.flops += 4.0 * n * rows * cols;
     }
   }
@@ -330,13 +359,8 @@ static int begin_step(sfb_ctx* ctx) {
   }
   if (c.model != SFB_SC) return SFB_OK;
   CK(stamp(ctx->stream, take_stamp(ctx)));
-  float* G = ctx->lay.G ? ctx->at<float>(ctx->lay.G) : nullptr;
-  if (c.precision == SFB_PREC_FP32 && G && !ctx->h16) {
-    EpiArgs e{};
-    e.C = G; e.ldc = c.cols;
-    CK(sgemm(ctx->stream, false, false, EPI_SYM, c.cols, c.cols, c.rows, ctx->W, c.cols, ctx->W, c.cols, e));
-    ctx->stats.flops += static_cast<double>(c.cols) * c.cols * c.rows;
-  }
+  float* G = ctx->lay.G && !(c.sc_lipschitz > 0.f) ? ctx->at<float>(ctx->lay.G) : nullptr;
+  if (ctx->lay.Gd) CK(gram64_begin(ctx, G));
   if (!(c.sc_lipschitz > 0.f))
     CK(estimate_lipschitz(ctx->stream, ctx->W, G, c.rows, c.cols, ctx->at<char>(ctx->lay.pi),
                           ctx->at<Scalars>(ctx->lay.scalars), ctx->at<uint32_t>(ctx->lay.status), 50));

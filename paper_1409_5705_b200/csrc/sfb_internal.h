@@ -16,6 +16,7 @@ inline void count_launch(int n = 1) { g_kernel_launches.fetch_add(n, std::memory
 
 // Multiprocessors of the current device (looked up once per device ordinal).
 int sm_count();
+constexpr int kModelSms = 148;        // what the cost models count with
 
 // ---------------------------------------------------------------------------------------------------------
 // Launches.  A step is a chain of dependent kernels, several of them only microseconds long: each is launched with
@@ -120,6 +121,7 @@ struct Layout {
   // sparse coding: the dictionary's Gram matrix (when the coder iterates on it), W^T x, the codes of odd iterations, and
   // the scratch of the power iteration
   size_t G, Gs, Bx, V2, As2, pi;
+  size_t Wd, Gd, Xd, Bd, Ad;          // in fp64: W, W^T W, the samples, W^T x and the codes, transposed (see sfb_gram64.cu)
   int64_t ldu;                        // row pitch of the fp32 U buffer (rows rounded up to 4; rows itself with tf32 pairs)
   int64_t colsp, rowsp;               // cols, rows rounded up to 64
   int64_t Kp;                         // K rounded up to the contraction block of the update product
@@ -131,7 +133,10 @@ struct Layout {
 };
 
 Layout make_layout(const sfb_config& c);
-bool sc_use_gram(const sfb_config& c);
+bool sc_use_gram(const sfb_config& c);        // the coder on W^T W: bf16 mode;
+bool sc_use_gram64(const sfb_config& c);      //   FMA kernels of the fp32 mode, in fp64
+bool sc_on_pairs(const sfb_config& c);
+bool sc_estimate_on_gram(const sfb_config& c, double form);     // L estimated on a W^T W that costs `form` cycles
 inline int64_t round_up(int64_t x, int64_t m) { return (x + m - 1) / m * m; }
 
 // Which kernels the products of an fp32 mode run on.  Pairs of tf32 words when asked for (logistic models).  SFB_PREC_FP32 runs
@@ -147,7 +152,7 @@ bool sparse_on_fma(const sfb_config& c);      // sparse samples: see sfb_sparse.
 inline bool use_h16(const sfb_config& c) {
   if (c.precision != SFB_PREC_FP32 || c.rows < 64 || c.cols < 64 || sparse_on_fma(c)) return false;
   const double K = static_cast<double>(c.workers) * c.batch, macs = K * static_cast<double>(c.rows) * static_cast<double>(c.cols);
-  if (c.model == SFB_SC) return macs >= 2.8e8;
+  if (c.model == SFB_SC) return sc_on_pairs(c);
   return c.cols >= 256 && (macs >= 1e9 || macs * (1.0 - 24.0 / K) >= 1.8e8);
 }
 
@@ -155,7 +160,7 @@ struct Scalars {                      // device-resident scalars
   float loss_mean;
   float L;                            // ||W||_2^2 used by the coder
   float invL;
-  float iWT, iWT2, iG, iU;            // inverse scales: W^T and its square, W^T W, u (see sfb_split.cu)
+  float iWT, iWT2, iU;                // inverse scales: W^T and its square, u (see sfb_split.cu)
   unsigned long long copy_pieces;     // 64-byte row pieces of the bf16 operand copy the update passes went over ...
   unsigned long long copy_written;    // ... and how many of them they had to rewrite (the others already held bf16(W))
   unsigned long long ns[4];           // global time at the start of the step, of its gather and of its update, and at its end
@@ -224,10 +229,10 @@ inline Stamp take_stamp(sfb_ctx* ctx) { return ctx->take_pending(); }
 // fp32 FMA matrix products:  C (M x N) = sum_k A(m,k) * B(n,k)  followed by an epilogue.
 // A_KC: A(m,k) at A[m*lda + k] (k contiguous), else at A[k*lda + m].  Same for B with n.
 //   EPI_STORE  C = acc                                     EPI_SUB    C = acc - aux
-//   EPI_RMW    C = prox(C + alpha acc)                     EPI_SYM    C = acc for a symmetric result (half of the tiles)
-//   EPI_ISTA   C = soft(cur - (acc - aux) / L, lam / L)    EPI_ISTA0  C = soft(acc / L, lam / L), C2 = acc
+//   EPI_RMW    C = prox(C + alpha acc)
+//   EPI_ISTA   C = soft(cur - acc / L, lam / L)            EPI_ISTA0  C = soft(acc / L, lam / L), C2 = acc
 // ---------------------------------------------------------------------------------------------------------
-enum Epilogue { EPI_STORE = 0, EPI_SUB = 1, EPI_RMW = 2, EPI_ISTA = 3, EPI_ISTA0 = 4, EPI_SYM = 5 };
+enum Epilogue { EPI_STORE = 0, EPI_SUB = 1, EPI_RMW = 2, EPI_ISTA = 3, EPI_ISTA0 = 4 };
 
 // Entry-wise proximal operator fused into the update: kind 1 soft-threshold by a, kind 2 multiply by a.
 __host__ __device__ __forceinline__ float prox_entry(float w, int kind, float a) {
@@ -249,7 +254,7 @@ struct EpiArgs {
   int64_t ldc;
   float* C2;           // EPI_ISTA0 (may be null)
   int64_t ldc2;
-  const float* aux;    // EPI_SUB, EPI_ISTA (there: may be null)
+  const float* aux;    // EPI_SUB
   int64_t ldaux;
   const float* cur;    // EPI_ISTA
   int64_t ldcur;
@@ -257,13 +262,22 @@ struct EpiArgs {
 };
 
 struct GemmShape { int tile, split; };               // tile edge; parts the contraction is cut into
-double gemm_cost(int tile, int split, int64_t M, int64_t N, int64_t Kc, bool sym);
-GemmShape pick_gemm_shape(int64_t M, int64_t N, int64_t Kc, bool sym = false);
+double gemm_cost(int tile, int split, int64_t M, int64_t N, int64_t Kc);
+GemmShape pick_gemm_shape(int64_t M, int64_t N, int64_t Kc);
+double gemm_cycles(int64_t M, int64_t N, int64_t Kc);               // in the better tile
 
 // M_split (0: M): the row count that decides how the contraction is split; callers that compute a product in slices of
 // rows pass the whole product's, so that a row has the same bits whichever slice it is computed in.
 cudaError_t sgemm(cudaStream_t s, bool a_kc, bool b_kc, Epilogue epi, int64_t M, int64_t N, int64_t Kc,
                   const float* A, int64_t lda, const float* B, int64_t ldb, const EpiArgs& e, int64_t M_split = 0);
+
+// The coder of the fp32 mode on W^T W in fp64 (sfb_gram64.cu): cycles of a product, and of W^T W with W widened; buffers (of W^T W
+// alone without coder); W^T W (G32, may be null: also in fp32); the codes of n samples to V.
+double gram64_cost(int64_t N, int64_t M, int64_t Kc);
+double gram64_form_cost(int64_t D, int64_t A);
+void gram64_extend_layout(const sfb_config& c, bool coder, Layout& L, size_t& off);
+cudaError_t gram64_begin(sfb_ctx* ctx, float* G32);
+cudaError_t gram64_codes(sfb_ctx* ctx, int64_t n, const float* X, float* V);
 
 // ---------------------------------------------------------------------------------------------------------
 // Factor kernels (pack, softmax, pair residual, prox, power iteration)
@@ -336,7 +350,6 @@ int sparse_stage(sfb_ctx* ctx, int64_t off, int64_t n, const int64_t* indptr, co
                  int64_t nnz);
 // fp32 FMA mode: rows of W per block of the row-wise forward over sparse samples (0: the rows do not fit), and that product
 bool sparse_forward_wanted(const sfb_ctx* ctx, int64_t n);
-double gemm_cycles(int64_t M, int64_t N, int64_t Kc);               // of a product on the FMA kernels
 int sparse_forward(sfb_ctx* ctx, int64_t off, int64_t n, float* Z, int64_t ldz);
 int sparse_build_csc(sfb_ctx* ctx);
 int sparse_update(sfb_ctx* ctx);

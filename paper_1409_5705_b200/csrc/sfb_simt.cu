@@ -97,26 +97,26 @@ struct GemmParams {
 
 template <int EPI>
 __device__ __forceinline__ float epi_one(float acc, float cur, float aux, const EpiArgs& e, float invL) {
-  if (EPI == EPI_STORE || EPI == EPI_SYM) return acc;
+  if (EPI == EPI_STORE) return acc;
   if (EPI == EPI_SUB) return acc - aux;
   if (EPI == EPI_RMW) return prox_entry(fmaf(e.alpha, acc, cur), e.prox_kind, e.prox_a);
   if (EPI == EPI_ISTA0) return soft(acc * invL, e.lam * invL);
-  return soft(fmaf(-(acc - aux), invL, cur), e.lam * invL);       // EPI_ISTA
+  return soft(fmaf(-acc, invL, cur), e.lam * invL);               // EPI_ISTA
 }
 template <int EPI>
 constexpr bool kReadsCur = EPI == EPI_RMW || EPI == EPI_ISTA;
 
 // four neighbouring outputs of row m (n a multiple of 4) or one output
 template <int EPI>
-__device__ __forceinline__ void epilogue4(const GemmParams& p, int m, int n, float4 acc, float invL, bool mirror) {
+__device__ __forceinline__ void epilogue4(const GemmParams& p, int m, int n, float4 acc, float invL) {
   const EpiArgs& e = p.e;
   float* c = e.C + m * e.ldc + n;
-  const float* x = e.aux ? e.aux + m * e.ldaux + n : nullptr;
+  const float* x = EPI == EPI_SUB ? e.aux + m * e.ldaux + n : nullptr;
   const float* q = EPI == EPI_RMW ? c : kReadsCur<EPI> ? e.cur + m * e.ldcur + n : nullptr;
   if (p.c_vec && n + 3 < p.N) {
     float4 cur = make_float4(0.f, 0.f, 0.f, 0.f), aux = cur, out;
     if (kReadsCur<EPI>) cur = *reinterpret_cast<const float4*>(q);
-    if ((EPI == EPI_SUB || EPI == EPI_ISTA) && x) aux = *reinterpret_cast<const float4*>(x);
+    if (EPI == EPI_SUB) aux = *reinterpret_cast<const float4*>(x);
     out.x = epi_one<EPI>(acc.x, cur.x, aux.x, e, invL);
     out.y = epi_one<EPI>(acc.y, cur.y, aux.y, e, invL);
     out.z = epi_one<EPI>(acc.z, cur.z, aux.z, e, invL);
@@ -129,16 +129,10 @@ __device__ __forceinline__ void epilogue4(const GemmParams& p, int m, int n, flo
     for (int j = 0; j < 4; ++j)
       if (n + j < p.N) {
         const float cur = kReadsCur<EPI> ? q[j] : 0.f;
-        const float aux = (EPI == EPI_SUB || EPI == EPI_ISTA) && x ? x[j] : 0.f;
+        const float aux = EPI == EPI_SUB ? x[j] : 0.f;
         c[j] = epi_one<EPI>(a[j], cur, aux, e, invL);
         if (EPI == EPI_ISTA0 && e.C2) e.C2[m * e.ldc2 + n + j] = a[j];
       }
-  }
-  if (EPI == EPI_SYM && mirror) {
-    const float a[4] = {acc.x, acc.y, acc.z, acc.w};
-#pragma unroll
-    for (int j = 0; j < 4; ++j)
-      if (n + j < p.N) e.C[(n + j) * e.ldc + m] = a[j];
   }
 }
 
@@ -163,7 +157,6 @@ __global__ void __launch_bounds__(NT, 2) sgemm_kernel(const __grid_constant__ Ge
   pdl_launch_dependents();
   pdl_wait();
   if (EPI == EPI_RMW) stamp_begin(p.e.begin);
-  if (EPI == EPI_SYM && tn < tm) return;              // the mirror image of (tn, tm): uniform over the cluster
   const int m0 = tm * BT, n0 = tn * BT;
   // parts of the contraction end at multiples of 32 whatever the tile, so that a product has one summation order
   const int units = (p.Kc + 31) / 32;
@@ -220,7 +213,6 @@ __global__ void __launch_bounds__(NT, 2) sgemm_kernel(const __grid_constant__ Ge
 
   float invL = 0.f;
   if (EPI == EPI_ISTA || EPI == EPI_ISTA0) invL = p.e.sc->invL;
-  const bool mirror = tn > tm;
   if (S == 1) {
 #pragma unroll
     for (int i = 0; i < T; ++i) {
@@ -230,7 +222,7 @@ __global__ void __launch_bounds__(NT, 2) sgemm_kernel(const __grid_constant__ Ge
       for (int h = 0; h < T / 4; ++h) {
         const int n = n0 + h * 64 + tx * 4;
         const float2 lo = unpack2(acc[i][2 * h]), hi = unpack2(acc[i][2 * h + 1]);
-        if (n < p.N) epilogue4<EPI>(p, m, n, make_float4(lo.x, lo.y, hi.x, hi.y), invL, mirror);
+        if (n < p.N) epilogue4<EPI>(p, m, n, make_float4(lo.x, lo.y, hi.x, hi.y), invL);
       }
     }
     if (EPI == EPI_RMW) stamp_end(p.e.end);
@@ -263,7 +255,7 @@ __global__ void __launch_bounds__(NT, 2) sgemm_kernel(const __grid_constant__ Ge
       asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(w.x), "=f"(w.y), "=f"(w.z), "=f"(w.w) : "r"(peer));
       v.x += w.x; v.y += w.y; v.z += w.z; v.w += w.w;
     }
-    epilogue4<EPI>(p, m, n, v, invL, mirror);
+    epilogue4<EPI>(p, m, n, v, invL);
   }
   if (EPI == EPI_RMW) stamp_end(p.e.end);
   // no CTA leaves while a peer still reads its tile
@@ -301,10 +293,10 @@ cudaError_t launch(cudaStream_t s, int64_t M, int64_t N, int64_t Kc, const float
   p.b_vec = aligned16(B) && ldb % 4 == 0;
   p.c_vec = aligned16(e.C) && e.ldc % 4 == 0 && (!e.aux || (aligned16(e.aux) && e.ldaux % 4 == 0)) &&
             (!e.cur || (aligned16(e.cur) && e.ldcur % 4 == 0)) && (!e.C2 || (aligned16(e.C2) && e.ldc2 % 4 == 0));
-  const GemmShape g = pick_gemm_shape(M_split > 0 ? M_split : M, N, Kc, EPI == EPI_SYM);
+  const GemmShape g = pick_gemm_shape(M_split > 0 ? M_split : M, N, Kc);
   p.split = g.split;
   // the split belongs to the product (it fixes the summation order); the tile follows the rows of this call
-  const bool big = gemm_cost(128, g.split, M, N, Kc, EPI == EPI_SYM) <= gemm_cost(64, g.split, M, N, Kc, EPI == EPI_SYM);
+  const bool big = gemm_cost(128, g.split, M, N, Kc) <= gemm_cost(64, g.split, M, N, Kc);
   const int BT = big ? 128 : 64;
   const int64_t tilesM = (M + BT - 1) / BT, tilesN = (N + BT - 1) / BT, tiles = tilesM * tilesN;
   if (tiles * p.split > 0x7fffffffLL) return cudaErrorInvalidValue;
@@ -318,10 +310,10 @@ cudaError_t launch(cudaStream_t s, int64_t M, int64_t N, int64_t Kc, const float
 // either tile per SM) times the cycles of a part.  A pair of 128-wide tiles takes about 300 cycles per k on an SM (85 % of
 // its FMA rate), a pair of 64-wide ones 100; a tile that has its SM to itself 185 and 65.  A part also pays for filling its
 // ring and for the exchange.
-double gemm_cost(int BT, int split, int64_t M, int64_t N, int64_t Kc, bool sym) {
+double gemm_cost(int BT, int split, int64_t M, int64_t N, int64_t Kc) {
   const double tm = static_cast<double>((M + BT - 1) / BT), tn = static_cast<double>((N + BT - 1) / BT);
-  const double tiles = (sym ? 0.5 * tm * (tn + 1.0) : tm * tn) * split;
-  const double sms = sm_count();
+  const double tiles = tm * tn * split;
+  const double sms = kModelSms;
   const double k = static_cast<double>(Kc) / split;
   const int64_t per_sm = static_cast<int64_t>((tiles + sms - 1.0) / sms);       // tiles of the busiest SM
   const double pairs = static_cast<double>(per_sm / 2), single = static_cast<double>(per_sm % 2);
@@ -329,13 +321,13 @@ double gemm_cost(int BT, int split, int64_t M, int64_t N, int64_t Kc, bool sym) 
   return k * per_k + (pairs + single) * (BT == 128 ? 4000.0 : 2000.0) + (split > 1 ? 2500.0 : 0.0);
 }
 
-GemmShape pick_gemm_shape(int64_t M, int64_t N, int64_t Kc, bool sym) {
+GemmShape pick_gemm_shape(int64_t M, int64_t N, int64_t Kc) {
   GemmShape best{128, 1};
-  double cost = gemm_cost(128, 1, M, N, Kc, sym);
+  double cost = gemm_cost(128, 1, M, N, Kc);
   for (int bt = 128; bt >= 64; bt -= 64)
     for (int s = 1; s <= 8; s *= 2) {
       if (s > 1 && Kc < 64 * s) break;                // at least two 32-deep blocks per part
-      const double c = gemm_cost(bt, s, M, N, Kc, sym);
+      const double c = gemm_cost(bt, s, M, N, Kc);
       if (c < 0.97 * cost) { cost = c; best = {bt, s}; }
     }
   return best;
@@ -343,7 +335,7 @@ GemmShape pick_gemm_shape(int64_t M, int64_t N, int64_t Kc, bool sym) {
 
 double gemm_cycles(int64_t M, int64_t N, int64_t Kc) {
   const GemmShape g = pick_gemm_shape(M, N, Kc);
-  return std::min(gemm_cost(128, g.split, M, N, Kc, false), gemm_cost(64, g.split, M, N, Kc, false));
+  return std::min(gemm_cost(128, g.split, M, N, Kc), gemm_cost(64, g.split, M, N, Kc));
 }
 
 cudaError_t sgemm(cudaStream_t s, bool a_kc, bool b_kc, Epilogue epi, int64_t M, int64_t N, int64_t Kc,
@@ -358,7 +350,6 @@ cudaError_t sgemm(cudaStream_t s, bool a_kc, bool b_kc, Epilogue epi, int64_t M,
   } else if (!b_kc) {
     if (epi == EPI_STORE) SFB_GO(false, false, EPI_STORE);
     if (epi == EPI_RMW) SFB_GO(false, false, EPI_RMW);
-    if (epi == EPI_SYM) SFB_GO(false, false, EPI_SYM);
   }
 #undef SFB_GO
   return cudaErrorInvalidValue;                       // a combination no step uses

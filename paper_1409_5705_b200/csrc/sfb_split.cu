@@ -31,9 +31,12 @@ constexpr float kLoScale = 2048.f;                  // of the lo word in the fp1
 //   F_ISTA     C <- soft(C - D / L, lambda / L) in place, also as a pair              (ISTA step)
 //   F_ISTAG    C <- soft(C - (D - C2) / L, lambda / L) in place, also as a pair       (the same on W^T W; C2 = W^T x)
 //   F_ISTA0    C2 (unless null) = D and C = soft(D / L, lambda / L), also as a pair   (first iterate)
-//   F_GRAM     C (unless null) = D and D as a pair, of a symmetric D: only the tiles that reach the diagonal or lie above it
-//              are formed, the others are written as their mirror images              (W^T W)
+//   F_GRAM     C (unless null) = D and, in the bf16 form, D as a pair, of a symmetric D: only the tiles that reach the diagonal or
+//              lie above it are formed, the others are written as their mirror images (W^T W)
 enum FwdEpi { F_STORE = 0, F_SUB = 1, F_ISTA = 2, F_ISTAG = 3, F_ISTA0 = 4, F_GRAM = 5 };
+// The result also goes out as an operand.  (fp32 mode has W^T W for the power iteration only.)
+template <int EPI, bool F16>
+constexpr bool kPairOut = EPI != F_STORE && !(EPI == F_GRAM && F16);
 template <int EPI>
 constexpr bool kIsta = EPI == F_ISTA || EPI == F_ISTAG || EPI == F_ISTA0;
 
@@ -56,16 +59,14 @@ struct SplitParams {
   int32_t aux_row0;            // aux's map
   const Scalars* sc;           // F_ISTA*: 1 / L
   float lam;                   // F_ISTA*: lambda
-  uint16_t* split;             // all but F_STORE: [M x ld_split] receives hi at column n and lo at column split_half + n
+  uint16_t* split;             // where kPairOut: [M x ld_split] receives hi at column n and lo at column split_half + n
   int64_t ld_split;
   int32_t split_half;          // padded N (a multiple of 64); columns N..split_half-1 are written as zeros
-  // fp16 form: inverse scales of A per row, of B per column of D, a factor for all, and of the pair that goes out (per row, or
-  // one for all); null: 1
+  // fp16 form: inverse scales of A per row, of B per column of D, a factor for all (null: 1), and of the pair that goes out per row
   const float* ia;
   const float* ib;
   const float* iab;
   const float* io;
-  const float* ios;
   uint32_t* status;
 };
 
@@ -131,7 +132,11 @@ constexpr int kChunk = 32, kEpi = 8;
 constexpr int kStagesMax = 6;
 constexpr int kRegion = 192 << 10;                  // of the operand ring
 constexpr int kSlot = 32 * kChunk * 4;              // per epilogue warp: 32 rows x 32 columns of fp32
-constexpr int kDrain = 8;
+// k-blocks of A_hi B_hi per drain.  Sparse coding in fp32 mode drains every one: the gradient of its iterations cancels, and the
+// rounding towards zero of the 32 instructions of eight k-blocks made the codes up to 2.5 times less exact than those of the FMA
+// kernels (676 x 1,148, K = 649, 20 iterations; one drain a k-block: 0.95).
+template <int EPI, bool F16>
+constexpr int kDrain = F16 && EPI != F_STORE ? 1 : 8;
 constexpr int kThreads = 128 + 32 * kEpi;
 constexpr int kInputs = 3;                          // buffers per epilogue warp for what the end of the last tile reads
 static_assert((4 + kInputs - 1) * kEpi * kSlot <= kRegion, "see there");
@@ -289,7 +294,7 @@ split_product_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
         const Segment sg = segs.get(i);
         const int nk = sg.k1 - sg.k0;
         for (int kb = 0; kb < nk; ++kb) {
-          const int kc = kb % kDrain;
+          const int kc = kb % kDrain<EPI, F16>;
           if (!mbar_wait(&full[s], ph, abort_flag) || (kc == 0 && !mbar_wait(mempty, (g & 1) ^ 1, abort_flag)) ||
               (kb == 0 && !mbar_wait(cempty, (i & 1) ^ 1, abort_flag))) { ok = false; break; }
           tc_fence_after();
@@ -302,7 +307,7 @@ split_product_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
             umma_bf16_pair(d_main, dah + adv, dbh + adv, idesc, (kc | k) != 0 ? 1u : 0u);      // A_hi B_hi
             umma_bf16_pair(d_cross, dah + adv, dbl + adv, idesc, (kb | k) != 0 ? 1u : 0u);     // A_hi B_lo
           }
-          if (kc == kDrain - 1 || kb + 1 == nk) {
+          if (kc == kDrain<EPI, F16> - 1 || kb + 1 == nk) {
             umma_commit_pair(mfull, 3);
             ++g;
           }
@@ -351,7 +356,7 @@ split_product_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
       if constexpr (F16) {
         if (p.ia) v = scale4(v, p.ia[row]);
         v = make_float4(v.x * o.fb.x, v.y * o.fb.y, v.z * o.fb.z, v.w * o.fb.w);
-        if constexpr (EPI != F_STORE) so = __frcp_rn(p.io ? p.io[row] : *p.ios);
+        if constexpr (kPairOut<EPI, F16>) so = __frcp_rn(p.io[row]);
       }
       // (N, hence every pitch, is a multiple of 4 for the products over atoms)
       if constexpr (EPI == F_ISTAG) v = make_float4(v.x - b.x, v.y - b.y, v.z - b.z, v.w - b.w);
@@ -374,7 +379,7 @@ split_product_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
           if (o.col + 2 < p.N) to[2] = v.z;
         }
       }
-      if constexpr (EPI != F_STORE) {                // the operand of the next product, zero in the padding past N
+      if constexpr (kPairOut<EPI, F16>) {            // the operand of the next product, zero in the padding past N
         if (o.col < p.split_half) {
           if (!o.in4) v = make_float4(o.col < p.N ? v.x : 0.f, o.col + 1 < p.N ? v.y : 0.f, o.col + 2 < p.N ? v.z : 0.f, 0.f);
           put_pair4<F16>(p.split + static_cast<int64_t>(row) * p.ld_split + o.col, p.split_half, F16 ? scale4(v, so) : v);
@@ -414,17 +419,19 @@ split_product_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
       const int row = m0 + row0 + lane, col0 = n0 + c * kChunk;
       if (row >= p.M) return;
       const int own_end = (row / p.bn + 1) * p.bn;                  // end of the column block that row lies in
-      const float f = F16 && p.iab ? *p.iab : 1.f, s = F16 ? __frcp_rn(*p.ios) : 1.f;
+      const float f = F16 ? *p.iab : 1.f;
 #pragma unroll
       for (int j = 0; j < 32; ++j) {
         const int n = col0 + j;
         if (n >= p.N || own_end > n / PM * PM) continue;
         const float v = __uint_as_float(acc[j]) * f;
-        uint32_t hi, lo;
-        split2<F16>(v * s, 0.f, hi, lo);
-        uint16_t* mp = p.split + static_cast<int64_t>(n) * p.ld_split + row;
-        mp[0] = static_cast<uint16_t>(hi);
-        mp[p.split_half] = static_cast<uint16_t>(lo);
+        if constexpr (kPairOut<EPI, F16>) {
+          uint32_t hi, lo;
+          split2<F16>(v, 0.f, hi, lo);
+          uint16_t* mp = p.split + static_cast<int64_t>(n) * p.ld_split + row;
+          mp[0] = static_cast<uint16_t>(hi);
+          mp[p.split_half] = static_cast<uint16_t>(lo);
+        }
         if (p.C) p.C[static_cast<int64_t>(n) * p.ldc + row] = v;
       }
     };
@@ -459,7 +466,7 @@ split_product_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
         __syncwarp();
         if (lane == 0) mbar_arrive_cluster(done);
       };
-      for (int kb = 0; kb < nk && ok; kb += kDrain, ++g) {
+      for (int kb = 0; kb < nk && ok; kb += kDrain<EPI, F16>, ++g) {
         ok = __all_sync(0xffffffffu, mbar_wait(mfull, g & 1, abort_flag));
         if (ok) drain(0, 1.f, mempty_leader);
       }
@@ -897,8 +904,7 @@ __global__ void __launch_bounds__(kPackThreads, 1) pack_long_kernel(const __grid
   }
 }
 
-// fp16 form, sparse coding: one scale for W^T (the smallest of W's rows) and one for W^T W, whose entries are at most
-// rows * max |w|^2.  iw: inverse scales of W's rows.
+// fp16 form, sparse coding: one scale for W^T (the smallest of W's rows).  iw: inverse scales of W's rows.
 __global__ void __launch_bounds__(1024) sc_scales_kernel(const float* __restrict__ iw, int rows, Scalars* sc) {
   pdl_launch_dependents();
   pdl_wait(iw);
@@ -911,10 +917,8 @@ __global__ void __launch_bounds__(1024) sc_scales_kernel(const float* __restrict
   __syncthreads();
   if (threadIdx.x == 0) {
     for (int w = 1; w < 32; ++w) m = fmaxf(m, sh[w]);
-    const float most = m * 16384.f;                    // of |w|
     sc->iWT = m;
     sc->iWT2 = m * m;
-    sc->iG = 1.f / pow2_scale(static_cast<float>(rows) * most * most, 13);
   }
 }
 
@@ -987,12 +991,13 @@ __global__ void __launch_bounds__(256) pack_u_kernel(const float* __restrict__ U
 // and to take over a part of a tile: a last round of tiles is cut when that gains more, and not into parts of less than
 // four k-blocks.
 struct ProductPlan { int bn; int64_t tiles, whole, pairs; double cost; };
-ProductPlan plan_width(int64_t M, int64_t N, int64_t Kc, bool sym, int bn, int64_t max_pairs) {
+// fine: drained at every k-block, which the MMAs of a third of it do not hide.
+ProductPlan plan_width(int64_t M, int64_t N, int64_t Kc, bool sym, bool fine, int bn, int64_t max_pairs) {
   ProductPlan p{};
   p.bn = bn;
   const int tm = static_cast<int>((M + PM - 1) / PM), tn = static_cast<int>((N + bn - 1) / bn);
   p.tiles = sym ? sym_tiles(tm, tn, bn) : static_cast<int64_t>(tm) * tn;
-  const double per_kb = std::max(7.2 * bn, (2.0 * kBytesA + bn * BK * 2.0) / 38.0);
+  const double per_kb = std::max(7.2 * bn, (2.0 * kBytesA + bn * BK * 2.0) / 38.0) + (fine ? 7.0 * bn : 0.0);
   const int64_t kseg = (Kc + BK - 1) / BK, rounds = p.tiles / max_pairs, rest = p.tiles % max_pairs;
   p.whole = p.tiles;
   p.pairs = std::min(p.tiles, max_pairs);
@@ -1009,11 +1014,11 @@ ProductPlan plan_width(int64_t M, int64_t N, int64_t Kc, bool sym, int bn, int64
   p.cost = kb * per_kb + 12000.0 + static_cast<double>(rounds) * 1500.0;
   return p;
 }
-ProductPlan plan_product(int64_t M, int64_t N, int64_t Kc, bool sym, int64_t max_pairs) {
-  if (N <= 64) return plan_width(M, N, Kc, sym, static_cast<int>(round_up(N, 32)), max_pairs);
+ProductPlan plan_product(int64_t M, int64_t N, int64_t Kc, bool sym, bool fine, int64_t max_pairs) {
+  if (N <= 64) return plan_width(M, N, Kc, sym, fine, static_cast<int>(round_up(N, 32)), max_pairs);
   ProductPlan best{};
   for (int bn = kMaxN; bn >= 64; bn -= 32) {
-    const ProductPlan p = plan_width(M, N, Kc, sym, bn, max_pairs);
+    const ProductPlan p = plan_width(M, N, Kc, sym, fine, bn, max_pairs);
     if (bn == kMaxN || p.cost < best.cost) best = p;
   }
   return best;
@@ -1024,7 +1029,7 @@ template <int EPI, bool F16>
 int split_product(sfb_ctx* ctx, int64_t off, int64_t n, const uint16_t* A, const uint16_t* B, int64_t N, int64_t Cp,
                   SplitParams p) {
   TcState* st = static_cast<TcState*>(ctx->tc);
-  const ProductPlan plan = plan_product(n, N, Cp, EPI == F_GRAM, std::min<int64_t>(st->max_pairs, sm_count() / 2));
+  const ProductPlan plan = plan_product(n, N, Cp, EPI == F_GRAM, kDrain<EPI, F16> == 1, std::min<int64_t>(st->max_pairs, sm_count() / 2));
   p.bn = plan.bn;
   p.whole = static_cast<int32_t>(plan.whole);
   p.partial = ctx->at<float>(ctx->lay.partial);
@@ -1162,7 +1167,7 @@ int factors_sc(sfb_ctx* ctx, int64_t off, int64_t n, const float* X) {
   }
   for (int t = 2; t <= T; ++t) {
     if (gram) {
-      rc = split_product<F_ISTAG, F16>(ctx, off, n, as[(t - 1) & 1], ctx->at<uint16_t>(L.Gs), cols, L.colsp, ista(t, iC, &sc->iG));
+      if constexpr (!F16) rc = split_product<F_ISTAG, F16>(ctx, off, n, as[(t - 1) & 1], ctx->at<uint16_t>(L.Gs), cols, L.colsp, ista(t, nullptr, nullptr));
     } else {
       if ((rc = residual(as[0])) != SFB_OK) return rc;
       rc = split_product<F_ISTA, F16>(ctx, off, n, Rs, WTs, cols, L.rowsp, ista(t, iR, &sc->iWT));  // a <- soft(a - W^T r / L)
@@ -1193,20 +1198,23 @@ int begin_operands(sfb_ctx* ctx) {
   if (F16) CKC(launch_kernel(sc_scales_kernel, dim3(1), dim3(1024), 0, s, 1, ctx->at<float>(L.iW), static_cast<int>(rows), sc));
   CKC(launch_kernel(pack_t_kernel<F16>, dim3(static_cast<unsigned>((cols + 63) / 64), static_cast<unsigned>(L.rowsp / 64)),
                     dim3(256), 0, s, 1, ctx->W, rows, cols, cols, WTs, L.rowsp, &sc->iWT));
-  if (!L.Gs) return SFB_OK;
+  if (!(F16 ? L.G : L.Gs)) return SFB_OK;
   SplitParams p{};
   p.four = rows <= kPreciseRows;
   p.C = c.sc_lipschitz > 0.f ? nullptr : ctx->at<float>(L.G);
   p.ldc = cols;
-  p.split = ctx->at<uint16_t>(L.Gs); p.ld_split = 2 * L.colsp; p.split_half = static_cast<int32_t>(L.colsp);
-  if (F16) { p.iab = &sc->iWT2; p.ios = &sc->iG; }
+  if (F16) {
+    p.iab = &sc->iWT2;
+  } else {
+    p.split = ctx->at<uint16_t>(L.Gs); p.ld_split = 2 * L.colsp; p.split_half = static_cast<int32_t>(L.colsp);
+  }
   return split_product<F_GRAM, F16>(ctx, 0, cols, WTs, WTs, cols, L.rowsp, p);
 }
 
 }  // namespace
 
-double split_product_cost(int64_t M, int64_t N, int64_t Kc, bool sym) {
-  return plan_product(M, N, Kc, sym, sm_count() / 2).cost;
+double split_product_cost(int64_t M, int64_t N, int64_t Kc, bool sym, bool fine) {
+  return plan_product(M, N, Kc, sym, fine, kModelSms / 2).cost;
 }
 
 void split_extend_layout(const sfb_config& c, Layout& L, size_t& off) {
@@ -1234,6 +1242,7 @@ void split_extend_layout(const sfb_config& c, Layout& L, size_t& off) {
     L.iC = take(K * 4);
   }
   L.WTs = take(static_cast<size_t>(c.cols) * 2 * L.rowsp * 2);        // W^T, atoms x (hi | lo)
+  if (f16 && sc_estimate_on_gram(c, split_product_cost(c.cols, c.cols, c.rows, true, true))) L.G = take(static_cast<size_t>(c.cols) * c.cols * 4);
   if (sc_use_gram(c)) {
     L.Gs = take(static_cast<size_t>(c.cols) * 2 * L.colsp * 2);       // W^T W, atoms x (hi | lo)
     L.G = take(c.sc_lipschitz > 0.f ? 0 : static_cast<size_t>(c.cols) * c.cols * 4);   // in fp32 for the power iteration

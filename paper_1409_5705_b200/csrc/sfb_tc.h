@@ -53,7 +53,7 @@ int split_factors_sc(sfb_ctx* ctx, int64_t off, int64_t n, const float* X);
 int split_pack_received(sfb_ctx* ctx, int64_t off, int64_t n);
 int split_gather(sfb_ctx* ctx);
 const uint16_t* split_v(const sfb_ctx* ctx);
-double split_product_cost(int64_t M, int64_t N, int64_t Kc, bool sym);
+double split_product_cost(int64_t M, int64_t N, int64_t Kc, bool sym, bool fine = false);     // fine: sparse coding in fp32 mode
 int tc_update(sfb_ctx* ctx);
 int tc_get_factors(sfb_ctx* ctx, const void** U, const void** V, int32_t* dtype, int32_t* layout, int64_t* ldu,
                    int64_t* ldv);
