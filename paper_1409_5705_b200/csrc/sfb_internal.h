@@ -115,7 +115,7 @@ struct Layout {
   // (hi | lo) operands of the split products
   size_t Ws, WTs, As, Rs;             // W by rows, W transposed, the A operand (v or the codes), the residual
   size_t partial, ready;              // parts of the tiles of a split product
-  size_t iW, iA, iR, iC, q;           // fp32 mode: inverse scales of the rows of W, of the pairs; see sfb_split.cu
+  size_t iW, iA, iR, iC, q, mR, mC;   // fp32 mode: inverse scales of the rows of W, of the pairs, what they are taken from; see sfb_split.cu
   // sparse factors (MLR, csr_nnz_max > 0): the step's (sample, column, value) triples and their column-major form
   size_t coo_i, coo_c, coo_x, coo_cx, row_beg, row_end, csc_cnt, csc_cur, csc_ptr, csc_tmp, csc_ent;
   // sparse coding: the dictionary's Gram matrix (when the coder iterates on it), W^T x, the codes of odd iterations, and

@@ -62,11 +62,16 @@ struct SplitParams {
   uint16_t* split;             // where kPairOut: [M x ld_split] receives hi at column n and lo at column split_half + n
   int64_t ld_split;
   int32_t split_half;          // padded N (a multiple of 64); columns N..split_half-1 are written as zeros
-  // fp16 form: inverse scales of A per row, of B per column of D, a factor for all (null: 1), and of the pair that goes out per row
+  // fp16 form: inverse scales of A per row, of B per column of D, a factor for all (null: 1)
   const float* ia;
   const float* ib;
   const float* iab;
-  const float* io;
+  // ... and of the pair that goes out, per row: from the largest value so far, most_in, whose inverse scale goes to io and which
+  // with the values of this product becomes most_out.  (Iterations that diverge, on an L below ||W||^2 / 2, keep their precision as
+  // long as no value grows by more than 2^12 in one of them.)
+  const float* most_in;
+  float* most_out;
+  float* io;
   uint32_t* status;
 };
 
@@ -80,6 +85,7 @@ __device__ __forceinline__ float pow2_scale(float m, int top) {
   if (ex == 128) return 1.f;
   return __int_as_float((min(max(top - ex, -120), 120) + 127) << 23);
 }
+constexpr int kTop = 3;                             // of the largest value so far of a sample's codes and residuals
 // two neighbouring values (already scaled in the fp16 form) as packed words
 template <bool F16>
 __device__ __forceinline__ void split2(float f0, float f1, uint32_t& hi, uint32_t& lo) {
@@ -352,11 +358,9 @@ split_product_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
       return o;
     };
     auto put = [&](const Place& o, int row, float4 v, const float4& x, const float4& b) {
-      float so = 1.f;
       if constexpr (F16) {
         if (p.ia) v = scale4(v, p.ia[row]);
         v = make_float4(v.x * o.fb.x, v.y * o.fb.y, v.z * o.fb.z, v.w * o.fb.w);
-        if constexpr (kPairOut<EPI, F16>) so = __frcp_rn(p.io[row]);
       }
       // (N, hence every pitch, is a multiple of 4 for the products over atoms)
       if constexpr (EPI == F_ISTAG) v = make_float4(v.x - b.x, v.y - b.y, v.z - b.z, v.w - b.w);
@@ -382,7 +386,18 @@ split_product_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
       if constexpr (kPairOut<EPI, F16>) {            // the operand of the next product, zero in the padding past N
         if (o.col < p.split_half) {
           if (!o.in4) v = make_float4(o.col < p.N ? v.x : 0.f, o.col + 1 < p.N ? v.y : 0.f, o.col + 2 < p.N ? v.z : 0.f, 0.f);
-          put_pair4<F16>(p.split + static_cast<int64_t>(row) * p.ld_split + o.col, p.split_half, F16 ? scale4(v, so) : v);
+          uint16_t* to = p.split + static_cast<int64_t>(row) * p.ld_split + o.col;
+          if constexpr (F16) {
+            const float most = p.most_in[row], so = pow2_scale(most, kTop);
+            const float here = fmaxf(fmaxf(fabsf(v.x), fabsf(v.y)), fmaxf(fabsf(v.z), fabsf(v.w)));
+            if (here > most) atomicMax(reinterpret_cast<int*>(p.most_out + row), __float_as_int(here));
+            if (o.col == 0) {
+              atomicMax(reinterpret_cast<int*>(p.most_out + row), __float_as_int(most));
+              p.io[row] = 1.f / so;
+            }
+            v = scale4(v, so);
+          }
+          put_pair4<F16>(to, p.split_half, v);
         }
       }
     };
@@ -724,22 +739,23 @@ struct Pack16 {
   int64_t dimp;
   float* inv;
   float* inv2;                 // the same again (may be null)
-  // sparse coding: inverse scales of the sample's residuals (at most ||x||) and of its codes: an ISTA step moves a code by at
-  // most ||W^T r|| / L <= ||x|| / sqrt(L), so T of them stay below T ||x|| / sqrt(L).  Both bounds hold for L >= ||W||^2; they
-  // go to 2^4, so an iteration that diverges on a smaller L has a factor of 2^11 left.
-  float* inv_res;
+  // sparse coding: what the sample's residuals and codes begin with as their largest values, ||x|| and ||x|| / sqrt(L), in both of
+  // the buffers that the iterations take in turn (of `samples` each), and the inverse scale of codes that no iteration makes
+  float* res;
+  float* code;
   float* inv_code;
+  int64_t samples;
   const Scalars* sc;
-  float iters;
   Stamp stamp;
 };
 __device__ __forceinline__ void row_scales(const Pack16& p, int64_t r, float s, float ss) {
   p.inv[r] = 1.f / s;
   if (p.inv2) p.inv2[r] = 1.f / s;
-  if (p.inv_res) {
-    const float norm = sqrtf(ss);
-    p.inv_res[r] = 1.f / pow2_scale(norm, 4);
-    p.inv_code[r] = 1.f / pow2_scale(p.iters * norm * sqrtf(p.sc->invL), 4);
+  if (p.res) {
+    const float norm = sqrtf(ss), code = norm * sqrtf(p.sc->invL);
+    p.res[r] = p.res[p.samples + r] = norm;
+    p.code[r] = p.code[p.samples + r] = code;
+    p.inv_code[r] = 1.f / pow2_scale(code, kTop);
   }
 }
 template <int TPR>
@@ -767,7 +783,7 @@ __global__ void __launch_bounds__(256) pack16_kernel(const __grid_constant__ Pac
   float m = 0.f, ss = 0.f;
   auto look = [&](const float4& v) {
     m = fmaxf(m, fmaxf(fmaxf(fabsf(v.x), fabsf(v.y)), fmaxf(fabsf(v.z), fabsf(v.w))));
-    if (p.inv_res) ss = fmaf(v.x, v.x, fmaf(v.y, v.y, fmaf(v.z, v.z, fmaf(v.w, v.w, ss))));
+    if (p.res) ss = fmaf(v.x, v.x, fmaf(v.y, v.y, fmaf(v.z, v.z, fmaf(v.w, v.w, ss))));
   };
   float4 held[kHeld];
   if (vec) {
@@ -870,7 +886,7 @@ __global__ void __launch_bounds__(kPackThreads, 1) pack_long_kernel(const __grid
           row[q] = v;                                    // (this thread reads it again)
         }
         m = fmaxf(m, fmaxf(fmaxf(fabsf(v.x), fabsf(v.y)), fmaxf(fabsf(v.z), fabsf(v.w))));
-        if (p.inv_res) ss = fmaf(v.x, v.x, fmaf(v.y, v.y, fmaf(v.z, v.z, fmaf(v.w, v.w, ss))));
+        if (p.res) ss = fmaf(v.x, v.x, fmaf(v.y, v.y, fmaf(v.z, v.z, fmaf(v.w, v.w, ss))));
       }
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) {
@@ -1120,9 +1136,12 @@ int factors_sc(sfb_ctx* ctx, int64_t off, int64_t n, const float* X) {
   Scalars* sc = ctx->at<Scalars>(L.scalars);
   // the iterates as operands: with the Gram matrix a product reads one and writes the next, so two buffers in turn
   uint16_t* as[2] = {ctx->at<uint16_t>(L.As), ctx->at<uint16_t>(gram ? L.As2 : L.As)};
+  const int64_t K = ctx->K;
   const float* iX = F16 ? ctx->at<float>(L.iA) : nullptr;
-  const float* iR = F16 ? ctx->at<float>(L.iR) : nullptr;
-  const float* iC = F16 ? ctx->at<float>(L.iC) : nullptr;
+  float* iR = F16 ? ctx->at<float>(L.iR) : nullptr;
+  float* iC = F16 ? ctx->at<float>(L.iC) : nullptr;                  // [2][K]: of odd and even iterations
+  float* mR = F16 ? ctx->at<float>(L.mR) : nullptr;                  // [2][K], as mC
+  float* mC = F16 ? ctx->at<float>(L.mC) : nullptr;
   auto ista = [&](int t, const float* ia, const float* iab) {
     SplitParams q{};
     q.C = V; q.ldc = cols;
@@ -1130,15 +1149,19 @@ int factors_sc(sfb_ctx* ctx, int64_t off, int64_t n, const float* X) {
     q.C2 = gram ? ctx->at<float>(L.Bx) : nullptr;
     q.sc = sc; q.lam = c.sc_lambda;
     q.split = as[t & 1]; q.ld_split = 2 * L.colsp; q.split_half = static_cast<int32_t>(L.colsp);
-    if (F16) { q.ia = ia; q.iab = iab; q.io = iC; }
+    if (F16) { q.ia = ia; q.iab = iab; q.most_in = mC + ((t + 1) & 1) * K; q.most_out = mC + (t & 1) * K; q.io = iC + (t & 1) * K; }
     return q;
   };
-  auto residual = [&](uint16_t* a) {                                                    // r = W a - x
+  auto residual = [&](int t) {                                                          // r = W a_t - x
+    uint16_t* a = as[gram ? t & 1 : 0];
     SplitParams q{};
     q.C = ctx->at<float>(L.U); q.ldc = L.ldu;
     q.aux = X - off * rows; q.ldaux = rows; q.aux_row0 = static_cast<int32_t>(off);          // X holds this worker's samples: index it by the global row
     q.split = Rs; q.ld_split = 2 * L.rowsp; q.split_half = static_cast<int32_t>(L.rowsp);
-    if (F16) { q.ia = iC; q.ib = ctx->at<float>(L.iW); q.io = iR; }
+    if (F16) {
+      q.ia = iC + (t & 1) * K; q.ib = ctx->at<float>(L.iW);
+      q.most_in = mR + ((t + 1) & 1) * K; q.most_out = mR + (t & 1) * K; q.io = iR;
+    }
     return split_product<F_SUB, F16>(ctx, off, n, a, Ws, rows, L.colsp, q);
   };
   int rc = SFB_OK;
@@ -1146,8 +1169,8 @@ int factors_sc(sfb_ctx* ctx, int64_t off, int64_t n, const float* X) {
     Pack16 p{};
     p.F = X; p.n = n; p.dim = p.ld = rows; p.dst = Rs + off * 2 * L.rowsp; p.dimp = L.rowsp;
     p.inv = ctx->at<float>(L.iA) + off;
-    p.inv_res = ctx->at<float>(L.iR) + off; p.inv_code = ctx->at<float>(L.iC) + off;
-    p.sc = sc; p.iters = static_cast<float>(T);
+    p.res = mR + off; p.code = mC + off; p.inv_code = iC + off; p.samples = K;
+    p.sc = sc;
     CKC(pack16(ctx, p));
   }
   if (T == 0) {
@@ -1169,12 +1192,12 @@ int factors_sc(sfb_ctx* ctx, int64_t off, int64_t n, const float* X) {
     if (gram) {
       if constexpr (!F16) rc = split_product<F_ISTAG, F16>(ctx, off, n, as[(t - 1) & 1], ctx->at<uint16_t>(L.Gs), cols, L.colsp, ista(t, nullptr, nullptr));
     } else {
-      if ((rc = residual(as[0])) != SFB_OK) return rc;
+      if ((rc = residual(t - 1)) != SFB_OK) return rc;
       rc = split_product<F_ISTA, F16>(ctx, off, n, Rs, WTs, cols, L.rowsp, ista(t, iR, &sc->iWT));  // a <- soft(a - W^T r / L)
     }
     if (rc) return rc;
   }
-  return residual(as[T & 1]);                                                           // u = W a - x
+  return residual(T);                                                                   // u = W a - x
 }
 
 template <bool F16>
@@ -1239,7 +1262,9 @@ void split_extend_layout(const sfb_config& c, Layout& L, size_t& off) {
   if (c.model != SFB_SC) return;
   if (f16) {
     L.iR = take(K * 4);
-    L.iC = take(K * 4);
+    L.iC = take(2 * K * 4);
+    L.mR = take(2 * K * 4);
+    L.mC = take(2 * K * 4);
   }
   L.WTs = take(static_cast<size_t>(c.cols) * 2 * L.rowsp * 2);        // W^T, atoms x (hi | lo)
   if (f16 && sc_estimate_on_gram(c, split_product_cost(c.cols, c.cols, c.rows, true, true))) L.G = take(static_cast<size_t>(c.cols) * c.cols * 4);
@@ -1307,7 +1332,10 @@ const uint16_t* split_v(const sfb_ctx* ctx) {
   const bool odd = ctx->cfg.model == SFB_SC && L.Gs != 0 && (ctx->cfg.sc_ista_iters & 1);     // which buffer the last iterate is in
   return ctx->at<uint16_t>(odd ? L.As2 : L.As);
 }
-static float* inv_v(const sfb_ctx* ctx) { return ctx->at<float>(ctx->cfg.model == SFB_SC ? ctx->lay.iC : ctx->lay.iA); }
+static float* inv_v(const sfb_ctx* ctx) {
+  if (ctx->cfg.model != SFB_SC) return ctx->at<float>(ctx->lay.iA);
+  return ctx->at<float>(ctx->lay.iC) + (ctx->cfg.sc_ista_iters & 1) * ctx->K;
+}
 
 int split_pack_received(sfb_ctx* ctx, int64_t off, int64_t n) {
   const sfb_config& c = ctx->cfg;

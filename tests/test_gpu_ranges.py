@@ -124,3 +124,30 @@ def test_codes_of_fitted_samples(rows, cols, P, B):
         c = np.sign(g) * np.maximum(np.abs(g) - 0.1 / L, 0)
     assert np.linalg.norm(V - c) <= 10 * 2.0 ** -24 * np.linalg.norm(c)
     assert np.linalg.norm(U - (c @ Wd.T - X)) <= 10 * 2.0 ** -24 * np.linalg.norm(X)
+
+
+# An L below ||W||^2 / 2, on which the iterations diverge (values of 1e8 and more here): still the iterates, to the precision of the mode, on
+# pairs of words with scales, in fp64 and on the FMA kernels.
+@pytest.mark.parametrize("rows,cols,P,B,T", [(772, 1280, 2, 467, 20), (772, 1280, 2, 467, 7), (2000, 1000, 1, 128, 20), (2000, 1400, 4, 128, 20), (90, 64, 1, 8, 12)])
+def test_codes_of_diverging_iterations(rows, cols, P, B, T):
+    rng = np.random.default_rng(rows + cols)
+    W0 = rng.standard_normal((rows, cols)).astype(np.float32)
+    W0 /= np.linalg.norm(W0, axis=0, keepdims=True)
+    K = P * B
+    X = rng.standard_normal((K, rows)).astype(np.float32)
+    X[1] *= 1e-3
+    Wd = W0.astype(np.float64)
+    L = float(np.float32(np.linalg.norm(Wd, 2) ** 2 / 6))
+    W = to_dev(W0, torch)
+    ctx = S.Context(S.make_config(S.SC, rows, cols, P, B, 1e-3, S.PREC_FP32, sc_lambda=0.1, sc_ista_iters=T, sc_lipschitz=L), W)
+    ctx.sfb_compute_factors(-1, to_dev(X, torch))
+    U, V = (t.cpu().numpy().astype(np.float64) for t in ctx.factors_as_tensors())
+    assert ctx.sfb_get_status() == 0
+    ctx.close()
+    c = np.zeros((K, cols))
+    for _ in range(T):
+        g = c - (c @ Wd.T - X) @ Wd / L
+        c = np.sign(g) * np.maximum(np.abs(g) - 0.1 / L, 0)
+    assert np.linalg.norm(V - c) <= 1e-5 * np.linalg.norm(c)
+    u = c @ Wd.T - X
+    assert np.linalg.norm(U - u) <= 1e-5 * np.linalg.norm(u)
