@@ -16,7 +16,7 @@ inline void count_launch(int n = 1) { g_kernel_launches.fetch_add(n, std::memory
 
 // Multiprocessors of the current device (looked up once per device ordinal).
 int sm_count();
-constexpr int kModelSms = 148;        // what the cost models count with
+constexpr int kModelSms = 148;        // what the cost models, hence the layout of a workspace, count with: no CUDA call
 
 // ---------------------------------------------------------------------------------------------------------
 // Launches.  A step is a chain of dependent kernels, several of them only microseconds long: each is launched with

@@ -631,7 +631,7 @@ int sparse_forward_rows(const sfb_config& c, int64_t n) {
 // scattered samples 160,000.  For the room for entries, so that a slice of the mini-batch takes the same kernel.
 static double row_wise_cycles(const sfb_config& c, int rb) {
   const double K = static_cast<double>(c.workers) * c.batch, entries = static_cast<double>(c.csr_nnz_max) / K;
-  const double rounds = static_cast<double>(((c.rows + rb - 1) / rb + sm_count() - 1) / sm_count());
+  const double rounds = static_cast<double>(((c.rows + rb - 1) / rb + kModelSms - 1) / kModelSms);
   return rounds * (std::ceil(K / kSfWarps) * (900.0 + 40.0 * entries * rb / 32.0) + static_cast<double>(rb * c.cols) * 4.0 / 25.0);
 }
 // Whether the row-wise forward is faster than the FMA product.

@@ -1045,7 +1045,7 @@ template <int EPI, bool F16>
 int split_product(sfb_ctx* ctx, int64_t off, int64_t n, const uint16_t* A, const uint16_t* B, int64_t N, int64_t Cp,
                   SplitParams p) {
   TcState* st = static_cast<TcState*>(ctx->tc);
-  const ProductPlan plan = plan_product(n, N, Cp, EPI == F_GRAM, kDrain<EPI, F16> == 1, std::min<int64_t>(st->max_pairs, sm_count() / 2));
+  const ProductPlan plan = plan_product(n, N, Cp, EPI == F_GRAM, kDrain<EPI, F16> == 1, std::min<int64_t>(st->max_pairs, std::min(sm_count(), kModelSms) / 2));
   p.bn = plan.bn;
   p.whole = static_cast<int32_t>(plan.whole);
   p.partial = ctx->at<float>(ctx->lay.partial);
@@ -1252,8 +1252,8 @@ void split_extend_layout(const sfb_config& c, Layout& L, size_t& off) {
   L.Rs = take(K * 2 * static_cast<size_t>(L.rowsp) * 2);              // u (SC: first x, then the residuals)
   L.Ws = take(static_cast<size_t>(c.rows) * 2 * L.colsp * 2);         // W, rows x (hi | lo)
   L.As = take(K * 2 * static_cast<size_t>(L.colsp) * 2);              // v (MLR, DML) or the codes a (SC)
-  L.partial = take(static_cast<size_t>(sm_count() / 2) * 2 * kEpi * 4 * kSlot);      // parts of tiles (see split_product_kernel)
-  L.ready = take(static_cast<size_t>(sm_count() / 2) * 2 * kEpi * 4);
+  L.partial = take(static_cast<size_t>(kModelSms / 2) * 2 * kEpi * 4 * kSlot);      // parts of tiles (see split_product_kernel)
+  L.ready = take(static_cast<size_t>(kModelSms / 2) * 2 * kEpi * 4);
   if (f16) {
     L.iW = take((static_cast<size_t>(c.rows) + 32) * 4);              // inverse scales: rows of W, pairs
     L.iA = take(K * 4);
@@ -1278,7 +1278,7 @@ void split_extend_layout(const sfb_config& c, Layout& L, size_t& off) {
 
 // A launch that ran into a wait limit may have left flags set.
 cudaError_t split_reset(sfb_ctx* ctx) {
-  return cudaMemsetAsync(ctx->at<char>(ctx->lay.ready), 0, static_cast<size_t>(sm_count() / 2) * 2 * kEpi * 4, ctx->stream);
+  return cudaMemsetAsync(ctx->at<char>(ctx->lay.ready), 0, static_cast<size_t>(kModelSms / 2) * 2 * kEpi * 4, ctx->stream);
 }
 
 // Pad columns of the operands are never written by the kernels: cleared once.

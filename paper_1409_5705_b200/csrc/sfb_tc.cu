@@ -777,7 +777,7 @@ static int forward_stages(int bn) { return std::min(S_MAX, S * (kBytesA + kBytes
 static double forward_cost(int64_t n, int64_t rows, int64_t cols, int bn, int split) {
   const double kb = static_cast<double>((cols + BK - 1) / BK), ar = static_cast<double>(std::min<int64_t>(BM, round_up(n, 8)));
   const int64_t ctas = ((n + BM - 1) / BM) * ((rows + bn - 1) / bn) * split;
-  const double rounds = static_cast<double>((ctas + sm_count() - 1) / sm_count());
+  const double rounds = static_cast<double>((ctas + kModelSms - 1) / kModelSms);
   const double per_kb = std::max(std::max(2.0 * bn, (ar + bn) * BK * 2 / 60.0), 1200.0 / forward_stages(bn));
   return rounds * (kb / split * per_kb + 2500.0 + (split > 1 ? 3000.0 : 0.0));
 }
