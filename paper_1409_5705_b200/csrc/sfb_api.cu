@@ -46,7 +46,7 @@ bool sc_use_gram(const sfb_config& c) {
 // The power iteration on W^T W, whose rows stay on chip, or on W, which comes from L2 or memory twice an iteration, with a barrier
 // between (2,500 x 1,000: 2.6 us an iteration against 21).
 bool sc_estimate_on_gram(const sfb_config& c, double form) {
-  if (c.sc_lipschitz > 0.f || c.cols > kMostAtoms) return false;
+  if (c.sc_lipschitz > 0.f || c.cols > kMostAtoms || !derived_fit(c, 8.0)) return false;
   const double D = static_cast<double>(c.rows), A = static_cast<double>(c.cols);
   return form + 50.0 * (4000.0 + A * A * 4.0 / 3000.0) < 50.0 * (10000.0 + D * A * 8.0 / 640.0);
 }
@@ -59,7 +59,7 @@ static double sc_fma_cost(const sfb_config& c, bool& gram64) {
   gram64 = false;
   if (it < 0) return last + there;
   const double two = gemm_cycles(K, A, D) + it * (gemm_cycles(K, D, A) + gemm_cycles(K, A, D)) + last + there;
-  if (it < 1 || A > kMostAtoms) return two;
+  if (it < 1 || A > kMostAtoms || !derived_fit(c, 8.0)) return two;
   const double one = form + gram64_cost(A, K, D) + it * gram64_cost(A, K, A) + last + 10000.0;
   gram64 = one < two;
   return std::min(one, two);

@@ -3,6 +3,10 @@ import os
 import subprocess
 import sys
 
+import pytest
+
+import paper_1409_5705_b200 as S
+
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
 
@@ -21,3 +25,13 @@ print("asked")
     out = subprocess.run([sys.executable, "-c", prog], cwd=ROOT, env=dict(os.environ, LD_DEBUG="libs"), capture_output=True, text=True)
     assert out.returncode == 0 and "asked" in out.stdout, out.stderr[-500:]
     assert "libcuda.so" not in out.stderr
+
+
+@pytest.mark.parametrize("model,rows,cols,K", [(S.MLR, 1_100_000, 20_000, 64), (S.DML, 200_000, 110_000, 64), (S.SC, 1_000_000, 20_000, 8),
+                                               (S.SC, 700_000, 20_000, 64), (S.L2MLR, 2_000_000, 11_000, 100)])
+def test_fp32_contexts_fit_the_gpu_where_w_does(model, rows, cols, K):
+    """The pairs of W that the fp32 mode derives must not be what keeps a matrix from fitting the 180 GB."""
+    kw = dict(sdca_lambda=0.1, sdca_n=1) if model == S.L2MLR else {}
+    assert 4 * rows * cols + S.sfb_workspace_bytes(S.make_config(model, rows, cols, 1, K, 0.1, S.PREC_FP32, **kw)) <= 165e9
+    # (and are still derived where they fit)
+    assert S.sfb_workspace_bytes(S.make_config(model, rows // 4, cols, 1, 200, 0.1, S.PREC_FP32, **kw)) >= rows * cols
