@@ -253,7 +253,9 @@ int sfb_step(sfb_ctx* ctx, const float* X_dev, const float* Y_dev, const int32_t
 /* The same step for callers whose minibatch lives in HOST memory (pinned memory recommended): copies
  * X_host [K x in_dim] (and Y_host, labels_host when the model uses them) to staging buffers inside the
  * workspace, runs the step, copies the step's mean loss (MLR; 0 otherwise) and the status word back, and
- * waits for the stream.  loss_out and status_out may be NULL. */
+ * waits for the stream.  loss_out and status_out may be NULL.  The first call of a context makes a stream for the copies,
+ * nine events and a page of page-locked host memory, which sfb_destroy frees.  On an error the call still waits for the copies
+ * it has enqueued: the host buffers are the caller's again when it returns. */
 int sfb_step_host(sfb_ctx* ctx, const float* X_host, const float* Y_host, const int32_t* labels_host,
                   float* loss_out, uint32_t* status_out);
 

@@ -824,18 +824,13 @@ extern "C" int sfb_step(sfb_ctx* ctx, const float* X_dev, const float* Y_dev, co
   return sfb_apply_update(ctx);
 }
 
-extern "C" int sfb_step_host(sfb_ctx* ctx, const float* X_host, const float* Y_host, const int32_t* labels_host,
-                             float* loss_out, uint32_t* status_out) {
-  if (!ctx || !X_host) return SFB_ERR_ARG;
-  if (ctx->sdca) return SFB_ERR_UNSUPPORTED;
+// The copies in, the step and the copy of what is read back, all enqueued.
+static int enqueue_host_step(sfb_ctx* ctx, const float* X_host, const float* Y_host, const int32_t* labels_host) {
   const sfb_config& c = ctx->cfg;
-  if (c.model == SFB_DML && (!Y_host || !labels_host)) return SFB_ERR_ARG;
-  if (c.model == SFB_MLR && !labels_host) return SFB_ERR_ARG;
+  HostSide& h = *ctx->host;
   float* Xs = ctx->at<float>(ctx->lay.stageX);
   float* Ys = ctx->at<float>(ctx->lay.stageY);
   int32_t* Ls = ctx->at<int32_t>(ctx->lay.stageL);
-  if (!ctx->host) CK(make_host_side(ctx));
-  HostSide& h = *ctx->host;
   // MLR in bf16 mode: the logits of a part of the samples are formed while the next part is copied (20,000 x 4,000, K = 512: the
   // copy's 178 us in line with the step's 330 before).
   const int parts = c.precision == SFB_PREC_BF16 ? tc_host_parts(ctx) : 1;
@@ -858,12 +853,27 @@ extern "C" int sfb_step_host(sfb_ctx* ctx, const float* X_host, const float* Y_h
   h.parts = parts;
   const int rc = sfb_step(ctx, Xs, c.model == SFB_DML ? Ys : nullptr, c.model != SFB_SC ? Ls : nullptr);
   h.parts = 0;
-  if (rc) {
-    if (parts > 1) cudaStreamSynchronize(h.copies);      // the caller's buffer is not read after the return
-    return rc;
-  }
+  if (rc) return rc;
   // status word and scalars lie side by side: one copy, to page-locked memory
   CK(cudaMemcpyAsync(h.back, ctx->at<char>(ctx->lay.status), ctx->lay.loss - ctx->lay.status, cudaMemcpyDeviceToHost, ctx->stream));
+  return SFB_OK;
+}
+
+extern "C" int sfb_step_host(sfb_ctx* ctx, const float* X_host, const float* Y_host, const int32_t* labels_host,
+                             float* loss_out, uint32_t* status_out) {
+  if (!ctx || !X_host) return SFB_ERR_ARG;
+  if (ctx->sdca) return SFB_ERR_UNSUPPORTED;
+  const sfb_config& c = ctx->cfg;
+  if (c.model == SFB_DML && (!Y_host || !labels_host)) return SFB_ERR_ARG;
+  if (c.model == SFB_MLR && !labels_host) return SFB_ERR_ARG;
+  if (!ctx->host) CK(make_host_side(ctx));
+  HostSide& h = *ctx->host;
+  const int rc = enqueue_host_step(ctx, X_host, Y_host, labels_host);
+  if (rc) {                                              // whatever failed: the caller's buffers are not read after the return
+    cudaStreamSynchronize(h.copies);
+    cudaStreamSynchronize(ctx->stream);
+    return rc;
+  }
   CK(cudaStreamSynchronize(ctx->stream));
   const Scalars* sc = reinterpret_cast<const Scalars*>(h.back + (ctx->lay.scalars - ctx->lay.status));
   if (loss_out) *loss_out = sc->loss_mean;

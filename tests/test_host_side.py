@@ -35,3 +35,88 @@ def test_fp32_contexts_fit_the_gpu_where_w_does(model, rows, cols, K):
     assert 4 * rows * cols + S.sfb_workspace_bytes(S.make_config(model, rows, cols, 1, K, 0.1, S.PREC_FP32, **kw)) <= 165e9
     # (and are still derived where they fit)
     assert S.sfb_workspace_bytes(S.make_config(model, rows // 4, cols, 1, 200, 0.1, S.PREC_FP32, **kw)) >= rows * cols
+
+
+# csrc/sfb_api.cu against a fake of the CUDA runtime that counts the copies in flight: the n-th fallible call fails.
+FAKE = r"""
+#include <cmath>
+#include <cstdio>
+#include <cstdlib>
+#include <cstring>
+#include <map>
+static std::map<void*, int> in_flight;      // host copies enqueued per stream
+static int calls = 0, fail_at = -1, step_rc = 0, host_parts = 4;
+static bool joined = false;
+static bool failing() { return calls++ == fail_at; }
+#include "sfb_api.cu"
+extern "C" {
+cudaError_t cudaStreamCreateWithFlags(cudaStream_t* s, unsigned) { *s = reinterpret_cast<cudaStream_t>(2); return cudaSuccess; }
+cudaError_t cudaStreamDestroy(cudaStream_t) { return cudaSuccess; }
+cudaError_t cudaEventCreateWithFlags(cudaEvent_t* e, unsigned) { *e = reinterpret_cast<cudaEvent_t>(1); return cudaSuccess; }
+cudaError_t cudaEventDestroy(cudaEvent_t) { return cudaSuccess; }
+cudaError_t cudaHostAlloc(void** p, size_t n, unsigned) { *p = calloc(1, n); return cudaSuccess; }
+cudaError_t cudaFreeHost(void* p) { free(p); return cudaSuccess; }
+cudaError_t cudaEventRecord(cudaEvent_t, cudaStream_t) { return failing() ? cudaErrorUnknown : cudaSuccess; }
+cudaError_t cudaStreamWaitEvent(cudaStream_t, cudaEvent_t, unsigned) { return failing() ? cudaErrorUnknown : cudaSuccess; }
+cudaError_t cudaMemcpyAsync(void*, const void*, size_t, cudaMemcpyKind k, cudaStream_t s) {
+  if (failing()) return cudaErrorUnknown;
+  if (k == cudaMemcpyHostToDevice) in_flight[s]++;
+  return cudaSuccess;
+}
+cudaError_t cudaStreamSynchronize(cudaStream_t s) {
+  in_flight[s] = 0;
+  if (joined && s == reinterpret_cast<cudaStream_t>(1)) in_flight[reinterpret_cast<cudaStream_t>(2)] = 0;
+  return cudaSuccess;
+}
+}
+namespace sfb {
+int tc_host_parts(const sfb_ctx*) { return host_parts; }
+int tc_factors(sfb_ctx*, int64_t, int64_t, const float*, const float*, const int32_t*, bool, float*) {
+  joined = step_rc == 0;                    // the step's stream has waited for the copies' events
+  return step_rc;
+}
+int tc_update(sfb_ctx*) { return SFB_OK; }
+void tc_destroy(sfb_ctx*) {}
+}
+int main() {
+  for (int parts : {4, 1})
+    for (step_rc = 0; step_rc >= -1; --step_rc)
+      for (fail_at = -1; fail_at < 24; ++fail_at) {
+        sfb_ctx* ctx = new sfb_ctx();
+        ctx->cfg.model = SFB_MLR; ctx->cfg.precision = SFB_PREC_BF16;
+        ctx->cfg.rows = 8; ctx->cfg.cols = 8; ctx->cfg.workers = 1; ctx->cfg.batch = 512;
+        ctx->K = 512; ctx->in_dim = 8;
+        alignas(1024) static char ws[1 << 16];
+        ctx->ws = ws;
+        ctx->lay.loss = 4096; ctx->lay.scalars = 1024; ctx->lay.stageX = 8192; ctx->lay.stageL = 32768;
+        ctx->stream = reinterpret_cast<cudaStream_t>(1);
+        calls = 0;
+        joined = false;
+        host_parts = parts;
+        in_flight.clear();
+        alignas(16) static float X[512 * 8];
+        static int32_t y[512];
+        float loss;
+        uint32_t status;
+        const int rc = sfb_step_host(ctx, X, nullptr, y, &loss, &status);
+        for (auto& f : in_flight)
+          if (f.second) { printf("rc %d with %d copies in flight (call %d failed, step %d)\n", rc, f.second, fail_at, step_rc); return 1; }
+        if (ctx->host && ctx->host->parts) { printf("parts left set\n"); return 1; }
+        if ((rc != 0) != (step_rc != 0 || (fail_at >= 0 && fail_at < calls))) { printf("rc %d, call %d\n", rc, fail_at); return 1; }
+        sfb_destroy(ctx);
+      }
+  printf("ok\n");
+  return 0;
+}
+"""
+
+
+def test_host_step_returns_no_buffer_that_is_still_read(tmp_path):
+    src, exe = tmp_path / "fake.cpp", tmp_path / "fake"
+    src.write_text(FAKE)
+    csrc = os.path.join(ROOT, "paper_1409_5705_b200", "csrc")
+    cuda = next(p for p in ("/usr/local/cuda", "/usr/local/cuda-12.9") if os.path.exists(os.path.join(p, "include", "cuda_runtime.h")))
+    subprocess.check_call(["g++", "-std=c++17", "-w", "-I", os.path.join(ROOT, "include"), "-I", csrc, "-I", os.path.join(cuda, "include"), str(src),
+                           "-o", str(exe), "-Wl,--unresolved-symbols=ignore-all"])
+    out = subprocess.run([str(exe)], capture_output=True, text=True)
+    assert out.returncode == 0, out.stdout + out.stderr
