@@ -654,7 +654,7 @@ __global__ void __launch_bounds__(256) pack_t_kernel(const float* __restrict__ F
   pdl_launch_dependents();
   pdl_wait(inv);
   __shared__ float tile[64][65];
-  const int64_t i0 = static_cast<int64_t>(blockIdx.y) * 64, c0 = static_cast<int64_t>(blockIdx.x) * 64;
+  const int64_t cblocks = (dim + 63) / 64, i0 = blockIdx.x / cblocks * 64, c0 = blockIdx.x % cblocks * 64;
   const int t = threadIdx.x;
   const float s = F16 ? 1.f / *inv : 1.f;
 #pragma unroll
@@ -1219,8 +1219,9 @@ int begin_operands(sfb_ctx* ctx) {
   if (c.model != SFB_SC) return SFB_OK;
   uint16_t* WTs = ctx->at<uint16_t>(L.WTs);
   if (F16) CKC(launch_kernel(sc_scales_kernel, dim3(1), dim3(1024), 0, s, 1, ctx->at<float>(L.iW), static_cast<int>(rows), sc));
-  CKC(launch_kernel(pack_t_kernel<F16>, dim3(static_cast<unsigned>((cols + 63) / 64), static_cast<unsigned>(L.rowsp / 64)),
-                    dim3(256), 0, s, 1, ctx->W, rows, cols, cols, WTs, L.rowsp, &sc->iWT));
+  const int64_t blocks = ((cols + 63) / 64) * (L.rowsp / 64);
+  if (blocks > 0x7fffffffLL) return SFB_ERR_SHAPE;
+  CKC(launch_kernel(pack_t_kernel<F16>, dim3(static_cast<unsigned>(blocks)), dim3(256), 0, s, 1, ctx->W, rows, cols, cols, WTs, L.rowsp, &sc->iWT));
   if (!(F16 ? L.G : L.Gs)) return SFB_OK;
   SplitParams p{};
   p.four = rows <= kPreciseRows;

@@ -151,3 +151,23 @@ def test_codes_of_diverging_iterations(rows, cols, P, B, T):
     assert np.linalg.norm(V - c) <= 1e-5 * np.linalg.norm(c)
     u = c @ Wd.T - X
     assert np.linalg.norm(U - u) <= 1e-5 * np.linalg.norm(u)
+
+
+# More than 65,535 blocks of 64 features.
+@pytest.mark.parametrize("prec", [pytest.param(S.PREC_FP32, id="fp32"), pytest.param(S.PREC_BF16, id="bf16")])
+def test_sparse_coding_of_millions_of_features(prec):
+    rows, cols, K, T = 4_194_400, 64, 128, 3
+    g = torch.Generator(device="cuda").manual_seed(1)
+    W = torch.randn(rows, cols, generator=g, device="cuda") / np.sqrt(rows)
+    X = torch.randn(K, rows, generator=g, device="cuda") / np.sqrt(rows) + torch.randn(K, cols, generator=g, device="cuda") @ W.t()
+    Wd, Xd, L = W.double(), X.double(), 1.1
+    c = torch.zeros(K, cols, dtype=torch.float64, device="cuda")
+    for _ in range(T):
+        a = c - (c @ Wd.t() - Xd) @ Wd / L
+        c = torch.sign(a) * (a.abs() - 0.1 / L).clamp_min(0)
+    ctx = S.Context(S.make_config(S.SC, rows, cols, 1, K, 1e-3, prec, sc_lambda=0.1, sc_ista_iters=T, sc_lipschitz=L), W)
+    ctx.sfb_compute_factors(-1, X)
+    V = ctx.factors_as_tensors()[1]
+    assert ctx.sfb_get_status() == 0
+    ctx.close()
+    assert float((V.double() - c).norm()) <= (1e-5 if prec == S.PREC_FP32 else 1e-4) * float(c.norm())
