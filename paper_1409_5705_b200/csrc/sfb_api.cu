@@ -954,6 +954,10 @@ extern "C" int sfb_get_operand_copy(sfb_ctx* ctx, const void** copy_dev, int32_t
 
 extern "C" int sfb_get_stats(sfb_ctx* ctx, sfb_stats* out) {
   if (!ctx || !out) return SFB_ERR_ARG;
+  const sfb_config& c = ctx->cfg;
+  // MLR in bf16 mode forms the mean loss with the label rows, in the update: asked for after the gather already, here
+  if (ctx->gathered && c.model == SFB_MLR && c.precision == SFB_PREC_BF16 && ctx->labels == sfb_ctx::kLabelsNone)
+    CK(mean_of(ctx->stream, ctx->at<float>(ctx->lay.loss), ctx->K, &ctx->at<Scalars>(ctx->lay.scalars)->loss_mean, Stamp{}));
   CK(cudaStreamSynchronize(ctx->stream));
   if (ctx->stats.steps > 0) {
     Scalars h{};

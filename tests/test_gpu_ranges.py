@@ -171,3 +171,27 @@ def test_sparse_coding_of_millions_of_features(prec):
     assert ctx.sfb_get_status() == 0
     ctx.close()
     assert float((V.double() - c).norm()) <= (1e-5 if prec == S.PREC_FP32 else 1e-4) * float(c.norm())
+
+
+# The loss of a step can be read after the gather, before the update.
+@pytest.mark.parametrize("prec", [pytest.param(S.PREC_FP32, id="fp32"), pytest.param(S.PREC_BF16, id="bf16")])
+def test_loss_after_the_gather(prec):
+    wl = I.scaled(I.WORKLOADS["mlr_mid"], "loss", rows=333, cols=260, workers=3, batch=37, eta=0.05, w_std=0.05, x_scale="unit")
+    W0 = I.initial_W(wl)
+    W = to_dev(W0, torch)
+    ctx = S.Context(config_for(wl, prec), W)
+    Wt = W0
+    for t in range(3):
+        inp = I.step_inputs(wl, t)
+        X, lab = to_dev(inp.X, torch), to_dev(inp.labels, torch)
+        for p in range(wl.workers):
+            r = slice(p * wl.batch, (p + 1) * wl.batch)
+            ctx.sfb_compute_factors(p, X[r], None, lab[r])
+        ctx.sfb_gather_factors()
+        if t:                                                    # (the read-outs begin with the first completed step)
+            assert abs(ctx.sfb_get_stats().last_loss - O.mlr_loss(Wt, inp.X, inp.labels).mean()) < 2e-3
+        ctx.sfb_apply_update()
+        Wt = W.cpu().numpy()
+        assert abs(ctx.sfb_get_stats().last_loss - O.mlr_loss(I.initial_W(wl) if t == 0 else Wprev, inp.X, inp.labels).mean()) < 2e-3
+        Wprev = Wt
+    ctx.close()
