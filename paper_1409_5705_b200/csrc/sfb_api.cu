@@ -194,6 +194,9 @@ extern "C" int sfb_init(const sfb_config* cfg, float* W_dev, void* workspace_dev
   ctx->tf32 = use_tf32(*cfg);
   ctx->h16 = use_h16(*cfg);
   if (cfg->precision != SFB_PREC_BF16) ctx->cfg.precision = SFB_PREC_FP32;      // one fp32 family; tf32, h16 say which kernels
+  ctx->sparse_fma = ctx->h16 && sparse_on_fma(*cfg);
+  ctx->fma_mask = 0;
+  ctx->update_fma = false;
   ctx->sdca = cfg->model == SFB_L2MLR;
   if (ctx->sdca) ctx->cfg.model = SFB_MLR;            // the products, buffers and the update are those of MLR
   ctx->dualQ = nullptr;
@@ -275,8 +278,8 @@ extern "C" int sfb_destroy(sfb_ctx* ctx) {
 // fp32-operand path
 // ---------------------------------------------------------------------------------------------------------
 // v = x (or x - y) of n pairs at offset off, and z = W v into U.
-static int logits_fp32(sfb_ctx* ctx, int64_t off, int64_t n, const float* X, const float* Y) {
-  if (ctx->h16) return split_logits(ctx, off, n, X, Y);
+static int logits_fp32(sfb_ctx* ctx, int64_t off, int64_t n, const float* X, const float* Y, bool pairs) {
+  if (pairs) return split_logits(ctx, off, n, X, Y);
   const sfb_config& c = ctx->cfg;
   float* V = ctx->at<float>(ctx->lay.V) + off * c.cols;
   CK(pack_copy(ctx->stream, V, X, Y, n * c.cols, take_stamp(ctx)));
@@ -288,7 +291,7 @@ static int logits_fp32(sfb_ctx* ctx, int64_t off, int64_t n, const float* X, con
 }
 
 static int factors_fp32(sfb_ctx* ctx, int64_t off, int64_t n, const float* X, const float* Y,
-                        const int32_t* labels, bool sparse_fwd = false, float* dml_norm_out = nullptr) {
+                        const int32_t* labels, bool pairs, bool sparse_fwd = false, float* dml_norm_out = nullptr) {
   const sfb_config& c = ctx->cfg;
   const int64_t rows = c.rows, cols = c.cols, ldu = ctx->lay.ldu, K = ctx->K;
   float* V = ctx->at<float>(ctx->lay.V) + off * cols;
@@ -303,7 +306,7 @@ static int factors_fp32(sfb_ctx* ctx, int64_t off, int64_t n, const float* X, co
       const int rc = sparse_forward(ctx, off, n, ctx->at<float>(ctx->lay.U), ldu);
       if (rc) return rc;
     } else {
-      const int rc = logits_fp32(ctx, off, n, X, c.model == SFB_DML ? Y : nullptr);
+      const int rc = logits_fp32(ctx, off, n, X, c.model == SFB_DML ? Y : nullptr, pairs);
       if (rc) return rc;
     }
     if (c.model == SFB_MLR)
@@ -370,7 +373,7 @@ static int begin_step(sfb_ctx* ctx) {
 static int update_fp32(sfb_ctx* ctx) {
   const sfb_config& c = ctx->cfg;
   if (ctx->sparse_v) return sparse_update(ctx);
-  if (ctx->h16) return tc_update(ctx);
+  if (ctx->h16 && !ctx->update_fma) return tc_update(ctx);
   EpiArgs e{};
   e.C = ctx->W; e.ldc = c.cols; e.alpha = -ctx->step;
   e.prox_kind = ctx->prox_kind; e.prox_a = ctx->prox_a;
@@ -400,7 +403,7 @@ static int compute_factors(sfb_ctx* ctx, int32_t worker, const float* X_dev, con
   const int64_t off = worker < 0 ? 0 : static_cast<int64_t>(worker) * c.batch;
   const int64_t n = worker < 0 ? ctx->K : c.batch;
   if (ctx->committed == 0) {
-    ctx->sparse_mask = 0;
+    ctx->sparse_mask = ctx->fma_mask = 0;
     ctx->csr_fill = 0;
     begin_phase(ctx, 0);
   }
@@ -412,12 +415,13 @@ static int compute_factors(sfb_ctx* ctx, int32_t worker, const float* X_dev, con
   // bf16 mode: every product runs on the tensor cores; DML and SC, whose u comes from a cancelling residual,
   // carry each value as a (hi, lo) pair of bf16 (fp32-class products)
   rc = ctx->tf32 ? tc32_factors(ctx, off, n, X_dev, labels_dev, nullptr, 0.f)
-       : c.precision == SFB_PREC_FP32 ? factors_fp32(ctx, off, n, X_dev, Y_dev, labels_dev)
+       : c.precision == SFB_PREC_FP32 ? factors_fp32(ctx, off, n, X_dev, Y_dev, labels_dev, ctx->h16)
                                       : tc_factors(ctx, off, n, X_dev, Y_dev, labels_dev, fused);
   if (rc) return rc;
   const uint64_t all = c.workers == 64 ? ~0ull : ((1ull << c.workers) - 1);
   ctx->committed |= worker < 0 ? all : (1ull << worker);
   ctx->sparse_mask &= ~(worker < 0 ? all : (1ull << worker));       // these samples are dense
+  ctx->fma_mask &= ~(worker < 0 ? all : (1ull << worker));
   ctx->gathered = false;
   return SFB_OK;
 }
@@ -442,7 +446,7 @@ static int compute_factors_csr(sfb_ctx* ctx, int32_t worker, const int64_t* indp
   const uint64_t all = c.workers == 64 ? ~0ull : ((1ull << c.workers) - 1);
   const uint64_t bits = worker < 0 ? all : (1ull << worker);
   if (ctx->committed == 0) {
-    ctx->sparse_mask = 0;
+    ctx->sparse_mask = ctx->fma_mask = 0;
     ctx->csr_fill = 0;
   }
   if (ctx->sparse_mask & bits) return SFB_ERR_STATE;                // its triples are already in the step's list
@@ -452,7 +456,8 @@ static int compute_factors_csr(sfb_ctx* ctx, int32_t worker, const int64_t* indp
   if (ctx->committed == 0) begin_phase(ctx, 0);
   if (starts_over(ctx, worker)) ctx->begun = false;
   int rc = SFB_OK;
-  if (!ctx->begun) {
+  const bool pairs = ctx->h16 && !ctx->sparse_fma;
+  if (!ctx->begun && (pairs || !ctx->h16)) {              // (on the FMA kernels these samples need no pairs of W)
     if ((rc = begin_step(ctx)) != SFB_OK) return rc;
     ctx->begun = true;
   }
@@ -460,11 +465,12 @@ static int compute_factors_csr(sfb_ctx* ctx, int32_t worker, const int64_t* indp
   if (rc) return rc;
   const float* X = ctx->at<float>(ctx->lay.stageX) + off * c.cols;
   rc = ctx->tf32 ? tc32_factors(ctx, off, n, X, labels_dev, nullptr, 0.f)
-       : c.precision == SFB_PREC_FP32 ? factors_fp32(ctx, off, n, X, nullptr, labels_dev, sparse_forward_wanted(ctx, n))
+       : c.precision == SFB_PREC_FP32 ? factors_fp32(ctx, off, n, X, nullptr, labels_dev, pairs, sparse_forward_wanted(ctx, n))
                                       : tc_factors(ctx, off, n, X, nullptr, labels_dev, fused);
   if (rc) return rc;
   ctx->csr_fill += nnz;
   ctx->sparse_mask |= bits;
+  if (ctx->sparse_fma) ctx->fma_mask |= bits;
   ctx->committed |= bits;
   ctx->gathered = false;
   return SFB_OK;
@@ -507,7 +513,7 @@ extern "C" int sfb_forward_partials(sfb_ctx* ctx, const float* X_dev, const int3
   if (!al16(partials_dev)) return SFB_ERR_ALIGN;
   const sfb_config& c = ctx->cfg;
   ctx->committed = 0;
-  ctx->sparse_mask = 0;
+  ctx->sparse_mask = ctx->fma_mask = 0;
   ctx->csr_fill = 0;
   ctx->gathered = false;
   begin_phase(ctx, 0);
@@ -518,7 +524,7 @@ extern "C" int sfb_forward_partials(sfb_ctx* ctx, const float* X_dev, const int3
   } else {
     const int64_t K = ctx->K, ldu = ctx->lay.ldu;
     float* U = ctx->at<float>(ctx->lay.U);
-    if ((rc = begin_step(ctx)) != SFB_OK || (rc = logits_fp32(ctx, 0, K, X_dev, nullptr)) != SFB_OK) return rc;    // z_i = W_shard x_i
+    if ((rc = begin_step(ctx)) != SFB_OK || (rc = logits_fp32(ctx, 0, K, X_dev, nullptr, ctx->h16)) != SFB_OK) return rc;    // z_i = W_shard x_i
     // the class ids are kept for the finish (the caller's buffer may change before it)
     CK(cudaMemcpyAsync(ctx->at<int32_t>(ctx->lay.stageL), labels_dev, static_cast<size_t>(K) * 4, cudaMemcpyDeviceToDevice,
                        ctx->stream));
@@ -538,7 +544,7 @@ extern "C" int sfb_forward_partials_pairs(sfb_ctx* ctx, const float* X_dev, cons
   if (!partials_dev) return SFB_ERR_ARG;
   const sfb_config& c = ctx->cfg;
   ctx->committed = 0;
-  ctx->sparse_mask = 0;
+  ctx->sparse_mask = ctx->fma_mask = 0;
   ctx->csr_fill = 0;
   ctx->gathered = false;
   begin_phase(ctx, 0);
@@ -546,7 +552,7 @@ extern "C" int sfb_forward_partials_pairs(sfb_ctx* ctx, const float* X_dev, cons
   CK(cudaMemcpyAsync(ctx->at<int32_t>(ctx->lay.stageL), similar_dev, static_cast<size_t>(ctx->K) * 4, cudaMemcpyDeviceToDevice,
                      ctx->stream));
   if ((rc = begin_step(ctx)) != SFB_OK) return rc;
-  rc = c.precision == SFB_PREC_FP32 ? factors_fp32(ctx, 0, ctx->K, X_dev, Y_dev, similar_dev, false, partials_dev)
+  rc = c.precision == SFB_PREC_FP32 ? factors_fp32(ctx, 0, ctx->K, X_dev, Y_dev, similar_dev, ctx->h16, false, partials_dev)
                                     : tc_factors(ctx, 0, ctx->K, X_dev, Y_dev, similar_dev, false, partials_dev);
   if (rc) return rc;
   ctx->partials_ready = true;
@@ -616,6 +622,7 @@ extern "C" int sfb_set_factors(sfb_ctx* ctx, int32_t worker, const float* U_dev,
   }
   ctx->committed |= 1ull << worker;
   ctx->sparse_mask &= ~(1ull << worker);             // received factors are dense
+  ctx->fma_mask &= ~(1ull << worker);
   ctx->gathered = false;
   return SFB_OK;
 }
@@ -658,6 +665,7 @@ extern "C" int sfb_gather_factors(sfb_ctx* ctx) {
   // Every worker wrote its pairs at row offset p*B of the shared buffers, so the gathered operands are
   // complete; what remains is the per-step read-out over all K pairs.
   // all K samples sparse: the v become their column-major form (and the dense update operands are not needed)
+  ctx->update_fma = ctx->fma_mask != 0;
   ctx->sparse_v = c.model == SFB_MLR && c.csr_nnz_max > 0 && ctx->sparse_mask == all && sparse_update_wanted(ctx);
   if (ctx->sparse_v) {
     CK(stamp(ctx->stream, take_stamp(ctx)));
@@ -667,7 +675,7 @@ extern "C" int sfb_gather_factors(sfb_ctx* ctx) {
     CK(stamp(ctx->stream, take_stamp(ctx)));
     int rc = tc32_gather(ctx);
     if (rc) return rc;
-  } else if (ctx->h16) {
+  } else if (ctx->h16 && !ctx->update_fma) {
     const int rc = split_gather(ctx);
     if (rc) return rc;
   }
@@ -707,7 +715,7 @@ extern "C" int sfb_apply_update(sfb_ctx* ctx) {
   if (rc) return rc;
   ctx->committed = 0;
   ctx->begun = false;
-  ctx->sparse_mask = 0;               // the next step starts with no sparse samples staged
+  ctx->sparse_mask = ctx->fma_mask = 0;               // the next step starts with no sparse samples staged
   ctx->csr_fill = 0;
   ctx->gathered = false;
   ctx->stats.steps += 1;
@@ -764,7 +772,7 @@ static int sdca_compute_factors(sfb_ctx* ctx, int32_t worker, const float* X_dev
       if (rc) return rc;
       ctx->begun = true;
     }
-    const int rc = logits_fp32(ctx, off, n, X_dev, nullptr);                                          // z_i = W a_i
+    const int rc = logits_fp32(ctx, off, n, X_dev, nullptr, ctx->h16);                                       // z_i = W a_i
     if (rc) return rc;
     SdcaArgs a = sdca_args(ctx, off, n, X_dev, labels_dev, sample_ids_dev, inv_lam_n);
     a.Z = U; a.ldz = ldu; a.out = U; a.ldo = ldu;                                                     // u_i = du_i

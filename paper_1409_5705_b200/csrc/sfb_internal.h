@@ -148,19 +148,20 @@ inline int64_t round_up(int64_t x, int64_t m) { return (x + m - 1) / m * m; }
 inline bool use_tf32(const sfb_config& c) {
   return c.precision == SFB_PREC_TF32X3 && (c.model == SFB_MLR || c.model == SFB_L2MLR);
 }
-bool sparse_on_fma(const sfb_config& c);      // sparse samples: see sfb_sparse.cu
 // Whether W and operands derived from it of `per_entry` bytes an entry leave room in the 180 GB of a GPU for samples and factors; the
 // FMA kernels need none (1,000,000 x 20,000: W 80 GB, its pairs as much again, those of W^T for sparse coding 80 more).
 inline bool derived_fit(const sfb_config& c, double per_entry) {
   return (4.0 + per_entry) * static_cast<double>(c.rows) * static_cast<double>(c.cols) <= 150e9;
 }
 inline bool use_h16(const sfb_config& c) {
-  if (c.precision != SFB_PREC_FP32 || c.rows < 64 || c.cols < 64 || sparse_on_fma(c)) return false;
+  if (c.precision != SFB_PREC_FP32 || c.rows < 64 || c.cols < 64) return false;
   if (!derived_fit(c, c.model == SFB_SC ? 8.0 : 4.0)) return false;
   const double K = static_cast<double>(c.workers) * c.batch, macs = K * static_cast<double>(c.rows) * static_cast<double>(c.cols);
   if (c.model == SFB_SC) return sc_on_pairs(c);
   return c.cols >= 256 && (macs >= 1e9 || macs * (1.0 - 24.0 / K) >= 1.8e8);
 }
+
+bool sparse_on_fma(const sfb_config& c);      // sparse samples of such a context: on the FMA kernels all the same (see sfb_sparse.cu)
 
 struct Scalars {                      // device-resident scalars
   float loss_mean;
@@ -199,6 +200,9 @@ struct sfb_ctx {
   int64_t global_rows;                //   of a matrix with global_rows rows (class ids are global); 0, rows when unsharded
   bool partials_ready;                // sfb_forward_partials has run since the last update
   bool tf32, h16;                     // fp32 modes with their products on the tensor cores (see use_tf32, use_h16)
+  bool sparse_fma;                    // h16, but sparse samples take the FMA kernels; bit p of fma_mask: worker p's of this step did
+  uint64_t fma_mask;
+  bool update_fma;                    // the gathered factors are not all there as pairs: the update takes the FMA kernels
   bool sdca;                          // SFB_L2MLR: the factors are dual changes; cfg.model is kept as SFB_MLR internally
   float* dualQ;                       // SDCA dual state [dual_n x rows], caller-owned
   int64_t dual_n;

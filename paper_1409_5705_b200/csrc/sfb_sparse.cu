@@ -559,7 +559,7 @@ bool sparse_update_wanted(const sfb_ctx* ctx) {
   const bool bf16 = c.precision == SFB_PREC_BF16;
   if (c.csr_update == 2 || slab_smem(ctx->K, bf16) < 0) return false;
   if (c.csr_update == 1) return true;
-  if (!bf16 && !ctx->tf32 && !ctx->h16) {
+  if (!bf16 && !ctx->tf32 && (!ctx->h16 || ctx->sparse_fma)) {
     // FMA kernels, in SM cycles: the column-major form takes 38,000 (five small launches), the dense update at least its pass over W
     // at 2.5 TB/s.  us per step, sparse / dense update: 1,000 x 1,000 K = 128 57 / 42, 91,238 x 148 K = 176 519 / 441, 20,000 x 4,000
     // K = 16 371 / 458, 10,000 x 20,000 K = 128 874 / 1531.
@@ -637,7 +637,7 @@ static double row_wise_cycles(const sfb_config& c, int rb) {
 // Whether the row-wise forward is faster than the FMA product.
 bool sparse_forward_wanted(const sfb_ctx* ctx, int64_t n) {
   const int rb = sparse_forward_rows(ctx->cfg, n);
-  return rb > 0 && !ctx->h16 && row_wise_cycles(ctx->cfg, rb) < gemm_cycles(ctx->K, ctx->cfg.rows, ctx->cfg.cols);
+  return rb > 0 && (!ctx->h16 || ctx->sparse_fma) && row_wise_cycles(ctx->cfg, rb) < gemm_cycles(ctx->K, ctx->cfg.rows, ctx->cfg.cols);
 }
 // Whether sparse samples in fp32 mode are better off on the FMA kernels and the sparse update than on pairs of fp16 words (the
 // packing of W at 4.5 TB/s, the dense product, the cheaper update; in units of 2.6 ps per entry of W as below).  us per step, FMA / pairs:

@@ -195,3 +195,52 @@ def test_loss_after_the_gather(prec):
         assert abs(ctx.sfb_get_stats().last_loss - O.mlr_loss(I.initial_W(wl) if t == 0 else Wprev, inp.X, inp.labels).mean()) < 2e-3
         Wprev = Wt
     ctx.close()
+
+
+# A context with room for sparse samples whose products of dense samples belong on the tensor cores and those of sparse ones on the FMA
+# kernels: dense, sparse and mixed steps in turn on one context, factors received and an update replayed between them.
+def test_dense_and_sparse_steps_on_one_fp32_context():
+    rows, cols, P, B = 2000, 4000, 4, 32
+    wl = I.scaled(I.WORKLOADS["mlr_mid"], "mixed", rows=rows, cols=cols, workers=P, batch=B, eta=0.05, w_std=0.01, x_scale="inv_sqrt_d")
+    W0 = I.initial_W(wl)
+    W = to_dev(W0, torch)
+    ctx = S.Context(S.make_config(S.MLR, rows, cols, P, B, wl.eta, S.PREC_FP32, csr_nnz_max=8 * wl.K * 2), W)
+    Wt, flops = W0, []
+    for t, form in enumerate(["dense", "sparse", "dense", "mixed", "sparse", "received", "mixed", "dense"]):
+        inp = I.step_inputs(wl, t)
+        sp = I.sparse_samples(wl.seed, t, wl.K, cols, 8.0)
+        X, lab = inp.X.copy(), inp.labels
+        ld = to_dev(lab, torch)
+        before = ctx.sfb_get_stats().flops
+        if form == "dense":
+            ctx.sfb_step(to_dev(X, torch), None, ld)
+        elif form == "sparse":
+            X = I.densify(sp, cols)
+            ctx.sfb_step_csr(to_dev(sp.indptr, torch), to_dev(sp.indices, torch), to_dev(sp.values, torch), sp.nnz, ld)
+        else:
+            for p in range(P):
+                r = slice(p * B, (p + 1) * B)
+                if p % 2 == 0:
+                    X[r] = I.densify(sp, cols)[r]
+                    ip = sp.indptr[p * B:(p + 1) * B + 1]
+                    lo, hi = int(ip[0]), int(ip[-1])
+                    ctx.sfb_compute_factors_csr(p, to_dev(ip - lo, torch), to_dev(sp.indices[lo:hi], torch), to_dev(sp.values[lo:hi], torch), hi - lo, ld[r])
+                else:
+                    ctx.sfb_compute_factors(p, to_dev(X[r], torch), None, ld[r])
+                if form == "received" and p != 1:
+                    U, V = torch.empty(B, rows, device="cuda"), torch.empty(B, cols, device="cuda")
+                    ctx.sfb_export_factors(p, U, V)
+                    ctx.sfb_set_factors(p, U, V)
+            ctx.sfb_gather_factors()
+            ctx.sfb_apply_update()
+        assert ctx.sfb_get_status() == 0
+        flops.append(ctx.sfb_get_stats().flops - before)
+        Wg, ref = W.cpu().numpy(), O.sfb_step(wl.model, Wt, X, None, lab, workers=P, eta=wl.eta)
+        assert rel_err(Wg, ref, Wt) <= 1e-5, form
+        if t == 3 or t == 5:
+            ctx.sfb_replay_update()
+            assert rel_err(W.cpu().numpy(), Wg.astype(np.float64) + (ref - Wt), Wt) <= 2e-5, form
+            Wg = W.cpu().numpy()
+        Wt = Wg
+    ctx.close()
+    assert flops[0] >= 7.5 * wl.K * rows * cols                   # three products a term in the logits of dense samples
