@@ -171,7 +171,7 @@ int sfb_compute_factors(sfb_ctx* ctx, int32_t worker, const float* X_dev, const 
  * then counts K*rows*element size for the u and 8 bytes per non-zero for the v.  A mini-batch too large for the
  * kernel's on-chip factor slab (K above about 1200 in the fp32 modes, 2400 in bf16 mode) takes the dense update, and
  * so does, unless cfg.csr_update says otherwise, one whose columns hold so many non-zeros that the tensor-core update
- * over the scattered samples is the faster of the two (in bf16 mode always up to K = 1024; in the fp32 modes from about
+ * over the scattered samples is the faster of the two (in bf16 mode always up to K = 1024 and 200,000 rows; in the fp32 modes from about
  * 30 non-zeros per column with tf32 pairs, fewer with fp16 pairs). */
 int sfb_compute_factors_csr(sfb_ctx* ctx, int32_t worker, const int64_t* indptr_dev, const int32_t* indices_dev,
                             const float* values_dev, int64_t nnz, const int32_t* labels_dev);

@@ -550,8 +550,9 @@ void sparse_extend_layout(const sfb_config& c, Layout& L, size_t& off) {
 }
 
 // Cost model, in time per entry of W relative to the dense update of K = 1024 pairs in bf16 (325,000 x 10,000: 8.5 ms): the
-// sparse update costs a fixed 1.0 for its pass over W in bf16 mode (0.83 where the operand copy hardly changes, 1.4 at
-// 10,000 x 20,000 where all of it does, and the column-major form of the samples comes on top) and 1.57 in the tensor-core
+// sparse update costs a fixed 1.0 for its pass over W in bf16 mode and 0.9 from 200,000 rows on, where the probabilities are small
+// and less than a tenth of the operand copy changes (ms a step of K = 1024 with 10 non-zeros, sparse / dense: 325,000 x 10,000 12.9 /
+// 12.9, 200,000 x 20,000 14.4 / 15.2, 100,000 x 10,000 4.15 / 3.87, 10,000 x 20,000 1.19 / 1.00), and 1.57 in the tensor-core
 // fp32 mode, whose 8-byte operand copy it also writes, plus 0.089 per non-zero of an average column; the dense update costs
 // K/1024 in bf16 mode, 4.4 K/1024 with tf32 pairs, 2.2 K/1024 with fp16 pairs, and far more on the FMA kernels.
 bool sparse_update_wanted(const sfb_ctx* ctx) {
@@ -570,7 +571,7 @@ bool sparse_update_wanted(const sfb_ctx* ctx) {
   }
   const double per_col = static_cast<double>(ctx->csr_fill) / static_cast<double>(c.cols);
   const double k = static_cast<double>(ctx->K) / 1024.0;
-  const double sparse = (ctx->tf32 ? 1.57 : 1.0) + 0.089 * per_col;
+  const double sparse = (ctx->tf32 ? 1.57 : bf16 && c.rows >= 200000 ? 0.9 : 1.0) + 0.089 * per_col;
   return sparse < (bf16 ? 1.0 : ctx->tf32 ? 4.4 : 2.2) * k;
 }
 

@@ -244,3 +244,16 @@ def test_dense_and_sparse_steps_on_one_fp32_context():
         Wt = Wg
     ctx.close()
     assert flops[0] >= 7.5 * wl.K * rows * cols                   # three products a term in the logits of dense samples
+
+
+# Which update a step of sparse samples takes in bf16 mode: from 200,000 rows on the sparse one again, below one non-zero per column.
+@pytest.mark.parametrize("rows,sparse", [(200_000, True), (199_999, False)])
+def test_choice_of_the_update_by_rows(rows, sparse):
+    cols, K = 2048, 1024
+    sp = I.sparse_samples(3, 0, K, cols, 0.4)                     # one entry a sample
+    lab = np.arange(K, dtype=np.int32)
+    W = torch.zeros((rows, cols), device="cuda")
+    ctx = S.Context(S.make_config(S.MLR, rows, cols, 16, 64, 0.05, S.PREC_BF16, csr_nnz_max=sp.nnz), W)
+    ctx.sfb_step_csr(to_dev(sp.indptr, torch), to_dev(sp.indices, torch), to_dev(sp.values, torch), sp.nnz, to_dev(lab, torch))
+    assert ctx.sfb_get_status() == 0 and ctx.sfb_get_stats().sparse_updates == int(sparse)
+    ctx.close()
