@@ -51,7 +51,7 @@ def check(wl, prec, per_worker=False, scale=1.0, L=None):
 
 
 # Ragged tiles of 256 x bn; the two forms of the update (384 and 385 pairs); rows of 2048 and 2052 columns (one warp or a block with
-# bulk copies per row) and of 26,628 (registers, the rest from memory); several tiles per pair of CTAs.
+# bulk copies per row) and of 26,628 (registers, the rest from memory); an update of several tiles per pair of CTAs.
 @pytest.mark.parametrize("shape", [(701, 1028, 3, 101), (530, 1000, 1, 384), (530, 1000, 5, 77), (640, 2048, 2, 90), (641, 2052, 2, 90),
                                    (65, 26628, 2, 70), (9001, 256, 1, 257)])
 def test_regression_in_fp32(shape):
@@ -71,6 +71,17 @@ def test_metric_learning(shape, prec):
                                          ((257, 1092, 5, 211), 1), ((257, 1092, 5, 211), 0)])
 def test_sparse_coding(shape, iters, prec):
     check(workload("sc", *shape, sc_iters=iters), prec)
+
+
+# Products of more tiles than pairs of CTAs (74): at 256 columns, the widest, already ceil(K / 256) x ceil(columns / 256) of them, with the
+# logits, the residual, both forms of an iteration and the first iterate.  (The coder on W^T W: bf16 mode, no more atoms than features.)
+@pytest.mark.parametrize("name,shape,prec,kw", [("mlr", (5200, 516, 2, 512), S.PREC_FP32, {}), ("dml", (5200, 516, 2, 512), S.PREC_BF16, {}),
+                                                ("sc", (2700, 2600, 8, 232), S.PREC_BF16, {"sc_iters": 4}),
+                                                ("sc", (2564, 2700, 8, 232), S.PREC_BF16, {"sc_iters": 3}),
+                                                ("sc", (2564, 2600, 8, 232), S.PREC_FP32, {"sc_iters": 3})])
+def test_several_tiles_per_pair(name, shape, prec, kw):
+    assert -(-shape[2] * shape[3] // 256) * -(-min(shape[:2] if name == "sc" else shape[:1]) // 256) > 74
+    check(workload(name, *shape, **kw), prec, scale=0.06 if name == "dml" else 1.0)
 
 
 @pytest.mark.parametrize("name,shape", [("mlr", (701, 1028, 3, 101)), ("dml", (711, 1020, 6, 57)), ("sc", (700, 400, 3, 341))])
