@@ -61,7 +61,7 @@ __device__ __forceinline__ float block_max(float v, float* sh) {
 __global__ void pack_kernel(float* __restrict__ dst, const float* __restrict__ x, const float* __restrict__ y,
                             int64_t n4, int64_t n, const Stamp st) {
   pdl_launch_dependents();
-  pdl_wait();
+  pdl_wait(dst, x, y);
   stamp_begin(st);
   const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
   for (int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; i < n4; i += stride) {
@@ -78,14 +78,14 @@ __global__ void pack_kernel(float* __restrict__ dst, const float* __restrict__ x
 
 __global__ void zero_kernel(float* __restrict__ dst, int64_t n) {
   pdl_launch_dependents();
-  pdl_wait();
+  pdl_wait(dst);
   const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
   for (int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; i < n; i += stride) dst[i] = 0.f;
 }
 
 __global__ void prox_entries_kernel(float* __restrict__ w, int64_t n, int kind, float a) {
   pdl_launch_dependents();
-  pdl_wait();
+  pdl_wait(w);
   const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
   for (int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; i < n; i += stride)
     w[i] = prox_entry(w[i], kind, a);
@@ -93,7 +93,7 @@ __global__ void prox_entries_kernel(float* __restrict__ w, int64_t n, int kind, 
 
 __global__ void axpy_kernel(float* __restrict__ y, const float* __restrict__ x, float alpha, int64_t n) {
   pdl_launch_dependents();
-  pdl_wait();
+  pdl_wait(y, x);
   const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
   for (int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; i < n; i += stride)
     y[i] = fmaf(alpha, x[i], y[i]);
@@ -107,7 +107,7 @@ __global__ void __launch_bounds__(NTHREADS) mlr_softmax_kernel(float* __restrict
                                                                const int32_t* __restrict__ labels,
                                                                float* __restrict__ loss, uint32_t* status) {
   pdl_launch_dependents();
-  pdl_wait(labels);
+  pdl_wait(Z, labels, loss);
   __shared__ float sh[32];
   float* z = Z + static_cast<int64_t>(blockIdx.x) * ldz;
   float m = -INFINITY;
@@ -141,7 +141,7 @@ __global__ void __launch_bounds__(NTHREADS) mlr_shard_partials_kernel(const floa
                                                                       const int32_t* __restrict__ labels, int64_t row_off,
                                                                       float4* __restrict__ part) {
   pdl_launch_dependents();
-  pdl_wait(labels);
+  pdl_wait(Z, labels, part);
   __shared__ float sh[32];
   const float* z = Z + static_cast<int64_t>(blockIdx.x) * ldz;
   float m = -INFINITY;
@@ -183,7 +183,7 @@ __global__ void __launch_bounds__(NTHREADS) mlr_shard_finish_kernel(float* __res
                                                                     const float4* __restrict__ parts, int shards, int64_t K,
                                                                     float* __restrict__ loss, uint32_t* status) {
   pdl_launch_dependents();
-  pdl_wait(labels, parts);
+  pdl_wait(Z, labels, parts, loss);
   __shared__ float sh_lse;
   float* z = Z + static_cast<int64_t>(blockIdx.x) * ldz;
   if (threadIdx.x == 0) {
@@ -375,7 +375,7 @@ __global__ void __launch_bounds__(NTHREADS) dml_scale_kernel(float* __restrict__
                                                              int64_t split_half, const float* __restrict__ inv_v,
                                                              float* __restrict__ most) {
   pdl_launch_dependents();
-  pdl_wait(similar, norms_all, inv_v);
+  pdl_wait(Z, similar, norm_out, norms_all, split, inv_v, most);
   __shared__ float sh[32];
   float* z = Z + static_cast<int64_t>(blockIdx.x) * ld;
   float q = 0.f;
@@ -410,7 +410,7 @@ __global__ void __launch_bounds__(NTHREADS) dml_scale_kernel(float* __restrict__
 
 __global__ void mean_kernel(const float* __restrict__ v, int64_t n, float* out, const Stamp st) {
   pdl_launch_dependents();
-  pdl_wait();
+  pdl_wait(v);
   stamp_begin(st);
   __shared__ float sh[32];
   float s = 0.f;
@@ -424,7 +424,7 @@ __global__ void mean_kernel(const float* __restrict__ v, int64_t n, float* out, 
 __global__ void __launch_bounds__(kThreads) col_sumsq_kernel(const float* __restrict__ W, int64_t rows, int64_t cols,
                                                              double* __restrict__ part, int64_t slab_rows) {
   pdl_launch_dependents();
-  pdl_wait();
+  pdl_wait(W, part);
   __shared__ double sh[8][128];
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
   const int64_t c0 = static_cast<int64_t>(blockIdx.x) * 128 + tx * 4;
@@ -458,7 +458,7 @@ __global__ void __launch_bounds__(kThreads) prox_scale_kernel(float* __restrict_
                                                               const double* __restrict__ part, int nslabs,
                                                               int64_t slab_rows, unsigned long long* end) {
   pdl_launch_dependents();
-  pdl_wait(part);
+  pdl_wait(W, part);
   __shared__ double scale[128];
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
   if (threadIdx.x < 128) {

@@ -33,14 +33,14 @@ struct Stamp {                        // the first block stores the time to at[0
 };
 #ifdef __CUDACC__
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-// ... with the kernel's `const __restrict__` parameters: the compiler may read through those at any time, before the wait too
-// (a scalar was), unless it cannot tell where they point until after it.
-template <typename T>
-__device__ __forceinline__ void pdl_hide(T& p) { asm volatile("" : "+l"(p) :: "memory"); }
+// ... with all of the kernel's `__restrict__` parameters: nothing the wait may touch can alias those, so the compiler may move their
+// loads and stores above it (a load of a scalar was), unless their addresses come from something that it learns after the wait.
 template <typename... P>
 __device__ __forceinline__ void pdl_wait(P&... p) {
   pdl_wait();
-  (pdl_hide(p), ...);
+  int64_t zero = 0;
+  asm volatile("" : "+l"(zero) :: "memory");
+  ((p += zero), ...);
 }
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 

@@ -72,7 +72,7 @@ __global__ void __launch_bounds__(256) csr_stage_kernel(const int64_t* __restric
                                                         int32_t* __restrict__ row_beg,
                                                         int32_t* __restrict__ row_end, uint32_t* __restrict__ status) {
   pdl_launch_dependents();
-  pdl_wait();
+  pdl_wait(indptr, idx, val, Xd, coo_i, coo_c, coo_x, coo_cx, row_beg, row_end, status);
   const int64_t i = (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (i >= n) return;
@@ -113,7 +113,7 @@ __global__ void __launch_bounds__(256) csr_stage_kernel(const int64_t* __restric
 // ---------------------------------------------------------------------------------------------------------
 __global__ void __launch_bounds__(256) csc_count_kernel(const int32_t* __restrict__ coo_c, int64_t nnz, int32_t* __restrict__ cnt) {
   pdl_launch_dependents();
-  pdl_wait();
+  pdl_wait(coo_c, cnt);
   const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
   for (int64_t t = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; t < nnz; t += stride) {
     const int32_t c = coo_c[t];
@@ -123,7 +123,7 @@ __global__ void __launch_bounds__(256) csc_count_kernel(const int32_t* __restric
 
 __global__ void __launch_bounds__(1024) csc_scan_kernel(const int32_t* __restrict__ cnt, int64_t cols, int32_t* __restrict__ ptr) {
   pdl_launch_dependents();
-  pdl_wait(cnt);
+  pdl_wait(cnt, ptr);
   __shared__ int32_t part[1024];
   const int t = threadIdx.x;
   const int64_t chunk = (cols + 1023) / 1024;
@@ -151,7 +151,7 @@ __global__ void __launch_bounds__(256) csc_fill_kernel(const int32_t* __restrict
                                                        const int32_t* __restrict__ ptr, int32_t* __restrict__ cur,
                                                        int2* __restrict__ tmp) {
   pdl_launch_dependents();
-  pdl_wait(ptr);
+  pdl_wait(coo_i, coo_c, coo_x, ptr, cur, tmp);
   const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
   for (int64_t t = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; t < nnz; t += stride) {
     const int32_t c = coo_c[t];
@@ -166,7 +166,7 @@ __global__ void __launch_bounds__(128) csc_sort_kernel(const int2* __restrict__ 
                                                        const int32_t* __restrict__ cnt, int64_t cols, int32_t K,
                                                        int2* __restrict__ ent) {
   pdl_launch_dependents();
-  pdl_wait(ptr, cnt);
+  pdl_wait(tmp, ptr, cnt, ent);
   for (int64_t d = blockIdx.x; d < cols; d += gridDim.x) {
     const int32_t n = cnt[d], b = ptr[d];
     for (int32_t e = threadIdx.x; e < n; e += blockDim.x) {
@@ -226,7 +226,7 @@ __global__ void __launch_bounds__(kSfThreads, 1) sparse_forward_kernel(const flo
                                                                        const int2* __restrict__ cx, int64_t off, int32_t n,
                                                                        float* __restrict__ Z, int64_t ldz) {
   pdl_launch_dependents();
-  pdl_wait();
+  pdl_wait(W, row_beg, row_end, cx, Z);
   extern __shared__ __align__(16) uint8_t sf_smem[];
   constexpr int EP = 32 / RB;                        // entries of a sample worked on at once
   float* ws = reinterpret_cast<float*>(sf_smem);     // RB rows of W, row pitch `pitch` floats

@@ -652,7 +652,7 @@ template <bool F16>
 __global__ void __launch_bounds__(256) pack_t_kernel(const float* __restrict__ F, int64_t n, int64_t dim, int64_t ld,
                                                      uint16_t* __restrict__ FT, int64_t Kp, const float* __restrict__ inv) {
   pdl_launch_dependents();
-  pdl_wait(inv);
+  pdl_wait(F, FT, inv);
   __shared__ float tile[64][65];
   const int64_t cblocks = (dim + 63) / 64, i0 = blockIdx.x / cblocks * 64, c0 = blockIdx.x % cblocks * 64;
   const int t = threadIdx.x;
@@ -688,7 +688,7 @@ __global__ void __launch_bounds__(256) pack_rows_kernel(const float* __restrict_
                                                         int64_t ld, float* __restrict__ V, uint16_t* __restrict__ dst, int64_t dimp,
                                                         const Stamp stamp) {
   pdl_launch_dependents();
-  pdl_wait();
+  pdl_wait(F, Y, V, dst);
   stamp_begin(stamp);
   const int64_t r = static_cast<int64_t>(blockIdx.x) * (256 / TPR) + threadIdx.x / TPR;
   const int t = threadIdx.x % TPR, quads = dim / 4;
@@ -942,7 +942,7 @@ __global__ void __launch_bounds__(1024) sc_scales_kernel(const float* __restrict
 __global__ void __launch_bounds__(256) row_most_kernel(const float* __restrict__ U, int64_t ldu, int64_t rows,
                                                        const float* __restrict__ inv, float* __restrict__ q) {
   pdl_launch_dependents();
-  pdl_wait(inv);
+  pdl_wait(U, inv, q);
   __shared__ float sh[8];
   const float* u = U + static_cast<int64_t>(blockIdx.x) * ldu;
   float m = 0.f;
@@ -964,7 +964,7 @@ __global__ void __launch_bounds__(256) pack_u_kernel(const float* __restrict__ U
                                                      const float* __restrict__ q, const float* __restrict__ inv_v,
                                                      uint16_t* __restrict__ dst, int64_t rowsp, Scalars* sc, const Stamp stamp) {
   pdl_launch_dependents();
-  pdl_wait(q, inv_v);
+  pdl_wait(U, q, inv_v, dst);
   stamp_begin(stamp);
   __shared__ float sh[8];
   float m = 0.f;

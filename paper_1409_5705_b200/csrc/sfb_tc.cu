@@ -275,7 +275,7 @@ __device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
 __global__ void __launch_bounds__(256) convert_rows_kernel(const float* __restrict__ src, int64_t rows, int64_t cols,
                                                            __nv_bfloat16* __restrict__ dst, int64_t ld) {
   pdl_launch_dependents();
-  pdl_wait();
+  pdl_wait(src, dst);
   const int64_t quads = cols / 4;
   const int64_t total = rows * quads;
   const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
@@ -298,7 +298,7 @@ __global__ void __launch_bounds__(256) pack_mlr_kernel(const float* __restrict__
                                                        float* __restrict__ Xf, const int32_t* labels, int32_t* labels_out,
                                                        int32_t* __restrict__ slot, int64_t rows, const Stamp stamp) {
   pdl_launch_dependents();
-  pdl_wait();
+  pdl_wait(X, Xb, Xf, slot);
   stamp_begin(stamp);
   const uint32_t quads = static_cast<uint32_t>(cols / 4);
   const int64_t total = n * quads, stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
@@ -336,7 +336,7 @@ __global__ void __launch_bounds__(256) mlr_lse_kernel(const float2* __restrict__
                                                       float* __restrict__ coef, int32_t* __restrict__ slot,
                                                       uint32_t* status) {
   pdl_launch_dependents();
-  pdl_wait(part, labels);
+  pdl_wait(part, Z, labels, lse, loss, coef, slot);
   const int64_t i = static_cast<int64_t>(blockIdx.x) * 8 + (threadIdx.x >> 5);
   if (i >= n) return;
   const int lane = threadIdx.x & 31;
@@ -507,7 +507,7 @@ __global__ void __launch_bounds__(256) label_delta_kernel(const LabelArgs a) {
 __global__ void __launch_bounds__(256) label_slots_kernel(const int32_t* __restrict__ labels, int32_t K, int64_t rows,
                                                           int32_t* __restrict__ slot, const Stamp stamp) {
   pdl_launch_dependents();
-  pdl_wait(labels);
+  pdl_wait(labels, slot);
   stamp_begin(stamp);
   const int i = blockIdx.x * 256 + threadIdx.x;
   if (i >= K) return;
@@ -523,7 +523,7 @@ __global__ void __launch_bounds__(256) mlr_shard_partials_tc_kernel(const float2
                                                                     const int32_t* __restrict__ labels, int64_t row_off,
                                                                     int64_t n, float4* __restrict__ out) {
   pdl_launch_dependents();
-  pdl_wait(part, labels);
+  pdl_wait(part, Z, labels, out);
   const int64_t i = static_cast<int64_t>(blockIdx.x) * 8 + (threadIdx.x >> 5);
   if (i >= n) return;
   const int lane = threadIdx.x & 31;
@@ -552,7 +552,7 @@ __global__ void __launch_bounds__(256) mlr_shard_finish_tc_kernel(const float4* 
                                                                   float* __restrict__ lse, float* __restrict__ loss,
                                                                   float* __restrict__ coef, uint32_t* status) {
   pdl_launch_dependents();
-  pdl_wait(parts);
+  pdl_wait(parts, labels, lse, loss, coef);
   const int64_t i = static_cast<int64_t>(blockIdx.x) * 256 + threadIdx.x;
   if (i >= n) return;
   float M = -INFINITY;
@@ -588,7 +588,7 @@ __global__ void __launch_bounds__(256) mlr_emit_p_kernel(const float* __restrict
                                                          const int32_t* __restrict__ labels, __nv_bfloat16* __restrict__ P,
                                                          int64_t ldp, int lab_blocks, const LabelArgs lab) {
   pdl_launch_dependents();
-  pdl_wait(lse, labels);
+  pdl_wait(Z, lse, labels, P);
   if (static_cast<int>(blockIdx.x) < lab_blocks) return label_delta(lab, blockIdx.x, lab_blocks);
   const uint32_t octs = static_cast<uint32_t>((rows + 7) / 8);
   const int64_t total = n * octs, stride = static_cast<int64_t>(gridDim.x - lab_blocks) * blockDim.x;
@@ -614,7 +614,7 @@ __global__ void __launch_bounds__(256) mlr_lse_emit_kernel(const float2* __restr
                                                            float* __restrict__ loss, float* __restrict__ coef,
                                                            __nv_bfloat16* __restrict__ P, int64_t ldp, uint32_t* status) {
   pdl_launch_dependents();
-  pdl_wait(part, labels);
+  pdl_wait(part, Z, labels, lse, loss, coef, P);
   __shared__ float sh[16];
   const int t = threadIdx.x;
   const int64_t i = blockIdx.y, s = off + i;
@@ -674,7 +674,7 @@ __device__ __forceinline__ float to_tf32(float x) {
 __global__ void __launch_bounds__(256) split32_rows_kernel(const float* __restrict__ F, int64_t n, int64_t dim, int64_t ld,
                                                            float* __restrict__ dst, int64_t dimp) {
   pdl_launch_dependents();
-  pdl_wait();
+  pdl_wait(F, dst);
   const int64_t quads = dim / 4, total = n * quads;
   const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
   for (int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; i < total; i += stride) {
@@ -693,7 +693,7 @@ __global__ void __launch_bounds__(256) split32_rows_kernel(const float* __restri
 __global__ void __launch_bounds__(256) split32_t_kernel(const float* __restrict__ F, int64_t n, int64_t dim, int64_t ld,
                                                         float* __restrict__ FT, int64_t Kp) {
   pdl_launch_dependents();
-  pdl_wait();
+  pdl_wait(F, FT);
   __shared__ float tile[64][65];
   const int64_t i0 = static_cast<int64_t>(blockIdx.y) * 64, c0 = static_cast<int64_t>(blockIdx.x) * 64;
   const int t = threadIdx.x;
@@ -724,7 +724,7 @@ __global__ void __launch_bounds__(256) mlr_finish_u_kernel(const float* __restri
                                                            const int32_t* __restrict__ labels,
                                                            float* __restrict__ U) {
   pdl_launch_dependents();
-  pdl_wait(lse, labels);
+  pdl_wait(Z, lse, labels, U);
   const int64_t i = blockIdx.y;
   const float l = lse[i];
   const int64_t y = labels[i];
@@ -1129,7 +1129,7 @@ __global__ void __launch_bounds__(256) mlr_export_u_kernel(const float* __restri
                                                            const int32_t* __restrict__ labels,
                                                            int64_t off, float* __restrict__ U_out) {
   pdl_launch_dependents();
-  pdl_wait(lse, labels);
+  pdl_wait(Z, lse, labels, U_out);
   const int64_t i = blockIdx.y;
   const float l = lse[off + i];
   const int32_t y = labels[off + i];
@@ -1147,7 +1147,7 @@ __global__ void __launch_bounds__(256) mlr_import_labels_kernel(const float* __r
                                                                 int32_t* __restrict__ labels, float* __restrict__ coef,
                                                                 float* __restrict__ loss, int32_t* __restrict__ slot) {
   pdl_launch_dependents();
-  pdl_wait();
+  pdl_wait(U_in, labels, coef, loss, slot);
   __shared__ float sv[256];
   __shared__ int32_t si[256];
   const int64_t i = blockIdx.x;

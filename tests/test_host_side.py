@@ -120,3 +120,20 @@ def test_host_step_returns_no_buffer_that_is_still_read(tmp_path):
                            "-o", str(exe), "-Wl,--unresolved-symbols=ignore-all"])
     out = subprocess.run([str(exe)], capture_output=True, text=True)
     assert out.returncode == 0, out.stdout + out.stderr
+
+
+def test_kernels_read_nothing_before_their_wait():
+    """A kernel launched ahead of the one before it waits for that one.  Its `__restrict__` parameters all go through the wait: the compiler
+    may move accesses through the others above it."""
+    import glob
+    import re
+    seen = 0
+    for path in glob.glob(os.path.join(ROOT, "paper_1409_5705_b200", "csrc", "*.cu")):
+        src = open(path).read()
+        for m in re.finditer(r"__global__[^;{]*?\(((?:[^(){}]|\([^()]*\))*)\)\s*\{", src):
+            names = re.findall(r"__restrict__\s+(\w+)", m.group(0))
+            if names:
+                wait = re.search(r"pdl_wait\(([^)]*)\);", src[m.end():])
+                assert wait and sorted(names) == sorted(wait.group(1).replace(" ", "").split(",")), (os.path.basename(path), m.group(0)[:120])
+                seen += 1
+    assert seen >= 30
