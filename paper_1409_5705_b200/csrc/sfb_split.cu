@@ -46,7 +46,7 @@ struct SplitParams {
   int32_t a_rows;              // rows of A per box (fewer than 128 for a slice of few samples)
   int32_t stages, kseg;        // operand ring; k-blocks
   int32_t a_lo, b_lo;          // first column of the lo halves
-  int32_t whole;               // tiles [0, whole) are taken whole, pair by pair; the k-blocks of the others are shared out
+  int32_t cut;                 // the k-blocks are shared out; else the tiles are taken whole, pair by pair
   float* partial;              // [pairs][2][kEpi][4][8][32] float4: sums of the tile that a pair leaves to another one ...
   uint32_t* ready;             // [pairs][2][kEpi]: ... and that they are there
   int32_t four;                // F_GRAM: with the fourth term A_lo B_lo
@@ -122,14 +122,14 @@ __device__ __forceinline__ float4 scale4(float4 v, float s) { return make_float4
 // The tensor core rounds an fp32 accumulator towards zero at every instruction, so the error grows with the instructions that
 // add to one.  Hence the cross terms have an accumulator of their own (2^-8 or 2^-11 of the size), and A_hi B_hi is drained
 // every eight k-blocks, while the A_lo B_hi of the last of them run: the epilogue warps add it to sums in their registers.
-// The tiles that do not fill a last round of the SMs are cut along the contraction: their k-blocks are shared out evenly, a pair
+// A product of fewer tiles than pairs is cut along the contraction: its k-blocks are shared out evenly, a pair
 // has a run of them that begins within one tile and ends within another (or the same).  The part at the end of a run, which
 // does not reach the end of its tile, is computed first and left in memory; the part at the beginning, which completes a tile,
 // last: the parts that it waits for come from the pairs before this one.  The sums are in the order of the pairs, so they do
 // not depend on timing.
 // Warps: 0 TMA producer, 1 MMA issuer (leader CTA) and TMEM owner, 4..11 epilogue; the first four give their registers to
 // the epilogue (384 threads x 168 = 128 x 40 + 256 x 232).
-// Rates: see pair_cost.
+// Rates: see plan_width.
 // ---------------------------------------------------------------------------------------------------------
 constexpr int PM = 256, BM = 128, BK = 64, UMMA_K = 16;
 constexpr int kMaxN = 256;
@@ -177,39 +177,36 @@ __device__ __forceinline__ void tile_coords(const SplitParams& p, int tile, int&
   n0 = tn * p.bn;
 }
 
-// What a pair computes, in its order: the part of a tile that another pair completes, its whole tiles, the tiles that it
+// What a pair computes, in its order: whole tiles, or the part of a tile that another pair completes and then the tiles that it
 // completes (the one it completes for others last).  k-blocks [k0, k1) of each.
 struct Segment { int tile, k0, k1; };
 struct Segments {
-  int pair, pairs, whole, kseg, nwhole, t0, nt, n;
-  int64_t units, beg, end;             // of the k-blocks of the tiles whole, whole + 1, ...
-  bool leaves;
+  int pair, pairs, kseg, t0, n;
+  int64_t units, beg, end;             // k-blocks of all tiles; of this pair (none: whole tiles)
+  bool cut, leaves;
   __device__ Segments(const SplitParams& p, int ntiles, int pair_, int pairs_)
-      : pair(pair_), pairs(pairs_), whole(p.whole), kseg(p.kseg), units(static_cast<int64_t>(ntiles - p.whole) * p.kseg) {
-    nwhole = pair < whole ? (whole - 1 - pair) / pairs + 1 : 0;
+      : pair(pair_), pairs(pairs_), kseg(p.kseg), units(static_cast<int64_t>(ntiles) * p.kseg), cut(p.cut != 0) {
     beg = units * pair / pairs;
     end = units * (pair + 1) / pairs;
     t0 = static_cast<int>(beg / kseg);
-    nt = end > beg ? static_cast<int>((end - 1) / kseg) - t0 + 1 : 0;
-    leaves = end > beg && end % kseg != 0;
-    n = nwhole + nt;
+    leaves = cut && end > beg && end % kseg != 0;
+    n = cut ? (end > beg ? static_cast<int>((end - 1) / kseg) - t0 + 1 : 0) : pair < ntiles ? (ntiles - 1 - pair) / pairs + 1 : 0;
   }
   __device__ Segment get(int i) const {
+    if (!cut) return Segment{pair + i * pairs, 0, kseg};
     if (leaves) {
-      const int64_t first = static_cast<int64_t>(t0 + nt - 1) * kseg;
-      if (i == 0) return Segment{whole + t0 + nt - 1, static_cast<int>((beg > first ? beg : first) - first), static_cast<int>(end - first)};
+      const int64_t first = static_cast<int64_t>(t0 + n - 1) * kseg;
+      if (i == 0) return Segment{t0 + n - 1, static_cast<int>((beg > first ? beg : first) - first), static_cast<int>(end - first)};
       --i;
     }
-    if (i < nwhole) return Segment{pair + i * pairs, 0, kseg};
-    i -= nwhole;
-    const int mine = nt - (leaves ? 1 : 0), t = i < mine - 1 ? t0 + 1 + i : t0;
+    const int mine = n - (leaves ? 1 : 0), t = i < mine - 1 ? t0 + 1 + i : t0;
     const int64_t first = static_cast<int64_t>(t) * kseg;
-    return Segment{whole + t, beg > first ? static_cast<int>(beg - first) : 0, kseg};
+    return Segment{t, beg > first ? static_cast<int>(beg - first) : 0, kseg};
   }
   // of the pairs that have a part of the tile which this one completes
   __device__ int first_part(const Segment& sg) const {
     if (sg.k0 == 0) return pair;
-    const int64_t first = static_cast<int64_t>(sg.tile - whole) * kseg;
+    const int64_t first = static_cast<int64_t>(sg.tile) * kseg;
     int j = pair - 1;
     while (j > 0 && units * j / pairs > first) --j;
     return j;
@@ -1001,12 +998,13 @@ __global__ void __launch_bounds__(256) pack_u_kernel(const float* __restrict__ U
     }                                                   \
   } while (0)
 
-// Tiles of a product that are taken whole, and the SM cycles of the product.  A k-block takes the longer of its MMAs (6 cycles per
+// Tile width of a product, whether its contraction is cut, and its SM cycles.  A k-block takes the longer of its MMAs (6 cycles per
 // column by their rate, 7.2 as measured at 256 columns: 1,838) and of its bytes from L2 at 38 a cycle and SM (192 columns: 1,485;
 // 160: 1,395; 64: 1,100).  12,000 cycles from the start to the first MMA and from the last one to the results; 8,000 to leave
-// and to take over a part of a tile: a last round of tiles is cut when that gains more, and not into parts of less than
-// four k-blocks.
-struct ProductPlan { int bn; int64_t tiles, whole, pairs; double cost; };
+// and to take over a part of a tile: a product of fewer tiles than
+// pairs is cut when that gains more, and not into parts of less than four k-blocks.  (Cutting only the last of several rounds took
+// fewer cycles at a lower clock: 908 -> 1013 us.)
+struct ProductPlan { int bn; int64_t tiles, pairs; bool cut; double cost; };
 // fine: drained at every k-block, which the MMAs of a third of it do not hide.
 ProductPlan plan_width(int64_t M, int64_t N, int64_t Kc, bool sym, bool fine, int bn, int64_t max_pairs) {
   ProductPlan p{};
@@ -1014,20 +1012,19 @@ ProductPlan plan_width(int64_t M, int64_t N, int64_t Kc, bool sym, bool fine, in
   const int tm = static_cast<int>((M + PM - 1) / PM), tn = static_cast<int>((N + bn - 1) / bn);
   p.tiles = sym ? sym_tiles(tm, tn, bn) : static_cast<int64_t>(tm) * tn;
   const double per_kb = std::max(7.2 * bn, (2.0 * kBytesA + bn * BK * 2.0) / 38.0) + (fine ? 7.0 * bn : 0.0);
-  const int64_t kseg = (Kc + BK - 1) / BK, rounds = p.tiles / max_pairs, rest = p.tiles % max_pairs;
-  p.whole = p.tiles;
+  const int64_t kseg = (Kc + BK - 1) / BK, rounds = (p.tiles + max_pairs - 1) / max_pairs;
   p.pairs = std::min(p.tiles, max_pairs);
-  double kb = static_cast<double>((rounds + (rest > 0 ? 1 : 0)) * kseg);
-  if (rest > 0) {
-    const int64_t pairs = rounds > 0 ? max_pairs : std::max<int64_t>(1, std::min(max_pairs, rest * kseg / 4));
-    const double cut = static_cast<double>(rounds * kseg + (rest * kseg + pairs - 1) / pairs);
-    if (!sym && rounds == 0 && (kb - cut) * per_kb > 8000.0) {
-      p.whole = rounds * max_pairs;
+  double kb = static_cast<double>(rounds * kseg);
+  if (!sym && p.tiles < max_pairs) {
+    const int64_t pairs = std::max<int64_t>(1, std::min(max_pairs, p.tiles * kseg / 4));
+    const double shared = static_cast<double>((p.tiles * kseg + pairs - 1) / pairs);
+    if ((kb - shared) * per_kb > 8000.0) {
+      p.cut = true;
       p.pairs = pairs;
-      kb = cut + 8000.0 / per_kb;
+      kb = shared + 8000.0 / per_kb;
     }
   }
-  p.cost = kb * per_kb + 12000.0 + static_cast<double>(rounds) * 1500.0;
+  p.cost = kb * per_kb + 12000.0 + static_cast<double>(p.tiles / max_pairs) * 1500.0;
   return p;
 }
 ProductPlan plan_product(int64_t M, int64_t N, int64_t Kc, bool sym, bool fine, int64_t max_pairs) {
@@ -1047,7 +1044,7 @@ int split_product(sfb_ctx* ctx, int64_t off, int64_t n, const uint16_t* A, const
   TcState* st = static_cast<TcState*>(ctx->tc);
   const ProductPlan plan = plan_product(n, N, Cp, EPI == F_GRAM, kDrain<EPI, F16> == 1, std::min<int64_t>(st->max_pairs, std::min(sm_count(), kModelSms) / 2));
   p.bn = plan.bn;
-  p.whole = static_cast<int32_t>(plan.whole);
+  p.cut = plan.cut;
   p.partial = ctx->at<float>(ctx->lay.partial);
   p.ready = ctx->at<uint32_t>(ctx->lay.ready);
   p.stages = ring_stages(p.bn);

@@ -36,10 +36,6 @@ constexpr int kThreads = 64 + 32 * kEpiWarps;
 constexpr int kBars = 2 * S_MAX + 4;
 constexpr int kSmem = S * (kBytesA + kBytesB) + kEpiWarps * R * kSlotBytes + kBars * 8 + 16 + 1024;
 
-// Epilogues of the product  D (samples x N) = A * B^T:
-//   F_SOFTMAX  store D as fp32 logits and the softmax partials per (sample, pw columns)
-enum FwdEpi { F_SOFTMAX = 0 };
-
 struct TcParams {
   int32_t M, N, Kc;            // extents of the product: samples, output columns, contraction
   int32_t m_off;               // first sample handled by this launch (per-worker slices)
@@ -47,15 +43,15 @@ struct TcParams {
   int32_t a_rows;              // rows of A per box (fewer than 128 for a slice of few samples; the rest of a
                                // tile's samples are then never stored)
   int32_t stages;              // forward_kernel: stages of the operand ring
-  int32_t pw;                  // F_SOFTMAX: columns per softmax partial, a divisor of bn
+  int32_t pw;                  // columns per softmax partial, a divisor of bn
   int32_t bn;                  // columns per tile, at most BN, a multiple of 32 (chosen so that the tiles fill the SMs)
   // The contraction runs over nseg segments of kseg k-blocks; segment s reads A from column a_off<s> and B from
-  // column b_off<s> of their tensors: one segment is the plain product, three segments over [hi | lo] operand
-  // halves form the split-bf16 product hi*hi + hi*lo + lo*hi.  (Scalars: an indexed array would send the whole
-  // parameter block to local memory.)
+  // column b_off<s> of their tensors: one segment is the plain product, three segments over [big | small] tf32 operand
+  // halves form big*small + small*big + big*big.  (Scalars: an indexed array would send the whole parameter block to local
+  // memory.)
   int32_t nseg, kseg;
   int32_t a_off0, a_off1, a_off2, b_off0, b_off1, b_off2;
-  float2* part;                // F_SOFTMAX: [N / pw][part_ld] (max, sum exp) per sample and pw rows of W
+  float2* part;                // [N / pw][part_ld] (max, sum exp) per sample and pw rows of W
   int64_t part_ld;
   int32_t kparts;              // the contraction of a tile is cut over a cluster of this many CTAs (1: persistent CTAs)
   uint32_t* status;
@@ -71,7 +67,7 @@ __device__ __forceinline__ void tile_coords(const TcParams& p, int tile, int& m0
 
 // TF32: the operands are 32-bit words read as tf32 (a k-block of 128 bytes is then 32 elements and one MMA contracts
 // 8 of them); everything else -- stages, descriptors, epilogues -- is the same.
-template <int EPI, bool TF32 = false>
+template <bool TF32>
 __global__ void __launch_bounds__(kThreads, 1)
 forward_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                const __grid_constant__ CUtensorMap tmC, const TcParams p) {
@@ -171,26 +167,24 @@ forward_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     uint8_t* ring = sRing + q * R * kSlotBytes;
     const int my_tiles = tile0 < ntiles ? (ntiles - 1 - tile0) / tile_step + 1 : 0;
     bool ok = true;
-    // The fp32 result goes out through the ring by TMA; F_SOFTMAX keeps a running (max, sum exp) per sample.
+    // The fp32 result goes out through the ring by TMA; the epilogue keeps a running (max, sum exp) per sample.
     uint32_t gs = 0;                       // stores issued so far: consecutive stores alternate ring slots
     float mx = -INFINITY, sum = 0.f;
     auto finish = [&](uint32_t (&acc)[32], int m0, int n0, int c) {
       uint8_t* sl = ring + (gs % R) * kSlotBytes;
       const int col0 = n0 + c * kChunk, row = m0 + q * 32 + lane;
       if (col0 < p.N) {
-        if constexpr (EPI == F_SOFTMAX) {
-          float cm = -INFINITY;
+        float cm = -INFINITY;
 #pragma unroll
-          for (int j = 0; j < 32; ++j)
-            if (col0 + j < p.N) cm = fmaxf(cm, __uint_as_float(acc[j]));
-          const float nm = fmaxf(mx, cm);
-          float cs = 0.f;
+        for (int j = 0; j < 32; ++j)
+          if (col0 + j < p.N) cm = fmaxf(cm, __uint_as_float(acc[j]));
+        const float nm = fmaxf(mx, cm);
+        float cs = 0.f;
 #pragma unroll
-          for (int j = 0; j < 32; ++j)
-            if (col0 + j < p.N) cs += __expf(__uint_as_float(acc[j]) - nm);
-          sum = sum * __expf(mx - nm) + cs;
-          mx = nm;
-        }
+        for (int j = 0; j < 32; ++j)
+          if (col0 + j < p.N) cs += __expf(__uint_as_float(acc[j]) - nm);
+        sum = sum * __expf(mx - nm) + cs;
+        mx = nm;
         if (lane == 0) tma_wait_group_read<R - 1>();   // the store that last used this slot has read it
         __syncwarp();
 #pragma unroll
@@ -205,7 +199,7 @@ forward_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         }
         ++gs;
       }
-      if (EPI == F_SOFTMAX && ((c + 1) * kChunk) % p.pw == 0) {      // the end of a group of pw columns
+      if (((c + 1) * kChunk) % p.pw == 0) {      // the end of a group of pw columns
         const int grp = (n0 + (c + 1) * kChunk) / p.pw - 1;
         if (grp * p.pw < p.N && row < p.M) p.part[static_cast<int64_t>(grp) * p.part_ld + row] = make_float2(mx, sum);
         mx = -INFINITY;
@@ -738,22 +732,22 @@ __global__ void __launch_bounds__(256) mlr_finish_u_kernel(const float* __restri
 // ---------------------------------------------------------------------------------------------------------
 // Host side
 // ---------------------------------------------------------------------------------------------------------
-template <int EPI, bool TF32 = false>
+template <bool TF32>
 cudaError_t launch_forward(sfb_ctx* ctx, const CUtensorMap& a, const CUtensorMap& b, const CUtensorMap& c, TcParams p) {
   TcState* st = static_cast<TcState*>(ctx->tc);
   const int64_t tiles = static_cast<int64_t>(p.tilesM) * p.tilesN;
   if (tiles <= 0) return cudaSuccess;
   const unsigned grid = static_cast<unsigned>(p.kparts > 1 ? tiles * p.kparts : std::min<int64_t>(tiles, st->sms));
-  return launch_kernel_if(tiles * p.kparts <= st->sms, forward_kernel<EPI, TF32>, dim3(grid), dim3(kThreads), kSmem, ctx->stream,
+  return launch_kernel_if(tiles * p.kparts <= st->sms, forward_kernel<TF32>, dim3(grid), dim3(kThreads), kSmem, ctx->stream,
                           p.kparts, a, b, c, p);
 }
 
 // The shared-memory opt-in is a per-device attribute of each kernel: set for every instantiation when a context is
 // created (with its device current), not once per process.
 cudaError_t prepare_forward_kernels() {
-  cudaError_t e = cudaFuncSetAttribute(forward_kernel<F_SOFTMAX>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
+  cudaError_t e = cudaFuncSetAttribute(forward_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
   if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(forward_kernel<F_SOFTMAX, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
+    e = cudaFuncSetAttribute(forward_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
   return e;
 }
 
@@ -935,7 +929,7 @@ static int mlr32_forward(sfb_ctx* ctx, int64_t off, int64_t n, const float* X, i
   p.nseg = 3; p.kseg = static_cast<int32_t>(L.colsp / (BK / 2));          // cross terms first, big*big last
   p.a_off0 = 0; p.a_off1 = static_cast<int32_t>(L.colsp); p.a_off2 = 0;
   p.b_off0 = static_cast<int32_t>(L.colsp); p.b_off1 = 0; p.b_off2 = 0;
-  CKC((launch_forward<F_SOFTMAX, true>(ctx, ma, mb, mc, p)));                                // z_i = W x_i
+  CKC((launch_forward<true>(ctx, ma, mb, mc, p)));                                // z_i = W x_i
   ctx->stats.flops += 3.0 * 2.0 * n * rows * cols;
   *tiles_n = p.tilesN;
   return SFB_OK;
@@ -977,7 +971,7 @@ int tc32_factors(sfb_ctx* ctx, int64_t off, int64_t n, const float* X, const int
                  float inv_lam_n) {
   const sfb_config& c = ctx->cfg;
   const Layout& L = ctx->lay;
-  const int64_t rows = c.rows, cols = c.cols, K = ctx->K;
+  const int64_t rows = c.rows, K = ctx->K;
   const int64_t ldz = round_up(rows, 32);
   cudaStream_t s = ctx->stream;
   float* Z = ctx->at<float>(L.ZT);
@@ -1048,7 +1042,7 @@ static int mlr_forward(sfb_ctx* ctx, int64_t off, int64_t n, const float* X, con
   p.tilesN = static_cast<int32_t>((rows + bn - 1) / bn);
   p.part = ctx->at<float2>(L.part); p.part_ld = K; p.status = ctx->at<uint32_t>(L.status);
   p.nseg = 1; p.kseg = (p.Kc + BK - 1) / BK;
-  CKC(launch_forward<F_SOFTMAX>(ctx, ma, mb, mc, p));
+  CKC(launch_forward<false>(ctx, ma, mb, mc, p));
   ctx->stats.flops += 2.0 * n * rows * cols;
   *parts = static_cast<int>((rows + L.pw - 1) / L.pw);
   return SFB_OK;
@@ -1190,8 +1184,8 @@ int tc_export_factors(sfb_ctx* ctx, int64_t off, int64_t n, float* U_out, float*
   return SFB_OK;
 }
 
-// Received fp32 factors take a worker's place in the bf16 layout: v into V^T (bf16) and the fp32 sample copy, u into U^T
-// (bf16, 0 at the class entry), the class entry into the fp32 label coefficients.
+// Received fp32 factors take a worker's place in the bf16 layout: v as the bf16 operand and the fp32 sample copy, u as the bf16
+// operand (0 at the class entry), the class entry into the fp32 label coefficients.
 int tc_import_factors(sfb_ctx* ctx, int64_t off, int64_t n, const float* U_in, const float* V_in) {
   const sfb_config& c = ctx->cfg;
   const Layout& L = ctx->lay;

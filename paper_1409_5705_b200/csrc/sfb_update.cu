@@ -52,7 +52,7 @@ struct UpdParams {
   int32_t rows, cols;          // shape of W
   int32_t tilesM, tilesN;      // pair tiles: 256 rows x bn columns
   int32_t bn;                  // 256 or 128
-  int32_t nseg, kseg;          // contraction: nseg segments of kseg k-blocks (3 segments: split-bf16 product)
+  int32_t nseg, kseg;          // contraction: nseg segments of kseg k-blocks (3 segments: tf32 pairs)
   // Segment s reads U^T from column a_off<s> and V^T from column b_off<s>.  Scalars, not arrays: indexing an
   // array of a kernel parameter with a run-time index moves the whole parameter block to local memory.
   int32_t a_off0, a_off1, a_off2, b_off0, b_off1, b_off2;
