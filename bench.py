@@ -222,24 +222,6 @@ def run_reference(args, wl, rank):
     print(json.dumps(line), flush=True)
 
 
-# DRAM bytes per launch of the update kernel at the paper-scale MLR shape, from the one-pass ncu capture summarised in
-# profiles/ncu_update_pair_kernel_mlr_large_dram.md (dram__bytes_read.sum + dram__bytes_write.sum of one launch of the
-# full-size bench).  The bf16 copy of W is rewritten only where its rounding changed, so the traffic depends on the data
-# and does not scale with the rows: the figure applies to this workload only.  "kernel_unchanged_since" names the
-# commit of the kernel's sources (csrc/sfb_update.cu, csrc/sfb_ptx.cuh) the counters were taken at: when the kernel is edited
-# this entry has to be re-captured
-# or set to None.
-NCU_UPDATE_TRAFFIC = {"rows": 325000, "cols": 10000, "K": 1024, "bytes": 15.29e9 + 13.85e9,
-                      "kernel_unchanged_since": "d08beef"}
-
-
-def ncu_traffic_per_launch(wl, prec):
-    t = NCU_UPDATE_TRAFFIC
-    if t["bytes"] is None or wl.model != I.MLR or wl.cols != t["cols"] or wl.K != t["K"] or wl.rows != t["rows"]             or prec != 0:
-        return None
-    return t["bytes"]
-
-
 def workload_config(wl, dtype):
     return {"workload": wl.name, "family": ["mlr", "dml", "sc"][wl.model], "rows": wl.rows, "cols": wl.cols,
             "workers_P": wl.workers, "batch_B": wl.batch, "K": wl.K, "eta": wl.eta, "operands": dtype,
@@ -251,25 +233,10 @@ def precision_code(S, name):
     return {"bf16": S.PREC_BF16, "fp32": S.PREC_FP32, "tf32": S.PREC_TF32X3, "ffma": S.PREC_FP32_FFMA}[name]
 
 
-def dtype_name(wl, name):
-    """The arithmetic type of the products: bf16, f32 (FFMA), or f16x3 / tf32x3 (fp32 values as pairs of fp16 or tf32 words)."""
-    if name == "bf16":
-        return "bf16"
-    return "tf32x3" if runs_tf32(wl, name) else "f16x3" if runs_fp16_pairs(wl, name) else "f32"
-
-
-def runs_tf32(wl, name):
-    return name == "tf32" and wl.model == I.MLR
-
-
-def runs_fp16_pairs(wl, name):
-    """Whether the fp32 mode runs this workload's products on the tensor cores as pairs of fp16 words (the library's own rule)."""
-    if name != "fp32" or wl.rows < 64 or wl.cols < 64:
-        return False
-    macs = float(wl.K) * wl.rows * wl.cols
-    if wl.model == I.SC:
-        return macs >= 2.8e8
-    return wl.cols >= 256 and (macs >= 1e9 or macs * (1 - 24 / wl.K) >= 1.8e8)
+def dtype_name(name, form):
+    """The arithmetic type of the products: bf16, f32 (FFMA, or the sums over sparse samples), or f16x3 / tf32x3 (fp32 values as pairs
+    of fp16 or tf32 words), by what the library says its update ran on."""
+    return "bf16" if name == "bf16" else {3: "f16x3", 4: "tf32x3"}.get(form, "f32")
 
 
 NOMINAL_BF16_TFLOPS = 2250.0        # dense bf16, vendor figure (context only)
@@ -318,8 +285,7 @@ def update_roofline(wl, prec_bf16, ms_u, peaks, clocks, sustained=True, tf32=Fal
         roof = {"bound": "alu", "achieved": upd_flops / (ms_u * 1e-3) / 1e12, "peak": peak, "unit": "TFLOP/s"}
         roof["roof_ms"] = upd_flops / (peak * 1e12) * 1e3
     roof["frac"] = roof["achieved"] / roof["peak"]
-    roof["traffic"] = ncu_traffic_per_launch(wl, 0 if prec_bf16 else 1)
-    roof["traffic_captured_at"] = NCU_UPDATE_TRAFFIC["kernel_unchanged_since"] if roof["traffic"] else None
+    roof["traffic"] = None                       # (no DRAM counters have been taken of the kernel as it is)
     roof["kernel"] = "update_pair_kernel (sfb_apply_update)" if prec_bf16 \
         else "update_pair_kernel<tf32 pairs> (sfb_apply_update)" if tf32 else "update_split_kernel (sfb_apply_update)" if pairs else "sgemm_kernel EPI_RMW (sfb_apply_update)"
     roof["ms"] = ms_u
@@ -433,20 +399,18 @@ def run_sharded(args, wl, rank, world, local):
     launches = st.kernel_launches - launches0
     status = ctx.sfb_get_status()
     ms_u = st.ms_update
+    form = ctx.sfb_get_update_form()
     total_ms, ms_u = max_over_ranks([total_ms, ms_u], dev, world)
     if rank == 0:
         value = K * args.steps / (total_ms * 1e-3)                          # one problem: K samples per step in all
         shard = I.scaled(wl, wl.name, rows=r1 - r0)
-        roof = update_roofline(shard, prec == S.PREC_BF16, ms_u, peaks, clocks, tf32=runs_tf32(shard, args.precision),
-                          pairs=runs_fp16_pairs(shard, args.precision))
-        roof["traffic"] = None
-        roof["traffic_captured_at"] = None
+        roof = update_roofline(shard, prec == S.PREC_BF16, ms_u, peaks, clocks, tf32=form == 4, pairs=form == 3)
         model = exchange_model_bytes(wl.workers, wl.batch, wl.rows, wl.cols, world)
         line = {"metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
                 "warmup": args.warmup, "ms_per_step": total_ms / args.steps, "higher_is_better": True,
-                "scaling": "strong", "vs_baseline": None, "dtype": dtype_name(wl, args.precision),
+                "scaling": "strong", "vs_baseline": None, "dtype": dtype_name(args.precision, form),
                 "data": "synthetic",
-                "config": dict(workload_config(wl, dtype_name(wl, args.precision)),
+                "config": dict(workload_config(wl, dtype_name(args.precision, form)),
                                parallelism=f"rows{world}", rows_per_rank=r1 - r0),
                 "roofline": roof, "cpu_baseline": None, "e2e": None, "gpu_launches": int(launches), "clocks": clocks,
                 "exchange": {"measured_bytes_received_per_rank": moved.total if moved else 0,
@@ -617,6 +581,7 @@ def main():
         # the L2 flush runs between the steps; the value counts the steps' own device intervals
         total_ms = sum(e[0].elapsed_time(e[3]) for e in evs)
     st1 = ctx.sfb_get_stats()
+    form = ctx.sfb_get_update_form()
     launches = st1.kernel_launches - launches0
     copy_stats = {"row_pieces_per_step": (st1.copy_pieces - st0.copy_pieces) / args.steps,
                   "rewritten_per_step": (st1.copy_written - st0.copy_written) / args.steps,
@@ -679,7 +644,7 @@ def main():
         update_loop = {"launches": reps, "ms": ms_loop, "seconds": ms_loop * reps * 1e-3, "clocks": ck,
                        "ms_x_sm_mhz": ms_loop * ck["sm_mhz"] if ck.get("sm_mhz") else None,
                        "roofline": update_roofline(wl, prec == S.PREC_BF16, ms_loop, peaks, ck,
-                                                   tf32=runs_tf32(wl, args.precision), pairs=runs_fp16_pairs(wl, args.precision))}
+                                                   tf32=form == 4, pairs=form == 3)}
 
     # ---- end to end: host minibatch -> sfb_step_host -> loss back on the host, every step (sparse samples: the three
     # arrays and the labels copied from pinned memory, sfb_step_csr, the loss read back through sfb_get_stats)
@@ -748,7 +713,7 @@ def main():
         h2d = int(sum(8 * (K + 1) + 8 * n for _, _, _, n in hS) / nb) + K * 4
 
     # ---- roofline of the dominant kernel (the fused update), timed inside the long step: sustained tensor figure
-    roof = update_roofline(wl, prec == S.PREC_BF16, ms_u, peaks, clocks, tf32=runs_tf32(wl, args.precision), pairs=runs_fp16_pairs(wl, args.precision),
+    roof = update_roofline(wl, prec == S.PREC_BF16, ms_u, peaks, clocks, tf32=form == 4, pairs=form == 3,
                            copy_fraction=min(1.0, copy_stats["rewritten_per_step"] / (wl.rows * math.ceil(wl.cols / 32)))
                            if copy_stats else 1.0)
     sparse_ran = sparse and st1.sparse_updates > st0.sparse_updates
@@ -783,7 +748,7 @@ def main():
     if prec == S.PREC_BF16 and wl.model != I.MLR:
         esz = 4
     one_copy = K * (wl.rows + wl.cols) * esz
-    cfg_line = workload_config(wl, dtype_name(wl, args.precision))
+    cfg_line = workload_config(wl, dtype_name(args.precision, form))
     if sparse:
         one_copy = K * wl.rows * esz + 8 * sum(n for _, _, _, n in hS) / nb
         cfg_line["features"] = (f"compressed sparse rows, about {args.sparse_nnz:g} non-zeros per sample "
@@ -791,7 +756,7 @@ def main():
         cfg_line["update"] = ("sparse" if sparse_ran else "dense") + f" ({args.sparse_update})"
     line = {"metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
             "warmup": args.warmup, "ms_per_step": total_ms / args.steps, "higher_is_better": True,
-            "scaling": "weak", "vs_baseline": None, "dtype": dtype_name(wl, args.precision),
+            "scaling": "weak", "vs_baseline": None, "dtype": dtype_name(args.precision, form),
             "data": "synthetic", "config": cfg_line,
             "roofline": roof, "roofline_forward": roof_fwd, "roofline_step": roof_step, "cpu_baseline": cpu,
             "e2e": {"value": e2e_value, "unit": UNIT, "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": 8,

@@ -110,7 +110,7 @@ typedef struct sfb_stats {
   double  gather_bytes;       /* bytes of gathered factors, one copy: K*(rows+cols)*element size        */
   double  gather_bytes_p2p;   /* the paper's peer-to-peer count: P*(P-1)*B*(rows+cols)*element size     */
   double  dense_sync_bytes;   /* what full-matrix sync would move: P*rows*cols*4 (Section 5 cost table) */
-  float   ms_factors, ms_gather, ms_update;  /* device time of the last step's phases (CUDA events)     */
+  float   ms_factors, ms_gather, ms_update;  /* device time of the last step's phases (kernels' stamps)  */
   float   last_loss;          /* MLR: mean over the last step's K samples of -log p(y_i); else 0        */
   float   sc_lipschitz;       /* SC: the L = ||W||_2^2 the coder used in the last step                  */
   int64_t kernel_launches;    /* kernels this library has launched in this process                      */
@@ -302,7 +302,7 @@ int sfb_dense_sync_step(sfb_ctx* ctx, const float* X_dev, const float* Y_dev, co
                         float* scratch_dev, size_t scratch_bytes);
 
 /* The gathered factor buffers of the last gather, for inspection.  dtype: 0 = fp32, 1 = bf16.
- * layout: 0 = pair-major (U [K x ldu], V [K x ldv]); 1 = transposed (U^T [rows x ldu], V^T [cols x ldv]).
+ * layout: 0 = pair-major (U [K x ldu], V [K x ldv]).
  * DML and SC return their fp32 pair-major factors in both modes.
  * MLR in bf16 mode splits u_i = p_i - onehot(y_i) in two: the buffer holds the probabilities p_i in bf16 with a 0
  * at the label entry (i, y_i); that entry, p_iy - 1, is kept in fp32 and applied to row y_i of W separately
@@ -315,6 +315,10 @@ int sfb_get_factors(sfb_ctx* ctx, const void** U_dev, const void** V_dev, int32_
  * ld/2 + c.  SFB_ERR_UNSUPPORTED where no persistent copy exists (the other models and SFB_PREC_FP32 rebuild theirs
  * every step; the FFMA kernels read W itself). */
 int sfb_get_operand_copy(sfb_ctx* ctx, const void** copy_dev, int32_t* dtype, int64_t* ld);
+
+/* Which products the last gathered update runs on: 0 fp32 FMAs, 1 bf16, 2 pairs of bf16 words, 3 pairs of fp16 words, 4 pairs of
+ * tf32 words, 5 the sums over sparse samples.  SFB_ERR_STATE before the first gather. */
+int sfb_get_update_form(sfb_ctx* ctx, int32_t* form);
 
 /* Waits for the stream, then fills the counters. */
 int sfb_get_stats(sfb_ctx* ctx, sfb_stats* out);

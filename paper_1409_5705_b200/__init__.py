@@ -19,7 +19,7 @@ STATUS_LABEL_RANGE, STATUS_TIMEOUT, STATUS_SAMPLE_RANGE, STATUS_INDEX_RANGE = 0x
 
 EXPORTS = ("sfb_workspace_bytes", "sfb_init", "sfb_compute_factors", "sfb_gather_factors", "sfb_apply_update",
            "sfb_step", "sfb_step_host", "sfb_dense_sync_step", "sfb_get_factors", "sfb_get_stats",
-           "sfb_get_status", "sfb_strerror", "sfb_last_cuda_error", "sfb_destroy", "sfb_prox_columns_noalloc",
+           "sfb_get_update_form", "sfb_get_status", "sfb_strerror", "sfb_last_cuda_error", "sfb_destroy", "sfb_prox_columns_noalloc",
            "sfb_selftest_wait_timeout", "sfb_set_row_shard", "sfb_forward_partials", "sfb_finish_factors",
            "sfb_replay_update", "sfb_refresh_operands", "sfb_sdca_set_dual", "sfb_sdca_compute_factors",
            "sfb_sdca_step", "sfb_set_factors", "sfb_set_eta", "sfb_get_operand_copy", "sfb_compute_factors_csr",
@@ -220,7 +220,7 @@ class Context:
                                            scratch.numel() * scratch.element_size()), "sfb_dense_sync_step")
 
     def sfb_get_factors(self):
-        """(U address, V address, dtype 0 fp32 / 1 bf16, layout 0 pair-major / 1 transposed, ldu, ldv)."""
+        """(U address, V address, dtype 0 fp32 / 1 bf16, layout 0 pair-major, ldu, ldv)."""
         U, V = ctypes.c_void_p(), ctypes.c_void_p()
         dt, lo = ctypes.c_int32(), ctypes.c_int32()
         ldu, ldv = ctypes.c_int64(), ctypes.c_int64()
@@ -241,9 +241,7 @@ class Context:
             off = addr - ws0
             flat = self.workspace[off:off + n0 * ld * esz].view(tdt)
             return flat.view(n0, ld)
-        if lo == 0:
-            return view(U, K, ldu)[:, :rows].float(), view(V, K, ldv)[:, :cols].float()
-        return view(U, rows, ldu)[:, :K].t().float(), view(V, cols, ldv)[:, :K].t().float()
+        return view(U, K, ldu)[:, :rows].float(), view(V, K, ldv)[:, :cols].float()
 
     def capture(self, calls):
         """Captures the library calls made by ``calls()`` on this context's stream into one CUDA graph and returns it
@@ -272,6 +270,12 @@ class Context:
         st = sfb_stats()
         self._ck(lib().sfb_get_stats(self._h, ctypes.byref(st)), "sfb_get_stats")
         return st
+
+    def sfb_get_update_form(self) -> int:
+        """Products of the last gathered update: 0 fp32 FMAs, 1 bf16, 2 / 3 / 4 pairs of bf16 / fp16 / tf32 words, 5 sparse sums."""
+        form = ctypes.c_int32(0)
+        self._ck(lib().sfb_get_update_form(self._h, ctypes.byref(form)), "sfb_get_update_form")
+        return form.value
 
     def sfb_get_status(self) -> int:
         st = ctypes.c_uint32(0)

@@ -960,6 +960,14 @@ extern "C" int sfb_get_operand_copy(sfb_ctx* ctx, const void** copy_dev, int32_t
   return SFB_OK;
 }
 
+extern "C" int sfb_get_update_form(sfb_ctx* ctx, int32_t* form) {
+  if (!ctx || !form) return SFB_ERR_ARG;
+  if (ctx->stats.gather_bytes == 0.0) return SFB_ERR_STATE;
+  const sfb_config& c = ctx->cfg;
+  *form = ctx->sparse_v ? 5 : ctx->tf32 ? 4 : c.precision == SFB_PREC_BF16 ? (c.model == SFB_MLR ? 1 : 2) : ctx->h16 && !ctx->update_fma ? 3 : 0;
+  return SFB_OK;
+}
+
 extern "C" int sfb_get_stats(sfb_ctx* ctx, sfb_stats* out) {
   if (!ctx || !out) return SFB_ERR_ARG;
   const sfb_config& c = ctx->cfg;
