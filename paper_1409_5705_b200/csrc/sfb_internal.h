@@ -141,8 +141,9 @@ inline int64_t round_up(int64_t x, int64_t m) { return (x + m - 1) / m * m; }
 
 // Which kernels the products of an fp32 mode run on.  Pairs of tf32 words when asked for (logistic models).  SFB_PREC_FP32 runs
 // on pairs of fp16 words with fp32 scales (sfb_split.cu) where the products are large enough to repay the packing of their
-// operands (W once per step, as much work as 24 more pairs), else on the FMA kernels.  us per step, fp16 pairs / FMAs: sparse
-// coding 2,000 x 1,000 K = 128 459 / 425, 6,000 x 3,000 K = 16 1242 / 2568; metric learning 300 x 1,000 K = 500 55 / 49,
+// operands (W once per step, as much work as 24 more pairs), else on the FMA kernels.  Sparse coding by the
+// costs of its forms (sc_on_pairs).  us per step, fp16 pairs / FMAs: sparse coding 814 x 1,252 K = 620 1311 / 2240, 2,422 x 760 K = 209
+// 1201 / 723; metric learning 300 x 1,000 K = 500 55 / 49,
 // 500 x 4,000 K = 100 66 / 77; regression 2,000 x 5,000 K = 16 128 / 90, 3,000 x 600 K = 130 50 / 64, 10,000 x 20,000 K = 16
 // 1306 / 1583, 50,000 x 64 K = 256 192 / 148 (bound by u, which is packed too).
 inline bool use_tf32(const sfb_config& c) {
