@@ -231,7 +231,7 @@ split_product_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + kBars);
   volatile uint32_t* abort_flag = tmem_slot + 1;
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_index(), lane = threadIdx.x & 31;
   const uint32_t rank = cluster_ctarank();
   const int ST = p.stages, half = p.bn / 2;
   const int bytesB = half * BK * 2, stage_bytes = 2 * kBytesA + 2 * bytesB;
@@ -260,7 +260,7 @@ split_product_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
 
   if (warp < 4) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 40;");
-    if (warp == 0 && lane == 0) {
+    if (warp == 0) {
       // ---------------- TMA producer ----------------
       const uint64_t pol_keep = policy_evict_last(), pol_norm = policy_evict_normal();
       uint32_t s = 0, ph = 0;
@@ -272,22 +272,24 @@ split_product_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
         const int ma = m0 + static_cast<int>(rank) * BM, nb = n0 + static_cast<int>(rank) * half;
         for (int k = sg.k0; k < sg.k1; ++k) {
           const int x = k * BK;
-          if (!mbar_wait(&empty[s], ph ^ 1, abort_flag)) { ok = false; break; }
-          if (k + 4 < sg.k1) {                          // B streams from HBM when it is larger than L2: asked for early
-            tma_prefetch_2d(&tmB, x + 4 * BK, nb);
-            tma_prefetch_2d(&tmB, p.b_lo + x + 4 * BK, nb);
+          if (!mbar_wait_warp(&empty[s], ph ^ 1, abort_flag)) { ok = false; break; }
+          if (elect_one()) {
+            if (k + 4 < sg.k1) {                        // B streams from HBM when it is larger than L2: asked for early
+              tma_prefetch_2d(&tmB, x + 4 * BK, nb);
+              tma_prefetch_2d(&tmB, p.b_lo + x + 4 * BK, nb);
+            }
+            if (rank == 0) mbar_expect_tx(&full[s], 2 * (2 * p.a_rows * BK * 2 + 2 * bytesB));
+            const uint32_t bar = mapa_u32(smem_u32(&full[s]), 0);
+            uint8_t* st = smem + s * stage_bytes;
+            tma_load_2d_pair(st, &tmA, x, ma, bar, pol_keep);
+            tma_load_2d_pair(st + kBytesA, &tmA, p.a_lo + x, ma, bar, pol_keep);
+            tma_load_2d_pair(st + 2 * kBytesA, &tmB, x, nb, bar, pol_norm);
+            tma_load_2d_pair(st + 2 * kBytesA + bytesB, &tmB, p.b_lo + x, nb, bar, pol_norm);
           }
-          if (rank == 0) mbar_expect_tx(&full[s], 2 * (2 * p.a_rows * BK * 2 + 2 * bytesB));
-          const uint32_t bar = mapa_u32(smem_u32(&full[s]), 0);
-          uint8_t* st = smem + s * stage_bytes;
-          tma_load_2d_pair(st, &tmA, x, ma, bar, pol_keep);
-          tma_load_2d_pair(st + kBytesA, &tmA, p.a_lo + x, ma, bar, pol_keep);
-          tma_load_2d_pair(st + 2 * kBytesA, &tmB, x, nb, bar, pol_norm);
-          tma_load_2d_pair(st + 2 * kBytesA + bytesB, &tmB, p.b_lo + x, nb, bar, pol_norm);
           if (++s == static_cast<uint32_t>(ST)) { s = 0; ph ^= 1; }
         }
       }
-    } else if (warp == 1 && lane == 0 && rank == 0) {
+    } else if (warp == 1 && rank == 0) {
       // ---------------- MMA issuer ----------------
       const uint32_t idesc = F16 ? umma_idesc_fp16(PM, p.bn) : umma_idesc_bf16(PM, p.bn);
       const uint32_t d_main = tmem_base, d_cross = tmem_base + kMaxN;
@@ -298,32 +300,33 @@ split_product_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
         const int nk = sg.k1 - sg.k0;
         for (int kb = 0; kb < nk; ++kb) {
           const int kc = kb % kDrain<EPI, F16>;
-          if (!mbar_wait(&full[s], ph, abort_flag) || (kc == 0 && !mbar_wait(mempty, (g & 1) ^ 1, abort_flag)) ||
-              (kb == 0 && !mbar_wait(cempty, (i & 1) ^ 1, abort_flag))) { ok = false; break; }
+          if (!mbar_wait_warp(&full[s], ph, abort_flag) || (kc == 0 && !mbar_wait_warp(mempty, (g & 1) ^ 1, abort_flag)) ||
+              (kb == 0 && !mbar_wait_warp(cempty, (i & 1) ^ 1, abort_flag))) { ok = false; break; }
           tc_fence_after();
-          uint8_t* st = smem + s * stage_bytes;
-          const uint64_t dah = umma_desc_k128(smem_u32(st)), dal = umma_desc_k128(smem_u32(st + kBytesA));
-          const uint64_t dbh = umma_desc_k128(smem_u32(st + 2 * kBytesA)), dbl = umma_desc_k128(smem_u32(st + 2 * kBytesA + bytesB));
+          const bool drained = kc == kDrain<EPI, F16> - 1 || kb + 1 == nk;
+          if (elect_one()) {
+            uint8_t* st = smem + s * stage_bytes;
+            const uint64_t dah = umma_desc_k128(smem_u32(st)), dal = umma_desc_k128(smem_u32(st + kBytesA));
+            const uint64_t dbh = umma_desc_k128(smem_u32(st + 2 * kBytesA)), dbl = umma_desc_k128(smem_u32(st + 2 * kBytesA + bytesB));
 #pragma unroll
-          for (int k = 0; k < BK / UMMA_K; ++k) {
-            const uint64_t adv = static_cast<uint64_t>(k * UMMA_K * 2 / 16);
-            umma_bf16_pair(d_main, dah + adv, dbh + adv, idesc, (kc | k) != 0 ? 1u : 0u);      // A_hi B_hi
-            umma_bf16_pair(d_cross, dah + adv, dbl + adv, idesc, (kb | k) != 0 ? 1u : 0u);     // A_hi B_lo
-          }
-          if (kc == kDrain<EPI, F16> - 1 || kb + 1 == nk) {
-            umma_commit_pair(mfull, 3);
-            ++g;
-          }
+            for (int k = 0; k < BK / UMMA_K; ++k) {
+              const uint64_t adv = static_cast<uint64_t>(k * UMMA_K * 2 / 16);
+              umma_bf16_pair(d_main, dah + adv, dbh + adv, idesc, (kc | k) != 0 ? 1u : 0u);      // A_hi B_hi
+              umma_bf16_pair(d_cross, dah + adv, dbl + adv, idesc, (kb | k) != 0 ? 1u : 0u);     // A_hi B_lo
+            }
+            if (drained) umma_commit_pair(mfull, 3);
 #pragma unroll
-          for (int k = 0; k < BK / UMMA_K; ++k) {
-            const uint64_t adv = static_cast<uint64_t>(k * UMMA_K * 2 / 16);
-            umma_bf16_pair(d_cross, dal + adv, dbh + adv, idesc, 1u);                          // A_lo B_hi
-            if (EPI == F_GRAM && !F16 && p.four) umma_bf16_pair(d_cross, dal + adv, dbl + adv, idesc, 1u);
+            for (int k = 0; k < BK / UMMA_K; ++k) {
+              const uint64_t adv = static_cast<uint64_t>(k * UMMA_K * 2 / 16);
+              umma_bf16_pair(d_cross, dal + adv, dbh + adv, idesc, 1u);                          // A_lo B_hi
+              if (EPI == F_GRAM && !F16 && p.four) umma_bf16_pair(d_cross, dal + adv, dbl + adv, idesc, 1u);
+            }
+            umma_commit_pair(&empty[s], 3);
           }
-          umma_commit_pair(&empty[s], 3);
+          if (drained) ++g;
           if (++s == static_cast<uint32_t>(ST)) { s = 0; ph ^= 1; }
         }
-        if (ok) umma_commit_pair(cfull, 3);
+        if (ok && elect_one()) umma_commit_pair(cfull, 3);
       }
     }
     __syncwarp();

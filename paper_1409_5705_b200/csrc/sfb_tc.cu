@@ -84,7 +84,7 @@ forward_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + kBars);
   volatile uint32_t* abort_flag = tmem_slot + 1;
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_index(), lane = threadIdx.x & 31;
   const int ntiles = p.tilesM * p.tilesN;
   // With a split contraction a CTA has one tile and the k-blocks [kbeg, kend) of its nseg * kseg; else all of them and the
   // tiles blockIdx.x, blockIdx.x + gridDim.x, ...
@@ -110,43 +110,43 @@ forward_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
 
   if (warp == 0) {
     // ---------------- TMA producer ----------------
-    if (lane == 0) {
-      // A (the K samples) is the small operand every tile re-reads: pinned in L2.
-      const uint64_t pol_keep = policy_evict_last();
-      uint32_t s = 0, ph = 0;
-      bool ok = true;
-      for (int tile = tile0; tile < ntiles && ok; tile += tile_step) {
-        int m0, n0;
-        tile_coords(p, tile, m0, n0);
-        for (int seg = 0; seg < p.nseg && ok; ++seg) {
-          const int xa0 = seg == 0 ? p.a_off0 : seg == 1 ? p.a_off1 : p.a_off2;
-          const int xb0 = seg == 0 ? p.b_off0 : seg == 1 ? p.b_off1 : p.b_off2;
-          const int kl1 = min(p.kseg, kend - seg * p.kseg);
-          for (int kl = max(0, kbeg - seg * p.kseg); kl < kl1; ++kl) {
-            if (!mbar_wait(&empty[s], ph ^ 1, abort_flag)) { ok = false; break; }
+    // A (the K samples) is the small operand every tile re-reads: pinned in L2.
+    const uint64_t pol_keep = policy_evict_last();
+    uint32_t s = 0, ph = 0;
+    bool ok = true;
+    for (int tile = tile0; tile < ntiles && ok; tile += tile_step) {
+      int m0, n0;
+      tile_coords(p, tile, m0, n0);
+      for (int seg = 0; seg < p.nseg && ok; ++seg) {
+        const int xa0 = seg == 0 ? p.a_off0 : seg == 1 ? p.a_off1 : p.a_off2;
+        const int xb0 = seg == 0 ? p.b_off0 : seg == 1 ? p.b_off1 : p.b_off2;
+        const int kl1 = min(p.kseg, kend - seg * p.kseg);
+        for (int kl = max(0, kbeg - seg * p.kseg); kl < kl1; ++kl) {
+          if (!mbar_wait_warp(&empty[s], ph ^ 1, abort_flag)) { ok = false; break; }
+          if (elect_one()) {
             uint8_t* st = smem + s * stage_bytes;
             mbar_expect_tx(&full[s], (p.a_rows + p.bn) * BK * 2);
             tma_load_2d_hint(st, &tmA, xa0 + kl * (TF32 ? BK / 2 : BK), m0, &full[s], pol_keep);
             tma_load_2d(st + kBytesA, &tmB, xb0 + kl * (TF32 ? BK / 2 : BK), n0, &full[s]);
-            if (++s == static_cast<uint32_t>(ST)) { s = 0; ph ^= 1; }
           }
+          if (++s == static_cast<uint32_t>(ST)) { s = 0; ph ^= 1; }
         }
       }
     }
   } else if (warp == 1) {
     // ---------------- MMA issuer ----------------
-    if (lane == 0) {
-      const uint32_t idesc = TF32 ? umma_idesc_tf32(BM, p.bn) : umma_idesc_bf16(BM, p.bn);
-      uint32_t s = 0, ph = 0, tl = 0;
-      bool ok = true;
-      for (int tile = tile0; tile < ntiles && ok; tile += tile_step, ++tl) {
-        const uint32_t a = tl & 1, aph = (tl >> 1) & 1;
-        if (!mbar_wait(&tempty[a], aph ^ 1, abort_flag)) { ok = false; break; }
+    const uint32_t idesc = TF32 ? umma_idesc_tf32(BM, p.bn) : umma_idesc_bf16(BM, p.bn);
+    uint32_t s = 0, ph = 0, tl = 0;
+    bool ok = true;
+    for (int tile = tile0; tile < ntiles && ok; tile += tile_step, ++tl) {
+      const uint32_t a = tl & 1, aph = (tl >> 1) & 1;
+      if (!mbar_wait_warp(&tempty[a], aph ^ 1, abort_flag)) { ok = false; break; }
+      tc_fence_after();
+      const uint32_t d_tmem = tmem_base + a * BN;
+      for (int kb = 0; kb < kend - kbeg; ++kb) {
+        if (!mbar_wait_warp(&full[s], ph, abort_flag)) { ok = false; break; }
         tc_fence_after();
-        const uint32_t d_tmem = tmem_base + a * BN;
-        for (int kb = 0; kb < kend - kbeg; ++kb) {
-          if (!mbar_wait(&full[s], ph, abort_flag)) { ok = false; break; }
-          tc_fence_after();
+        if (elect_one()) {
           const uint64_t da = umma_desc_k128(smem_u32(smem + s * stage_bytes));
           const uint64_t db = umma_desc_k128(smem_u32(smem + s * stage_bytes + kBytesA));
 #pragma unroll
@@ -156,10 +156,10 @@ forward_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
             else umma_bf16(d_tmem, da + adv, db + adv, idesc, (kb | k) != 0 ? 1u : 0u);
           }
           umma_commit(&empty[s]);          // the stage is free once these MMAs have read it
-          if (++s == static_cast<uint32_t>(ST)) { s = 0; ph ^= 1; }
         }
-        if (ok) umma_commit(&tfull[a]);    // the accumulator is complete once every MMA of the tile is
+        if (++s == static_cast<uint32_t>(ST)) { s = 0; ph ^= 1; }
       }
+      if (ok && elect_one()) umma_commit(&tfull[a]);    // the accumulator is complete once every MMA of the tile is
     }
   } else {
     // ---------------- epilogue: warps 2..5, TMEM lane quarter q ----------------

@@ -116,7 +116,7 @@ update_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + kBars);
   volatile uint32_t* abort_flag = tmem_slot + 1;
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_index(), lane = threadIdx.x & 31;
   const uint32_t rank = cluster_ctarank();
   const int pair = blockIdx.x >> 1, npairs = gridDim.x >> 1;
   const int ntiles = p.tilesM * p.tilesN;
@@ -146,29 +146,28 @@ update_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
 
   if (warp == 0) {
     // ---------------- TMA producer (each CTA loads its own rows of U^T and its own half of the V^T rows) ---------
-    if (lane == 0) {
-      const uint64_t pol_keep = policy_evict_last(), pol_norm = policy_evict_normal();
-      uint32_t it = 0;
-      bool ok = true;
-      for (int tl = 0; tl < my_tiles && ok; ++tl) {
-        int m0, n0;
-        tile_origin(p, pair + tl * npairs, m0, n0);
-        for (int seg = 0; seg < p.nseg && ok; ++seg) {
-          for (int kl = 0; kl < p.kseg; ++kl, ++it) {
-            const uint32_t s = it % kStages, ph = (it / kStages) & 1;
-            if (!mbar_wait(&empty[s], ph ^ 1, abort_flag)) { ok = false; break; }
+    const uint64_t pol_keep = policy_evict_last(), pol_norm = policy_evict_normal();
+    uint32_t it = 0;
+    bool ok = true;
+    for (int tl = 0; tl < my_tiles && ok; ++tl) {
+      int m0, n0;
+      tile_origin(p, pair + tl * npairs, m0, n0);
+      const int ma = m0 + static_cast<int>(rank) * UM, nb = n0 + static_cast<int>(rank) * half;
+      for (int seg = 0; seg < p.nseg && ok; ++seg) {
+        const int xa = seg == 0 ? p.a_off0 : seg == 1 ? p.a_off1 : p.a_off2;
+        const int xb = seg == 0 ? p.b_off0 : seg == 1 ? p.b_off1 : p.b_off2;
+        for (int kl = 0; kl < p.kseg; ++kl, ++it) {
+          const uint32_t s = it % kStages, ph = (it / kStages) & 1;
+          if (!mbar_wait_warp(&empty[s], ph ^ 1, abort_flag)) { ok = false; break; }
+          if (elect_one()) {
             if (rank == 0) mbar_expect_tx(&full[s], 2 * (kBytesA + half * UK * 2));
             const uint32_t full_leader = mapa_u32(smem_u32(&full[s]), 0);
-            const int xa = seg == 0 ? p.a_off0 : seg == 1 ? p.a_off1 : p.a_off2;
-            const int xb = seg == 0 ? p.b_off0 : seg == 1 ? p.b_off1 : p.b_off2;
-            const int ma = m0 + static_cast<int>(rank) * UM, nb = n0 + static_cast<int>(rank) * half;
             if (MN) {                          // boxes of 64 rows (columns) of W x 64 pairs
 #pragma unroll
               for (int h = 0; h < 2; ++h) {
                 tma_load_2d_pair(sA + s * kBytesA + h * (kBytesA / 2), &tmA, xa + ma + 64 * h, kl * UK, full_leader, pol_norm);
                 if (64 * h < half)
-                  tma_load_2d_pair(sB + s * kBytesB + h * (kBytesB / 2), &tmB, xb + nb + 64 * h, kl * UK, full_leader,
-                  pol_keep);
+                  tma_load_2d_pair(sB + s * kBytesB + h * (kBytesB / 2), &tmB, xb + nb + 64 * h, kl * UK, full_leader, pol_keep);
               }
             } else {
               tma_load_2d_pair(sA + s * kBytesA, &tmA, xa + kl * (UK / 2), ma, full_leader, pol_norm);
@@ -180,30 +179,32 @@ update_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
     }
   } else if (warp == 1) {
     // ---------------- MMA issuer: one thread of the leader CTA drives both SMs ----------------
-    if (lane == 0 && rank == 0) {
+    if (rank == 0) {
       const uint32_t idesc = TF32 ? umma_idesc_tf32(2 * UM, p.bn) : umma_idesc_bf16(2 * UM, p.bn) | kIdescMnMajor;
       uint32_t it = 0;
       bool ok = true;
       for (int tl = 0; tl < my_tiles && ok; ++tl) {
         const uint32_t a = tl & 1, aph = (tl >> 1) & 1;
-        if (!mbar_wait(&tempty[a], aph ^ 1, abort_flag)) { ok = false; break; }
+        if (!mbar_wait_warp(&tempty[a], aph ^ 1, abort_flag)) { ok = false; break; }
         tc_fence_after();
         const uint32_t d_tmem = tmem_base + a * UN;
         for (int kb = 0; kb < numK; ++kb, ++it) {
           const uint32_t s = it % kStages, ph = (it / kStages) & 1;
-          if (!mbar_wait(&full[s], ph, abort_flag)) { ok = false; break; }
+          if (!mbar_wait_warp(&full[s], ph, abort_flag)) { ok = false; break; }
           tc_fence_after();
-          const uint64_t da = MN ? umma_desc_mn128(smem_u32(sA + s * kBytesA)) : umma_desc_k128(smem_u32(sA + s * kBytesA));
-          const uint64_t db = MN ? umma_desc_mn128(smem_u32(sB + s * kBytesB)) : umma_desc_k128(smem_u32(sB + s * kBytesB));
+          if (elect_one()) {
+            const uint64_t da = MN ? umma_desc_mn128(smem_u32(sA + s * kBytesA)) : umma_desc_k128(smem_u32(sA + s * kBytesA));
+            const uint64_t db = MN ? umma_desc_mn128(smem_u32(sB + s * kBytesB)) : umma_desc_k128(smem_u32(sB + s * kBytesB));
 #pragma unroll
-          for (int k = 0; k < UK / UMMA_K; ++k) {          // four MMAs of 16 pairs (bf16) or 8 (tf32) each
-            const uint64_t adv = static_cast<uint64_t>(MN ? k * 2048 / 16 : k * 32 / 16);
-            if (TF32) umma_tf32_pair(d_tmem, da + adv, db + adv, idesc, (kb | k) != 0 ? 1u : 0u);
-            else umma_bf16_pair(d_tmem, da + adv, db + adv, idesc, (kb | k) != 0 ? 1u : 0u);
+            for (int k = 0; k < UK / UMMA_K; ++k) {          // four MMAs of 16 pairs (bf16) or 8 (tf32) each
+              const uint64_t adv = static_cast<uint64_t>(MN ? k * 2048 / 16 : k * 32 / 16);
+              if (TF32) umma_tf32_pair(d_tmem, da + adv, db + adv, idesc, (kb | k) != 0 ? 1u : 0u);
+              else umma_bf16_pair(d_tmem, da + adv, db + adv, idesc, (kb | k) != 0 ? 1u : 0u);
+            }
+            umma_commit_pair(&empty[s], 3);          // both CTAs' stage s is free once these MMAs have read it
           }
-          umma_commit_pair(&empty[s], 3);          // both CTAs' stage s is free once these MMAs have read it
         }
-        if (ok) umma_commit_pair(&tfull[a], 3);    // both CTAs' halves of the accumulator are complete
+        if (ok && elect_one()) umma_commit_pair(&tfull[a], 3);    // both CTAs' halves of the accumulator are complete
       }
     }
   } else {
@@ -419,7 +420,7 @@ update_split_kernel(const __grid_constant__ CUtensorMap tmU, const __grid_consta
   volatile uint32_t* abort_flag = tmem_slot + 1;
 
   const UpdParams& p = sp.t;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_index(), lane = threadIdx.x & 31;
   const uint32_t rank = cluster_ctarank();
   const int pair = blockIdx.x >> 1, npairs = gridDim.x >> 1;
   const int ntiles = p.tilesM * p.tilesN;
@@ -448,17 +449,17 @@ update_split_kernel(const __grid_constant__ CUtensorMap tmU, const __grid_consta
 
   if (warp == 0) {
     // ---------------- TMA producer: U_hi, U_lo, V_hi, V_lo of a k-block, boxes of 64 columns ----------------
-    if (lane == 0) {
-      const uint64_t pol_keep = policy_evict_last(), pol_norm = policy_evict_normal();
-      uint32_t it = 0;
-      bool ok = true;
-      for (int tl = 0; tl < my_tiles && ok; ++tl) {
-        int m0, n0;
-        tile_origin(p, pair + tl * npairs, m0, n0);
-        const int mu = m0 + static_cast<int>(rank) * UM, nv = n0 + static_cast<int>(rank) * half;
-        for (int kb = 0; kb < nk; ++kb, ++it) {
-          const uint32_t s = it % SU_STAGES, ph = (it / SU_STAGES) & 1;
-          if (!mbar_wait(&empty[s], ph ^ 1, abort_flag)) { ok = false; break; }
+    const uint64_t pol_keep = policy_evict_last(), pol_norm = policy_evict_normal();
+    uint32_t it = 0;
+    bool ok = true;
+    for (int tl = 0; tl < my_tiles && ok; ++tl) {
+      int m0, n0;
+      tile_origin(p, pair + tl * npairs, m0, n0);
+      const int mu = m0 + static_cast<int>(rank) * UM, nv = n0 + static_cast<int>(rank) * half;
+      for (int kb = 0; kb < nk; ++kb, ++it) {
+        const uint32_t s = it % SU_STAGES, ph = (it / SU_STAGES) & 1;
+        if (!mbar_wait_warp(&empty[s], ph ^ 1, abort_flag)) { ok = false; break; }
+        if (elect_one()) {
           if (rank == 0) mbar_expect_tx(&full[s], 2 * (2 * kSuBytes + 2 * half * SU_UK * 2));
           const uint32_t bar = mapa_u32(smem_u32(&full[s]), 0);
           uint8_t* st = smem + s * kSuStage;
@@ -476,7 +477,7 @@ update_split_kernel(const __grid_constant__ CUtensorMap tmU, const __grid_consta
     }
   } else if (warp == 1) {
     // ---------------- MMA issuer: one thread of the leader CTA ----------------
-    if (lane == 0 && rank == 0) {
+    if (rank == 0) {
       const uint32_t idesc = (sp.fp16 ? umma_idesc_fp16(2 * UM, p.bn) : umma_idesc_bf16(2 * UM, p.bn)) | kIdescMnMajor;
       const uint32_t d_main = tmem_base, d_cross = tmem_base + UN;
       uint32_t it = 0, g = 0;
@@ -485,34 +486,37 @@ update_split_kernel(const __grid_constant__ CUtensorMap tmU, const __grid_consta
         for (int kb = 0; kb < nk; ++kb, ++it) {
           const uint32_t s = it % SU_STAGES, ph = (it / SU_STAGES) & 1;
           const int kc = kb % SU_DRAIN;
-          if (!mbar_wait(&full[s], ph, abort_flag)) { ok = false; break; }
-          if (kc == 0 && !mbar_wait(mempty, (g & 1) ^ 1, abort_flag)) { ok = false; break; }
+          if (!mbar_wait_warp(&full[s], ph, abort_flag)) { ok = false; break; }
+          if (kc == 0 && !mbar_wait_warp(mempty, (g & 1) ^ 1, abort_flag)) { ok = false; break; }
           tc_fence_after();
           uint8_t* st = smem + s * kSuStage;
           const uint64_t duh = umma_desc_mn128(smem_u32(st), kSuBox), dul = umma_desc_mn128(smem_u32(st + kSuBytes), kSuBox);
           const uint64_t dvh = umma_desc_mn128(smem_u32(st + 2 * kSuBytes), kSuBox), dvl = umma_desc_mn128(smem_u32(st + 3 * kSuBytes), kSuBox);
+          const bool drained = kc == SU_DRAIN - 1 || kb + 1 == nk;
+          if (elect_one()) {
 #pragma unroll
-          for (int k = 0; k < SU_UK / UMMA_K; ++k) {
-            const uint64_t adv = static_cast<uint64_t>(k * 2048 / 16);
-            umma_bf16_pair(d_main, duh + adv, dvh + adv, idesc, (kc | k) != 0 ? 1u : 0u);
+            for (int k = 0; k < SU_UK / UMMA_K; ++k) {
+              const uint64_t adv = static_cast<uint64_t>(k * 2048 / 16);
+              umma_bf16_pair(d_main, duh + adv, dvh + adv, idesc, (kc | k) != 0 ? 1u : 0u);
+            }
+            if (drained) umma_commit_pair(mfull, 3);
           }
-          if (kc == SU_DRAIN - 1 || kb + 1 == nk) {
-            umma_commit_pair(mfull, 3);
-            ++g;
-          }
+          if (drained) ++g;
           if (kb == 0) {
-            if (!mbar_wait(cempty, (tl & 1) ^ 1, abort_flag)) { ok = false; break; }
+            if (!mbar_wait_warp(cempty, (tl & 1) ^ 1, abort_flag)) { ok = false; break; }
             tc_fence_after();
           }
+          if (elect_one()) {
 #pragma unroll
-          for (int k = 0; k < SU_UK / UMMA_K; ++k) {
-            const uint64_t adv = static_cast<uint64_t>(k * 2048 / 16);
-            umma_bf16_pair(d_cross, dul + adv, dvh + adv, idesc, (kb | k) != 0 ? 1u : 0u);
-            umma_bf16_pair(d_cross, duh + adv, dvl + adv, idesc, 1u);
+            for (int k = 0; k < SU_UK / UMMA_K; ++k) {
+              const uint64_t adv = static_cast<uint64_t>(k * 2048 / 16);
+              umma_bf16_pair(d_cross, dul + adv, dvh + adv, idesc, (kb | k) != 0 ? 1u : 0u);
+              umma_bf16_pair(d_cross, duh + adv, dvl + adv, idesc, 1u);
+            }
+            umma_commit_pair(&empty[s], 3);
           }
-          umma_commit_pair(&empty[s], 3);
         }
-        if (ok) umma_commit_pair(cfull, 3);
+        if (ok && elect_one()) umma_commit_pair(cfull, 3);
       }
     }
   } else {
