@@ -159,6 +159,11 @@ __device__ __forceinline__ void tma_store_2d_hint(const CUtensorMap* m, const vo
                ::"l"(reinterpret_cast<uint64_t>(m)), "r"(smem_u32(src)), "r"(x), "r"(y), "l"(pol)
                : "memory");
 }
+__device__ __forceinline__ void tma_store_2d_at(const CUtensorMap* m, uint32_t src, int32_t x, int32_t y, uint64_t pol) {
+  asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group.L2::cache_hint [%0, {%2, %3}], [%1], %4;"
+               ::"l"(reinterpret_cast<uint64_t>(m)), "r"(src), "r"(x), "r"(y), "l"(pol)
+               : "memory");
+}
 __device__ __forceinline__ void tma_commit_group() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
 template <int N>
 __device__ __forceinline__ void tma_wait_group_read() {
@@ -316,6 +321,11 @@ __device__ __forceinline__ void tma_load_2d_at(uint32_t dst, const CUtensorMap* 
   asm volatile(
       "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
       ::"r"(dst), "l"(reinterpret_cast<uint64_t>(m)), "r"(smem_u32(bar)), "r"(x), "r"(y) : "memory");
+}
+// 32 bytes, a whole sector, from one lane (32-byte aligned)
+__device__ __forceinline__ void st_global_v8(void* dst, const uint32_t (&v)[16], int first) {
+  asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(dst), "r"(v[first]), "r"(v[first + 1]), "r"(v[first + 2]),
+               "r"(v[first + 3]), "r"(v[first + 4]), "r"(v[first + 5]), "r"(v[first + 6]), "r"(v[first + 7]) : "memory");
 }
 // Orders this thread's generic accesses (and what it has acquired) and asynchronous ones, in every state space.
 __device__ __forceinline__ void fence_proxy_async_all() { asm volatile("fence.proxy.async;" ::: "memory"); }

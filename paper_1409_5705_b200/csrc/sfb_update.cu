@@ -13,11 +13,11 @@
 // a sixth of a step of metric learning at 1,000 x 20,000).  The tf32 words are K-major (U^T, V^T).
 // Warps of a CTA: 0 = TMA producer, 1 = MMA issuer (leader CTA only) and TMEM owner, 2..9 = epilogue.
 // Epilogue warp (q, h): TMEM lane quarter q (32 rows of W), column half h (128 columns), in four chunks of
-// 32 x 32.  Each warp owns a ring of three 4 KB slots: the W chunk lands there by TMA (two chunks in flight per
-// warp, 64 KB per SM), is combined in place with the accumulator chunk and goes back by TMA from the same slot;
-// the bf16 copy of the new chunk is read back from the slot and stored as 64-byte row pieces.  Shared memory is
-// the scarce resource: 4 operand stages (128 KB) + the rings (96 KB).  Measured: a fourth operand stage gains
-// more (the operand loads slow down when they share L2 with the stream of W) than a fourth ring slot.
+// 32 x 32.  Each warp owns a ring of 4 KB slots: the W chunk lands there by TMA (two chunks in flight per warp, 64 KB per SM, or
+// four), is combined in place with the accumulator chunk and goes back by TMA from the same slot; a lane has a row of the
+// chunk and stores its 32 roundings of the bf16 copy as two sectors.  (The copy by rows, read back from the slot with 8 lanes a row,
+// was a third of a warp's chain per chunk: 10,000 x 20,000, 64 pairs 480 us of the pass, 420 without, 374 where few rows change.)
+// Shared memory is the scarce resource: see UpShape.
 #include <cuda.h>
 #include <cuda_bf16.h>
 
@@ -25,6 +25,7 @@
 
 #include "sfb_ptx.cuh"
 #include "sfb_tc.h"
+#include "sfb_tile.cuh"
 
 namespace sfb {
 namespace {
@@ -34,19 +35,26 @@ using namespace ptx;
 constexpr int UM = 128;                 // rows of W per CTA (256 per pair)
 constexpr int UN = 256;                 // columns of W per tile, at most (128 for small matrices, see tile_width)
 constexpr int UK = 64, UMMA_K = 16;
-constexpr int kStages = 4;
 constexpr int kBytesA = UM * UK * 2;          // 16 KB: this CTA's rows of U^T
 constexpr int kBytesB = (UN / 2) * UK * 2;    // 16 KB: this CTA's half of the V^T rows
 constexpr int kStageBytes = kBytesA + kBytesB;
 constexpr int kChunk = 32;
 constexpr int kSlotBytes = 32 * kChunk * 4;   // 4 KB
-constexpr int kRing = 3;                      // slots per epilogue warp
 constexpr int kPend = 1;                      // TMA stores of a warp that may still be reading their slots
 constexpr int kEpiWarps = 8;
 constexpr int kThreads = 64 + 32 * kEpiWarps;
 constexpr int kTmemCols = 512;
-constexpr int kBars = 2 * kStages + 4 + kEpiWarps * kRing;
-constexpr int kSmem = kStages * kStageBytes + kEpiWarps * kRing * kSlotBytes + kBars * 8 + 16 + 1024;
+// Two splits of the shared memory.  Many pairs: four operand stages and a ring of three slots per epilogue warp.  FEW pairs (up to
+// kFewPairs), where the pass over W is what takes the time: two stages and five slots.  us of the pass, 4 + 3 / 2 + 5, of
+// 10,000 x 20,000: 64 pairs 374 / 378, 192 388 / 381, 256 392 / 384, 320 391 / 393, 1,024 472 / 713; of 5,000 x 3,000 (in
+// L2): 64 pairs 38 / 33, 256 41 / 37.  (3 + 4: 1,024 pairs 552; 5 + 2: 64 pairs 480, 1,024 495.)
+constexpr int kFewPairs = 256;
+template <bool FEW>
+struct UpShape {
+  static constexpr int kStages = FEW ? 2 : 4, kRing = FEW ? 5 : 3;
+  static constexpr int kBars = 2 * kStages + 4 + kEpiWarps * kRing;
+  static constexpr int kSmem = kStages * kStageBytes + kEpiWarps * kRing * kSlotBytes + kBars * 8 + 16 + 1024;
+};
 
 struct UpdParams {
   int32_t rows, cols;          // shape of W
@@ -98,10 +106,11 @@ __device__ __forceinline__ void tile_origin(const UpdParams& p, int tile, int& m
 // TF32: the operands are 32-bit words read as tf32 (32 elements per 128-byte k-block), see the forward kernel.
 // SHADOW: the operand copy of the new W that the epilogue writes beside it for the next forward product:
 // 1 bf16, 2 the (big | small) pair of tf32 words of the fp32-on-tensor-cores mode.
-template <int SHADOW, bool TF32 = false>
+template <int SHADOW, bool TF32 = false, bool FEW = false>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
 update_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                    const __grid_constant__ CUtensorMap tmC, const UpdParams p) {
+  constexpr int kStages = UpShape<FEW>::kStages, kRing = UpShape<FEW>::kRing, kBars = UpShape<FEW>::kBars;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint8_t* sA = smem;
@@ -220,20 +229,21 @@ update_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
     const uint32_t tempty_leader0 = mapa_u32(smem_u32(&tempty[0]), 0), tempty_leader1 = mapa_u32(smem_u32(&tempty[1]), 0);
     const int row_in_tile = static_cast<int>(rank) * UM + q * 32;
     bool ok = true;
-    uint32_t copy_written = 0;           // row pieces of the bf16 copy this warp rewrote
-    uint32_t lg = 0;                     // next chunk to request
+    uint32_t copy_written = 0;           // row pieces of the bf16 copy this lane rewrote
+    uint32_t lg = 0;                     // next chunk to request, by the whole warp
+    int lm0 = 0, ln0 = 0;                // ... and its tile
     auto issue_load = [&]() {
       if (lg >= nchunks) return;
-      int m0, n0;
-      tile_origin(p, pair + static_cast<int>(lg >> cshift) * npairs, m0, n0);
+      if ((lg & (cpw - 1)) == 0) tile_origin(p, pair + static_cast<int>(lg >> cshift) * npairs, lm0, ln0);
       const uint32_t slot = lg % kRing;
-      mbar_expect_tx(&rf[slot], kSlotBytes);
-      tma_load_2d_hint(ring + slot * kSlotBytes, &tmC, n0 + h * half + static_cast<int>(lg & (cpw - 1)) * kChunk,
-                       m0 + row_in_tile, &rf[slot], pol_w);
+      if (elect_one()) {
+        mbar_expect_tx(&rf[slot], kSlotBytes);
+        tma_load_2d_hint(ring + slot * kSlotBytes, &tmC, ln0 + h * half + static_cast<int>(lg & (cpw - 1)) * kChunk,
+                         lm0 + row_in_tile, &rf[slot], pol_w);
+      }
       ++lg;
     };
-    if (lane == 0)
-      for (int i = 0; i < kRing - kPend; ++i) issue_load();
+    for (int i = 0; i < kRing - kPend; ++i) issue_load();
     uint32_t g = 0;
     for (int tl = 0; tl < my_tiles && ok; ++tl) {
       int m0, n0;
@@ -255,46 +265,52 @@ update_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
           if (lane == 0) mbar_arrive_cluster(a ? tempty_leader1 : tempty_leader0);
         }
         const uint32_t rs = g % kRing;
-        uint8_t* sl = ring + rs * kSlotBytes;
+        const uint32_t sl = smem_u32(ring + rs * kSlotBytes);
         const int x0 = n0 + h * half + c * kChunk;
         if (!__all_sync(0xffffffffu, mbar_wait(&rf[rs], (g / kRing) & 1, abort_flag))) return false;
-        uint32_t differs = 0;      // SHADOW == 1: does the bf16 rounding of any of this row's 32 values change?
+        // All of the row's reads, then the arithmetic, then the writes: with two epilogue warps to a scheduler a chunk's time is its
+        // chain of latencies.
+        float4 w[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) w[j] = ld_shared_f4(slot_addr(sl, lane, j));
+        uint32_t now[16];          // SHADOW == 1: the bf16 rounding of this row's 32 new values
+        uint32_t differs = 0;      //   does any of them change?
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
-          float4* wp = reinterpret_cast<float4*>(sl + lane * 128 + ((j ^ (lane & 7)) << 4));
-          float4 w = *wp;
           uint32_t o01 = 0, o23 = 0;
-          if (SHADOW == 1) { o01 = pack2(w.x, w.y); o23 = pack2(w.z, w.w); }
-          w.x = fmaf(p.alpha, __uint_as_float(acc[4 * j + 0]), w.x);
-          w.y = fmaf(p.alpha, __uint_as_float(acc[4 * j + 1]), w.y);
-          w.z = fmaf(p.alpha, __uint_as_float(acc[4 * j + 2]), w.z);
-          w.w = fmaf(p.alpha, __uint_as_float(acc[4 * j + 3]), w.w);
+          if (SHADOW == 1) { o01 = pack2(w[j].x, w[j].y); o23 = pack2(w[j].z, w[j].w); }
+          w[j].x = fmaf(p.alpha, __uint_as_float(acc[4 * j + 0]), w[j].x);
+          w[j].y = fmaf(p.alpha, __uint_as_float(acc[4 * j + 1]), w[j].y);
+          w[j].z = fmaf(p.alpha, __uint_as_float(acc[4 * j + 2]), w[j].z);
+          w[j].w = fmaf(p.alpha, __uint_as_float(acc[4 * j + 3]), w[j].w);
           if (p.prox_kind != 0) {
-            w.x = prox_entry(w.x, p.prox_kind, p.prox_a); w.y = prox_entry(w.y, p.prox_kind, p.prox_a);
-            w.z = prox_entry(w.z, p.prox_kind, p.prox_a); w.w = prox_entry(w.w, p.prox_kind, p.prox_a);
+            w[j].x = prox_entry(w[j].x, p.prox_kind, p.prox_a); w[j].y = prox_entry(w[j].y, p.prox_kind, p.prox_a);
+            w[j].z = prox_entry(w[j].z, p.prox_kind, p.prox_a); w[j].w = prox_entry(w[j].w, p.prox_kind, p.prox_a);
           }
-          *wp = w;
-          if (SHADOW == 1) differs |= (o01 ^ pack2(w.x, w.y)) | (o23 ^ pack2(w.z, w.w));
+          if (SHADOW == 1) {
+            now[2 * j] = pack2(w[j].x, w[j].y);
+            now[2 * j + 1] = pack2(w[j].z, w[j].w);
+            differs |= (o01 ^ now[2 * j]) | (o23 ^ now[2 * j + 1]);
+          }
         }
-        // The bf16 copy holds bf16(W) when the pass starts (set-up, refresh and this kernel keep it so): a
-        // row piece whose 32 roundings all stay the same already holds bf16 of the new values and is not rewritten.
-        // With updates of a few fp32 spacings per entry that is most of the matrix; the copy stays exact either way.
-        const uint32_t rowmask = SHADOW == 1 ? __ballot_sync(0xffffffffu, differs != 0) : 0u;
+#pragma unroll
+        for (int j = 0; j < 8; ++j) st_shared_f4(slot_addr(sl, lane, j), w[j]);
         fence_proxy_async_smem();
         __syncwarp();                                        // every lane has rewritten its row of the slot
-        if (lane == 0) {
-          if (x0 < p.cols && y0 < p.rows) tma_store_2d_hint(&tmC, sl, x0, y0, pol_w);
+        if (elect_one()) {                                   // (the same lane every time: bulk groups are a thread's)
+          if (x0 < p.cols && y0 < p.rows) tma_store_2d_at(&tmC, sl, x0, y0, pol_w);
           tma_commit_group();
           if (g >= kPend) tma_wait_group_read<kPend>();      // the store of chunk g-kPend has read its slot:
-          issue_load();                                      // refill it with chunk g + kRing - kPend
         }
+        __syncwarp();
+        issue_load();                                        // refill it with chunk g + kRing - kPend
         if (SHADOW == 2) {
           // (big | small) tf32 copy of the chunk, read back from the slot with 8 lanes per row: 128-byte row pieces
           const int sub = lane >> 3, jj = lane & 7;
 #pragma unroll
           for (int r0 = 0; r0 < 32; r0 += 4) {
             const int r = r0 + sub;
-            const float4 w = *reinterpret_cast<const float4*>(sl + r * 128 + ((jj ^ (r & 7)) << 4));
+            const float4 w = ld_shared_f4(slot_addr(sl, r, jj));
             const int col = x0 + 4 * jj;
             if (y0 + r < p.rows && col < p.cols) {
               const float4 b = make_float4(to_tf32(w.x), to_tf32(w.y), to_tf32(w.z), to_tf32(w.w));
@@ -306,37 +322,17 @@ update_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
           }
         }
         if (SHADOW == 1) {
-          // bf16 copy of the chunk, read back from the slot with 8 lanes per row (4 rows per pass): each row's
-          // 32 values leave as one 64-byte piece instead of 32 lanes storing 16 bytes to 32 different rows.
-          const int sub = lane >> 3, jj = lane & 7;
-          if (__popc(rowmask) > 12) {
-            // most rows changed: all 32 in eight fixed passes (cheaper than picking them one by one)
-            copy_written += 32;
-#pragma unroll
-            for (int r0 = 0; r0 < 32; r0 += 4) {
-              const int r = r0 + sub;
-              const float4 w = *reinterpret_cast<const float4*>(sl + r * 128 + ((jj ^ (r & 7)) << 4));
-              const int col = x0 + 4 * jj;
-              if (y0 + r < p.rows && col < p.shadow_ld)
-                *reinterpret_cast<uint2*>(p.shadow + static_cast<int64_t>(y0 + r) * p.shadow_ld + col) =
-                    make_uint2(pack2(w.x, w.y), pack2(w.z, w.w));
-            }
-          } else {
-          copy_written += __popc(rowmask);
-          // the changed rows, four per pass: lane group `sub` takes the (sub+1)-th changed row still to do
-#pragma unroll 1
-          for (uint32_t todo = rowmask; todo != 0;) {
-            const uint32_t r = __fns(todo, 0, sub + 1);           // 0xffffffff when fewer than sub+1 rows are left
-            if (r < 32u) {
-              const float4 w = *reinterpret_cast<const float4*>(sl + r * 128 + ((jj ^ (r & 7)) << 4));
-              const int col = x0 + 4 * jj;
-              if (y0 + static_cast<int>(r) < p.rows && col < p.shadow_ld)
-                *reinterpret_cast<uint2*>(p.shadow + static_cast<int64_t>(y0 + r) * p.shadow_ld + col) =
-                    make_uint2(pack2(w.x, w.y), pack2(w.z, w.w));
-            }
-            todo &= todo - 1; todo &= todo - 1; todo &= todo - 1; todo &= todo - 1;    // drop the four lowest set bits
+          // The bf16 copy holds bf16(W) when the pass starts (set-up, refresh and this kernel keep it so): a row piece whose 32
+          // roundings all stay the same already holds bf16 of the new values and is not rewritten.  With updates of a few
+          // fp32 spacings per entry that is most of the matrix; the copy stays exact either way.  (x0 and the copy's pitch are
+          // multiples of 32: a piece is inside or outside as a whole.)
+          const bool rewrite = differs != 0 && y0 + lane < p.rows && x0 < p.shadow_ld;
+          if (rewrite) {
+            __nv_bfloat16* d = p.shadow + static_cast<int64_t>(y0 + lane) * p.shadow_ld + x0;
+            st_global_v8(d, now, 0);
+            st_global_v8(d + 16, now, 8);
           }
-          }
+          copy_written += rewrite;
         }
         ++g;
         return true;
@@ -347,10 +343,13 @@ update_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
         if (ok) ok = process(acc1, acc0, c + 1);
       }
     }
-    if (lane == 0) tma_wait_group<0>();
-    if (SHADOW == 1 && lane == 0 && p.copy_counters) {
-      atomicAdd(&p.copy_counters[0], 32ull * nchunks);
-      atomicAdd(&p.copy_counters[1], static_cast<unsigned long long>(copy_written));
+    if (elect_one()) tma_wait_group<0>();
+    if (SHADOW == 1 && p.copy_counters) {
+      const uint32_t written = __reduce_add_sync(0xffffffffu, copy_written);
+      if (lane == 0) {
+        atomicAdd(&p.copy_counters[0], 32ull * nchunks);
+        atomicAdd(&p.copy_counters[1], static_cast<unsigned long long>(written));
+      }
     }
   }
 
@@ -627,7 +626,8 @@ update_split_kernel(const __grid_constant__ CUtensorMap tmU, const __grid_consta
 
 // Tile width: 128 where 256-wide tiles leave the pairs short of work.  Cycles of a tile: its k-blocks at the MMA or operand
 // rate (measured about 620 a k-block of 64 pairs for 256 columns, 450 for 128; 1600 and 900 with four operand halves) and its
-// epilogue.
+// epilogue.  (Counted with the cycles of the pass over W instead, more shapes take 128, whose half rows it moves more slowly: 4,999 x
+// 3,004 with 259 pairs 36.7 -> 41.9 us, 30,000 x 500 with 300 42 -> 50.)
 int tile_width(int64_t rows, int64_t cols, int64_t kblocks, int pairs, bool split) {
   auto cost = [&](int bn) {
     const int64_t tiles = ((rows + 2 * UM - 1) / (2 * UM)) * ((cols + bn - 1) / bn);
@@ -670,10 +670,11 @@ static cudaError_t prepare_kernel(Kernel kernel, int smem, int* max_pairs) {
 
 int tc_update_init(sfb_ctx* ctx, TcState* st) {
   int n = 1 << 30;
-  CKC(prepare_kernel(update_pair_kernel<1>, kSmem, &n));
+  CKC(prepare_kernel(update_pair_kernel<1>, UpShape<false>::kSmem, &n));
+  CKC(prepare_kernel(update_pair_kernel<1, false, true>, UpShape<true>::kSmem, &n));
   CKC(prepare_kernel(update_split_kernel<false>, SuShape<false>::kSmem, &n));
   CKC(prepare_kernel(update_split_kernel<true>, SuShape<true>::kSmem, &n));
-  CKC(prepare_kernel(update_pair_kernel<2, true>, kSmem, &n));
+  CKC(prepare_kernel(update_pair_kernel<2, true>, UpShape<false>::kSmem, &n));
   st->max_pairs = n;
   if (n < 1) return SFB_ERR_ARCH;                 // the device cannot host a CTA pair of these kernels
   return SFB_OK;
@@ -713,7 +714,7 @@ int tc32_update(sfb_ctx* ctx) {
   p.shadow = nullptr; p.shadow32 = ctx->at<float>(L.Ws); p.shadow_ld = 2 * L.colsp; p.shadow_half = L.colsp;
   const int64_t tiles = static_cast<int64_t>(p.tilesM) * p.tilesN;
   const unsigned grid = 2u * static_cast<unsigned>(std::min<int64_t>(tiles, st->max_pairs));
-  CKC(launch_kernel_if(tiles <= st->max_pairs, (update_pair_kernel<2, true>), dim3(grid), dim3(kThreads), kSmem, ctx->stream, 1, ma, mb, mc, p));
+  CKC(launch_kernel_if(tiles <= st->max_pairs, (update_pair_kernel<2, true>), dim3(grid), dim3(kThreads), UpShape<false>::kSmem, ctx->stream, 1, ma, mb, mc, p));
   return SFB_OK;
 }
 
@@ -763,7 +764,11 @@ int tc_update(sfb_ctx* ctx) {
   p.nseg = 1;
   p.shadow = ctx->at<__nv_bfloat16>(L.Wb); p.shadow_ld = L.colsb;
   p.copy_counters = &ctx->at<Scalars>(L.scalars)->copy_pieces;
-  CKC(launch_kernel_if(tiles <= st->max_pairs, update_pair_kernel<1>, dim3(grid), dim3(kThreads), kSmem, ctx->stream, 1, ma, mb, mc, p));
+  CKC(ctx->K <= kFewPairs
+          ? launch_kernel_if(tiles <= st->max_pairs, (update_pair_kernel<1, false, true>), dim3(grid), dim3(kThreads),
+                             UpShape<true>::kSmem, ctx->stream, 1, ma, mb, mc, p)
+          : launch_kernel_if(tiles <= st->max_pairs, update_pair_kernel<1>, dim3(grid), dim3(kThreads), UpShape<false>::kSmem,
+                             ctx->stream, 1, ma, mb, mc, p));
   return SFB_OK;
 }
 

@@ -1,0 +1,40 @@
+"""Regression in bf16 mode at the sizes where the choice of its kernels changes and their tiles end, against the oracle at the mode's
+tolerance; the operand copy of W must be bf16(W) bit for bit after the step."""
+import pytest
+
+import paper_1409_5705_b200 as S
+import sfb_inputs as I
+from _parity import TOL, config_for, oracle_step, rel_err, to_dev
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+
+
+def check(rows, cols, workers, batch, per_worker=False):
+    wl = I.scaled(I.WORKLOADS["mlr_mid"], "mlr_forms", rows=rows, cols=cols, workers=workers, batch=batch, w_std=0.05,
+                  x_scale="unit", eta=0.05)
+    W0, inp = I.initial_W(wl), I.step_inputs(wl, 1)
+    W = to_dev(W0, torch)
+    ctx = S.Context(config_for(wl, S.PREC_BF16), W)
+    X, lab = to_dev(inp.X, torch), to_dev(inp.labels, torch)
+    if per_worker:
+        for p in reversed(range(workers)):
+            r = slice(p * batch, (p + 1) * batch)
+            ctx.sfb_compute_factors(p, X[r], None, lab[r])
+        ctx.sfb_gather_factors()
+        ctx.sfb_apply_update()
+    else:
+        ctx.sfb_step(X, None, lab)
+    assert ctx.sfb_get_status() == 0
+    assert torch.equal(ctx.operand_copy_as_tensor()[:, :cols], W.to(torch.bfloat16))
+    Wg = W.cpu().numpy()
+    ctx.close()
+    err = rel_err(Wg, oracle_step(wl, W0, inp), W0)
+    print(f"{rows} x {cols} K={wl.K}: rel err {err:.3e}")
+    assert err <= TOL[S.PREC_BF16]
+
+
+# The two forms of the update (256 and 257 pairs), one ragged tile, one row more than a tile, several tiles per pair of CTAs.
+@pytest.mark.parametrize("shape", [(5, 4, 1, 1), (257, 260, 4, 64), (257, 260, 1, 257), (1030, 2500, 5, 51), (6001, 2052, 2, 120)])
+def test_update_forms(shape):
+    check(*shape)
