@@ -1,0 +1,345 @@
+// Logits of multiclass logistic regression in bf16 mode for more than 128 samples, on pairs of CTAs:  Z (samples x rows of W) = X W^T
+// with the softmax partials of each sample.  (Fewer samples, and the tf32 words: forward_kernel in sfb_tc.cu.)
+//
+// A pair (cta_group::2) owns a tile of 256 samples x bn classes, a CTA 128 of the samples in its TMEM; it loads its own samples and its
+// half of the classes, 32 KB a k-block where a CTA with a 128 x 256 tile of its own loads 48 KB.  Two accumulators: the end of a
+// tile runs beside the next one's products.
+// What bounds the product is the MMA, as long as no pair waits: 160 tiles of 10,000 x 20,000 with 1,024 samples are 2.2 rounds of the
+// 74 pairs, and a third round for twelve tiles took 85 of 390 us.  So the tiles of all rounds but the last whole one are taken
+// whole, in step (the tiles that run at the same time share a block of W), and the k-blocks of the rest are shared out evenly, at
+// most two tiles a pair and few parts a tile (Segments in sfb_tile.cuh).
+// Warps: 0 TMA producer, 1 MMA issuer (leader CTA) and TMEM owner, 2..9 epilogue (TMEM lane quarter q, half h of the columns).
+#include <cuda.h>
+#include <cuda_bf16.h>
+
+#include <algorithm>
+
+#include "sfb_tc.h"
+#include "sfb_tile.cuh"
+
+namespace sfb {
+namespace {
+
+using namespace ptx;
+
+constexpr int PM = 256, BM = 128, BK = 64, UMMA_K = 16;
+constexpr int kMaxN = 256, kChunk = 32, kEpi = 8;
+constexpr int kStages = 5, kRing = 2;               // operand stages; slots per epilogue warp for the chunks of Z on their way out
+constexpr int kInputs = 4;                          // parts of tiles on their way in, per epilogue warp
+constexpr int kBytesA = BM * BK * 2, kBytesB = (kMaxN / 2) * BK * 2, kStage = kBytesA + kBytesB;
+constexpr int kSlot = 32 * kChunk * 4;
+constexpr int kThreads = 64 + 32 * kEpi;
+constexpr int kBars = 2 * kStages + 4 + kEpi * kInputs;
+constexpr int kSmem = kStages * kStage + kEpi * kRing * kSlot + kBars * 8 + 16 + 1024;
+constexpr int kTmemCols = 512;
+static_assert(kEpi * kInputs * kSlot <= kStages * kStage, "the parts land in the operand ring");
+
+struct PairParams {
+  int32_t M, N, m_off;         // samples end at M and begin at m_off; classes
+  int32_t tilesM, tilesN, bn;  // tiles of 256 samples x bn classes, bn a multiple of 64
+  int32_t kseg;                // k-blocks
+  int32_t cut, whole;          // see Segments
+  float2* part;                // [ceil(N / (bn / 2))][part_ld] (max, sum exp) per sample and half a tile's classes
+  int64_t part_ld;
+  float* partial;              // [pairs][2][kEpi][4] slots: what a pair leaves of a tile that another one completes ...
+  uint32_t* ready;             // [pairs][2][kEpi]: ... and that it is there
+  uint32_t* status;
+};
+
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
+forward_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
+                    const __grid_constant__ CUtensorMap tmC, const __grid_constant__ PairParams p) {
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  uint8_t* sRing = smem + kStages * kStage;
+  uint64_t* bars = reinterpret_cast<uint64_t*>(sRing + kEpi * kRing * kSlot);
+  uint64_t* full = bars;                             // full, tempty: the leader's are in use
+  uint64_t* empty = bars + kStages;
+  uint64_t* tfull = bars + 2 * kStages;
+  uint64_t* tempty = tfull + 2;
+  uint64_t* ifull = tfull + 4;                       // per epilogue warp and input buffer
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + kBars);
+  volatile uint32_t* abort_flag = tmem_slot + 1;
+
+  const int warp = warp_index(), lane = threadIdx.x & 31;
+  const uint32_t rank = cluster_ctarank();
+  const int pair = blockIdx.x >> 1, half = p.bn / 2;
+  const Segments segs(p.kseg, p.cut != 0, p.whole, p.tilesM * p.tilesN, pair, gridDim.x >> 1);
+  // Sample block fastest: the tiles that run at the same time share blocks of W.
+  auto tile_coords = [&](int tile, int& m0, int& n0) {
+    const int tn = tile / p.tilesM;
+    m0 = p.m_off + (tile - tn * p.tilesM) * PM;
+    n0 = tn * p.bn;
+  };
+  pdl_launch_dependents();
+
+  if (threadIdx.x == 0) {
+    for (int i = 0; i < kStages; ++i) { mbar_init(&full[i], 1); mbar_init(&empty[i], 1); }
+    for (int i = 0; i < 2; ++i) { mbar_init(&tfull[i], 1); mbar_init(&tempty[i], 2 * kEpi); }
+    for (int i = 0; i < kEpi * kInputs; ++i) mbar_init(&ifull[i], 1);
+    *abort_flag = 0;
+    fence_barrier_init();
+    prefetch_tmap(&tmA); prefetch_tmap(&tmB); prefetch_tmap(&tmC);
+  }
+  if (warp == 1) { tmem_alloc_pair(tmem_slot, kTmemCols); tmem_relinquish_pair(); }
+  tc_fence_before();
+  __syncthreads();
+  cluster_arrive();          // both CTAs' barriers exist and both have their TMEM before anyone signals the peer
+  cluster_wait();
+  tc_fence_after();
+  const uint32_t tmem_base = *tmem_slot;
+  pdl_wait();
+
+  if (warp == 0) {
+    // ---------------- TMA producer ----------------
+    const uint64_t pol_keep = policy_evict_last(), pol_norm = policy_evict_normal();    // every tile reads the samples again
+    uint32_t s = 0, ph = 0;
+    bool ok = true;
+    for (int i = 0; i < segs.n && ok; ++i) {
+      const Segment sg = segs.get(i);
+      int m0, n0;
+      tile_coords(sg.tile, m0, n0);
+      const int ma = m0 + static_cast<int>(rank) * BM, nb = n0 + static_cast<int>(rank) * half;
+      for (int k = sg.k0; k < sg.k1; ++k) {
+        if (!mbar_wait_warp(&empty[s], ph ^ 1, abort_flag)) { ok = false; break; }
+        if (elect_one()) {
+          if (rank == 0) mbar_expect_tx(&full[s], 2 * (kBytesA + half * BK * 2));
+          const uint32_t bar = mapa_u32(smem_u32(&full[s]), 0);
+          uint8_t* st = smem + s * kStage;
+          tma_load_2d_pair(st, &tmA, k * BK, ma, bar, pol_keep);
+          tma_load_2d_pair(st + kBytesA, &tmB, k * BK, nb, bar, pol_norm);
+        }
+        if (++s == static_cast<uint32_t>(kStages)) { s = 0; ph ^= 1; }
+      }
+    }
+  } else if (warp == 1) {
+    // ---------------- MMA issuer ----------------
+    if (rank == 0) {
+      const uint32_t idesc = umma_idesc_bf16(PM, p.bn);
+      uint32_t s = 0, ph = 0;
+      bool ok = true;
+      for (int i = 0; i < segs.n && ok; ++i) {
+        const Segment sg = segs.get(i);
+        const uint32_t a = i & 1, aph = (i >> 1) & 1, d_tmem = tmem_base + a * kMaxN;
+        if (!mbar_wait_warp(&tempty[a], aph ^ 1, abort_flag)) { ok = false; break; }
+        tc_fence_after();
+        for (int kb = 0; kb < sg.k1 - sg.k0; ++kb) {
+          if (!mbar_wait_warp(&full[s], ph, abort_flag)) { ok = false; break; }
+          tc_fence_after();
+          if (elect_one()) {
+            const uint64_t da = umma_desc_k128(smem_u32(smem + s * kStage)), db = umma_desc_k128(smem_u32(smem + s * kStage + kBytesA));
+#pragma unroll
+            for (int k = 0; k < BK / UMMA_K; ++k) {
+              const uint64_t adv = static_cast<uint64_t>(k * UMMA_K * 2 / 16);
+              umma_bf16_pair(d_tmem, da + adv, db + adv, idesc, (kb | k) != 0 ? 1u : 0u);
+            }
+            umma_commit_pair(&empty[s], 3);
+          }
+          if (++s == static_cast<uint32_t>(kStages)) { s = 0; ph ^= 1; }
+        }
+        if (ok && elect_one()) umma_commit_pair(&tfull[a], 3);
+      }
+    }
+  } else {
+    // ---------------- epilogue ----------------
+    const int e = warp - 2, q = warp & 3, h = e >> 2, cpw = half / kChunk;
+    const uint32_t ring = smem_u32(sRing + e * kRing * kSlot);
+    const int row0 = static_cast<int>(rank) * BM + q * 32;           // first of this warp's 32 samples within the tile
+    const int at = static_cast<int>(rank) * kEpi + e;
+    const uint32_t tempty_leader0 = mapa_u32(smem_u32(&tempty[0]), 0), tempty_leader1 = mapa_u32(smem_u32(&tempty[1]), 0);
+    uint32_t stores = 0;
+    bool ok = true;
+    // a chunk from registers (a sample per lane) to a slot, when the copy that last used the slot has read it
+    auto to_slot = [&](const uint32_t (&acc)[32]) {
+      const uint32_t sl = ring + (stores % kRing) * kSlot;
+      if (elect_one()) tma_wait_group_read<kRing - 1>();
+      __syncwarp();
+      slot_put(sl, lane, acc);
+      fence_proxy_async_smem();
+      __syncwarp();
+      ++stores;
+      return sl;
+    };
+    for (int i = 0; i < segs.n && ok; ++i) {
+      const Segment sg = segs.get(i);
+      int m0, n0;
+      tile_coords(sg.tile, m0, n0);
+      const uint32_t a = i & 1, aph = (i >> 1) & 1;
+      if (!__all_sync(0xffffffffu, mbar_wait(&tfull[a], aph, abort_flag))) { ok = false; break; }
+      tc_fence_after();
+      const uint32_t t_addr = tmem_base + (static_cast<uint32_t>(q * 32) << 16) + a * kMaxN + h * half;
+      const bool leave = sg.k1 < p.kseg;
+      const int from = leave ? pair : segs.first_part(sg), parts = pair - from, asks = parts * cpw;
+      // Parts of the tile from the pairs before this one (the last tile of a pair): their sums come by bulk copies, kInputs of them
+      // under way per warp, into the operand ring, which nothing uses any more.
+      const uint32_t room = smem_u32(smem) + e * kInputs * kSlot;
+      uint64_t* bar = ifull + e * kInputs;
+      int asked = 0;
+      auto ask = [&]() {                             // the next one: chunk by chunk, each from all of them in their order
+        if (asked >= asks) return;
+        const int c = asked / parts, w = asked - c * parts, b = asked % kInputs;
+        if (elect_one()) {
+          mbar_expect_tx(&bar[b], kSlot);
+          bulk_load(room + b * kSlot, p.partial + ((static_cast<int64_t>(from + w) * 2 * kEpi + at) * 4 + c) * (kSlot / 4), kSlot, &bar[b]);
+        }
+        ++asked;
+      };
+      if (parts > 0) {
+        for (int j = from; j < pair && ok; ++j) ok = __all_sync(0xffffffffu, lane != 0 || flag_wait(p.ready + j * 2 * kEpi + at, abort_flag));
+        if (!ok) break;
+        if (elect_one())
+          for (int j = from; j < pair; ++j) p.ready[j * 2 * kEpi + at] = 0;             // for the next launch
+        fence_proxy_async_all();
+        __syncwarp();
+        for (int b = 0; b < kInputs; ++b) ask();
+      }
+      float mx = -INFINITY, sum = 0.f;
+      int taken = 0;
+      const int row = m0 + row0 + lane;
+#pragma unroll 1
+      for (int c = 0; c < cpw && ok; ++c) {
+        uint32_t acc[32];
+        tmem_ld_32x32(t_addr + c * kChunk, acc);
+        tmem_ld_wait();
+        if (c + 1 == cpw) {                          // the last read of the accumulator: hand it back
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive_cluster(a ? tempty_leader1 : tempty_leader0);
+        }
+        if (leave) {
+          const uint32_t sl = to_slot(acc);
+          if (elect_one()) {
+            bulk_store(p.partial + ((static_cast<int64_t>(pair) * 2 * kEpi + at) * 4 + c) * (kSlot / 4), sl, kSlot);
+            tma_commit_group();
+          }
+          continue;
+        }
+        for (int w = 0; w < parts && ok; ++w, ++taken) {
+          const int b = taken % kInputs;
+          ok = __all_sync(0xffffffffu, mbar_wait(&bar[b], (taken / kInputs) & 1, abort_flag));
+          if (!ok) break;
+#pragma unroll
+          for (int j = 0; j < 8; ++j) {
+            const float4 t = ld_shared_f4(slot_addr(room + b * kSlot, lane, j));
+            acc[4 * j] = __float_as_uint(__uint_as_float(acc[4 * j]) + t.x);
+            acc[4 * j + 1] = __float_as_uint(__uint_as_float(acc[4 * j + 1]) + t.y);
+            acc[4 * j + 2] = __float_as_uint(__uint_as_float(acc[4 * j + 2]) + t.z);
+            acc[4 * j + 3] = __float_as_uint(__uint_as_float(acc[4 * j + 3]) + t.w);
+          }
+          __syncwarp();
+          ask();
+        }
+        if (!ok) break;
+        const int col0 = n0 + h * half + c * kChunk;
+        if (col0 >= p.N) continue;
+        // running (max, sum exp) of the sample over this warp's classes of the tile
+        float cm = -INFINITY;
+#pragma unroll
+        for (int j = 0; j < 32; ++j)
+          if (col0 + j < p.N) cm = fmaxf(cm, __uint_as_float(acc[j]));
+        const float nm = fmaxf(mx, cm);
+        float cs = 0.f;
+#pragma unroll
+        for (int j = 0; j < 32; ++j)
+          if (col0 + j < p.N) cs += __expf(__uint_as_float(acc[j]) - nm);
+        sum = sum * __expf(mx - nm) + cs;
+        mx = nm;
+        const uint32_t sl = to_slot(acc);
+        if (elect_one()) {
+          tma_store_2d_at(&tmC, sl, col0, m0 + row0);
+          tma_commit_group();
+        }
+      }
+      if (leave && ok) {
+        if (elect_one()) {
+          tma_wait_group<0>();
+          fence_proxy_async_all();
+          __threadfence();
+          st_release(p.ready + pair * 2 * kEpi + at, 1u);
+        }
+        __syncwarp();
+      } else if (ok && n0 + h * half < p.N && row < p.M) {
+        p.part[static_cast<int64_t>(n0 / half + h) * p.part_ld + row] = make_float2(mx, sum);
+      }
+    }
+    if (elect_one()) tma_wait_group<0>();
+  }
+
+  // ---------------- teardown ----------------
+  __syncwarp();
+  tc_fence_before();
+  __syncthreads();
+  if (*abort_flag) {
+    // A wait ran out: report it and give copies in flight a bounded time to land.
+    if (threadIdx.x == 0) atomicOr(p.status, SFB_STATUS_TIMEOUT);
+    for (int i = 0; i < 64; ++i) __nanosleep(1000);
+    __syncthreads();
+  }
+  cluster_arrive();          // neither CTA frees its TMEM or exits while the other may still signal or write it
+  cluster_wait();
+  if (warp == 1) { tc_fence_after(); tmem_dealloc_pair(tmem_base, kTmemCols); }
+}
+
+// Cycles of a plan: its k-blocks on a pair at the MMAs' rate or 60 bytes a cycle and SM, at least the 8,000 that the end of a tile of 256
+// classes takes; 7,000 from the start to the first MMA and from the last one to the results; 13,000 and 1,000 a part to leave and to
+// take over parts of tiles.  (Fitted to 47 shapes, 64 to 100,000 classes, 170 to 20,000 features, 129 to 1,024 samples: against
+// the best of forward_kernel, whole tiles and cut ones the choice loses 3 % in the middle of the factors' time, 31 % at most, of 12 us;
+// forward_kernel alone 11 %.  us of the product, forward_kernel / here: 10,000 x 20,000 with 1,024 samples 376 / 283, 11,133 x
+// 3,364 with 1,024 79 / 67.)
+constexpr int64_t kNarrowRows = 4096;               // up to which narrower tiles are looked at (they have more partials)
+struct PairPlan { int bn, cut, whole, pairs; double cost; };
+PairPlan plan_pairs(int64_t n, int64_t rows, int64_t cols, int64_t max_pairs) {
+  PairPlan best{};
+  const int64_t kseg = (cols + BK - 1) / BK, tm = (n + PM - 1) / PM;
+  for (int bn = kMaxN; bn >= (rows <= kNarrowRows ? 64 : kMaxN); bn -= 64) {
+    const int64_t tiles = tm * ((rows + bn - 1) / bn), rounds = (tiles + max_pairs - 1) / max_pairs, full = tiles / max_pairs;
+    const double per_kb = std::max(2.1 * bn, (BM + bn / 2) * BK * 2 / 60.0);
+    const double tile = std::max(static_cast<double>(kseg) * per_kb, 8000.0 * bn / kMaxN);
+    PairPlan p{bn, 0, 0, static_cast<int>(std::min(tiles, max_pairs)), static_cast<double>(rounds) * tile + 7000.0};
+    const int64_t whole = std::max<int64_t>(0, full - 1) * max_pairs, rest = tiles - whole;
+    const int64_t pairs = full > 0 ? max_pairs : std::max<int64_t>(1, std::min(max_pairs, rest * kseg / 4));
+    const int64_t shared = (rest * kseg + pairs - 1) / pairs;
+    const double cost = static_cast<double>(whole / max_pairs) * tile + static_cast<double>(shared) * per_kb + 20000.0 +
+                        1000.0 * static_cast<double>((pairs + rest - 1) / rest);
+    if (cost < p.cost && rest % pairs != 0) p = PairPlan{bn, 1, static_cast<int>(whole), static_cast<int>(pairs), cost};
+    if (bn == kMaxN || p.cost < 0.97 * best.cost) best = p;
+  }
+  return best;
+}
+PairPlan plan_pairs(const sfb_ctx* ctx, int64_t n) {
+  const int64_t most = std::min(static_cast<TcState*>(ctx->tc)->max_pairs, std::min(sm_count(), kModelSms) / 2);
+  return plan_pairs(n, ctx->cfg.rows, ctx->cfg.cols, most);
+}
+
+}  // namespace
+
+double forward_pair_cost(int64_t n, int64_t rows, int64_t cols) { return plan_pairs(n, rows, cols, kModelSms / 2).cost; }
+int64_t forward_pair_groups(int64_t rows) { return rows <= kNarrowRows ? (rows + 31) / 32 : (rows + kMaxN / 2 - 1) / (kMaxN / 2); }
+size_t forward_pair_partial_bytes() { return static_cast<size_t>(kModelSms / 2) * 2 * kEpi * 4 * kSlot; }
+size_t forward_pair_ready_bytes() { return static_cast<size_t>(kModelSms / 2) * 2 * kEpi * 4; }
+
+cudaError_t forward_pair_prepare(int* max_pairs) { return prepare_pair_kernel(forward_pair_kernel, kThreads, kSmem, max_pairs); }
+
+cudaError_t forward_pair(sfb_ctx* ctx, int64_t off, int64_t n, int* pw) {
+  TcState* st = static_cast<TcState*>(ctx->tc);
+  const Layout& L = ctx->lay;
+  const int64_t rows = ctx->cfg.rows, cols = ctx->cfg.cols;
+  const PairPlan plan = plan_pairs(ctx, n);
+  CUtensorMap ma, mb, mc;
+  if (!make_map(st, &ma, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, ctx->at<uint16_t>(L.Xb), cols, ctx->K, L.colsb * 2, BK, BM) ||
+      !make_map(st, &mb, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, ctx->at<uint16_t>(L.Wb), cols, rows, L.colsb * 2, BK, plan.bn / 2) ||
+      !make_map(st, &mc, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, ctx->at<float>(L.ZT), rows, off + n, round_up(rows, 32) * 4, kChunk, 32))
+    return cudaErrorInvalidValue;
+  PairParams p{};
+  p.M = static_cast<int32_t>(off + n); p.N = static_cast<int32_t>(rows); p.m_off = static_cast<int32_t>(off);
+  p.tilesM = static_cast<int32_t>((n + PM - 1) / PM); p.tilesN = static_cast<int32_t>((rows + plan.bn - 1) / plan.bn);
+  p.bn = plan.bn; p.kseg = static_cast<int32_t>((cols + BK - 1) / BK);
+  p.cut = plan.cut; p.whole = plan.whole;
+  p.part = ctx->at<float2>(L.part); p.part_ld = ctx->K;
+  p.partial = ctx->at<float>(L.partial); p.ready = ctx->at<uint32_t>(L.ready); p.status = ctx->at<uint32_t>(L.status);
+  *pw = plan.bn / 2;
+  return launch_kernel_if(p.tilesM * p.tilesN <= plan.pairs, forward_pair_kernel, dim3(2u * static_cast<unsigned>(plan.pairs)),
+                          dim3(kThreads), kSmem, ctx->stream, 1, ma, mb, mc, p);
+}
+
+}  // namespace sfb

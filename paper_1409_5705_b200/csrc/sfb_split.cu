@@ -177,42 +177,6 @@ __device__ __forceinline__ void tile_coords(const SplitParams& p, int tile, int&
   n0 = tn * p.bn;
 }
 
-// What a pair computes, in its order: whole tiles, or the part of a tile that another pair completes and then the tiles that it
-// completes (the one it completes for others last).  k-blocks [k0, k1) of each.
-struct Segment { int tile, k0, k1; };
-struct Segments {
-  int pair, pairs, kseg, t0, n;
-  int64_t units, beg, end;             // k-blocks of all tiles; of this pair (none: whole tiles)
-  bool cut, leaves;
-  __device__ Segments(const SplitParams& p, int ntiles, int pair_, int pairs_)
-      : pair(pair_), pairs(pairs_), kseg(p.kseg), units(static_cast<int64_t>(ntiles) * p.kseg), cut(p.cut != 0) {
-    beg = units * pair / pairs;
-    end = units * (pair + 1) / pairs;
-    t0 = static_cast<int>(beg / kseg);
-    leaves = cut && end > beg && end % kseg != 0;
-    n = cut ? (end > beg ? static_cast<int>((end - 1) / kseg) - t0 + 1 : 0) : pair < ntiles ? (ntiles - 1 - pair) / pairs + 1 : 0;
-  }
-  __device__ Segment get(int i) const {
-    if (!cut) return Segment{pair + i * pairs, 0, kseg};
-    if (leaves) {
-      const int64_t first = static_cast<int64_t>(t0 + n - 1) * kseg;
-      if (i == 0) return Segment{t0 + n - 1, static_cast<int>((beg > first ? beg : first) - first), static_cast<int>(end - first)};
-      --i;
-    }
-    const int mine = n - (leaves ? 1 : 0), t = i < mine - 1 ? t0 + 1 + i : t0;
-    const int64_t first = static_cast<int64_t>(t) * kseg;
-    return Segment{t, beg > first ? static_cast<int>(beg - first) : 0, kseg};
-  }
-  // of the pairs that have a part of the tile which this one completes
-  __device__ int first_part(const Segment& sg) const {
-    if (sg.k0 == 0) return pair;
-    const int64_t first = static_cast<int64_t>(sg.tile) * kseg;
-    int j = pair - 1;
-    while (j > 0 && units * j / pairs > first) --j;
-    return j;
-  }
-};
-
 template <int EPI, bool F16>
 __global__ void __launch_bounds__(kThreads, 1)
 split_product_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
@@ -237,7 +201,7 @@ split_product_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
   const int bytesB = half * BK * 2, stage_bytes = 2 * kBytesA + 2 * bytesB;
   const int ntiles = EPI == F_GRAM ? sym_tiles(p.tilesM, p.tilesN, p.bn) : p.tilesM * p.tilesN;
   const int pair = blockIdx.x >> 1;
-  const Segments segs(p, ntiles, pair, gridDim.x >> 1);
+  const Segments segs(p.kseg, p.cut != 0, 0, ntiles, pair, gridDim.x >> 1);
 
   pdl_launch_dependents();
   if (threadIdx.x == 0) {

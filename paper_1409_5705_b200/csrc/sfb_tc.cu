@@ -799,6 +799,16 @@ static int pick_forward_split(int64_t K, int64_t rows, int64_t cols) {
   return best;
 }
 
+// Whether the logits of n samples take the kernel of CTA pairs.  Not beyond five rounds of its tiles, where an uneven last one matters
+// little and the step is at the power limit (325,000 x 10,000 with 1,024 samples: 5,280 us of the factors' time here, 5,470 there).  A
+// contraction split over a cluster costs 24,000 cycles more than forward_cost has for it (989 x 2,036 with 193 samples 40 us
+// of the factors' time, 18 on pairs; 873 x 2,800 with 634 38 and 25).
+static bool forward_on_pairs(const sfb_config& c, const Layout& L, int64_t n) {
+  if (n <= BM || !L.partial || ((n + 255) / 256) * ((c.rows + 255) / 256) >= 5 * (kModelSms / 2)) return false;
+  const int bn = pick_forward_width(n, c.rows, c.cols, L.pw, L.split);
+  return forward_pair_cost(n, c.rows, c.cols) < forward_cost(n, c.rows, c.cols, bn, L.split) + (L.split > 1 ? 24000.0 : 0.0);
+}
+
 // fp32 mode on the tensor cores (MLR): fp32 pair-major factors as in the FFMA path, plus the (big | small) tf32
 // operands of the two products and the logits.
 void tc32_extend_layout(const sfb_config& c, Layout& L, size_t& off) {
@@ -830,7 +840,12 @@ void tc_extend_layout(const sfb_config& c, Layout& L, size_t& off) {
   const size_t ldz = static_cast<size_t>(round_up(c.rows, 32));
   L.split = pick_forward_split(static_cast<int64_t>(K), c.rows, c.cols);
   L.pw = L.split > 1 ? 32 : pick_forward_width(c.batch, c.rows, c.cols, 32, 1);
-  const size_t nblk = static_cast<size_t>((c.rows + L.pw - 1) / L.pw);
+  size_t nblk = static_cast<size_t>((c.rows + L.pw - 1) / L.pw);
+  if (K > BM) {                                  // for the kernel of CTA pairs
+    nblk = std::max(nblk, static_cast<size_t>(forward_pair_groups(c.rows)));
+    L.partial = take(forward_pair_partial_bytes());
+    L.ready = take(forward_pair_ready_bytes());
+  }
   L.Wb = take(static_cast<size_t>(c.rows) * L.colsb * 2);
   L.Xb = take(K * L.colsb * 2);
   L.ZT = take(K * ldz * 4);                      // logits Z, sample-major [K x ldz]
@@ -872,6 +887,7 @@ int tc_init(sfb_ctx* ctx) {
     return tc_refresh_operands(ctx);
   }
   if (c.model != SFB_MLR || ctx->h16) return split_init(ctx);
+  if (ctx->lay.partial) CKC(cudaMemsetAsync(ctx->at<char>(ctx->lay.ready), 0, forward_pair_ready_bytes(), ctx->stream));
   CKC(cudaMemsetAsync(ctx->at<char>(ctx->lay.labels), 0xff, static_cast<size_t>(ctx->K) * 4, ctx->stream));
   CKC(cudaMemsetAsync(ctx->at<char>(ctx->lay.slot), 0x7f, static_cast<size_t>(c.rows) * 4, ctx->stream));
   // bf16 copy of W for the forward product; afterwards the update's epilogue keeps it current
@@ -1026,6 +1042,13 @@ static int mlr_forward(sfb_ctx* ctx, int64_t off, int64_t n, const float* X, con
                     fused ? nullptr : ctx->at<float>(L.Xf), labels, ctx->at<int32_t>(L.labels), ctx->at<int32_t>(L.slot),
                     rows,
                     take_stamp(ctx)));
+  ctx->stats.flops += 2.0 * n * rows * cols;
+  if (forward_on_pairs(c, L, n)) {
+    int pw = 0;
+    CKC(forward_pair(ctx, off, n, &pw));
+    *parts = static_cast<int>((rows + pw - 1) / pw);
+    return SFB_OK;
+  }
   // samples on the lanes (A), rows of W on the accumulator columns (B)
   const int bn = pick_forward_width(n, rows, cols, L.pw, L.split);
   const int ar = static_cast<int>(std::min<int64_t>(BM, round_up(n, 8)));
@@ -1043,7 +1066,6 @@ static int mlr_forward(sfb_ctx* ctx, int64_t off, int64_t n, const float* X, con
   p.part = ctx->at<float2>(L.part); p.part_ld = K; p.status = ctx->at<uint32_t>(L.status);
   p.nseg = 1; p.kseg = (p.Kc + BK - 1) / BK;
   CKC(launch_forward<false>(ctx, ma, mb, mc, p));
-  ctx->stats.flops += 2.0 * n * rows * cols;
   *parts = static_cast<int>((rows + L.pw - 1) / L.pw);
   return SFB_OK;
 }
@@ -1239,7 +1261,8 @@ int tc_host_parts(const sfb_ctx* ctx) {
   auto total = [&](int parts) {
     const int64_t n = ctx->K / parts;
     const double copy = 4.0 * static_cast<double>(n) * static_cast<double>(c.cols) / 45e9 + 4e-6;
-    const double cycles = forward_cost(n, c.rows, c.cols, pick_forward_width(n, c.rows, c.cols, ctx->lay.pw, 1), 1);
+    const double cycles = forward_on_pairs(c, ctx->lay, n) ? forward_pair_cost(n, c.rows, c.cols)
+                                                           : forward_cost(n, c.rows, c.cols, pick_forward_width(n, c.rows, c.cols, ctx->lay.pw, 1), 1);
     const double product = std::max(cycles / 1.7e9, 2.0 * static_cast<double>(c.rows) * static_cast<double>(c.cols) / 5e12) + 5e-6;
     // (a product that takes much longer than its copy has little to gain, and a pass over W per part to lose)
     return parts > 1 && product > 2. * copy ? 1e9 : copy + (parts - 1) * std::max(copy, product) + product;

@@ -58,6 +58,15 @@ int tc_update(sfb_ctx* ctx);
 int tc_get_factors(sfb_ctx* ctx, const void** U, const void** V, int32_t* dtype, int32_t* layout, int64_t* ldu,
                    int64_t* ldv);
 
+// The forward product on pairs of CTAs (sfb_forward.cu): its cycles; its buffers (parts of tiles, their flags); the logits of n packed
+// samples at pair offset off, *pw: classes per softmax partial.
+double forward_pair_cost(int64_t n, int64_t rows, int64_t cols);
+int64_t forward_pair_groups(int64_t rows);           // most softmax partials of a sample
+size_t forward_pair_partial_bytes();
+size_t forward_pair_ready_bytes();
+cudaError_t forward_pair_prepare(int* max_pairs);
+cudaError_t forward_pair(sfb_ctx* ctx, int64_t off, int64_t n, int* pw);
+
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
                                   const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
                                   CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);

@@ -43,6 +43,46 @@ __device__ __forceinline__ void xchg_sum(uint8_t* smem, int c, int row, int part
   }
 }
 
+// What a pair of CTAs computes of a product's tiles, in its order: whole tiles (the `whole` first of them, a multiple of the pairs;
+// all when nothing is cut), then, of the others, whose k-blocks are shared out evenly, the part of a tile that another pair
+// completes and the tiles that it completes (the one it completes for others last).  k-blocks [k0, k1) of each.
+struct Segment { int tile, k0, k1; };
+struct Segments {
+  int pair, pairs, kseg, whole, own, t0, n;      // own: whole tiles of this pair ahead of its part of the others
+  int64_t units, beg, end;                       // k-blocks of the tiles that are shared out; of this pair
+  bool cut, leaves;
+  __device__ Segments(int kseg_, bool cut_, int whole_, int ntiles, int pair_, int pairs_)
+      : pair(pair_), pairs(pairs_), kseg(kseg_), whole(whole_), units(static_cast<int64_t>(ntiles - whole_) * kseg_), cut(cut_) {
+    own = whole / pairs;
+    beg = units * pair / pairs;
+    end = units * (pair + 1) / pairs;
+    t0 = static_cast<int>(beg / kseg);
+    leaves = cut && end > beg && end % kseg != 0;
+    n = cut ? own + (end > beg ? static_cast<int>((end - 1) / kseg) - t0 + 1 : 0) : pair < ntiles ? (ntiles - 1 - pair) / pairs + 1 : 0;
+  }
+  __device__ Segment get(int i) const {
+    if (!cut || i < own) return Segment{pair + i * pairs, 0, kseg};
+    i -= own;
+    if (leaves) {
+      const int last = t0 + n - own - 1;
+      const int64_t first = static_cast<int64_t>(last) * kseg;
+      if (i == 0) return Segment{whole + last, static_cast<int>((beg > first ? beg : first) - first), static_cast<int>(end - first)};
+      --i;
+    }
+    const int mine = n - own - (leaves ? 1 : 0), t = i < mine - 1 ? t0 + 1 + i : t0;
+    const int64_t first = static_cast<int64_t>(t) * kseg;
+    return Segment{whole + t, beg > first ? static_cast<int>(beg - first) : 0, kseg};
+  }
+  // of the pairs that have a part of the tile which this one completes
+  __device__ int first_part(const Segment& sg) const {
+    if (sg.k0 == 0) return pair;
+    const int64_t first = static_cast<int64_t>(sg.tile - whole) * kseg;
+    int j = pair - 1;
+    while (j > 0 && units * j / pairs > first) --j;
+    return j;
+  }
+};
+
 __device__ __forceinline__ float soft_threshold(float w, float t) {
   const float a = fabsf(w) - t;
   return a > 0.f ? copysignf(a, w) : 0.f;
@@ -52,6 +92,27 @@ __device__ __forceinline__ float soft_threshold(float w, float t) {
 inline unsigned grid1d(int64_t items, int per_block) {
   const int64_t g = (items + per_block - 1) / per_block;
   return static_cast<unsigned>(std::max<int64_t>(1, std::min<int64_t>(g, static_cast<int64_t>(sm_count()) * 16)));
+}
+
+// Opts a kernel of CTA pairs (thread blocks of a fixed cluster of two) into `smem` bytes; at most *max_pairs of them at a time.
+template <typename Kernel>
+cudaError_t prepare_pair_kernel(Kernel kernel, int threads, int smem, int* max_pairs) {
+  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (e != cudaSuccess) return e;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(2, 1, 1);
+  cfg.blockDim = dim3(threads, 1, 1);
+  cfg.dynamicSmemBytes = smem;
+  cudaLaunchAttribute attr{};
+  attr.id = cudaLaunchAttributeClusterDimension;
+  attr.val.clusterDim.x = 2; attr.val.clusterDim.y = 1; attr.val.clusterDim.z = 1;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  int n = 0;
+  e = cudaOccupancyMaxActiveClusters(&n, kernel, &cfg);
+  if (e != cudaSuccess) return e;
+  *max_pairs = std::min(*max_pairs, n);
+  return cudaSuccess;
 }
 
 }  // namespace sfb

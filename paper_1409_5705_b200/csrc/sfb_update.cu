@@ -648,33 +648,14 @@ int tile_width(int64_t rows, int64_t cols, int64_t kblocks, int pairs, bool spli
     }                                                   \
   } while (0)
 
-template <typename Kernel>
-static cudaError_t prepare_kernel(Kernel kernel, int smem, int* max_pairs) {
-  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  if (e != cudaSuccess) return e;
-  cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3(2, 1, 1);
-  cfg.blockDim = dim3(kThreads, 1, 1);
-  cfg.dynamicSmemBytes = smem;
-  cudaLaunchAttribute attr{};
-  attr.id = cudaLaunchAttributeClusterDimension;
-  attr.val.clusterDim.x = 2; attr.val.clusterDim.y = 1; attr.val.clusterDim.z = 1;
-  cfg.attrs = &attr;
-  cfg.numAttrs = 1;
-  int n = 0;
-  e = cudaOccupancyMaxActiveClusters(&n, kernel, &cfg);
-  if (e != cudaSuccess) return e;
-  *max_pairs = std::min(*max_pairs, n);
-  return cudaSuccess;
-}
-
 int tc_update_init(sfb_ctx* ctx, TcState* st) {
   int n = 1 << 30;
-  CKC(prepare_kernel(update_pair_kernel<1>, UpShape<false>::kSmem, &n));
-  CKC(prepare_kernel(update_pair_kernel<1, false, true>, UpShape<true>::kSmem, &n));
-  CKC(prepare_kernel(update_split_kernel<false>, SuShape<false>::kSmem, &n));
-  CKC(prepare_kernel(update_split_kernel<true>, SuShape<true>::kSmem, &n));
-  CKC(prepare_kernel(update_pair_kernel<2, true>, UpShape<false>::kSmem, &n));
+  CKC(prepare_pair_kernel(update_pair_kernel<1>, kThreads, UpShape<false>::kSmem, &n));
+  CKC((prepare_pair_kernel(update_pair_kernel<1, false, true>, kThreads, UpShape<true>::kSmem, &n)));
+  CKC(prepare_pair_kernel(update_split_kernel<false>, kThreads, SuShape<false>::kSmem, &n));
+  CKC(prepare_pair_kernel(update_split_kernel<true>, kThreads, SuShape<true>::kSmem, &n));
+  CKC((prepare_pair_kernel(update_pair_kernel<2, true>, kThreads, UpShape<false>::kSmem, &n)));
+  CKC(forward_pair_prepare(&n));
   st->max_pairs = n;
   if (n < 1) return SFB_ERR_ARCH;                 // the device cannot host a CTA pair of these kernels
   return SFB_OK;

@@ -11,7 +11,9 @@ torch = pytest.importorskip("torch")
 
 
 def check(rows, cols, workers, batch, per_worker=False):
-    wl = I.scaled(I.WORKLOADS["mlr_mid"], "mlr_forms", rows=rows, cols=cols, workers=workers, batch=batch, w_std=0.05,
+    # logits of about 1: those of size s carry 2^-9 s of rounding in bf16 operands, and the probabilities with them (with s = 4.8 the
+    # update is 3.0e-3 off on any kernel)
+    wl = I.scaled(I.WORKLOADS["mlr_mid"], "mlr_forms", rows=rows, cols=cols, workers=workers, batch=batch, w_std=cols ** -0.5,
                   x_scale="unit", eta=0.05)
     W0, inp = I.initial_W(wl), I.step_inputs(wl, 1)
     W = to_dev(W0, torch)
@@ -38,3 +40,28 @@ def check(rows, cols, workers, batch, per_worker=False):
 @pytest.mark.parametrize("shape", [(5, 4, 1, 1), (257, 260, 4, 64), (257, 260, 1, 257), (1030, 2500, 5, 51), (6001, 2052, 2, 120)])
 def test_update_forms(shape):
     check(*shape)
+
+
+# The logits on pairs of CTAs: whole tiles of 64 and 192 classes; a contraction shared out over all pairs, most of them in the middle of a
+# tile; more tiles than pairs, the rest of the second and of the third round shared out; the last sample and the last class alone in a tile.
+@pytest.mark.parametrize("shape", [(873, 2800, 2, 317), (190, 708, 1, 513), (791, 9276, 4, 140), (9001, 4004, 2, 257), (10100, 5004, 5, 180),
+                                   (2305, 1028, 1, 129)])
+def test_logits_on_pairs(shape):
+    check(*shape)
+
+
+def test_logits_on_pairs_repeat():
+    """The sums of a shared-out tile are in the order of the pairs: the same bits every time."""
+    rows, cols, K = 9001, 4004, 514
+    W0 = torch.randn(rows, cols, device="cuda") * 0.05
+    X, lab = torch.randn(K, cols, device="cuda") / cols ** 0.5, torch.randint(0, rows, (K,), device="cuda", dtype=torch.int32)
+    got = []
+    for _ in range(2):
+        W = W0.clone()
+        ctx = S.Context(S.make_config(S.MLR, rows, cols, 1, K, 0.05, S.PREC_BF16), W)
+        for _ in range(3):
+            ctx.sfb_step(X, None, lab)
+        assert ctx.sfb_get_status() == 0
+        got.append(W)
+        ctx.close()
+    assert torch.equal(got[0], got[1])
