@@ -343,3 +343,219 @@ cudaError_t forward_pair(sfb_ctx* ctx, int64_t off, int64_t n, int* pw) {
 }
 
 }  // namespace sfb
+
+// ---------------------------------------------------------------------------------------------------------
+// Logits of up to 64 samples, a worker's mini-batch: the classes are the rows of the accumulator (128 of them a CTA), the samples its
+// columns.
+// Such a product is bound by the way of W to the SMs and by latency.  With the samples as rows, 128 of which the MMA computes
+// whatever their number, an SM had 64 classes and issued four MMAs of 64 columns a k-block of 8 KB of W: 79 CTAs at 400 cycles a
+// k-block for 4,999 x 3,004.  Here an MMA has as many columns as there are samples, a k-block is 16 KB of W, and the contraction
+// is cut over clusters of up to four CTAs as long as all of them are resident.  us of a worker's call, forward_kernel / here:
+// 4,999 x 3,004 with 8, 37, 64 samples 20.5, 20.6, 21.7 / 12.7, 14.5, 17.9; 500 x 3,004 18.2, 28.6, 28.9 / 11.2, 12.6, 13.0.  (With
+// the rounding of the samples in this kernel instead of one of its own before it, eight k-blocks of loads under way: 11.4, 16.3,
+// 20.9; every CTA then reads all samples in fp32.)
+// Warps: 0 TMA producer, 1 MMA issuer and TMEM owner, 2..9 epilogue: parts through shared memory, Z by rows, softmax partials of 32
+// classes.
+// ---------------------------------------------------------------------------------------------------------
+namespace sfb {
+namespace {
+
+constexpr int kFewN = 64, kFewStages = 8, kFewParts = 4;
+constexpr int kFewA = BM * BK * 2, kFewB = kFewN * BK * 2, kFewStage = kFewA + kFewB;
+constexpr int kFewXchg = 4 * kFewN * 32 * 4;        // [lane quarter][sample][32 classes] fp32
+constexpr int kFewBars = 2 * kFewStages + 1;
+constexpr int kFewSmem = kFewStages * kFewStage + kFewXchg + kFewBars * 8 + 16 + 1024;
+constexpr int kFewTmem = 64;
+
+struct FewParams {
+  int32_t n, off;              // samples of this call, first pair
+  int32_t rows, tiles;         // classes; tiles of 128 of them
+  int32_t kseg, parts;         // k-blocks; CTAs of a cluster, which share them
+  float* Z;
+  int64_t ldz;
+  float2* part;
+  int64_t part_ld;
+  uint32_t* status;
+};
+
+__global__ void __launch_bounds__(kThreads, 1)
+forward_few_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmX, const __grid_constant__ FewParams p) {
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  uint8_t* xchg = smem + kFewStages * kFewStage;
+  uint64_t* bars = reinterpret_cast<uint64_t*>(xchg + kFewXchg);
+  uint64_t* full = bars;
+  uint64_t* empty = bars + kFewStages;
+  uint64_t* done = bars + 2 * kFewStages;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + kFewBars);
+  volatile uint32_t* abort_flag = tmem_slot + 1;
+
+  const int warp = warp_index(), lane = threadIdx.x & 31;
+  const int tile = static_cast<int>(blockIdx.x) / p.parts, mine = static_cast<int>(blockIdx.x) % p.parts;     // (its rank in the cluster)
+  const int kbeg = mine * p.kseg / p.parts, nk = (mine + 1) * p.kseg / p.parts - kbeg;
+  pdl_launch_dependents();
+  if (threadIdx.x == 0) {
+    for (int i = 0; i < kFewStages; ++i) { mbar_init(&full[i], 1); mbar_init(&empty[i], 1); }
+    mbar_init(done, 1);
+    *abort_flag = 0;
+    fence_barrier_init();
+    prefetch_tmap(&tmW); prefetch_tmap(&tmX);
+  }
+  if (warp == 1) { tmem_alloc(tmem_slot, kFewTmem); tmem_relinquish(); }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem_base = *tmem_slot;
+  pdl_wait();
+
+  if (warp == 0) {
+    const uint64_t pol_keep = policy_evict_last();      // every tile reads the samples
+    bool ok = true;
+    for (int k = 0; k < nk && ok; ++k) {
+      const uint32_t s = k % kFewStages, ph = (k / kFewStages) & 1;
+      ok = mbar_wait_warp(&empty[s], ph ^ 1, abort_flag);
+      if (ok && elect_one()) {
+        mbar_expect_tx(&full[s], kFewA + ((p.n + 7) & ~7) * BK * 2);
+        tma_load_2d(smem + s * kFewStage, &tmW, (kbeg + k) * BK, tile * BM, &full[s]);
+        tma_load_2d_hint(smem + s * kFewStage + kFewA, &tmX, (kbeg + k) * BK, p.off, &full[s], pol_keep);
+      }
+    }
+  } else if (warp == 1) {
+    const uint32_t idesc = umma_idesc_bf16(BM, (static_cast<uint32_t>(p.n) + 15u) & ~15u);
+    bool ok = true;
+    for (int k = 0; k < nk && ok; ++k) {
+      const uint32_t s = k % kFewStages, ph = (k / kFewStages) & 1;
+      ok = mbar_wait_warp(&full[s], ph, abort_flag);
+      tc_fence_after();
+      if (ok && elect_one()) {
+        const uint64_t da = umma_desc_k128(smem_u32(smem + s * kFewStage)), db = umma_desc_k128(smem_u32(smem + s * kFewStage + kFewA));
+#pragma unroll
+        for (int j = 0; j < BK / UMMA_K; ++j) {
+          const uint64_t adv = static_cast<uint64_t>(j * UMMA_K * 2 / 16);
+          umma_bf16(tmem_base, da + adv, db + adv, idesc, (k | j) != 0 ? 1u : 0u);
+        }
+        umma_commit(&empty[s]);
+      }
+    }
+    if (ok && elect_one()) umma_commit(done);
+  } else {
+    const int e = warp - 2, q = warp & 3, h = e >> 2;
+    const int r4 = lane >> 3, c8 = lane & 7;         // eight lanes take 32 classes of a sample
+    // ---------------- the accumulator: lane = class, column = sample ----------------
+    if (mbar_wait_warp(done, 0, abort_flag) && h * 32 < p.n) {
+      tc_fence_after();
+      uint32_t acc[32];
+      tmem_ld_32x32(tmem_base + (static_cast<uint32_t>(q * 32) << 16) + h * 32, acc);
+      tmem_ld_wait();
+      float* out = reinterpret_cast<float*>(xchg) + (q * kFewN + h * 32) * 32 + lane;
+#pragma unroll
+      for (int j = 0; j < 32; ++j)
+        if (h * 32 + j < p.n) out[j * 32] = __uint_as_float(acc[j]);
+    }
+    __syncwarp();
+    if (p.parts > 1) { cluster_arrive(); cluster_wait(); }
+    else asm volatile("bar.sync 1, 256;" ::: "memory");
+    // units of 4 samples x 32 classes, 8 lanes a sample; a unit's sums are in rank order
+    const int units = 4 * ((p.n + 3) / 4);
+    for (int u = mine * kEpi + e; u < units; u += p.parts * kEpi) {
+      const int uq = u & 3, j = (u >> 2) * 4 + r4, grp = tile * 4 + uq;
+      const int64_t r0 = static_cast<int64_t>(grp) * 32 + 4 * c8;
+      const uint32_t at = smem_u32(xchg) + ((uq * kFewN + j) * 32 + 4 * c8) * 4;      // (j < 64: n is at most that)
+      float4 v = ld_cluster_f4(at, 0);
+      for (int r = 1; r < p.parts; ++r) {
+        const float4 t = ld_cluster_f4(at, r);
+        v.x += t.x; v.y += t.y; v.z += t.z; v.w += t.w;
+      }
+      const int left = p.rows - static_cast<int>(r0);                                   // classes from here on
+      float mx = left > 0 ? v.x : -INFINITY;
+      if (left > 1) mx = fmaxf(mx, v.y);
+      if (left > 2) mx = fmaxf(mx, v.z);
+      if (left > 3) mx = fmaxf(mx, v.w);
+#pragma unroll
+      for (int o = 4; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+      float sum = (left > 0 ? __expf(v.x - mx) : 0.f) + (left > 1 ? __expf(v.y - mx) : 0.f) + (left > 2 ? __expf(v.z - mx) : 0.f) +
+                  (left > 3 ? __expf(v.w - mx) : 0.f);
+#pragma unroll
+      for (int o = 4; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+      if (j < p.n && grp * 32 < p.rows) {
+        *reinterpret_cast<float4*>(p.Z + (p.off + j) * p.ldz + r0) = v;               // (its pitch is a multiple of 32)
+        if (c8 == 0) p.part[static_cast<int64_t>(grp) * p.part_ld + p.off + j] = make_float2(mx, sum);
+      }
+    }
+  }
+  if (p.parts > 1) {
+    __syncwarp();
+    if (warp < 2) { cluster_arrive(); cluster_wait(); }                // (the others have been there)
+    cluster_arrive();                                                  // no CTA leaves while a peer still reads its part
+    cluster_wait();
+  }
+  __syncwarp();
+  tc_fence_before();
+  __syncthreads();
+  if (*abort_flag) {
+    if (threadIdx.x == 0) atomicOr(p.status, SFB_STATUS_TIMEOUT);
+    for (int i = 0; i < 64; ++i) __nanosleep(1000);
+    __syncthreads();
+  }
+  if (warp == 1) { tc_fence_after(); tmem_dealloc(tmem_base, kFewTmem); }
+}
+
+// CTAs of a cluster: as many as keep all of them resident and leave each four k-blocks.
+int few_parts(int64_t tiles, int64_t kseg, const int (&most)[kFewParts + 1]) {
+  int best = 1;
+  for (int s = 2; s <= kFewParts; ++s)
+    if (tiles <= most[s] && kseg >= 4 * s) best = s;
+  return best;
+}
+
+}  // namespace
+
+// Where two CTAs share a tile (up to 74 tiles); fewer than one tile per SM leaves SMs idle, which pays for few samples or where W comes from
+// HBM.  us of a worker's call, forward_kernel / here, 3,004 features: 9,400 classes with 37 and 64 samples 23.2, 24.9 / 21.5, 24.2; 10,000
+// with 8 and 64 23.5, 26.0 / 19.4, 29.8; 15,000 with 16 and 37 25.0, 27.3 / 22.0, 30.8; 10,000 x 20,000 with 8 and 64 119, 128 / 80, 88.
+bool forward_few_fits(int64_t n, int64_t rows, int64_t cols) {
+  const int64_t tiles = (rows + BM - 1) / BM;
+  return n <= kFewN && (tiles <= kModelSms / 2 || (tiles <= 118 && (n <= 24 || rows * cols >= 100000000)));
+}
+int64_t forward_few_groups(int64_t rows) { return (rows + 31) / 32; }
+
+cudaError_t forward_few_prepare(int (&most)[5]) {
+  static_assert(kFewParts + 1 == 5, "");
+  cudaError_t e = cudaFuncSetAttribute(forward_few_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kFewSmem);
+  for (int s = 1; s <= kFewParts && e == cudaSuccess; ++s) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(s, 1, 1);
+    cfg.blockDim = dim3(kThreads, 1, 1);
+    cfg.dynamicSmemBytes = kFewSmem;
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = s; attr.val.clusterDim.y = 1; attr.val.clusterDim.z = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    e = cudaOccupancyMaxActiveClusters(&most[s], forward_few_kernel, &cfg);
+  }
+  return e;
+}
+
+cudaError_t forward_few(sfb_ctx* ctx, int64_t off, int64_t n) {
+  TcState* st = static_cast<TcState*>(ctx->tc);
+  const Layout& L = ctx->lay;
+  const int64_t rows = ctx->cfg.rows, cols = ctx->cfg.cols;
+  CUtensorMap mw, mx;
+  if (!make_map(st, &mw, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, ctx->at<uint16_t>(L.Wb), cols, rows, L.colsb * 2, BK, BM) ||
+      !make_map(st, &mx, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, ctx->at<uint16_t>(L.Xb), cols, ctx->K, L.colsb * 2, BK,
+                static_cast<int>(round_up(n, 8))))
+    return cudaErrorInvalidValue;
+  FewParams p{};
+  p.n = static_cast<int32_t>(n); p.off = static_cast<int32_t>(off);
+  p.rows = static_cast<int32_t>(rows); p.tiles = static_cast<int32_t>((rows + BM - 1) / BM);
+  p.kseg = static_cast<int32_t>((cols + BK - 1) / BK);
+  p.parts = few_parts(p.tiles, p.kseg, st->few);
+  p.Z = ctx->at<float>(L.ZT); p.ldz = round_up(rows, 32);
+  p.part = ctx->at<float2>(L.part); p.part_ld = ctx->K;
+  p.status = ctx->at<uint32_t>(L.status);
+  return launch_kernel(forward_few_kernel, dim3(static_cast<unsigned>(p.tiles * p.parts)), dim3(kThreads), kFewSmem, ctx->stream, p.parts,
+                       mw, mx, p);
+}
+
+}  // namespace sfb

@@ -841,6 +841,7 @@ void tc_extend_layout(const sfb_config& c, Layout& L, size_t& off) {
   L.split = pick_forward_split(static_cast<int64_t>(K), c.rows, c.cols);
   L.pw = L.split > 1 ? 32 : pick_forward_width(c.batch, c.rows, c.cols, 32, 1);
   size_t nblk = static_cast<size_t>((c.rows + L.pw - 1) / L.pw);
+  if (forward_few_fits(c.batch, c.rows, c.cols)) nblk = std::max(nblk, static_cast<size_t>(forward_few_groups(c.rows)));
   if (K > BM) {                                  // for the kernel of CTA pairs
     nblk = std::max(nblk, static_cast<size_t>(forward_pair_groups(c.rows)));
     L.partial = take(forward_pair_partial_bytes());
@@ -874,6 +875,7 @@ int tc_init(sfb_ctx* ctx) {
   CKC(cudaGetDevice(&dev));
   CKC(cudaDeviceGetAttribute(&st->sms, cudaDevAttrMultiProcessorCount, dev));
   CKC(prepare_forward_kernels());
+  CKC(forward_few_prepare(st->few));
   {
     const int rc = tc_update_init(ctx, st);
     if (rc) return rc;
@@ -1035,6 +1037,7 @@ static int mlr_forward(sfb_ctx* ctx, int64_t off, int64_t n, const float* X, con
   const int64_t ldz = round_up(rows, 32);
   __nv_bfloat16* Xb = ctx->at<__nv_bfloat16>(L.Xb);
   ctx->labels = sfb_ctx::kLabelsNone;
+  ctx->stats.flops += 2.0 * n * rows * cols;
   // (samples that come by a copy on another stream: that one has to be complete before the kernel starts at all)
   const bool early = !ctx->host || ctx->host->parts <= 1;
   CKC(launch_kernel_if(early, pack_mlr_kernel, dim3(grid1d(n * cols / 4, 256)), dim3(256), 0, ctx->stream, 1, X, n, cols, Xb,
@@ -1042,7 +1045,11 @@ static int mlr_forward(sfb_ctx* ctx, int64_t off, int64_t n, const float* X, con
                     fused ? nullptr : ctx->at<float>(L.Xf), labels, ctx->at<int32_t>(L.labels), ctx->at<int32_t>(L.slot),
                     rows,
                     take_stamp(ctx)));
-  ctx->stats.flops += 2.0 * n * rows * cols;
+  if (forward_few_fits(n, rows, cols)) {
+    CKC(forward_few(ctx, off, n));
+    *parts = static_cast<int>(forward_few_groups(rows));
+    return SFB_OK;
+  }
   if (forward_on_pairs(c, L, n)) {
     int pw = 0;
     CKC(forward_pair(ctx, off, n, &pw));

@@ -67,6 +67,13 @@ size_t forward_pair_ready_bytes();
 cudaError_t forward_pair_prepare(int* max_pairs);
 cudaError_t forward_pair(sfb_ctx* ctx, int64_t off, int64_t n, int* pw);
 
+// The same for up to 64 samples (forward_few_kernel): whether it takes these sizes; softmax partials, of 32 classes; most resident
+// clusters of 1 to 4 CTAs.
+bool forward_few_fits(int64_t n, int64_t rows, int64_t cols);
+int64_t forward_few_groups(int64_t rows);
+cudaError_t forward_few_prepare(int (&most)[5]);
+cudaError_t forward_few(sfb_ctx* ctx, int64_t off, int64_t n);
+
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
                                   const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
                                   CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
@@ -88,6 +95,7 @@ struct TcState {
   CUtensorMap map[kMaps];
   EncodeTiledFn encode;      // cuTensorMapEncodeTiled, obtained through the runtime's driver entry point query
   int sms;                   // multiprocessors of the device
+  int few[5];                // resident clusters of 1 to 4 CTAs of forward_few_kernel
   int max_pairs;             // CTA pairs (clusters of 2) of the update kernel that can be resident at once
 };
 

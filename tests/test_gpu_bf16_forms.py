@@ -65,3 +65,12 @@ def test_logits_on_pairs_repeat():
         got.append(W)
         ctx.close()
     assert torch.equal(got[0], got[1])
+
+
+# The logits of up to 64 samples: one sample, two classes; a contraction in 1, 2, 3 and 4 parts; the last tile of one class; 64 samples and 65;
+# more classes than that, with few samples; samples of one call and of several workers.
+@pytest.mark.parametrize("shape", [(2, 4, 1, 1), (200, 12004, 1, 37), (129, 68, 1, 33), (64, 256, 4, 32), (385, 1028, 3, 37), (4999, 3004, 2, 37), (7100, 516, 1, 17),
+                                   (9000, 772, 2, 64), (9000, 772, 1, 65), (9473, 772, 1, 24), (15104, 132, 2, 9), (15105, 132, 2, 9)])
+@pytest.mark.parametrize("per_worker", [False, True])
+def test_logits_of_few_samples(shape, per_worker):
+    check(*shape, per_worker=per_worker)
