@@ -599,6 +599,134 @@ __global__ void __launch_bounds__(256) mlr_emit_p_kernel(const float* __restrict
   }
 }
 
+// Merged softmax of a small mini-batch (up to 256 samples, few partials): one launch instead of mlr_lse_kernel and mlr_emit_p_kernel,
+// 3 of the 20 us of a step at 64 x 256 with 128 samples.  Every block merges the partials of all samples itself (the same sums as
+// mlr_lse_kernel's); the label blocks find a class's first sample in shared memory, as its slots are only just being set here.
+constexpr int kMergeSamples = 256, kMergePartials = 2048;
+__global__ void __launch_bounds__(256) mlr_merged_kernel(const float2* __restrict__ part, int64_t part_ld, int nblocks,
+                                                         const float* __restrict__ Z, int64_t ldz, int64_t rows, int32_t n,
+                                                         const int32_t* __restrict__ labels, float* __restrict__ lse,
+                                                         float* __restrict__ loss, float* __restrict__ coef, int32_t* __restrict__ slot,
+                                                         __nv_bfloat16* __restrict__ P, int64_t ldp, uint32_t* status, int lab_blocks,
+                                                         const LabelArgs lab) {
+  pdl_launch_dependents();
+  pdl_wait(part, Z, labels, lse, loss, coef, slot, P);
+  __shared__ float sh_lse[kMergeSamples], sh_coef[kMergeSamples], sh_loss[kMergeSamples];
+  __shared__ int32_t sh_y[kMergeSamples], sh_next[kMergeSamples];
+  __shared__ bool sh_first[kMergeSamples];
+  const int t = threadIdx.x, lane = t & 31;
+  // lanes of a sample: the power of two that the partials fill, at most 32
+  int width = 32;
+  while (width > 1 && width / 2 >= nblocks) width /= 2;
+  const int sub = t % width;
+  for (int i = t / width; i < (n + 256 / width - 1) / (256 / width) * (256 / width); i += 256 / width) {
+    float m = -INFINITY, sum = 0.f;
+    if (i < n)
+      for (int b = sub; b < nblocks; b += width) m = fmaxf(m, part[static_cast<int64_t>(b) * part_ld + i].x);
+    for (int o = width / 2; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+    if (i < n)
+      for (int b = sub; b < nblocks; b += width) {
+        const float2 v = part[static_cast<int64_t>(b) * part_ld + i];
+        sum += v.y * __expf(v.x - m);
+      }
+    for (int o = width / 2; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+    if (sub == 0 && i < n) {
+      const float l = m + logf(sum);
+      const int32_t y = labels[i];
+      const bool ok = y >= 0 && y < rows;
+      const float zy = ok ? Z[i * ldz + y] : 0.f;
+      sh_lse[i] = l;
+      sh_y[i] = ok ? y : -1;
+      sh_loss[i] = ok ? l - zy : 0.f;
+      sh_coef[i] = ok ? -expm1f(zy - l) : 0.f;
+    }
+  }
+  __syncthreads();
+  const int blk = static_cast<int>(blockIdx.x);
+  if ((blk < lab_blocks || blk == gridDim.x - 1) && t < n) {       // the first sample of this one's class, and the next one
+    const int32_t y = sh_y[t];
+    int first = n, next = n;
+#pragma unroll 8
+    for (int j = n - 1; j >= 0; --j)
+      if (sh_y[j] == y) {
+        first = j;
+        if (j > t) next = j;
+      }
+    sh_first[t] = y >= 0 && first == t;
+    sh_next[t] = next;
+  }
+  __syncthreads();
+  if (blk == gridDim.x - 1)                          // for the calls that come after
+    for (int i = t; i < n; i += 256) {
+      lse[i] = sh_lse[i]; loss[i] = sh_loss[i]; coef[i] = sh_coef[i];
+      if (sh_y[i] < 0) atomicOr(status, SFB_STATUS_LABEL_RANGE);
+      if (sh_first[i]) slot[sh_y[i]] = i;
+    }
+  if (blk < lab_blocks) {
+    if (blk == lab_blocks - 1) {                     // the mean loss, in label_delta's order
+      __shared__ float lsum[8];
+      float v = t < n ? sh_loss[t] : 0.f;
+      v = warp_sum(v);
+      if (lane == 0) lsum[t >> 5] = v;
+      __syncthreads();
+      if (t == 0) {
+        float mean = 0.f;
+        for (int w = 0; w < 8; ++w) mean += lsum[w];
+        *lab.loss_mean = mean / static_cast<float>(n);
+      }
+    }
+    const int chunks = static_cast<int>((lab.cols + kLabelCols - 1) / kLabelCols);
+    for (int u = blk; u < n * chunks; u += lab_blocks) {
+      const int i = u / chunks;
+      if (!sh_first[i]) continue;
+      const int32_t y = sh_y[i];
+      const int64_t c = static_cast<int64_t>(u % chunks) * kLabelCols + 4 * t;
+      if (c >= lab.cols) continue;
+      float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+      float* wp = lab.W + static_cast<int64_t>(y) * lab.cols + c;
+      float4 w = *reinterpret_cast<const float4*>(wp);
+      const float* X = lab.X + c;
+      auto add = [&](float cf, const float4& x) {
+        s.x = fmaf(cf, x.x, s.x); s.y = fmaf(cf, x.y, s.y); s.z = fmaf(cf, x.z, s.z); s.w = fmaf(cf, x.w, s.w);
+      };
+      for (int j = i; j < n;) {
+        if (sh_next[j] >= n) {                       // the last one by itself
+          add(sh_coef[j], *reinterpret_cast<const float4*>(X + static_cast<int64_t>(j) * lab.cols));
+          break;
+        }
+        float4 x[kLabelBatch];
+        const float* xp[kLabelBatch];
+        float cf[kLabelBatch];
+#pragma unroll
+        for (int e = 0; e < kLabelBatch; ++e) {
+          xp[e] = X + static_cast<int64_t>(j < n ? j : i) * lab.cols;
+          cf[e] = j < n ? sh_coef[j] : 0.f;
+          if (j < n) j = sh_next[j];
+        }
+        load8(x, xp);
+#pragma unroll
+        for (int e = 0; e < kLabelBatch; ++e) add(cf[e], x[e]);
+      }
+      *reinterpret_cast<float4*>(lab.dL + static_cast<int64_t>(i) * lab.cols + c) = s;
+      w.x = fmaf(lab.step, s.x, w.x); w.y = fmaf(lab.step, s.y, w.y); w.z = fmaf(lab.step, s.z, w.z); w.w = fmaf(lab.step, s.w, w.w);
+      *reinterpret_cast<float4*>(wp) = w;
+      *reinterpret_cast<uint2*>(lab.Wb + static_cast<int64_t>(y) * lab.ldw + c) = make_uint2(pack_bf16(w.x, w.y), pack_bf16(w.z, w.w));
+    }
+    return;
+  }
+  const int octs = static_cast<int>((rows + 7) / 8), emit = static_cast<int>(gridDim.x) - lab_blocks;
+  for (int q = (blk - lab_blocks) * 256 + t; q < n * octs; q += emit * 256) {
+    const int i = q / octs, r = (q - i * octs) * 8, yrel = sh_y[i] - r;
+    const float l = sh_lse[i];
+    const float4 a = *reinterpret_cast<const float4*>(Z + i * ldz + r), b = *reinterpret_cast<const float4*>(Z + i * ldz + r + 4);
+    float z[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+#pragma unroll
+    for (int k = 0; k < 8; ++k) z[k] = k == yrel ? 0.f : __expf(z[k] - l);
+    *reinterpret_cast<uint4*>(P + i * ldp + r) =
+        make_uint4(pack_bf16(z[0], z[1]), pack_bf16(z[2], z[3]), pack_bf16(z[4], z[5]), pack_bf16(z[6], z[7]));
+  }
+}
+
 // Both for a worker's samples whose label rows are summed later: every block merges the partials of its sample itself, which
 // saves a launch (3 us of a call of 37 samples against 4,999 x 3,004).  One sample per grid row, its classes over the grid's
 // columns.
@@ -1310,6 +1438,15 @@ int tc_factors(sfb_ctx* ctx, int64_t off, int64_t n, const float* X, const float
     CKC(launch_kernel(mlr_lse_emit_kernel, dim3(static_cast<unsigned>(std::min(most, want)), static_cast<unsigned>(n)), dim3(256), 0,
                       ctx->stream, 1, ctx->at<float2>(L.part), K, tiles_n, Z, ldz, rows, labels, off, lse, ctx->at<float>(L.loss),
                       ctx->at<float>(L.coef), ctx->at<__nv_bfloat16>(L.P), L.ldp, ctx->at<uint32_t>(L.status)));
+    return SFB_OK;
+  }
+  if (fused && n == K && n <= kMergeSamples && n * tiles_n <= kMergePartials) {
+    const int lab = label_blocks(ctx);
+    CKC(launch_kernel(mlr_merged_kernel, dim3(grid1d(n * ((rows + 7) / 8), 256) + lab), dim3(256), 0, ctx->stream, 1,
+                      ctx->at<float2>(L.part), K, tiles_n, Z, ldz, rows, static_cast<int32_t>(n), labels, lse, ctx->at<float>(L.loss),
+                      ctx->at<float>(L.coef), ctx->at<int32_t>(L.slot), ctx->at<__nv_bfloat16>(L.P), L.ldp, ctx->at<uint32_t>(L.status),
+                      lab, label_args(ctx, X)));
+    ctx->labels = sfb_ctx::kLabelsApplied;
     return SFB_OK;
   }
   CKC(launch_kernel(mlr_lse_kernel, dim3(static_cast<unsigned>((n + 7) / 8)), dim3(256), 0, ctx->stream, 1,

@@ -74,3 +74,34 @@ def test_logits_on_pairs_repeat():
 @pytest.mark.parametrize("per_worker", [False, True])
 def test_logits_of_few_samples(shape, per_worker):
     check(*shape, per_worker=per_worker)
+
+
+# The softmax of a small mini-batch in one launch: 256 samples and 257, 1 to 32 partials and more than a warp has lanes, classes of one sample
+# and (two classes) of more than eight; a class out of range; the update repeated on the sums that the launch keeps.
+@pytest.mark.parametrize("shape", [(2, 1028, 1, 30), (64, 256, 4, 32), (300, 68, 8, 32), (300, 68, 1, 257), (1030, 260, 1, 40), (2000, 132, 1, 30)])
+def test_merged_softmax(shape):
+    check(*shape)
+
+
+def test_merged_softmax_out_of_range_and_repeated():
+    rows, cols, K = 40, 132, 50
+    W0 = torch.randn(rows, cols, device="cuda") * 0.05
+    X, lab = torch.randn(K, cols, device="cuda"), torch.randint(0, rows, (K,), device="cuda", dtype=torch.int32)
+    lab[7], lab[8] = -1, rows
+    got = []
+    for repeats in (1, 2):
+        W = W0.clone()
+        ctx = S.Context(S.make_config(S.MLR, rows, cols, 1, K, 0.05, S.PREC_BF16), W)
+        ctx.sfb_step(X, None, lab)
+        for _ in range(repeats - 1):
+            ctx.sfb_replay_update()
+        assert ctx.sfb_get_status() == S.STATUS_LABEL_RANGE
+        got.append(W.double())
+        ctx.close()
+    z = X.double() @ W0.double().t()
+    p = torch.softmax(z, 1)
+    ok = (lab >= 0) & (lab < rows)
+    p[ok, lab[ok].long()] -= 1
+    step = -0.05 * p.t() @ X.double()
+    for n, W in enumerate(got, 1):                    # operands in bf16: 2e-3 of the update
+        assert float((W - W0.double() - n * step).norm() / (n * step).norm()) < 2e-3
