@@ -281,8 +281,8 @@ forward_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
 }
 
 // Cycles of a plan: its k-blocks on a pair at the MMAs' rate or 60 bytes a cycle and SM, at least the 8,000 that the end of a tile of 256
-// classes takes; 7,000 from the start to the first MMA and from the last one to the results; 13,000 and 1,000 a part to leave and to
-// take over parts of tiles.  (Fitted to 47 shapes, 64 to 100,000 classes, 170 to 20,000 features, 129 to 1,024 samples: against
+// classes takes; 7,000 from the start to the first MMA and from the last one to the results; 9,000 and 2,000 a part to leave and to
+// take over parts of tiles, of which there are no more than pay for that.  (Fitted to 47 shapes, 64 to 100,000 classes, 170 to 20,000 features, 129 to 1,024 samples: against
 // the best of forward_kernel, whole tiles and cut ones the choice loses 3 % in the middle of the factors' time, 31 % at most, of 12 us;
 // forward_kernel alone 11 %.  us of the product, forward_kernel / here: 10,000 x 20,000 with 1,024 samples 376 / 283, 11,133 x
 // 3,364 with 1,024 79 / 67.)
@@ -297,11 +297,12 @@ PairPlan plan_pairs(int64_t n, int64_t rows, int64_t cols, int64_t max_pairs) {
     const double tile = std::max(static_cast<double>(kseg) * per_kb, 8000.0 * bn / kMaxN);
     PairPlan p{bn, 0, 0, static_cast<int>(std::min(tiles, max_pairs)), static_cast<double>(rounds) * tile + 7000.0};
     const int64_t whole = std::max<int64_t>(0, full - 1) * max_pairs, rest = tiles - whole;
-    const int64_t pairs = full > 0 ? max_pairs : std::max<int64_t>(1, std::min(max_pairs, rest * kseg / 4));
-    const int64_t shared = (rest * kseg + pairs - 1) / pairs;
-    const double cost = static_cast<double>(whole / max_pairs) * tile + static_cast<double>(shared) * per_kb + 20000.0 +
-                        1000.0 * static_cast<double>((pairs + rest - 1) / rest);
-    if (cost < p.cost && rest % pairs != 0) p = PairPlan{bn, 1, static_cast<int>(whole), static_cast<int>(pairs), cost};
+    const int64_t most = full > 0 ? max_pairs : std::max<int64_t>(1, std::min(max_pairs, rest * kseg / 4));
+    for (int64_t parts = 2; (parts - 1) * rest < most; ++parts) {             // of a tile
+      const int64_t pairs = full > 0 ? max_pairs : std::min(most, parts * rest), shared = (rest * kseg + pairs - 1) / pairs;
+      const double cost = static_cast<double>(whole / max_pairs) * tile + static_cast<double>(shared) * per_kb + 16000.0 + 2000.0 * static_cast<double>(parts);
+      if (cost < p.cost && rest % pairs != 0) p = PairPlan{bn, 1, static_cast<int>(whole), static_cast<int>(pairs), cost};
+    }
     if (bn == kMaxN || p.cost < 0.97 * best.cost) best = p;
   }
   return best;

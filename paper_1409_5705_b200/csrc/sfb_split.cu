@@ -967,10 +967,13 @@ __global__ void __launch_bounds__(256) pack_u_kernel(const float* __restrict__ U
 
 // Tile width of a product, whether its contraction is cut, and its SM cycles.  A k-block takes the longer of its MMAs (6 cycles per
 // column by their rate, 7.2 as measured at 256 columns: 1,838) and of its bytes from L2 at 38 a cycle and SM (192 columns: 1,485;
-// 160: 1,395; 64: 1,100).  12,000 cycles from the start to the first MMA and from the last one to the results; 8,000 to leave
-// and to take over a part of a tile: a product of fewer tiles than
-// pairs is cut when that gains more, and not into parts of less than four k-blocks.  (Cutting only the last of several rounds took
-// fewer cycles at a lower clock: 908 -> 1013 us.)
+// 160: 1,395; 64: 1,100).  12,000 cycles from the start to the first MMA and from the last one to the results; 4,000 and 4,500 a part to
+// leave and to take over the parts of a tile, whose adding up waits for one copy after another: a product of fewer tiles than pairs is
+// cut into as many parts a tile as that pays for, and not into parts of less than four k-blocks.  (With 8,000 cycles whatever the
+// parts' number, all pairs took part: metric learning 500 x 8,000 with 256 pairs 31 parts a tile, 95 us a step, 56 now; sparse coding 3,000
+// x 2,000 with 256 samples 888, 503 now; 6,000 x 3,000 with 150 1,178, 897 now; fp32 2,200 x 700 with 600 1,536, 1,076 now; with 3,000
+// and 6,500 cycles a part within a few per cent of this.  Cutting only the last of several rounds took fewer cycles at a lower
+// clock: 908 -> 1013 us.)
 struct ProductPlan { int bn; int64_t tiles, pairs; bool cut; double cost; };
 // fine: drained at every k-block, which the MMAs of a third of it do not hide.
 ProductPlan plan_width(int64_t M, int64_t N, int64_t Kc, bool sym, bool fine, int bn, int64_t max_pairs) {
@@ -983,13 +986,18 @@ ProductPlan plan_width(int64_t M, int64_t N, int64_t Kc, bool sym, bool fine, in
   p.pairs = std::min(p.tiles, max_pairs);
   double kb = static_cast<double>(rounds * kseg);
   if (!sym && p.tiles < max_pairs) {
-    const int64_t pairs = std::max<int64_t>(1, std::min(max_pairs, p.tiles * kseg / 4));
-    const double shared = static_cast<double>((p.tiles * kseg + pairs - 1) / pairs);
-    if ((kb - shared) * per_kb > 8000.0) {
-      p.cut = true;
-      p.pairs = pairs;
-      kb = shared + 8000.0 / per_kb;
+    const int64_t most = std::max<int64_t>(1, std::min(max_pairs, p.tiles * kseg / 4));
+    double least = kb * per_kb;
+    for (int64_t parts = 2; (parts - 1) * p.tiles < most; ++parts) {          // of a tile
+      const int64_t pairs = std::min(most, parts * p.tiles);
+      const double shared = static_cast<double>((p.tiles * kseg + pairs - 1) / pairs), extra = 4000.0 + 4500.0 * static_cast<double>(parts);
+      if (shared * per_kb + extra < least) {
+        least = shared * per_kb + extra;
+        p.cut = true;
+        p.pairs = pairs;
+      }
     }
+    kb = least / per_kb;
   }
   p.cost = kb * per_kb + 12000.0 + static_cast<double>(p.tiles / max_pairs) * 1500.0;
   return p;
