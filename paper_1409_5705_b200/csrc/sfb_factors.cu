@@ -421,6 +421,7 @@ __global__ void mean_kernel(const float* __restrict__ v, int64_t n, float* out, 
 
 // Column sums of squares in fp64 (the prox must resolve norms to far better than fp32's 6e-8, because the
 // rescaling multiplies every entry of W while the step's update is ~1e-3 of ||W||).
+constexpr int kProxLoads = 4;         // rows that a thread of the two passes has under way: 10,000 x 5,000, the scaling 95 us with one, 84 with four
 __global__ void __launch_bounds__(kThreads) col_sumsq_kernel(const float* __restrict__ W, int64_t rows, int64_t cols,
                                                              double* __restrict__ part, int64_t slab_rows) {
   pdl_launch_dependents();
@@ -432,12 +433,18 @@ __global__ void __launch_bounds__(kThreads) col_sumsq_kernel(const float* __rest
   const int64_t r1 = min(rows, r0 + slab_rows);
   double a0 = 0., a1 = 0., a2 = 0., a3 = 0.;
   if (c0 < cols) {
-    for (int64_t r = r0 + ty; r < r1; r += 8) {
-      const float4 w = *reinterpret_cast<const float4*>(W + r * cols + c0);
-      a0 = fma(static_cast<double>(w.x), static_cast<double>(w.x), a0);
-      a1 = fma(static_cast<double>(w.y), static_cast<double>(w.y), a1);
-      a2 = fma(static_cast<double>(w.z), static_cast<double>(w.z), a2);
-      a3 = fma(static_cast<double>(w.w), static_cast<double>(w.w), a3);
+    for (int64_t r = r0 + ty; r < r1; r += 8 * kProxLoads) {
+      float4 w[kProxLoads];
+#pragma unroll
+      for (int k = 0; k < kProxLoads; ++k)
+        w[k] = r + 8 * k < r1 ? *reinterpret_cast<const float4*>(W + (r + 8 * k) * cols + c0) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+      for (int k = 0; k < kProxLoads; ++k) {
+        a0 = fma(static_cast<double>(w[k].x), static_cast<double>(w[k].x), a0);
+        a1 = fma(static_cast<double>(w[k].y), static_cast<double>(w[k].y), a1);
+        a2 = fma(static_cast<double>(w[k].z), static_cast<double>(w[k].z), a2);
+        a3 = fma(static_cast<double>(w[k].w), static_cast<double>(w[k].w), a3);
+      }
     }
   }
   sh[ty][tx * 4 + 0] = a0; sh[ty][tx * 4 + 1] = a1; sh[ty][tx * 4 + 2] = a2; sh[ty][tx * 4 + 3] = a3;
@@ -476,14 +483,20 @@ __global__ void __launch_bounds__(kThreads) prox_scale_kernel(float* __restrict_
   if (s0 == 1. && s1 == 1. && s2 == 1. && s3 == 1.) return;
   const int64_t r0 = static_cast<int64_t>(blockIdx.y) * slab_rows;
   const int64_t r1 = min(rows, r0 + slab_rows);
-  for (int64_t r = r0 + ty; r < r1; r += 8) {
-    float4* p = reinterpret_cast<float4*>(W + r * cols + c0);
-    float4 w = *p;
-    if (s0 != 1.) w.x = static_cast<float>(static_cast<double>(w.x) * s0);
-    if (s1 != 1.) w.y = static_cast<float>(static_cast<double>(w.y) * s1);
-    if (s2 != 1.) w.z = static_cast<float>(static_cast<double>(w.z) * s2);
-    if (s3 != 1.) w.w = static_cast<float>(static_cast<double>(w.w) * s3);
-    *p = w;
+  for (int64_t r = r0 + ty; r < r1; r += 8 * kProxLoads) {
+    float4 w[kProxLoads];
+#pragma unroll
+    for (int k = 0; k < kProxLoads; ++k)
+      if (r + 8 * k < r1) w[k] = *reinterpret_cast<const float4*>(W + (r + 8 * k) * cols + c0);
+#pragma unroll
+    for (int k = 0; k < kProxLoads; ++k) {
+      if (r + 8 * k >= r1) break;
+      if (s0 != 1.) w[k].x = static_cast<float>(static_cast<double>(w[k].x) * s0);
+      if (s1 != 1.) w[k].y = static_cast<float>(static_cast<double>(w[k].y) * s1);
+      if (s2 != 1.) w[k].z = static_cast<float>(static_cast<double>(w[k].z) * s2);
+      if (s3 != 1.) w[k].w = static_cast<float>(static_cast<double>(w[k].w) * s3);
+      *reinterpret_cast<float4*>(W + (r + 8 * k) * cols + c0) = w[k];
+    }
   }
 }
 
