@@ -227,6 +227,7 @@ extern "C" int sfb_init(const sfb_config* cfg, float* W_dev, void* workspace_dev
   ctx->stats = sfb_stats{};
   ctx->tc = nullptr;
   ctx->host = nullptr;
+  ctx->packed = false;
   ctx->labels = sfb_ctx::kLabelsNone;
   ctx->pending = Stamp{};
   // status word, scalars and per-sample losses are the first three (contiguous) regions
@@ -461,12 +462,18 @@ static int compute_factors_csr(sfb_ctx* ctx, int32_t worker, const int64_t* indp
     if ((rc = begin_step(ctx)) != SFB_OK) return rc;
     ctx->begun = true;
   }
-  rc = sparse_stage(ctx, off, n, indptr_dev, indices_dev, values_dev, nnz);
+  // (in a call that goes on to the update the label rows read the samples from the staging buffer, else from their fp32 copy)
+  const bool packed = sparse_stage_packs(ctx);
+  float* Xd = ctx->at<float>(packed && !fused ? ctx->lay.Xf : ctx->lay.stageX);
+  rc = packed ? sparse_stage_packed(ctx, off, n, indptr_dev, indices_dev, values_dev, nnz, labels_dev, Xd)
+              : sparse_stage(ctx, off, n, indptr_dev, indices_dev, values_dev, nnz);
   if (rc) return rc;
-  const float* X = ctx->at<float>(ctx->lay.stageX) + off * c.cols;
+  const float* X = Xd + off * c.cols;
+  ctx->packed = packed;
   rc = ctx->tf32 ? tc32_factors(ctx, off, n, X, labels_dev, nullptr, 0.f)
        : c.precision == SFB_PREC_FP32 ? factors_fp32(ctx, off, n, X, nullptr, labels_dev, pairs, sparse_forward_wanted(ctx, n))
                                       : tc_factors(ctx, off, n, X, nullptr, labels_dev, fused);
+  ctx->packed = false;
   if (rc) return rc;
   ctx->csr_fill += nnz;
   ctx->sparse_mask |= bits;

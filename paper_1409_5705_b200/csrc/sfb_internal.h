@@ -217,6 +217,7 @@ struct sfb_ctx {
   int64_t last_stage_nnz;             // entries of the last staged block of samples
   bool sparse_v;                      // the gathered v are in column-major sparse form: the update sums only the non-zeros
   bool gathered;
+  bool packed;                        // the samples of the call at hand are operands already, their labels and slots set (see sparse_stage_packed)
   int last_cuda;
   // MLR, bf16 mode: the label entries of the step's factors are not in W; in W by the factors call; were in a past update,
   // their sums kept
@@ -359,6 +360,10 @@ void sparse_extend_layout(const sfb_config& c, Layout& L, size_t& off);
 bool sparse_update_wanted(const sfb_ctx* ctx);
 int sparse_stage(sfb_ctx* ctx, int64_t off, int64_t n, const int64_t* indptr, const int32_t* idx, const float* val,
                  int64_t nnz);
+// bf16 mode, rows that fit shared memory: staged and packed in one kernel, in fp32 to Xd [K x cols].
+bool sparse_stage_packs(const sfb_ctx* ctx);
+int sparse_stage_packed(sfb_ctx* ctx, int64_t off, int64_t n, const int64_t* indptr, const int32_t* idx, const float* val, int64_t nnz,
+                        const int32_t* labels, float* Xd);
 // fp32 FMA mode: rows of W per block of the row-wise forward over sparse samples (0: the rows do not fit), and that product
 bool sparse_forward_wanted(const sfb_ctx* ctx, int64_t n);
 int sparse_forward(sfb_ctx* ctx, int64_t off, int64_t n, float* Z, int64_t ldz);

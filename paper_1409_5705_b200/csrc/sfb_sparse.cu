@@ -105,6 +105,69 @@ __global__ void __launch_bounds__(256) csr_stage_kernel(const int64_t* __restric
   }
 }
 
+// bf16 mode: the same with what pack_mlr_kernel does, a block per sample: its row is put together in shared memory and leaves as fp32
+// (for the label rows) and as the bf16 operand, each written once.  Against clearing the staging buffer, scattering into it and
+// packing it: 10,000 x 20,000, 1,024 samples of 30 entries, 27 us instead of 46; a step of 2,000 x 3,000 with 240 samples 59 -> 51 us.
+constexpr int kRowThreads = 512, kRowSmem = 200 << 10;
+struct RowArgs {
+  const int64_t* indptr;
+  const int32_t* idx;
+  const float* val;
+  int64_t nnz, cols, off;
+  float* Xd;                   // [K x cols]
+  uint16_t* Xb;                // [K x ldx] bf16
+  int64_t ldx;
+  const int32_t* labels;
+  int32_t* labels_out;
+  int32_t* slot;
+  int64_t rows;
+  int32_t* coo_i;
+  int32_t* coo_c;
+  float* coo_x;
+  Stamp stamp;
+  uint32_t* status;
+};
+__global__ void __launch_bounds__(kRowThreads) csr_rows_kernel(const RowArgs a) {
+  pdl_launch_dependents();
+  pdl_wait();
+  stamp_begin(a.stamp);
+  extern __shared__ float4 row4[];
+  float* row = reinterpret_cast<float*>(row4);
+  const int t = threadIdx.x, quads = static_cast<int>(a.cols / 4);
+  const int64_t i = blockIdx.x, s = a.off + i;
+  for (int q = t; q < quads; q += kRowThreads) row4[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+  const int64_t base = a.indptr[0];
+  int64_t b = a.indptr[i] - base, e = a.indptr[i + 1] - base;
+  const bool bad = b < 0 || e < b || e > a.nnz;    // row pointers that do not describe nnz entries: sample left empty
+  if (bad) b = e = 0;
+  __syncthreads();
+  for (int64_t k = b + t; k < e; k += kRowThreads) {
+    const int32_t c = a.idx[base + k];
+    const float x = a.val[base + k];
+    if (c < 0 || c >= a.cols) {                    // entry skipped (its slot keeps the "no entry" mark)
+      atomicOr(a.status, SFB_STATUS_INDEX_RANGE);
+      continue;
+    }
+    row[c] = x;
+    a.coo_i[k] = static_cast<int32_t>(s);
+    a.coo_c[k] = c;
+    a.coo_x[k] = x;
+  }
+  if (t == 0) {
+    if (bad) atomicOr(a.status, SFB_STATUS_INDEX_RANGE);
+    const int32_t old = a.labels_out[s];
+    if (old >= 0 && old < a.rows) a.slot[old] = kNoSlot;
+    a.labels_out[s] = a.labels[i];
+  }
+  __syncthreads();
+  for (int q = t; q < quads; q += kRowThreads) {
+    const float4 v = row4[q];
+    reinterpret_cast<float4*>(a.Xd + s * a.cols)[q] = v;
+    const __nv_bfloat162 lo = __floats2bfloat162_rn(v.x, v.y), hi = __floats2bfloat162_rn(v.z, v.w);
+    reinterpret_cast<uint2*>(a.Xb + s * a.ldx)[q] = make_uint2(*reinterpret_cast<const uint32_t*>(&lo), *reinterpret_cast<const uint32_t*>(&hi));
+  }
+}
+
 // ---------------------------------------------------------------------------------------------------------
 // Column-major form of the step's K samples: a counting sort of the triples by column, then every column's
 // entries in ascending sample order (so that the sums of the update have one order, whatever order the atomics
@@ -588,6 +651,27 @@ int sparse_stage(sfb_ctx* ctx, int64_t off, int64_t n, const int64_t* indptr, co
                     ctx->at<int32_t>(L.coo_c) + ctx->csr_fill, ctx->at<float>(L.coo_x) + ctx->csr_fill,
                     ctx->at<int2>(L.coo_cx) + ctx->csr_fill, static_cast<int32_t>(ctx->csr_fill),
                     ctx->at<int32_t>(L.row_beg), ctx->at<int32_t>(L.row_end), ctx->at<uint32_t>(L.status)));
+  ctx->last_stage_nnz = nnz;
+  return SFB_OK;
+}
+
+bool sparse_stage_packs(const sfb_ctx* ctx) { return ctx->cfg.precision == SFB_PREC_BF16 && ctx->cfg.cols * 4 <= kRowSmem; }
+int sparse_stage_packed(sfb_ctx* ctx, int64_t off, int64_t n, const int64_t* indptr, const int32_t* idx, const float* val, int64_t nnz,
+                        const int32_t* labels, float* Xd) {
+  const Layout& L = ctx->lay;
+  cudaStream_t s = ctx->stream;
+  if (nnz > 0) CKS(cudaMemsetAsync(ctx->at<int32_t>(L.coo_c) + ctx->csr_fill, 0xff, static_cast<size_t>(nnz) * 4, s));   // "no entry"
+  RowArgs a{};
+  a.indptr = indptr; a.idx = idx; a.val = val; a.nnz = nnz; a.cols = ctx->cfg.cols; a.off = off;
+  a.Xd = Xd;
+  a.Xb = ctx->at<uint16_t>(L.Xb); a.ldx = L.colsb;
+  a.labels = labels; a.labels_out = ctx->at<int32_t>(L.labels); a.slot = ctx->at<int32_t>(L.slot); a.rows = ctx->cfg.rows;
+  a.coo_i = ctx->at<int32_t>(L.coo_i) + ctx->csr_fill;
+  a.coo_c = ctx->at<int32_t>(L.coo_c) + ctx->csr_fill;
+  a.coo_x = ctx->at<float>(L.coo_x) + ctx->csr_fill;
+  a.stamp = take_stamp(ctx); a.status = ctx->at<uint32_t>(L.status);
+  CKS(allow_smem<csr_rows_kernel>(kRowSmem));
+  CKS(launch_kernel(csr_rows_kernel, dim3(static_cast<unsigned>(n)), dim3(kRowThreads), static_cast<size_t>(a.cols) * 4, s, 1, a));
   ctx->last_stage_nnz = nnz;
   return SFB_OK;
 }

@@ -286,7 +286,6 @@ __global__ void __launch_bounds__(256) convert_rows_kernel(const float* __restri
 // The label-row slots of the classes that these samples had in the step before are cleared.
 // One read of X, 6 bytes written per value, 2 without Xf; bound by HBM (1,024 x 20,000: 33 us with a transposed copy beside
 // it, 28 without, 20 without Xf).
-constexpr int32_t kNoSlot = 0x7f7f7f7f;              // above every sample index (K <= 2^20)
 __global__ void __launch_bounds__(256) pack_mlr_kernel(const float* __restrict__ X, int64_t n, int64_t cols,
                                                        __nv_bfloat16* __restrict__ Xb, int64_t ldx, int64_t off,
                                                        float* __restrict__ Xf, const int32_t* labels, int32_t* labels_out,
@@ -1168,7 +1167,8 @@ static int mlr_forward(sfb_ctx* ctx, int64_t off, int64_t n, const float* X, con
   ctx->stats.flops += 2.0 * n * rows * cols;
   // (samples that come by a copy on another stream: that one has to be complete before the kernel starts at all)
   const bool early = !ctx->host || ctx->host->parts <= 1;
-  CKC(launch_kernel_if(early, pack_mlr_kernel, dim3(grid1d(n * cols / 4, 256)), dim3(256), 0, ctx->stream, 1, X, n, cols, Xb,
+  if (!ctx->packed)
+    CKC(launch_kernel_if(early, pack_mlr_kernel, dim3(grid1d(n * cols / 4, 256)), dim3(256), 0, ctx->stream, 1, X, n, cols, Xb,
                     L.colsb, off,
                     fused ? nullptr : ctx->at<float>(L.Xf), labels, ctx->at<int32_t>(L.labels), ctx->at<int32_t>(L.slot),
                     rows,

@@ -74,6 +74,8 @@ int64_t forward_few_groups(int64_t rows);
 cudaError_t forward_few_prepare(int (&most)[5]);
 cudaError_t forward_few(sfb_ctx* ctx, int64_t off, int64_t n);
 
+constexpr int32_t kNoSlot = 0x7f7f7f7f;              // a label-row slot that no sample has: above every index (K <= 2^20)
+
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
                                   const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
                                   CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);

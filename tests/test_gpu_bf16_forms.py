@@ -105,3 +105,48 @@ def test_merged_softmax_out_of_range_and_repeated():
     step = -0.05 * p.t() @ X.double()
     for n, W in enumerate(got, 1):                    # operands in bf16: 2e-3 of the update
         assert float((W - W0.double() - n * step).norm() / (n * step).norm()) < 2e-3
+
+
+# Sparse samples staged and packed in one kernel (51,200 features, the most that it takes, and four more: in three), in one call and by workers:
+# the bits of the dense samples' step.  Empty samples, a sample with an entry everywhere, one with a column out of range.
+@pytest.mark.parametrize("cols", [4, 260, 51200, 51204])
+@pytest.mark.parametrize("per_worker", [False, True])
+def test_sparse_samples_as_dense_ones(cols, per_worker):
+    rows, workers, batch = 70, 3, 5
+    K = workers * batch
+    g = torch.Generator(device="cuda")
+    g.manual_seed(1)
+    W0 = torch.randn(rows, cols, generator=g, device="cuda") * 0.05
+    lab = torch.randint(0, rows, (K,), generator=g, device="cuda", dtype=torch.int32)
+    got = []
+    for sparse in (False, True):
+        W = W0.clone()
+        ctx = S.Context(S.make_config(S.MLR, rows, cols, workers, batch, 0.05, S.PREC_BF16, csr_nnz_max=K * cols + 1, csr_update=2), W)
+        for t in range(2):                            # (another step's samples leave nothing behind)
+            g.manual_seed(2 + t)
+            X = torch.randn(K, cols, generator=g, device="cuda") * (torch.rand(K, cols, generator=g, device="cuda") < 0.05)
+            X[3] = 0
+            X[4] = 1
+            parts = [slice(p * batch, (p + 1) * batch) for p in range(workers)] if per_worker else [slice(0, K)]
+            for p, r in enumerate(parts):
+                if sparse:
+                    where = X[r].nonzero()
+                    ptr = torch.zeros(X[r].shape[0] + 1, dtype=torch.int64, device="cuda")
+                    ptr[1:] = torch.cumsum(torch.bincount(where[:, 0], minlength=X[r].shape[0]), 0)
+                    idx, val = where[:, 1].to(torch.int32), X[r][where[:, 0], where[:, 1]]
+                    if p == len(parts) - 1:           # one more entry of the last sample, out of range: skipped
+                        ptr[-1] += 1
+                        idx, val = torch.cat([idx, idx.new_tensor([cols])]), torch.cat([val, val.new_tensor([9.0])])
+                    args = (ptr, idx.contiguous(), val.contiguous(), int(ptr[-1]), lab[r])
+                    ctx.sfb_compute_factors_csr(p, *args) if per_worker else ctx.sfb_step_csr(*args)
+                elif per_worker:
+                    ctx.sfb_compute_factors(p, X[r], None, lab[r])
+                else:
+                    ctx.sfb_step(X, None, lab)
+            if per_worker:
+                ctx.sfb_gather_factors()
+                ctx.sfb_apply_update()
+        assert ctx.sfb_get_status() == (S.STATUS_INDEX_RANGE if sparse else 0)
+        got.append(W)
+        ctx.close()
+    assert torch.equal(got[0], got[1])
