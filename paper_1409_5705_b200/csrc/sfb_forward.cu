@@ -298,7 +298,7 @@ PairPlan plan_pairs(int64_t n, int64_t rows, int64_t cols, int64_t max_pairs) {
     PairPlan p{bn, 0, 0, static_cast<int>(std::min(tiles, max_pairs)), static_cast<double>(rounds) * tile + 7000.0};
     const int64_t whole = std::max<int64_t>(0, full - 1) * max_pairs, rest = tiles - whole;
     const int64_t most = full > 0 ? max_pairs : std::max<int64_t>(1, std::min(max_pairs, rest * kseg / 4));
-    for (int64_t parts = 2; (parts - 1) * rest < most; ++parts) {             // of a tile
+    for (int64_t parts = 2; (full > 0 && parts == 2) || (parts - 1) * rest < most; ++parts) {      // of a tile
       const int64_t pairs = full > 0 ? max_pairs : std::min(most, parts * rest), shared = (rest * kseg + pairs - 1) / pairs;
       const double cost = static_cast<double>(whole / max_pairs) * tile + static_cast<double>(shared) * per_kb + 16000.0 + 2000.0 * static_cast<double>(parts);
       if (cost < p.cost && rest % pairs != 0) p = PairPlan{bn, 1, static_cast<int>(whole), static_cast<int>(pairs), cost};
