@@ -2,7 +2,8 @@
 // logistic regression (Sections 1 and 2: u = softmax(W x) - onehot(y), v = x) and the operand packing of the
 // update product.  The update product itself is in sfb_update.cu, the products of (hi | lo) pairs in sfb_split.cu.
 //
-// Forward product: one persistent, warp-specialised kernel computes  Z (K x rows) = X (K x cols) * W^T  with bf16
+// Forward product (of 65 to 128 samples or many rounds of tiles, and of tf32 words; the others: sfb_forward.cu): one persistent,
+// warp-specialised kernel computes  Z (K x rows) = X (K x cols) * W^T  with bf16
 // operands staged by TMA into 128-byte-swizzled shared memory, tcgen05.mma accumulating in TMEM (two 128 x 256
 // fp32 accumulators, so the epilogue of one tile overlaps the main loop of the next).  The epilogue stores Z as
 // fp32 and, per (sample, 256-row block), the softmax partials (max, sum of exp).
@@ -598,10 +599,12 @@ __global__ void __launch_bounds__(256) mlr_emit_p_kernel(const float* __restrict
   }
 }
 
-// Merged softmax of a small mini-batch (up to 256 samples, few partials): one launch instead of mlr_lse_kernel and mlr_emit_p_kernel,
-// 3 of the 20 us of a step at 64 x 256 with 128 samples.  Every block merges the partials of all samples itself (the same sums as
-// mlr_lse_kernel's); the label blocks find a class's first sample in shared memory, as its slots are only just being set here.
-constexpr int kMergeSamples = 256, kMergePartials = 2048;
+// Merged softmax of a small mini-batch (up to 128 samples, eight partials): one launch instead of mlr_lse_kernel and mlr_emit_p_kernel,
+// 1.6 of the 20 us of a step at 64 x 256 with 128 samples.  Every block merges the partials of all samples itself, a sample per
+// thread with all loads under way, in the order of mlr_lse_kernel's lanes; the label blocks find a class's samples in shared
+// memory, as its slots are only just being set here.  (With more partials, a sample's over several lanes and so the samples in several
+// passes: 405 x 940 with 102 samples and 13 partials 28 -> 38 us; with more samples the search for a class: 191 x 140 with 225 25.6 -> 28.4.)
+constexpr int kMergeSamples = 128, kMergePartials = 8;
 __global__ void __launch_bounds__(256) mlr_merged_kernel(const float2* __restrict__ part, int64_t part_ld, int nblocks,
                                                          const float* __restrict__ Z, int64_t ldz, int64_t rows, int32_t n,
                                                          const int32_t* __restrict__ labels, float* __restrict__ lse,
@@ -614,31 +617,29 @@ __global__ void __launch_bounds__(256) mlr_merged_kernel(const float2* __restric
   __shared__ int32_t sh_y[kMergeSamples], sh_next[kMergeSamples];
   __shared__ bool sh_first[kMergeSamples];
   const int t = threadIdx.x, lane = t & 31;
-  // lanes of a sample: the power of two that the partials fill, at most 32
-  int width = 32;
-  while (width > 1 && width / 2 >= nblocks) width /= 2;
-  const int sub = t % width;
-  for (int i = t / width; i < (n + 256 / width - 1) / (256 / width) * (256 / width); i += 256 / width) {
-    float m = -INFINITY, sum = 0.f;
-    if (i < n)
-      for (int b = sub; b < nblocks; b += width) m = fmaxf(m, part[static_cast<int64_t>(b) * part_ld + i].x);
-    for (int o = width / 2; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-    if (i < n)
-      for (int b = sub; b < nblocks; b += width) {
-        const float2 v = part[static_cast<int64_t>(b) * part_ld + i];
-        sum += v.y * __expf(v.x - m);
-      }
-    for (int o = width / 2; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-    if (sub == 0 && i < n) {
-      const float l = m + logf(sum);
-      const int32_t y = labels[i];
-      const bool ok = y >= 0 && y < rows;
-      const float zy = ok ? Z[i * ldz + y] : 0.f;
-      sh_lse[i] = l;
-      sh_y[i] = ok ? y : -1;
-      sh_loss[i] = ok ? l - zy : 0.f;
-      sh_coef[i] = ok ? -expm1f(zy - l) : 0.f;
-    }
+  if (t < n) {
+    float2 v[kMergePartials];
+#pragma unroll
+    for (int b = 0; b < kMergePartials; ++b)
+      v[b] = b < nblocks ? part[static_cast<int64_t>(b) * part_ld + t] : make_float2(-INFINITY, 0.f);
+    const int32_t y = labels[t];
+    const bool ok = y >= 0 && y < rows;
+    const float zy = ok ? Z[t * ldz + y] : 0.f;
+    float m = v[0].x;
+#pragma unroll
+    for (int b = 1; b < kMergePartials; ++b) m = fmaxf(m, v[b].x);
+    float e[kMergePartials];
+#pragma unroll
+    for (int b = 0; b < kMergePartials; ++b) e[b] = b < nblocks ? v[b].y * __expf(v[b].x - m) : 0.f;
+#pragma unroll
+    for (int o = kMergePartials / 2; o > 0; o >>= 1)
+#pragma unroll
+      for (int b = 0; b < o; ++b) e[b] += e[b + o];
+    const float l = m + logf(e[0]);
+    sh_lse[t] = l;
+    sh_y[t] = ok ? y : -1;
+    sh_loss[t] = ok ? l - zy : 0.f;
+    sh_coef[t] = ok ? -expm1f(zy - l) : 0.f;
   }
   __syncthreads();
   const int blk = static_cast<int>(blockIdx.x);
@@ -1440,7 +1441,7 @@ int tc_factors(sfb_ctx* ctx, int64_t off, int64_t n, const float* X, const float
                       ctx->at<float>(L.coef), ctx->at<__nv_bfloat16>(L.P), L.ldp, ctx->at<uint32_t>(L.status)));
     return SFB_OK;
   }
-  if (fused && n == K && n <= kMergeSamples && n * tiles_n <= kMergePartials) {
+  if (fused && n == K && n <= kMergeSamples && tiles_n <= kMergePartials) {
     const int lab = label_blocks(ctx);
     CKC(launch_kernel(mlr_merged_kernel, dim3(grid1d(n * ((rows + 7) / 8), 256) + lab), dim3(256), 0, ctx->stream, 1,
                       ctx->at<float2>(L.part), K, tiles_n, Z, ldz, rows, static_cast<int32_t>(n), labels, lse, ctx->at<float>(L.loss),
