@@ -19,7 +19,7 @@ STATUS_LABEL_RANGE, STATUS_TIMEOUT, STATUS_SAMPLE_RANGE, STATUS_INDEX_RANGE = 0x
 
 EXPORTS = ("sfb_workspace_bytes", "sfb_init", "sfb_compute_factors", "sfb_gather_factors", "sfb_apply_update",
            "sfb_step", "sfb_step_host", "sfb_dense_sync_step", "sfb_get_factors", "sfb_get_stats",
-           "sfb_get_update_form", "sfb_get_status", "sfb_strerror", "sfb_last_cuda_error", "sfb_destroy", "sfb_prox_columns_noalloc",
+           "sfb_get_update_form", "sfb_get_plan", "sfb_get_status", "sfb_strerror", "sfb_last_cuda_error", "sfb_destroy", "sfb_prox_columns_noalloc",
            "sfb_selftest_wait_timeout", "sfb_set_row_shard", "sfb_forward_partials", "sfb_finish_factors",
            "sfb_replay_update", "sfb_refresh_operands", "sfb_sdca_set_dual", "sfb_sdca_compute_factors",
            "sfb_sdca_step", "sfb_set_factors", "sfb_set_eta", "sfb_get_operand_copy", "sfb_compute_factors_csr",
@@ -76,6 +76,7 @@ def lib() -> ctypes.CDLL:
         L.sfb_get_factors.argtypes = [vp, ctypes.POINTER(vp), ctypes.POINTER(vp), ctypes.POINTER(i32),
                                       ctypes.POINTER(i32), ctypes.POINTER(i64), ctypes.POINTER(i64)]
         L.sfb_get_stats.argtypes = [vp, ctypes.POINTER(sfb_stats)]
+        L.sfb_get_plan.argtypes = [cfgp, i64] + [ctypes.POINTER(i32)] * 3
         L.sfb_get_status.argtypes = [vp, ctypes.POINTER(ctypes.c_uint32)]
         L.sfb_strerror.argtypes = [ctypes.c_int]
         L.sfb_strerror.restype = ctypes.c_char_p
@@ -122,6 +123,15 @@ def sfb_workspace_bytes(cfg: sfb_config) -> int:
     if rc:
         raise SfbError(rc, "sfb_workspace_bytes")
     return out.value
+
+
+def sfb_get_plan(cfg: sfb_config, samples: int):
+    """(product, parts, merged) of a factors call of ``samples`` samples; see include/sfb.h."""
+    out = [ctypes.c_int32(0) for _ in range(3)]
+    rc = lib().sfb_get_plan(ctypes.byref(cfg), samples, *(ctypes.byref(o) for o in out))
+    if rc:
+        raise SfbError(rc, "sfb_get_plan")
+    return tuple(o.value for o in out)
 
 
 def _ptr(t):

@@ -975,6 +975,35 @@ extern "C" int sfb_get_update_form(sfb_ctx* ctx, int32_t* form) {
   return SFB_OK;
 }
 
+extern "C" int sfb_get_plan(const sfb_config* cfg, int64_t samples, int32_t* product, int32_t* parts, int32_t* merged) {
+  const int rc = check_config(cfg);
+  if (rc) return rc;
+  if (!product || !parts || !merged) return SFB_ERR_ARG;
+  sfb_config c = *cfg;
+  if (samples < 1 || samples > static_cast<int64_t>(c.workers) * c.batch) return SFB_ERR_SHAPE;
+  if (c.model == SFB_L2MLR) c.model = SFB_MLR;
+  int form = 0, cut = 1;
+  bool one = false;
+  if (use_tf32(c)) {
+    form = 4;
+  } else if (c.model == SFB_SC && !use_h16(c) && c.precision != SFB_PREC_BF16) {
+    form = sc_use_gram64(c) ? 7 : 0;
+  } else if (c.model == SFB_SC) {
+    form = sc_use_gram(c) ? 6 : 5;
+    cut = split_product_parts(samples, form == 6 ? c.cols : c.rows, c.cols, c.precision != SFB_PREC_BF16);
+  } else if (use_h16(c) || (c.precision == SFB_PREC_BF16 && c.model == SFB_DML)) {
+    form = 5;
+    cut = split_product_parts(samples, c.rows, c.cols, false);
+  } else if (c.precision == SFB_PREC_BF16) {
+    form = tc_logits_plan(c, make_layout(*cfg), samples, &cut, &one);
+    one = one && cfg->model == SFB_MLR && samples == static_cast<int64_t>(c.workers) * c.batch;
+  }
+  *product = form;
+  *parts = cut;
+  *merged = one;
+  return SFB_OK;
+}
+
 extern "C" int sfb_get_stats(sfb_ctx* ctx, sfb_stats* out) {
   if (!ctx || !out) return SFB_ERR_ARG;
   const sfb_config& c = ctx->cfg;

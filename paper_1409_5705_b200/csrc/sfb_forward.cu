@@ -315,6 +315,20 @@ PairPlan plan_pairs(const sfb_ctx* ctx, int64_t n) {
 }  // namespace
 
 double forward_pair_cost(int64_t n, int64_t rows, int64_t cols) { return plan_pairs(n, rows, cols, kModelSms / 2).cost; }
+// Against a product of `other` cycles (by forward_cost) with `other_groups` softmax partials a sample.  The two models were fitted apart: held
+// against each other, on 1,278 shapes of 129 to 2,048 samples, 2 to 300,000 classes and 32 to 24,000 features, the pairs are the better
+// ones where a third more, 13,000 cycles where tiles are cut, and 2,400 per 32 partials that the softmax has to merge (a pair's tile
+// of 256 classes leaves two) still come to less.  With that the choice costs a step, fused or by calls, more than 3 % in 29 of 2,556 cases,
+// by the models as they are in 271: 36,667 x 912 with 364 samples 145 us on forward_kernel, 174 on pairs, 78,798 x 1,716 with 156
+// 396 and 458, 121 x 3,772 with 180 35.8 and 39.6.
+bool forward_pair_pays(int64_t n, int64_t rows, int64_t cols, double other, int64_t other_groups, int* parts) {
+  const PairPlan p = plan_pairs(n, rows, cols, kModelSms / 2);
+  const int64_t half = p.bn / 2, tiles = (n + PM - 1) / PM * ((rows + p.bn - 1) / p.bn);
+  const double groups = static_cast<double>((rows + half - 1) / half - other_groups);
+  if (1.35 * p.cost + (p.cut ? 13000.0 : 0.0) + 2400.0 * groups / 32.0 >= other) return false;
+  *parts = p.cut ? std::max(2, static_cast<int>((p.pairs + tiles - p.whole - 1) / (tiles - p.whole))) : 1;
+  return true;
+}
 int64_t forward_pair_groups(int64_t rows) { return rows <= kNarrowRows ? (rows + 31) / 32 : (rows + kMaxN / 2 - 1) / (kMaxN / 2); }
 size_t forward_pair_partial_bytes() { return static_cast<size_t>(kModelSms / 2) * 2 * kEpi * 4 * kSlot; }
 size_t forward_pair_ready_bytes() { return static_cast<size_t>(kModelSms / 2) * 2 * kEpi * 4; }

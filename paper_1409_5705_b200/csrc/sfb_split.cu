@@ -1221,6 +1221,11 @@ double split_product_cost(int64_t M, int64_t N, int64_t Kc, bool sym, bool fine)
   return plan_product(M, N, Kc, sym, fine, kModelSms / 2).cost;
 }
 
+int split_product_parts(int64_t M, int64_t N, int64_t Kc, bool fine) {
+  const ProductPlan p = plan_product(M, N, Kc, false, fine, kModelSms / 2);
+  return p.cut ? std::max(2, static_cast<int>((p.pairs + p.tiles - 1) / p.tiles)) : 1;
+}
+
 void split_extend_layout(const sfb_config& c, Layout& L, size_t& off) {
   auto take = [&](size_t bytes) { size_t o = off; off += (bytes + kAlign - 1) / kAlign * kAlign; return o; };
   const size_t K = static_cast<size_t>(c.workers) * c.batch;

@@ -928,13 +928,39 @@ static int pick_forward_split(int64_t K, int64_t rows, int64_t cols) {
 }
 
 // Whether the logits of n samples take the kernel of CTA pairs.  Not beyond five rounds of its tiles, where an uneven last one matters
-// little and the step is at the power limit (325,000 x 10,000 with 1,024 samples: 5,280 us of the factors' time here, 5,470 there).  A
-// contraction split over a cluster costs 24,000 cycles more than forward_cost has for it (989 x 2,036 with 193 samples 40 us
-// of the factors' time, 18 on pairs; 873 x 2,800 with 634 38 and 25).
-static bool forward_on_pairs(const sfb_config& c, const Layout& L, int64_t n) {
+// little and the step is at the power limit (325,000 x 10,000 with 1,024 samples: 5,280 us of the factors' time here, 5,470 there).
+// What forward_cost has for a split contraction chooses among splits; against another kernel it needs 22,000 cycles more, and its rounds are
+// those of the clusters that are resident at a time (15 of eight CTAs, 120 of the 148 SMs: the factors of 281 x 7,060 with 146 samples,
+// 144 CTAs, 33.6 us, 22.9 on pairs; 870 x 1,012 with 218, 112 CTAs, 16.5 and 14.0).
+static bool forward_on_pairs(const sfb_config& c, const Layout& L, int64_t n, int* parts) {
   if (n <= BM || !L.partial || ((n + 255) / 256) * ((c.rows + 255) / 256) >= 5 * (kModelSms / 2)) return false;
   const int bn = pick_forward_width(n, c.rows, c.cols, L.pw, L.split);
-  return forward_pair_cost(n, c.rows, c.cols) < forward_cost(n, c.rows, c.cols, bn, L.split) + (L.split > 1 ? 24000.0 : 0.0);
+  double cost = forward_cost(n, c.rows, c.cols, bn, L.split);
+  if (L.split > 1) {
+    const int64_t clusters = ((n + BM - 1) / BM) * ((c.rows + bn - 1) / bn), resident = L.split == 2 ? 74 : L.split == 4 ? 33 : 15;
+    const int64_t by_ctas = (clusters * L.split + kModelSms - 1) / kModelSms, rounds = (clusters + resident - 1) / resident;
+    cost = (cost / static_cast<double>(by_ctas) - 3000.0 + 22000.0) * static_cast<double>(rounds);
+  }
+  return forward_pair_pays(n, c.rows, c.cols, cost, (c.rows + L.pw - 1) / L.pw, parts);
+}
+
+// The kernel that forms the logits of n samples, in bf16 mode.
+enum LogitsKernel { kLogitsTiles = 1, kLogitsPairs = 2, kLogitsFew = 3 };
+static LogitsKernel logits_kernel(const sfb_config& c, const Layout& L, int64_t n, int* parts) {
+  *parts = L.split;
+  if (forward_few_fits(n, c.rows, c.cols)) return kLogitsFew;
+  return forward_on_pairs(c, L, n, parts) ? kLogitsPairs : kLogitsTiles;
+}
+
+// Whether the softmax of a step's n samples, `partials` of each, is merged by mlr_merged_kernel.
+static bool softmax_merged(int64_t n, int64_t partials) { return n <= kMergeSamples && partials <= kMergePartials; }
+
+int tc_logits_plan(const sfb_config& c, const Layout& L, int64_t n, int* parts, bool* merged) {
+  const LogitsKernel k = logits_kernel(c, L, n, parts);
+  const int64_t pw = k == kLogitsFew ? 32 : L.pw;
+  *merged = k != kLogitsPairs && softmax_merged(n, (c.rows + pw - 1) / pw);
+  if (k == kLogitsFew) *parts = 1;
+  return k;
 }
 
 // fp32 mode on the tensor cores (MLR): fp32 pair-major factors as in the FFMA path, plus the (big | small) tf32
@@ -1174,12 +1200,14 @@ static int mlr_forward(sfb_ctx* ctx, int64_t off, int64_t n, const float* X, con
                     fused ? nullptr : ctx->at<float>(L.Xf), labels, ctx->at<int32_t>(L.labels), ctx->at<int32_t>(L.slot),
                     rows,
                     take_stamp(ctx)));
-  if (forward_few_fits(n, rows, cols)) {
+  int cut = 1;
+  const LogitsKernel kernel = logits_kernel(c, L, n, &cut);
+  if (kernel == kLogitsFew) {
     CKC(forward_few(ctx, off, n));
     *parts = static_cast<int>(forward_few_groups(rows));
     return SFB_OK;
   }
-  if (forward_on_pairs(c, L, n)) {
+  if (kernel == kLogitsPairs) {
     int pw = 0;
     CKC(forward_pair(ctx, off, n, &pw));
     *parts = static_cast<int>((rows + pw - 1) / pw);
@@ -1397,8 +1425,10 @@ int tc_host_parts(const sfb_ctx* ctx) {
   auto total = [&](int parts) {
     const int64_t n = ctx->K / parts;
     const double copy = 4.0 * static_cast<double>(n) * static_cast<double>(c.cols) / 45e9 + 4e-6;
-    const double cycles = forward_on_pairs(c, ctx->lay, n) ? forward_pair_cost(n, c.rows, c.cols)
-                                                           : forward_cost(n, c.rows, c.cols, pick_forward_width(n, c.rows, c.cols, ctx->lay.pw, 1), 1);
+    int cut = 1;
+    const double cycles = logits_kernel(c, ctx->lay, n, &cut) == kLogitsPairs
+                              ? forward_pair_cost(n, c.rows, c.cols)
+                              : forward_cost(n, c.rows, c.cols, pick_forward_width(n, c.rows, c.cols, ctx->lay.pw, 1), 1);
     const double product = std::max(cycles / 1.7e9, 2.0 * static_cast<double>(c.rows) * static_cast<double>(c.cols) / 5e12) + 5e-6;
     // (a product that takes much longer than its copy has little to gain, and a pass over W per part to lose)
     return parts > 1 && product > 2. * copy ? 1e9 : copy + (parts - 1) * std::max(copy, product) + product;
@@ -1441,7 +1471,7 @@ int tc_factors(sfb_ctx* ctx, int64_t off, int64_t n, const float* X, const float
                       ctx->at<float>(L.coef), ctx->at<__nv_bfloat16>(L.P), L.ldp, ctx->at<uint32_t>(L.status)));
     return SFB_OK;
   }
-  if (fused && n == K && n <= kMergeSamples && tiles_n <= kMergePartials) {
+  if (fused && n == K && softmax_merged(n, tiles_n)) {
     const int lab = label_blocks(ctx);
     CKC(launch_kernel(mlr_merged_kernel, dim3(grid1d(n * ((rows + 7) / 8), 256) + lab), dim3(256), 0, ctx->stream, 1,
                       ctx->at<float2>(L.part), K, tiles_n, Z, ldz, rows, static_cast<int32_t>(n), labels, lse, ctx->at<float>(L.loss),

@@ -54,6 +54,9 @@ int split_pack_received(sfb_ctx* ctx, int64_t off, int64_t n);
 int split_gather(sfb_ctx* ctx);
 const uint16_t* split_v(const sfb_ctx* ctx);
 double split_product_cost(int64_t M, int64_t N, int64_t Kc, bool sym, bool fine = false);     // fine: sparse coding in fp32 mode
+int split_product_parts(int64_t M, int64_t N, int64_t Kc, bool fine);                         // that a tile is cut into, at most
+// MLR, bf16 mode: the kernel of the logits of n samples (see sfb_get_plan) and the parts of a tile; whether the softmax is merged in one launch.
+int tc_logits_plan(const sfb_config& c, const Layout& L, int64_t n, int* parts, bool* merged);
 int tc_update(sfb_ctx* ctx);
 int tc_get_factors(sfb_ctx* ctx, const void** U, const void** V, int32_t* dtype, int32_t* layout, int64_t* ldu,
                    int64_t* ldv);
@@ -61,6 +64,7 @@ int tc_get_factors(sfb_ctx* ctx, const void** U, const void** V, int32_t* dtype,
 // The forward product on pairs of CTAs (sfb_forward.cu): its cycles; its buffers (parts of tiles, their flags); the logits of n packed
 // samples at pair offset off, *pw: classes per softmax partial.
 double forward_pair_cost(int64_t n, int64_t rows, int64_t cols);
+bool forward_pair_pays(int64_t n, int64_t rows, int64_t cols, double other, int64_t other_groups, int* parts);
 int64_t forward_pair_groups(int64_t rows);           // most softmax partials of a sample
 size_t forward_pair_partial_bytes();
 size_t forward_pair_ready_bytes();

@@ -1,0 +1,38 @@
+"""Which kernels a configuration takes (host arithmetic; no GPU)."""
+import ctypes
+
+import pytest
+
+import paper_1409_5705_b200 as S
+
+TILES, PAIRS, FEW = 1, 2, 3
+
+
+def bf16(rows, cols, samples, workers=1, **more):
+    return S.make_config(S.MLR, rows, cols, workers, samples // workers, 0.05, S.PREC_BF16, **more)
+
+
+def test_arguments():
+    cfg = bf16(64, 256, 128)
+    assert S.sfb_get_plan(cfg, 128)[0] == TILES and S.sfb_get_plan(cfg, 64)[0] == FEW
+    for n in (0, 129):
+        with pytest.raises(S.SfbError):
+            S.sfb_get_plan(cfg, n)
+    assert S.lib().sfb_get_plan(ctypes.byref(cfg), 1, None, None, None) == -1
+    assert S.sfb_get_plan(S.make_config(S.MLR, 64, 256, 1, 8, 0.1, S.PREC_TF32X3), 8) == (4, 1, 0)
+    assert S.sfb_get_plan(S.make_config(S.MLR, 64, 256, 1, 8, 0.1, S.PREC_FP32_FFMA), 8) == (0, 1, 0)
+
+
+# Logits where pairs of CTAs take longer than forward_kernel: many classes with few features, whose softmax has twice the partials to
+# merge; two and a half rounds of short tiles; a few tiles of a long contraction, which clusters of eight cut as well.
+@pytest.mark.parametrize("rows,cols,samples", [(36_667, 912, 364), (78_798, 1_716, 156), (44_790, 2_884, 237), (121, 3_772, 180),
+                                               (3, 6_764, 244), (89, 6_608, 533), (9_760, 200, 300), (190, 708, 513)])
+def test_logits_that_pairs_would_slow_down(rows, cols, samples):
+    assert S.sfb_get_plan(bf16(rows, cols, samples), samples)[0] == TILES
+
+
+# ... and where they are the faster ones: uneven rounds of long tiles, clusters that are not all resident.
+@pytest.mark.parametrize("rows,cols,samples", [(10_000, 20_000, 1_024), (10_000, 4_000, 512), (20_000, 4_000, 256), (281, 7_060, 146),
+                                               (2_220, 2_588, 144), (873, 2_800, 634)])
+def test_logits_on_pairs(rows, cols, samples):
+    assert S.sfb_get_plan(bf16(rows, cols, samples), samples)[0] == PAIRS
