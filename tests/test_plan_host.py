@@ -14,7 +14,7 @@ def bf16(rows, cols, samples, workers=1, **more):
 
 def test_arguments():
     cfg = bf16(64, 256, 128)
-    assert S.sfb_get_plan(cfg, 128)[0] == TILES and S.sfb_get_plan(cfg, 64)[0] == FEW
+    assert S.sfb_get_plan(cfg, 128)[0] == TILES and S.sfb_get_plan(cfg, 32)[0] == FEW
     for n in (0, 129):
         with pytest.raises(S.SfbError):
             S.sfb_get_plan(cfg, n)
@@ -36,3 +36,11 @@ def test_logits_that_pairs_would_slow_down(rows, cols, samples):
                                                (2_220, 2_588, 144), (873, 2_800, 634)])
 def test_logits_on_pairs(rows, cols, samples):
     assert S.sfb_get_plan(bf16(rows, cols, samples), samples)[0] == PAIRS
+
+
+# Up to 64 samples: the kernel of few samples, but for more than 40 with fewer than 12 k-blocks and for the longest contractions of a few tiles.
+@pytest.mark.parametrize("rows,cols,samples,few", [(64, 64, 40, True), (64, 64, 41, False), (300, 708, 64, True), (300, 704, 64, False), (3_048, 268, 56, False),
+                                                   (107, 84, 44, False), (4_999, 3_004, 64, True), (4_999, 3_004, 65, False),
+                                                   (512, 18_000, 8, True), (512, 18_004, 8, False), (513, 24_000, 64, True)])
+def test_logits_of_few_samples(rows, cols, samples, few):
+    assert (S.sfb_get_plan(bf16(rows, cols, samples), samples)[0] == FEW) == few
