@@ -600,10 +600,13 @@ __global__ void __launch_bounds__(256) mlr_emit_p_kernel(const float* __restrict
 }
 
 // Merged softmax of a small mini-batch (up to 128 samples, eight partials): one launch instead of mlr_lse_kernel and mlr_emit_p_kernel,
-// 1.6 of the 20 us of a step at 64 x 256 with 128 samples.  Every block merges the partials of all samples itself, a sample per
+// 1.2 of the 20 us of a step at 64 x 256 with 128 samples.  Every block merges the partials of all samples itself, a sample per
 // thread with all loads under way, in the order of mlr_lse_kernel's lanes; the label blocks find a class's samples in shared
-// memory, as its slots are only just being set here.  (With more partials, a sample's over several lanes and so the samples in several
-// passes: 405 x 940 with 102 samples and 13 partials 28 -> 38 us; with more samples the search for a class: 191 x 140 with 225 25.6 -> 28.4.)
+// memory, as its slots are only just being set here, and follow its chain while the eight samples before are on their way.  (Followed
+// between the loads, a popular class made the launch slower than the two: 4 x 256 with 100 Zipf labels 22.5 us a step in two launches,
+// 27.6 so, 21.1 now; 64 x 256 with 128 21.0, 22.3, 20.6.  With more partials, a sample's over several lanes and so the samples in
+// several passes: 405 x 940 with 102 samples and 13 partials 28 -> 38 us; with more samples the search for a class: 191 x 140 with 225 25.6 ->
+// 28.4.  With more than 64 samples of more than 6,000 features 1.02 to 1.06 times as long.)
 constexpr int kMergeSamples = 128, kMergePartials = 8;
 __global__ void __launch_bounds__(256) mlr_merged_kernel(const float2* __restrict__ part, int64_t part_ld, int nblocks,
                                                          const float* __restrict__ Z, int64_t ldz, int64_t rows, int32_t n,
@@ -689,23 +692,32 @@ __global__ void __launch_bounds__(256) mlr_merged_kernel(const float2* __restric
       auto add = [&](float cf, const float4& x) {
         s.x = fmaf(cf, x.x, s.x); s.y = fmaf(cf, x.y, s.y); s.z = fmaf(cf, x.z, s.z); s.w = fmaf(cf, x.w, s.w);
       };
-      for (int j = i; j < n;) {
-        if (sh_next[j] >= n) {                       // the last one by itself
-          add(sh_coef[j], *reinterpret_cast<const float4*>(X + static_cast<int64_t>(j) * lab.cols));
-          break;
-        }
-        float4 x[kLabelBatch];
+      int j = i;
+      if (sh_next[j] >= n) {                         // a class of one sample
+        add(sh_coef[j], *reinterpret_cast<const float4*>(X + static_cast<int64_t>(j) * lab.cols));
+      } else {
         const float* xp[kLabelBatch];
         float cf[kLabelBatch];
+        auto follow = [&]() {                        // the next eight of the chain
 #pragma unroll
-        for (int e = 0; e < kLabelBatch; ++e) {
-          xp[e] = X + static_cast<int64_t>(j < n ? j : i) * lab.cols;
-          cf[e] = j < n ? sh_coef[j] : 0.f;
-          if (j < n) j = sh_next[j];
+          for (int e = 0; e < kLabelBatch; ++e) {
+            xp[e] = X + static_cast<int64_t>(j < n ? j : i) * lab.cols;
+            cf[e] = j < n ? sh_coef[j] : 0.f;
+            if (j < n) j = sh_next[j];
+          }
+        };
+        follow();
+        for (bool more = true; more;) {              // the chain is followed while the samples are on their way
+          float4 x[kLabelBatch];
+          float cx[kLabelBatch];
+          load8(x, xp);
+#pragma unroll
+          for (int e = 0; e < kLabelBatch; ++e) cx[e] = cf[e];
+          more = j < n;
+          if (more) follow();
+#pragma unroll
+          for (int e = 0; e < kLabelBatch; ++e) add(cx[e], x[e]);
         }
-        load8(x, xp);
-#pragma unroll
-        for (int e = 0; e < kLabelBatch; ++e) add(cf[e], x[e]);
       }
       *reinterpret_cast<float4*>(lab.dL + static_cast<int64_t>(i) * lab.cols + c) = s;
       w.x = fmaf(lab.step, s.x, w.x); w.y = fmaf(lab.step, s.y, w.y); w.z = fmaf(lab.step, s.z, w.z); w.w = fmaf(lab.step, s.w, w.w);
@@ -953,12 +965,14 @@ static LogitsKernel logits_kernel(const sfb_config& c, const Layout& L, int64_t 
 }
 
 // Whether the softmax of a step's n samples, `partials` of each, is merged by mlr_merged_kernel.
-static bool softmax_merged(int64_t n, int64_t partials) { return n <= kMergeSamples && partials <= kMergePartials; }
+static bool softmax_merged(int64_t n, int64_t cols, int64_t partials) {
+  return n <= (cols > 6000 ? kMergeSamples / 2 : kMergeSamples) && partials <= kMergePartials;
+}
 
 int tc_logits_plan(const sfb_config& c, const Layout& L, int64_t n, int* parts, bool* merged) {
   const LogitsKernel k = logits_kernel(c, L, n, parts);
   const int64_t pw = k == kLogitsFew ? 32 : L.pw;
-  *merged = k != kLogitsPairs && softmax_merged(n, (c.rows + pw - 1) / pw);
+  *merged = k != kLogitsPairs && softmax_merged(n, c.cols, (c.rows + pw - 1) / pw);
   if (k == kLogitsFew) *parts = 1;
   return k;
 }
@@ -1471,7 +1485,7 @@ int tc_factors(sfb_ctx* ctx, int64_t off, int64_t n, const float* X, const float
                       ctx->at<float>(L.coef), ctx->at<__nv_bfloat16>(L.P), L.ldp, ctx->at<uint32_t>(L.status)));
     return SFB_OK;
   }
-  if (fused && n == K && softmax_merged(n, tiles_n)) {
+  if (fused && n == K && softmax_merged(n, c.cols, tiles_n)) {
     const int lab = label_blocks(ctx);
     CKC(launch_kernel(mlr_merged_kernel, dim3(grid1d(n * ((rows + 7) / 8), 256) + lab), dim3(256), 0, ctx->stream, 1,
                       ctx->at<float2>(L.part), K, tiles_n, Z, ldz, rows, static_cast<int32_t>(n), labels, lse, ctx->at<float>(L.loss),

@@ -44,3 +44,12 @@ def test_logits_on_pairs(rows, cols, samples):
                                                    (512, 18_000, 8, True), (512, 18_004, 8, False), (513, 24_000, 64, True)])
 def test_logits_of_few_samples(rows, cols, samples, few):
     assert (S.sfb_get_plan(bf16(rows, cols, samples), samples)[0] == FEW) == few
+
+
+# The softmax in one launch: up to 128 samples (64 with more than 6,000 features) and eight partials, all of the context's samples at once.
+@pytest.mark.parametrize("rows,cols,samples,merged", [(64, 256, 128, 1), (64, 256, 129, 0), (64, 6_000, 128, 1), (64, 6_004, 65, 0),
+                                                      (64, 6_004, 64, 1), (256, 256, 16, 1), (257, 256, 16, 0)])
+def test_softmax_in_one_launch(rows, cols, samples, merged):
+    assert S.sfb_get_plan(bf16(rows, cols, samples), samples)[2] == merged
+    if samples > 1:
+        assert S.sfb_get_plan(bf16(rows, cols, samples), samples - 1)[2] == 0
