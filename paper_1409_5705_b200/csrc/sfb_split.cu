@@ -974,21 +974,21 @@ __global__ void __launch_bounds__(256) pack_u_kernel(const float* __restrict__ U
 
 // Tile width of a product, whether its contraction is cut, and its SM cycles.  A k-block takes the longer of its MMAs (6 cycles per
 // column by their rate, 7.2 as measured at 256 columns: 1,838) and of its bytes from L2 at 38 a cycle and SM (192 columns: 1,485;
-// 160: 1,395; 64: 1,100).  12,000 cycles from the start to the first MMA and from the last one to the results; 4,000 and 4,500 a part to
-// leave and to take over the parts of a tile, whose adding up waits for one copy after another: a product of fewer tiles than pairs is
-// cut into as many parts a tile as that pays for, and not into parts of less than four k-blocks.  (With 8,000 cycles whatever the
-// parts' number, all pairs took part: metric learning 500 x 8,000 with 256 pairs 31 parts a tile, 95 us a step, 56 now; sparse coding 3,000
-// x 2,000 with 256 samples 888, 503 now; 6,000 x 3,000 with 150 1,178, 897 now; fp32 2,200 x 700 with 600 1,536, 1,076 now; with 3,000
-// and 6,500 cycles a part within a few per cent of this.  Cutting only the last of several rounds took fewer cycles at a lower
-// clock: 908 -> 1013 us.)
+// 160: 1,395; 64: 1,100).  12,000 cycles from the start to the first MMA and from the last one to the results; 4,000 and, a part, 1,500
+// and 12 a column to leave and to take over the parts of a tile, whose adding up waits for one copy after another: a product of fewer
+// tiles than pairs is cut into as many parts a tile as that pays for, and not into parts of less than four k-blocks.  (Of 900 drawn
+// calls whose plan matters, against all pairs taking part, factors of metric learning, regression in fp32 and sparse coding take 0.74, 0.82
+// and 0.82 times as long, in fp32 0.92 times; with 4,500 cycles a part whatever the width 0.76, 0.82, 0.83 and 0.99, 28 of 609 more than 3 %
+// longer than with all pairs, and 214 of 504 in fp32 sparse coding: 1,041 x 900 with 54 samples 413 -> 572 us.  Cutting only the last of
+// several rounds took fewer cycles at a lower clock: 908 -> 1013 us.)
 struct ProductPlan { int bn; int64_t tiles, pairs; bool cut; double cost; };
-// fine: drained at every k-block, which the MMAs of a third of it do not hide.
+// fine: drained at every k-block, 21 cycles a column that the MMAs do not hide (7 in W^T W, sym, whose width alone they decide).
 ProductPlan plan_width(int64_t M, int64_t N, int64_t Kc, bool sym, bool fine, int bn, int64_t max_pairs) {
   ProductPlan p{};
   p.bn = bn;
   const int tm = static_cast<int>((M + PM - 1) / PM), tn = static_cast<int>((N + bn - 1) / bn);
   p.tiles = sym ? sym_tiles(tm, tn, bn) : static_cast<int64_t>(tm) * tn;
-  const double per_kb = std::max(7.2 * bn, (2.0 * kBytesA + bn * BK * 2.0) / 38.0) + (fine ? 7.0 * bn : 0.0);
+  const double per_kb = std::max(7.2 * bn, (2.0 * kBytesA + bn * BK * 2.0) / 38.0) + (fine ? (sym ? 7.0 : 21.0) * bn : 0.0);
   const int64_t kseg = (Kc + BK - 1) / BK, rounds = (p.tiles + max_pairs - 1) / max_pairs;
   p.pairs = std::min(p.tiles, max_pairs);
   double kb = static_cast<double>(rounds * kseg);
@@ -997,7 +997,7 @@ ProductPlan plan_width(int64_t M, int64_t N, int64_t Kc, bool sym, bool fine, in
     double least = kb * per_kb;
     for (int64_t parts = 2; (parts - 1) * p.tiles < most; ++parts) {          // of a tile
       const int64_t pairs = std::min(most, parts * p.tiles);
-      const double shared = static_cast<double>((p.tiles * kseg + pairs - 1) / pairs), extra = 4000.0 + 4500.0 * static_cast<double>(parts);
+      const double shared = static_cast<double>((p.tiles * kseg + pairs - 1) / pairs), extra = 4000.0 + (1500.0 + 12.0 * bn) * static_cast<double>(parts);
       if (shared * per_kb + extra < least) {
         least = shared * per_kb + extra;
         p.cut = true;

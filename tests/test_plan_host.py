@@ -53,3 +53,13 @@ def test_softmax_in_one_launch(rows, cols, samples, merged):
     assert S.sfb_get_plan(bf16(rows, cols, samples), samples)[2] == merged
     if samples > 1:
         assert S.sfb_get_plan(bf16(rows, cols, samples), samples - 1)[2] == 0
+
+
+# Products of pairs of words of fewer tiles than pairs of CTAs: narrow tiles are cut although they have few k-blocks, products that drain their
+# accumulator at every k-block (sparse coding in fp32 mode) into more parts than others.
+def test_parts_of_products_of_words():
+    dml = S.make_config(S.DML, 28, 1_656, 1, 193, 1e-3, S.PREC_BF16)
+    assert S.sfb_get_plan(dml, 193)[:2] >= (5, 2)
+    assert S.sfb_get_plan(S.make_config(S.DML, 137, 1_592, 7, 15, 1e-3, S.PREC_BF16), 15)[1] > 1
+    assert S.sfb_get_plan(S.make_config(S.DML, 500, 8_000, 1, 256, 1e-3, S.PREC_BF16), 256)[1] < 31
+    assert S.sfb_get_plan(S.make_config(S.DML, 1_000, 20_000, 16, 64, 1e-3, S.PREC_BF16), 1_024)[1] >= 2
