@@ -39,8 +39,8 @@ bool sc_use_gram(const sfb_config& c) {
   const int64_t K = static_cast<int64_t>(c.workers) * c.batch, D = c.rows, A = c.cols;
   const double it = sc_iterations(c);
   if (c.precision != SFB_PREC_BF16 || it < 1 || A > D || A > kMostAtoms) return false;
-  return split_product_cost(A, A, D, true) + it * split_product_cost(K, A, A, false) <
-         it * (split_product_cost(K, D, A, false) + split_product_cost(K, A, D, false));
+  return split_form_cost(A, A, D, true) + it * split_form_cost(K, A, A, false) <
+         it * (split_form_cost(K, D, A, false) + split_form_cost(K, A, D, false));
 }
 
 // The power iteration on W^T W, whose rows stay on chip, or on W, which comes from L2 or memory twice an iteration, with a barrier
@@ -70,14 +70,19 @@ bool sc_use_gram64(const sfb_config& c) {
   return gram64;
 }
 // Whether the products of sparse coding in fp32 mode are better off as pairs of fp16 words: the packing of W and W^T at 4.5 TB/s, two
-// products an iteration.
+// products an iteration.  Against W^T W in fp64 by the plans' cost: 88 drawn dictionaries on this side of the line that lay on the other
+// by split_form_cost take 0.64 times as long in fp64, and their codes are 0.12 times as far from 64 bits.  Against two products of FMAs by
+// split_form_cost: 199 on the other side of that line take 0.99 times as long, 97 of them more than 3 % longer, and their codes are up to 2.1
+// times as far off (4,960 x 820, 5 iterations: 2.3e-7 on pairs, 4.6e-7).
 bool sc_on_pairs(const sfb_config& c) {
   const int64_t K = static_cast<int64_t>(c.workers) * c.batch, D = c.rows, A = c.cols;
-  const double it = sc_iterations(c), size = static_cast<double>(D) * static_cast<double>(A), form = split_product_cost(A, A, D, true, true);
-  const double toD = split_product_cost(K, D, A, false, true), toA = split_product_cost(K, A, D, false, true);
-  const double pairs = toD + size * 16.0 / 4.5e12 * 1.9e9 + 20000.0 + (it >= 0 ? toA + it * (toD + toA) : 0.0) + (sc_estimate_on_gram(c, form) ? form : 0.0);
   bool gram64;
-  return pairs < sc_fma_cost(c, gram64);
+  const double fma = sc_fma_cost(c, gram64);
+  auto product = [&](int64_t N, int64_t Kc) { return gram64 ? split_product_cost(K, N, Kc, false, true) : split_form_cost(K, N, Kc, false, true); };
+  const double it = sc_iterations(c), size = static_cast<double>(D) * static_cast<double>(A), form = split_product_cost(A, A, D, true, true);
+  const double toD = product(D, A), toA = product(A, D);
+  const double pairs = toD + size * 16.0 / 4.5e12 * 1.9e9 + 20000.0 + (it >= 0 ? toA + it * (toD + toA) : 0.0) + (sc_estimate_on_gram(c, form) ? form : 0.0);
+  return pairs < fma;
 }
 
 Layout make_layout(const sfb_config& cfg) {

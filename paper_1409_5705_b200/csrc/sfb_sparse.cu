@@ -735,7 +735,7 @@ bool sparse_on_fma(const sfb_config& c) {
   const double size = static_cast<double>(c.rows) * static_cast<double>(c.cols), unit = 2.6e-12 * 1.9e9 * size;
   const double sparse = 1.0 + 0.089 * static_cast<double>(c.csr_nnz_max) / static_cast<double>(c.cols);
   const double fma = (rb > 0 ? std::min(row_wise_cycles(c, rb), gemm_cycles(K, c.rows, c.cols)) : gemm_cycles(K, c.rows, c.cols)) + sparse * unit;
-  const double pairs = size * 8.0 / 4.5e12 * 1.9e9 + split_product_cost(K, c.rows, c.cols, false) +
+  const double pairs = size * 8.0 / 4.5e12 * 1.9e9 + split_form_cost(K, c.rows, c.cols, false) +
                        std::min(sparse, std::max(0.7, 1.75 * static_cast<double>(K) / 1024.0)) * unit;
   return fma < 1.1 * pairs;
 }

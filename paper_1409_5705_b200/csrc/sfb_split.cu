@@ -981,7 +981,8 @@ __global__ void __launch_bounds__(256) pack_u_kernel(const float* __restrict__ U
 // and 0.82 times as long, in fp32 0.92 times; with 4,500 cycles a part whatever the width 0.76, 0.82, 0.83 and 0.99, 28 of 609 more than 3 %
 // longer than with all pairs, and 214 of 504 in fp32 sparse coding: 1,041 x 900 with 54 samples 413 -> 572 us.  Cutting only the last of
 // several rounds took fewer cycles at a lower clock: 908 -> 1013 us.)
-struct ProductPlan { int bn; int64_t tiles, pairs; bool cut; double cost; };
+// flat: cycles with all pairs taking part, at 8,000 for the parts (see split_form_cost).
+struct ProductPlan { int bn; int64_t tiles, pairs; bool cut; double cost, flat; };
 // fine: drained at every k-block, 21 cycles a column that the MMAs do not hide (7 in W^T W, sym, whose width alone they decide).
 ProductPlan plan_width(int64_t M, int64_t N, int64_t Kc, bool sym, bool fine, int bn, int64_t max_pairs) {
   ProductPlan p{};
@@ -992,8 +993,12 @@ ProductPlan plan_width(int64_t M, int64_t N, int64_t Kc, bool sym, bool fine, in
   const int64_t kseg = (Kc + BK - 1) / BK, rounds = (p.tiles + max_pairs - 1) / max_pairs;
   p.pairs = std::min(p.tiles, max_pairs);
   double kb = static_cast<double>(rounds * kseg);
+  const double rate = fine ? std::max(7.2 * bn, (2.0 * kBytesA + bn * BK * 2.0) / 38.0) + 7.0 * bn : per_kb;
+  p.flat = kb * rate;
   if (!sym && p.tiles < max_pairs) {
     const int64_t most = std::max<int64_t>(1, std::min(max_pairs, p.tiles * kseg / 4));
+    const double all = static_cast<double>((p.tiles * kseg + most - 1) / most) * rate + 8000.0;
+    p.flat = std::min(p.flat, all);
     double least = kb * per_kb;
     for (int64_t parts = 2; (parts - 1) * p.tiles < most; ++parts) {          // of a tile
       const int64_t pairs = std::min(most, parts * p.tiles);
@@ -1006,7 +1011,9 @@ ProductPlan plan_width(int64_t M, int64_t N, int64_t Kc, bool sym, bool fine, in
     }
     kb = least / per_kb;
   }
-  p.cost = kb * per_kb + 12000.0 + static_cast<double>(p.tiles / max_pairs) * 1500.0;
+  const double rest = 12000.0 + static_cast<double>(p.tiles / max_pairs) * 1500.0;
+  p.cost = kb * per_kb + rest;
+  p.flat += rest;
   return p;
 }
 ProductPlan plan_product(int64_t M, int64_t N, int64_t Kc, bool sym, bool fine, int64_t max_pairs) {
@@ -1219,6 +1226,15 @@ int begin_operands(sfb_ctx* ctx) {
 
 double split_product_cost(int64_t M, int64_t N, int64_t Kc, bool sym, bool fine) {
   return plan_product(M, N, Kc, sym, fine, kModelSms / 2).cost;
+}
+double split_form_cost(int64_t M, int64_t N, int64_t Kc, bool sym, bool fine) {
+  if (N <= 64) return plan_width(M, N, Kc, sym, fine, static_cast<int>(round_up(N, 32)), kModelSms / 2).flat;
+  double best = 0.0;
+  for (int bn = kMaxN; bn >= 64; bn -= 32) {
+    const double c = plan_width(M, N, Kc, sym, fine, bn, kModelSms / 2).flat;
+    if (bn == kMaxN || c < best) best = c;
+  }
+  return best;
 }
 
 int split_product_parts(int64_t M, int64_t N, int64_t Kc, bool fine) {

@@ -54,6 +54,8 @@ int split_pack_received(sfb_ctx* ctx, int64_t off, int64_t n);
 int split_gather(sfb_ctx* ctx);
 const uint16_t* split_v(const sfb_ctx* ctx);
 double split_product_cost(int64_t M, int64_t N, int64_t Kc, bool sym, bool fine = false);     // fine: sparse coding in fp32 mode
+// The same as the forms of the coder are chosen by: the line between forms that round differently does not move with the plans.
+double split_form_cost(int64_t M, int64_t N, int64_t Kc, bool sym, bool fine = false);
 int split_product_parts(int64_t M, int64_t N, int64_t Kc, bool fine);                         // that a tile is cut into, at most
 // MLR, bf16 mode: the kernel of the logits of n samples (see sfb_get_plan) and the parts of a tile; whether the softmax is merged in one launch.
 int tc_logits_plan(const sfb_config& c, const Layout& L, int64_t n, int* parts, bool* merged);

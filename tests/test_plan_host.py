@@ -63,3 +63,15 @@ def test_parts_of_products_of_words():
     assert S.sfb_get_plan(S.make_config(S.DML, 137, 1_592, 7, 15, 1e-3, S.PREC_BF16), 15)[1] > 1
     assert S.sfb_get_plan(S.make_config(S.DML, 500, 8_000, 1, 256, 1e-3, S.PREC_BF16), 256)[1] < 31
     assert S.sfb_get_plan(S.make_config(S.DML, 1_000, 20_000, 16, 64, 1e-3, S.PREC_BF16), 1_024)[1] >= 2
+
+
+# The form of the coder where forms round differently.  bf16: two products an iteration where W^T W would have larger errors (five iterations
+# of 3,445 x 3,172, K = 156: the codes 5.1e-6 from 64 bits, 7.8e-6 on W^T W); fp32: pairs of words rather than two products of FMAs, W^T W
+# in fp64 rather than either where it is the faster one.
+@pytest.mark.parametrize("rows,cols,samples,iters,prec,product", [
+    (3_445, 3_172, 156, 5, S.PREC_BF16, 5), (8_078, 84, 10, 5, S.PREC_BF16, 5), (10_000, 5_000, 512, 20, S.PREC_BF16, 6),
+    (4_960, 820, 29, 5, S.PREC_FP32, 5), (1_130, 1_156, 251, 20, S.PREC_FP32, 5), (198, 1_408, 685, 5, S.PREC_FP32, 5),
+    (5_521, 116, 82, 5, S.PREC_FP32, 7), (2_000, 1_000, 128, 20, S.PREC_FP32, 7), (1_720, 1_148, 230, 20, S.PREC_FP32, 7)])
+def test_form_of_the_coder(rows, cols, samples, iters, prec, product):
+    cfg = S.make_config(S.SC, rows, cols, 1, samples, 1e-3, prec, sc_ista_iters=iters, sc_prox=1, sc_lipschitz=1.0)
+    assert S.sfb_get_plan(cfg, samples)[0] == product
