@@ -108,7 +108,9 @@ __global__ void __launch_bounds__(256) csr_stage_kernel(const int64_t* __restric
 // bf16 mode: the same with what pack_mlr_kernel does, a block per sample: its row is put together in shared memory and leaves as fp32
 // (for the label rows) and as the bf16 operand, each written once.  Against clearing the staging buffer, scattering into it and
 // packing it: 10,000 x 20,000, 1,024 samples of 30 entries, 27 us instead of 46; a step of 2,000 x 3,000 with 240 samples 59 -> 51 us.
-constexpr int kRowThreads = 512, kRowSmem = 200 << 10;
+// 512 threads a sample, four samples an SM; where that is more than one round of blocks, a thread has two quads of the row or more: 1,415 samples
+// of 76 features took 93 us a step with 512, 87 in three kernels; 134 x 36 with 2,269 77.1, 71.4, now 71.5.
+constexpr int kRowThreads = 512, kRowSmem = 200 << 10;     // at most
 struct RowArgs {
   const int64_t* indptr;
   const int32_t* idx;
@@ -133,15 +135,15 @@ __global__ void __launch_bounds__(kRowThreads) csr_rows_kernel(const RowArgs a) 
   stamp_begin(a.stamp);
   extern __shared__ float4 row4[];
   float* row = reinterpret_cast<float*>(row4);
-  const int t = threadIdx.x, quads = static_cast<int>(a.cols / 4);
+  const int t = threadIdx.x, threads = blockDim.x, quads = static_cast<int>(a.cols / 4);
   const int64_t i = blockIdx.x, s = a.off + i;
-  for (int q = t; q < quads; q += kRowThreads) row4[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+  for (int q = t; q < quads; q += threads) row4[q] = make_float4(0.f, 0.f, 0.f, 0.f);
   const int64_t base = a.indptr[0];
   int64_t b = a.indptr[i] - base, e = a.indptr[i + 1] - base;
   const bool bad = b < 0 || e < b || e > a.nnz;    // row pointers that do not describe nnz entries: sample left empty
   if (bad) b = e = 0;
   __syncthreads();
-  for (int64_t k = b + t; k < e; k += kRowThreads) {
+  for (int64_t k = b + t; k < e; k += threads) {
     const int32_t c = a.idx[base + k];
     const float x = a.val[base + k];
     if (c < 0 || c >= a.cols) {                    // entry skipped (its slot keeps the "no entry" mark)
@@ -160,7 +162,7 @@ __global__ void __launch_bounds__(kRowThreads) csr_rows_kernel(const RowArgs a) 
     a.labels_out[s] = a.labels[i];
   }
   __syncthreads();
-  for (int q = t; q < quads; q += kRowThreads) {
+  for (int q = t; q < quads; q += threads) {
     const float4 v = row4[q];
     reinterpret_cast<float4*>(a.Xd + s * a.cols)[q] = v;
     const __nv_bfloat162 lo = __floats2bfloat162_rn(v.x, v.y), hi = __floats2bfloat162_rn(v.z, v.w);
@@ -671,7 +673,8 @@ int sparse_stage_packed(sfb_ctx* ctx, int64_t off, int64_t n, const int64_t* ind
   a.coo_x = ctx->at<float>(L.coo_x) + ctx->csr_fill;
   a.stamp = take_stamp(ctx); a.status = ctx->at<uint32_t>(L.status);
   CKS(allow_smem<csr_rows_kernel>(kRowSmem));
-  CKS(launch_kernel(csr_rows_kernel, dim3(static_cast<unsigned>(n)), dim3(kRowThreads), static_cast<size_t>(a.cols) * 4, s, 1, a));
+  const int64_t threads = n <= 4 * sm_count() ? kRowThreads : std::min<int64_t>(kRowThreads, std::max<int64_t>(32, (a.cols / 8 + 31) / 32 * 32));
+  CKS(launch_kernel(csr_rows_kernel, dim3(static_cast<unsigned>(n)), dim3(static_cast<unsigned>(threads)), static_cast<size_t>(a.cols) * 4, s, 1, a));
   ctx->last_stage_nnz = nnz;
   return SFB_OK;
 }

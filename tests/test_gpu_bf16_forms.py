@@ -150,3 +150,31 @@ def test_sparse_samples_as_dense_ones(cols, per_worker):
         got.append(W)
         ctx.close()
     assert torch.equal(got[0], got[1])
+
+
+# Sparse samples in more than one round of blocks, whose rows then have fewer threads: the bits of the dense samples' step.
+@pytest.mark.parametrize("cols", [4, 252, 260, 4100])
+def test_many_sparse_samples_as_dense_ones(cols):
+    rows, K = 40, 700
+    g = torch.Generator(device="cuda")
+    g.manual_seed(3)
+    W0 = torch.randn(rows, cols, generator=g, device="cuda") * 0.05
+    lab = torch.randint(0, rows, (K,), generator=g, device="cuda", dtype=torch.int32)
+    X = torch.randn(K, cols, generator=g, device="cuda") * (torch.rand(K, cols, generator=g, device="cuda") < 0.1)
+    X[5] = 0
+    X[6] = 1
+    where = X.nonzero()
+    ptr = torch.zeros(K + 1, dtype=torch.int64, device="cuda")
+    ptr[1:] = torch.cumsum(torch.bincount(where[:, 0], minlength=K), 0)
+    got = []
+    for sparse in (False, True):
+        W = W0.clone()
+        ctx = S.Context(S.make_config(S.MLR, rows, cols, 1, K, 0.05, S.PREC_BF16, csr_nnz_max=K * cols, csr_update=2), W)
+        if sparse:
+            ctx.sfb_step_csr(ptr, where[:, 1].to(torch.int32).contiguous(), X[where[:, 0], where[:, 1]].contiguous(), int(ptr[-1]), lab)
+        else:
+            ctx.sfb_step(X, None, lab)
+        assert ctx.sfb_get_status() == 0
+        got.append(W)
+        ctx.close()
+    assert torch.equal(got[0], got[1])
