@@ -330,7 +330,11 @@ bool forward_pair_pays(int64_t n, int64_t rows, int64_t cols, double other, int6
   return true;
 }
 int64_t forward_pair_groups(int64_t rows) { return rows <= kNarrowRows ? (rows + 31) / 32 : (rows + kMaxN / 2 - 1) / (kMaxN / 2); }
-size_t forward_pair_partial_bytes() { return static_cast<size_t>(kModelSms / 2) * 2 * kEpi * 4 * kSlot; }
+size_t forward_pair_partial_bytes(int64_t pairs) { return static_cast<size_t>(pairs) * 2 * kEpi * 4 * kSlot; }
+int64_t forward_pair_cut(int64_t n, int64_t rows, int64_t cols) {
+  const PairPlan p = plan_pairs(n, rows, cols, kModelSms / 2);
+  return p.cut ? p.pairs : 0;
+}
 size_t forward_pair_ready_bytes() { return static_cast<size_t>(kModelSms / 2) * 2 * kEpi * 4; }
 
 cudaError_t forward_pair_prepare(int* max_pairs) { return prepare_pair_kernel(forward_pair_kernel, kThreads, kSmem, max_pairs); }
@@ -339,7 +343,12 @@ cudaError_t forward_pair(sfb_ctx* ctx, int64_t off, int64_t n, int* pw) {
   TcState* st = static_cast<TcState*>(ctx->tc);
   const Layout& L = ctx->lay;
   const int64_t rows = ctx->cfg.rows, cols = ctx->cfg.cols;
-  const PairPlan plan = plan_pairs(ctx, n);
+  PairPlan plan = plan_pairs(ctx, n);
+  if (plan.cut && plan.pairs > L.cut_pairs) {      // (a device with fewer pairs than the workspace was laid out for: whole tiles)
+    const int64_t tiles = (n + PM - 1) / PM * ((rows + plan.bn - 1) / plan.bn);
+    plan.cut = plan.whole = 0;
+    plan.pairs = static_cast<int>(std::min<int64_t>(tiles, plan.pairs));
+  }
   CUtensorMap ma, mb, mc;
   if (!make_map(st, &ma, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, ctx->at<uint16_t>(L.Xb), cols, ctx->K, L.colsb * 2, BK, BM) ||
       !make_map(st, &mb, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, ctx->at<uint16_t>(L.Wb), cols, rows, L.colsb * 2, BK, plan.bn / 2) ||

@@ -127,6 +127,8 @@ struct Layout {
   int64_t Kp;                         // K rounded up to the contraction block of the update product
   int32_t split;                      // parts that the bf16 forward product of MLR cuts its contraction into
   int32_t pw;                         // columns per softmax partial of the bf16 forward product
+  bool on_pairs;                      // some call's logits take the kernel of CTA pairs
+  int32_t cut_pairs;                  //   and of those, pairs that leave parts of tiles, at most
   int64_t ldp;                        // row pitch of P: rows rounded up to 64
   int64_t colsb;                      // cols rounded up to the contraction block of the forward product
   size_t total;

@@ -945,7 +945,7 @@ static int pick_forward_split(int64_t K, int64_t rows, int64_t cols) {
 // those of the clusters that are resident at a time (15 of eight CTAs, 120 of the 148 SMs: the factors of 281 x 7,060 with 146 samples,
 // 144 CTAs, 33.6 us, 22.9 on pairs; 870 x 1,012 with 218, 112 CTAs, 16.5 and 14.0).
 static bool forward_on_pairs(const sfb_config& c, const Layout& L, int64_t n, int* parts) {
-  if (n <= BM || !L.partial || ((n + 255) / 256) * ((c.rows + 255) / 256) >= 5 * (kModelSms / 2)) return false;
+  if (n <= BM || ((n + 255) / 256) * ((c.rows + 255) / 256) >= 5 * (kModelSms / 2)) return false;
   const int bn = pick_forward_width(n, c.rows, c.cols, L.pw, L.split);
   double cost = forward_cost(n, c.rows, c.cols, bn, L.split);
   if (L.split > 1) {
@@ -1010,9 +1010,18 @@ void tc_extend_layout(const sfb_config& c, Layout& L, size_t& off) {
   L.pw = L.split > 1 ? 32 : pick_forward_width(c.batch, c.rows, c.cols, 32, 1);
   size_t nblk = static_cast<size_t>((c.rows + L.pw - 1) / L.pw);
   if (forward_few_fits(c.batch, c.rows, c.cols)) nblk = std::max(nblk, static_cast<size_t>(forward_few_groups(c.rows)));
-  if (K > BM) {                                  // for the kernel of CTA pairs
-    nblk = std::max(nblk, static_cast<size_t>(forward_pair_groups(c.rows)));
-    L.partial = take(forward_pair_partial_bytes());
+  // For the kernel of CTA pairs, where a worker's call, one of all samples or a part of sfb_step_host's takes it: parts of tiles, 256 KB
+  // a pair that leaves some (19 MB in all; whatever the context, 325,000 x 10,000 had them for nothing).
+  for (int64_t parts = 0; parts <= HostSide::kParts; parts = parts ? 2 * parts : 1) {
+    const int64_t n = parts ? static_cast<int64_t>(K) / parts : c.batch;
+    int cut = 1;
+    if (n < 1 || logits_kernel(c, L, n, &cut) != kLogitsPairs) continue;
+    L.on_pairs = true;
+    L.cut_pairs = std::max(L.cut_pairs, static_cast<int32_t>(forward_pair_cut(n, c.rows, c.cols)));
+  }
+  if (L.on_pairs) nblk = std::max(nblk, static_cast<size_t>(forward_pair_groups(c.rows)));
+  if (L.cut_pairs > 0) {
+    L.partial = take(forward_pair_partial_bytes(L.cut_pairs));
     L.ready = take(forward_pair_ready_bytes());
   }
   L.Wb = take(static_cast<size_t>(c.rows) * L.colsb * 2);
@@ -1057,7 +1066,7 @@ int tc_init(sfb_ctx* ctx) {
     return tc_refresh_operands(ctx);
   }
   if (c.model != SFB_MLR || ctx->h16) return split_init(ctx);
-  if (ctx->lay.partial) CKC(cudaMemsetAsync(ctx->at<char>(ctx->lay.ready), 0, forward_pair_ready_bytes(), ctx->stream));
+  if (ctx->lay.ready) CKC(cudaMemsetAsync(ctx->at<char>(ctx->lay.ready), 0, forward_pair_ready_bytes(), ctx->stream));
   CKC(cudaMemsetAsync(ctx->at<char>(ctx->lay.labels), 0xff, static_cast<size_t>(ctx->K) * 4, ctx->stream));
   CKC(cudaMemsetAsync(ctx->at<char>(ctx->lay.slot), 0x7f, static_cast<size_t>(c.rows) * 4, ctx->stream));
   // bf16 copy of W for the forward product; afterwards the update's epilogue keeps it current
@@ -1221,7 +1230,7 @@ static int mlr_forward(sfb_ctx* ctx, int64_t off, int64_t n, const float* X, con
     *parts = static_cast<int>(forward_few_groups(rows));
     return SFB_OK;
   }
-  if (kernel == kLogitsPairs) {
+  if (kernel == kLogitsPairs && L.on_pairs) {
     int pw = 0;
     CKC(forward_pair(ctx, off, n, &pw));
     *parts = static_cast<int>((rows + pw - 1) / pw);

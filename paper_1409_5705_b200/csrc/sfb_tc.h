@@ -68,7 +68,8 @@ int tc_get_factors(sfb_ctx* ctx, const void** U, const void** V, int32_t* dtype,
 double forward_pair_cost(int64_t n, int64_t rows, int64_t cols);
 bool forward_pair_pays(int64_t n, int64_t rows, int64_t cols, double other, int64_t other_groups, int* parts);
 int64_t forward_pair_groups(int64_t rows);           // most softmax partials of a sample
-size_t forward_pair_partial_bytes();
+int64_t forward_pair_cut(int64_t n, int64_t rows, int64_t cols);      // pairs that leave parts of tiles
+size_t forward_pair_partial_bytes(int64_t pairs);
 size_t forward_pair_ready_bytes();
 cudaError_t forward_pair_prepare(int* max_pairs);
 cudaError_t forward_pair(sfb_ctx* ctx, int64_t off, int64_t n, int* pw);

@@ -75,3 +75,15 @@ def test_parts_of_products_of_words():
 def test_form_of_the_coder(rows, cols, samples, iters, prec, product):
     cfg = S.make_config(S.SC, rows, cols, 1, samples, 1e-3, prec, sc_ista_iters=iters, sc_prox=1, sc_lipschitz=1.0)
     assert S.sfb_get_plan(cfg, samples)[0] == product
+
+
+# Room for parts of tiles only where some call's logits take pairs of CTAs that leave some.
+def test_workspace_of_the_logits_on_pairs():
+    size = lambda *a, **k: S.sfb_workspace_bytes(bf16(*a, **k))  # noqa: E731
+    assert size(64, 256, 129) - size(64, 256, 128) < 100_000
+    rows, cols, K = 325_000, 10_000, 1_024             # operands, logits, probabilities, samples (staged, fp32, bf16, label sums), partials
+    need = rows * 10_048 * 2 + K * rows * 6 + K * cols * 14 + K * rows // 256 * 8
+    assert need < size(rows, cols, K) < need + 10_000_000
+    cfg = bf16(10_000, 20_000, 1_024)
+    assert S.sfb_get_plan(cfg, 1_024)[:2] == (PAIRS, 2)
+    assert size(10_000, 20_000, 1_024, workers=16) > 10_000 * 20_032 * 2 + 1_024 * (10_000 * 6 + 20_000 * 14) + 19_000_000
