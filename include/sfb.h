@@ -320,8 +320,8 @@ int sfb_get_operand_copy(sfb_ctx* ctx, const void** copy_dev, int32_t* dtype, in
  * tf32 words, 5 the sums over sparse samples.  SFB_ERR_STATE before the first gather. */
 int sfb_get_update_form(sfb_ctx* ctx, int32_t* form);
 
-/* Which kernels a context with this config takes for the factors of `samples` samples (one call's: B, K, or a part of
- * them; SFB_ERR_SHAPE outside 1..K).  Host-only; no CUDA call.
+/* Which kernels a context with this config takes for the factors of `samples` samples: K in a step (sfb_step, ...), fewer in a
+ * factors call of their own (SFB_ERR_SHAPE outside 1..K).  Host-only; no CUDA call.
  *   product  0 fp32 FMAs | bf16: 1 tiles of one CTA, 2 of pairs of CTAs, 3 up to 64 samples | 4 pairs of tf32 words | 5 pairs of
  *            bf16 or fp16 words | sparse coding on W^T W: 6 in such pairs, 7 in fp64
  *   parts    that a tile's contraction is cut into in the products 1, 2 and 5 (6: of an iteration; 2 where any is cut); 1 elsewhere

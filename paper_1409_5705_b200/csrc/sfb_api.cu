@@ -1000,8 +1000,9 @@ extern "C" int sfb_get_plan(const sfb_config* cfg, int64_t samples, int32_t* pro
     form = 5;
     cut = split_product_parts(samples, c.rows, c.cols, false);
   } else if (c.precision == SFB_PREC_BF16) {
-    form = tc_logits_plan(c, make_layout(*cfg), samples, &cut, &one);
-    one = one && cfg->model == SFB_MLR && samples == static_cast<int64_t>(c.workers) * c.batch;
+    const bool step = samples == static_cast<int64_t>(c.workers) * c.batch;
+    form = tc_logits_plan(c, make_layout(*cfg), samples, step, &cut, &one);
+    one = one && step && cfg->model == SFB_MLR;
   }
   *product = form;
   *parts = cut;

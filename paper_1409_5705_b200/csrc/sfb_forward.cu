@@ -538,12 +538,13 @@ int few_parts(int64_t tiles, int64_t kseg, const int (&most)[kFewParts + 1]) {
 // HBM.  us of a worker's call, forward_kernel / here, 3,004 features: 9,400 classes with 37 and 64 samples 23.2, 24.9 / 21.5, 24.2; 10,000
 // with 8 and 64 23.5, 26.0 / 19.4, 29.8; 15,000 with 16 and 37 25.0, 27.3 / 22.0, 30.8; 10,000 x 20,000 with 8 and 64 119, 128 / 80, 88.
 // Above 40 samples the end of a tile (Z and partials, by rows, through shared memory) takes longer than forward_kernel's, which fewer than 12
-// k-blocks do not repay: factors with 49 to 64 samples, up to 500 features 1.06 to 1.18 times as long as with forward_kernel, 1,000 to 1,500
-// 0.84 times; 33 to 40 samples 1.02 and 0.85.  And forward_kernel cuts the longest contractions into eight parts where there are few
+// k-blocks do not repay in a call of its own: factors with 49 to 64 samples, up to 500 features 1.06 to 1.20 times as long as with
+// forward_kernel, 1,000 to 1,500 0.84 times; 33 to 40 samples 1.02 and 0.85.  (In a step, beside the kernels around it, the same sizes
+// take 0.90 to 1.04 times as long.)  And forward_kernel cuts the longest contractions into eight parts where there are few
 // tiles: up to 512 classes, 20,000 to 24,000 features 1.04 times as long here, 14,000 to 18,000 0.95.
-bool forward_few_fits(int64_t n, int64_t rows, int64_t cols) {
+bool forward_few_fits(int64_t n, int64_t rows, int64_t cols, bool step) {
   const int64_t tiles = (rows + BM - 1) / BM, kseg = (cols + BK - 1) / BK;
-  if (n > kFewN || (n > 40 && kseg < 12) || (tiles <= 4 && cols > 18000)) return false;
+  if (n > kFewN || (!step && n > 40 && kseg < 12) || (tiles <= 4 && cols > 18000)) return false;
   return tiles <= kModelSms / 2 || (tiles <= 118 && (n <= 24 || rows * cols >= 100000000));
 }
 int64_t forward_few_groups(int64_t rows) { return (rows + 31) / 32; }

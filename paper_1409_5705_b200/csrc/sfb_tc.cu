@@ -956,11 +956,11 @@ static bool forward_on_pairs(const sfb_config& c, const Layout& L, int64_t n, in
   return forward_pair_pays(n, c.rows, c.cols, cost, (c.rows + L.pw - 1) / L.pw, parts);
 }
 
-// The kernel that forms the logits of n samples, in bf16 mode.
+// The kernel that forms the logits of n samples, in bf16 mode; step: in a call that goes on to the update.
 enum LogitsKernel { kLogitsTiles = 1, kLogitsPairs = 2, kLogitsFew = 3 };
-static LogitsKernel logits_kernel(const sfb_config& c, const Layout& L, int64_t n, int* parts) {
+static LogitsKernel logits_kernel(const sfb_config& c, const Layout& L, int64_t n, bool step, int* parts) {
   *parts = L.split;
-  if (forward_few_fits(n, c.rows, c.cols)) return kLogitsFew;
+  if (forward_few_fits(n, c.rows, c.cols, step)) return kLogitsFew;
   return forward_on_pairs(c, L, n, parts) ? kLogitsPairs : kLogitsTiles;
 }
 
@@ -969,8 +969,8 @@ static bool softmax_merged(int64_t n, int64_t cols, int64_t partials) {
   return n <= (cols > 6000 ? kMergeSamples / 2 : kMergeSamples) && partials <= kMergePartials;
 }
 
-int tc_logits_plan(const sfb_config& c, const Layout& L, int64_t n, int* parts, bool* merged) {
-  const LogitsKernel k = logits_kernel(c, L, n, parts);
+int tc_logits_plan(const sfb_config& c, const Layout& L, int64_t n, bool step, int* parts, bool* merged) {
+  const LogitsKernel k = logits_kernel(c, L, n, step, parts);
   const int64_t pw = k == kLogitsFew ? 32 : L.pw;
   *merged = k != kLogitsPairs && softmax_merged(n, c.cols, (c.rows + pw - 1) / pw);
   if (k == kLogitsFew) *parts = 1;
@@ -1009,13 +1009,13 @@ void tc_extend_layout(const sfb_config& c, Layout& L, size_t& off) {
   L.split = pick_forward_split(static_cast<int64_t>(K), c.rows, c.cols);
   L.pw = L.split > 1 ? 32 : pick_forward_width(c.batch, c.rows, c.cols, 32, 1);
   size_t nblk = static_cast<size_t>((c.rows + L.pw - 1) / L.pw);
-  if (forward_few_fits(c.batch, c.rows, c.cols)) nblk = std::max(nblk, static_cast<size_t>(forward_few_groups(c.rows)));
+  if (forward_few_fits(c.batch, c.rows, c.cols, true)) nblk = std::max(nblk, static_cast<size_t>(forward_few_groups(c.rows)));
   // For the kernel of CTA pairs, where a worker's call, one of all samples or a part of sfb_step_host's takes it: parts of tiles, 256 KB
   // a pair that leaves some (19 MB in all; whatever the context, 325,000 x 10,000 had them for nothing).
   for (int64_t parts = 0; parts <= HostSide::kParts; parts = parts ? 2 * parts : 1) {
     const int64_t n = parts ? static_cast<int64_t>(K) / parts : c.batch;
     int cut = 1;
-    if (n < 1 || logits_kernel(c, L, n, &cut) != kLogitsPairs) continue;
+    if (n < 1 || logits_kernel(c, L, n, parts != 0, &cut) != kLogitsPairs) continue;
     L.on_pairs = true;
     L.cut_pairs = std::max(L.cut_pairs, static_cast<int32_t>(forward_pair_cut(n, c.rows, c.cols)));
   }
@@ -1224,7 +1224,7 @@ static int mlr_forward(sfb_ctx* ctx, int64_t off, int64_t n, const float* X, con
                     rows,
                     take_stamp(ctx)));
   int cut = 1;
-  const LogitsKernel kernel = logits_kernel(c, L, n, &cut);
+  const LogitsKernel kernel = logits_kernel(c, L, n, fused, &cut);
   if (kernel == kLogitsFew) {
     CKC(forward_few(ctx, off, n));
     *parts = static_cast<int>(forward_few_groups(rows));
@@ -1449,7 +1449,7 @@ int tc_host_parts(const sfb_ctx* ctx) {
     const int64_t n = ctx->K / parts;
     const double copy = 4.0 * static_cast<double>(n) * static_cast<double>(c.cols) / 45e9 + 4e-6;
     int cut = 1;
-    const double cycles = logits_kernel(c, ctx->lay, n, &cut) == kLogitsPairs
+    const double cycles = logits_kernel(c, ctx->lay, n, true, &cut) == kLogitsPairs
                               ? forward_pair_cost(n, c.rows, c.cols)
                               : forward_cost(n, c.rows, c.cols, pick_forward_width(n, c.rows, c.cols, ctx->lay.pw, 1), 1);
     const double product = std::max(cycles / 1.7e9, 2.0 * static_cast<double>(c.rows) * static_cast<double>(c.cols) / 5e12) + 5e-6;

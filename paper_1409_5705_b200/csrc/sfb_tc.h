@@ -58,7 +58,7 @@ double split_product_cost(int64_t M, int64_t N, int64_t Kc, bool sym, bool fine 
 double split_form_cost(int64_t M, int64_t N, int64_t Kc, bool sym, bool fine = false);
 int split_product_parts(int64_t M, int64_t N, int64_t Kc, bool fine);                         // that a tile is cut into, at most
 // MLR, bf16 mode: the kernel of the logits of n samples (see sfb_get_plan) and the parts of a tile; whether the softmax is merged in one launch.
-int tc_logits_plan(const sfb_config& c, const Layout& L, int64_t n, int* parts, bool* merged);
+int tc_logits_plan(const sfb_config& c, const Layout& L, int64_t n, bool step, int* parts, bool* merged);
 int tc_update(sfb_ctx* ctx);
 int tc_get_factors(sfb_ctx* ctx, const void** U, const void** V, int32_t* dtype, int32_t* layout, int64_t* ldu,
                    int64_t* ldv);
@@ -76,7 +76,7 @@ cudaError_t forward_pair(sfb_ctx* ctx, int64_t off, int64_t n, int* pw);
 
 // The same for up to 64 samples (forward_few_kernel): whether it takes these sizes; softmax partials, of 32 classes; most resident
 // clusters of 1 to 4 CTAs.
-bool forward_few_fits(int64_t n, int64_t rows, int64_t cols);
+bool forward_few_fits(int64_t n, int64_t rows, int64_t cols, bool step);      // step: in a call that goes on to the update
 int64_t forward_few_groups(int64_t rows);
 cudaError_t forward_few_prepare(int (&most)[5]);
 cudaError_t forward_few(sfb_ctx* ctx, int64_t off, int64_t n);

@@ -38,12 +38,15 @@ def test_logits_on_pairs(rows, cols, samples):
     assert S.sfb_get_plan(bf16(rows, cols, samples), samples)[0] == PAIRS
 
 
-# Up to 64 samples: the kernel of few samples, but for more than 40 with fewer than 12 k-blocks and for the longest contractions of a few tiles.
-@pytest.mark.parametrize("rows,cols,samples,few", [(64, 64, 40, True), (64, 64, 41, False), (300, 708, 64, True), (300, 704, 64, False), (3_048, 268, 56, False),
-                                                   (107, 84, 44, False), (4_999, 3_004, 64, True), (4_999, 3_004, 65, False),
-                                                   (512, 18_000, 8, True), (512, 18_004, 8, False), (513, 24_000, 64, True)])
-def test_logits_of_few_samples(rows, cols, samples, few):
-    assert (S.sfb_get_plan(bf16(rows, cols, samples), samples)[0] == FEW) == few
+# Up to 64 samples: the kernel of few samples, but in a worker's call for more than 40 with fewer than 12 k-blocks, and for the longest
+# contractions of a few tiles.
+@pytest.mark.parametrize("rows,cols,samples,call,step", [
+    (64, 64, 40, True, True), (64, 64, 41, False, True), (300, 708, 64, True, True), (300, 704, 64, False, True), (3_048, 268, 56, False, True),
+    (107, 84, 44, False, True), (4_999, 3_004, 64, True, True), (4_999, 3_004, 65, False, False), (512, 18_000, 8, True, True),
+    (512, 18_004, 8, False, False), (513, 24_000, 64, True, True)])
+def test_logits_of_few_samples(rows, cols, samples, call, step):
+    assert (S.sfb_get_plan(bf16(rows, cols, 2 * samples, workers=2), samples)[0] == FEW) == call
+    assert (S.sfb_get_plan(bf16(rows, cols, samples), samples)[0] == FEW) == step
 
 
 # The softmax in one launch: up to 128 samples (64 with more than 6,000 features) and eight partials, all of the context's samples at once.
