@@ -282,9 +282,8 @@ forward_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
 
 // Cycles of a plan: its k-blocks on a pair at the MMAs' rate or 60 bytes a cycle and SM, at least the 8,000 that the end of a tile of 256
 // classes takes; 7,000 from the start to the first MMA and from the last one to the results; 9,000 and 2,000 a part to leave and to
-// take over parts of tiles, of which there are no more than pay for that.  (Fitted to 47 shapes, 64 to 100,000 classes, 170 to 20,000 features, 129 to 1,024 samples: against
-// the best of forward_kernel, whole tiles and cut ones the choice loses 3 % in the middle of the factors' time, 31 % at most, of 12 us;
-// forward_kernel alone 11 %.  us of the product, forward_kernel / here: 10,000 x 20,000 with 1,024 samples 376 / 283, 11,133 x
+// take over parts of tiles, of which there are no more than pay for that.  (Fitted to 47 shapes, 64 to 100,000 classes, 170 to 20,000 features, 129 to 1,024 samples; whether
+// the pairs are taken at all: forward_pair_pays.  us of the product, forward_kernel / here: 10,000 x 20,000 with 1,024 samples 376 / 283, 11,133 x
 // 3,364 with 1,024 79 / 67.)
 constexpr int64_t kNarrowRows = 4096;               // up to which narrower tiles are looked at (they have more partials)
 struct PairPlan { int bn, cut, whole, pairs; double cost; };
@@ -319,7 +318,8 @@ double forward_pair_cost(int64_t n, int64_t rows, int64_t cols) { return plan_pa
 // against each other, on 1,278 shapes of 129 to 2,048 samples, 2 to 300,000 classes and 32 to 24,000 features, the pairs are the better
 // ones where a third more, 13,000 cycles where tiles are cut, and 2,400 per 32 partials that the softmax has to merge (a pair's tile
 // of 256 classes leaves two) still come to less.  With that the choice costs a step, fused or by calls, more than 3 % in 29 of 2,556 cases,
-// by the models as they are in 271: 36,667 x 912 with 364 samples 145 us on forward_kernel, 174 on pairs, 78,798 x 1,716 with 156
+// by the models as they are in 271 (4,047 more shapes, against the better of the two: steps 0.7 % longer, 2.1 % by the models as they are,
+// 2.9 % on forward_kernel alone): 36,667 x 912 with 364 samples 145 us on forward_kernel, 174 on pairs, 78,798 x 1,716 with 156
 // 396 and 458, 121 x 3,772 with 180 35.8 and 39.6.
 bool forward_pair_pays(int64_t n, int64_t rows, int64_t cols, double other, int64_t other_groups, int* parts) {
   const PairPlan p = plan_pairs(n, rows, cols, kModelSms / 2);
@@ -537,6 +537,8 @@ int few_parts(int64_t tiles, int64_t kseg, const int (&most)[kFewParts + 1]) {
 // Where two CTAs share a tile (up to 74 tiles); fewer than one tile per SM leaves SMs idle, which pays for few samples or where W comes from
 // HBM.  us of a worker's call, forward_kernel / here, 3,004 features: 9,400 classes with 37 and 64 samples 23.2, 24.9 / 21.5, 24.2; 10,000
 // with 8 and 64 23.5, 26.0 / 19.4, 29.8; 15,000 with 16 and 37 25.0, 27.3 / 22.0, 30.8; 10,000 x 20,000 with 8 and 64 119, 128 / 80, 88.
+// (118 tiles are the 15,000 classes up to which it was measured.  From 15,105 to 30,000 up to 8 samples would take 0.74 to 0.90 times as long
+// here too, 9 to 16 0.83 to 0.97, 17 to 32 0.94 to 1.06, more 1.08 to 1.39.)
 // Above 40 samples the end of a tile (Z and partials, by rows, through shared memory) takes longer than forward_kernel's, which fewer than 12
 // k-blocks do not repay in a call of its own: factors with 49 to 64 samples, up to 500 features 1.06 to 1.20 times as long as with
 // forward_kernel, 1,000 to 1,500 0.84 times; 33 to 40 samples 1.02 and 0.85.  (In a step, beside the kernels around it, the same sizes

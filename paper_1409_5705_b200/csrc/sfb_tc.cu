@@ -928,7 +928,8 @@ static int pick_forward_width(int64_t n, int64_t rows, int64_t cols, int least, 
   return best;
 }
 // Parts that the contraction of the forward product is cut into when the tiles of all K samples do not fill the SMs (72 rows of
-// 14,240 columns: 223 k-blocks in a row on one SM, 68 us).  One choice per context: it fixes the order of the sums.
+// 14,240 columns: 223 k-blocks in a row on one SM, 68 us).  One choice per context, for the calls that forward_kernel takes: its sums
+// then have one order.  (By their number of samples others go to the kernels of sfb_forward.cu, whose sums have another one.)
 static int pick_forward_split(int64_t K, int64_t rows, int64_t cols) {
   int best = 1;
   double cost = forward_cost(K, rows, cols, pick_forward_width(K, rows, cols, 32, 1), 1);
@@ -940,7 +941,9 @@ static int pick_forward_split(int64_t K, int64_t rows, int64_t cols) {
 }
 
 // Whether the logits of n samples take the kernel of CTA pairs.  Not beyond five rounds of its tiles, where an uneven last one matters
-// little and the step is at the power limit (325,000 x 10,000 with 1,024 samples: 5,280 us of the factors' time here, 5,470 there).
+// little (325,000 x 10,000 with 1,024 samples: 5,280 us of the factors' time here, 5,470 there) and the softmax has twice the partials to
+// merge: from 30,000 classes on, steps with 129 to 200 samples of up to 1,000 features take 1.5 to 1.7 times as long on pairs, with 300 to 500
+// 1.45, with more than 1,000 1.02 to 1.05, although their factors by calls take 0.91 to 1.03.
 // What forward_cost has for a split contraction chooses among splits; against another kernel it needs 22,000 cycles more, and its rounds are
 // those of the clusters that are resident at a time (15 of eight CTAs, 120 of the 148 SMs: the factors of 281 x 7,060 with 146 samples,
 // 144 CTAs, 33.6 us, 22.9 on pairs; 870 x 1,012 with 218, 112 CTAs, 16.5 and 14.0).
