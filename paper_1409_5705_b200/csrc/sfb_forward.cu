@@ -1,4 +1,4 @@
-// Logits of multiclass logistic regression in bf16 mode for more than 128 samples, on pairs of CTAs:  Z (samples x rows of W) = X W^T
+// Logits of multiclass logistic regression in bf16 mode for more than 128 samples, on pairs of CTAs where these are the faster ones:  Z (samples x rows of W) = X W^T
 // with the softmax partials of each sample.  (Fewer samples, and the tf32 words: forward_kernel in sfb_tc.cu.)
 //
 // A pair (cta_group::2) owns a tile of 256 samples x bn classes, a CTA 128 of the samples in its TMEM; it loads its own samples and its

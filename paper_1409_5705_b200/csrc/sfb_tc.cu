@@ -2,8 +2,8 @@
 // logistic regression (Sections 1 and 2: u = softmax(W x) - onehot(y), v = x) and the operand packing of the
 // update product.  The update product itself is in sfb_update.cu, the products of (hi | lo) pairs in sfb_split.cu.
 //
-// Forward product (of 65 to 128 samples or many rounds of tiles, and of tf32 words; the others: sfb_forward.cu): one persistent,
-// warp-specialised kernel computes  Z (K x rows) = X (K x cols) * W^T  with bf16
+// Forward product (of 65 to 128 samples, of others where logits_kernel does not prefer those of sfb_forward.cu, and of tf32 words): one
+// persistent, warp-specialised kernel computes  Z (K x rows) = X (K x cols) * W^T  with bf16
 // operands staged by TMA into 128-byte-swizzled shared memory, tcgen05.mma accumulating in TMEM (two 128 x 256
 // fp32 accumulators, so the epilogue of one tile overlaps the main loop of the next).  The epilogue stores Z as
 // fp32 and, per (sample, 256-row block), the softmax partials (max, sum of exp).
