@@ -49,19 +49,39 @@ def plan(rows, cols, workers, batch, samples):
 PAIRS = 2
 
 
-# The logits on pairs of CTAs.  Whole tiles of 64 and 192 classes; a contraction shared out over most pairs, most of them in the middle of a
+# More than 128 samples, on pairs of CTAs or near the line between these and forward_kernel: long and short contractions, several rounds of
+# tiles, the last sample and the last class alone in a tile.
+@pytest.mark.parametrize("shape", [(873, 2800, 2, 317), (190, 708, 1, 513), (791, 9276, 4, 140), (9001, 4004, 2, 257), (10100, 5004, 5, 180),
+                                   (2305, 1028, 1, 129)])
+def test_logits_on_pairs(shape):
+    check(*shape)
+
+
+# (forward_kernel's size by now: of a shared-out tile the same is tested below.)
+def test_logits_on_pairs_repeat():
+    """The sums of a shared-out tile are in the order of the pairs: the same bits every time."""
+    rows, cols, K = 9001, 4004, 514
+    W0 = torch.randn(rows, cols, device="cuda") * 0.05
+    X, lab = torch.randn(K, cols, device="cuda") / cols ** 0.5, torch.randint(0, rows, (K,), device="cuda", dtype=torch.int32)
+    got = []
+    for _ in range(2):
+        W = W0.clone()
+        ctx = S.Context(S.make_config(S.MLR, rows, cols, 1, K, 0.05, S.PREC_BF16), W)
+        for _ in range(3):
+            ctx.sfb_step(X, None, lab)
+        assert ctx.sfb_get_status() == 0
+        got.append(W)
+        ctx.close()
+    assert torch.equal(got[0], got[1])
+
+
+# Those that are on pairs.  Whole tiles of 64 and 192 classes; a contraction shared out over most pairs, most of them in the middle of a
 # tile; more tiles than pairs, the rest of the third round shared out; the last sample and the last class alone in a tile, whole
 # and cut.
 @pytest.mark.parametrize("shape", [(873, 2800, 2, 317), (65, 972, 1, 257), (791, 9276, 4, 140), (10100, 5004, 5, 180), (65, 1108, 1, 129),
                                    (257, 4188, 1, 129), (65, 4168, 1, 1025), (321, 4264, 1, 257)])
-def test_logits_on_pairs(shape):
+def test_logits_whose_plan_is_pairs(shape):
     assert plan(*shape, shape[2] * shape[3])[0] == PAIRS
-    check(*shape)
-
-
-# ... and sizes whose plan has been theirs: forward_kernel now.
-@pytest.mark.parametrize("shape", [(190, 708, 1, 513), (9001, 4004, 2, 257), (2305, 1028, 1, 129)])
-def test_logits_near_the_choice(shape):
     check(*shape)
 
 
