@@ -604,10 +604,13 @@ __global__ void __launch_bounds__(256) mlr_emit_p_kernel(const float* __restrict
 // thread with all loads under way, in the order of mlr_lse_kernel's lanes; the label blocks find a class's samples in shared
 // memory, as its slots are only just being set here, and follow its chain while the eight samples before are on their way.  (Followed
 // between the loads, a popular class made the launch slower than the two: 4 x 256 with 100 Zipf labels 22.5 us a step in two launches,
-// 27.6 so, 21.1 now; 64 x 256 with 128 21.0, 22.3, 20.6.  With more partials, a sample's over several lanes and so the samples in
+// 24.9 so, 20.6 now; 64 x 256 with 128 21.0, 21.1, 20.4; 4 x 2,000 with 128 uniform ones 34.0 so, 30.8 now.  The next eight as bytes:
+// with pointers and coefficients in registers 64 x 1,024 with 128 23.9, 22.9 now.  64 x 256 with 128 uniform labels 18.4 to 20 so,
+// 20.2 now.  With more partials, a sample's over several lanes and so the samples in
 // several passes: 405 x 940 with 102 samples and 13 partials 28 -> 38 us; with more samples the search for a class: 191 x 140 with 225 25.6 ->
 // 28.4.  With more than 64 samples of more than 6,000 features 1.02 to 1.06 times as long.)
 constexpr int kMergeSamples = 128, kMergePartials = 8;
+static_assert(kMergeSamples < 255 && kLabelBatch == 8, "");
 __global__ void __launch_bounds__(256) mlr_merged_kernel(const float2* __restrict__ part, int64_t part_ld, int nblocks,
                                                          const float* __restrict__ Z, int64_t ldz, int64_t rows, int32_t n,
                                                          const int32_t* __restrict__ labels, float* __restrict__ lse,
@@ -696,27 +699,27 @@ __global__ void __launch_bounds__(256) mlr_merged_kernel(const float2* __restric
       if (sh_next[j] >= n) {                         // a class of one sample
         add(sh_coef[j], *reinterpret_cast<const float4*>(X + static_cast<int64_t>(j) * lab.cols));
       } else {
-        const float* xp[kLabelBatch];
-        float cf[kLabelBatch];
-        auto follow = [&]() {                        // the next eight of the chain
+        uint32_t at[kLabelBatch / 4], ahead[kLabelBatch / 4];
+        auto follow = [&](uint32_t (&q)[kLabelBatch / 4]) {        // the next eight of the chain, a byte each: 255 behind its end
+          q[0] = q[1] = 0;
 #pragma unroll
           for (int e = 0; e < kLabelBatch; ++e) {
-            xp[e] = X + static_cast<int64_t>(j < n ? j : i) * lab.cols;
-            cf[e] = j < n ? sh_coef[j] : 0.f;
+            q[e / 4] |= static_cast<uint32_t>(j < n ? j : 255) << (8 * (e % 4));
             if (j < n) j = sh_next[j];
           }
         };
-        follow();
+        auto sample = [&](int e) { return static_cast<int>((at[e / 4] >> (8 * (e % 4))) & 255u); };
+        follow(at);
         for (bool more = true; more;) {              // the chain is followed while the samples are on their way
           float4 x[kLabelBatch];
-          float cx[kLabelBatch];
-          load8(x, xp);
 #pragma unroll
-          for (int e = 0; e < kLabelBatch; ++e) cx[e] = cf[e];
+          for (int e = 0; e < kLabelBatch; ++e)
+            x[e] = __ldg(reinterpret_cast<const float4*>(X + (sample(e) < n ? sample(e) : i) * lab.cols));
           more = j < n;
-          if (more) follow();
+          if (more) follow(ahead);
 #pragma unroll
-          for (int e = 0; e < kLabelBatch; ++e) add(cx[e], x[e]);
+          for (int e = 0; e < kLabelBatch; ++e) add(sample(e) < n ? sh_coef[sample(e)] : 0.f, x[e]);
+          at[0] = ahead[0]; at[1] = ahead[1];
         }
       }
       *reinterpret_cast<float4*>(lab.dL + static_cast<int64_t>(i) * lab.cols + c) = s;
