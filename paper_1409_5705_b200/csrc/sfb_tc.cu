@@ -602,15 +602,17 @@ __global__ void __launch_bounds__(256) mlr_emit_p_kernel(const float* __restrict
 // Merged softmax of a small mini-batch (up to 128 samples, eight partials): one launch instead of mlr_lse_kernel and mlr_emit_p_kernel,
 // 1.2 of the 20 us of a step at 64 x 256 with 128 samples.  Every block merges the partials of all samples itself, a sample per
 // thread with all loads under way, in the order of mlr_lse_kernel's lanes; the label blocks find a class's samples in shared
-// memory, as its slots are only just being set here, and follow its chain while the eight samples before are on their way.  (Followed
+// memory, as its slots are only just being set here, and follow its chain, LONG while the eight samples before are on their way.  (Followed
 // between the loads, a popular class made the launch slower than the two: 4 x 256 with 100 Zipf labels 22.5 us a step in two launches,
-// 24.9 so, 20.6 now; 64 x 256 with 128 21.0, 21.1, 20.4; 4 x 2,000 with 128 uniform ones 34.0 so, 30.8 now.  The next eight as bytes:
-// with pointers and coefficients in registers 64 x 1,024 with 128 23.9, 22.9 now.  64 x 256 with 128 uniform labels 18.4 to 20 so,
-// 20.2 now.  With more partials, a sample's over several lanes and so the samples in
+// 24.9 so, 20.6 now; 4 x 2,000 with 128 uniform ones 34.0 so, 30.8 now.  The next eight as bytes:
+// with pointers and coefficients in registers 4 x 256 21.1.  With more partials, a sample's over several lanes and so the samples in
 // several passes: 405 x 940 with 102 samples and 13 partials 28 -> 38 us; with more samples the search for a class: 191 x 140 with 225 25.6 ->
 // 28.4.  With more than 64 samples of more than 6,000 features 1.02 to 1.06 times as long.)
+// LONG: the chain is followed ahead, which takes 80 registers instead of 40; where classes have more than four samples on average. (64 x 256 with
+// 128 uniform labels 18.4 us without it, 20.1 with it; 4 x 256 and 4 x 2,000 as above.)
 constexpr int kMergeSamples = 128, kMergePartials = 8;
 static_assert(kMergeSamples < 255 && kLabelBatch == 8, "");
+template <bool LONG>
 __global__ void __launch_bounds__(256) mlr_merged_kernel(const float2* __restrict__ part, int64_t part_ld, int nblocks,
                                                          const float* __restrict__ Z, int64_t ldz, int64_t rows, int32_t n,
                                                          const int32_t* __restrict__ labels, float* __restrict__ lse,
@@ -698,6 +700,25 @@ __global__ void __launch_bounds__(256) mlr_merged_kernel(const float2* __restric
       int j = i;
       if (sh_next[j] >= n) {                         // a class of one sample
         add(sh_coef[j], *reinterpret_cast<const float4*>(X + static_cast<int64_t>(j) * lab.cols));
+      } else if (!LONG) {
+        while (j < n) {
+          if (sh_next[j] >= n) {                     // the last one by itself
+            add(sh_coef[j], *reinterpret_cast<const float4*>(X + static_cast<int64_t>(j) * lab.cols));
+            break;
+          }
+          float4 x[kLabelBatch];
+          const float* xp[kLabelBatch];
+          float cf[kLabelBatch];
+#pragma unroll
+          for (int e = 0; e < kLabelBatch; ++e) {
+            xp[e] = X + static_cast<int64_t>(j < n ? j : i) * lab.cols;
+            cf[e] = j < n ? sh_coef[j] : 0.f;
+            if (j < n) j = sh_next[j];
+          }
+          load8(x, xp);
+#pragma unroll
+          for (int e = 0; e < kLabelBatch; ++e) add(cf[e], x[e]);
+        }
       } else {
         uint32_t at[kLabelBatch / 4], ahead[kLabelBatch / 4];
         auto follow = [&](uint32_t (&q)[kLabelBatch / 4]) {        // the next eight of the chain, a byte each: 255 behind its end
@@ -1502,7 +1523,7 @@ int tc_factors(sfb_ctx* ctx, int64_t off, int64_t n, const float* X, const float
   }
   if (fused && n == K && softmax_merged(n, c.cols, tiles_n)) {
     const int lab = label_blocks(ctx);
-    CKC(launch_kernel(mlr_merged_kernel, dim3(grid1d(n * ((rows + 7) / 8), 256) + lab), dim3(256), 0, ctx->stream, 1,
+    CKC(launch_kernel(n > 4 * rows ? mlr_merged_kernel<true> : mlr_merged_kernel<false>, dim3(grid1d(n * ((rows + 7) / 8), 256) + lab), dim3(256), 0, ctx->stream, 1,
                       ctx->at<float2>(L.part), K, tiles_n, Z, ldz, rows, static_cast<int32_t>(n), labels, lse, ctx->at<float>(L.loss),
                       ctx->at<float>(L.coef), ctx->at<int32_t>(L.slot), ctx->at<__nv_bfloat16>(L.P), L.ldp, ctx->at<uint32_t>(L.status),
                       lab, label_args(ctx, X)));
