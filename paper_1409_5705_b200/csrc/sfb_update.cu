@@ -13,14 +13,11 @@
 // a sixth of a step of metric learning at 1,000 x 20,000).  The tf32 words are K-major (U^T, V^T).
 // Warps of a CTA: 0 = TMA producer, 1 = MMA issuer (leader CTA only) and TMEM owner, 2..9 = epilogue.
 // Epilogue warp (q, h): TMEM lane quarter q (32 rows of W), column half h (128 columns), in four chunks of
-// 32 x 32.  Each warp owns a ring of three 4 KB slots: the W chunk lands there by TMA (two chunks in flight per warp, 64 KB per SM),
-// is combined in place with the accumulator chunk and goes back by TMA from the same slot; a lane has a row of the
+// 32 x 32.  Each warp owns a ring of 4 KB slots: the W chunk lands there by TMA (two chunks in flight per warp, 64 KB per SM, or
+// four), is combined in place with the accumulator chunk and goes back by TMA from the same slot; a lane has a row of the
 // chunk and stores its 32 roundings of the bf16 copy as two sectors.  (The copy by rows, read back from the slot with 8 lanes a row,
 // was a third of a warp's chain per chunk: 10,000 x 20,000, 64 pairs 480 us of the pass, 420 without, 374 where few rows change.)
-// Shared memory is the scarce resource: 4 operand stages (128 KB) + the rings (96 KB).  us of an update, these / two stages and five slots,
-// which have four chunks in flight: 5,000 x 3,000 with 64, 128, 256 pairs 35.4, 38.3, 41.4 / 34.9, 37.1, 41.1; 10,000 x 20,000 366, 373, 405 /
-// 367, 377, 396; 78,798 x 1,716 252, 262, 272 / 259, 270, 284; 300,000 x 500 272, 285, 310 / 279, 292, 324; 1,024 pairs of 10,000 x
-// 20,000 472 / 713.  (3 + 4: 552; 5 + 2: 495.)
+// Shared memory is the scarce resource: see UpShape.
 #include <cuda.h>
 #include <cuda_bf16.h>
 
@@ -47,9 +44,19 @@ constexpr int kPend = 1;                      // TMA stores of a warp that may s
 constexpr int kEpiWarps = 8;
 constexpr int kThreads = 64 + 32 * kEpiWarps;
 constexpr int kTmemCols = 512;
-constexpr int kStages = 4, kRing = 3;         // operand stages; slots per epilogue warp
-constexpr int kBars = 2 * kStages + 4 + kEpiWarps * kRing;
-constexpr int kSmem = kStages * kStageBytes + kEpiWarps * kRing * kSlotBytes + kBars * 8 + 16 + 1024;
+// Two splits of the shared memory.  Four operand stages and a ring of three slots per epilogue warp; FEW, where every tile has a pair of CTAs of
+// its own and the contraction fits two stages (up to kFewPairs pairs): two stages and five slots, so that all four chunks of a warp are under
+// way at once.  us of a step, 4 + 3 / 2 + 5: 64 x 256 with 128 samples 20.5 / 18.2 to 19.5, 500 x 1,000 28.3 / 28.15, 1,000 x 1,000 30.2 / 30.1,
+// 512 x 2,048 with 64 24.7 / 24.6; beyond: 1,000 x 1,000 with 256 30.5 / 31.2, 2,000 x 500 with 256 27.4 / 28.1.  us of an update:
+// 5,000 x 3,000 with 128, 256 pairs 31.2, 34.8 / 32.7, 36.3; 10,000 x 20,000 with 64 366 / 367, 1,024 472 / 713;
+// 78,798 x 1,716 with 256 272 / 284.  (3 + 4: 552; 5 + 2: 495.)
+constexpr int kFewPairs = 128;
+template <bool FEW>
+struct UpShape {
+  static constexpr int kStages = FEW ? 2 : 4, kRing = FEW ? 5 : 3;
+  static constexpr int kBars = 2 * kStages + 4 + kEpiWarps * kRing;
+  static constexpr int kSmem = kStages * kStageBytes + kEpiWarps * kRing * kSlotBytes + kBars * 8 + 16 + 1024;
+};
 
 struct UpdParams {
   int32_t rows, cols;          // shape of W
@@ -101,10 +108,11 @@ __device__ __forceinline__ void tile_origin(const UpdParams& p, int tile, int& m
 // TF32: the operands are 32-bit words read as tf32 (32 elements per 128-byte k-block), see the forward kernel.
 // SHADOW: the operand copy of the new W that the epilogue writes beside it for the next forward product:
 // 1 bf16, 2 the (big | small) pair of tf32 words of the fp32-on-tensor-cores mode.
-template <int SHADOW, bool TF32 = false>
+template <int SHADOW, bool TF32 = false, bool FEW = false>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
 update_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                    const __grid_constant__ CUtensorMap tmC, const UpdParams p) {
+  constexpr int kStages = UpShape<FEW>::kStages, kRing = UpShape<FEW>::kRing, kBars = UpShape<FEW>::kBars;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint8_t* sA = smem;
@@ -644,10 +652,11 @@ int tile_width(int64_t rows, int64_t cols, int64_t kblocks, int pairs, bool spli
 
 int tc_update_init(sfb_ctx* ctx, TcState* st) {
   int n = 1 << 30;
-  CKC(prepare_pair_kernel(update_pair_kernel<1>, kThreads, kSmem, &n));
+  CKC(prepare_pair_kernel(update_pair_kernel<1>, kThreads, UpShape<false>::kSmem, &n));
+  CKC((prepare_pair_kernel(update_pair_kernel<1, false, true>, kThreads, UpShape<true>::kSmem, &n)));
   CKC(prepare_pair_kernel(update_split_kernel<false>, kThreads, SuShape<false>::kSmem, &n));
   CKC(prepare_pair_kernel(update_split_kernel<true>, kThreads, SuShape<true>::kSmem, &n));
-  CKC((prepare_pair_kernel(update_pair_kernel<2, true>, kThreads, kSmem, &n)));
+  CKC((prepare_pair_kernel(update_pair_kernel<2, true>, kThreads, UpShape<false>::kSmem, &n)));
   CKC(forward_pair_prepare(&n));
   st->max_pairs = n;
   if (n < 1) return SFB_ERR_ARCH;                 // the device cannot host a CTA pair of these kernels
@@ -688,7 +697,7 @@ int tc32_update(sfb_ctx* ctx) {
   p.shadow = nullptr; p.shadow32 = ctx->at<float>(L.Ws); p.shadow_ld = 2 * L.colsp; p.shadow_half = L.colsp;
   const int64_t tiles = static_cast<int64_t>(p.tilesM) * p.tilesN;
   const unsigned grid = 2u * static_cast<unsigned>(std::min<int64_t>(tiles, st->max_pairs));
-  CKC(launch_kernel_if(tiles <= st->max_pairs, (update_pair_kernel<2, true>), dim3(grid), dim3(kThreads), kSmem, ctx->stream, 1, ma, mb, mc, p));
+  CKC(launch_kernel_if(tiles <= st->max_pairs, (update_pair_kernel<2, true>), dim3(grid), dim3(kThreads), UpShape<false>::kSmem, ctx->stream, 1, ma, mb, mc, p));
   return SFB_OK;
 }
 
@@ -738,7 +747,11 @@ int tc_update(sfb_ctx* ctx) {
   p.nseg = 1;
   p.shadow = ctx->at<__nv_bfloat16>(L.Wb); p.shadow_ld = L.colsb;
   p.copy_counters = &ctx->at<Scalars>(L.scalars)->copy_pieces;
-  CKC(launch_kernel_if(tiles <= st->max_pairs, update_pair_kernel<1>, dim3(grid), dim3(kThreads), kSmem, ctx->stream, 1, ma, mb, mc, p));
+  CKC(ctx->K <= kFewPairs && tiles <= st->max_pairs
+          ? launch_kernel((update_pair_kernel<1, false, true>), dim3(grid), dim3(kThreads),
+                             UpShape<true>::kSmem, ctx->stream, 1, ma, mb, mc, p)
+          : launch_kernel_if(tiles <= st->max_pairs, update_pair_kernel<1>, dim3(grid), dim3(kThreads), UpShape<false>::kSmem,
+                             ctx->stream, 1, ma, mb, mc, p));
   return SFB_OK;
 }
 
